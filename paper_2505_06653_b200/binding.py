@@ -1,14 +1,17 @@
-"""ctypes binding of ``libbof4.so``: argument marshalling only.
+"""Binding of ``libbof4.so``: argument marshalling only.
 
 Every function here has the name of the C entry point it calls (see ``include/bof4.h``) and
 does nothing but turn torch CUDA tensors into device pointers, allocate the outputs with torch
 (device memory and streams are the only things torch is used for) and check the status code.
-All arithmetic of the method runs in the CUDA kernels; there is no CPU fallback: if the shared
+The calls that sit in a user's inner loop do this in native code (``csrc/torch_host.cpp``, loaded
+as ``_bof4_torch``: a call on a small tensor is bound by its host side); the others through ctypes.
+All arithmetic of the method runs in the CUDA kernels; there is no CPU fallback: if a shared
 library is missing or no CUDA device is present, the calls raise.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import List, Optional, Sequence, Tuple
 
@@ -17,6 +20,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libbof4.so")
+HOST_PATH = os.path.join(_HERE, "_bof4_torch.so")
 
 F32, BF16 = 0, 1
 NORM_ABS, NORM_SIGNED = 0, 1
@@ -129,6 +133,25 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_host = None
+
+
+def _native():
+    """The native half of the binding.  Raises if it has not been built."""
+    global _host
+    if _host is None:
+        lib()
+        if not os.path.exists(HOST_PATH):
+            raise ImportError("%s not found: run `python -m paper_2505_06653_b200.build`" % HOST_PATH)
+        spec = importlib.util.spec_from_file_location("_bof4_torch", HOST_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        m.set_hooks(Bof4Error, _codebook)
+        m.set_allocator(_allocator)
+        _host = m
+    return _host
+
+
 def _check(rc: int):
     if rc != 0:
         raise Bof4Error(rc, lib().bof4_last_error().decode())
@@ -163,6 +186,8 @@ def set_output_allocator(fn) -> None:
     harness uses it to surround each buffer with guard bands."""
     global _allocator
     _allocator = fn
+    if _host is not None:
+        _host.set_allocator(fn)
 
 
 def _new(numel: int, dtype, device, zero: bool = False) -> torch.Tensor:
@@ -318,26 +343,7 @@ def bof4_fit_codebook(weights, block_size: int, norm: int, metric: int, levels, 
     """``iters`` Lloyd iterations; returns (levels, err_log) as device tensors (fp32[16],
     fp64[iters]).  With sync=False nothing waits for the stream.  `out` = (fp32[16], fp64[>= iters])
     device tensors to hold the results instead of fresh allocations."""
-    ws, dt, ptrs, sizes = _tensor_list(weights)
-    dev = ws[0].device
-    if out is not None:
-        cb, log = _dev(out[0], "out[0]"), _dev(out[1], "out[1]")
-        if cb.dtype != torch.float32 or cb.numel() != LEVELS or log.dtype != torch.float64 or log.numel() < iters:
-            raise ValueError("out must be (float32[16], float64[>= iters])")
-        src = _codebook(levels, dev)
-        if src.data_ptr() != cb.data_ptr():  # levels may be the output buffer itself: continue in place
-            cb.copy_(src)
-    else:
-        cb = _codebook(levels, dev).clone()
-        log = _new(max(iters, 1), torch.float64, dev, zero=True)
-    wsp = workspace if workspace is not None else _workspace(
-        OP_EM, sum(w.numel() for w in ws), block_size, metric, dev)
-    with torch.cuda.device(dev):
-        _check(lib().bof4_fit_codebook(ptrs, sizes, len(ws), dt, block_size, norm, metric, _ptr(cb),
-                                       fixed_mask, iters, _ptr(log), _ptr(wsp), wsp.numel(), _stream()))
-    if sync:
-        torch.cuda.current_stream(dev).synchronize()
-    return cb, log[:iters]
+    return _native().fit_codebook(weights, block_size, norm, metric, levels, fixed_mask, iters, workspace, sync, out)
 
 
 def bof4_theoretical_codebook(block_size: int, norm: int, metric: int, levels, fixed_mask: int,
@@ -400,19 +406,7 @@ def bof4_quantize(w: torch.Tensor, block_size: int, norm: int, levels,
                   scale_dtype: Optional[int] = None,
                   out: Optional[Tuple[torch.Tensor, torch.Tensor]] = None):
     """-> (codes uint8[n/2], scales [n/block_size])."""
-    w = _dev(w, "w").reshape(-1)
-    n, dt = w.numel(), _dt(w)
-    sd = dt if scale_dtype is None else scale_dtype
-    cb = _codebook(levels, w.device)
-    if out is None:
-        codes = _new((n + 1) // 2, torch.uint8, w.device)
-        scales = _new(-(-n // max(block_size, 1)), _torch_dt(sd), w.device)
-    else:
-        codes, scales = out
-    with torch.cuda.device(w.device):
-        _check(lib().bof4_quantize(_ptr(w), dt, n, block_size, norm, _ptr(cb), _ptr(codes),
-                                   _ptr(scales), sd, _stream()))
-    return codes, scales
+    return _native().quantize(w, block_size, norm, levels, scale_dtype, out)
 
 
 def bof4_dequantize(codes: torch.Tensor, scales: torch.Tensor, block_size: int, levels,
@@ -420,47 +414,14 @@ def bof4_dequantize(codes: torch.Tensor, scales: torch.Tensor, block_size: int, 
                     out: Optional[torch.Tensor] = None, n: Optional[int] = None) -> torch.Tensor:
     """-> dequantised tensor [n]; `outliers` = (idx int32, val bf16, n_out int64[1]) for OPQ.
     `n` = number of weights when it is odd (default: twice the number of code bytes)."""
-    codes = _dev(codes, "codes")
-    scales = _dev(scales, "scales")
-    n = codes.numel() * 2 if n is None else int(n)
-    if (n + 1) // 2 != codes.numel():
-        raise ValueError("codes must hold (n + 1) // 2 bytes")
-    cb = _codebook(levels, codes.device)
-    if out is None:
-        out = _new(n, _torch_dt(out_dtype), codes.device)
-    idx = val = cnt = None
-    cap = 0
-    if outliers is not None:
-        idx, val, cnt = outliers
-        cap = idx.numel()
-    with torch.cuda.device(codes.device):
-        _check(lib().bof4_dequantize(_ptr(codes), _ptr(scales), _dt(scales), n, block_size, _ptr(cb),
-                                     _ptr(idx), _ptr(val), _ptr(cnt), cap, _ptr(out), out_dtype,
-                                     _stream()))
-    return out
+    return _native().dequantize(codes, scales, block_size, levels, out_dtype, outliers, out, n)
 
 
 def bof4_gemv(codes: torch.Tensor, scales: torch.Tensor, rows: int, cols: int, block_size: int, levels,
               x: torch.Tensor, outliers: Optional[Tuple[torch.Tensor, torch.Tensor, torch.Tensor]] = None,
               out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """-> y fp32 [rows] = W_q x for the rows x cols matrix held as (codes, scales[, outliers])."""
-    codes = _dev(codes, "codes")
-    scales = _dev(scales, "scales")
-    x = _dev(x, "x")
-    if codes.numel() * 2 != rows * cols or x.numel() != cols:
-        raise ValueError("codes must hold rows * cols weights and x cols values")
-    cb = _codebook(levels, codes.device)
-    if out is None:
-        out = _new(rows, torch.float32, codes.device)
-    idx = val = cnt = None
-    cap = 0
-    if outliers is not None:
-        idx, val, cnt = outliers
-        cap = idx.numel()
-    with torch.cuda.device(codes.device):
-        _check(lib().bof4_gemv(_ptr(codes), _ptr(scales), _dt(scales), rows, cols, block_size, _ptr(cb),
-                               _ptr(x), _dt(x), _ptr(idx), _ptr(val), _ptr(cnt), cap, _ptr(out), _stream()))
-    return out
+    return _native().gemv(codes, scales, rows, cols, block_size, levels, x, outliers, out)
 
 
 def opq_split(w: torch.Tensor, block_size: int, tau: float, capacity: int,
@@ -485,128 +446,38 @@ def bof4_gemm_tc(codes: torch.Tensor, scales: torch.Tensor, rows: int, cols: int
                  outliers: Optional[Tuple[torch.Tensor, torch.Tensor, torch.Tensor]] = None):
     """Y fp32 [rows, n_rhs] = W_q X^T on the tensor cores for x bf16 [n_rhs, cols].
     -> (y, status int32[1]); status 0 unless a bounded wait inside the kernel ran out."""
-    codes = _dev(codes, "codes")
-    scales = _dev(scales, "scales")
-    x = _dev(x, "x")
-    if x.dtype != torch.bfloat16 or x.dim() != 2 or x.shape[1] != cols or codes.numel() * 2 != rows * cols:
-        raise ValueError("x must be bf16 [n_rhs, cols] and codes must hold rows * cols weights")
-    n_rhs = x.shape[0]
-    cb = _codebook(levels, codes.device)
-    y = _new(rows * n_rhs, torch.float32, codes.device).view(rows, n_rhs)
-    status = _new(1, torch.int32, codes.device, zero=True)
-    ws = workspace if workspace is not None else (_new(8 * rows * n_rhs * 4, torch.uint8, codes.device) if split else None)
-    with torch.cuda.device(codes.device):
-        idx = val = cnt = None
-        cap = 0
-        if outliers is not None:
-            idx, val, cnt = (_dev(t, "outliers") for t in outliers)
-            cap = idx.numel()
-        _check(lib().bof4_gemm_tc(_ptr(codes), _ptr(scales), _dt(scales), rows, cols, block_size, _ptr(cb), _ptr(x),
-                                  n_rhs, _ptr(idx), _ptr(val), _ptr(cnt), cap, _ptr(y), _ptr(status), _ptr(ws),
-                                  ws.numel() if ws is not None else 0, _stream()))
-    return y, status
+    return _native().gemm_tc(codes, scales, rows, cols, block_size, levels, x, workspace, split, outliers)
 
 
 def bof4_outlier_count(n_out: torch.Tensor, capacity: int) -> int:
     """Waits for the current stream and returns the true outlier count; raises Bof4Error
     (BOF4_ERR_CAPACITY) when it exceeds `capacity`, i.e. when outliers were dropped."""
-    n_out = _dev(n_out, "n_out")
-    if n_out.dtype != torch.int64 or n_out.numel() != 1:
-        raise ValueError("n_out must be the int64[1] count tensor of an OPQ call")
-    host = ctypes.c_int64(0)
-    with torch.cuda.device(n_out.device):
-        _check(lib().bof4_outlier_count(_ptr(n_out), int(capacity), ctypes.byref(host), _stream()))
-    return int(host.value)
-
-
-def _ptr_array(tensors):
-    return (ctypes.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
+    return _native().outlier_count(n_out, capacity)
 
 
 def bof4_quantize_batch(weights, block_size: int, norm: int, levels, scale_dtype: Optional[int] = None, out=None):
     """bof4_quantize over a list of tensors in few launches -> (list of codes, list of scales).
     `out` = (codes list, scales list) to write into instead of fresh allocations."""
-    ws, dt, ptrs, sizes = _tensor_list(weights)
-    dev = ws[0].device
-    cb = _codebook(levels, dev)
-    sd = dt if scale_dtype is None else scale_dtype
-    if out is not None:
-        codes, scales = [_dev(c, "codes") for c in out[0]], [_dev(s, "scales") for s in out[1]]
-    else:
-        codes = [_new((w.numel() + 1) // 2, torch.uint8, dev) for w in ws]
-        scales = [_new(-(-w.numel() // max(block_size, 1)), _torch_dt(sd), dev) for w in ws]
-    for w, c, sc in zip(ws, codes, scales):
-        if c.numel() != (w.numel() + 1) // 2 or sc.numel() != -(-w.numel() // max(block_size, 1)) or _dt(sc) != sd:
-            raise ValueError("out buffers do not match the tensors")
-    with torch.cuda.device(dev):
-        _check(lib().bof4_quantize_batch(ptrs, sizes, len(ws), dt, block_size, norm, _ptr(cb), _ptr_array(codes),
-                                         _ptr_array(scales), sd, _stream()))
-    return codes, scales
+    return _native().quantize_batch(weights, block_size, norm, levels, scale_dtype, out)
 
 
 def bof4_dequantize_batch(codes, scales, sizes, block_size: int, levels, out_dtype: int = BF16, out=None):
     """bof4_dequantize (no outlier list) over a list of tensors in few launches -> list of outputs."""
-    codes = [_dev(c, "codes") for c in codes]
-    scales = [_dev(s, "scales") for s in scales]
-    dev = codes[0].device
-    cb = _codebook(levels, dev)
-    outs = [_dev(o, "out") for o in out] if out is not None else [_new(int(n), _torch_dt(out_dtype), dev) for n in sizes]
-    ns = (ctypes.c_int64 * len(codes))(*[int(n) for n in sizes])
-    for c, sc, o, n in zip(codes, scales, outs, sizes):
-        if c.numel() != (n + 1) // 2 or sc.numel() != -(-n // max(block_size, 1)) or o.numel() != n \
-                or _dt(o) != out_dtype or _dt(sc) != _dt(scales[0]):
-            raise ValueError("buffers do not match the sizes")
-    with torch.cuda.device(dev):
-        _check(lib().bof4_dequantize_batch(_ptr_array(codes), _ptr_array(scales), _dt(scales[0]), ns, len(codes),
-                                           block_size, _ptr(cb), _ptr_array(outs), out_dtype, _stream()))
-    return outs
+    return _native().dequantize_batch(codes, scales, sizes, block_size, levels, out_dtype, out)
 
 
 def bof4_scales_compress(scales: torch.Tensor, norm: int):
     """Double quantisation of block constants -> (q uint8[B], group fp32[ceil(B/256)], sign uint8[ceil(B/8)] or None)."""
-    scales = _dev(scales, "scales")
-    B = scales.numel()
-    dev = scales.device
-    q = _new(B, torch.uint8, dev)
-    g = _new((B + 255) // 256, torch.float32, dev)
-    sign = _new((B + 7) // 8, torch.uint8, dev) if norm == NORM_SIGNED else None
-    with torch.cuda.device(dev):
-        _check(lib().bof4_scales_compress(_ptr(scales), _dt(scales), B, norm, _ptr(q), _ptr(g),
-                                          _ptr(sign) if sign is not None else None, _stream()))
-    return q, g, sign
+    return _native().scales_compress(scales, norm)
 
 
 def bof4_scales_expand(q: torch.Tensor, group: torch.Tensor, sign: Optional[torch.Tensor]) -> torch.Tensor:
     """The decoder's fp32 block constants from their double-quantised form."""
-    q = _dev(q, "q")
-    out = _new(q.numel(), torch.float32, q.device)
-    with torch.cuda.device(q.device):
-        _check(lib().bof4_scales_expand(_ptr(q), _ptr(_dev(group, "group")),
-                                        _ptr(_dev(sign, "sign")) if sign is not None else None, q.numel(),
-                                        _ptr(out), _stream()))
-    return out
+    return _native().scales_expand(q, group, sign)
 
 
 def bof4_quantize_opq(w: torch.Tensor, block_size: int, norm: int, levels, tau: float,
                       capacity: int, scale_dtype: Optional[int] = None,
                       workspace: Optional[torch.Tensor] = None, out=None):
     """-> (codes, scales, idx int32[capacity], val bf16[capacity], n_out int64[1])."""
-    w = _dev(w, "w").reshape(-1)
-    n, dt = w.numel(), _dt(w)
-    dev = w.device
-    sd = dt if scale_dtype is None else scale_dtype
-    cb = _codebook(levels, dev)
-    wsp = workspace if workspace is not None else _workspace(OP_OPQ, n, block_size, 0, dev)
-    if out is None:
-        codes = _new((n + 1) // 2, torch.uint8, dev)
-        scales = _new(-(-n // max(block_size, 1)), _torch_dt(sd), dev)
-        idx = _new(capacity, torch.int32, dev)
-        val = _new(capacity, torch.bfloat16, dev)
-        cnt = _new(1, torch.int64, dev, zero=True)
-    else:
-        codes, scales, idx, val, cnt = out
-    with torch.cuda.device(dev):
-        _check(lib().bof4_quantize_opq(_ptr(w), dt, n, block_size, norm, _ptr(cb), tau, _ptr(codes),
-                                       _ptr(scales), sd, _ptr(idx), _ptr(val), capacity, _ptr(cnt),
-                                       _ptr(wsp), wsp.numel(), _stream()))
-    return codes, scales, idx, val, cnt
+    return _native().quantize_opq(w, block_size, norm, levels, tau, capacity, scale_dtype, workspace, out)
