@@ -73,6 +73,7 @@ extern "C" {
 
 #define BOF4_OP_EM 0  /* bof4_em_step / bof4_fit_codebook workspace */
 #define BOF4_OP_OPQ 1 /* opq_split / bof4_quantize_opq workspace    */
+#define BOF4_OP_EM_BF16 2 /* the same as BOF4_OP_EM where all tensors are bf16 (smaller) */
 
 #define BOF4_LEVELS 16
 
@@ -112,9 +113,12 @@ typedef struct bof4_em_stats {
  *                     metric = MAE, the per-level selection histograms and candidate lists.
  *                     n_max = the TOTAL number of weights of the tensor list.  The candidate lists
  *                     grow with it (n_max / 8 bytes, between 8 MiB and 1 GiB); any workspace of at
- *                     least bof4_workspace_bytes(BOF4_OP_EM, 0, ...) is accepted, a smaller one
- *                     than asked for here only costs the MAE fit one more pass over the data per
- *                     iteration.  Results do not depend on the workspace size.
+ *                     least bof4_workspace_bytes(BOF4_OP_EM, 0, ...) is accepted.  A fit of four or
+ *                     more iterations puts its samples in order once (16 bytes per weight up to 2^26
+ *                     weights; bf16 data of 2^22 weights and more: about 90 MB and 10 bytes per block,
+ *                     BOF4_OP_EM_BF16); with a smaller workspace than asked for here it streams the data
+ *                     in every iteration.  Medians do not depend on the workspace size, sums only by
+ *                     their rounding.
  *   op = BOF4_OP_OPQ: per-tile outlier staging and tile offsets of the ordered compaction.
  */
 BOF4_API size_t bof4_workspace_bytes(int op, int64_t n_max, int block_size, int metric);

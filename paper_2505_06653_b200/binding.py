@@ -26,7 +26,7 @@ F32, BF16 = 0, 1
 NORM_ABS, NORM_SIGNED = 0, 1
 METRIC_MSE, METRIC_MAE = 0, 1
 METRIC_MSE_NORMALIZED, METRIC_MAE_NORMALIZED = 2, 3  # App. D: errors of the normalised weights
-OP_EM, OP_OPQ = 0, 1
+OP_EM, OP_OPQ, OP_EM_BF16 = 0, 1, 2
 LEVELS = 16
 
 # kernels one MAE iteration enqueues: setup, 2 x (data pass + bin selection), then 2 data passes

@@ -12,6 +12,7 @@
 // bit-reproducible.  The COUNT variant also keeps the member count of every region.
 #include "common.cuh"
 #include "em_common.cuh"
+#include "em_sorted.cuh"
 #include "lane32.cuh"
 #include "layout.h"
 
@@ -902,6 +903,11 @@ extern "C" int bof4_fit_codebook(const void* const* h_w, const int64_t* h_n, int
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     double* partials = static_cast<double*>(d_ws);
+    // Four or more iterations: put the samples in order once (em_cells.cu, em_sorted.cu); fewer, or a
+    // workspace that does not hold them: stream the data in every iteration.
+    bool done = false;
+    if ((rc = cells_fit(a, d_codebook, fixed_mask, iters, d_err_log, d_ws, ws_bytes, st, &done)) || done) return rc;
+    if ((rc = sorted_fit(a, d_codebook, fixed_mask, iters, d_err_log, d_ws, ws_bytes, st, &done)) || done) return rc;
     if (metric == BOF4_METRIC_MSE || metric == BOF4_METRIC_MSE_NORMALIZED) {
         if (iters > 0 && (rc = reset_ticket(partials, st))) return rc;
         for (int t = 0; t < iters; ++t) {

@@ -1,0 +1,678 @@
+// Codebook fit of bf16 data over its distinct normalised weights (see em_sorted.cuh).
+//
+// A bf16 number has an 8-bit significand, so w / m is (a / b) 2^e with a and b in 128 ... 255: whatever
+// the size of the data, the normalised weights of magnitude 2^-40 and more take at most 128 * 128 * 2 * 40
+// values, and the fit only needs the sum of the sample weights (m^2 or |m|) of each.  The data is read
+// twice, once for the block constants and once for the counts; then a fit of any number of iterations
+// works on at most 1.3 million samples (about 0.4 million for near-Gaussian data).
+//
+//   blocks      block constants (bf16, stored) and the number of blocks per magnitude; HBM bound
+//   plan        first position of every magnitude, units of work
+//   order       block addresses grouped by magnitude
+//   accumulate  a unit is some blocks of ONE magnitude |m|: with m fixed, the cell of a weight is the
+//               difference of the two bit patterns, so the counts of a unit are 10240 words of shared
+//               memory and a weight costs a subtraction, a comparison and one shared-memory reduction
+//               (about 3.5 wavefronts per 32 weights on random banks, which bounds the pass); when the
+//               unit is done its counts times the weight of |m| are added to the cells
+//   items       the occupied cells in a fixed order, as samples for the ordering passes
+//
+// A cell is (significand of m, sign, distance of the bit patterns).  Cell sums are integers (128 bits, a
+// fixed-point scale relative to the largest |m|; exact while |m| is within 2^-38 of it), so they do not
+// depend on the order of the additions.  Normalised weights below 2^-40 in magnitude count as zero.
+#include "em_sorted.cuh"
+#include "lane32.cuh"
+
+namespace bof4 {
+
+constexpr int kCellDepth = 40 * 128;              // bit-pattern distances told apart: 40 binades
+constexpr int kCellRow = 2 * kCellDepth + 1;      // positive, negative, zero
+constexpr int kCells = 128 * kCellRow;
+constexpr int kMags = 32768;                      // magnitudes of a bf16 number
+constexpr int kCellThreads = 512;
+constexpr int kCellCtas = 3;                      // per SM
+constexpr int kCellScan = 2048;                   // cells per CTA of the items pass
+constexpr int kCellScans = (kCells + kCellScan - 1) / kCellScan;
+constexpr int64_t kCellsMinN = (int64_t)1 << 22;  // below: one sample per weight is cheaper (measured)
+constexpr int kMagTiny = 48 * 128;                // |m| below 2^-79: subnormal weights within 40 binades
+
+bool cells_apply(int w_dtype, int64_t n) { return w_dtype == BOF4_BF16 && n >= kCellsMinN; }
+
+struct CellUnit {
+    uint32_t mag, first, count;  // bit pattern of |m|, first block in the ordered list, blocks
+};
+struct CellsWs {
+    uint32_t* hist;      // [kMags] blocks per magnitude
+    uint32_t* cursor;    // [kMags] next free position of the ordered list
+    uint32_t* scal;      // [0] units, [1] next unit, [2] largest magnitude of the short last blocks, [3] of all
+    uint32_t* scans;     // [kCellScans]
+    ulonglong2* acc;     // [kCells]
+    unsigned long long* acc_a;
+    CellUnit* units;
+    unsigned long long* order;  // [blocks] address, sign of the constant in bit 63
+    uint16_t* consts;           // [blocks]
+    SortWs sort;
+};
+
+constexpr int kMaxExtraUnits = 16 * kSMs;  // units beyond one per magnitude: blocks / unit size
+
+static int unit_blocks(int64_t blocks, int block_size)
+{
+    const int64_t least = 131072 / block_size, even = (blocks + kMaxExtraUnits - 1) / kMaxExtraUnits;
+    return (int)(even > least ? even : least);
+}
+
+static size_t cells_layout(void* base, int64_t n, int block_size, CellsWs* W)
+{
+    char* p = static_cast<char*>(base);
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* q = p ? p + off : nullptr;
+        off += align_up(bytes, 256);
+        return q;
+    };
+    const size_t blocks = (size_t)(n / block_size) + 1;
+    CellsWs L;
+    L.hist = reinterpret_cast<uint32_t*>(take((size_t)kMags * 4));
+    L.scal = reinterpret_cast<uint32_t*>(take(256));
+    L.acc = reinterpret_cast<ulonglong2*>(take((size_t)kCells * 16));
+    L.acc_a = reinterpret_cast<unsigned long long*>(take((size_t)kCells * 8));  // the four arrays above are cleared together
+    L.cursor = reinterpret_cast<uint32_t*>(take((size_t)kMags * 4));
+    L.scans = reinterpret_cast<uint32_t*>(take((size_t)kCellScans * 4));
+    L.units = reinterpret_cast<CellUnit*>(take((size_t)(kMags + kMaxExtraUnits) * sizeof(CellUnit)));
+    L.order = reinterpret_cast<unsigned long long*>(take(blocks * 8));
+    L.consts = reinterpret_cast<uint16_t*>(take(blocks * 2));
+    char* rest = p ? p + off : nullptr;
+    off += sorted_layout(rest, kCells, true, &L.sort);
+    if (W) *W = L;
+    return off;
+}
+
+size_t cells_workspace_bytes(int64_t n, int block_size)
+{
+    return n >= kCellsMinN ? cells_layout(nullptr, n, block_size, nullptr) : 0;
+}
+
+// ---------------------------------------------------------------- weights and cells of one magnitude
+
+// Bit pattern of a bf16 value scaled by 2^64 (exact; makes subnormal values normal).
+__device__ __forceinline__ uint32_t scaled16(uint32_t bits)
+{
+    return __float_as_uint(__uint_as_float(bits << 16) * 0x1p64f) >> 16;
+}
+
+// The sample weight of |m| (per weight) as an integer times 2^shift.
+struct MagWeight {
+    uint32_t b;       // significand, 128 ... 255
+    uint32_t base;    // b^2, b or 1
+    int shift;
+    uint32_t fixed;   // MAE: weight of the median
+};
+constexpr int kMseScale = 76, kMaeScale = 84;  // 2^33 weights of the largest |m| stay below 2^128
+
+__device__ __forceinline__ int true_exponent(uint32_t mag)  // biased exponent, extended below the normal range
+{
+    return mag < (uint32_t)kMagTiny ? (int)(scaled16(mag) >> 7) - 64 : (int)(mag >> 7);
+}
+__device__ __forceinline__ MagWeight mag_weight(uint32_t mag, uint32_t max_mag, int metric)
+{
+    MagWeight r;
+    const uint32_t s = mag < (uint32_t)kMagTiny ? scaled16(mag) : mag;
+    r.b = 128u + (s & 127u);
+    const int k = true_exponent(max_mag) - true_exponent(mag);
+    if (metric >= 2) {
+        r.base = 1u;
+        r.shift = kMaeScale;
+        r.fixed = 1u;
+    } else if (metric == BOF4_METRIC_MSE) {
+        r.base = r.b * r.b;
+        r.shift = kMseScale - 2 * k;
+        r.fixed = 0u;
+    } else {
+        r.base = r.b;
+        r.shift = kMaeScale - k;
+        r.fixed = sort_fixed_weight(__uint_as_float(mag << 16), max_mag << 16);
+    }
+    return r;
+}
+__device__ __forceinline__ double cell_scale(uint32_t max_mag, int metric)
+{
+    if (metric >= 2) return ldexp(1.0, -kMaeScale);
+    const int e = true_exponent(max_mag) - 134;  // |m| = b 2^(exponent - 134)
+    return metric == BOF4_METRIC_MSE ? ldexp(1.0, 2 * e - kMseScale) : ldexp(1.0, e - kMaeScale);
+}
+
+__device__ __forceinline__ void cell_add(const CellsWs& W, uint32_t cell, unsigned long long count, const MagWeight& m, bool mae)
+{
+    const unsigned long long v = count * m.base;
+    unsigned long long lo, hi = 0ull;
+    if (m.shift >= 64) {
+        lo = 0ull;
+        hi = v << (m.shift - 64);
+    } else if (m.shift > 0) {
+        lo = v << m.shift;
+        hi = v >> (64 - m.shift);
+    } else {
+        lo = m.shift > -64 ? v >> (-m.shift) : 0ull;
+    }
+    unsigned long long* p = reinterpret_cast<unsigned long long*>(W.acc + cell);
+    if (lo) {
+        const unsigned long long old = atomicAdd(p, lo);
+        if (old + lo < old) ++hi;
+    }
+    if (hi) atomicAdd(p + 1, hi);
+    if (mae && m.fixed) atomicAdd(W.acc_a + cell, count * m.fixed);
+}
+
+// ---------------------------------------------------------------- block constants
+
+template <int I, bool SIGNED>
+__global__ void __launch_bounds__(1024, 1)
+cells_blocks_kernel(const EmTensors T, const int64_t first_block, uint32_t* __restrict__ hist, uint16_t* __restrict__ consts)
+{
+    extern __shared__ uint32_t s_hist[];  // [kMags]
+    __shared__ WideScratch s_wide;
+    __shared__ const void* s_ptr[kEmMaxTensors];
+    __shared__ int64_t s_n[kEmMaxTensors], s_row_end[kEmMaxTensors], s_block0[kEmMaxTensors];
+    const int tid = threadIdx.x;
+    for (int k = tid; k < kMags; k += 1024) s_hist[k] = 0u;
+    if (tid < T.count) {
+        s_ptr[tid] = T.ptr[tid];
+        s_n[tid] = T.n[tid];
+        s_row_end[tid] = T.row_end[tid];
+    }
+    if (tid == 0) {
+        int64_t b = first_block;
+        for (int t = 0; t < T.count; ++t) {
+            s_block0[t] = b;
+            b += T.n[t] / I;
+        }
+    }
+    __syncthreads();
+    const int64_t total_rows = T.row_end[T.count - 1];
+    int t_cur = 0;
+    auto fetch = [&](int64_t g, int64_t& block) -> Raw32 {  // block: this lane's block, or -1 past the end
+        block = -1;
+        if (g < total_rows) {
+            while (g >= s_row_end[t_cur]) ++t_cur;
+            const int64_t r = g - (t_cur ? s_row_end[t_cur - 1] : 0);
+            const int64_t idx = (r * 1024 + tid) * kLW;
+            if (idx < s_n[t_cur]) {
+                block = s_block0[t_cur] + idx / I;
+                if (idx & (I - 1)) block |= (int64_t)1 << 62;  // not the block's first lane
+                return load_raw32(s_ptr[t_cur], idx);
+            }
+        }
+        return zero_raw32();
+    };
+    auto row = [&](const Raw32& raw, int64_t block) {
+        uint32_t u[16];
+        words_of(raw, u);
+        float mx, mn, g;
+        lane_minmax32(u, mx, mn);
+        const float m = block_constant32<I, SIGNED>(u, mx, mn, g, &s_wide);
+        if (block >= 0 && !(block >> 62)) {
+            const uint32_t b = __float_as_uint(m) >> 16;
+            consts[block] = (uint16_t)b;
+            atomicAdd(&s_hist[b & 0x7fffu], 1u);
+        }
+    };
+    int64_t g = blockIdx.x, ba, bb;
+    const int64_t GS = gridDim.x;
+    Raw32 a = fetch(g, ba), b;
+    while (g < total_rows) {  // two row buffers used in turn
+        b = fetch(g + GS, bb);
+        row(a, ba);
+        g += GS;
+        if (g >= total_rows) break;
+        a = fetch(g + GS, ba);
+        row(b, bb);
+        g += GS;
+    }
+    __syncthreads();
+    for (int k = tid; k < kMags; k += 1024)
+        if (s_hist[k]) atomicAdd(&hist[k], s_hist[k]);
+}
+
+// ---------------------------------------------------------------- plan
+
+// One CTA, 32 magnitudes per thread: positions of the magnitudes in the ordered list, the units of work,
+// the largest magnitude and the scale of the cell sums.
+__global__ void __launch_bounds__(1024)
+cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __restrict__ head)
+{
+    __shared__ uint32_t s_blocks[32], s_units[32], s_top;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_top = W.scal[2];
+    uint32_t c[32], blocks = 0u, units = 0u, top = 0u;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const uint4 v = reinterpret_cast<const uint4*>(W.hist)[tid * 8 + q];
+        c[4 * q] = v.x, c[4 * q + 1] = v.y, c[4 * q + 2] = v.z, c[4 * q + 3] = v.w;
+    }
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        blocks += c[k];
+        if (c[k]) {
+            units += (c[k] + per_unit - 1) / per_unit;
+            top = (uint32_t)(tid * 32 + k);
+        }
+    }
+    uint32_t ib = blocks, iu = units;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t x = __shfl_up_sync(kFull, ib, off), y = __shfl_up_sync(kFull, iu, off);
+        if (lane >= off) {
+            ib += x;
+            iu += y;
+        }
+    }
+    __syncthreads();
+    if (lane == 31) {
+        s_blocks[warp] = ib;
+        s_units[warp] = iu;
+    }
+    atomicMax(&s_top, top);
+    __syncthreads();
+    for (int k = 0; k < warp; ++k) {
+        ib += s_blocks[k];
+        iu += s_units[k];
+    }
+    uint32_t at = ib - blocks, u = iu - units;
+#pragma unroll
+    for (int k = 0; k < 32; k += 4) {
+        const uint32_t a1 = c[k], a2 = a1 + c[k + 1], a3 = a2 + c[k + 2];
+        reinterpret_cast<uint4*>(W.cursor)[(tid * 32 + k) >> 2] = make_uint4(at, at + a1, at + a2, at + a3);
+        at += a3 + c[k + 3];
+    }
+    at = ib - blocks;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        const uint32_t mag = (uint32_t)(tid * 32 + k);
+        for (uint32_t done = 0; done < c[k]; done += per_unit)
+            W.units[u++] = CellUnit{mag, at + done, min(per_unit, c[k] - done)};
+        at += c[k];
+    }
+    if (tid == 1023) {
+        W.scal[0] = iu;
+        W.scal[1] = 0u;
+    }
+    if (tid == 0) {
+        W.scal[3] = s_top;
+        head[1] = s_top << 16;
+        *reinterpret_cast<double*>(head + 2) = cell_scale(s_top, metric);
+    }
+}
+
+// ---------------------------------------------------------------- order
+
+// Every CTA takes a contiguous part of the blocks: counts its magnitudes, reserves room for them in the
+// list, then writes the addresses.  The order inside a magnitude does not matter (sums of integers).
+__global__ void __launch_bounds__(1024, 1)
+cells_order_kernel(const EmTensors T, const int64_t first_block, const int64_t n_blocks, int block_size, const CellsWs W)
+{
+    extern __shared__ uint32_t s_pos[];  // [kMags]
+    __shared__ const char* s_ptr[kEmMaxTensors];
+    __shared__ int64_t s_end[kEmMaxTensors];  // first block behind the tensor
+    const int tid = threadIdx.x;
+    for (int k = tid; k < kMags; k += 1024) s_pos[k] = 0u;
+    if (tid == 0) {
+        int64_t b = first_block;
+        for (int t = 0; t < T.count; ++t) {
+            // address that block 0 would have
+            s_ptr[t] = static_cast<const char*>(T.ptr[t]) - b * block_size * 2;
+            b += T.n[t] / block_size;
+            s_end[t] = b;
+        }
+    }
+    __syncthreads();
+    const int64_t part = (n_blocks + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = first_block + (int64_t)blockIdx.x * part;
+    const int64_t hi = min(first_block + n_blocks, lo + part);
+#pragma unroll 4
+    for (int64_t i = lo + tid; i < hi; i += 1024) atomicAdd(&s_pos[W.consts[i] & 0x7fffu], 1u);
+    __syncthreads();
+    for (int k = tid; k < kMags; k += 1024)
+        if (s_pos[k]) s_pos[k] = atomicAdd(&W.cursor[k], s_pos[k]);
+    __syncthreads();
+    int t = 0;
+#pragma unroll 4
+    for (int64_t i = lo + tid; i < hi; i += 1024) {
+        while (i >= s_end[t]) ++t;
+        const uint32_t c = W.consts[i];
+        const unsigned long long p = reinterpret_cast<unsigned long long>(s_ptr[t] + i * block_size * 2);
+        W.order[atomicAdd(&s_pos[c & 0x7fffu], 1u)] = p | ((unsigned long long)(c >> 15) << 63);
+    }
+}
+
+// ---------------------------------------------------------------- accumulate
+
+__device__ __forceinline__ void cell_count(uint32_t base, uint32_t w, uint32_t mag)
+{
+    const uint32_t d = mag - (w & 0x7fffu);
+    // positive weights at distance d, negative ones kCellDepth further on; a zero (or smaller than 2^-40 of
+    // the constant) is not counted: the zeros of a unit are what is missing from its number of weights
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.lt.u32 p, %0, %2;\n\t"
+        "@p red.shared.add.u32 [%1], 1;\n\t}" ::"r"(d),
+        "r"(base + d * 4u + ((w & 0x8000u) ? (uint32_t)kCellDepth * 4u : 0u)), "n"(kCellDepth)
+        : "memory");
+}
+
+__global__ void __launch_bounds__(kCellThreads, kCellCtas)
+cells_accumulate_kernel(const CellsWs W, int lanes_shift, int metric)
+{
+    extern __shared__ uint32_t s_cnt[];  // [2 * kCellDepth]
+    __shared__ CellUnit s_unit;
+    __shared__ uint32_t s_seen[kCellThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(s_cnt);
+    const uint32_t units = W.scal[0], max_mag = W.scal[3];
+    const bool mae = metric == BOF4_METRIC_MAE || metric == BOF4_METRIC_MAE_NORMALIZED;
+    for (int k = tid; k < 2 * kCellDepth; k += kCellThreads) s_cnt[k] = 0u;
+    while (true) {
+        __syncthreads();
+        if (tid == 0) {
+            const uint32_t u = atomicAdd(&W.scal[1], 1u);
+            s_unit = (u < units) ? W.units[u] : CellUnit{0u, 0u, 0u};
+        }
+        __syncthreads();
+        const CellUnit U = s_unit;
+        if (U.count == 0u) break;
+        const unsigned long long* list = W.order + U.first;
+        const uint32_t pieces = U.count << lanes_shift, mask = (1u << lanes_shift) - 1u;  // pieces of 16 weights
+        auto load = [&](uint32_t q, uint32_t& flip) -> Raw8 {
+            const unsigned long long p = __ldg(list + (q >> lanes_shift));
+            flip = (p >> 63) ? 0x80008000u : 0u;
+            return ld_stream256(reinterpret_cast<const char*>(p & 0x7fffffffffffffffull) + (q & mask) * 32u);
+        };
+        if (U.mag == 0u) {
+            // all-zero blocks: every weight is a zero (below)
+        } else if (U.mag >= (uint32_t)kMagTiny) {
+            auto use = [&](const Raw8& r, uint32_t flip) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const uint32_t u = r.u[k] ^ flip;
+                    cell_count(base, u & 0xffffu, U.mag);
+                    cell_count(base, u >> 16, U.mag);
+                }
+            };
+            uint32_t fa, fb, q = tid;
+            Raw8 a, b;
+            if (q < pieces) a = load(q, fa);
+            while (q < pieces) {  // two buffers used in turn
+                if (q + kCellThreads < pieces) b = load(q + kCellThreads, fb);
+                use(a, fa);
+                q += kCellThreads;
+                if (q >= pieces) break;
+                if (q + kCellThreads < pieces) a = load(q + kCellThreads, fa);
+                use(b, fb);
+                q += kCellThreads;
+            }
+        } else {  // subnormal weights may occur: compare scaled bit patterns
+            const uint32_t mag = scaled16(U.mag);
+            for (uint32_t q = tid; q < pieces; q += kCellThreads) {
+                uint32_t flip;
+                const Raw8 r = load(q, flip);
+                for (int k = 0; k < 8; ++k) {
+                    const uint32_t u = r.u[k] ^ flip;
+                    cell_count(base, scaled16(u & 0xffffu), mag);
+                    cell_count(base, scaled16(u >> 16), mag);
+                }
+            }
+        }
+        __syncthreads();
+        const MagWeight m = mag_weight(U.mag, max_mag, metric);
+        const uint32_t row = (m.b - 128u) * (uint32_t)kCellRow;
+        uint32_t seen = 0u;
+        for (int k = tid; k < 2 * kCellDepth; k += kCellThreads) {
+            const uint32_t v = s_cnt[k];
+            if (v) {
+                s_cnt[k] = 0u;
+                seen += v;
+                cell_add(W, row + (uint32_t)k, v, m, mae);
+            }
+        }
+#pragma unroll
+        for (int off = 16; off; off >>= 1) seen += __shfl_xor_sync(kFull, seen, off);
+        if (lane == 0) s_seen[warp] = seen;
+        __syncthreads();
+        if (tid == 0) {
+            for (int k = 1; k < kCellThreads / 32; ++k) seen += s_seen[k];
+            const uint32_t zeros = pieces * 16u - seen;
+            // an all-zero block has weight zero, except where every sample weighs one
+            if (zeros && (U.mag != 0u || metric >= 2)) cell_add(W, row + 2 * kCellDepth, zeros, m, mae);
+        }
+    }
+}
+
+// The short last blocks: `add` = 0 takes the largest magnitude (before the plan), 1 adds their weights.
+template <bool SIGNED>
+__global__ void __launch_bounds__(kEmTailThreads)
+cells_tail_kernel(const EmTails Q, const CellsWs W, int metric, int add)
+{
+    __shared__ float s_w[4096];
+    __shared__ unsigned long long s_red[kEmTailThreads / 32];
+    const bool mae = metric == BOF4_METRIC_MAE || metric == BOF4_METRIC_MAE_NORMALIZED;
+    for (int q = 0; q < Q.count; ++q) {
+        const int len = Q.len[q];
+        const float m = load_short_block<BF16, SIGNED>(Q.ptr[q], len, s_w, s_red);
+        const uint32_t mag = (__float_as_uint(m) >> 16) & 0x7fffu;
+        if (!add) {
+            if (threadIdx.x == 0) atomicMax(&W.scal[2], mag);
+        } else if (mag != 0u || metric >= 2) {
+            const MagWeight mw = mag_weight(mag, W.scal[3], metric);
+            const bool tiny = mag < (uint32_t)kMagTiny;
+            const uint32_t ms = tiny ? scaled16(mag) : mag;
+            for (int i = threadIdx.x; i < len; i += kEmTailThreads) {
+                uint32_t w = (__float_as_uint(s_w[i]) >> 16) ^ ((__float_as_uint(m) >> 16) & 0x8000u);
+                if (tiny) w = scaled16(w);
+                const uint32_t d = ms - (w & 0x7fffu);
+                const uint32_t at = (mag == 0u || d >= (uint32_t)kCellDepth) ? 2u * kCellDepth : d + ((w & 0x8000u) ? kCellDepth : 0u);
+                cell_add(W, (mw.b - 128u) * (uint32_t)kCellRow + at, 1ull, mw, mae);
+            }
+        }
+        __syncthreads();  // before the next block overwrites s_w
+    }
+}
+
+// ---------------------------------------------------------------- items
+
+// Occupied cells per CTA of the items pass.  A cell of weight zero (|m| far below the largest) has no say.
+__global__ void __launch_bounds__(512)
+cells_scan_kernel(const CellsWs W)
+{
+    __shared__ uint32_t s_n[16];
+    const int tid = threadIdx.x;
+    uint32_t n = 0u;
+#pragma unroll
+    for (int k = 0; k < kCellScan / 512; ++k) {
+        const int c = blockIdx.x * kCellScan + k * 512 + tid;
+        if (c < kCells) {
+            const ulonglong2 v = W.acc[c];
+            n += (v.x | v.y) ? 1u : 0u;
+        }
+    }
+    n = __reduce_add_sync(kFull, n);
+    if ((tid & 31) == 0) s_n[tid >> 5] = n;
+    __syncthreads();
+    if (tid == 0) {
+        for (int k = 1; k < 16; ++k) n += s_n[k];
+        W.scans[blockIdx.x] = n;
+    }
+}
+
+// Writes the samples {x, cell} of the occupied cells in the order of the cells, and the sums of m^2 x^2 for
+// the error of the MSE metrics.
+__global__ void __launch_bounds__(512)
+cells_items_kernel(const CellsWs W)
+{
+    constexpr int PER = kCellScan / 512;
+    __shared__ uint32_t s_warp[16], s_before[16];
+    __shared__ double s_sum[16];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t before = 0u;
+    for (int k = tid; k < (int)blockIdx.x; k += 512) before += W.scans[k];
+    before = __reduce_add_sync(kFull, before);
+    if (lane == 0) s_before[warp] = before;
+    const double scale = *reinterpret_cast<const double*>(W.sort.n_items + 2);
+    const int c0 = blockIdx.x * kCellScan + tid * PER;
+    ulonglong2 v[PER];
+    uint32_t mine = 0u;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        v[k] = (c0 + k < kCells) ? W.acc[c0 + k] : make_ulonglong2(0ull, 0ull);
+        mine += (v[k].x | v[k].y) ? 1u : 0u;
+    }
+    uint32_t incl = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl, off);
+        if (lane >= off) incl += t;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    before = 0u;
+    for (int k = 0; k < 16; ++k) before += s_before[k] + (k < warp ? s_warp[k] : 0u);
+    uint32_t at = before + incl - mine;
+    double sum = 0.0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (!(v[k].x | v[k].y)) continue;
+        const uint32_t cell = (uint32_t)(c0 + k), b = cell / kCellRow, r = cell % kCellRow;
+        float x = 0.0f;
+        if (r < 2u * kCellDepth) {
+            const bool neg = r >= (uint32_t)kCellDepth;
+            const uint32_t mb = 0x3f80u + b, wb = mb - (neg ? r - kCellDepth : r);
+            const float m = __uint_as_float(mb << 16), w = __uint_as_float(wb << 16);
+            x = __fdiv_rn(neg ? -w : w, m);
+            const double e = (double)x;
+            sum += ((double)v[k].y * 18446744073709551616.0 + (double)v[k].x) * scale * e * e;
+        }
+        W.sort.a[at++] = make_float2(x, __uint_as_float(cell));
+    }
+#pragma unroll
+    for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+    if (lane == 0) s_sum[warp] = sum;
+    __syncthreads();
+    if (tid == 0) {
+        for (int k = 1; k < 16; ++k) sum += s_sum[k];
+        reinterpret_cast<double*>(W.sort.counts)[blockIdx.x] = sum;  // folded by the next kernel
+        if (blockIdx.x == gridDim.x - 1) {
+            uint32_t n = before;  // of all earlier CTAs (warp 0 has added nothing of its own CTA)
+            for (int k = 0; k < 16; ++k) n += s_warp[k];
+            W.sort.n_items[0] = n;
+        }
+    }
+}
+
+// The CTAs' sums of squares into the slots that the iterations add up.
+__global__ void __launch_bounds__(320)
+cells_square_kernel(const CellsWs W)
+{
+    const double* part = reinterpret_cast<const double*>(W.sort.counts);
+    for (int k = threadIdx.x; k < kSortParts; k += blockDim.x) {
+        double a = 0.0;
+        for (int c = k; c < kCellScans; c += kSortParts) a += part[c];
+        W.sort.w2[k] = a;
+    }
+}
+static_assert((size_t)kCellScans * 8 <= (size_t)kSortGrid * 256 * 4, "partial sums fit the ordering passes' counters");
+
+// ---------------------------------------------------------------- host side
+
+namespace {
+
+template <bool SG>
+int blocks_pass(const EmTensors& T, int block_size, int64_t first, const CellsWs& W, cudaStream_t st)
+{
+    constexpr int smem = kMags * 4;
+#define BOF4_CELLS_I(I_)                                                                  \
+    case I_: {                                                                            \
+        constexpr auto kern = cells_blocks_kernel<I_, SG>;                                \
+        if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;                    \
+        kern<<<kSMs, 1024, smem, st>>>(T, first, W.hist, W.consts);                       \
+        break;                                                                            \
+    }
+    switch (block_size) {
+        BOF4_CELLS_I(32) BOF4_CELLS_I(64) BOF4_CELLS_I(128) BOF4_CELLS_I(256) BOF4_CELLS_I(512) BOF4_CELLS_I(1024)
+        BOF4_CELLS_I(2048) BOF4_CELLS_I(4096)
+    }
+#undef BOF4_CELLS_I
+    BOF4_CUDA_TRY(cudaGetLastError());
+    return BOF4_OK;
+}
+
+}  // namespace
+
+int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters, double* d_err_log, void* d_ws,
+              size_t ws_bytes, cudaStream_t st, bool* done)
+{
+    *done = false;
+    if (!cells_apply(a.w_dtype, a.n_total) || iters < kSortMinIters) return BOF4_OK;
+    CellsWs W;
+    if (cells_layout(d_ws, a.n_total, a.block_size, &W) > ws_bytes) return BOF4_OK;
+    *done = true;
+    int64_t blocks = 0;
+    for (int t = 0; t < a.n_tensors; ++t) blocks += a.h_n[t] / a.block_size;
+    const bool sg = a.norm == BOF4_NORM_SIGNED;
+    BOF4_CUDA_TRY(cudaMemsetAsync(W.hist, 0, reinterpret_cast<char*>(W.cursor) - reinterpret_cast<char*>(W.hist), st));
+    auto tails = [&](int add) {
+        return for_each_tail_chunk(a, [&](const EmTails& Q) -> int {
+            if (sg) cells_tail_kernel<true><<<1, kEmTailThreads, 0, st>>>(Q, W, a.metric, add);
+            else cells_tail_kernel<false><<<1, kEmTailThreads, 0, st>>>(Q, W, a.metric, add);
+            BOF4_CUDA_TRY(cudaGetLastError());
+            return BOF4_OK;
+        });
+    };
+    auto of = [&](const EmTensors& T) {
+        int64_t b = 0;
+        for (int t = 0; t < T.count; ++t) b += T.n[t] / a.block_size;
+        return b;
+    };
+    int rc = tails(0), calls = 0;
+    if (rc) return rc;
+    int64_t first = 0;
+    rc = for_each_tensor_chunk(a, 1024 * kLW, [&](const EmTensors& T) -> int {
+        const int64_t f = first;
+        first += of(T);
+        return sg ? blocks_pass<true>(T, a.block_size, f, W, st) : blocks_pass<false>(T, a.block_size, f, W, st);
+    }, &calls);
+    if (rc) return rc;
+    cells_plan_kernel<<<1, 1024, 0, st>>>(W, (uint32_t)unit_blocks(blocks, a.block_size), a.metric, W.sort.n_items);
+    BOF4_CUDA_TRY(cudaGetLastError());
+    first = 0;
+    rc = for_each_tensor_chunk(a, 1024 * kLW, [&](const EmTensors& T) -> int {
+        const int64_t f = first, nb = of(T);
+        first += nb;
+        if (const int e = ensure_dynamic_smem<cells_order_kernel>(kMags * 4)) return e;
+        cells_order_kernel<<<kSMs, 1024, kMags * 4, st>>>(T, f, nb, a.block_size, W);
+        BOF4_CUDA_TRY(cudaGetLastError());
+        return BOF4_OK;
+    }, &calls);
+    if (rc) return rc;
+    int shift = 0;
+    while ((16 << shift) < a.block_size) ++shift;
+    constexpr int smem = 2 * kCellDepth * 4;
+    if ((rc = ensure_dynamic_smem<cells_accumulate_kernel>(smem))) return rc;
+    cells_accumulate_kernel<<<kCellCtas * kSMs, kCellThreads, smem, st>>>(W, shift, a.metric);
+    BOF4_CUDA_TRY(cudaGetLastError());
+    if ((rc = tails(1))) return rc;
+    cells_scan_kernel<<<kCellScans, 512, 0, st>>>(W);
+    cells_items_kernel<<<kCellScans, 512, 0, st>>>(W);
+    cells_square_kernel<<<1, 320, 0, st>>>(W);
+    BOF4_CUDA_TRY(cudaGetLastError());
+    SortFit F{};
+    F.acc = reinterpret_cast<const unsigned long long*>(W.acc);
+    F.acc_a = W.acc_a;
+    F.metric = a.metric;
+    F.n_total = a.n_total;
+    F.n_max = kCells;
+    F.codebook = d_codebook;
+    F.fixed_mask = fixed_mask;
+    F.iters = iters;
+    F.err_log = d_err_log;
+    return sorted_run(W.sort, F, st);
+}
+
+}  // namespace bof4

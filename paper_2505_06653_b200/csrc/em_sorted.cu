@@ -1,0 +1,779 @@
+// Codebook fit over ordered samples (see em_sorted.cuh): one sample per weight, the ordering passes,
+// the sums per bin and the iterations.
+//
+// Launches of a fit, whatever its number of iterations: samples (one per 64 tensors), two ordering
+// passes of eight bits (count and scatter each, least significant digit first, stable), first sample of
+// every bin, sums of the bins in two steps, iterations.  Nothing depends on the order in which CTAs run:
+// the samples' order, the order of every sum and hence the result are reproducible.
+#include "em_sorted.cuh"
+
+namespace bof4 {
+
+constexpr int kSortThreads = 1024;
+constexpr int kSortPerThread = 8;
+constexpr int kSortTile = kSortThreads * kSortPerThread;
+
+size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W)
+{
+    char* p = static_cast<char*>(base);
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* q = p ? p + off : nullptr;
+        off += align_up(bytes, 256);
+        return q;
+    };
+    const size_t chunks = (size_t)((n + kSortChunk - 1) / kSortChunk) + 1;
+    SortWs L;
+    L.n_items = reinterpret_cast<uint32_t*>(take(256));
+    L.w2 = reinterpret_cast<double*>(take(kSortParts * 8));
+    L.counts = reinterpret_cast<uint32_t*>(take((size_t)kSortGrid * 256 * 4));
+    L.start = reinterpret_cast<uint32_t*>(take((size_t)(kSortBins + 1) * 4));
+    L.bin = reinterpret_cast<SortSums*>(take((size_t)kSortBins * sizeof(SortSums)));
+    L.group = reinterpret_cast<SortSums*>(take((size_t)kSortGroups * sizeof(SortSums)));
+    L.lead = reinterpret_cast<SortSums*>(take(chunks * sizeof(SortSums)));
+    L.trail = reinterpret_cast<SortSums*>(take(chunks * sizeof(SortSums)));
+    L.a = reinterpret_cast<float2*>(take((size_t)n * 8));
+    L.b = reinterpret_cast<float2*>(take((size_t)n * 8));
+    L.cell_s = cells ? reinterpret_cast<double*>(take((size_t)n * 8)) : nullptr;
+    L.cell_a = cells ? reinterpret_cast<unsigned long long*>(take((size_t)n * 8)) : nullptr;
+    if (W) *W = L;
+    return off;
+}
+
+// ---------------------------------------------------------------- samples, one per weight
+
+// Every lane owns 16 consecutive weights; x = RN(w / m) and |m| (1 for the normalised-domain metrics) go
+// to the sample array in the order of the weights.  Bound by its stores (8 bytes per weight).
+template <class DT, int I, bool SIGNED>
+__global__ void __launch_bounds__(512, 2)
+sort_samples_kernel(const EmTensors T, const uint32_t first, float2* __restrict__ items, uint32_t* __restrict__ head,
+                    double* __restrict__ w2)
+{
+    constexpr int NT = 512;
+    __shared__ WideScratch s_wide;
+    __shared__ uint32_t s_item0[kEmMaxTensors];
+    __shared__ double s_sum[NT / 32];
+    __shared__ uint32_t s_max[NT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        uint32_t at = first;
+        for (int t = 0; t < T.count; ++t) {
+            s_item0[t] = at;
+            at += (uint32_t)T.n[t];
+        }
+    }
+    __syncthreads();
+    const int64_t total_rows = T.row_end[T.count - 1];
+    const bool unit = T.unit != 0;
+    double sum = 0.0;
+    float top = 0.0f;
+    int t = 0;
+    for (int64_t g = blockIdx.x; g < total_rows; g += gridDim.x) {
+        while (g >= T.row_end[t]) ++t;
+        const int64_t r = g - (t ? T.row_end[t - 1] : 0);
+        const int64_t idx = (r * NT + tid) * kLaneW;
+        const bool ok = idx < T.n[t];
+        float v[kLaneW], x[kLaneW], gmax;
+        widen(ok ? load_raw<DT>(T.ptr[t], idx) : zero_raw<DT>(), v);
+        const float m = block_constant<I, SIGNED>(v, gmax, &s_wide);
+        const bool safe = row_is_safe(gmax, ok);
+        normalise16<true>(v, m, safe && DT::code == BF16::code, x);
+        if (!ok) continue;
+        top = fmaxf(top, gmax);
+        const float am = unit ? 1.0f : fabsf(m);
+#pragma unroll
+        for (int k = 0; k < kLaneW; ++k) {  // (m x)^2: with the x of the other sums the error is free of cancellation
+            const double e = (double)x[k] * (double)am;
+            sum = fma(e, e, sum);
+        }
+        float4* dst = reinterpret_cast<float4*>(items + s_item0[t] + idx);
+#pragma unroll
+        for (int k = 0; k < kLaneW; k += 2) dst[k >> 1] = make_float4(x[k], am, x[k + 1], am);
+    }
+    uint32_t bits = __float_as_uint(top);
+#pragma unroll
+    for (int off = 16; off; off >>= 1) {
+        sum += __shfl_xor_sync(kFull, sum, off);
+        bits = max(bits, __shfl_xor_sync(kFull, bits, off));
+    }
+    if (lane == 0) {
+        s_sum[warp] = sum;
+        s_max[warp] = bits;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double a = 0.0;
+        for (int k = 0; k < NT / 32; ++k) {
+            a += s_sum[k];
+            bits = max(bits, s_max[k]);
+        }
+        w2[blockIdx.x] = T.accumulate ? w2[blockIdx.x] + a : a;
+        atomicMax(head + 1, bits);  // non-negative floats order like their bits
+    }
+}
+
+// The short last blocks, after all whole blocks in the sample array: one CTA.
+template <class DT, bool SIGNED>
+__global__ void __launch_bounds__(kEmTailThreads)
+sort_tail_kernel(const EmTails Q, uint32_t at, float2* __restrict__ items, uint32_t* __restrict__ head,
+                 double* __restrict__ w2)
+{
+    __shared__ float s_w[4096];
+    __shared__ unsigned long long s_red[kEmTailThreads / 32];
+    __shared__ double s_sum[kEmTailThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double sum = 0.0;
+    for (int q = 0; q < Q.count; ++q) {
+        const int len = Q.len[q];
+        const float m = load_short_block<DT, SIGNED>(Q.ptr[q], len, s_w, s_red);
+        for (int i = tid; i < len; i += kEmTailThreads) {
+            const float x = normalise(s_w[i], m), am = Q.unit ? 1.0f : fabsf(m);
+            const double e = (double)x * (double)am;
+            sum = fma(e, e, sum);
+            items[at + i] = make_float2(x, am);
+        }
+        at += (uint32_t)len;
+        if (tid == 0) atomicMax(head + 1, __float_as_uint(fabsf(m)));
+        __syncthreads();  // before the next block overwrites s_w
+    }
+#pragma unroll
+    for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+    if (lane == 0) s_sum[warp] = sum;
+    __syncthreads();
+    if (tid == 0) {
+        double a = 0.0;
+        for (int k = 0; k < kEmTailThreads / 32; ++k) a += s_sum[k];
+        w2[kSortParts - 1] = Q.accumulate ? w2[kSortParts - 1] + a : a;
+    }
+}
+
+__global__ void sort_head_kernel(uint32_t* head, uint32_t n, double* w2)
+{
+    if (threadIdx.x == 0) {
+        head[0] = n;
+        head[1] = 0u;
+    }
+    for (int k = threadIdx.x; k < kSortParts; k += blockDim.x) w2[k] = 0.0;
+}
+
+// ---------------------------------------------------------------- ordering passes
+
+// Samples [lo, hi) of CTA c.
+__device__ __forceinline__ void sort_part(uint32_t n, uint32_t c, uint32_t& lo, uint32_t& hi)
+{
+    const uint32_t len = (n + kSortGrid - 1) / kSortGrid;
+    lo = min(n, c * len);
+    hi = min(n, lo + len);
+}
+
+template <int SHIFT>
+__global__ void __launch_bounds__(kSortThreads)
+sort_count_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ head, uint32_t* __restrict__ counts)
+{
+    __shared__ uint32_t s_hist[4][256];  // a copy per eight warps: fewer collisions on crowded digits
+    const int tid = threadIdx.x;
+    (&s_hist[0][0])[tid] = 0u;
+    __syncthreads();
+    uint32_t lo, hi;
+    sort_part(*head, blockIdx.x, lo, hi);
+    for (uint32_t i = lo + tid; i < hi; i += kSortThreads)
+        atomicAdd(&s_hist[tid >> 8][(sort_bin(in[i].x) >> SHIFT) & 255], 1u);
+    __syncthreads();
+    if (tid < 256) counts[blockIdx.x * 256 + tid] = s_hist[0][tid] + s_hist[1][tid] + s_hist[2][tid] + s_hist[3][tid];
+}
+
+// Stable scatter by one digit.  A sample goes to: samples with a smaller digit + samples of the same
+// digit in earlier CTAs + in earlier tiles of this CTA + in earlier warps of the tile + earlier in the
+// warp (each warp owns 256 consecutive samples of a tile, 32 at a time).
+template <int SHIFT>
+__global__ void __launch_bounds__(kSortThreads)
+sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ head, const uint32_t* __restrict__ counts,
+                    float2* __restrict__ out)
+{
+    __shared__ uint32_t s_cnt[32][256];
+    __shared__ uint32_t s_base[256], s_warp[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t lo, hi;
+    sort_part(*head, blockIdx.x, lo, hi);
+    {
+        const int seg = tid >> 8, d = tid & 255;
+        uint32_t before = 0u, all = 0u;
+#pragma unroll
+        for (int k = 0; k < (kSortGrid + 3) / 4; ++k) {  // all loads at once: one round trip to L2
+            const int c = seg + 4 * k;
+            const uint32_t v = c < kSortGrid ? __ldcg(counts + c * 256 + d) : 0u;
+            all += v;
+            before += (c < (int)blockIdx.x) ? v : 0u;
+        }
+        s_cnt[seg][d] = before;
+        s_cnt[4 + seg][d] = all;
+        __syncthreads();
+        uint32_t mine = 0u, incl = 0u;
+        if (tid < 256) {
+            mine = s_cnt[4][tid] + s_cnt[5][tid] + s_cnt[6][tid] + s_cnt[7][tid];
+            incl = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, incl, off);
+                if (lane >= off) incl += t;
+            }
+            if (lane == 31) s_warp[warp] = incl;
+        }
+        __syncthreads();
+        if (tid < 256) {
+            for (int k = 0; k < warp; ++k) incl += s_warp[k];
+            s_base[tid] = incl - mine + s_cnt[0][tid] + s_cnt[1][tid] + s_cnt[2][tid] + s_cnt[3][tid];
+        }
+        __syncthreads();
+    }
+    for (uint32_t t0 = lo; t0 < hi; t0 += kSortTile) {
+        float2 item[kSortPerThread];
+        uint32_t rank[kSortPerThread];
+        const uint32_t i0 = t0 + warp * (32 * kSortPerThread) + lane;
+#pragma unroll
+        for (int k = 0; k < kSortPerThread; ++k) {
+            const uint32_t i = i0 + 32 * k;
+            item[k] = (i < hi) ? in[i] : make_float2(0.0f, 0.0f);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s_cnt[warp][lane + 32 * k] = 0u;
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < kSortPerThread; ++k) {
+            const bool ok = i0 + 32 * k < hi;
+            const uint32_t d = ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u;
+            unsigned peers = __ballot_sync(kFull, ok);
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const unsigned with = __ballot_sync(kFull, (d >> b) & 1u);
+                peers &= ((d >> b) & 1u) ? with : ~with;
+            }
+            const uint32_t old = s_cnt[warp][d];
+            __syncwarp();
+            if (ok && lane == __ffs(peers) - 1) s_cnt[warp][d] = old + __popc(peers);
+            __syncwarp();
+            rank[k] = old + __popc(peers & ((1u << lane) - 1u));
+        }
+        __syncthreads();
+        if (tid < 256) {
+            uint32_t c[32], run = s_base[tid];
+#pragma unroll
+            for (int w = 0; w < 32; ++w) c[w] = s_cnt[w][tid];
+#pragma unroll
+            for (int w = 0; w < 32; ++w) {
+                s_cnt[w][tid] = run;
+                run += c[w];
+            }
+            s_base[tid] = run;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kSortPerThread; ++k) {
+            const uint32_t d = ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u;
+            if (i0 + 32 * k < hi) out[s_cnt[warp][d] + rank[k]] = item[k];
+        }
+        __syncthreads();  // s_cnt is cleared for the next tile
+    }
+}
+
+// ---------------------------------------------------------------- sums of the bins
+
+// What a sample contributes.
+template <bool MAE, bool CELLS>
+struct SampleWeight {
+    uint32_t max_bits;
+    bool unit;
+    double scale;                    // CELLS: undoes the fixed-point scale of the weights
+    const ulonglong2* acc;           // CELLS, by cell
+    const unsigned long long* acc_a;
+    // A direct sample's payload is its |m|; a cell's is its number.
+    __device__ __forceinline__ void operator()(float2 it, double& s, unsigned long long& a) const
+    {
+        a = 0ull;
+        if (CELLS) {
+            const uint32_t cell = __float_as_uint(it.y);
+            const ulonglong2 v = acc[cell];
+            s = ((double)v.y * 18446744073709551616.0 + (double)v.x) * scale;
+            if (MAE) a = acc_a[cell];
+        } else {
+            const double m = (double)it.y;
+            s = MAE ? m : m * m;
+            if (MAE) a = unit ? 1ull : (unsigned long long)sort_fixed_weight(it.y, max_bits);
+        }
+    }
+};
+
+__global__ void __launch_bounds__(256)
+sort_start_kernel(const float2* __restrict__ items, const uint32_t* __restrict__ head, uint32_t* __restrict__ start)
+{
+    const uint32_t n = *head;
+    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+        const int b = sort_bin(items[i].x), prev = i ? sort_bin(items[i - 1].x) : -1;
+        for (int t = prev + 1; t <= b; ++t) start[t] = i;
+        if (i == n - 1)
+            for (int t = b + 1; t <= kSortBins; ++t) start[t] = n;
+    }
+}
+
+template <bool MAE>
+__device__ __forceinline__ void sums_reduce(SortSums& t)
+{
+#pragma unroll
+    for (int off = 16; off; off >>= 1) {
+        t.s += __shfl_xor_sync(kFull, t.s, off);
+        t.sx += __shfl_xor_sync(kFull, t.sx, off);
+        if (MAE) t.a += __shfl_xor_sync(kFull, t.a, off);
+    }
+}
+__device__ __forceinline__ void sums_add(SortSums& t, const SortSums& v)
+{
+    t.s += v.s;
+    t.sx += v.sx;
+    t.a += v.a;
+}
+
+// One warp per kSortChunk ordered samples, 32 at a time: a segmented scan over the runs of equal bins.
+// A run that lies inside the chunk is a bin's sum; parts of runs that cross the chunk's edges go to
+// lead / trail and are put together by sort_group_kernel.  The work is even whatever the distribution (the bins
+// of x = +-1 hold 1 / I of the data; a bin of small data is mostly empty).
+template <bool MAE, bool CELLS>
+__global__ void __launch_bounds__(256)
+sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
+{
+    constexpr int STEPS = kSortChunk / 32, kNone = 1 << 20;
+    const uint32_t n = W.n_items[0];
+    weight.max_bits = W.n_items[1];
+    if (CELLS) weight.scale = *reinterpret_cast<const double*>(W.n_items + 2);
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = gridDim.x * 8u;
+    for (uint32_t c = blockIdx.x * 8u + (threadIdx.x >> 5); (uint64_t)c * kSortChunk < n; c += warps) {
+        const uint32_t lo = c * kSortChunk, hi = min(n, lo + kSortChunk);
+        float2 it[STEPS];
+        SortSums v[STEPS];
+        int key[STEPS];
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) {
+            const uint32_t i = lo + 32 * k + lane;
+            it[k] = (i < hi) ? W.b[i] : make_float2(0.0f, 0.0f);
+        }
+        const int before = lo ? sort_bin(W.b[lo - 1].x) : -1, behind = (hi < n) ? sort_bin(W.b[hi].x) : kNone;
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) {
+            const uint32_t i = lo + 32 * k + lane;
+            v[k] = SortSums{0.0, 0.0, 0ull};
+            key[k] = kNone;
+            if (i < hi) {
+                key[k] = sort_bin(it[k].x);
+                weight(it[k], v[k].s, v[k].a);
+                v[k].sx = v[k].s * (double)it[k].x;
+            }
+        }
+        if (CELLS) {
+#pragma unroll
+            for (int k = 0; k < STEPS; ++k) {
+                const uint32_t i = lo + 32 * k + lane;
+                if (i < hi) {
+                    W.cell_s[i] = v[k].s;
+                    if (MAE) W.cell_a[i] = v[k].a;
+                }
+            }
+        }
+        SortSums open{0.0, 0.0, 0ull};  // the run that reaches the end of the steps so far (the same in all lanes)
+        int open_key = before;
+        bool early = true;              // it began before this chunk
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) {
+            int left = __shfl_up_sync(kFull, key[k], 1);
+            if (lane == 0) left = open_key;
+            const unsigned heads = __ballot_sync(kFull, key[k] != left);
+            if ((heads & 1u) && k > 0 && lane == 0 && open_key != kNone) (early ? W.lead[c] : W.bin[open_key]) = open;
+            const unsigned upto = heads & ((2u << lane) - 1u);
+            const int from = upto ? 31 - __clz(upto) : 0;
+            SortSums t = v[k];
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const double s = __shfl_up_sync(kFull, t.s, off), sx = __shfl_up_sync(kFull, t.sx, off);
+                const unsigned long long a = MAE ? __shfl_up_sync(kFull, t.a, off) : 0ull;
+                if (lane >= from + off) {
+                    t.s += s;
+                    t.sx += sx;
+                    t.a += a;
+                }
+            }
+            if (!upto) sums_add(t, open);
+            if (lane < 31 && ((heads >> (lane + 1)) & 1u) && key[k] != kNone) ((early && !upto) ? W.lead[c] : W.bin[key[k]]) = t;
+            open.s = __shfl_sync(kFull, t.s, 31);
+            open.sx = __shfl_sync(kFull, t.sx, 31);
+            if (MAE) open.a = __shfl_sync(kFull, t.a, 31);
+            open_key = __shfl_sync(kFull, key[k], 31);
+            early = early && heads == 0u;
+        }
+        if (lane == 0 && open_key != kNone) (early ? W.lead[c] : open_key == behind ? W.trail[c] : W.bin[open_key]) = open;
+    }
+}
+
+// One warp per group of 32 bins: empty bins are cleared, bins that cross chunks put together (in the
+// order of the chunks), and the group's sums formed.
+template <bool MAE>
+__global__ void __launch_bounds__(256)
+sort_group_kernel(const SortWs W)
+{
+    const int lane = threadIdx.x & 31, g = blockIdx.x * 8 + (threadIdx.x >> 5), b = g * kSortGroup + lane;
+    const uint32_t s = W.start[b], e = W.start[b + 1];
+    SortSums t{0.0, 0.0, 0ull};
+    const uint32_t c0 = s / kSortChunk, c1 = (e > s) ? (e - 1) / kSortChunk : c0;
+    if (e > s && c0 == c1) t = W.bin[b];
+    unsigned spans = __ballot_sync(kFull, e > s && c0 != c1);
+    while (spans) {
+        const int who = __ffs(spans) - 1;
+        spans &= spans - 1u;
+        const uint32_t f = __shfl_sync(kFull, c0, who), l = __shfl_sync(kFull, c1, who);
+        SortSums u{0.0, 0.0, 0ull};
+#pragma unroll 4
+        for (uint32_t c = f + lane; c <= l; c += 32) sums_add(u, (c == f) ? W.trail[c] : W.lead[c]);
+        __syncwarp();
+        sums_reduce<MAE>(u);
+        if (lane == who) t = u;
+    }
+    W.bin[b] = t;
+    sums_reduce<MAE>(t);
+    if (lane == 0) W.group[g] = t;
+}
+
+// ---------------------------------------------------------------- all iterations
+//
+// One CTA.  Warp 2 l + h owns half h of region l: the samples from the region's lower threshold to its
+// level (h = 0) or from the level to the upper threshold (h = 1); the split is what the MAE error needs.
+// An iteration is a chain of latencies (thresholds -> first samples of the two cut bins -> those samples
+// -> butterfly -> level update), so everything that does not depend on one another is requested
+// together; the cut bins are mostly those of the iteration before and come from L1.  When an iteration
+// leaves every level unchanged the remaining ones would repeat it bit for bit: their entries of the
+// error log are filled in and the loop ends.
+template <bool MAE, bool CELLS>
+__global__ void __launch_bounds__(1024, 1)
+sort_fit_kernel(const SortWs W, const SortFit F)
+{
+    extern __shared__ __align__(16) SortSums s_group[];
+    __shared__ float s_level[2][kLevels], s_med[kLevels];
+    __shared__ SortSums s_half[32];
+    __shared__ int s_stop;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    SampleWeight<MAE, false> weight;
+    weight.max_bits = W.n_items[1];
+    weight.unit = F.metric >= 2;
+    for (int k = tid; k < kSortGroups; k += 1024) s_group[k] = W.group[k];
+    if (tid < kLevels) s_level[0][tid] = F.codebook[tid];
+    double w2 = 0.0;
+    if (warp == 1) {  // the warp that works out the errors
+        for (int k = lane; k < kSortParts; k += 32) w2 += W.w2[k];
+#pragma unroll
+        for (int off = 16; off; off >>= 1) w2 += __shfl_xor_sync(kFull, w2, off);
+    }
+    if (tid == 0) s_stop = 0;
+    __syncthreads();
+    const int l = warp >> 1, h = warp & 1;
+    const float inf = __int_as_float(0x7f800000);
+    auto use = [&](uint32_t i, float2 it, double& s, unsigned long long& a) {
+        if (CELLS) {
+            s = __ldg(W.cell_s + i);
+            a = MAE ? __ldg(W.cell_a + i) : 0ull;
+        } else {
+            weight(it, s, a);
+        }
+    };
+    auto bin_sums = [&](int b) {
+        SortSums v;
+        v.s = __ldg(&W.bin[b].s);
+        v.sx = __ldg(&W.bin[b].sx);
+        v.a = MAE ? __ldg(&W.bin[b].a) : 0ull;
+        return v;
+    };
+    int now = 0;
+    for (int iter = 0; iter < F.iters; ++iter, now ^= 1) {
+        const float* s_lv = s_level[now];
+        const float lv = s_lv[l];
+        const float lo = l ? __fmul_rn(__fadd_rn(s_lv[l - 1], lv), 0.5f) : -inf;
+        const float hi = l < kLevels - 1 ? __fmul_rn(__fadd_rn(lv, s_lv[l + 1]), 0.5f) : inf;
+        const float mid = fminf(fmaxf(lv, lo), hi);
+        const float p = h ? mid : lo, q = h ? hi : mid;  // this warp: samples with p <= x < q
+        const int bp = (p == -inf) ? -1 : sort_bin(p), bq = (q == inf) ? kSortBins : sort_bin(q);
+        // bins strictly inside, as whole groups with up to 31 single bins on either side
+        const int b0 = bp + 1, b1 = max(bq, b0);
+        const int g0 = (b0 + kSortGroup - 1) / kSortGroup, g1 = b1 / kSortGroup;
+        const int head_end = min(b1, g0 * kSortGroup), tail0 = (g1 >= g0) ? g1 * kSortGroup : b1;
+        const bool cut_p = bp >= 0, cut_q = bq < kSortBins && bq != bp;
+        const bool one_p = one_value_bin(bp), one_q = one_value_bin(bq);
+        SortSums t{0.0, 0.0, 0ull};
+        // the cut bins' samples: the first 32 of both are on their way before anything is added up
+        uint32_t sp = 0u, ep = 0u, sq = 0u, eq = 0u;
+        if (cut_p && !one_p) sp = __ldg(W.start + bp) + lane, ep = __ldg(W.start + bp + 1);
+        if (cut_q && !one_q) sq = __ldg(W.start + bq) + lane, eq = __ldg(W.start + bq + 1);
+        const bool in_p = sp < ep, in_q = sq < eq;
+        float2 ip = make_float2(0.0f, 0.0f), iq = ip;
+        if (in_p) ip = __ldg(W.b + sp);
+        if (in_q) iq = __ldg(W.b + sq);
+        auto take = [&](uint32_t i, float2 it) {
+            if (!(it.x >= p && it.x < q)) return;
+            double s;
+            unsigned long long a;
+            use(i, it, s, a);
+            t.s += s;
+            t.sx += s * (double)it.x;
+            t.a += a;
+        };
+        if (b0 + lane < head_end) sums_add(t, bin_sums(b0 + lane));
+        if (tail0 + lane < b1) sums_add(t, bin_sums(tail0 + lane));
+        for (int g = g0 + lane; g < g1; g += 32) sums_add(t, s_group[g]);
+        if (lane == 0) {  // bins of one value are in or out as a whole
+            if (cut_p && one_p && value_of_bin(bp) >= p && value_of_bin(bp) < q) sums_add(t, bin_sums(bp));
+            if (cut_q && one_q && value_of_bin(bq) >= p && value_of_bin(bq) < q) sums_add(t, bin_sums(bq));
+        }
+        if (in_p) {
+            take(sp, ip);
+            for (uint32_t i = sp + 32; i < ep; i += 32) take(i, __ldg(W.b + i));
+        }
+        if (in_q) {
+            take(sq, iq);
+            for (uint32_t i = sq + 32; i < eq; i += 32) take(i, __ldg(W.b + i));
+        }
+        __syncwarp();
+        sums_reduce<MAE>(t);
+        if (lane == 0) s_half[warp] = t;
+        __syncthreads();
+        if (MAE) {
+            // The warp whose half holds the crossing of half the region's weight finds the sample.
+            const unsigned long long below = s_half[2 * l].a, total = below + s_half[2 * l + 1].a;
+            const bool in_lower = 2ull * below >= total;
+            if (total > 0ull && in_lower == (h == 0) && !((F.fixed_mask >> l) & 1u)) {
+                unsigned long long before = h ? below : 0ull;
+                // the samples of bin b inside [p, q): smallest key with 2 (before + weight up to it) >= total;
+                // false (and `before` advanced) if the crossing lies behind them
+                auto pick = [&](int b) -> bool {
+                    if (one_value_bin(b)) {
+                        const float x = value_of_bin(b);
+                        const unsigned long long a = (x >= p && x < q) ? bin_sums(b).a : 0ull;
+                        if (a == 0ull || 2ull * (before + a) < total) {
+                            before += a;
+                            return false;
+                        }
+                        if (lane == 0) s_med[l] = x;
+                        return true;
+                    }
+                    constexpr int R = 4;
+                    const uint32_t s0 = __ldg(W.start + b), e = __ldg(W.start + b + 1);
+                    uint32_t key[R], kmin = 0xffffffffu, kmax = 0u;
+                    unsigned long long wt[R], sum = 0ull;
+                    auto get = [&](uint32_t i, uint32_t& k, unsigned long long& a) {
+                        k = 0xffffffffu;
+                        a = 0ull;
+                        if (i < e) {
+                            const float2 it = __ldg(W.b + i);
+                            double s;
+                            if (it.x >= p && it.x < q) {
+                                use(i, it, s, a);
+                                k = sort_key(it.x);
+                            }
+                        }
+                    };
+#pragma unroll
+                    for (int r = 0; r < R; ++r) get(s0 + 32 * r + lane, key[r], wt[r]);
+                    auto each = [&](auto fn) {
+#pragma unroll
+                        for (int r = 0; r < R; ++r) fn(key[r], wt[r]);
+                        for (uint32_t i = s0 + 32 * R + lane; i < e; i += 32) {
+                            uint32_t k;
+                            unsigned long long a;
+                            get(i, k, a);
+                            fn(k, a);
+                        }
+                        __syncwarp();
+                    };
+                    each([&](uint32_t k, unsigned long long a) {
+                        if (k != 0xffffffffu) {
+                            kmin = min(kmin, k);
+                            kmax = max(kmax, k);
+                        }
+                        sum += a;
+                    });
+#pragma unroll
+                    for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+                    if (2ull * (before + sum) < total || sum == 0ull) {
+                        before += sum;
+                        return false;
+                    }
+                    uint32_t k0 = __reduce_min_sync(kFull, kmin), k1 = __reduce_max_sync(kFull, kmax);
+                    while (k0 < k1) {
+                        const uint32_t km = k0 + ((k1 - k0) >> 1);
+                        sum = 0ull;
+                        each([&](uint32_t k, unsigned long long a) { sum += (k <= km) ? a : 0ull; });
+#pragma unroll
+                        for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+                        if (2ull * (before + sum) >= total) k1 = km;
+                        else k0 = km + 1u;
+                    }
+                    if (lane == 0) s_med[l] = sort_key_value(k0);
+                    return true;
+                };
+                // 32 entries, this lane's `mine`: the first that reaches half, or -1; `before` advanced past those in front
+                auto first_of = [&](unsigned long long mine) -> int {
+                    unsigned long long incl = mine;
+#pragma unroll
+                    for (int off = 1; off < 32; off <<= 1) {
+                        const unsigned long long v = __shfl_up_sync(kFull, incl, off);
+                        if (lane >= off) incl += v;
+                    }
+                    const unsigned hit = __ballot_sync(kFull, 2ull * (before + incl) >= total && mine > 0ull);
+                    const int at = __ffs(hit) - 1;
+                    const unsigned long long upto = __shfl_sync(kFull, incl, at < 0 ? 31 : at);
+                    before += (at < 0) ? upto : upto - __shfl_sync(kFull, mine, at);
+                    return at;
+                };
+                auto bins = [&](int from, int to) -> bool {  // at most 32 whole bins
+                    const int at = first_of((from + lane < to) ? bin_sums(from + lane).a : 0ull);
+                    return at >= 0 && pick(from + at);
+                };
+                bool found = cut_p && pick(bp);
+                if (!found && b0 < head_end) found = bins(b0, head_end);
+                for (int g = g0; !found && g < g1; g += 32) {
+                    const int at = first_of((g + lane < g1) ? s_group[g + lane].a : 0ull);
+                    if (at >= 0) found = bins((g + at) * kSortGroup, (g + at + 1) * kSortGroup);
+                }
+                if (!found && tail0 < b1) found = bins(tail0, b1);
+                if (!found && cut_q) pick(bq);
+            }
+            __syncthreads();
+        }
+        double err = 0.0;
+        if (warp < 2 && lane < kLevels) {
+            const SortSums u = s_half[2 * lane], v = s_half[2 * lane + 1];
+            const float old = s_lv[lane];
+            const double o = (double)old, s1 = u.sx + v.sx, s0 = u.s + v.s;
+            if (warp == 0) {
+                float next = old;
+                if (!((F.fixed_mask >> lane) & 1u)) {
+                    if (MAE) next = (u.a + v.a > 0ull) ? s_med[lane] : old;
+                    else next = (s0 > 0.0) ? (float)(s1 / s0) : old;
+                }
+                s_level[now ^ 1][lane] = next;
+                const bool same = __all_sync(0xffffu, __float_as_uint(next) == __float_as_uint(old));
+                if (lane == 0) s_stop = same ? 1 : 0;
+            } else {
+                err = MAE ? (o * u.s - u.sx) + (v.sx - o * v.s) : o * (2.0 * s1 - o * s0);
+#pragma unroll
+                for (int off = 8; off; off >>= 1) err += __shfl_xor_sync(0xffffu, err, off);
+                if (!MAE) err = w2 - err;
+                err = fmax(err, 0.0) / (double)F.n_total;
+                if (lane == 0 && F.err_log) F.err_log[iter] = err;
+            }
+        }
+        __syncthreads();
+        if (s_stop) {
+            if (warp == 1 && lane < kLevels && F.err_log)
+                for (int k = iter + 1 + lane; k < F.iters; k += kLevels) F.err_log[k] = err;
+            now ^= 1;
+            break;
+        }
+    }
+    if (tid < kLevels && !((F.fixed_mask >> tid) & 1u)) F.codebook[tid] = s_level[now][tid];
+}
+
+// ---------------------------------------------------------------- host side
+
+namespace {
+
+template <bool MAE, bool CELLS>
+int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
+{
+    SampleWeight<MAE, CELLS> weight{};
+    weight.unit = F.metric >= 2;
+    weight.acc = reinterpret_cast<const ulonglong2*>(F.acc);
+    weight.acc_a = F.acc_a;
+    const int64_t ctas = (F.n_max + 8 * kSortChunk - 1) / (8 * kSortChunk);
+    sort_sums_kernel<MAE, CELLS><<<(int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st>>>(W, weight);
+    sort_group_kernel<MAE><<<kSortGroups / 8, 256, 0, st>>>(W);
+    constexpr int smem = kSortGroups * (int)sizeof(SortSums);
+    constexpr auto kern = sort_fit_kernel<MAE, CELLS>;
+    if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
+    kern<<<1, 1024, smem, st>>>(W, F);
+    BOF4_CUDA_TRY(cudaGetLastError());
+    return BOF4_OK;
+}
+
+template <class DT, bool SG>
+int samples(const EmTensors& T, int block_size, uint32_t first, const SortWs& W, cudaStream_t st)
+{
+#define BOF4_SORT_I(I_) \
+    case I_: sort_samples_kernel<DT, I_, SG><<<2 * kSMs, 512, 0, st>>>(T, first, W.a, W.n_items, W.w2); break;
+    switch (block_size) {
+        BOF4_SORT_I(32) BOF4_SORT_I(64) BOF4_SORT_I(128) BOF4_SORT_I(256) BOF4_SORT_I(512) BOF4_SORT_I(1024)
+        BOF4_SORT_I(2048) BOF4_SORT_I(4096)
+    }
+#undef BOF4_SORT_I
+    BOF4_CUDA_TRY(cudaGetLastError());
+    return BOF4_OK;
+}
+
+}  // namespace
+
+int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
+{
+    sort_count_kernel<0><<<kSortGrid, kSortThreads, 0, st>>>(W.a, W.n_items, W.counts);
+    sort_scatter_kernel<0><<<kSortGrid, kSortThreads, 0, st>>>(W.a, W.n_items, W.counts, W.b);
+    sort_count_kernel<8><<<kSortGrid, kSortThreads, 0, st>>>(W.b, W.n_items, W.counts);
+    sort_scatter_kernel<8><<<kSortGrid, kSortThreads, 0, st>>>(W.b, W.n_items, W.counts, W.a);
+    SortWs V = W;  // the ordered samples are in the first array
+    V.a = W.b;
+    V.b = W.a;
+    const int64_t ctas = (F.n_max + 255) / 256;
+    sort_start_kernel<<<(int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st>>>(V.b, V.n_items, V.start);
+    BOF4_CUDA_TRY(cudaGetLastError());
+    const bool mae = F.metric == BOF4_METRIC_MAE || F.metric == BOF4_METRIC_MAE_NORMALIZED;
+    if (F.acc) return mae ? sums_and_iterations<true, true>(V, F, st) : sums_and_iterations<false, true>(V, F, st);
+    return mae ? sums_and_iterations<true, false>(V, F, st) : sums_and_iterations<false, false>(V, F, st);
+}
+
+int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters, double* d_err_log, void* d_ws,
+               size_t ws_bytes, cudaStream_t st, bool* done)
+{
+    *done = false;
+    if (iters < kSortMinIters || a.n_total < 1 || a.n_total > kSortMaxDirect) return BOF4_OK;
+    SortWs W;
+    if (sorted_layout(d_ws, a.n_total, false, &W) > ws_bytes) return BOF4_OK;
+    *done = true;
+    sort_head_kernel<<<1, 320, 0, st>>>(W.n_items, (uint32_t)a.n_total, W.w2);
+    const bool sg = a.norm == BOF4_NORM_SIGNED;
+    uint32_t at = 0;
+    int calls = 0;
+    int rc = for_each_tensor_chunk(a, 512 * kLaneW, [&](const EmTensors& T) -> int {
+        const uint32_t first = at;
+        for (int t = 0; t < T.count; ++t) at += (uint32_t)T.n[t];
+        if (a.w_dtype == BOF4_F32)
+            return sg ? samples<F32, true>(T, a.block_size, first, W, st) : samples<F32, false>(T, a.block_size, first, W, st);
+        return sg ? samples<BF16, true>(T, a.block_size, first, W, st) : samples<BF16, false>(T, a.block_size, first, W, st);
+    }, &calls);
+    if (rc) return rc;
+    rc = for_each_tail_chunk(a, [&](const EmTails& Q) -> int {
+        if (a.w_dtype == BOF4_F32) {
+            if (sg) sort_tail_kernel<F32, true><<<1, kEmTailThreads, 0, st>>>(Q, at, W.a, W.n_items, W.w2);
+            else sort_tail_kernel<F32, false><<<1, kEmTailThreads, 0, st>>>(Q, at, W.a, W.n_items, W.w2);
+        } else {
+            if (sg) sort_tail_kernel<BF16, true><<<1, kEmTailThreads, 0, st>>>(Q, at, W.a, W.n_items, W.w2);
+            else sort_tail_kernel<BF16, false><<<1, kEmTailThreads, 0, st>>>(Q, at, W.a, W.n_items, W.w2);
+        }
+        for (int q = 0; q < Q.count; ++q) at += (uint32_t)Q.len[q];
+        BOF4_CUDA_TRY(cudaGetLastError());
+        return BOF4_OK;
+    });
+    if (rc) return rc;
+    SortFit F{};
+    F.metric = a.metric;
+    F.n_total = a.n_total;
+    F.n_max = a.n_total;
+    F.codebook = d_codebook;
+    F.fixed_mask = fixed_mask;
+    F.iters = iters;
+    F.err_log = d_err_log;
+    return sorted_run(W, F, st);
+}
+
+}  // namespace bof4

@@ -1,0 +1,119 @@
+// Codebook fit over samples that are put in order ONCE: interface between the two ways of making the
+// samples (em_sorted.cu: one per weight; em_cells.cu: one per distinct normalised weight of bf16
+// data) and what follows them (order, sums per bin, all iterations in one launch).
+//
+// The normalised weights x and the block constants do not change from one Lloyd iteration to the next;
+// only the thresholds move.  With the samples in ascending order of a 16-bit bin of x and the sums of
+// every bin at hand, an iteration needs no pass over the data: a region's sums are those of the bins
+// inside it plus the few samples of the two bins that its thresholds cut, and the weighted median is
+// found the same way.  An iteration costs about as much as a handful of L2 accesses, whatever the size
+// of the data.
+#pragma once
+
+#include "common.cuh"
+#include "em_common.cuh"
+#include "layout.h"
+
+namespace bof4 {
+
+constexpr int kSortGrid = 148;               // CTAs of the ordering passes, a contiguous part of the samples each
+constexpr int kSortBins = 1 << 16;           // bins of x; bin 0 stays empty
+constexpr int kSortGroup = 32;               // bins per group sum
+constexpr int kSortGroups = kSortBins / kSortGroup;
+constexpr int kSortChunk = 128;              // samples per warp of the bin sums
+// Below four iterations putting the samples in order costs more than streaming the data does (one
+// streaming iteration of small data is a 14 us launch, the ordering 35 us; of large data, see em_cells.cu).
+constexpr int kSortMinIters = 4;
+constexpr int64_t kSortMaxDirect = (int64_t)1 << 26;  // one sample per weight: 16 bytes of workspace each
+constexpr int kSortParts = 2 * kSMs + 1;     // partial sums of w^2: CTAs of the sample kernels, and the short last blocks
+
+// A sample is {x, payload}: the magnitude of its block constant, or (em_cells.cu) the number of its cell.
+struct SortSums {      // per bin, per group, or per part of a bin
+    double s, sx;      // sum of the sample weights, sum of weight * x
+    unsigned long long a;  // MAE: sum of the fixed-point weights of the median
+};
+
+struct SortWs {
+    uint32_t* n_items;    // device: [0] samples, [1] bits of the largest block constant, [2..3] scale (em_cells.cu)
+    double* w2;           // [kSortParts]
+    uint32_t* counts;     // [kSortGrid][256]
+    uint32_t* start;      // [kSortBins + 1] first sample of every bin
+    SortSums *bin, *group;
+    SortSums *lead, *trail;  // [chunks] part of a bin that began in an earlier chunk / that goes on in the next
+    float2 *a, *b;        // samples, ordered samples
+    double* cell_s;       // em_cells.cu: weights of the ordered samples (else NULL)
+    unsigned long long* cell_a;
+};
+
+// Bytes of workspace of the two ways (cells: 0 where they do not apply).
+size_t cells_workspace_bytes(int64_t n, int block_size);
+bool cells_apply(int w_dtype, int64_t n);
+
+// Carves the workspace for up to n samples; returns the bytes used.
+size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W);
+
+struct SortFit {
+    const unsigned long long* acc;   // em_cells.cu: [cell] {low, high} 128-bit sum of weights, else NULL
+    const unsigned long long* acc_a; // [cell] fixed-point weights (MAE)
+    int metric;
+    int64_t n_total;
+    int64_t n_max;                   // at most this many samples
+    float* codebook;
+    uint32_t fixed_mask;
+    int iters;
+    double* err_log;
+};
+
+// Samples are in W.a, their number in *W.n_items: orders them, sums the bins, runs the iterations.
+int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st);
+
+// The whole fit by one of the two ways; *done tells whether it was taken (workspace, size, type,
+// number of iterations).
+int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters, double* d_err_log, void* d_ws,
+               size_t ws_bytes, cudaStream_t st, bool* done);
+int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters, double* d_err_log, void* d_ws,
+              size_t ws_bytes, cudaStream_t st, bool* done);
+
+// Bin of a normalised weight, monotone in x: 32768 +- the bin of |x|, which is 0 for x = 0 alone, eight
+// bins per binade below 2^-7 (1 ... 254, all of |x| < 2^-38 in the first), bins of width 1 / 32767 from there on, and
+// 32767 for |x| = 1 alone.  Zeros (sparse data) and ones (a weight per block) are the only values that
+// data is likely to hold in any number, and no threshold ever has to look into a bin of one value.
+constexpr int kBinMinus = 1, kBinZero = 32768, kBinPlus = 65535;
+__device__ __forceinline__ int sort_bin(float x)
+{
+    const float a = fminf(fabsf(x), 1.0f);
+    int m;
+    if (a >= 0.0078125f) {
+        m = (int)(a * 32767.0f);
+    } else {
+        m = 255 - (960 - (int)(__float_as_uint(a) >> 20));
+        m = (a == 0.0f) ? 0 : max(m, 1);
+    }
+    return x < 0.0f ? kBinZero - m : kBinZero + m;
+}
+__device__ __forceinline__ bool one_value_bin(int b) { return b == kBinMinus || b == kBinZero || b == kBinPlus; }
+__device__ __forceinline__ float value_of_bin(int b) { return b == kBinMinus ? -1.0f : b == kBinPlus ? 1.0f : 0.0f; }
+
+// Order-preserving key of x and back; -0 and +0 share a key.
+__device__ __forceinline__ uint32_t sort_key(float x)
+{
+    const uint32_t u = __float_as_uint(x + 0.0f);
+    return u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float sort_key_value(uint32_t k)
+{
+    return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+
+// |m| as a 31-bit fixed-point integer relative to the largest magnitude of the data (see em_mae.cu).
+__device__ __forceinline__ uint32_t sort_fixed_weight(float m, uint32_t max_bits)
+{
+    const uint32_t b = __float_as_uint(fabsf(m));
+    const int e = max((int)(b >> 23), 1), emax = max((int)(max_bits >> 23), 1);
+    const uint32_t mant = (b & 0x7fffffu) | ((b >> 23) ? 0x800000u : 0u);
+    const int sh = e - emax + 7;
+    if (sh >= 0) return mant << min(sh, 7);
+    return (-sh >= 32) ? 0u : (mant >> (-sh));
+}
+
+}  // namespace bof4

@@ -4,6 +4,7 @@
 #include <stdio.h>
 
 #include "common.cuh"
+#include "em_sorted.cuh"
 #include "layout.h"
 
 namespace bof4 {
@@ -33,9 +34,17 @@ const char* bof4_last_error(void) { return bof4::g_err; }
 size_t bof4_workspace_bytes(int op, int64_t n_max, int block_size, int metric)
 {
     if (n_max < 0 || !bof4::valid_block_size(block_size)) return 0;
-    if (op == BOF4_OP_EM) {
+    if (op == BOF4_OP_EM || op == BOF4_OP_EM_BF16) {
         if (metric < BOF4_METRIC_MSE || metric > BOF4_METRIC_MAE_NORMALIZED) return 0;
-        return bof4::em_workspace_bytes_for(n_max);
+        size_t need = bof4::em_workspace_bytes_for(n_max);
+        const size_t cells = bof4::cells_workspace_bytes(n_max, block_size);
+        if (need < cells) need = cells;
+        // one sample per weight: fp32 data, and bf16 data too small for the other way
+        if (n_max >= 1 && n_max <= bof4::kSortMaxDirect && (op == BOF4_OP_EM || cells == 0)) {
+            const size_t direct = bof4::sorted_layout(nullptr, n_max, false, nullptr);
+            if (need < direct) need = direct;
+        }
+        return need;
     }
     if (op == BOF4_OP_OPQ) return bof4::opq_layout(n_max).total;
     return 0;

@@ -531,7 +531,7 @@ PyObject* fit_codebook(PyObject* const* a)
         if (!done) cb = codebook(a[4], w.d).clone();
         log = make(iters > 1 ? iters : 1, at::kDouble, w.d, iters < 1);  // the fit writes every entry
     }
-    const at::Tensor ws = workspace(a[7], BOF4_OP_EM, w.total, block, metric, w.d);
+    const at::Tensor ws = workspace(a[7], w.dt == BOF4_BF16 ? BOF4_OP_EM_BF16 : BOF4_OP_EM, w.total, block, metric, w.d);
     check(bof4_fit_codebook(w.ptr.data(), w.n.data(), (int)w.ptr.size(), w.dt, block, norm, metric,
                             static_cast<float*>(cb.data_ptr()), (uint32_t)integer(a[5]), (int)iters,
                             static_cast<double*>(log.data_ptr()), ws.data_ptr(), (size_t)ws.numel(), st));

@@ -1,0 +1,78 @@
+"""Fits of four and more iterations, which put the samples in order once: one sample per weight (fp32,
+small bf16) and one per distinct normalised weight (bf16 from 2^22 weights), against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bof4():
+    import __graft_entry__ as entry
+    entry.build()
+    import paper_2505_06653_b200 as m
+    assert torch.cuda.is_available()
+    return m
+
+
+def _weights(n, dtype, seed, kind):
+    w = workloads.gaussian(n, 0.02, seed, torch.float32)
+    g = torch.Generator().manual_seed(seed + 1)
+    if kind == "sparse":       # many exact zeros
+        w *= (torch.rand(n, generator=g) < 0.3)
+    elif kind == "grid":       # few distinct values
+        w = torch.round(w * 200) / 200
+    elif kind == "scales":     # block constants over sixty binades
+        w *= torch.exp2(torch.randint(-30, 30, ((n + 63) // 64,), generator=g).float()).repeat_interleave(64)[:n]
+    elif kind == "subnormal":  # bf16 weights below the normal range
+        w *= 1e-37
+    return w.to(dtype)
+
+
+def _check(bof4, ws, I, norm, metric, iters, mask=None):
+    lv, m = bof4.bof4_default_init(norm)
+    mask = m if mask is None else mask
+    dev = [w.cuda() for w in ws]
+    cb, log = bof4.bof4_fit_codebook(dev, I, norm, metric, lv, mask, iters)
+    again, log2 = bof4.bof4_fit_codebook(dev, I, norm, metric, lv, mask, iters)
+    assert torch.equal(cb, again) and torch.equal(log, log2)
+    ref, ref_log = oracle.fit(ws, I, norm, metric, lv, mask, iters)
+    if metric == bof4.METRIC_MAE:
+        assert np.array_equal(cb.cpu().numpy(), ref)
+    else:
+        np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5, atol=1e-7)
+    np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5, atol=1e-12)
+
+
+@pytest.mark.parametrize("sizes", [(1,), (31,), (129,), (4096, 33), (8192 * 148 + 5,), (1 << 20, 70001)])
+@pytest.mark.parametrize("metric", [0, 1])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_one_sample_per_weight(bof4, sizes, metric, dtype):
+    """Lengths around the edges of warps, chunks and tiles of the ordering passes."""
+    _check(bof4, [_weights(n, dtype, 100 + k, "plain") for k, n in enumerate(sizes)], 64, sum(sizes) % 2, metric, 4)
+
+
+@pytest.mark.parametrize("n,I,kind,mask", [((1 << 22), 64, "plain", None), ((1 << 22) + 37, 32, "sparse", 0),
+                                           ((1 << 22) + 4095, 4096, "grid", 0), ((1 << 22) + 64, 64, "scales", None),
+                                           ((1 << 22) + 1, 1024, "subnormal", None)])
+@pytest.mark.parametrize("metric", [0, 1])
+@pytest.mark.parametrize("norm", [0, 1])
+def test_one_sample_per_distinct_weight(bof4, n, I, kind, mask, metric, norm):
+    _check(bof4, [_weights(n, torch.bfloat16, 7, kind)], I, norm, metric, 4, mask)
+
+
+def test_converged_fit_fills_the_rest_of_the_log(bof4):
+    """Three distinct magnitudes: the levels settle at once, and every further entry is the same."""
+    w = torch.tensor([1.0, -0.5, 0.25, 0.0] * 4096)
+    _check(bof4, [w], 64, 0, 0, 50)
+
+
+def test_many_tensors(bof4):
+    """More tensors than one launch takes, with and without short last blocks."""
+    ws = [_weights(70000 + 13 * k, torch.bfloat16, k, "plain") for k in range(70)]
+    _check(bof4, ws, 128, 1, 1, 4)
+    _check(bof4, ws[:66], 128, 0, 0, 4)
