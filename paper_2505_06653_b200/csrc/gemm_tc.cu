@@ -7,38 +7,58 @@
 // weight rounded to bf16, bit for bit what bof4_dequantize writes (Eq. 3, then round to nearest
 // even), X is bf16, products are exact and the sums are accumulated in fp32 by the tensor cores.
 //
-// One CTA owns 128 rows of W and a range of K.  Eight producer warps decode, per k-block of 64
-// weights, the 128 x 64 tile (4 KiB of codes) into shared memory as bf16 in the K-major
-// 128-byte-swizzled layout that the tcgen05 shared-memory descriptor names (8-row groups of 1024
-// bytes, 16-byte chunk c of row r stored at chunk c ^ (r & 7)) and copy the matching 64 columns
-// of X the same way; each warp then arrives on the stage's "full" mbarrier.  One thread of a ninth
-// warp waits for a full stage and issues four tcgen05.mma (M = 128, N = batch, K = 16 each) that
-// accumulate into tensor memory; its tcgen05.commit arrives on the stage's "empty" mbarrier when
-// the tensor cores have read the stage, which the producers wait for before they overwrite it
-// (three stages).  No CTA-wide barrier inside the loop.  Every wait is bounded: a time-out sets
-// the status word, the issuing thread still commits and waits (bounded) for what it has issued,
-// and the kernel frees its tensor memory and returns.  The epilogue reads the accumulator with
-// tcgen05.ld (one row per thread) and writes fp32.
+// One CTA owns 128 rows of W and a range of K.  The codes come by TMA, four k-blocks of 64 weights (a
+// 128-byte line of every row) at a time into a ring; two warps bring the block constants beside them.
+// Sixteen producer warps, four groups of four with a k-block each and a thread per row, decode to bf16 and
+// store the row into TENSOR MEMORY (tcgen05.st, two weights per 32-bit column), from where tcgen05.mma takes
+// its A operand: the decoded matrix never touches shared memory, whose bandwidth (16 KiB written by the
+// producers and read again by the tensor cores per k-block, 256 cycles) bound the earlier form.  The
+// producers have no global load in flight either: publishing a k-block waited for it.
+//
+// Decode: the products of a block constant with the 16 levels are formed once per row and k-block, rounded
+// to bf16 and split into a table of low and a table of high bytes (four registers each); eight codes are
+// then looked up with byte permutes: two per table half, one that chooses between the halves by the
+// code's top bit, one that interleaves low and high bytes.  About 3 instructions per weight, on the half-rate
+// integer pipe, which bounds the kernel: 370 cycles per k-block and SM.
+//
+// OPQ (Sec. 3.3, decoding side): a position in the outlier list holds its stored bf16 value instead of
+// the decoded weight; the producer warp replaces it in tensor memory.  Two more warps find the list's part
+// for the tile and the entries of every row meanwhile.
+//
+// The 64 columns of X of a k-block come by TMA in the K-major 128-byte-swizzled layout that the tcgen05
+// shared-memory descriptor names; their bytes and one arrival per producer warp complete the stage's
+// "full" mbarrier.  One thread waits for the stages in order and issues four tcgen05.mma each (M = 128,
+// N = batch, K = 16); its tcgen05.commit arrives on the stage's "empty" mbarrier.  No CTA-wide barrier in
+// the loop.  Every wait is bounded: a time-out sets the status word, the issuing thread still commits and
+// waits (bounded) for what it has issued, and the kernel frees its tensor memory and returns.
+//
+// Matrices with few row tiles are split along K over the CTAs of a cluster (up to 8), whose partial products
+// are summed in rank order through distributed shared memory: no workspace and no second launch.
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "common.cuh"
 
 namespace bof4 {
 
-constexpr int kTcProducerWarps = 8;
-constexpr int kTcProducers = kTcProducerWarps * 32;  // threads that decode
-constexpr int kTcThreads = 32 + kTcProducers;        // and one warp that issues the tensor-core instructions
+constexpr int kTcGroups = 4;      // producer groups of four warps, a k-block each; k-blocks of a code line
 constexpr int kTcM = 128;         // rows per CTA = tensor-memory lanes
 constexpr int kTcK = 64;          // weights per k-block: one 128-byte swizzle row of bf16
-constexpr int kTcStages = 3;
-constexpr int kTcCtasPerSm = 2;   // 106 KiB of shared memory and 64 tensor-memory columns each
-constexpr int kTcMaxN = 64;
-constexpr int kTcTmemCols = 64;   // power of two >= 32 and >= N
-constexpr int kTcABytes = kTcM * kTcK * 2;     // 16 KiB
-constexpr int kTcBBytes = kTcMaxN * kTcK * 2;  // 8 KiB
-constexpr int kTcTableBytes = 256 * 16 * 8;    // level pairs per code byte, one column per lane pair (L, L + 16)
-constexpr int kTcSmem = kTcStages * (kTcABytes + kTcBBytes) + 1024 + kTcTableBytes;  // + slack to align to 1024 bytes
-constexpr uint32_t kTcSpinLimit = 1u << 16;    // try_wait calls before a wait gives up (a k-block takes microseconds)
+constexpr int kTcStages = 8;
+constexpr int kTcLines = 4;       // ring of code lines
+constexpr int kTcMaxN = 64;       // columns of the accumulator
+constexpr int kTcACols = kTcK / 2;               // tensor-memory columns of a stage of A
+constexpr int kTcTmemCols = 512;                 // power of two >= accumulator and stages of A
+static_assert(kTcMaxN + kTcStages * kTcACols <= kTcTmemCols, "tensor memory");
+constexpr int kTcBBytes = kTcMaxN * kTcK * 2;    // 8 KiB
+constexpr int kTcLineBytes = kTcM * 128;         // 16 KiB
+constexpr int kTcScaleFloats = 2 * kTcGroups * kTcM;  // constants of a line (two per k-block for blocks of 32 weights)
+constexpr int kTcSmem = kTcStages * kTcBBytes + kTcLines * (kTcLineBytes + kTcScaleFloats * 4) + 1024;  // + slack to align to 1024 bytes
+constexpr uint32_t kTcSpinLimit = 1u << 16;      // try_wait calls before a wait gives up (a k-block takes microseconds)
+constexpr int kTcMaxSplit = 8;                   // CTAs of a cluster (portable size)
+// warps: 0 issues, 1 ... 16 produce, 17 requests code lines, 18 X, 19 and 20 bring constants, 21 and 22 look outlier rows up
+constexpr int kTcFinders = 64;
+__host__ __device__ constexpr int tc_threads(bool opq) { return 32 * (kTcGroups * 4 + 5) + (opq ? kTcFinders : 0); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -68,10 +88,10 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity)
         uint32_t ok;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok)
-            : "r"(bar), "r"(parity)
+            : "r"(bar), "r"(parity), "r"(1000u)  // suspended for up to a microsecond instead of polling
             : "memory");
         if (ok) return true;
     }
@@ -91,47 +111,149 @@ __device__ __forceinline__ float tc_scale<BF16>(const void* scales, int64_t b)
     return __uint_as_float((uint32_t)__ldg(static_cast<const uint16_t*>(scales) + b) << 16);
 }
 
-template <class ST>
-__global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm)
-gemm_tc_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t cols, int block_shift,
-               const float* __restrict__ levels, const __grid_constant__ CUtensorMap x_map, int n_rhs,
-               float* __restrict__ y, int kb_per_split, int* __restrict__ status)
+__device__ __forceinline__ uint32_t tc_prmt(uint32_t a, uint32_t b, uint32_t sel)
 {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+    return d;
+}
+
+// The 16 levels times a block constant, rounded to bf16 (Eq. 3 and the operand's rounding), as a table of
+// low bytes and one of high bytes.
+struct TcTable {
+    uint32_t lo[4], hi[4];
+};
+__device__ __forceinline__ TcTable tc_table(float m, const float2 (&lv)[8])
+{
+    TcTable t;
+    uint32_t p[8];
+    const float2 mm = make_float2(m, m);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float2 v = __fmul2_rn(mm, lv[k]);
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[k]) : "f"(v.y), "f"(v.x));
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        t.lo[k] = tc_prmt(p[2 * k], p[2 * k + 1], 0x6420u);
+        t.hi[k] = tc_prmt(p[2 * k], p[2 * k + 1], 0x7531u);
+    }
+    return t;
+}
+// Eight codes (even element in the high nibble of its byte) to eight bf16 values.
+__device__ __forceinline__ void tc_decode8(uint32_t w, const TcTable& t, uint32_t* o)
+{
+    const uint32_t sel = w & 0x77777777u, half = ((w >> 1) & 0x44444444u) | 0x32103210u;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t s = h ? sel >> 16 : sel, c = h ? half >> 16 : half;
+        const uint32_t lo = tc_prmt(tc_prmt(t.lo[0], t.lo[1], s), tc_prmt(t.lo[2], t.lo[3], s), c);
+        const uint32_t hi = tc_prmt(tc_prmt(t.hi[0], t.hi[1], s), tc_prmt(t.hi[2], t.hi[3], s), c);
+        o[2 * h] = tc_prmt(lo, hi, 0x4051u);      // bytes of codes 1 0 3 2: low half of a pair is the even one
+        o[2 * h + 1] = tc_prmt(lo, hi, 0x6273u);
+    }
+}
+
+// First entry of the ascending list with idx >= key, by one warp: a guess from the key's place in the
+// matrix narrows the range to 32 entries in one step for lists of evenly spread outliers; any other list
+// takes steps of a factor of 32.
+__device__ __forceinline__ int64_t tc_lower_bound(const int32_t* __restrict__ idx, int64_t k_end, int64_t key, int64_t n, int lane)
+{
+    int64_t lo = 0, hi = k_end;  // the answer lies in [lo, hi]
+    int64_t g = (int64_t)((double)k_end * ((double)key / (double)n)) - 512;
+    g = g < 0 ? 0 : g;
+    for (int step = 0; hi > lo; ++step) {
+        // 32 probes; the entries before the last probe that is below the key are below it as well
+        const int64_t first = step == 0 ? g : lo, stride = step == 0 ? 32 : (hi - lo + 31) / 32;
+        const int64_t at = first + lane * stride;
+        const int cnt = __popc(__ballot_sync(kFull, at < hi && (int64_t)__ldg(idx + at) < key));
+        const int64_t above = first + (int64_t)cnt * stride;  // the first probe that is not below the key
+        if (cnt > 0) lo = above - stride + 1;
+        if (cnt < 32 && above < hi) hi = above;
+        if (step > 0 && stride == 1) break;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ void tc_arrive(unsigned long long* bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tc_load_box(uint32_t dst, const CUtensorMap* map, unsigned long long* bar, uint32_t bytes, int x, int y)
+{
+    const uint32_t b = smem_u32(bar);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+                 :
+                 : "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(b), "r"(x), "r"(y)
+                 : "memory");
+}
+// Sixteen 32-bit columns of the warp's 32 rows in tensor memory.
+__device__ __forceinline__ void tc_store16(uint32_t addr, const uint32_t (&v)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        :
+        : "r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+          "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+        : "memory");
+}
+
+template <class ST, bool HALF, bool OPQ>  // HALF: blocks of 32 weights, two constants per row and k-block
+__global__ void __launch_bounds__(tc_threads(OPQ), 1)
+gemm_tc_kernel(const __grid_constant__ CUtensorMap code_map, const void* __restrict__ scales, int64_t cols, int block_shift,
+               const float* __restrict__ levels, const __grid_constant__ CUtensorMap x_map, int n_rhs,
+               float* __restrict__ y, int* __restrict__ status, const int32_t* __restrict__ out_idx,
+               const uint16_t* __restrict__ out_val, const int64_t* __restrict__ n_out, int64_t capacity)
+{
+    constexpr int NT = tc_threads(OPQ);
     extern __shared__ unsigned char s_dyn[];
-    // full[s]: the producers have filled stage s (one arrival per producer warp); empty[s]: the tensor
-    // cores have read it (tcgen05.commit); done: every instruction of the CTA has completed
-    __shared__ __align__(8) unsigned long long s_full[kTcStages], s_empty[kTcStages], s_done;
+    // full[s]: stage s holds a k-block (one arrival per producer warp; one and the TMA bytes for X); empty[s]: the
+    // tensor cores have read it (tcgen05.commit); line_full / line_empty: the same for the ring of code lines
+    // and constants; done: every instruction of the CTA has completed; rows: s_beg and s_end are set
+    __shared__ __align__(8) unsigned long long s_full[kTcStages], s_empty[kTcStages], s_line_full[kTcLines], s_line_empty[kTcLines],
+        s_done, s_rows;
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
+    __shared__ int s_beg[kTcM], s_end[kTcM];  // OPQ: the list entries of every row of the tile inside the CTA's columns
+    __shared__ long long s_part[2];           // OPQ: the tile's part of the list
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t tiles = (smem_u32(s_dyn) + 1023u) & ~1023u;  // 1024-byte aligned: the swizzle atoms start here
     unsigned char* tiles_ptr = s_dyn + (tiles - smem_u32(s_dyn));
+    const uint32_t code_ring = tiles + kTcStages * kTcBBytes;
+    float* const scale_ring = reinterpret_cast<float*>(tiles_ptr + kTcStages * kTcBBytes + kTcLines * kTcLineBytes);
     const int64_t row0 = (int64_t)blockIdx.x * kTcM;
-    // blockIdx.y selects a range of k-blocks (split along K so that matrices with few row tiles still
-    // fill the machine); its partial product goes to slab blockIdx.y of y
-    const int kblocks = kb_per_split, kb0 = (int)blockIdx.y * kb_per_split;
-    y += (int64_t)blockIdx.y * ((int64_t)gridDim.x * kTcM) * n_rhs;
+    // the CTA's k-blocks: its share of the cluster's, in whole lines
+    const int splits = (int)gridDim.y, rank = (int)blockIdx.y, kb_all = (int)(cols / kTcK);
+    const int lines_all = (kb_all + kTcGroups - 1) / kTcGroups;
+    const int line0 = (int)((int64_t)lines_all * rank / splits), lines = (int)((int64_t)lines_all * (rank + 1) / splits) - line0;
+    const int kb0 = line0 * kTcGroups, kblocks = min(kb_all - kb0, lines * kTcGroups);
+    // wait of a whole warp; false (and the failure noted): it ran out
+    auto warp_wait = [&](unsigned long long* bar, uint32_t parity) -> bool {
+        if (__all_sync(kFull, tc_wait(smem_u32(bar), parity))) return true;
+        if (lane == 0) s_fail = 1;
+        return false;
+    };
 
-    // Level pairs of a code byte (Eq. 3's xhat for its two weights), one 8-byte column per pair of
-    // lanes L and L + 16: an 8-byte read is served half a warp at a time, so the 16 lanes of a half
-    // never share a bank whatever their code bytes are.
-    unsigned char* tab_ptr = tiles_ptr + kTcStages * (kTcABytes + kTcBBytes);
-    __shared__ float s_lv[kLevels];
-    if (tid < kLevels) s_lv[tid] = levels[tid];
-    __syncthreads();  // the table is filled from shared memory: no global read per entry
-    for (int e = tid; e < 256 * 16; e += kTcThreads)
-        reinterpret_cast<float2*>(tab_ptr)[e] = make_float2(s_lv[e >> 8], s_lv[(e >> 4) & 15]);
-    const uint32_t tab = smem_u32(tab_ptr) + (uint32_t)(lane & 15) * 8u;
     if (tid == 0) {
+        if (blockIdx.x == 0 && rank == 0) *status = 0;  // long before any wait can have run out
         s_fail = 0;
+        auto init = [&](unsigned long long* bar, int count) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+        };
         for (int s = 0; s < kTcStages; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_full[s])), "r"(kTcProducerWarps + 1) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_empty[s])), "r"(1) : "memory");
+            init(&s_full[s], 4 + 1);
+            init(&s_empty[s], 1);
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_done)), "r"(1) : "memory");
+        for (int s = 0; s < kTcLines; ++s) {
+            init(&s_line_full[s], 2);
+            init(&s_line_empty[s], 4 * kTcGroups);
+        }
+        init(&s_done, 1);
+        init(&s_rows, kTcFinders / 32);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) {  // tensor memory for the 128 x N fp32 accumulator
+    if (warp == 0) {  // tensor memory: the 128 x N fp32 accumulator, then the stages of A
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                      "r"(kTcTmemCols)
                      : "memory");
@@ -148,24 +270,24 @@ gemm_tc_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scale
         if (lane == 0) {
             const uint32_t idesc = tc_instr_desc(n_rhs);
             bool ok = true;
-            for (int kb = 0; kb < kblocks && ok; ++kb) {
+            for (int kb = 0; kb < kblocks; ++kb) {
                 const int s = kb % kTcStages;
                 if (!tc_wait(smem_u32(&s_full[s]), (uint32_t)((kb / kTcStages) & 1))) {
                     ok = false;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t sa = tiles + (uint32_t)s * (kTcABytes + kTcBBytes);
-                const uint64_t da = tc_smem_desc(sa), db = tc_smem_desc(sa + kTcABytes);
+                const uint32_t a = tmem + (uint32_t)(kTcMaxN + s * kTcACols);
+                const uint64_t db = tc_smem_desc(tiles + (uint32_t)s * kTcBBytes);
 #pragma unroll
-                for (int kk = 0; kk < kTcK / 16; ++kk) {  // 32 bytes of K per instruction: +2 in the address field
+                for (int kk = 0; kk < kTcK / 16; ++kk) {  // 16 of K: eight columns of A, +2 in the address field of B
                     const uint32_t acc = (kb > 0 || kk > 0) ? 1u : 0u;
                     asm volatile(
                         "{\n\t.reg .pred p;\n\t"
                         "setp.ne.b32 p, %4, 0;\n\t"
-                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
+                        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}"
                         :
-                        : "r"(tmem), "l"(da + (uint64_t)(2 * kk)), "l"(db + (uint64_t)(2 * kk)), "r"(idesc), "r"(acc), "r"(0u)
+                        : "r"(tmem), "r"(a + (uint32_t)(8 * kk)), "l"(db + (uint64_t)(2 * kk)), "r"(idesc), "r"(acc), "r"(0u)
                         : "memory");
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -179,92 +301,151 @@ gemm_tc_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scale
             if (!ok) s_fail = 1;
             if (!tc_wait(smem_u32(&s_done), 0u)) s_fail = 1;
         }
-    } else {
-        // ---- producer warps: thread t decodes half a row (32 weights = 16 code bytes = four 16-byte
-        // chunks) of the 128 x 64 tile; the first of them also requests the X tile
-        const int t = tid - 32;
-        const int a_row = t >> 1, a_half = t & 1;
-        const uint8_t* a_codes = codes + ((row0 + a_row) * cols) / 2 + a_half * 16;
-        const int64_t a_first = (row0 + a_row) * cols + a_half * 32;  // flat index of its first weight in k-block 0
-        const uint32_t a_off = (uint32_t)((a_row >> 3) * 1024 + (a_row & 7) * 128);
-        struct Fetched {
-            uint4 cc;
-            float m;
+    } else if (warp <= kTcGroups * 4) {
+        // ---- producers: group g decodes k-blocks g, g + 4, ...; the thread's row of a k-block is 64 weights.
+        // A warp reaches the 32 rows of tensor memory that its number modulo 4 names.
+        const int group = (warp - 1) >> 2, a_row = (warp & 3) * 32 + lane;
+        const uint32_t a_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)kTcMaxN;
+        float2 lv[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) lv[k] = __ldg(reinterpret_cast<const float2*>(levels) + k);
+        // OPQ: the row's next list entry, as a column of this CTA, and its value
+        int at = 0, end = 0, next = INT32_MAX;
+        uint32_t value = 0u;
+        const int base = OPQ ? (int)((row0 + a_row) * cols + (int64_t)kb0 * kTcK) : 0;  // indices fit 31 bits
+        auto entry = [&]() {
+            next = at < end ? __ldg(out_idx + at) - base : INT32_MAX;
+            value = at < end ? (uint32_t)__ldg(out_val + at) : 0u;
         };
-        auto fetch = [&](int kb) {  // what the thread reads from global memory for one k-block
-            Fetched f;
-            kb += kb0;
-            // a row's codes are read 32 bytes per k-block (two threads); the hint brings the whole 128-byte
-            // line into L2 at the first touch, so DRAM sees full lines instead of scattered sectors
-            asm volatile("ld.global.nc.L2::128B.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(f.cc.x), "=r"(f.cc.y), "=r"(f.cc.z), "=r"(f.cc.w)
-                         : "l"(a_codes + (int64_t)kb * (kTcK / 2)));
-            f.m = tc_scale<ST>(scales, (a_first + (int64_t)kb * kTcK) >> block_shift);
-            return f;
-        };
-        // One k-block: wait for the stage, request X, decode, publish.  false: a wait ran out.
-        auto step = [&](int kb, const Fetched& cur) -> bool {
-            const int s = kb % kTcStages;
-            unsigned char* sa = tiles_ptr + s * (kTcABytes + kTcBBytes);
-            unsigned char* sb = sa + kTcABytes;
-            if (kb >= kTcStages) {  // the tensor cores must have read what the stage held (k-block kb - stages)
-                int ok = 1;
-                if (lane == 0) ok = tc_wait(smem_u32(&s_empty[s]), (uint32_t)(((kb / kTcStages) - 1) & 1)) ? 1 : 0;
-                ok = __shfl_sync(kFull, ok, 0);
-                if (!ok) {
-                    if (lane == 0) s_fail = 1;
-                    return false;
+        for (int kb = group, line = 0; kb < kblocks; kb += kTcGroups, ++line) {
+            const int ls = line % kTcLines, s = kb % kTcStages;
+            if (!warp_wait(&s_line_full[ls], (uint32_t)((line / kTcLines) & 1))) break;
+            uint32_t w[8];
+            // the thread's 32 bytes: chunks 2 g and 2 g + 1 of its row's line (128-byte swizzle)
+            const uint32_t row = code_ring + (uint32_t)ls * kTcLineBytes + (uint32_t)a_row * 128u;
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(w[4 * h]), "=r"(w[4 * h + 1]), "=r"(w[4 * h + 2]), "=r"(w[4 * h + 3])
+                             : "r"(row + (uint32_t)(((2 * group + h) ^ (a_row & 7)) * 16)));
+            const float* sc = scale_ring + ls * kTcScaleFloats + (HALF ? 2 * group : group) * kTcM + a_row;
+            const float m = sc[0], m2 = HALF ? sc[kTcM] : 0.0f;
+            TcTable tab = tc_table(m, lv);
+            uint32_t v[16];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) tc_decode8(w[j], tab, v + 4 * j);
+            // the tensor cores must have read what the stage held (k-block kb - stages)
+            if (kb >= kTcStages && !warp_wait(&s_empty[s], (uint32_t)(((kb / kTcStages) - 1) & 1))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t dst = a_lane + (uint32_t)(s * kTcACols);
+            tc_store16(dst, v);
+            if (HALF) tab = tc_table(m2, lv);
+            uint32_t u[16];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) tc_decode8(w[4 + j], tab, u + 4 * j);
+            tc_store16(dst + 16u, u);
+            if (lane == 0) tc_arrive(&s_line_empty[ls]);
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            if (OPQ) {
+                if (kb == group) {  // the row's part of the list, found meanwhile
+                    if (!warp_wait(&s_rows, 0u)) break;
+                    at = s_beg[a_row], end = s_end[a_row];
+                    entry();
+                }
+                const int c0 = kb * kTcK;
+                while (next < c0) {  // the other groups' entries
+                    ++at;
+                    entry();
+                }
+                __syncwarp();
+                // one entry of one row at a time: the column it shares with its neighbour comes back from tensor
+                // memory, the row's half of it is replaced (about two entries per warp and k-block)
+                unsigned hits;
+                while ((hits = __ballot_sync(kFull, next < c0 + kTcK)) != 0u) {
+                    const int src = __ffs(hits) - 1, c = __shfl_sync(kFull, next, src) - c0;
+                    const uint32_t a = dst + (uint32_t)(c >> 1);
+                    uint32_t r;
+                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(a));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (lane == src) {
+                        r = (c & 1) ? (r & 0xffffu) | (value << 16) : (r & 0xffff0000u) | value;
+                        ++at;
+                        entry();
+                    }
+                    __syncwarp();
+                    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(a), "r"(r) : "memory");
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 }
             }
-            if (t == 0) {
-                // the X tile (n_rhs rows of 64 values) comes by TMA straight into the swizzled layout; its
-                // bytes count towards the stage's "full" barrier together with the producer warps' arrivals
-                const uint32_t bar = smem_u32(&s_full[s]);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)n_rhs * 128u)
-                             : "memory");
-                asm volatile(
-                    "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                    :
-                    : "r"(smem_u32(sb)), "l"(reinterpret_cast<uint64_t>(&x_map)), "r"(bar), "r"((kb0 + kb) * kTcK), "r"(0)
-                    : "memory");
-            }
-            const float2 mm = make_float2(cur.m, cur.m);
-            const uint32_t word[4] = {cur.cc.x, cur.cc.y, cur.cc.z, cur.cc.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {  // chunk j of this half: weights 8j .. 8j+7 = code bytes 4j .. 4j+3
-                uint32_t p[4];
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    // byte b of the word times 128 (the table's row size): one shift and one mask
-                    const uint32_t off = ((b == 0) ? (word[j] << 7) : (word[j] >> (8 * b - 7))) & 0x7f80u;
-                    float2 lv2;
-                    asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lv2.x), "=f"(lv2.y) : "r"(tab + off));
-                    const float2 w2 = __fmul2_rn(mm, lv2);  // Eq. 3 for the (even, odd) weight of the byte
-                    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[b]) : "f"(w2.y), "f"(w2.x));  // even weight in the low half
-                }
-                const int chunk = a_half * 4 + j;
-                *reinterpret_cast<uint4*>(sa + a_off + ((chunk ^ (a_row & 7)) * 16)) = make_uint4(p[0], p[1], p[2], p[3]);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> tensor-core reads
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&s_full[s])) : "memory");
-            return true;
-        };
-        // two fetch buffers used in turn (no register copies): the loads of k-block kb + 1 are in flight
-        // while k-block kb is decoded
-        {
-            Fetched fa = fetch(0), fb = fa;
-            int kb = 0;
-            while (kb < kblocks) {
-                if (kb + 1 < kblocks) fb = fetch(kb + 1);
-                if (!step(kb, fa)) break;
-                if (++kb >= kblocks) break;
-                if (kb + 1 < kblocks) fa = fetch(kb + 1);
-                if (!step(kb, fb)) break;
-                ++kb;
-            }
+            if (lane == 0) tc_arrive(&s_full[s]);
         }
+    } else if (warp == kTcGroups * 4 + 1) {
+        // ---- code lines: 128 bytes of each of the 128 rows
+        for (int line = 0; line < lines; ++line) {
+            const int ls = line % kTcLines;
+            if (line >= kTcLines && !warp_wait(&s_line_empty[ls], (uint32_t)(((line / kTcLines) - 1) & 1))) break;
+            if (lane == 0)
+                tc_load_box(code_ring + (uint32_t)ls * kTcLineBytes, &code_map, &s_line_full[ls], kTcLineBytes, (line0 + line) * 128, (int)row0);
+        }
+    } else if (warp == kTcGroups * 4 + 2) {
+        // ---- X: the 64 columns of a k-block
+        for (int kb = 0; kb < kblocks; ++kb) {
+            const int s = kb % kTcStages;
+            if (kb >= kTcStages && !warp_wait(&s_empty[s], (uint32_t)(((kb / kTcStages) - 1) & 1))) break;
+            if (lane == 0) tc_load_box(tiles + (uint32_t)s * kTcBBytes, &x_map, &s_full[s], (uint32_t)n_rhs * 128u, (kb0 + kb) * kTcK, 0);
+        }
+    } else if (warp <= kTcGroups * 4 + 4) {
+        // ---- block constants of every other line, as fp32 [k-block][row]
+        constexpr int PER = HALF ? 2 : 1;
+        for (int line = warp - (kTcGroups * 4 + 3); line < lines; line += 2) {
+            const int ls = line % kTcLines;
+            float v[4 * kTcGroups * PER];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int64_t first = (row0 + lane + 32 * r) * cols + (int64_t)kb0 * kTcK;
+#pragma unroll
+                for (int q = 0; q < kTcGroups * PER; ++q) {
+                    const int kb = min(line * kTcGroups + q / PER, kblocks - 1);
+                    v[q * 4 + r] = tc_scale<ST>(scales, (first + kb * kTcK + (q % PER) * 32) >> block_shift);
+                }
+            }
+            if (line >= kTcLines && !warp_wait(&s_line_empty[ls], (uint32_t)(((line / kTcLines) - 1) & 1))) break;
+#pragma unroll
+            for (int q = 0; q < kTcGroups * PER; ++q)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) scale_ring[ls * kTcScaleFloats + q * kTcM + lane + 32 * r] = v[q * 4 + r];
+            __syncwarp();
+            if (lane == 0) tc_arrive(&s_line_full[ls]);
+        }
+    } else if (OPQ) {
+        // ---- OPQ: the entries of every row of the tile inside the CTA's columns
+        const int f = tid - (kTcGroups * 4 + 5) * 32;
+        int64_t k_end = *n_out;
+        if (k_end > capacity) k_end = capacity;
+        const int64_t n = (int64_t)gridDim.x * kTcM * cols;
+        for (int r = f; r < kTcM; r += kTcFinders) s_beg[r] = s_end[r] = 0;
+        // first and last entry of the tile, a warp each
+        const int64_t p = tc_lower_bound(out_idx, k_end, (row0 + (f < 32 ? 0 : kTcM)) * cols, n, lane);
+        if (lane == 0) s_part[f >> 5] = p;
+        asm volatile("bar.sync 1, %0;" ::"n"(kTcFinders) : "memory");
+        const int64_t lo = s_part[0], hi = s_part[1];
+        const uint32_t tile = (uint32_t)(row0 * cols), c_lo = (uint32_t)kb0 * kTcK, c_hi = c_lo + (uint32_t)kblocks * kTcK, nc = (uint32_t)cols;
+        // row of entry k if it lies inside the CTA's columns, else -1 (also for what a list that is not ascending holds)
+        auto row_of = [&](int64_t k) -> int {
+            if (k < lo || k >= hi) return -1;
+            const uint32_t i = (uint32_t)__ldg(out_idx + k) - tile, r = i / nc, c = i - r * nc;
+            return (r < (uint32_t)kTcM && c >= c_lo && c < c_hi) ? (int)r : -1;
+        };
+        for (int64_t k = lo + f; k < hi; k += kTcFinders) {
+            const int r = row_of(k);
+            if (r < 0) continue;
+            if (row_of(k - 1) != r) s_beg[r] = (int)k;
+            if (row_of(k + 1) != r) s_end[r] = (int)k + 1;
+        }
+        __syncwarp();
+        if (lane == 0) tc_arrive(&s_rows);
     }
     // Every loop above is bounded, so every warp gets here.  After a time-out the issuing thread has
     // still committed and waited (bounded) for what it issued.
@@ -272,83 +453,56 @@ gemm_tc_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scale
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const bool failed = s_fail != 0;
-    if (!failed && warp < 4) {  // the accumulator, one row per thread (warp w reads lanes 32 w .. 32 w + 31)
-        float* yrow = y + (row0 + warp * 32 + lane) * n_rhs;
-        for (int c0 = 0; c0 < n_rhs; c0 += 8) {
-            uint32_t v[8];
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                         : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int c = 0; c < 8; ++c) yrow[c0 + c] = __uint_as_float(v[c]);
-        }
-    }
     if (failed) {
         // a TMA copy requested before the time-out may still be writing this CTA's shared memory: it
         // takes microseconds; give it a bounded 100 before the CTA goes away
         if (tid == 0) atomicExch(status, 1);
         for (int i = 0; i < 100; ++i) __nanosleep(1000);
     }
+    // the accumulator, one row per thread (warp w reads lanes 32 (w % 4) ...), through shared memory: the stages
+    // are free now.  Rows are padded by 16 bytes so that eight neighbouring rows fall into different banks.
+    float* part = reinterpret_cast<float*>(tiles_ptr);
+    const int pitch = n_rhs + 4;
+    if (!failed && warp < 16) {
+        float* prow = part + ((warp & 3) * 32 + lane) * pitch;
+        for (int c0 = (warp >> 2) * 8; c0 < n_rhs; c0 += 32) {
+            uint32_t v[8];
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                         : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0));
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            *reinterpret_cast<uint4*>(prow + c0) = make_uint4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<uint4*>(prow + c0 + 4) = make_uint4(v[4], v[5], v[6], v[7]);
+        }
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    if (splits > 1) cluster.sync();
+    else __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
-}
-
-// OPQ (Sec. 3.3, decoding side): an outlier position holds its stored bf16 value instead of the
-// decoded weight, so Y[r][b] += (val - decoded) * X[b][c] for every outlier (r, c).  One warp per
-// row: the row's outliers are a contiguous run of the ascending index list (two binary searches),
-// each lane owns right-hand sides b = lane, lane + 32 and adds the row's terms in list order.
-template <class ST>
-__global__ void __launch_bounds__(256)
-gemm_tc_outlier_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t rows, int64_t cols,
-                       int block_shift, const float* __restrict__ levels, const uint16_t* __restrict__ x, int n_rhs,
-                       const int32_t* __restrict__ idx, const uint16_t* __restrict__ val,
-                       const int64_t* __restrict__ n_out, int64_t capacity, float* __restrict__ y)
-{
-    int64_t k_end = *n_out;
-    if (k_end > capacity) k_end = capacity;
-    if (k_end <= 0) return;
-    auto lower_bound = [&](int64_t key) {  // first k with idx[k] >= key
-        int64_t lo = 0, hi = k_end;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if ((int64_t)idx[mid] < key) lo = mid + 1; else hi = mid;
-        }
-        return lo;
-    };
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += warps) {
-        const int64_t lo = lower_bound(r * cols), hi = lower_bound((r + 1) * cols);
-        if (lo == hi) continue;
-        for (int b = lane; b < n_rhs; b += 32) {
-            float acc = y[r * n_rhs + b];
-            for (int64_t k = lo; k < hi; ++k) {
-                const int64_t i = idx[k];
-                const uint32_t byte = codes[i >> 1];
-                const uint32_t c = (i & 1) ? (byte & 15u) : (byte >> 4);
-                const float q32 = __fmul_rn(tc_scale<ST>(scales, i >> block_shift), __ldg(levels + c));
-                uint32_t qb;
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(qb) : "f"(0.0f), "f"(q32));  // the operand the tile held
-                const float delta = __uint_as_float((uint32_t)val[k] << 16) - __uint_as_float(qb << 16);
-                const float xv = __uint_as_float((uint32_t)x[(int64_t)b * cols + (i - r * cols)] << 16);
-                acc = __fadd_rn(acc, __fmul_rn(delta, xv));
+    // the tile's 128 x n_rhs results are contiguous in y: each CTA of the cluster sums and writes its share
+    // of the rows, the ranks' parts in order
+    const int quads = n_rhs >> 2, rows_here = kTcM / splits;
+    for (int i = tid; i < rows_here * quads; i += NT) {
+        const int r = rank * rows_here + i / quads, c = (i % quads) * 4;
+        float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int q = 0; q < splits; ++q) {
+            const float* src = splits > 1 ? cluster.map_shared_rank(part, q) : part;
+            const float4 v = *reinterpret_cast<const float4*>(src + r * pitch + c);
+            if (q == 0) {
+                sum = v;
+            } else {
+                sum.x += v.x;
+                sum.y += v.y;
+                sum.z += v.z;
+                sum.w += v.w;
             }
-            y[r * n_rhs + b] = acc;
         }
+        *reinterpret_cast<float4*>(y + (row0 + r) * n_rhs + c) = sum;
     }
-}
-
-// Sum of the K-split partial products in slab order (fixed: the result does not depend on scheduling).
-__global__ void gemm_tc_reduce_kernel(const float* __restrict__ part, int splits, int64_t total, float* __restrict__ y)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        float a = part[i];
-        for (int s = 1; s < splits; ++s) a += part[(int64_t)s * total + i];
-        y[i] = a;
-    }
+    if (splits > 1) cluster.sync();  // nobody leaves while its part is being read
 }
 
 }  // namespace bof4
@@ -361,28 +515,30 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Tensor map of X (bf16 [n_rhs][cols]) with a box of 64 columns x n_rhs rows and the 128-byte swizzle:
-// one TMA load per k-block lands in the layout the tcgen05 descriptor of the B operand names.
-int make_x_map(const void* d_x, int64_t cols, int n_rhs, CUtensorMap* map)
+// Tensor map of a row-major matrix of 2-byte or 1-byte elements with a box of 128 bytes x box_rows and the
+// 128-byte swizzle: X lands in the layout that the tcgen05 descriptor of the B operand names, a code
+// line in one that sixteen-byte reads of neighbouring rows find without bank conflicts.
+int make_map(const void* p, bool bytes, int64_t cols, int64_t rows, int box_rows, CUtensorMap* map)
 {
     static EncodeTiledFn fn = nullptr;
     if (!fn) {
-        void* p = nullptr;
+        void* f = nullptr;
         cudaDriverEntryPointQueryResult q;
-        BOF4_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q));
-        if (!p || q != cudaDriverEntryPointSuccess) {
+        BOF4_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q));
+        if (!f || q != cudaDriverEntryPointSuccess) {
             set_error("bof4_gemm_tc: the driver does not provide cuTensorMapEncodeTiled");
             return BOF4_ERR_CUDA;
         }
-        fn = reinterpret_cast<EncodeTiledFn>(p);
+        fn = reinterpret_cast<EncodeTiledFn>(f);
     }
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)n_rhs};
-    const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kTcK, (cuuint32_t)n_rhs};
+    const int esize = bytes ? 1 : 2;
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)cols * esize};
+    const cuuint32_t box[2] = {(cuuint32_t)(128 / esize), (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(d_x), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = fn(map, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(p), dims,
+                          strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         set_error("bof4_gemm_tc: cuTensorMapEncodeTiled failed with code %d", (int)r);
         return BOF4_ERR_CUDA;
@@ -434,56 +590,55 @@ extern "C" int bof4_gemm_tc(const uint8_t* d_codes, const void* d_scales, int sc
         return BOF4_ERR_SHAPE;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    BOF4_CUDA_TRY(cudaMemsetAsync(d_status, 0, sizeof(int), st));
     if (cols == 0) {
+        BOF4_CUDA_TRY(cudaMemsetAsync(d_status, 0, sizeof(int), st));
         BOF4_CUDA_TRY(cudaMemsetAsync(d_y, 0, (size_t)rows * n_rhs * sizeof(float), st));
         return BOF4_OK;
     }
     const int grid = (int)(rows / kTcM);
-    // K split: enough CTAs to fill the SMs (kTcCtasPerSm each), a divisor of the number of k-blocks,
-    // partial products in the workspace (none: no split).  Measured: more and shorter CTAs than
-    // that cost more (table set-up, pipeline fill and drain, epilogue) than the fuller last wave gains.
+    // Split along K over a cluster: the choice with the least waves x (k-blocks per CTA + what a CTA costs
+    // beside them, about six k-blocks: set-up, pipeline fill and drain, epilogue).
     const int kblocks = (int)(cols / kTcK);
     int splits = 1;
-    const size_t slab = (size_t)rows * n_rhs * sizeof(float);
-    if (d_ws && !((uintptr_t)d_ws & 15u)) {
-        for (int cand = 2; cand <= 8; ++cand)
-            if (kblocks % cand == 0 && (size_t)cand * slab <= ws_bytes && (int64_t)grid * (cand - 1) < kSMs * 4)
-                splits = cand;
+    int64_t best = INT64_MAX;
+    for (int cand = 1; cand <= kTcMaxSplit && cand * kTcGroups <= kblocks + kTcGroups - 1; cand *= 2) {
+        const int64_t cost = (((int64_t)grid * cand + kSMs - 1) / kSMs) * ((kblocks + cand - 1) / cand + 6);
+        if (cost < best) best = cost, splits = cand;
     }
-    float* out = splits > 1 ? static_cast<float*>(d_ws) : d_y;
-    const dim3 g(grid, splits);
-    const int per = kblocks / splits;
     int rc, block_shift = 0;
     while ((1 << block_shift) < block_size) ++block_shift;
-    CUtensorMap x_map;
-    if ((rc = make_x_map(d_x, cols, n_rhs, &x_map))) return rc;
-    if (scale_dtype == BOF4_F32) {
-        constexpr auto kern = gemm_tc_kernel<F32>;
-        if ((rc = ensure_dynamic_smem<kern>(kTcSmem))) return rc;
-        kern<<<g, kTcThreads, kTcSmem, st>>>(d_codes, d_scales, cols, block_shift, d_codebook, x_map, n_rhs, out, per,
-                                             d_status);
-    } else {
-        constexpr auto kern = gemm_tc_kernel<BF16>;
-        if ((rc = ensure_dynamic_smem<kern>(kTcSmem))) return rc;
-        kern<<<g, kTcThreads, kTcSmem, st>>>(d_codes, d_scales, cols, block_shift, d_codebook, x_map, n_rhs, out, per,
-                                             d_status);
+    CUtensorMap x_map, code_map;
+    if ((rc = make_map(d_x, false, cols, n_rhs, n_rhs, &x_map)) || (rc = make_map(d_codes, true, cols / 2, rows, kTcM, &code_map)))
+        return rc;
+    const bool list = opq && capacity > 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, splits);
+    cfg.blockDim = dim3(tc_threads(list));
+    cfg.dynamicSmemBytes = kTcSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = (unsigned)splits;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const uint16_t* val = static_cast<const uint16_t*>(d_out_val);
+#define BOF4_TC_GO(ST_, HALF_, OPQ_)                                                                                        \
+    {                                                                                                                       \
+        constexpr auto kern = gemm_tc_kernel<ST_, HALF_, OPQ_>;                                                             \
+        if ((rc = ensure_dynamic_smem<kern>(kTcSmem))) return rc;                                                           \
+        BOF4_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, code_map, d_scales, cols, block_shift, d_codebook, x_map, n_rhs, d_y,  \
+                                         d_status, d_out_idx, val, d_n_out, capacity));                                     \
     }
-    BOF4_CUDA_TRY(cudaGetLastError());
-    if (splits > 1) {
-        gemm_tc_reduce_kernel<<<kSMs * 4, 256, 0, st>>>(out, splits, (int64_t)rows * n_rhs, d_y);
-        BOF4_CUDA_TRY(cudaGetLastError());
+#define BOF4_TC_ST(ST_)                                                             \
+    if (block_size == 32) {                                                         \
+        if (list) BOF4_TC_GO(ST_, true, true) else BOF4_TC_GO(ST_, true, false)     \
+    } else {                                                                        \
+        if (list) BOF4_TC_GO(ST_, false, true) else BOF4_TC_GO(ST_, false, false)   \
     }
-    if (opq && capacity > 0) {
-        const uint16_t* val = static_cast<const uint16_t*>(d_out_val);
-        const uint16_t* xb = static_cast<const uint16_t*>(d_x);
-        if (scale_dtype == BOF4_F32)
-            gemm_tc_outlier_kernel<F32><<<kSMs * 4, 256, 0, st>>>(d_codes, d_scales, rows, cols, block_shift, d_codebook, xb,
-                                                                  n_rhs, d_out_idx, val, d_n_out, capacity, d_y);
-        else
-            gemm_tc_outlier_kernel<BF16><<<kSMs * 4, 256, 0, st>>>(d_codes, d_scales, rows, cols, block_shift, d_codebook, xb,
-                                                                   n_rhs, d_out_idx, val, d_n_out, capacity, d_y);
-        BOF4_CUDA_TRY(cudaGetLastError());
-    }
+    if (scale_dtype == BOF4_F32) { BOF4_TC_ST(F32) } else { BOF4_TC_ST(BF16) }
+#undef BOF4_TC_ST
+#undef BOF4_TC_GO
     return BOF4_OK;
 }
