@@ -351,8 +351,10 @@ BOF4_API int bof4_gemv(const uint8_t* d_codes, const void* d_scales, int scale_d
  *   d_y        device, fp32 [rows][n_rhs], written
  *   d_status   device int, written: 0, or 1 when a bounded wait inside the kernel ran out (the result
  *              is then undefined; the kernel has still released its tensor memory and returned)
- *   d_ws, ws_bytes   not used (may be NULL, 0): matrices with few 128-row tiles are split along K over the
- *              CTAs of a cluster, which sum their partial products in a fixed order
+ *   d_ws       optional device workspace (16-byte aligned, any contents), or NULL: with it the work is cut evenly
+ *              over the SMs along rows and K (rows / 16 + 256 + 151552 n_rhs bytes serve every shape; with less,
+ *              fewer CTAs run) and the parts of a row tile are summed in a fixed order; without it every
+ *              128-row tile is one CTA's
  * One launch on `stream`; no synchronisation.
  */
 BOF4_API int bof4_gemm_tc(const uint8_t* d_codes, const void* d_scales, int scale_dtype, int64_t rows,

@@ -445,9 +445,8 @@ def bof4_gemm_tc(codes: torch.Tensor, scales: torch.Tensor, rows: int, cols: int
                  x: torch.Tensor, workspace: Optional[torch.Tensor] = None, split: bool = True,
                  outliers: Optional[Tuple[torch.Tensor, torch.Tensor, torch.Tensor]] = None):
     """Y fp32 [rows, n_rhs] = W_q X^T on the tensor cores for x bf16 [n_rhs, cols].
-    -> (y, status int32[1]); status 0 unless a bounded wait inside the kernel ran out.  The split along K
-    needs no workspace: `workspace` and `split` are accepted and not used."""
-    return _native().gemm_tc(codes, scales, rows, cols, block_size, levels, x, outliers)
+    -> (y, status int32[1]); status 0 unless a bounded wait inside the kernel ran out."""
+    return _native().gemm_tc(codes, scales, rows, cols, block_size, levels, x, workspace, split, outliers)
 
 
 def bof4_outlier_count(n_out: torch.Tensor, capacity: int) -> int:

@@ -305,7 +305,7 @@ PyObject* gemv(PyObject* const* a)
     return wrap(out);
 }
 
-// (codes, scales, rows, cols, block_size, levels, x, outliers)
+// (codes, scales, rows, cols, block_size, levels, x, workspace, split, outliers)
 PyObject* gemm_tc(PyObject* const* a)
 {
     const at::Tensor &codes = dev(a[0], "codes"), &scales = dev(a[1], "scales"), &x = dev(a[6], "x");
@@ -318,11 +318,16 @@ PyObject* gemm_tc(PyObject* const* a)
     const at::Tensor cb = codebook(a[5], d);
     const at::Tensor y = make(rows * n_rhs, at::kFloat, d).view({rows, n_rhs});
     const at::Tensor status = make(1, at::kInt, d, rows == 0);  // written by the call, unless there is nothing to do
-    const Outliers o(a[7]);
+    at::Tensor ws;
+    if (!none(a[7]))
+        ws = tensor(a[7], "workspace");
+    else if (PyObject_IsTrue(a[8]))
+        ws = make(rows / 16 + 256 + 148 * 2 * 128 * 4 * n_rhs, at::kByte, d);  // tickets; two parts of tiles per SM
+    const Outliers o(a[9]);
     check(bof4_gemm_tc(static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), rows,
                        cols, (int)integer(a[4]), levels_ptr(cb), x.const_data_ptr(), (int)n_rhs, o.idx, o.val, o.cnt, o.cap,
                        static_cast<float*>(y.data_ptr()), static_cast<int*>(status.data_ptr()),
-                       nullptr, 0, stream_of(d)));
+                       ws.defined() ? ws.data_ptr() : nullptr, ws.defined() ? (size_t)ws.numel() : 0, stream_of(d)));
     Ref ry(wrap(y)), rs(wrap(status));
     return PyTuple_Pack(2, ry.p, rs.p);
 }
@@ -557,7 +562,7 @@ PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n)
 #define BOF4_ENTRY(name, n) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&entry<name, n>)), METH_FASTCALL, nullptr}
 PyMethodDef g_methods[] = {
     BOF4_ENTRY(set_hooks, 2), BOF4_ENTRY(set_allocator, 1), BOF4_ENTRY(quantize, 6), BOF4_ENTRY(dequantize, 8),
-    BOF4_ENTRY(gemv, 9), BOF4_ENTRY(gemm_tc, 8), BOF4_ENTRY(quantize_opq, 9), BOF4_ENTRY(outlier_count, 2),
+    BOF4_ENTRY(gemv, 9), BOF4_ENTRY(gemm_tc, 10), BOF4_ENTRY(quantize_opq, 9), BOF4_ENTRY(outlier_count, 2),
     BOF4_ENTRY(quantize_batch, 6), BOF4_ENTRY(dequantize_batch, 7), BOF4_ENTRY(scales_compress, 2), BOF4_ENTRY(scales_expand, 3),
     BOF4_ENTRY(fit_codebook, 10), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_bof4_torch", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};

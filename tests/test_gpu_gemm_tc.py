@@ -128,3 +128,29 @@ def test_gemm_tc_argument_errors(bof4):
         c = torch.zeros(rows * cols // 2, dtype=torch.uint8, device="cuda")
         with pytest.raises(bof4.Bof4Error):
             bof4.bof4_gemm_tc(c, scales, rows, cols, 32 if cols % 64 else 64, lv, x)
+
+
+@pytest.mark.parametrize("rows,cols,n_rhs,I", [(128, 64, 64, 32), (128, 16384, 16, 64), (640, 4160, 32, 64), (3840, 320, 48, 64),
+                                               (19072, 256, 16, 256)])
+def test_work_cut_at_tile_edges(bof4, rows, cols, n_rhs, I):
+    """Parts of one to 148 CTAs that begin and end inside a row tile, rows whose last line of 256 columns is not
+    full, and outlier lists from empty to every weight (more than a batch holds), integer-valued: bit for bit,
+    whatever the workspace held before."""
+    lv, codes, scales, X = _exact_case(rows, cols, n_rhs, I, rows + cols)
+    args = (torch.from_numpy(codes).cuda(), torch.from_numpy(scales).cuda(), rows, cols, I, lv, torch.from_numpy(X).to(torch.bfloat16).cuda())
+    rng = np.random.default_rng(cols)
+    W = lv[np.stack([codes >> 4, codes & 15], 1).reshape(-1)].astype(np.float64) * np.repeat(scales.astype(np.float64), I)
+    ws = torch.full((rows // 16 + 256 + 151552 * n_rhs,), 255, dtype=torch.uint8, device="cuda")
+    for share in (0.0, 1e-3, 1.0 if rows * cols < 200000 else 0.05):
+        k = int(rows * cols * share)
+        idx = np.sort(rng.choice(rows * cols, k, replace=False)) if share < 1 else np.arange(rows * cols)
+        val = rng.integers(-2, 3, idx.size).astype(np.float32)
+        dense = W.copy()
+        dense[idx] = val
+        ref = dense.reshape(rows, cols) @ X.astype(np.float64).T
+        out = (torch.from_numpy(idx.astype(np.int32)).cuda(), torch.from_numpy(val).to(torch.bfloat16).cuda(),
+               torch.tensor([idx.size], dtype=torch.int64, device="cuda"))
+        for kw in ({}, {"workspace": ws}, {"split": False}):
+            y, status = bof4.bof4_gemm_tc(*args, outliers=out if idx.size else None, **kw)
+            assert int(status.item()) == 0
+            assert np.array_equal(y.cpu().numpy().astype(np.float64), ref), (share, list(kw))
