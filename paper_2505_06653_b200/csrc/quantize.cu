@@ -37,6 +37,62 @@ __device__ __forceinline__ void store_scale<BF16>(void* scales, int64_t b, float
     static_cast<uint16_t*>(scales)[b] = (uint16_t)(__float_as_uint(m) >> 16);  // exact: m is a bf16 value
 }
 
+// ---------------------------------------------------------------- short last block
+//
+// A tensor whose size is not a multiple of the block size ends in a shorter block.  It is one more "row"
+// of its tensor, taken by the CTA whose turn it is (a launch of its own cost 4 us, as much as a small
+// tensor): a thread owns up to four pairs of weights, the same arithmetic element by element.
+template <class DT>
+__device__ __forceinline__ float tail_load(const void* w, int64_t k);
+template <>
+__device__ __forceinline__ float tail_load<F32>(const void* w, int64_t k)
+{
+    return static_cast<const float*>(w)[k];
+}
+template <>
+__device__ __forceinline__ float tail_load<BF16>(const void* w, int64_t k)
+{
+    return __uint_as_float((uint32_t)static_cast<const uint16_t*>(w)[k] << 16);
+}
+
+template <class DT, bool SIGNED, class ST>
+__device__ __noinline__ void quantize_tail(const void* __restrict__ w, int64_t first, int len, const float* s_xi,
+                                           uint8_t* __restrict__ codes, void* __restrict__ scales, int64_t scale_index)
+{
+    constexpr int PAIRS = 4096 / 2 / kQThreads;
+    __shared__ unsigned long long s_red[kQThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    float v[2 * PAIRS];
+    unsigned long long best = 0ull;  // largest magnitude, lowest index on ties (Eq. 1 / Eq. 4)
+#pragma unroll
+    for (int k = 0; k < 2 * PAIRS; ++k) {
+        const int i = 2 * (tid + (k >> 1) * kQThreads) + (k & 1);
+        v[k] = i < len ? tail_load<DT>(w, first + i) : 0.0f;
+        const float a = fabsf(v[k]);
+        if (a > 0.0f) best = max(best, ((unsigned long long)__float_as_uint(a) << 32) | (0xffffffffu - (uint32_t)i));
+    }
+#pragma unroll
+    for (int off = 16; off; off >>= 1) best = max(best, __shfl_xor_sync(kFull, best, off));
+    __syncthreads();  // s_red may still be read from the previous tensor's block
+    if (lane == 0) s_red[tid >> 5] = best;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kQThreads / 32; ++k) best = max(best, s_red[k]);
+    float m = 0.0f;
+    if (best) {
+        m = tail_load<DT>(w, first + (int64_t)(0xffffffffu - (uint32_t)best));
+        if (!SIGNED) m = fabsf(m);
+    }
+    if (tid == 0) store_scale<ST>(scales, scale_index, m);
+#pragma unroll
+    for (int k = 0; k < PAIRS; ++k) {
+        const int j = tid + k * kQThreads;
+        if (2 * j >= len) continue;
+        const int hi = region_of(normalise(v[2 * k], m), s_xi), lo = region_of(normalise(v[2 * k + 1], m), s_xi);
+        codes[first / 2 + j] = (uint8_t)((hi << 4) | (2 * j + 1 < len ? lo : 0));
+    }
+}
+
 // Region setup shared by the quantising kernels: thresholds, levels and the one-probe table.
 struct QuantTables {
     float* xi;
@@ -118,6 +174,44 @@ __device__ __forceinline__ void quantize_row(const float (&v)[kLaneW], float mx,
     }
 }
 
+// Several tensors in one launch: the tables are built once per CTA, and the rows of all tensors
+// (a short last block counts as a row) are dealt round-robin over the CTAs as if they were one tensor
+// (tensor t starts with the CTA that follows the last row of tensor t - 1), so that small tensors
+// neither pay for a launch and a table build each nor leave part of the grid idle.
+constexpr int kQBatch = 64;  // tensors per launch (kernel parameter table)
+struct QuantBatch {
+    const void* w[kQBatch];
+    uint8_t* codes[kQBatch];
+    void* scales[kQBatch];
+    int64_t n[kQBatch];
+    int start[kQBatch];  // CTA that takes the tensor's first row
+    int count;
+};
+
+// The rows r0, r0 + G, ... of one tensor of n weights (G = CTAs of the grid), its short last block included.
+template <class DT, int I, bool SIGNED, class ST>
+__device__ __forceinline__ void quantize_rows(const void* __restrict__ w, int64_t n, uint8_t* __restrict__ codes,
+                                              void* __restrict__ scales, const int r0, const QuantTables& T,
+                                              uint32_t lut_base, WideScratch* ws)
+{
+    const int lane = threadIdx.x & 31, G = gridDim.x, tail = (int)(n & (I - 1));
+    const RowMap map(n - tail, kQRow, threadIdx.x);
+    int r = r0;
+    if (r < map.rows) {
+        RawRow<DT> raw = map.ok(r) ? load_raw<DT>(w, map.idx(r)) : zero_raw<DT>();
+        for (; r < map.rows; r += G) {
+            const int rn = r + G;
+            const RawRow<DT> next = map.ok(rn) ? load_raw<DT>(w, map.idx(rn)) : zero_raw<DT>();
+            float v[kLaneW], mx, mn;
+            widen(raw, v);
+            lane_minmax(v, mx, mn);
+            quantize_row<DT, I, SIGNED, ST>(v, mx, mn, map.idx(r), map.ok(r), T, lut_base, lane, codes, scales, ws);
+            raw = next;
+        }
+    }
+    if (tail && r == map.rows) quantize_tail<DT, SIGNED, ST>(w, n - tail, tail, T.xi, codes, scales, n / I);
+}
+
 template <class DT, int I, bool SIGNED, class ST>
 __global__ void __launch_bounds__(kQThreads, kQCtasPerSm)
 quantize_kernel(const void* __restrict__ w, int64_t n, const float* __restrict__ levels,
@@ -128,22 +222,22 @@ quantize_kernel(const void* __restrict__ w, int64_t n, const float* __restrict__
     __shared__ int s_multi;
     __shared__ WideScratch s_wide;
     const QuantTables T = setup_tables(levels, s_xi, s_lv, s_lut, &s_multi);
-    const int lane = threadIdx.x & 31;
-    const uint32_t lut_base = lut_lane_base(s_lut, lane);  // table base of this lane
-    const RowMap map(n, kQRow, threadIdx.x);
-    int r = blockIdx.x;
-    if (r >= map.rows) return;
-    RawRow<DT> raw = map.ok(r) ? load_raw<DT>(w, map.idx(r)) : zero_raw<DT>();
-    for (; r < map.rows; r += gridDim.x) {
-        const int rn = r + gridDim.x;
-        const RawRow<DT> next = map.ok(rn) ? load_raw<DT>(w, map.idx(rn)) : zero_raw<DT>();
-        float v[kLaneW], mx, mn;
-        widen(raw, v);
-        lane_minmax(v, mx, mn);
-        quantize_row<DT, I, SIGNED, ST>(v, mx, mn, map.idx(r), map.ok(r), T, lut_base, lane, codes, scales,
-                                        &s_wide);
-        raw = next;
-    }
+    quantize_rows<DT, I, SIGNED, ST>(w, n, codes, scales, (int)blockIdx.x, T, lut_lane_base(s_lut, threadIdx.x & 31), &s_wide);
+}
+
+template <class DT, int I, bool SIGNED, class ST>
+__global__ void __launch_bounds__(kQThreads, kQCtasPerSm)
+quantize_batch_kernel(const __grid_constant__ QuantBatch B, const float* __restrict__ levels)
+{
+    extern __shared__ __align__(16) unsigned char s_lut[];
+    __shared__ float s_xi[kLevels], s_lv[kLevels];
+    __shared__ int s_multi;
+    __shared__ WideScratch s_wide;
+    const QuantTables T = setup_tables(levels, s_xi, s_lv, s_lut, &s_multi);
+    const int G = gridDim.x;
+    for (int t = 0; t < B.count; ++t)
+        quantize_rows<DT, I, SIGNED, ST>(B.w[t], B.n[t], B.codes[t], B.scales[t], ((int)blockIdx.x + G - B.start[t]) % G, T,
+                                         lut_lane_base(s_lut, threadIdx.x & 31), &s_wide);
 }
 
 // ---------------------------------------------------------------- quantise, bf16 weights
@@ -267,29 +361,17 @@ quantize32_kernel(const void* __restrict__ w, int64_t n, const float* __restrict
 {
     extern __shared__ __align__(16) unsigned char s_lut[];
     __shared__ QuantShared32 S;
-    const RowMap32 map(n, kQRow32, threadIdx.x);
+    const int tail = (int)(n & (I - 1));
+    const RowMap32 map(n - tail, kQRow32, threadIdx.x);
     const int r = blockIdx.x;
-    if (r >= map.rows) return;
     const Raw32 first = map.ok(r) ? load_raw32(w, map.idx(r)) : zero_raw32();  // on its way while the tables are built
     const bool lut_ok = build_tables32(levels, S.xi, S.lv, s_lut, &S.info, [](int base) { return (uint32_t)base; });
     const bool fast_ok = lut_ok && !S.info.tiny;
     const uint32_t lut_base = lut_lane_base(s_lut, threadIdx.x & 31);
-    quantize32_rows<I, SIGNED, ST>(w, n, codes, scales, r, first, fast_ok, lut_base, &S);
+    if (r < map.rows) quantize32_rows<I, SIGNED, ST>(w, n - tail, codes, scales, r, first, fast_ok, lut_base, &S);
+    if (tail && r <= map.rows && (map.rows - r) % (int)gridDim.x == 0)
+        quantize_tail<BF16, SIGNED, ST>(w, n - tail, tail, S.xi, codes, scales, n / I);
 }
-
-// Several tensors in one launch: the tables are built once per CTA, and the rows of all tensors
-// are dealt round-robin over the CTAs as if they were one tensor (tensor t starts with the CTA
-// that follows the last row of tensor t - 1), so that small tensors neither pay for a launch and
-// a table build each nor leave part of the grid idle.
-constexpr int kQBatch = 64;  // tensors per launch (kernel parameter table)
-struct QuantBatch {
-    const void* w[kQBatch];
-    uint8_t* codes[kQBatch];
-    void* scales[kQBatch];
-    int64_t n[kQBatch];
-    int start[kQBatch];  // CTA that takes the tensor's first row
-    int count;
-};
 
 template <int I, bool SIGNED, class ST>
 __global__ void __launch_bounds__(kQThreads, kQCtasPerSm)
@@ -302,13 +384,17 @@ quantize32_batch_kernel(const QuantBatch B, const float* __restrict__ levels)
     const bool fast_ok = lut_ok && !S.info.tiny;
     const uint32_t lut_base = lut_lane_base(s_lut, threadIdx.x & 31);
     for (int t = 0; t < B.count; ++t) {
-        const int64_t n = B.n[t];
+        const int tail = (int)(B.n[t] & (I - 1));
+        const int64_t n = B.n[t] - tail;
         const RowMap32 map(n, kQRow32, threadIdx.x);
         const int r0 = ((int)blockIdx.x + G - B.start[t]) % G;
-        if (r0 >= map.rows) continue;  // uniform over the CTA
         const void* w = B.w[t];
-        const Raw32 first = map.ok(r0) ? load_raw32(w, map.idx(r0)) : zero_raw32();
-        quantize32_rows<I, SIGNED, ST>(w, n, B.codes[t], B.scales[t], r0, first, fast_ok, lut_base, &S);
+        if (r0 < map.rows) {  // uniform over the CTA
+            const Raw32 first = map.ok(r0) ? load_raw32(w, map.idx(r0)) : zero_raw32();
+            quantize32_rows<I, SIGNED, ST>(w, n, B.codes[t], B.scales[t], r0, first, fast_ok, lut_base, &S);
+        }
+        if (tail && r0 <= map.rows && (map.rows - r0) % G == 0)
+            quantize_tail<BF16, SIGNED, ST>(w, n, tail, S.xi, B.codes[t], B.scales[t], n / I);
     }
 }
 
@@ -350,12 +436,32 @@ __device__ __forceinline__ void build_pair_table(const float* __restrict__ level
     __syncthreads();
 }
 
+template <class ST, class OT>
+__device__ __forceinline__ void dequantize_tail(const uint8_t* __restrict__ codes, const void* __restrict__ scales,
+                                                int64_t first, int len, int64_t scale_index, const unsigned char* s_tab,
+                                                void* __restrict__ out)
+{
+    const float m = load_scale<ST>(scales, scale_index);
+    for (int i = threadIdx.x; i < len; i += kDThreads) {
+        const int64_t k = first + i;
+        const float2 lv = *reinterpret_cast<const float2*>(s_tab + (size_t)codes[k >> 1] * 256 + (threadIdx.x & 31u) * 8u);
+        const float v = __fmul_rn(m, (k & 1) ? lv.y : lv.x);
+        if (OT::code == BF16::code)
+            static_cast<uint16_t*>(out)[k] = (uint16_t)bf16_rne(v);
+        else
+            static_cast<float*>(out)[k] = v;
+    }
+}
+
 template <class ST, class OT, int I>
 __device__ __forceinline__ void dequantize_rows(const uint8_t* __restrict__ codes, const void* __restrict__ scales,
                                                 int64_t n, void* __restrict__ out, const unsigned char* s_tab, const int r0)
 {
+    const int tail = (int)(n & (I - 1));  // the short last block: one more row
+    n -= tail;
     const int64_t rows = (n + kDRow - 1) / kDRow;
     int64_t r = r0;
+    if (tail && rows >= r0 && (rows - r0) % gridDim.x == 0) dequantize_tail<ST, OT>(codes, scales, n, tail, n / I, s_tab, out);
     if (r >= rows) return;
     const uint32_t lane8 = (threadIdx.x & 31u) * 8u;
     // n is a multiple of 32, so a lane's 32 outputs are all inside the tensor or all outside
@@ -898,26 +1004,14 @@ using namespace bof4;
 
 // ================================================================= ragged last block
 //
-// A tensor whose size is not a multiple of the block size ends in a shorter block.  It is handled
-// by one CTA with plain loops (fewer than 4096 weights): the same arithmetic as the streaming
+// The OPQ calls handle the short last block by one CTA with plain loops (fewer than 4096 weights)
+// after the list of the whole blocks is complete: the same arithmetic as the streaming
 // kernels, written out element by element.  The block is its own unit: its own maximum, its own
 // mean and deviation over its own length; the two tree sums pad it with zeros to the next power
 // of two (neighbours first, as everywhere); a code byte with a single weight has a zero low nibble.
 
 constexpr int kTailThreads = 256;
 
-template <class DT>
-__device__ __forceinline__ float tail_load(const void* w, int64_t k);
-template <>
-__device__ __forceinline__ float tail_load<F32>(const void* w, int64_t k)
-{
-    return static_cast<const float*>(w)[k];
-}
-template <>
-__device__ __forceinline__ float tail_load<BF16>(const void* w, int64_t k)
-{
-    return __uint_as_float((uint32_t)static_cast<const uint16_t*>(w)[k] << 16);
-}
 template <class DT>
 __device__ __forceinline__ void tail_store(void* w, int64_t k, float v);  // v is exact in DT
 template <>
@@ -945,7 +1039,7 @@ __device__ __forceinline__ void tail_tree_sum(float* s_t, int P)
 // OPQ: outlier split (Sec. 3.3) of the block, appended to the list after the whole blocks'
 // outliers; QUANT: block constant, codes and scale.  first = flat index of the block's first
 // weight (a multiple of the block size), len = its length.
-template <class DT, bool SIGNED, class ST, bool QUANT, bool OPQ>
+template <class DT, bool SIGNED, class ST, bool QUANT>
 __global__ void __launch_bounds__(kTailThreads)
 tail_block_kernel(const void* __restrict__ w, int64_t first, int len, const float* __restrict__ levels,
                   float tau, uint8_t* __restrict__ codes, void* __restrict__ scales, int64_t scale_index,
@@ -959,7 +1053,7 @@ tail_block_kernel(const void* __restrict__ w, int64_t first, int len, const floa
     const int tid = threadIdx.x;
     for (int i = tid; i < len; i += kTailThreads) s_w[i] = tail_load<DT>(w, first + i);
     __syncthreads();
-    if (OPQ) {
+    {
         int P = 1;
         while (P < len) P <<= 1;
         for (int i = tid; i < P; i += kTailThreads) s_t[i] = (i < len) ? s_w[i] : 0.0f;
@@ -1015,25 +1109,6 @@ tail_block_kernel(const void* __restrict__ w, int64_t first, int len, const floa
             codes[first / 2 + k] = (uint8_t)((s_c[2 * k] << 4) | ((2 * k + 1 < len) ? s_c[2 * k + 1] : 0));
     }
 }
-
-template <class ST, class OT>
-__global__ void __launch_bounds__(kTailThreads)
-tail_dequantize_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t first, int len,
-                       int64_t scale_index, const float* __restrict__ levels, void* __restrict__ out)
-{
-    const float m = load_scale<ST>(scales, scale_index);
-    for (int i = threadIdx.x; i < len; i += kTailThreads) {
-        const int64_t k = first + i;
-        const uint32_t byte = codes[k >> 1];
-        const uint32_t c = (k & 1) ? (byte & 15u) : (byte >> 4);
-        const float v = __fmul_rn(m, levels[c]);
-        if (OT::code == BF16::code)
-            static_cast<uint16_t*>(out)[k] = (uint16_t)bf16_rne(v);
-        else
-            static_cast<float*>(out)[k] = v;
-    }
-}
-
 
 int grid_for(int64_t rows, int per_sm)
 {
@@ -1130,36 +1205,24 @@ extern "C" int bof4_quantize(const void* d_w, int w_dtype, int64_t n, int block_
     if ((rc = check_aligned("bof4_quantize", "d_w", d_w)) || (rc = check_aligned("bof4_quantize", "d_codes", d_codes)))
         return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int tail = (int)(n % block_size);  // a ragged last block goes to its own small kernel
-    const int64_t n_whole = n - tail;
-    n = n_whole;
-    if (n > 0) {
-        if (w_dtype == BOF4_BF16) {
-            const int grid = grid_for((n + kQRow32 - 1) / kQRow32, kQCtasPerSm);
-            BOF4_DISPATCH_ST(scale_dtype,
-                BOF4_DISPATCH_I(block_size,
-                    BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
-                        { constexpr auto kern = quantize32_kernel<I_, SG, ST>;
-                          if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                          kern<<<grid, kQThreads, kLutBytes, st>>>(d_w, n, d_codebook, d_codes, d_scales); })));
-        } else {
-            const int grid = grid_for((n + kQRow - 1) / kQRow, kQCtasPerSm);
+    const int64_t n_whole = n - n % block_size, more = n > n_whole ? 1 : 0;  // a short last block is one more row
+    if (w_dtype == BOF4_BF16) {
+        const int grid = grid_for((n_whole + kQRow32 - 1) / kQRow32 + more, kQCtasPerSm);
+        BOF4_DISPATCH_ST(scale_dtype,
             BOF4_DISPATCH_I(block_size,
                 BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
-                    { constexpr auto kern = quantize_kernel<F32, I_, SG, F32>;
+                    { constexpr auto kern = quantize32_kernel<I_, SG, ST>;
                       if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                      kern<<<grid, kQThreads, kLutBytes, st>>>(d_w, n, d_codebook, d_codes, d_scales); }));
-        }
-        BOF4_CUDA_TRY(cudaGetLastError());
-    }
-    if (tail) {
-        BOF4_DISPATCH_WS(w_dtype, scale_dtype,
+                      kern<<<grid, kQThreads, kLutBytes, st>>>(d_w, n, d_codebook, d_codes, d_scales); })));
+    } else {
+        const int grid = grid_for((n_whole + kQRow - 1) / kQRow + more, kQCtasPerSm);
+        BOF4_DISPATCH_I(block_size,
             BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
-                (tail_block_kernel<DT, SG, ST, true, false><<<1, kTailThreads, 0, st>>>(
-                    d_w, n_whole, tail, d_codebook, 0.0f, d_codes, d_scales, n_whole / block_size, nullptr, nullptr,
-                    nullptr, 0, nullptr))));
-        BOF4_CUDA_TRY(cudaGetLastError());
+                { constexpr auto kern = quantize_kernel<F32, I_, SG, F32>;
+                  if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
+                  kern<<<grid, kQThreads, kLutBytes, st>>>(d_w, n, d_codebook, d_codes, d_scales); }));
     }
+    BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;
 }
 
@@ -1193,21 +1256,14 @@ extern "C" int bof4_dequantize(const uint8_t* d_codes, const void* d_scales, int
     if ((rc = check_aligned("bof4_dequantize", "d_codes", d_codes)) || (rc = check_aligned("bof4_dequantize", "d_out", d_out)))
         return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int tail = (int)(n % block_size);  // a ragged last block goes to its own small kernel
-    const int64_t n_whole = n - tail;
-    const int64_t rows = (n_whole + kDRow - 1) / kDRow;
+    const int64_t n_whole = n - n % block_size;
+    const int64_t rows = (n_whole + kDRow - 1) / kDRow + (n > n_whole ? 1 : 0);  // a short last block is one more row
     const int grid = grid_for(rows, kDCtasPerSm);
 #define BOF4_DEQ(ST_, OT_)                                                                                   \
-    {                                                                                                        \
-        if (n_whole > 0)                                                                                     \
-            BOF4_DISPATCH_I(block_size, {                                                                    \
-                constexpr auto kern = dequantize_kernel<ST_, OT_, I_>;                                       \
-                if ((rc = ensure_dynamic_smem<kern>(kDTableBytes))) return rc;                               \
-                kern<<<grid, kDThreads, kDTableBytes, st>>>(d_codes, d_scales, n_whole, d_codebook, d_out); })  \
-        if (tail)                                                                                            \
-            tail_dequantize_kernel<ST_, OT_><<<1, kTailThreads, 0, st>>>(d_codes, d_scales, n_whole, tail,   \
-                                                                         n_whole / block_size, d_codebook, d_out); \
-    }
+    BOF4_DISPATCH_I(block_size, {                                                                            \
+        constexpr auto kern = dequantize_kernel<ST_, OT_, I_>;                                               \
+        if ((rc = ensure_dynamic_smem<kern>(kDTableBytes))) return rc;                                       \
+        kern<<<grid, kDThreads, kDTableBytes, st>>>(d_codes, d_scales, n, d_codebook, d_out); })
     if (scale_dtype == BOF4_F32 && out_dtype == BOF4_F32) { BOF4_DEQ(F32, F32) }
     else if (scale_dtype == BOF4_F32) { BOF4_DEQ(F32, BF16) }
     else if (out_dtype == BOF4_F32) { BOF4_DEQ(BF16, F32) }
@@ -1225,8 +1281,7 @@ extern "C" int bof4_dequantize(const uint8_t* d_codes, const void* d_scales, int
     return BOF4_OK;
 }
 
-// Many tensors per launch.  bf16 weights whose whole blocks go through the batch kernels, kQBatch
-// tensors per launch; fp32 weights and short last blocks take the single-tensor path.
+// Many tensors per launch, kQBatch of them.
 extern "C" int bof4_quantize_batch(const void* const* h_w, const int64_t* h_n, int n_tensors, int w_dtype,
                                    int block_size, int norm, const float* d_codebook, uint8_t* const* h_codes,
                                    void* const* h_scales, int scale_dtype, void* stream)
@@ -1252,52 +1307,43 @@ extern "C" int bof4_quantize_batch(const void* const* h_w, const int64_t* h_n, i
         if ((rc = check_aligned(fn, "a weight tensor", h_w[t])) || (rc = check_aligned(fn, "a code array", h_codes[t])))
             return rc;
     }
-    if (w_dtype != BOF4_BF16) {
-        for (int t = 0; t < n_tensors; ++t)
-            if ((rc = bof4_quantize(h_w[t], w_dtype, h_n[t], block_size, norm, d_codebook, h_codes[t], h_scales[t],
-                                    scale_dtype, stream)))
-                return rc;
-        return BOF4_OK;
-    }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     QuantBatch B;
     B.count = 0;
     int64_t rows = 0;
     const int G = kSMs * kQCtasPerSm;
+    const int64_t row = w_dtype == BOF4_BF16 ? kQRow32 : kQRow;
     for (int t = 0; t <= n_tensors; ++t) {
-        if (t < n_tensors) {
+        if (t < n_tensors && h_n[t] > 0) {
             const int64_t n_whole = h_n[t] - h_n[t] % block_size;
-            if (n_whole > 0) {
-                B.w[B.count] = h_w[t];
-                B.codes[B.count] = h_codes[t];
-                B.scales[B.count] = h_scales[t];
-                B.n[B.count] = n_whole;
-                B.start[B.count] = (int)(rows % G);
-                rows += (n_whole + kQRow32 - 1) / kQRow32;
-                ++B.count;
-            }
+            B.w[B.count] = h_w[t];
+            B.codes[B.count] = h_codes[t];
+            B.scales[B.count] = h_scales[t];
+            B.n[B.count] = h_n[t];
+            B.start[B.count] = (int)(rows % G);
+            rows += (n_whole + row - 1) / row + (h_n[t] > n_whole ? 1 : 0);
+            ++B.count;
         }
         if (B.count == kQBatch || (t == n_tensors && B.count > 0)) {
-            BOF4_DISPATCH_ST(scale_dtype,
+            const int grid = (int)(rows < G ? rows : G);  // start[] was taken modulo G: the same for fewer rows
+            if (w_dtype == BOF4_BF16) {
+                BOF4_DISPATCH_ST(scale_dtype,
+                    BOF4_DISPATCH_I(block_size,
+                        BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
+                            { constexpr auto kern = quantize32_batch_kernel<I_, SG, ST>;
+                              if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
+                              kern<<<grid, kQThreads, kLutBytes, st>>>(B, d_codebook); })));
+            } else {
                 BOF4_DISPATCH_I(block_size,
                     BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
-                        { constexpr auto kern = quantize32_batch_kernel<I_, SG, ST>;
+                        { constexpr auto kern = quantize_batch_kernel<F32, I_, SG, F32>;
                           if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                          kern<<<G, kQThreads, kLutBytes, st>>>(B, d_codebook); })));
+                          kern<<<grid, kQThreads, kLutBytes, st>>>(B, d_codebook); }));
+            }
             BOF4_CUDA_TRY(cudaGetLastError());
             B.count = 0;
+            rows = 0;
         }
-    }
-    for (int t = 0; t < n_tensors; ++t) {
-        const int tail = (int)(h_n[t] % block_size);
-        if (!tail) continue;
-        const int64_t n_whole = h_n[t] - tail;
-        BOF4_DISPATCH_ST(scale_dtype,
-            BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
-                (tail_block_kernel<BF16, SG, ST, true, false><<<1, kTailThreads, 0, st>>>(
-                    h_w[t], n_whole, tail, d_codebook, 0.0f, h_codes[t], h_scales[t], n_whole / block_size, nullptr,
-                    nullptr, nullptr, 0, nullptr))));
-        BOF4_CUDA_TRY(cudaGetLastError());
     }
     return BOF4_OK;
 }
@@ -1336,23 +1382,22 @@ extern "C" int bof4_dequantize_batch(const uint8_t* const* h_codes, const void* 
     int64_t rows = 0;
     const int G = kSMs * kDCtasPerSm;
     for (int t = 0; t <= n_tensors; ++t) {
-        if (t < n_tensors) {
+        if (t < n_tensors && h_n[t] > 0) {
             const int64_t n_whole = h_n[t] - h_n[t] % block_size;
-            if (n_whole > 0) {
-                B.codes[B.count] = h_codes[t];
-                B.scales[B.count] = h_scales[t];
-                B.out[B.count] = h_out[t];
-                B.n[B.count] = n_whole;
-                B.start[B.count] = (int)(rows % G);
-                rows += (n_whole + kDRow - 1) / kDRow;
-                ++B.count;
-            }
+            B.codes[B.count] = h_codes[t];
+            B.scales[B.count] = h_scales[t];
+            B.out[B.count] = h_out[t];
+            B.n[B.count] = h_n[t];
+            B.start[B.count] = (int)(rows % G);
+            rows += (n_whole + kDRow - 1) / kDRow + (h_n[t] > n_whole ? 1 : 0);
+            ++B.count;
         }
         if (B.count == kQBatch || (t == n_tensors && B.count > 0)) {
+            const int grid = (int)(rows < G ? rows : G);  // start[] was taken modulo G: the same for fewer rows
 #define BOF4_DEQB(ST_, OT_) BOF4_DISPATCH_I(block_size, {                                  \
         constexpr auto kern = dequantize_batch_kernel<ST_, OT_, I_>;                       \
         if ((rc = ensure_dynamic_smem<kern>(kDTableBytes))) return rc;                     \
-        kern<<<G, kDThreads, kDTableBytes, st>>>(B, d_codebook); })
+        kern<<<grid, kDThreads, kDTableBytes, st>>>(B, d_codebook); })
             if (scale_dtype == BOF4_F32 && out_dtype == BOF4_F32) { BOF4_DEQB(F32, F32) }
             else if (scale_dtype == BOF4_F32) { BOF4_DEQB(F32, BF16) }
             else if (out_dtype == BOF4_F32) { BOF4_DEQB(BF16, F32) }
@@ -1360,20 +1405,8 @@ extern "C" int bof4_dequantize_batch(const uint8_t* const* h_codes, const void* 
 #undef BOF4_DEQB
             BOF4_CUDA_TRY(cudaGetLastError());
             B.count = 0;
+            rows = 0;
         }
-    }
-    for (int t = 0; t < n_tensors; ++t) {
-        const int tail = (int)(h_n[t] % block_size);
-        if (!tail) continue;
-        const int64_t n_whole = h_n[t] - tail;
-#define BOF4_DEQT(ST_, OT_) tail_dequantize_kernel<ST_, OT_><<<1, kTailThreads, 0, st>>>( \
-        h_codes[t], h_scales[t], n_whole, tail, n_whole / block_size, d_codebook, h_out[t]);
-        if (scale_dtype == BOF4_F32 && out_dtype == BOF4_F32) { BOF4_DEQT(F32, F32) }
-        else if (scale_dtype == BOF4_F32) { BOF4_DEQT(F32, BF16) }
-        else if (out_dtype == BOF4_F32) { BOF4_DEQT(BF16, F32) }
-        else { BOF4_DEQT(BF16, BF16) }
-#undef BOF4_DEQT
-        BOF4_CUDA_TRY(cudaGetLastError());
     }
     return BOF4_OK;
 }
@@ -1476,7 +1509,7 @@ int launch_opq(const char* fn, const void* d_w, int w_dtype, int64_t n, int bloc
     if (tail) {  // after the gather kernel: its outliers follow those of the whole blocks
         BOF4_DISPATCH_WS(w_dtype, scale_dtype,
             BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
-                (tail_block_kernel<DT, SG, ST, QUANT, true><<<1, kTailThreads, 0, st>>>(
+                (tail_block_kernel<DT, SG, ST, QUANT><<<1, kTailThreads, 0, st>>>(
                     d_w, n_whole, tail, d_codebook, tau, d_codes, d_scales, n_whole / block_size, d_w_clean, d_out_idx,
                     out_val, capacity, d_n_out))));
         BOF4_CUDA_TRY(cudaGetLastError());
