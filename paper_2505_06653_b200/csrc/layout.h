@@ -58,7 +58,7 @@ inline uint32_t mae_cand_capacity(size_t ws_bytes)
 // count and a staging slot of kOpqStage outliers; tiles are scanned in chunks of kOpqChunk.
 constexpr int kOpqTile = 512;
 constexpr int kOpqStage = 16;
-constexpr int kOpqChunk = 2048;
+constexpr int kOpqChunk = 512;
 
 struct OpqLayout {
     int64_t tiles, chunks;

@@ -776,6 +776,16 @@ opq_pass1_kernel(const void* __restrict__ w, int64_t n, const float* __restrict_
 // kernel are those of the generic pass.  The two tree sums of the block statistics (App. E) keep
 // the balanced-tree order: neighbours first inside the lane (32 weights, five levels, the upper
 // four on packed pairs), then the lane butterfly, then the warps of a wide block.
+//
+// What bounds it is instructions, not memory, so the exact statistics are computed only where they decide
+// something.  A block within a warp first gets an interval [lo, hi] that contains its threshold, from the sum
+// and the sum of squares in one sweep of packed multiply-adds; a weight outside the interval is decided by it,
+// and a weight inside it (about one warp row in a thousand) sends the row to the exact sums.  A lane whose
+// largest weight is not below lo has its 32 weights put in shared memory, where the warp tests them one per
+// lane: the ballot is the outlier mask in index order, the places of the list follow from its bits, and the
+// cleaned weights and their extremes come back without a loop over all weights in every lane.
+// 28672 x 8192 weights, blocks of 64, 5 % of them with outliers: 225 us with the exact sums and a 32-step
+// outlier loop in every lane, NEWUS us this way; the plain quantiser takes 105.
 
 // Balanced tree sum of the lane's 32 values given as 16 pairs {even, odd}: every addition is a
 // separate fp32 RN operation; levels two to five add two independent partial sums per instruction.
@@ -812,97 +822,281 @@ __device__ __forceinline__ float outlier_threshold32(const uint32_t (&u)[16], fl
     float2 v[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = make_float2(bf_lo(u[k]), bf_hi(u[k]));
-    const float mean = __fmul_rn(block_tree_sum32<I>(lane_tree_sum32(v), ws->a), 1.0f / (float)I);  // exact: I = 2^k
+    const float mean = __fmul_rn(block_tree_sum32<I>(lane_tree_sum32(v), ws ? ws->a : nullptr), 1.0f / (float)I);  // exact: I = 2^k
     const float2 nm = make_float2(-mean, -mean);
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         const float2 d = __fadd2_rn(v[k], nm);
         v[k] = __fmul2_rn(d, d);
     }
-    const float sigma = __fsqrt_rn(__fdiv_rn(block_tree_sum32<I>(lane_tree_sum32(v), ws->b), (float)(I - 1)));
+    const float sigma = __fsqrt_rn(__fdiv_rn(block_tree_sum32<I>(lane_tree_sum32(v), ws ? ws->b : nullptr), (float)(I - 1)));
     return __fmul_rn(sigma, tau);
 }
 
-template <int I, bool SIGNED, class ST, bool QUANT>
-__global__ void __launch_bounds__(kQThreads, kQCtasPerSm)
-opq_pass1_32_kernel(const void* __restrict__ w, int64_t n, const float* __restrict__ levels, float tau,
-                    uint8_t* __restrict__ codes, void* __restrict__ scales, void* __restrict__ w_clean,
-                    int32_t* __restrict__ counts, unsigned long long* __restrict__ chunk_sum,
-                    int32_t* __restrict__ stage_idx, uint16_t* __restrict__ stage_val)
+// An interval [lo, hi] around the threshold of the lane's block (blocks within a warp), or false if this
+// estimate cannot bound it: a block that is zero, not finite, extreme, or whose mean is not small beside its
+// deviation.
+//
+// S = sum w and Q = sum w^2 are summed through at most 15 additions each (eight per partial sum, two to join
+// the four of a lane, five for the lanes), and the square of a bf16 value is exact in fp32, so with
+// e = 2^-24: |dS| <= 15 e sum |w|, |dQ| <= 15 e Q, and by Cauchy-Schwarz S^2 / I is off by at most
+// 30 e Q (plus the rounding of the two operations): V = Q - S^2 / I is off by at most 48 e Q, which is
+// 192 e V where V >= Q / 4.  The deviation is then off by at most 96 e, its square root, products and the
+// exact formula's own roundings (13 e in its sum, 2 e after it) by less than 20 e: less than 2^-17 in all.
+// The interval takes 2^-15 on either side.
+template <int I>
+__device__ __forceinline__ bool outlier_interval32(const uint32_t (&u)[16], float tau, float& lo, float& hi)
 {
-    static_assert(2 * kOpqTile == kWarpW32, "two tiles per warp iteration");
-    extern __shared__ __align__(16) unsigned char s_lut[];
+    static_assert(Geo32<I>::WPB == 1, "blocks within a warp");
+    float2 s0 = make_float2(bf_lo(u[0]), bf_hi(u[0])), s1 = make_float2(bf_lo(u[1]), bf_hi(u[1]));
+    float2 q0 = __fmul2_rn(s0, s0), q1 = __fmul2_rn(s1, s1);
+#pragma unroll
+    for (int k = 2; k < 16; k += 2) {
+        const float2 a = make_float2(bf_lo(u[k]), bf_hi(u[k])), b = make_float2(bf_lo(u[k + 1]), bf_hi(u[k + 1]));
+        s0 = __fadd2_rn(s0, a);
+        q0 = __ffma2_rn(a, a, q0);
+        s1 = __fadd2_rn(s1, b);
+        q1 = __ffma2_rn(b, b, q1);
+    }
+    s0 = __fadd2_rn(s0, s1);
+    q0 = __fadd2_rn(q0, q1);
+    float S = s0.x + s0.y, Q = q0.x + q0.y;
+#pragma unroll
+    for (int off = 1; off < Geo32<I>::LPB; off <<= 1) {
+        S += __shfl_xor_sync(kFull, S, off);
+        Q += __shfl_xor_sync(kFull, Q, off);
+    }
+    const float V = __fmaf_rn(S * (-1.0f / (float)I), S, Q);
+    float sigma;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(sigma) : "f"(V * (1.0f / (float)(I - 1))));
+    const float thr = sigma * tau;
+    lo = thr * (1.0f - 0x1p-15f);
+    hi = thr * (1.0f + 0x1p-15f);
+    return 4.0f * V >= Q && Q > 0x1p-80f && Q < 0x1p80f && thr > 0x1p-80f;
+}
+
+__device__ __forceinline__ float warp_max_nan(float x)
+{
+    float d;
+    asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(x));
+    return d;
+}
+__device__ __forceinline__ float warp_min(float x)
+{
+    float d;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(x));
+    return d;
+}
+
+struct OpqArgs {
+    const void* w;
+    int64_t n;
+    const float* levels;
+    float tau;
+    uint8_t* codes;
+    void *scales, *w_clean;
+    int32_t* counts;
+    unsigned long long* chunk_sum;
+    int32_t* stage_idx;
+    uint16_t* stage_val;
+};
+
+// A row that holds candidates: `cand` marks the lanes with a weight that is not below lo.  Writes the
+// staged outliers, zeroes them in u, replaces the marked lanes' mx and mn by those of the cleaned weights and
+// returns the outliers of lanes 0-15 and 16-31, or x = -1 (nothing done that a second run would not do again)
+// if a weight lies inside its interval.  tile = the warp row's first tile, idx = element index of lane 0.
+__device__ __forceinline__ int2 split_outliers32(uint32_t (&u)[16], unsigned cand, float lo, float hi, float& mx,
+                                                 float& mn, uint32_t s_words, int64_t tile, int64_t idx, int lane,
+                                                 const OpqArgs& A)
+{
+    // 64 bytes of shared memory per lane, its four 16-byte parts swapped about so that eight lanes hit all banks
+    const bool mine = (cand >> lane) & 1u;
+    const uint32_t own = s_words + lane * 64, sw = (lane >> 1) & 3;
+    if (mine) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(own + ((c ^ sw) << 4)), "r"(u[4 * c]),
+                         "r"(u[4 * c + 1]), "r"(u[4 * c + 2]), "r"(u[4 * c + 3])
+                         : "memory");
+    }
+    __syncwarp();
+    int2 found = make_int2(0, 0);
+    unsigned dirty = 0u;
+    for (unsigned left = cand; left; left &= left - 1u) {
+        const int L = __ffs(left) - 1;
+        const uint32_t at = s_words + L * 64 + ((((unsigned)lane >> 3) ^ ((L >> 1) & 3)) << 4) + (lane & 7) * 2;
+        uint32_t bits;
+        asm volatile("{\n\t.reg .u16 t;\n\tld.shared.u16 t, [%1];\n\tcvt.u32.u16 %0, t;\n\t}" : "=r"(bits) : "r"(at) : "memory");
+        const float v = bf_lo(bits), a = fabsf(v);
+        const unsigned o = __ballot_sync(kFull, a > __shfl_sync(kFull, hi, L));
+        if (o != __ballot_sync(kFull, a > __shfl_sync(kFull, lo, L))) return make_int2(-1, 0);
+        if (o == 0u) continue;  // uniform
+        const int half = L >> 4, before = half ? found.y : found.x;
+        if (half)
+            found.y += __popc(o);
+        else
+            found.x += __popc(o);
+        const bool out = (o >> lane) & 1u;
+        if (out) {
+            const int pos = before + __popc(o & ((1u << lane) - 1u));
+            if (pos < kOpqStage) {
+                A.stage_idx[(tile + half) * kOpqStage + pos] = (int32_t)(idx + L * kLW + lane);
+                A.stage_val[(tile + half) * kOpqStage + pos] = (uint16_t)bits;
+            }
+            asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"((unsigned short)0) : "memory");
+        }
+        const float c = out ? 0.0f : v, cmx = warp_max_nan(c), cmn = warp_min(c);
+        if (lane == L) {
+            mx = cmx;
+            mn = cmn;
+        }
+        dirty |= 1u << L;
+    }
+    __syncwarp();
+    if ((dirty >> lane) & 1u) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(u[4 * c]), "=r"(u[4 * c + 1]), "=r"(u[4 * c + 2]), "=r"(u[4 * c + 3])
+                         : "r"(own + ((c ^ sw) << 4))
+                         : "memory");
+    }
+    __syncwarp();  // before the next row's words are put there
+    return found;
+}
+
+// Outlier counts of the warp row's two tiles, and their share of the chunk's (integer: order-free).
+__device__ __forceinline__ void store_counts32(const OpqArgs& A, int2 found, int64_t tile, int lane)
+{
+    if (lane == 0 && found.x + found.y > 0)
+        atomicAdd(&A.chunk_sum[tile / kOpqChunk], (unsigned long long)(found.x + found.y));
+    if (lane < 2 && (tile + lane) * kOpqTile < A.n) A.counts[tile + lane] = lane ? found.y : found.x;
+}
+
+__device__ __forceinline__ void store_clean32(const OpqArgs& A, int64_t idx, const uint32_t (&u)[16])
+{
+    uint16_t* dst = static_cast<uint16_t*>(A.w_clean) + idx;
+    st_stream256(dst, Raw8{{u[0], u[1], u[2], u[3], u[4], u[5], u[6], u[7]}});
+    st_stream256(dst + 16, Raw8{{u[8], u[9], u[10], u[11], u[12], u[13], u[14], u[15]}});
+}
+
+// 24 warps of 80 registers an SM: with 32 of 64, the words of two rows and the candidates' state spill
+// (48 spilled words a row were half of the shared-memory and L1 traffic).
+constexpr int kOThreads = 384;
+constexpr int kORow = kOThreads * kLW;              // weights per CTA row
+constexpr int kOpqWordBytes = kOThreads * kLW * 2;  // shared memory for the weights of one row
+
+// One row with the exact statistics and any kind of weights, block constants or codebook; of blocks wider
+// than a warp every thread of the CTA takes part.
+template <int I, bool SIGNED, class ST, bool QUANT>
+__device__ __forceinline__ void opq_row_exact(const OpqArgs& A, const Raw32& raw, int64_t idx, bool ok, int64_t tile,
+                                              bool fast_ok, uint32_t lut_base, uint32_t s_words, QuantShared32* S)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t u[16];
+    words_of(raw, u);
+    float mx, mn;
+    lane_minmax32(u, mx, mn);
+    const float thr = outlier_threshold32<I>(u, A.tau, &S->wide);
+    const unsigned cand = __ballot_sync(kFull, !(fmaxf(mx, -mn) <= thr));  // a NaN is one, too
+    int2 found = make_int2(0, 0);
+    if (cand) found = split_outliers32(u, cand, thr, thr, mx, mn, s_words, tile, idx - lane * kLW, lane, A);
+    store_counts32(A, found, tile, lane);
+    if constexpr (QUANT)
+        quantize_row32<I, SIGNED, ST>(u, mx, mn, idx, ok, fast_ok, lut_base, S, A.codes, A.scales);
+    else if (A.w_clean != nullptr && ok)
+        store_clean32(A, idx, u);
+}
+
+// The same out of line, reading the row itself: the rows that the loop below leaves out, with nothing of the
+// loop's rows to be kept across the call.
+template <int I, bool SIGNED, class ST, bool QUANT>
+__device__ __noinline__ void opq_row_far(const OpqArgs& A, int64_t idx, bool ok, int64_t tile, bool fast_ok,
+                                         uint32_t lut_base, uint32_t s_words, QuantShared32* S)
+{
+    const Raw32 raw = ok ? load_raw32(A.w, idx) : zero_raw32();
+    opq_row_exact<I, SIGNED, ST, QUANT>(A, raw, idx, ok, tile, fast_ok, lut_base, s_words, S);
+}
+
+template <int I, bool SIGNED, class ST, bool QUANT>
+__global__ void __launch_bounds__(kOThreads, kQCtasPerSm) opq_pass1_32_kernel(const __grid_constant__ OpqArgs A)
+{
+    static_assert(2 * kOpqTile == kWarpW32 && kOpqChunk % 2 == 0, "two tiles of one chunk per warp iteration");
+    extern __shared__ __align__(16) unsigned char s_dyn[];  // candidate words, then the region table
     __shared__ QuantShared32 S;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const RowMap32 map(n, kQRow32, threadIdx.x);
-    const int G = gridDim.x;
+    const RowMap32 map(A.n, kORow, threadIdx.x);
+    const int G = gridDim.x, full = map.rows_full;
     int r = blockIdx.x;
     if (r >= map.rows) return;
-    auto fetch = [&](int rr) { return map.ok(rr) ? load_raw32(w, map.idx(rr)) : zero_raw32(); };
-    Raw32 a = fetch(r);
     bool fast_ok = false;
     uint32_t lut_base = 0u;
+    const uint32_t s_words = (uint32_t)__cvta_generic_to_shared(s_dyn) + warp * (32 * 64);
     if (QUANT) {
-        const bool lut_ok = build_tables32(levels, S.xi, S.lv, s_lut, &S.info, [](int base) { return (uint32_t)base; });
+        const bool lut_ok = build_tables32(A.levels, S.xi, S.lv, s_dyn + kOpqWordBytes, &S.info, [](int base) { return (uint32_t)base; });
         fast_ok = lut_ok && !S.info.tiny;
-        lut_base = lut_lane_base(s_lut, lane);
+        lut_base = lut_lane_base(s_dyn + kOpqWordBytes, lane);
     }
-    for (; r < map.rows; r += G) {
-        const Raw32 next = fetch(r + G);
-        const int64_t idx = map.idx(r);
-        const bool ok = map.ok(r);
-        // this lane's tile: lanes 0-15 the first, lanes 16-31 the second tile of the warp row
-        const int64_t tile = ((int64_t)r * (kQThreads / 32) + warp) * 2 + (lane >> 4);
-        const bool tile_ok = tile * kOpqTile < n;  // uniform over the half warp
-        uint32_t u[16];
-        words_of(a, u);
-        float mx, mn;
-        lane_minmax32(u, mx, mn);
-        const float thr = outlier_threshold32<I>(u, tau, &S.wide);
-        // A lane can only hold an outlier if its largest magnitude exceeds the threshold, so the
-        // per-element test runs only in warps where some lane does (a NaN maximum also enters).
-        const bool maybe = !(fmaxf(mx, -mn) <= thr);
-        int total_half = 0;
-        if (__any_sync(kFull, maybe)) {
-            unsigned o = 0u;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                o |= (fabsf(bf_lo(u[k])) > thr) ? (1u << (2 * k)) : 0u;
-                o |= (fabsf(bf_hi(u[k])) > thr) ? (2u << (2 * k)) : 0u;
+    auto tile_of = [&](int rr) { return ((int64_t)rr * (kOThreads / 32) + warp) * 2; };  // the warp row's first tile
+    if constexpr (Geo32<I>::WPB > 1) {
+        auto fetch = [&](int rr) { return map.ok(rr) ? load_raw32(A.w, map.idx(rr)) : zero_raw32(); };
+        Raw32 a = fetch(r);
+        for (; r < map.rows; r += G) {
+            const Raw32 next = fetch(r + G);
+            opq_row_exact<I, SIGNED, ST, QUANT>(A, a, map.idx(r), map.ok(r), tile_of(r), fast_ok, lut_base, s_words, &S);
+            a = next;
+        }
+    } else {
+        // Whole rows, two buffers used in turn.  False (of the whole warp): a row for the exact way.
+        auto row = [&](const Raw32& raw, int rr) -> bool {
+            uint32_t u[16];
+            words_of(raw, u);
+            float mx, mn, lo, hi;
+            lane_minmax32(u, mx, mn);
+            if (!__all_sync(kFull, outlier_interval32<I>(u, A.tau, lo, hi))) return false;
+            const int64_t idx = map.idx(rr), tile = tile_of(rr);
+            const unsigned cand = __ballot_sync(kFull, !(fmaxf(mx, -mn) <= lo));  // a NaN is one, too
+            int2 found = make_int2(0, 0);
+            if (cand) {
+                found = split_outliers32(u, cand, lo, hi, mx, mn, s_words, tile, idx - lane * kLW, lane, A);
+                if (found.x < 0) return false;
             }
-            if (__any_sync(kFull, o != 0u)) {
-                int total;
-                int pos = warp_excl_scan(__popc(o), lane, total);
-                const int lower = __shfl_sync(kFull, pos, 16);  // outliers of lanes 0-15
-                total_half = (lane >> 4) ? total - lower : lower;
-                if (lane >> 4) pos -= lower;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        if ((o >> (2 * k + h)) & 1u) {
-                            if (pos < kOpqStage) {
-                                stage_idx[tile * kOpqStage + pos] = (int32_t)(idx + 2 * k + h);
-                                stage_val[tile * kOpqStage + pos] = (uint16_t)(h ? (u[k] >> 16) : (u[k] & 0xffffu));
-                            }
-                            ++pos;
-                            u[k] &= h ? 0x0000ffffu : 0xffff0000u;  // the outlier becomes +0
-                        }
-                }
-                if ((lane & 15) == 0 && total_half > 0)
-                    atomicAdd(&chunk_sum[tile / kOpqChunk], (unsigned long long)total_half);  // integer: order-free
-                lane_minmax32(u, mx, mn);  // of the cleaned weights
+            if constexpr (QUANT) {
+                float g;
+                const float m = block_constant32<I, SIGNED>(u, mx, mn, g, nullptr);
+                if (!row_is_fast(g, m, true, fast_ok, &S.info)) return false;
+                uint32_t cw[4];
+                encode32_fast(u, m, lut_base, cw);
+                st_stream128(A.codes + idx / 2, cw[0], cw[1], cw[2], cw[3]);
+                if ((idx & (I - 1)) == 0) store_scale<ST>(A.scales, idx / I, m);
+            } else if (A.w_clean != nullptr) {
+                store_clean32(A, idx, u);
+            }
+            store_counts32(A, found, tile, lane);
+            return true;
+        };
+        while (r < full) {
+            Raw32 a = load_raw32(A.w, map.idx(r)), b = a;
+            bool done = true;
+            while (true) {
+                int rn = r + G;
+                if (rn < full) b = load_raw32(A.w, map.idx(rn));
+                if (!(done = row(a, r))) break;
+                r = rn;
+                if (r >= full) break;
+                rn = r + G;
+                if (rn < full) a = load_raw32(A.w, map.idx(rn));
+                if (!(done = row(b, r))) break;
+                r = rn;
+                if (r >= full) break;
+            }
+            if (!done) {
+                opq_row_far<I, SIGNED, ST, QUANT>(A, map.idx(r), true, tile_of(r), fast_ok, lut_base, s_words, &S);
+                r += G;
             }
         }
-        if ((lane & 15) == 0 && tile_ok) counts[tile] = total_half;
-        if (QUANT) {
-            quantize_row32<I, SIGNED, ST>(u, mx, mn, idx, ok, fast_ok, lut_base, &S, codes, scales);
-        } else if (w_clean != nullptr && ok) {
-            uint16_t* dst = static_cast<uint16_t*>(w_clean) + idx;
-            st_stream256(dst, Raw8{{u[0], u[1], u[2], u[3], u[4], u[5], u[6], u[7]}});
-            st_stream256(dst + 16, Raw8{{u[8], u[9], u[10], u[11], u[12], u[13], u[14], u[15]}});
-        }
-        a = next;
+        if (r == full && full < map.rows)  // the partial last row, by the CTA whose turn it is
+            opq_row_far<I, SIGNED, ST, QUANT>(A, map.idx(full), map.ok(full), tile_of(full), fast_ok, lut_base, s_words, &S);
     }
 }
 
@@ -1471,21 +1665,22 @@ int launch_opq(const char* fn, const void* d_w, int w_dtype, int64_t n, int bloc
         const OpqLayout Lw = opq_layout(n_whole);  // never larger than the layout of n
         const int64_t rows = (n_whole + kQRow - 1) / kQRow;
         const int grid = grid_for(rows, kQCtasPerSm);
-        const int smem = QUANT ? kLutBytes : 0;
+        const int smem = QUANT ? kLutBytes : 0;  // fp32 weights
         counts = reinterpret_cast<int32_t*>(ws + Lw.counts);
         chunk_sum = reinterpret_cast<unsigned long long*>(ws + Lw.chunk_off);
         stage_idx = reinterpret_cast<int32_t*>(ws + Lw.stage_idx);
         stage_val = reinterpret_cast<uint16_t*>(ws + Lw.stage_val);
         BOF4_CUDA_TRY(cudaMemsetAsync(chunk_sum, 0, (size_t)Lw.chunks * 8, st));
         if (w_dtype == BOF4_BF16) {
-            const int grid32 = grid_for((n_whole + kQRow32 - 1) / kQRow32, kQCtasPerSm);
+            const int grid32 = grid_for((n_whole + kORow - 1) / kORow, kQCtasPerSm);
             BOF4_DISPATCH_ST(scale_dtype,
                 BOF4_DISPATCH_I(block_size,
                     BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                         { constexpr auto kern = opq_pass1_32_kernel<I_, SG, ST, QUANT>;
-                          if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                          kern<<<grid32, kQThreads, smem, st>>>(d_w, n_whole, d_codebook, tau, d_codes, d_scales,
-                                                                d_w_clean, counts, chunk_sum, stage_idx, stage_val); })));
+                          constexpr int words = kOpqWordBytes + (QUANT ? kLutBytes : 0);
+                          if ((rc = ensure_dynamic_smem<kern>(words))) return rc;
+                          kern<<<grid32, kOThreads, words, st>>>(OpqArgs{d_w, n_whole, d_codebook, tau, d_codes, d_scales, d_w_clean,
+                                                                         counts, chunk_sum, stage_idx, stage_val}); })));
         } else {
             BOF4_DISPATCH_I(block_size,
                 BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
