@@ -169,6 +169,7 @@ template <int I, bool SIGNED>
 __global__ void __launch_bounds__(1024, 1)
 cells_blocks_kernel(const EmTensors T, const int64_t first_block, uint32_t* __restrict__ hist, uint16_t* __restrict__ consts)
 {
+    if (!after_previous()) return;
     extern __shared__ uint32_t s_hist[];  // [kMags]
     __shared__ WideScratch s_wide;
     __shared__ const void* s_ptr[kEmMaxTensors];
@@ -240,6 +241,7 @@ cells_blocks_kernel(const EmTensors T, const int64_t first_block, uint32_t* __re
 __global__ void __launch_bounds__(1024)
 cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __restrict__ head)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t s_blocks[32], s_units[32], s_top;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) s_top = W.scal[2];
@@ -310,6 +312,7 @@ cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __re
 __global__ void __launch_bounds__(1024, 1)
 cells_order_kernel(const EmTensors T, const int64_t first_block, const int64_t n_blocks, int block_size, const CellsWs W)
 {
+    if (!after_previous()) return;
     extern __shared__ uint32_t s_pos[];  // [kMags]
     __shared__ const char* s_ptr[kEmMaxTensors];
     __shared__ int64_t s_end[kEmMaxTensors];  // first block behind the tensor
@@ -362,6 +365,7 @@ __device__ __forceinline__ void cell_count(uint32_t base, uint32_t w, uint32_t m
 __global__ void __launch_bounds__(kCellThreads, kCellCtas)
 cells_accumulate_kernel(const CellsWs W, int lanes_shift, int metric)
 {
+    if (!after_previous()) return;
     extern __shared__ uint32_t s_cnt[];  // [2 * kCellDepth]
     __shared__ CellUnit s_unit;
     __shared__ uint32_t s_seen[kCellThreads / 32];
@@ -451,6 +455,7 @@ template <bool SIGNED>
 __global__ void __launch_bounds__(kEmTailThreads)
 cells_tail_kernel(const EmTails Q, const CellsWs W, int metric, int add)
 {
+    if (!after_previous()) return;
     __shared__ float s_w[4096];
     __shared__ unsigned long long s_red[kEmTailThreads / 32];
     const bool mae = metric == BOF4_METRIC_MAE || metric == BOF4_METRIC_MAE_NORMALIZED;
@@ -482,6 +487,7 @@ cells_tail_kernel(const EmTails Q, const CellsWs W, int metric, int add)
 __global__ void __launch_bounds__(512)
 cells_scan_kernel(const CellsWs W)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t s_n[16];
     const int tid = threadIdx.x;
     uint32_t n = 0u;
@@ -507,6 +513,7 @@ cells_scan_kernel(const CellsWs W)
 __global__ void __launch_bounds__(512)
 cells_items_kernel(const CellsWs W)
 {
+    if (!after_previous()) return;
     constexpr int PER = kCellScan / 512;
     __shared__ uint32_t s_warp[16], s_before[16];
     __shared__ double s_sum[16];
@@ -570,6 +577,7 @@ cells_items_kernel(const CellsWs W)
 __global__ void __launch_bounds__(320)
 cells_square_kernel(const CellsWs W)
 {
+    if (!after_previous()) return;
     const double* part = reinterpret_cast<const double*>(W.sort.counts);
     for (int k = threadIdx.x; k < kSortParts; k += blockDim.x) {
         double a = 0.0;
@@ -591,7 +599,7 @@ int blocks_pass(const EmTensors& T, int block_size, int64_t first, const CellsWs
     case I_: {                                                                            \
         constexpr auto kern = cells_blocks_kernel<I_, SG>;                                \
         if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;                    \
-        kern<<<kSMs, 1024, smem, st>>>(T, first, W.hist, W.consts);                       \
+        launch_after(kern, kSMs, 1024, smem, st, T, first, W.hist, W.consts);                       \
         break;                                                                            \
     }
     switch (block_size) {
@@ -619,8 +627,8 @@ int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters
     BOF4_CUDA_TRY(cudaMemsetAsync(W.hist, 0, reinterpret_cast<char*>(W.cursor) - reinterpret_cast<char*>(W.hist), st));
     auto tails = [&](int add) {
         return for_each_tail_chunk(a, [&](const EmTails& Q) -> int {
-            if (sg) cells_tail_kernel<true><<<1, kEmTailThreads, 0, st>>>(Q, W, a.metric, add);
-            else cells_tail_kernel<false><<<1, kEmTailThreads, 0, st>>>(Q, W, a.metric, add);
+            if (sg) launch_after(cells_tail_kernel<true>, 1, kEmTailThreads, 0, st, Q, W, a.metric, add);
+            else launch_after(cells_tail_kernel<false>, 1, kEmTailThreads, 0, st, Q, W, a.metric, add);
             BOF4_CUDA_TRY(cudaGetLastError());
             return BOF4_OK;
         });
@@ -639,14 +647,14 @@ int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters
         return sg ? blocks_pass<true>(T, a.block_size, f, W, st) : blocks_pass<false>(T, a.block_size, f, W, st);
     }, &calls);
     if (rc) return rc;
-    cells_plan_kernel<<<1, 1024, 0, st>>>(W, (uint32_t)unit_blocks(blocks, a.block_size), a.metric, W.sort.n_items);
+    launch_after(cells_plan_kernel, 1, 1024, 0, st, W, (uint32_t)unit_blocks(blocks, a.block_size), a.metric, W.sort.n_items);
     BOF4_CUDA_TRY(cudaGetLastError());
     first = 0;
     rc = for_each_tensor_chunk(a, 1024 * kLW, [&](const EmTensors& T) -> int {
         const int64_t f = first, nb = of(T);
         first += nb;
         if (const int e = ensure_dynamic_smem<cells_order_kernel>(kMags * 4)) return e;
-        cells_order_kernel<<<kSMs, 1024, kMags * 4, st>>>(T, f, nb, a.block_size, W);
+        launch_after(cells_order_kernel, kSMs, 1024, kMags * 4, st, T, f, nb, a.block_size, W);
         BOF4_CUDA_TRY(cudaGetLastError());
         return BOF4_OK;
     }, &calls);
@@ -655,12 +663,12 @@ int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters
     while ((16 << shift) < a.block_size) ++shift;
     constexpr int smem = 2 * kCellDepth * 4;
     if ((rc = ensure_dynamic_smem<cells_accumulate_kernel>(smem))) return rc;
-    cells_accumulate_kernel<<<kCellCtas * kSMs, kCellThreads, smem, st>>>(W, shift, a.metric);
+    launch_after(cells_accumulate_kernel, kCellCtas * kSMs, kCellThreads, smem, st, W, shift, a.metric);
     BOF4_CUDA_TRY(cudaGetLastError());
     if ((rc = tails(1))) return rc;
-    cells_scan_kernel<<<kCellScans, 512, 0, st>>>(W);
-    cells_items_kernel<<<kCellScans, 512, 0, st>>>(W);
-    cells_square_kernel<<<1, 320, 0, st>>>(W);
+    launch_after(cells_scan_kernel, kCellScans, 512, 0, st, W);
+    launch_after(cells_items_kernel, kCellScans, 512, 0, st, W);
+    launch_after(cells_square_kernel, 1, 320, 0, st, W);
     BOF4_CUDA_TRY(cudaGetLastError());
     SortFit F{};
     F.acc = reinterpret_cast<const unsigned long long*>(W.acc);

@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(512, 2)
 sort_samples_kernel(const EmTensors T, const uint32_t first, float2* __restrict__ items, uint32_t* __restrict__ head,
                     double* __restrict__ w2)
 {
+    if (!after_previous()) return;
     constexpr int NT = 512;
     __shared__ WideScratch s_wide;
     __shared__ uint32_t s_item0[kEmMaxTensors];
@@ -118,6 +119,7 @@ __global__ void __launch_bounds__(kEmTailThreads)
 sort_tail_kernel(const EmTails Q, uint32_t at, float2* __restrict__ items, uint32_t* __restrict__ head,
                  double* __restrict__ w2)
 {
+    if (!after_previous()) return;
     __shared__ float s_w[4096];
     __shared__ unsigned long long s_red[kEmTailThreads / 32];
     __shared__ double s_sum[kEmTailThreads / 32];
@@ -149,6 +151,7 @@ sort_tail_kernel(const EmTails Q, uint32_t at, float2* __restrict__ items, uint3
 
 __global__ void sort_head_kernel(uint32_t* head, uint32_t n, double* w2)
 {
+    if (!after_previous()) return;
     if (threadIdx.x == 0) {
         head[0] = n;
         head[1] = 0u;
@@ -170,6 +173,7 @@ template <int SHIFT>
 __global__ void __launch_bounds__(kSortThreads)
 sort_count_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ head, uint32_t* __restrict__ counts)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t s_hist[4][256];  // a copy per eight warps: fewer collisions on crowded digits
     const int tid = threadIdx.x;
     (&s_hist[0][0])[tid] = 0u;
@@ -190,6 +194,7 @@ __global__ void __launch_bounds__(kSortThreads)
 sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ head, const uint32_t* __restrict__ counts,
                     float2* __restrict__ out)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t s_cnt[32][256];
     __shared__ uint32_t s_base[256], s_warp[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -306,6 +311,7 @@ struct SampleWeight {
 __global__ void __launch_bounds__(256)
 sort_start_kernel(const float2* __restrict__ items, const uint32_t* __restrict__ head, uint32_t* __restrict__ start)
 {
+    if (!after_previous()) return;
     const uint32_t n = *head;
     for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
         const int b = sort_bin(items[i].x), prev = i ? sort_bin(items[i - 1].x) : -1;
@@ -340,6 +346,7 @@ template <bool MAE, bool CELLS>
 __global__ void __launch_bounds__(256)
 sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
 {
+    if (!after_previous()) return;
     constexpr int STEPS = kSortChunk / 32, kNone = 1 << 20;
     const uint32_t n = W.n_items[0];
     weight.max_bits = W.n_items[1];
@@ -418,6 +425,7 @@ template <bool MAE>
 __global__ void __launch_bounds__(256)
 sort_group_kernel(const SortWs W)
 {
+    if (!after_previous()) return;
     const int lane = threadIdx.x & 31, g = blockIdx.x * 8 + (threadIdx.x >> 5), b = g * kSortGroup + lane;
     const uint32_t s = W.start[b], e = W.start[b + 1];
     SortSums t{0.0, 0.0, 0ull};
@@ -453,6 +461,7 @@ template <bool MAE, bool CELLS>
 __global__ void __launch_bounds__(1024, 1)
 sort_fit_kernel(const SortWs W, const SortFit F)
 {
+    if (!after_previous()) return;
     extern __shared__ __align__(16) SortSums s_group[];
     __shared__ float s_level[2][kLevels], s_med[kLevels];
     __shared__ SortSums s_half[32];
@@ -689,12 +698,12 @@ int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
     weight.acc = reinterpret_cast<const ulonglong2*>(F.acc);
     weight.acc_a = F.acc_a;
     const int64_t ctas = (F.n_max + 8 * kSortChunk - 1) / (8 * kSortChunk);
-    sort_sums_kernel<MAE, CELLS><<<(int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st>>>(W, weight);
-    sort_group_kernel<MAE><<<kSortGroups / 8, 256, 0, st>>>(W);
+    launch_after(sort_sums_kernel<MAE, CELLS>, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, W, weight);
+    launch_after(sort_group_kernel<MAE>, kSortGroups / 8, 256, 0, st, W);
     constexpr int smem = kSortGroups * (int)sizeof(SortSums);
     constexpr auto kern = sort_fit_kernel<MAE, CELLS>;
     if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
-    kern<<<1, 1024, smem, st>>>(W, F);
+    launch_after(kern, 1, 1024, smem, st, W, F);
     BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;
 }
@@ -703,7 +712,7 @@ template <class DT, bool SG>
 int samples(const EmTensors& T, int block_size, uint32_t first, const SortWs& W, cudaStream_t st)
 {
 #define BOF4_SORT_I(I_) \
-    case I_: sort_samples_kernel<DT, I_, SG><<<2 * kSMs, 512, 0, st>>>(T, first, W.a, W.n_items, W.w2); break;
+    case I_: launch_after(sort_samples_kernel<DT, I_, SG>, 2 * kSMs, 512, 0, st, T, first, W.a, W.n_items, W.w2); break;
     switch (block_size) {
         BOF4_SORT_I(32) BOF4_SORT_I(64) BOF4_SORT_I(128) BOF4_SORT_I(256) BOF4_SORT_I(512) BOF4_SORT_I(1024)
         BOF4_SORT_I(2048) BOF4_SORT_I(4096)
@@ -717,15 +726,15 @@ int samples(const EmTensors& T, int block_size, uint32_t first, const SortWs& W,
 
 int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
 {
-    sort_count_kernel<0><<<kSortGrid, kSortThreads, 0, st>>>(W.a, W.n_items, W.counts);
-    sort_scatter_kernel<0><<<kSortGrid, kSortThreads, 0, st>>>(W.a, W.n_items, W.counts, W.b);
-    sort_count_kernel<8><<<kSortGrid, kSortThreads, 0, st>>>(W.b, W.n_items, W.counts);
-    sort_scatter_kernel<8><<<kSortGrid, kSortThreads, 0, st>>>(W.b, W.n_items, W.counts, W.a);
+    launch_after(sort_count_kernel<0>, kSortGrid, kSortThreads, 0, st, W.a, W.n_items, W.counts);
+    launch_after(sort_scatter_kernel<0>, kSortGrid, kSortThreads, 0, st, W.a, W.n_items, W.counts, W.b);
+    launch_after(sort_count_kernel<8>, kSortGrid, kSortThreads, 0, st, W.b, W.n_items, W.counts);
+    launch_after(sort_scatter_kernel<8>, kSortGrid, kSortThreads, 0, st, W.b, W.n_items, W.counts, W.a);
     SortWs V = W;  // the ordered samples are in the first array
     V.a = W.b;
     V.b = W.a;
     const int64_t ctas = (F.n_max + 255) / 256;
-    sort_start_kernel<<<(int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st>>>(V.b, V.n_items, V.start);
+    launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, V.b, V.n_items, V.start);
     BOF4_CUDA_TRY(cudaGetLastError());
     const bool mae = F.metric == BOF4_METRIC_MAE || F.metric == BOF4_METRIC_MAE_NORMALIZED;
     if (F.acc) return mae ? sums_and_iterations<true, true>(V, F, st) : sums_and_iterations<false, true>(V, F, st);
@@ -740,7 +749,7 @@ int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iter
     SortWs W;
     if (sorted_layout(d_ws, a.n_total, false, &W) > ws_bytes) return BOF4_OK;
     *done = true;
-    sort_head_kernel<<<1, 320, 0, st>>>(W.n_items, (uint32_t)a.n_total, W.w2);
+    launch_after(sort_head_kernel, 1, 320, 0, st, W.n_items, (uint32_t)a.n_total, W.w2);
     const bool sg = a.norm == BOF4_NORM_SIGNED;
     uint32_t at = 0;
     int calls = 0;
@@ -754,11 +763,11 @@ int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iter
     if (rc) return rc;
     rc = for_each_tail_chunk(a, [&](const EmTails& Q) -> int {
         if (a.w_dtype == BOF4_F32) {
-            if (sg) sort_tail_kernel<F32, true><<<1, kEmTailThreads, 0, st>>>(Q, at, W.a, W.n_items, W.w2);
-            else sort_tail_kernel<F32, false><<<1, kEmTailThreads, 0, st>>>(Q, at, W.a, W.n_items, W.w2);
+            if (sg) launch_after(sort_tail_kernel<F32, true>, 1, kEmTailThreads, 0, st, Q, at, W.a, W.n_items, W.w2);
+            else launch_after(sort_tail_kernel<F32, false>, 1, kEmTailThreads, 0, st, Q, at, W.a, W.n_items, W.w2);
         } else {
-            if (sg) sort_tail_kernel<BF16, true><<<1, kEmTailThreads, 0, st>>>(Q, at, W.a, W.n_items, W.w2);
-            else sort_tail_kernel<BF16, false><<<1, kEmTailThreads, 0, st>>>(Q, at, W.a, W.n_items, W.w2);
+            if (sg) launch_after(sort_tail_kernel<BF16, true>, 1, kEmTailThreads, 0, st, Q, at, W.a, W.n_items, W.w2);
+            else launch_after(sort_tail_kernel<BF16, false>, 1, kEmTailThreads, 0, st, Q, at, W.a, W.n_items, W.w2);
         }
         for (int q = 0; q < Q.count; ++q) at += (uint32_t)Q.len[q];
         BOF4_CUDA_TRY(cudaGetLastError());

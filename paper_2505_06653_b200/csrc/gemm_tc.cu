@@ -275,6 +275,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap code_map, const void* __restr
     __shared__ __align__(8) uint32_t s_head[2][OPQ ? kTcBatch : 1][2 * kTcIssue];
     __shared__ int s_batch_lines[2], s_count;       // lines of a batch, negative: more entries than there is room for
     __shared__ int2 s_bound[4];                     // brackets of the first list entry of the tiles tile0 + k, at k & 3
+    if (!after_previous()) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t tiles = (smem_u32(s_dyn) + 1023u) & ~1023u;  // 1024-byte aligned: the swizzle atoms start here
     unsigned char* tiles_ptr = s_dyn + (tiles - smem_u32(s_dyn));
@@ -867,9 +868,8 @@ extern "C" int bof4_gemm_tc(const uint8_t* d_codes, const void* d_scales, int sc
     {                                                                                                                      \
         constexpr auto kern = gemm_tc_kernel<ST_, HALF_, OPQ_, WIDE_>;                                                            \
         if ((rc = ensure_dynamic_smem<kern>(kTcSmem))) return rc;                                                          \
-        kern<<<work.ctas, kTcThreads, kTcSmem, st>>>(code_map, d_scales, cols, block_shift, d_codebook, x_map, n_rhs, d_y, \
-                                                     d_status, d_out_idx, val, d_n_out, capacity, work,                    \
-                                                     static_cast<unsigned char*>(d_ws));                                   \
+        launch_after(kern, work.ctas, kTcThreads, kTcSmem, st, code_map, d_scales, cols, block_shift, d_codebook, x_map, n_rhs, d_y, \
+                     d_status, d_out_idx, val, d_n_out, capacity, work, static_cast<unsigned char*>(d_ws));                          \
     }
 #define BOF4_TC_GO(ST_, HALF_, OPQ_) { if (n_rhs > 32) BOF4_TC_W(ST_, HALF_, OPQ_, true) else BOF4_TC_W(ST_, HALF_, OPQ_, false) }
 #define BOF4_TC_ST(ST_)                                                             \

@@ -145,6 +145,7 @@ gemv_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, 
             int block_shift, const float* __restrict__ levels, const void* __restrict__ x, float* __restrict__ y,
             int stripes, int groups)
 {
+    if (!after_previous()) return;
     constexpr int R = kGvRows, K = kGvDefer, S = kGvStages;
     extern __shared__ __align__(256) unsigned char s_dyn[];  // table, then the rings
     unsigned char* const s_tab = s_dyn;
@@ -318,6 +319,7 @@ gemv_outlier_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ 
                     const int32_t* __restrict__ idx, const uint16_t* __restrict__ val,
                     const int64_t* __restrict__ n_out, int64_t capacity, float* __restrict__ y)
 {
+    if (!after_previous()) return;
     __shared__ float s_term[256];
     __shared__ int s_row[256];
     int64_t k_end = *n_out;
@@ -373,7 +375,7 @@ static int launch_gemv_kernel(const uint8_t* d_codes, const void* d_scales, int6
     constexpr int smem = RING ? gv_smem(MAXT) : kGvTabBytes;
     constexpr auto kern = gemv_kernel<ST, XT, MAXT, RING>;
     if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
-    kern<<<grid, 32 * stripes * groups, smem, st>>>(d_codes, d_scales, rows, cols, block_shift, d_codebook,
+    launch_after(kern, grid, 32 * stripes * groups, smem, st, d_codes, d_scales, rows, cols, block_shift, d_codebook,
                                                              d_x, d_y, stripes, groups);
     BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;
@@ -393,7 +395,7 @@ static int launch_gemv(const uint8_t* d_codes, const void* d_scales, int64_t row
     if (opq && capacity > 0) {
         int block_shift = 0;
         while ((1 << block_shift) < block_size) ++block_shift;
-        gemv_outlier_kernel<ST, XT><<<2 * kSMs, 256, 0, st>>>(d_codes, d_scales, rows, cols, block_shift, d_codebook,
+        launch_after(gemv_outlier_kernel<ST, XT>, 2 * kSMs, 256, 0, st, d_codes, d_scales, rows, cols, block_shift, d_codebook,
                                                               d_x, d_out_idx, val, d_n_out, capacity, d_y);
         BOF4_CUDA_TRY(cudaGetLastError());
     }

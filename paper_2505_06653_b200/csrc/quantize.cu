@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kQThreads, kQCtasPerSm)
 quantize_kernel(const void* __restrict__ w, int64_t n, const float* __restrict__ levels,
                 uint8_t* __restrict__ codes, void* __restrict__ scales)
 {
+    if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_lut[];
     __shared__ float s_xi[kLevels], s_lv[kLevels];
     __shared__ int s_multi;
@@ -229,6 +230,7 @@ template <class DT, int I, bool SIGNED, class ST>
 __global__ void __launch_bounds__(kQThreads, kQCtasPerSm)
 quantize_batch_kernel(const __grid_constant__ QuantBatch B, const float* __restrict__ levels)
 {
+    if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_lut[];
     __shared__ float s_xi[kLevels], s_lv[kLevels];
     __shared__ int s_multi;
@@ -359,6 +361,7 @@ __global__ void __launch_bounds__(kQThreads, kQCtasPerSm)
 quantize32_kernel(const void* __restrict__ w, int64_t n, const float* __restrict__ levels,
                   uint8_t* __restrict__ codes, void* __restrict__ scales)
 {
+    if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_lut[];
     __shared__ QuantShared32 S;
     const int tail = (int)(n & (I - 1));
@@ -377,6 +380,7 @@ template <int I, bool SIGNED, class ST>
 __global__ void __launch_bounds__(kQThreads, kQCtasPerSm)
 quantize32_batch_kernel(const QuantBatch B, const float* __restrict__ levels)
 {
+    if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_lut[];
     __shared__ QuantShared32 S;
     const int G = gridDim.x;
@@ -524,6 +528,7 @@ __global__ void __launch_bounds__(kDThreads, kDCtasPerSm)
 dequantize_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t n,
                   const float* __restrict__ levels, void* __restrict__ out)
 {
+    if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_tab[];
     build_pair_table(levels, s_tab);
     dequantize_rows<ST, OT, I>(codes, scales, n, out, s_tab, (int)blockIdx.x);
@@ -544,6 +549,7 @@ template <class ST, class OT, int I>
 __global__ void __launch_bounds__(kDThreads, kDCtasPerSm)
 dequantize_batch_kernel(const DequantBatch B, const float* __restrict__ levels)
 {
+    if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_tab[];
     build_pair_table(levels, s_tab);
     const int G = gridDim.x;
@@ -558,6 +564,7 @@ __global__ void scatter_outliers_kernel(const int32_t* __restrict__ idx, const u
                                         const int64_t* __restrict__ n_out, int64_t capacity, int64_t n,
                                         void* __restrict__ out)
 {
+    if (!after_previous()) return;
     int64_t k_end = *n_out;
     if (k_end > capacity) k_end = capacity;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < k_end;
@@ -705,6 +712,7 @@ opq_pass1_kernel(const void* __restrict__ w, int64_t n, const float* __restrict_
                  int32_t* __restrict__ counts, unsigned long long* __restrict__ chunk_sum,
                  int32_t* __restrict__ stage_idx, uint16_t* __restrict__ stage_val)
 {
+    if (!after_previous()) return;
     static_assert(kOpqTile == kWarpW, "one tile per warp iteration");
     extern __shared__ __align__(16) unsigned char s_lut[];
     __shared__ float s_xi[kLevels], s_lv[kLevels];
@@ -785,7 +793,7 @@ opq_pass1_kernel(const void* __restrict__ w, int64_t n, const float* __restrict_
 // lane: the ballot is the outlier mask in index order, the places of the list follow from its bits, and the
 // cleaned weights and their extremes come back without a loop over all weights in every lane.
 // 28672 x 8192 weights, blocks of 64, 5 % of them with outliers: 225 us with the exact sums and a 32-step
-// outlier loop in every lane, NEWUS us this way; the plain quantiser takes 105.
+// outlier loop in every lane, 184 us this way; the plain quantiser takes 105.
 
 // Balanced tree sum of the lane's 32 values given as 16 pairs {even, odd}: every addition is a
 // separate fp32 RN operation; levels two to five add two independent partial sums per instruction.
@@ -1021,6 +1029,7 @@ __device__ __noinline__ void opq_row_far(const OpqArgs& A, int64_t idx, bool ok,
 template <int I, bool SIGNED, class ST, bool QUANT>
 __global__ void __launch_bounds__(kOThreads, kQCtasPerSm) opq_pass1_32_kernel(const __grid_constant__ OpqArgs A)
 {
+    if (!after_previous()) return;
     static_assert(2 * kOpqTile == kWarpW32 && kOpqChunk % 2 == 0, "two tiles of one chunk per warp iteration");
     extern __shared__ __align__(16) unsigned char s_dyn[];  // candidate words, then the region table
     __shared__ QuantShared32 S;
@@ -1112,6 +1121,7 @@ opq_gather_kernel(const void* __restrict__ w, int64_t n, float tau, const int32_
                   int32_t* __restrict__ out_idx, uint16_t* __restrict__ out_val, int64_t capacity,
                   int64_t* __restrict__ n_out)
 {
+    if (!after_previous()) return;
     constexpr int PER = kOpqChunk / 256;  // consecutive tiles per thread
     __shared__ int64_t s_warp[8];
     __shared__ unsigned long long s_base[8];
@@ -1240,6 +1250,7 @@ tail_block_kernel(const void* __restrict__ w, int64_t first, int len, const floa
                   void* __restrict__ w_clean, int32_t* __restrict__ out_idx, uint16_t* __restrict__ out_val,
                   int64_t capacity, int64_t* __restrict__ n_out)
 {
+    if (!after_previous()) return;
     __shared__ float s_w[4096], s_t[4096];
     __shared__ unsigned char s_c[4096];
     __shared__ float s_xi[kLevels], s_lv[kLevels];
@@ -1407,14 +1418,14 @@ extern "C" int bof4_quantize(const void* d_w, int w_dtype, int64_t n, int block_
                 BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                     { constexpr auto kern = quantize32_kernel<I_, SG, ST>;
                       if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                      kern<<<grid, kQThreads, kLutBytes, st>>>(d_w, n, d_codebook, d_codes, d_scales); })));
+                      launch_after(kern, grid, kQThreads, kLutBytes, st, d_w, n, d_codebook, d_codes, d_scales); })));
     } else {
         const int grid = grid_for((n_whole + kQRow - 1) / kQRow + more, kQCtasPerSm);
         BOF4_DISPATCH_I(block_size,
             BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                 { constexpr auto kern = quantize_kernel<F32, I_, SG, F32>;
                   if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                  kern<<<grid, kQThreads, kLutBytes, st>>>(d_w, n, d_codebook, d_codes, d_scales); }));
+                  launch_after(kern, grid, kQThreads, kLutBytes, st, d_w, n, d_codebook, d_codes, d_scales); }));
     }
     BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;
@@ -1457,7 +1468,7 @@ extern "C" int bof4_dequantize(const uint8_t* d_codes, const void* d_scales, int
     BOF4_DISPATCH_I(block_size, {                                                                            \
         constexpr auto kern = dequantize_kernel<ST_, OT_, I_>;                                               \
         if ((rc = ensure_dynamic_smem<kern>(kDTableBytes))) return rc;                                       \
-        kern<<<grid, kDThreads, kDTableBytes, st>>>(d_codes, d_scales, n, d_codebook, d_out); })
+        launch_after(kern, grid, kDThreads, kDTableBytes, st, d_codes, d_scales, n, d_codebook, d_out); })
     if (scale_dtype == BOF4_F32 && out_dtype == BOF4_F32) { BOF4_DEQ(F32, F32) }
     else if (scale_dtype == BOF4_F32) { BOF4_DEQ(F32, BF16) }
     else if (out_dtype == BOF4_F32) { BOF4_DEQ(BF16, F32) }
@@ -1467,9 +1478,9 @@ extern "C" int bof4_dequantize(const uint8_t* d_codes, const void* d_scales, int
     if (opq && capacity > 0) {
         const uint16_t* val = static_cast<const uint16_t*>(d_out_val);
         if (out_dtype == BOF4_F32)
-            scatter_outliers_kernel<F32><<<kSMs, 256, 0, st>>>(d_out_idx, val, d_n_out, capacity, n, d_out);
+            launch_after(scatter_outliers_kernel<F32>, kSMs, 256, 0, st, d_out_idx, val, d_n_out, capacity, n, d_out);
         else
-            scatter_outliers_kernel<BF16><<<kSMs, 256, 0, st>>>(d_out_idx, val, d_n_out, capacity, n, d_out);
+            launch_after(scatter_outliers_kernel<BF16>, kSMs, 256, 0, st, d_out_idx, val, d_n_out, capacity, n, d_out);
         BOF4_CUDA_TRY(cudaGetLastError());
     }
     return BOF4_OK;
@@ -1526,13 +1537,13 @@ extern "C" int bof4_quantize_batch(const void* const* h_w, const int64_t* h_n, i
                         BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                             { constexpr auto kern = quantize32_batch_kernel<I_, SG, ST>;
                               if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                              kern<<<grid, kQThreads, kLutBytes, st>>>(B, d_codebook); })));
+                              launch_after(kern, grid, kQThreads, kLutBytes, st, B, d_codebook); })));
             } else {
                 BOF4_DISPATCH_I(block_size,
                     BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                         { constexpr auto kern = quantize_batch_kernel<F32, I_, SG, F32>;
                           if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                          kern<<<grid, kQThreads, kLutBytes, st>>>(B, d_codebook); }));
+                          launch_after(kern, grid, kQThreads, kLutBytes, st, B, d_codebook); }));
             }
             BOF4_CUDA_TRY(cudaGetLastError());
             B.count = 0;
@@ -1591,7 +1602,7 @@ extern "C" int bof4_dequantize_batch(const uint8_t* const* h_codes, const void* 
 #define BOF4_DEQB(ST_, OT_) BOF4_DISPATCH_I(block_size, {                                  \
         constexpr auto kern = dequantize_batch_kernel<ST_, OT_, I_>;                       \
         if ((rc = ensure_dynamic_smem<kern>(kDTableBytes))) return rc;                     \
-        kern<<<grid, kDThreads, kDTableBytes, st>>>(B, d_codebook); })
+        launch_after(kern, grid, kDThreads, kDTableBytes, st, B, d_codebook); })
             if (scale_dtype == BOF4_F32 && out_dtype == BOF4_F32) { BOF4_DEQB(F32, F32) }
             else if (scale_dtype == BOF4_F32) { BOF4_DEQB(F32, BF16) }
             else if (out_dtype == BOF4_F32) { BOF4_DEQB(BF16, F32) }
@@ -1679,24 +1690,22 @@ int launch_opq(const char* fn, const void* d_w, int w_dtype, int64_t n, int bloc
                         { constexpr auto kern = opq_pass1_32_kernel<I_, SG, ST, QUANT>;
                           constexpr int words = kOpqWordBytes + (QUANT ? kLutBytes : 0);
                           if ((rc = ensure_dynamic_smem<kern>(words))) return rc;
-                          kern<<<grid32, kOThreads, words, st>>>(OpqArgs{d_w, n_whole, d_codebook, tau, d_codes, d_scales, d_w_clean,
+                          launch_after(kern, grid32, kOThreads, words, st, OpqArgs{d_w, n_whole, d_codebook, tau, d_codes, d_scales, d_w_clean,
                                                                          counts, chunk_sum, stage_idx, stage_val}); })));
         } else {
             BOF4_DISPATCH_I(block_size,
                 BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                     { constexpr auto kern = opq_pass1_kernel<F32, I_, SG, F32, QUANT>;
                       if ((rc = ensure_dynamic_smem<kern>(kLutBytes))) return rc;
-                      kern<<<grid, kQThreads, smem, st>>>(d_w, n_whole, d_codebook, tau, d_codes, d_scales, d_w_clean,
+                      launch_after(kern, grid, kQThreads, smem, st, d_w, n_whole, d_codebook, tau, d_codes, d_scales, d_w_clean,
                                                           counts, chunk_sum, stage_idx, stage_val); }));
         }
         BOF4_CUDA_TRY(cudaGetLastError());
         if (w_dtype == BOF4_F32) {
-            BOF4_DISPATCH_I(block_size, (opq_gather_kernel<F32, I_><<<(int)Lw.chunks, 256, 0, st>>>(
-                d_w, n_whole, tau, counts, Lw.tiles, chunk_sum, stage_idx, stage_val, d_out_idx, out_val, capacity,
+            BOF4_DISPATCH_I(block_size, (launch_after(opq_gather_kernel<F32, I_>, (int)Lw.chunks, 256, 0, st, d_w, n_whole, tau, counts, Lw.tiles, chunk_sum, stage_idx, stage_val, d_out_idx, out_val, capacity,
                 d_n_out)));
         } else {
-            BOF4_DISPATCH_I(block_size, (opq_gather_kernel<BF16, I_><<<(int)Lw.chunks, 256, 0, st>>>(
-                d_w, n_whole, tau, counts, Lw.tiles, chunk_sum, stage_idx, stage_val, d_out_idx, out_val, capacity,
+            BOF4_DISPATCH_I(block_size, (launch_after(opq_gather_kernel<BF16, I_>, (int)Lw.chunks, 256, 0, st, d_w, n_whole, tau, counts, Lw.tiles, chunk_sum, stage_idx, stage_val, d_out_idx, out_val, capacity,
                 d_n_out)));
         }
         BOF4_CUDA_TRY(cudaGetLastError());
@@ -1704,8 +1713,7 @@ int launch_opq(const char* fn, const void* d_w, int w_dtype, int64_t n, int bloc
     if (tail) {  // after the gather kernel: its outliers follow those of the whole blocks
         BOF4_DISPATCH_WS(w_dtype, scale_dtype,
             BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
-                (tail_block_kernel<DT, SG, ST, QUANT><<<1, kTailThreads, 0, st>>>(
-                    d_w, n_whole, tail, d_codebook, tau, d_codes, d_scales, n_whole / block_size, d_w_clean, d_out_idx,
+                (launch_after(tail_block_kernel<DT, SG, ST, QUANT>, 1, kTailThreads, 0, st, d_w, n_whole, tail, d_codebook, tau, d_codes, d_scales, n_whole / block_size, d_w_clean, d_out_idx,
                     out_val, capacity, d_n_out))));
         BOF4_CUDA_TRY(cudaGetLastError());
     }

@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(kDqGroup)
 scales_compress_kernel(const void* __restrict__ scales, int64_t n_blocks, uint8_t* __restrict__ q,
                        float* __restrict__ group, uint8_t* __restrict__ sign_bytes)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t s_max[kDqGroup / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int64_t k = blockIdx.x; k * kDqGroup < n_blocks; k += gridDim.x) {
@@ -66,6 +67,7 @@ __global__ void __launch_bounds__(kDqGroup)
 scales_expand_kernel(const uint8_t* __restrict__ q, const float* __restrict__ group,
                      const uint8_t* __restrict__ sign_bytes, int64_t n_blocks, float* __restrict__ out)
 {
+    if (!after_previous()) return;
     const int tid = threadIdx.x;
     for (int64_t k = blockIdx.x; k * kDqGroup < n_blocks; k += gridDim.x) {
         const int64_t b = k * kDqGroup + tid;
@@ -102,9 +104,9 @@ extern "C" int bof4_scales_compress(const void* d_scales, int scale_dtype, int64
     const int grid = (int)(groups < 148 * 8 ? groups : 148 * 8);
     uint8_t* sg = norm == BOF4_NORM_SIGNED ? d_sign : nullptr;
     if (scale_dtype == BOF4_F32)
-        scales_compress_kernel<F32><<<grid, kDqGroup, 0, st>>>(d_scales, n_blocks, d_q, d_group, sg);
+        launch_after(scales_compress_kernel<F32>, grid, kDqGroup, 0, st, d_scales, n_blocks, d_q, d_group, sg);
     else
-        scales_compress_kernel<BF16><<<grid, kDqGroup, 0, st>>>(d_scales, n_blocks, d_q, d_group, sg);
+        launch_after(scales_compress_kernel<BF16>, grid, kDqGroup, 0, st, d_scales, n_blocks, d_q, d_group, sg);
     BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;
 }
@@ -124,7 +126,7 @@ extern "C" int bof4_scales_expand(const uint8_t* d_q, const float* d_group, cons
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t groups = (n_blocks + kDqGroup - 1) / kDqGroup;
     const int grid = (int)(groups < 148 * 8 ? groups : 148 * 8);
-    scales_expand_kernel<<<grid, kDqGroup, 0, st>>>(d_q, d_group, d_sign, n_blocks, d_scales_out);
+    launch_after(scales_expand_kernel, grid, kDqGroup, 0, st, d_q, d_group, d_sign, n_blocks, d_scales_out);
     BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;
 }
