@@ -3,6 +3,8 @@
 #include <stdarg.h>
 #include <stdio.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "em_sorted.cuh"
 #include "layout.h"
@@ -23,6 +25,48 @@ int cuda_fail(cudaError_t e, const char* what)
 {
     set_error("CUDA error %d (%s) in %s", (int)e, cudaGetErrorString(e), what);
     return BOF4_ERR_CUDA;
+}
+
+// Where a count is read back: a page of host memory that the device writes, one line per waiting call.  A copy to
+// pageable memory and a stream synchronisation take 8 us after the kernels are done, a store seen by a
+// polling host 1 us.  The page is allocated once; with all its lines taken a call copies as before.
+struct CountSlots {
+    static constexpr int kSlots = 64;
+    std::atomic<uint64_t> taken{0};
+    char* page = nullptr;
+    int take()
+    {
+        uint64_t t = taken.load(std::memory_order_relaxed);
+        while (~t) {
+            const int k = __builtin_ctzll(~t);
+            if (taken.compare_exchange_weak(t, t | (1ull << k), std::memory_order_acquire)) return k;
+        }
+        return -1;
+    }
+    void give(int k) { taken.fetch_and(~(1ull << k), std::memory_order_release); }
+    volatile int64_t* slot(int k) { return reinterpret_cast<volatile int64_t*>(page + 64 * k); }
+};
+
+// The process's page, or NULL if none can be had.
+static CountSlots* count_slots()
+{
+    static CountSlots slots;
+    static const bool ok = [] {
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, 64 * CountSlots::kSlots, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        slots.page = static_cast<char*>(p);
+        return true;
+    }();
+    return ok ? &slots : nullptr;
+}
+
+__global__ void store_count_kernel(const int64_t* n_out, volatile int64_t* slot)
+{
+    if (!after_previous()) return;
+    *slot = *n_out;
 }
 
 }  // namespace bof4
@@ -60,8 +104,28 @@ int bof4_outlier_count(const int64_t* d_n_out, int64_t capacity, int64_t* h_n_ou
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int64_t count = 0;
-    BOF4_CUDA_TRY(cudaMemcpyAsync(&count, d_n_out, sizeof(count), cudaMemcpyDeviceToHost, st));
-    BOF4_CUDA_TRY(cudaStreamSynchronize(st));
+    bof4::CountSlots* slots = bof4::count_slots();
+    const int k = slots ? slots->take() : -1;
+    if (k < 0) {
+        BOF4_CUDA_TRY(cudaMemcpyAsync(&count, d_n_out, sizeof(count), cudaMemcpyDeviceToHost, st));
+        BOF4_CUDA_TRY(cudaStreamSynchronize(st));
+    } else {
+        // a slot is given back once its kernel is known to have run; after an error it is not
+        volatile int64_t* slot = slots->slot(k);
+        *slot = -1;
+        bof4::launch_after(bof4::store_count_kernel, 1, 1, 0, st, d_n_out, slot);
+        BOF4_CUDA_TRY(cudaGetLastError());
+        for (int polls = 0; (count = *slot) < 0; ++polls) {
+            if ((polls & 1023) != 1023) continue;
+            const cudaError_t e = cudaStreamQuery(st);
+            if (e == cudaErrorNotReady) continue;
+            BOF4_CUDA_TRY(e);
+            count = *slot;  // the stream is done: this is the count, whatever it is
+            break;
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        slots->give(k);
+    }
     if (h_n_out) *h_n_out = count;
     if (count > capacity) {
         bof4::set_error("outlier list overflow: %lld outliers found, capacity %lld (only the first %lld were "

@@ -759,7 +759,7 @@ opq_pass1_kernel(const void* __restrict__ w, int64_t n, const float* __restrict_
                     }
                 if (lane == 0) {
                     counts[tile] = total;
-                    atomicAdd(&chunk_sum[tile / kOpqChunk], (unsigned long long)total);  // integer: order-free
+                    if (chunk_sum != nullptr) atomicAdd(&chunk_sum[tile / kOpqChunk], (unsigned long long)total);  // integer: order-free
                 }
                 lane_minmax(v, mx, mn);  // of the cleaned weights
             } else if (lane == 0 && tile_ok) {
@@ -976,7 +976,7 @@ __device__ __forceinline__ int2 split_outliers32(uint32_t (&u)[16], unsigned can
 // Outlier counts of the warp row's two tiles, and their share of the chunk's (integer: order-free).
 __device__ __forceinline__ void store_counts32(const OpqArgs& A, int2 found, int64_t tile, int lane)
 {
-    if (lane == 0 && found.x + found.y > 0)
+    if (A.chunk_sum != nullptr && lane == 0 && found.x + found.y > 0)
         atomicAdd(&A.chunk_sum[tile / kOpqChunk], (unsigned long long)(found.x + found.y));
     if (lane < 2 && (tile + lane) * kOpqTile < A.n) A.counts[tile + lane] = lane ? found.y : found.x;
 }
@@ -1112,7 +1112,10 @@ __global__ void __launch_bounds__(kOThreads, kQCtasPerSm) opq_pass1_32_kernel(co
 // Pass 2: every tile's staged outliers are copied to their final, globally ascending position;
 // a tile with more than kOpqStage outliers is re-derived from the weights by one warp.  Each
 // CTA owns one chunk of tiles; its first output position is the sum of the earlier chunks'
-// outlier counts (accumulated by pass 1), and the last chunk's CTA also reports the total.
+// outlier counts (accumulated by pass 1; of a tensor of few chunks the earlier tiles' counts are summed
+// here, which costs nothing beside the wait for this chunk's and saves zeroing the sums), and the last chunk's
+// CTA also reports the total.  Loads that wait for one another bound it, so the first outlier of every tile is
+// requested before the positions are known.
 template <class DT, int I>
 __global__ void __launch_bounds__(256)
 opq_gather_kernel(const void* __restrict__ w, int64_t n, float tau, const int32_t* __restrict__ counts,
@@ -1138,6 +1141,19 @@ opq_gather_kernel(const void* __restrict__ w, int64_t n, float tau, const int32_
         c[k] = (t0 + k < tiles) ? counts[t0 + k] : 0;
         local += c[k];
     }
+    unsigned long long before = 0ull;  // outliers of all earlier chunks
+    if (chunk_sum != nullptr) {
+        for (int k = threadIdx.x; k < (int)blockIdx.x; k += 256) before += chunk_sum[k];
+    } else {
+        for (int k = threadIdx.x; k < (int)blockIdx.x * kOpqChunk; k += 256) before += (unsigned)counts[k];
+    }
+    int32_t first_idx[PER];
+    uint16_t first_val[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        first_idx[k] = c[k] > 0 ? stage_idx[(t0 + k) * kOpqStage] : 0;
+        first_val[k] = c[k] > 0 ? stage_val[(t0 + k) * kOpqStage] : (uint16_t)0;
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int wtotal;
     int excl = warp_excl_scan(local, lane, wtotal);
@@ -1145,9 +1161,6 @@ opq_gather_kernel(const void* __restrict__ w, int64_t n, float tau, const int32_
     __syncthreads();
     int rel = excl;
     for (int k = 0; k < warp; ++k) rel += (int)s_warp[k];
-    // first output position of this chunk: outliers of all earlier chunks
-    unsigned long long before = 0ull;
-    for (int k = threadIdx.x; k < (int)blockIdx.x; k += 256) before += chunk_sum[k];
 #pragma unroll
     for (int off = 16; off; off >>= 1) before += __shfl_xor_sync(kFull, before, off);
     if (lane == 0) s_base[warp] = before;
@@ -1155,7 +1168,7 @@ opq_gather_kernel(const void* __restrict__ w, int64_t n, float tau, const int32_
     before = 0ull;
     for (int k = 0; k < 8; ++k) before += s_base[k];
     const int64_t base = (int64_t)before;
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_out = base + (int64_t)chunk_sum[blockIdx.x];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 255) *n_out = base + rel + local;
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         if (c[k] > 0) {
@@ -1163,8 +1176,8 @@ opq_gather_kernel(const void* __restrict__ w, int64_t n, float tau, const int32_
                 for (int j = 0; j < c[k]; ++j) {
                     const int64_t dst = base + rel + j;
                     if (dst < capacity) {
-                        out_idx[dst] = stage_idx[(t0 + k) * kOpqStage + j];
-                        out_val[dst] = stage_val[(t0 + k) * kOpqStage + j];
+                        out_idx[dst] = j ? stage_idx[(t0 + k) * kOpqStage + j] : first_idx[k];
+                        out_val[dst] = j ? stage_val[(t0 + k) * kOpqStage + j] : first_val[k];
                     }
                 }
             } else {
@@ -1477,10 +1490,13 @@ extern "C" int bof4_dequantize(const uint8_t* d_codes, const void* d_scales, int
     BOF4_CUDA_TRY(cudaGetLastError());
     if (opq && capacity > 0) {
         const uint16_t* val = static_cast<const uint16_t*>(d_out_val);
+        // one entry per thread up to eight CTAs an SM: two loads and a store wait for one another
+        const int64_t ctas = (capacity + 255) / 256;
+        const int sgrid = (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs);
         if (out_dtype == BOF4_F32)
-            launch_after(scatter_outliers_kernel<F32>, kSMs, 256, 0, st, d_out_idx, val, d_n_out, capacity, n, d_out);
+            launch_after(scatter_outliers_kernel<F32>, sgrid, 256, 0, st, d_out_idx, val, d_n_out, capacity, n, d_out);
         else
-            launch_after(scatter_outliers_kernel<BF16>, kSMs, 256, 0, st, d_out_idx, val, d_n_out, capacity, n, d_out);
+            launch_after(scatter_outliers_kernel<BF16>, sgrid, 256, 0, st, d_out_idx, val, d_n_out, capacity, n, d_out);
         BOF4_CUDA_TRY(cudaGetLastError());
     }
     return BOF4_OK;
@@ -1618,6 +1634,10 @@ extern "C" int bof4_dequantize_batch(const uint8_t* const* h_codes, const void* 
 
 namespace {
 
+// Chunks up to which the gather kernel sums the counts of the earlier tiles itself: at 32 (2^23 weights) the last
+// CTA reads 64 KiB of them.  The memset it saves is 2 us of about 30.
+constexpr int kOpqDirect = 32;
+
 // Shared launcher of opq_split (QUANT = false) and bof4_quantize_opq (QUANT = true).
 template <bool QUANT>
 int launch_opq(const char* fn, const void* d_w, int w_dtype, int64_t n, int block_size, int norm,
@@ -1681,7 +1701,10 @@ int launch_opq(const char* fn, const void* d_w, int w_dtype, int64_t n, int bloc
         chunk_sum = reinterpret_cast<unsigned long long*>(ws + Lw.chunk_off);
         stage_idx = reinterpret_cast<int32_t*>(ws + Lw.stage_idx);
         stage_val = reinterpret_cast<uint16_t*>(ws + Lw.stage_val);
-        BOF4_CUDA_TRY(cudaMemsetAsync(chunk_sum, 0, (size_t)Lw.chunks * 8, st));
+        if (Lw.chunks <= kOpqDirect)
+            chunk_sum = nullptr;
+        else
+            BOF4_CUDA_TRY(cudaMemsetAsync(chunk_sum, 0, (size_t)Lw.chunks * 8, st));
         if (w_dtype == BOF4_BF16) {
             const int grid32 = grid_for((n_whole + kORow - 1) / kORow, kQCtasPerSm);
             BOF4_DISPATCH_ST(scale_dtype,
