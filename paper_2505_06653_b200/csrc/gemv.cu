@@ -24,10 +24,14 @@
 // 32-warp CTA of wider matrices has 64 registers per thread and no room for that: its codes
 // travel global -> shared memory by asynchronous 16-byte copies into a ring that each warp owns
 // (kGvStages batches); a lane later reads back exactly the 16 bytes it copied itself, so the
-// ring needs no barrier and costs no registers.  The per-lane partial sums of a
+// ring needs no barrier and costs no registers.  The row groups take kGvRows rows a round; the rows left
+// for a last round are dealt evenly over all groups (14336 rows: 25 instead of 28 for the busiest; 1024 rows: two
+// each on 128 SMs instead of four each on 64), and a round of one or two looks up no more than these.  The per-lane partial sums of a
 // batch are reduced over the warp with a halving butterfly, then every kGvDefer batches over the
 // stripes through shared memory in a fixed order.  Nothing is accumulated with atomics, so y is
 // bit-reproducible.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace bof4 {
@@ -155,17 +159,26 @@ gemv_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, 
     const int64_t c0 = (int64_t)stripe * kGvStripe + lane * kGvLane;  // this lane's first column
     const bool live = c0 < cols;  // cols is a multiple of 32: all of the lane's columns exist or none
     const uint32_t column = (uint32_t)lane * 8u;  // < 256: the low byte of every table offset
-    const int64_t batches = (rows + R - 1) / R;
-    const int64_t bstep = (int64_t)gridDim.x * groups;
+    const int64_t deal = (int64_t)gridDim.x * groups;             // row groups of the grid
+    const int64_t mine = (int64_t)blockIdx.x * groups + group;
+    const int64_t full = rows / (deal * R);                       // rounds of R rows a group
+    const int64_t rest = rows - full * deal * R;
+    const int last_rows = (int)((rest + deal - 1) / deal);        // rows a group of the last round, 0: there is none
+    const int64_t rounds = full + (last_rows > 0);
+    // a round's first row of this group and how many it takes (none past the end, none after the last round)
+    auto first_of = [&](int64_t i) { return i < full ? (i * deal + mine) * R : full * deal * R + mine * last_rows; };
+    auto count_of = [&](int64_t i) -> int64_t {
+        if (i < full) return R;
+        if (i >= rounds) return 0;
+        const int64_t left = rest - mine * last_rows;
+        return left < last_rows ? left : last_rows;
+    };
     // this lane's 16 bytes of (stage 0, row 0); a row is 512 bytes, a stage R rows
     const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_dyn + kGvTabBytes) + (uint32_t)warp * (S * R * 512) +
                           (uint32_t)lane * 16u;
     const uint32_t row_bytes = (uint32_t)(cols >> 1);             // codes of one row
     const uint32_t row_blocks = (uint32_t)(cols >> block_shift);  // block constants of one row
-    const int64_t step_bytes = bstep * R * (int64_t)row_bytes;    // from one of this warp's batches to the next
-    const int64_t step_blocks = bstep * R * (int64_t)row_blocks;
-    // Starts the copies of a batch into `stage`: `left` rows remain from its first row on, whose
-    // codes for this lane start at src.  Nothing is copied for rows past the end or dead lanes:
+    // Starts the copies of a batch of `left` rows into `stage`, whose codes for this lane start at src.  Nothing is copied for rows past the end or dead lanes:
     // whatever the slot then holds is multiplied by a zero block constant.
     auto issue = [&](const uint8_t* src, int64_t left, int stage) {
         if constexpr (RING) {
@@ -197,73 +210,69 @@ gemv_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, 
         for (int u = 0; u < R; ++u) m[u] = (live && u < left) ? gv_scale<ST>(scales, index + u * row_blocks) : 0.0f;
     };
 
-    int64_t b0 = (int64_t)blockIdx.x * groups;  // batch of group 0 in this iteration
-    const int64_t r_first = (b0 + group) * R;    // first row of this warp's first batch
-    int64_t left = rows - r_first;               // rows from the current batch's first row to the end (may be <= 0)
-    const int64_t step_rows = bstep * R;
-    const uint8_t* src = codes + ((r_first * cols + c0) >> 1);               // codes of the next batch to request
-    int64_t blk = (r_first * cols + c0) >> block_shift;                      // block of the next batch's constants
+    auto codes_at = [&](int64_t i) { return codes + ((first_of(i) * cols + c0) >> 1); };
+    auto block_at = [&](int64_t i) { return (first_of(i) * cols + c0) >> block_shift; };
     // The first codes, x and the levels are requested together: the cold misses overlap.
     uint4 cc[R];
     if (RING) {
 #pragma unroll
-        for (int sI = 0; sI < S - 1; ++sI) {
-            issue(src, left - sI * step_rows, sI);
-            src += step_bytes;
-        }
+        for (int sI = 0; sI < S - 1; ++sI) issue(codes_at(sI), count_of(sI), sI);
     } else {
-        fetch(src, left, cc);
-        src += step_bytes;
+        fetch(codes_at(0), count_of(0), cc);
     }
     float m[R];
-    block_constants(blk, left, m);
-    blk += step_blocks;
+    block_constants(block_at(0), count_of(0), m);
     uint64_t xr[16];
     load_x<XT>(x, c0, live, xr);
     {
-        const float mine = levels[threadIdx.x & 15];  // level l sits in the lanes with (lane & 15) == l
-        for (int e = threadIdx.x; e < 256 * 32; e += blockDim.x) {  // blockDim is a multiple of 32: e & 31 == lane
-            const int byte = e >> 5;
-            reinterpret_cast<float2*>(s_tab)[e] = make_float2(__shfl_sync(kFull, mine, byte >> 4),
-                                                              __shfl_sync(kFull, mine, byte & 15));
+        // a row of the table is the same pair 32 times: a warp writes rows in turn, the levels in its registers
+        float lv[16];
+#pragma unroll
+        for (int l = 0; l < 16; ++l) lv[l] = __ldg(levels + l);
+        for (int hi = warp; hi < 16; hi += (int)(blockDim.x >> 5)) {
+            float h = lv[15];
+#pragma unroll
+            for (int l = 14; l >= 0; --l) h = hi == l ? lv[l] : h;
+            float2* row = reinterpret_cast<float2*>(s_tab) + hi * (16 * 32) + lane;
+#pragma unroll
+            for (int l = 0; l < 16; ++l) row[l * 32] = make_float2(h, lv[l]);
         }
     }
     __syncthreads();
     int k = 0, buf = 0, stage = 0;
-    for (; b0 < batches; b0 += bstep) {
+    // One round: codes and constants of the next one are requested, this one's RR rows are multiplied.
+    auto round = [&](int64_t i, auto rr) {
+        constexpr int RR = decltype(rr)::value;
         // refill the slot consumed in the previous iteration, then wait for this iteration's batch
         // (registers: request the next batch before this one is used)
         uint4 cn[R];
         if (RING)
-            issue(src, left - (S - 1) * step_rows, stage == 0 ? S - 1 : stage - 1);
+            issue(codes_at(i + S - 1), count_of(i + S - 1), stage == 0 ? S - 1 : stage - 1);
         else
-            fetch(src, left - step_rows, cn);
-        src += step_bytes;
+            fetch(codes_at(i + 1), count_of(i + 1), cn);
         float mn[R];
-        block_constants(blk, left - step_rows, mn);  // block constants run one batch ahead in registers
-        blk += step_blocks;
-        left -= step_rows;
+        block_constants(block_at(i + 1), count_of(i + 1), mn);  // block constants run one batch ahead in registers
         uint32_t word[R][4];
         if (RING) {
             asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
 #pragma unroll
-            for (int u = 0; u < R; ++u)
+            for (int u = 0; u < RR; ++u)
                 asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
                              : "=r"(word[u][0]), "=r"(word[u][1]), "=r"(word[u][2]), "=r"(word[u][3])
                              : "r"(ring + (uint32_t)(stage * R + u) * 512u));
         } else {
 #pragma unroll
-            for (int u = 0; u < R; ++u)
+            for (int u = 0; u < RR; ++u)
                 word[u][0] = cc[u].x, word[u][1] = cc[u].y, word[u][2] = cc[u].z, word[u][3] = cc[u].w;
         }
         uint64_t a2[R];
 #pragma unroll
         for (int u = 0; u < R; ++u) a2[u] = 0ull;
-        // column pair j of all R rows before pair j + 1: R independent chains share one x register
+        // column pair j of all rows before pair j + 1: RR independent chains share one x register
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
 #pragma unroll
-            for (int u = 0; u < R; ++u) {
+            for (int u = 0; u < RR; ++u) {
                 // byte j holds the codes of columns 2j (high nibble) and 2j + 1 (low nibble);
                 // offset = byte * 256 + lane * 8 in one permute
                 const uint32_t off = __byte_perm(word[u][j >> 2], column, 0x5504u | ((uint32_t)(j & 3) << 4));
@@ -272,11 +281,10 @@ gemv_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, 
         }
         float part[R];
 #pragma unroll
-        for (int u = 0; u < R; ++u) part[u] = __fmul_rn(m[u], sum2(a2[u]));
+        for (int u = 0; u < R; ++u) part[u] = u < RR ? __fmul_rn(m[u], sum2(a2[u])) : 0.0f;
         reduce_rows<R>(part, lane);
         if ((lane & (32 / R - 1)) == 0) s_part[buf][k][lane / (32 / R)][warp] = part[0];
-        const bool last = b0 + bstep >= batches;
-        if (k == K - 1 || last) {
+        if (k == K - 1 || i + 1 == rounds) {
             __syncthreads();
             // Sum over the stripes for the k + 1 batches since the last reduction.  Two buffers:
             // whoever writes this buffer again has passed the next barrier, which the readers
@@ -284,8 +292,9 @@ gemv_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, 
             const int per = groups * R;
             for (int t = threadIdx.x; t < (k + 1) * per; t += blockDim.x) {
                 const int j = t / per, rem = t - j * per, g = rem / R, u = rem - g * R;
-                const int64_t r = (b0 - (int64_t)(k - j) * bstep + g) * R + u;
-                if (r < rows) {
+                const int64_t ri = i - (k - j), who = (int64_t)blockIdx.x * groups + g;
+                const int64_t r = ri < full ? (ri * deal + who) * R + u : full * deal * R + who * last_rows + u;
+                if (r < rows && (ri < full || u < last_rows)) {
                     float sum = 0.0f;
                     for (int sI = 0; sI < stripes; ++sI) sum += s_part[buf][j][u][g * stripes + sI];
                     y[r] = sum;
@@ -302,7 +311,14 @@ gemv_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, 
             m[u] = mn[u];
             if (!RING) cc[u] = cn[u];
         }
-    }
+    };
+    for (int64_t i = 0; i < full; ++i) round(i, std::integral_constant<int, R>{});
+    if (last_rows == 1)
+        round(full, std::integral_constant<int, 1>{});
+    else if (last_rows == 2)
+        round(full, std::integral_constant<int, 2>{});
+    else if (last_rows > 2)
+        round(full, std::integral_constant<int, R>{});
     if (RING) asm volatile("cp.async.wait_group 0;" ::: "memory");  // nothing of this CTA is in flight when it ends
 }
 
@@ -364,10 +380,9 @@ static int launch_gemv_kernel(const uint8_t* d_codes, const void* d_scales, int6
                               int block_size, const float* d_codebook, const void* d_x, float* d_y, int stripes,
                               cudaStream_t st)
 {
-    const int64_t batches = (rows + kGvRows - 1) / kGvRows;
     int groups = (MAXT / 32) / stripes;  // row groups per CTA, >= 1 by the caller's choice of MAXT
-    if (groups > batches) groups = (int)batches;
-    const int64_t want = (batches + groups - 1) / groups;
+    if (groups > rows) groups = (int)rows;
+    const int64_t want = (rows + groups - 1) / groups;
     const int grid = (int)(want < kSMs ? want : kSMs);  // one CTA per SM (its shared memory fills the SM)
     int block_shift = 0;
     while ((1 << block_shift) < block_size) ++block_shift;

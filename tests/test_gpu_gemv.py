@@ -169,3 +169,13 @@ def test_gemv_degenerate_shapes_and_errors(bof4):
     z = torch.zeros(4 * 64, dtype=torch.bfloat16, device=dev)
     c, s = bof4.bof4_quantize(z, 32, bof4.NORM_ABS, lv)
     assert torch.equal(bof4.bof4_gemv(c, s, 4, 64, 32, lv, x).cpu(), torch.zeros(4))
+
+
+@pytest.mark.parametrize("x_dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("cols,groups", [(1024, 16), (17408, 1)])
+def test_rows_left_for_the_last_round(bof4, cols, groups, x_dtype):
+    """148 * groups row groups take four rows a round and share the rest: none, one, two, three or four rows
+    each, the last group fewer."""
+    deal = 148 * groups
+    for rows in (1, deal, deal + 1, 3 * deal, 4 * deal - 1, 4 * deal, 4 * deal + 1, 5 * deal + 2):
+        _check(bof4, rows, cols, 64, torch.bfloat16, x_dtype, True, False, 31)
