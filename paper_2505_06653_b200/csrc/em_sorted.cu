@@ -5,6 +5,8 @@
 // passes of eight bits (count and scatter each, least significant digit first, stable), first sample of
 // every bin, sums of the bins in two steps, iterations.  Nothing depends on the order in which CTAs run:
 // the samples' order, the order of every sum and hence the result are reproducible.
+#include <type_traits>
+
 #include "em_sorted.cuh"
 
 namespace bof4 {
@@ -28,6 +30,10 @@ size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W)
     L.w2 = reinterpret_cast<double*>(take(kSortParts * 8));
     L.counts = reinterpret_cast<uint32_t*>(take((size_t)kSortGrid * 256 * 4));
     L.start = reinterpret_cast<uint32_t*>(take((size_t)(kSortBins + 1) * 4));
+    L.first = reinterpret_cast<uint32_t*>(take((size_t)(kSortGroups + 1) * 4));
+    L.off = reinterpret_cast<uint16_t*>(take((size_t)kSortBins * 2));
+    L.pre = reinterpret_cast<SortSums*>(take((size_t)kSortBins * sizeof(SortSums)));
+    L.suf = reinterpret_cast<SortSums*>(take((size_t)kSortBins * sizeof(SortSums)));
     L.bin = reinterpret_cast<SortSums*>(take((size_t)kSortBins * sizeof(SortSums)));
     L.group = reinterpret_cast<SortSums*>(take((size_t)kSortGroups * sizeof(SortSums)));
     L.lead = reinterpret_cast<SortSums*>(take(chunks * sizeof(SortSums)));
@@ -420,7 +426,7 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
 }
 
 // One warp per group of 32 bins: empty bins are cleared, bins that cross chunks put together (in the
-// order of the chunks), and the group's sums formed.
+// order of the chunks), and the sums of the group, of the bins in front of each and from each on formed.
 template <bool MAE>
 __global__ void __launch_bounds__(256)
 sort_group_kernel(const SortWs W)
@@ -444,11 +450,219 @@ sort_group_kernel(const SortWs W)
         if (lane == who) t = u;
     }
     W.bin[b] = t;
-    sums_reduce<MAE>(t);
-    if (lane == 0) W.group[g] = t;
+    SortSums up = t, down = t;  // this bin and those in front of it; and those behind it
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const SortSums u{__shfl_up_sync(kFull, up.s, o), __shfl_up_sync(kFull, up.sx, o), MAE ? __shfl_up_sync(kFull, up.a, o) : 0ull};
+        const SortSums d{__shfl_down_sync(kFull, down.s, o), __shfl_down_sync(kFull, down.sx, o),
+                         MAE ? __shfl_down_sync(kFull, down.a, o) : 0ull};
+        if (lane >= o) sums_add(up, u);
+        if (lane + o < 32) sums_add(down, d);
+    }
+    W.suf[b] = down;
+    if (lane == 0) W.pre[b] = SortSums{0.0, 0.0, 0ull};
+    if (lane < 31) W.pre[b + 1] = up;
+    else W.group[g] = up;
+    const uint32_t first = __shfl_sync(kFull, s, 0);
+    W.off[b] = (uint16_t)min(s - first, kFarBin);
+    if (lane == 0) W.first[g] = first;
+    if (b == kSortBins - 1) W.first[kSortGroups] = e;
 }
 
-// ---------------------------------------------------------------- all iterations
+// ---------------------------------------------------------------- all iterations, squared error
+//
+// One CTA.  An iteration is a chain of latencies, and what one SM can issue: 32 warps that each find their
+// thresholds' bins, samples and sums take 4000 cycles, most of them issue slots.  So the work is dealt out once:
+// warp 0 turns the levels into 15 cuts (bin, samples, neighbours; a cut per lane), warps 1 to 15 add up the
+// samples of a cut's bin on either side of it, warps 16 to 31 the whole bins of a region: groups from shared
+// memory, the bins beside whole groups as one sum each (pre, suf).  The first samples of all bins are in shared
+// memory as well (16 bits beside the group's first), which leaves one access to L2 in the chain.  Warp 0 divides,
+// compares and goes straight on to the next cuts; the error of an iteration is worked out while the others add up
+// the next.  Iterations of a fit of 2^20 weights, 50 of them: 115 us with
+// a warp per half region, 87 this way; of 2^26 bf16 weights, 100: 230 -> 165; of 2^24 fp32 weights, 30: 172 -> 129.
+//
+// When an iteration leaves every level unchanged the remaining ones would repeat it bit for bit: their entries
+// of the error log are filled in and the loop ends.
+struct SortCut {
+    float p, below, above;      // the threshold and the ones beside it
+    uint32_t from, to;          // samples of its bin (none: a bin of one value, which is in or out as a whole)
+    int end, begin;             // whole bins: the region below ends before `end`, the one above starts at `begin`
+    int low;                    // the bin's samples below p belong to this cut (no cut before it in the same bin)
+};
+constexpr int kMseOff = kSortGroups * 16;            // shared memory: group sums, first samples of the bins,
+constexpr int kMseFirst = kMseOff + kSortBins * 2;   // of the groups
+constexpr int kMseSmem = kMseFirst + (kSortGroups + 1) * 4;
+
+template <bool CELLS>
+__global__ void __launch_bounds__(1024, 1)
+sort_fit_mse_kernel(const SortWs W, const SortFit F)
+{
+    if (!after_previous()) return;
+    extern __shared__ __align__(16) unsigned char s_fit[];
+    double2* const s_group = reinterpret_cast<double2*>(s_fit);
+    uint16_t* const s_off = reinterpret_cast<uint16_t*>(s_fit + kMseOff);
+    uint32_t* const s_first = reinterpret_cast<uint32_t*>(s_fit + kMseFirst);
+    __shared__ SortCut s_cut[kLevels - 1];
+    __shared__ double2 s_low[kLevels], s_high[kLevels + 1], s_mid[kLevels];  // s_low[15] and s_high[0] stay zero
+    __shared__ int s_stop;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int k = tid; k < kSortBins / 8; k += 1024) reinterpret_cast<uint4*>(s_off)[k] = reinterpret_cast<const uint4*>(W.off)[k];
+    for (int k = tid; k < kSortGroups; k += 1024) s_group[k] = make_double2(W.group[k].s, W.group[k].sx);
+    for (int k = tid; k <= kSortGroups; k += 1024) s_first[k] = W.first[k];
+    if (tid == 0) {
+        s_stop = 0;
+        s_low[kLevels - 1] = s_high[0] = make_double2(0.0, 0.0);
+    }
+    double w2 = 0.0;
+    float lv = 0.0f;
+    const bool level = lane < kLevels;
+    if (warp == 0) {
+        for (int k = lane; k < kSortParts; k += 32) w2 += W.w2[k];
+#pragma unroll
+        for (int off = 16; off; off >>= 1) w2 += __shfl_xor_sync(kFull, w2, off);
+        lv = level ? F.codebook[lane] : 0.0f;
+    }
+    __syncthreads();
+    const float inf = __int_as_float(0x7f800000);
+    auto start_of = [&](int b) -> uint32_t {  // first sample of bin b <= kSortBins
+        if (b == kSortBins) return s_first[kSortGroups];
+        const uint32_t o = s_off[b];
+        return o == kFarBin ? __ldg(W.start + b) : s_first[b / kSortGroup] + o;
+    };
+    // the error of the iteration `at`, whose levels and sums lane l has (warp 0)
+    auto error_of = [&](float old, double s0, double s1, int at) -> double {
+        const double o = (double)old;
+        double err = level ? o * (2.0 * s1 - o * s0) : 0.0;
+#pragma unroll
+        for (int off = 8; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
+        err = fmax(w2 - err, 0.0) / (double)F.n_total;
+        if (lane == 0 && F.err_log) F.err_log[at] = err;
+        return err;
+    };
+    float old = 0.0f;
+    double s0 = 0.0, s1 = 0.0;
+    int iter = 0;
+    for (;; ++iter) {
+        // cuts of this iteration; the last one's stop
+        if (warp == 0) {
+            const float up = __shfl_down_sync(kFull, lv, 1);
+            const float p = (lane < kLevels - 1) ? __fmul_rn(__fadd_rn(lv, up), 0.5f) : inf;
+            const int b = sort_bin(p);
+            const float above = __shfl_down_sync(kFull, p, 1), below = __shfl_up_sync(kFull, p, 1);
+            const int before = __shfl_up_sync(kFull, b, 1);
+            if (lane < kLevels - 1) {
+                SortCut c;
+                const bool one = one_value_bin(b);
+                c.p = p, c.above = above, c.below = lane ? below : -inf;
+                c.from = one ? 0u : start_of(b);
+                c.to = one ? 0u : start_of(b + 1);
+                c.end = c.begin = b + 1;
+                if (!one || !(value_of_bin(b) < p)) c.end = b;
+                if (one) c.begin = c.end;
+                c.low = lane == 0 || before != b;
+                s_cut[lane] = c;
+            }
+        }
+        __syncthreads();
+        if (s_stop || iter == F.iters) break;
+        if (warp == 0) {
+            if (iter) error_of(old, s0, s1, iter - 1);
+        } else if (warp < kLevels) {
+            const SortCut c = s_cut[warp - 1];
+            double ls = 0.0, lx = 0.0, hs = 0.0, hx = 0.0;
+            // 64 samples at once, which is all of most bins, then 128
+            auto add = [&](auto count, uint32_t i) {
+                constexpr int U = decltype(count)::value;
+                float2 it[U];
+                double s[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool in = i + 32 * u < c.to;
+                    it[u] = in ? __ldg(W.b + i + 32 * u) : make_float2(__int_as_float(0x7fffffff), 0.0f);  // NaN: on neither side
+                    s[u] = (CELLS && in) ? __ldg(W.cell_s + i + 32 * u) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float x = it[u].x;
+                    const double m = (double)it[u].y, sv = CELLS ? s[u] : m * m, xv = sv * (double)x;
+                    if (x < c.p && x >= c.below && c.low) ls += sv, lx += xv;
+                    if (x >= c.p && x < c.above) hs += sv, hx += xv;
+                }
+            };
+            if (c.from < c.to) add(std::integral_constant<int, 2>{}, c.from + lane);
+            for (uint32_t at = c.from + 64; at < c.to; at += 128) add(std::integral_constant<int, 4>{}, at + lane);
+            __syncwarp();
+            // four sums at once: a quarter of the warp goes on with each
+            const bool a = lane & 16, q = lane & 8;
+            double u = (a ? hs : ls) + __shfl_xor_sync(kFull, a ? ls : hs, 16);
+            double v = (a ? hx : lx) + __shfl_xor_sync(kFull, a ? lx : hx, 16);
+            u = (q ? v : u) + __shfl_xor_sync(kFull, q ? u : v, 8);
+#pragma unroll
+            for (int off = 4; off; off >>= 1) u += __shfl_xor_sync(kFull, u, off);
+            if ((lane & 7) == 0) {
+                double2* to = a ? &s_high[warp] : &s_low[warp - 1];
+                (q ? to->y : to->x) = u;
+            }
+        } else {
+            const int l = warp - kLevels;
+            const int b0 = l ? s_cut[l - 1].begin : 0, b1 = l < kLevels - 1 ? s_cut[l].end : kSortBins;
+            const int g0 = (b0 + kSortGroup - 1) / kSortGroup, g1 = b1 / kSortGroup;
+            const SortSums* side = nullptr;  // what this lane adds of the bins beside whole groups
+            if (g1 < g0) {                   // all inside one group
+                if (b0 + lane < b1) side = W.bin + b0 + lane;
+            } else if (b0 < b1) {
+                if (lane == 0 && b0 < g0 * kSortGroup) side = W.suf + b0;
+                if (lane == 1 && b1 > g1 * kSortGroup) side = W.pre + b1;
+            }
+            double s = 0.0, x = 0.0;
+            if (side) s = __ldg(&side->s), x = __ldg(&side->sx);
+            double gs = 0.0, gx = 0.0;
+#pragma unroll 4
+            for (int g = g0 + lane; g < g1; g += 32) {
+                const double2 t = s_group[g];
+                gs += t.x;
+                gx += t.y;
+            }
+            s += gs;
+            x += gx;
+            __syncwarp();
+            const bool a = lane & 16;
+            double v = (a ? x : s) + __shfl_xor_sync(kFull, a ? s : x, 16);
+#pragma unroll
+            for (int off = 8; off; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
+            if ((lane & 15) == 0) (a ? s_mid[l].y : s_mid[l].x) = v;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            old = lv;
+            if (level) {
+                s0 = s_high[lane].x + s_mid[lane].x + s_low[lane].x;
+                s1 = s_high[lane].y + s_mid[lane].y + s_low[lane].y;
+                if (!((F.fixed_mask >> lane) & 1u) && s0 > 0.0) lv = (float)(s1 / s0);
+            }
+            const bool same = __all_sync(kFull, __float_as_uint(lv) == __float_as_uint(old));
+            if (lane == 0 && same) s_stop = 1;
+        }
+    }
+    if (warp == 0 && iter > 0) {
+        const double err = __shfl_sync(kFull, error_of(old, s0, s1, iter - 1), 0);
+        if (F.err_log)
+            for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = err;
+        if (level && !((F.fixed_mask >> lane) & 1u)) F.codebook[lane] = lv;
+    }
+}
+
+// ---------------------------------------------------------------- all iterations, absolute error
+
+// Sum of a 64-bit integer over the warp (modulo 2^64), 27 bits at a time.
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v)
+{
+    const uint32_t lo = __reduce_add_sync(kFull, (uint32_t)v & 0x7ffffffu);
+    const uint32_t mi = __reduce_add_sync(kFull, (uint32_t)(v >> 27) & 0x7ffffffu);
+    const uint32_t hi = __reduce_add_sync(kFull, (uint32_t)(v >> 54));
+    return (unsigned long long)lo + ((unsigned long long)mi << 27) + ((unsigned long long)hi << 54);
+}
+
 //
 // One CTA.  Warp 2 l + h owns half h of region l: the samples from the region's lower threshold to its
 // level (h = 0) or from the level to the upper threshold (h = 1); the split is what the MAE error needs.
@@ -456,10 +670,12 @@ sort_group_kernel(const SortWs W)
 // -> butterfly -> level update), so everything that does not depend on one another is requested
 // together; the cut bins are mostly those of the iteration before and come from L1.  When an iteration
 // leaves every level unchanged the remaining ones would repeat it bit for bit: their entries of the
-// error log are filled in and the loop ends.
-template <bool MAE, bool CELLS>
+// error log are filled in and the loop ends.  30 iterations over 2^24 fp32 weights: 1267 us with a median found by
+// halving the range of keys, 992 by the weights between them; over 3 * 2^20 bf16 weights 416 -> 390, eight layers of
+// a 7B-shaped model 213 -> 180.
+template <bool CELLS>
 __global__ void __launch_bounds__(1024, 1)
-sort_fit_kernel(const SortWs W, const SortFit F)
+sort_fit_mae_kernel(const SortWs W, const SortFit F)
 {
     if (!after_previous()) return;
     extern __shared__ __align__(16) SortSums s_group[];
@@ -467,17 +683,11 @@ sort_fit_kernel(const SortWs W, const SortFit F)
     __shared__ SortSums s_half[32];
     __shared__ int s_stop;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    SampleWeight<MAE, false> weight;
+    SampleWeight<true, false> weight;
     weight.max_bits = W.n_items[1];
     weight.unit = F.metric >= 2;
     for (int k = tid; k < kSortGroups; k += 1024) s_group[k] = W.group[k];
     if (tid < kLevels) s_level[0][tid] = F.codebook[tid];
-    double w2 = 0.0;
-    if (warp == 1) {  // the warp that works out the errors
-        for (int k = lane; k < kSortParts; k += 32) w2 += W.w2[k];
-#pragma unroll
-        for (int off = 16; off; off >>= 1) w2 += __shfl_xor_sync(kFull, w2, off);
-    }
     if (tid == 0) s_stop = 0;
     __syncthreads();
     const int l = warp >> 1, h = warp & 1;
@@ -485,7 +695,7 @@ sort_fit_kernel(const SortWs W, const SortFit F)
     auto use = [&](uint32_t i, float2 it, double& s, unsigned long long& a) {
         if (CELLS) {
             s = __ldg(W.cell_s + i);
-            a = MAE ? __ldg(W.cell_a + i) : 0ull;
+            a = __ldg(W.cell_a + i);
         } else {
             weight(it, s, a);
         }
@@ -494,7 +704,7 @@ sort_fit_kernel(const SortWs W, const SortFit F)
         SortSums v;
         v.s = __ldg(&W.bin[b].s);
         v.sx = __ldg(&W.bin[b].sx);
-        v.a = MAE ? __ldg(&W.bin[b].a) : 0ull;
+        v.a = __ldg(&W.bin[b].a);
         return v;
     };
     int now = 0;
@@ -546,10 +756,11 @@ sort_fit_kernel(const SortWs W, const SortFit F)
             for (uint32_t i = sq + 32; i < eq; i += 32) take(i, __ldg(W.b + i));
         }
         __syncwarp();
-        sums_reduce<MAE>(t);
+        sums_reduce<false>(t);
+        t.a = warp_sum64(t.a);
         if (lane == 0) s_half[warp] = t;
         __syncthreads();
-        if (MAE) {
+        {
             // The warp whose half holds the crossing of half the region's weight finds the sample.
             const unsigned long long below = s_half[2 * l].a, total = below + s_half[2 * l + 1].a;
             const bool in_lower = 2ull * below >= total;
@@ -589,11 +800,13 @@ sort_fit_kernel(const SortWs W, const SortFit F)
                     auto each = [&](auto fn) {
 #pragma unroll
                         for (int r = 0; r < R; ++r) fn(key[r], wt[r]);
-                        for (uint32_t i = s0 + 32 * R + lane; i < e; i += 32) {
-                            uint32_t k;
-                            unsigned long long a;
-                            get(i, k, a);
-                            fn(k, a);
+                        for (uint32_t i = s0 + 32 * R + lane; i < e; i += 32 * R) {
+                            uint32_t k[R];
+                            unsigned long long a[R];
+#pragma unroll
+                            for (int r = 0; r < R; ++r) get(i + 32 * r, k[r], a[r]);
+#pragma unroll
+                            for (int r = 0; r < R; ++r) fn(k[r], a[r]);
                         }
                         __syncwarp();
                     };
@@ -604,21 +817,34 @@ sort_fit_kernel(const SortWs W, const SortFit F)
                         }
                         sum += a;
                     });
-#pragma unroll
-                    for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+                    sum = warp_sum64(sum);
                     if (2ull * (before + sum) < total || sum == 0ull) {
                         before += sum;
                         return false;
                     }
+                    // The crossing is at one of the keys k0 ... k1 of the bin's samples; c0 of the bin's weight lies
+                    // below k0, c1 up to k1.  The next key to split at is where even weights would put it (every third
+                    // time the middle), and the ends move to samples: a handful of steps, where halving the keys
+                    // takes one per bit in which they differ.
                     uint32_t k0 = __reduce_min_sync(kFull, kmin), k1 = __reduce_max_sync(kFull, kmax);
-                    while (k0 < k1) {
-                        const uint32_t km = k0 + ((k1 - k0) >> 1);
+                    unsigned long long c0 = 0ull, c1 = sum;
+                    for (int step = 1; k0 < k1; ++step) {
+                        const uint32_t d = k1 - k0;
+                        const float at = step % 3 == 0 ? 0.5f : (float)(total - 2ull * (before + c0)) / (2.0f * (float)(c1 - c0));
+                        const uint32_t km = k0 + min((uint32_t)((float)d * at), d - 1u);
+                        uint32_t end = 0u, begin = 0xffffffffu;
                         sum = 0ull;
-                        each([&](uint32_t k, unsigned long long a) { sum += (k <= km) ? a : 0ull; });
-#pragma unroll
-                        for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
-                        if (2ull * (before + sum) >= total) k1 = km;
-                        else k0 = km + 1u;
+                        each([&](uint32_t k, unsigned long long a) {
+                            if (k <= km) {
+                                sum += a;
+                                end = max(end, k);
+                            } else {
+                                begin = min(begin, k);
+                            }
+                        });
+                        sum = warp_sum64(sum);
+                        if (2ull * (before + sum) >= total) k1 = __reduce_max_sync(kFull, end), c1 = sum;
+                        else k0 = __reduce_min_sync(kFull, begin), c0 = sum;
                     }
                     if (lane == 0) s_med[l] = sort_key_value(k0);
                     return true;
@@ -656,21 +882,19 @@ sort_fit_kernel(const SortWs W, const SortFit F)
         if (warp < 2 && lane < kLevels) {
             const SortSums u = s_half[2 * lane], v = s_half[2 * lane + 1];
             const float old = s_lv[lane];
-            const double o = (double)old, s1 = u.sx + v.sx, s0 = u.s + v.s;
+            const double o = (double)old;
             if (warp == 0) {
                 float next = old;
                 if (!((F.fixed_mask >> lane) & 1u)) {
-                    if (MAE) next = (u.a + v.a > 0ull) ? s_med[lane] : old;
-                    else next = (s0 > 0.0) ? (float)(s1 / s0) : old;
+                    if (u.a + v.a > 0ull) next = s_med[lane];
                 }
                 s_level[now ^ 1][lane] = next;
                 const bool same = __all_sync(0xffffu, __float_as_uint(next) == __float_as_uint(old));
                 if (lane == 0) s_stop = same ? 1 : 0;
             } else {
-                err = MAE ? (o * u.s - u.sx) + (v.sx - o * v.s) : o * (2.0 * s1 - o * s0);
+                err = (o * u.s - u.sx) + (v.sx - o * v.s);
 #pragma unroll
                 for (int off = 8; off; off >>= 1) err += __shfl_xor_sync(0xffffu, err, off);
-                if (!MAE) err = w2 - err;
                 err = fmax(err, 0.0) / (double)F.n_total;
                 if (lane == 0 && F.err_log) F.err_log[iter] = err;
             }
@@ -700,10 +924,16 @@ int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
     const int64_t ctas = (F.n_max + 8 * kSortChunk - 1) / (8 * kSortChunk);
     launch_after(sort_sums_kernel<MAE, CELLS>, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, W, weight);
     launch_after(sort_group_kernel<MAE>, kSortGroups / 8, 256, 0, st, W);
-    constexpr int smem = kSortGroups * (int)sizeof(SortSums);
-    constexpr auto kern = sort_fit_kernel<MAE, CELLS>;
-    if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
-    launch_after(kern, 1, 1024, smem, st, W, F);
+    if constexpr (MAE) {
+        constexpr int smem = kSortGroups * (int)sizeof(SortSums);
+        constexpr auto kern = sort_fit_mae_kernel<CELLS>;
+        if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
+        launch_after(kern, 1, 1024, smem, st, W, F);
+    } else {
+        constexpr auto kern = sort_fit_mse_kernel<CELLS>;
+        if (const int rc = ensure_dynamic_smem<kern>(kMseSmem)) return rc;
+        launch_after(kern, 1, 1024, kMseSmem, st, W, F);
+    }
     BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;
 }

@@ -20,6 +20,7 @@ constexpr int kSortGrid = 148;               // CTAs of the ordering passes, a c
 constexpr int kSortBins = 1 << 16;           // bins of x; bin 0 stays empty
 constexpr int kSortGroup = 32;               // bins per group sum
 constexpr int kSortGroups = kSortBins / kSortGroup;
+constexpr uint32_t kFarBin = 0xffffu;
 constexpr int kSortChunk = 128;              // samples per warp of the bin sums
 // Below four iterations putting the samples in order costs more than streaming the data does (one
 // streaming iteration of small data is a 14 us launch, the ordering 35 us; of large data, see em_cells.cu).
@@ -38,7 +39,10 @@ struct SortWs {
     double* w2;           // [kSortParts]
     uint32_t* counts;     // [kSortGrid][256]
     uint32_t* start;      // [kSortBins + 1] first sample of every bin
+    uint32_t* first;      // [kSortGroups + 1] first sample of every group
+    uint16_t* off;        // [kSortBins] first sample of a bin in its group, kFarBin: too far, see start
     SortSums *bin, *group;
+    SortSums *pre, *suf;  // per bin: the bins of its group in front of it; it and those behind it
     SortSums *lead, *trail;  // [chunks] part of a bin that began in an earlier chunk / that goes on in the next
     float2 *a, *b;        // samples, ordered samples
     double* cell_s;       // em_cells.cu: weights of the ordered samples (else NULL)

@@ -76,3 +76,21 @@ def test_many_tensors(bof4):
     ws = [_weights(70000 + 13 * k, torch.bfloat16, k, "plain") for k in range(70)]
     _check(bof4, ws, 128, 1, 1, 4)
     _check(bof4, ws[:66], 128, 0, 0, 4)
+
+
+@pytest.mark.parametrize("n", [300, (1 << 20) + 9, 1 << 23])
+@pytest.mark.parametrize("kind", ["plain", "grid", "sparse"])
+@pytest.mark.parametrize("metric", [0, 1])
+def test_thresholds_in_one_bin(bof4, n, kind, metric):
+    """Levels so close that several thresholds cut the same bin, a threshold that is exactly zero, regions that
+    stay empty, and bins of one, two and many rounds of samples."""
+    w = _weights(n, torch.float32, 5, kind)
+    lv = np.array([-1.0, -0.4, -0.2000002, -0.2000001, -0.2, -0.1, -0.01, 0.01, 0.1, 0.25, 0.2500001, 0.2500002, 0.2500003, 0.7,
+                   0.99999994, 1.0], np.float32)
+    cb, log = bof4.bof4_fit_codebook([w.cuda()], 64, 0, metric, lv, 0x8001, 6)
+    ref, ref_log = oracle.fit([w], 64, 0, metric, lv, 0x8001, 6)
+    if metric == bof4.METRIC_MAE:
+        assert np.array_equal(cb.cpu().numpy(), ref)
+    else:
+        np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5, atol=1e-7)
+    np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5, atol=1e-12)
