@@ -427,6 +427,9 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
 
 // One warp per group of 32 bins: empty bins are cleared, bins that cross chunks put together (in the
 // order of the chunks), and the sums of the group, of the bins in front of each and from each on formed.
+// Bound by the latency of its loads: with all crossing bins put together one after the other by the whole warp
+// it took 14.6 us for 2^20 samples, 3.7 with those of up to kSortFew chunks a lane each (cells of 2^26 weights 22.9, 10.5).
+constexpr uint32_t kSortFew = 16;
 template <bool MAE>
 __global__ void __launch_bounds__(256)
 sort_group_kernel(const SortWs W)
@@ -437,7 +440,14 @@ sort_group_kernel(const SortWs W)
     SortSums t{0.0, 0.0, 0ull};
     const uint32_t c0 = s / kSortChunk, c1 = (e > s) ? (e - 1) / kSortChunk : c0;
     if (e > s && c0 == c1) t = W.bin[b];
-    unsigned spans = __ballot_sync(kFull, e > s && c0 != c1);
+    // a bin of a few chunks by its lane, the lanes side by side; a longer one by the warp
+    const bool few = e > s && c0 != c1 && c1 - c0 <= kSortFew;
+    if (few) {
+        t = W.trail[c0];
+#pragma unroll 4
+        for (uint32_t c = c0 + 1; c <= c1; ++c) sums_add(t, W.lead[c]);
+    }
+    unsigned spans = __ballot_sync(kFull, e > s && c0 != c1 && !few);
     while (spans) {
         const int who = __ffs(spans) - 1;
         spans &= spans - 1u;
