@@ -115,7 +115,7 @@ typedef struct bof4_em_stats {
  *                     grow with it (n_max / 8 bytes, between 8 MiB and 1 GiB); any workspace of at
  *                     least bof4_workspace_bytes(BOF4_OP_EM, 0, ...) is accepted.  A fit of four or
  *                     more iterations puts its samples in order once (16 bytes per weight up to 2^26
- *                     weights; bf16 data of 2^22 weights and more: about 90 MB and 10 bytes per block,
+ *                     weights; bf16 data of 3 * 2^19 weights and more: about 90 MB and 10 bytes per block,
  *                     BOF4_OP_EM_BF16); with a smaller workspace than asked for here it streams the data
  *                     in every iteration.  Medians do not depend on the workspace size, sums only by
  *                     their rounding.

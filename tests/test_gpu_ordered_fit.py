@@ -1,5 +1,5 @@
 """Fits of four and more iterations, which put the samples in order once: one sample per weight (fp32,
-small bf16) and one per distinct normalised weight (bf16 from 2^22 weights), against the oracle."""
+small bf16) and one per distinct normalised weight (bf16 from 3 * 2^19 weights), against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -94,3 +94,9 @@ def test_thresholds_in_one_bin(bof4, n, kind, metric):
     else:
         np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5, atol=1e-7)
     np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5, atol=1e-12)
+
+
+@pytest.mark.parametrize("n", [(3 << 19) - 1, 3 << 19, (3 << 19) + 4097])
+@pytest.mark.parametrize("metric", [0, 1])
+def test_length_from_which_samples_are_distinct_weights(bof4, n, metric):
+    _check(bof4, [_weights(n, torch.bfloat16, 3, "plain")], 64, 1, metric, 4)
