@@ -71,9 +71,9 @@ extern "C" {
 #define BOF4_METRIC_MSE_NORMALIZED 2
 #define BOF4_METRIC_MAE_NORMALIZED 3
 
-#define BOF4_OP_EM 0  /* bof4_em_step / bof4_fit_codebook workspace */
+#define BOF4_OP_EM 0  /* bof4_em_step, and a bof4_fit_codebook that streams its data */
 #define BOF4_OP_OPQ 1 /* opq_split / bof4_quantize_opq workspace    */
-#define BOF4_OP_EM_BF16 2 /* the same as BOF4_OP_EM where all tensors are bf16 (smaller) */
+#define BOF4_OP_EM_BF16 2 /* bof4_fit_codebook over bf16 tensors, any number of iterations */
 
 #define BOF4_LEVELS 16
 
@@ -113,15 +113,23 @@ typedef struct bof4_em_stats {
  *                     metric = MAE, the per-level selection histograms and candidate lists.
  *                     n_max = the TOTAL number of weights of the tensor list.  The candidate lists
  *                     grow with it (n_max / 8 bytes, between 8 MiB and 1 GiB); any workspace of at
- *                     least bof4_workspace_bytes(BOF4_OP_EM, 0, ...) is accepted.  A fit of four or
- *                     more iterations puts its samples in order once (16 bytes per weight up to 2^26
- *                     weights; bf16 data of 3 * 2^19 weights and more: about 90 MB and 10 bytes per block,
- *                     BOF4_OP_EM_BF16); with a smaller workspace than asked for here it streams the data
- *                     in every iteration.  Medians do not depend on the workspace size, sums only by
- *                     their rounding.
+ *                     least bof4_workspace_bytes(BOF4_OP_EM, 0, ...) is accepted.  A fit that is given
+ *                     no more than this streams the data in every iteration; see
+ *                     bof4_fit_workspace_bytes for the workspace with which it does not have to.
+ *   op = BOF4_OP_EM_BF16: bof4_fit_workspace_bytes of bf16 tensors for the largest number of iterations.
  *   op = BOF4_OP_OPQ: per-tile outlier staging and tile offsets of the ordered compaction.
  */
 BOF4_API size_t bof4_workspace_bytes(int op, int64_t n_max, int block_size, int metric);
+
+/*
+ * Bytes of device workspace with which bof4_fit_codebook runs `iters` iterations over n_total weights of
+ * w_dtype the fastest way it has.  Never less than BOF4_OP_EM asks for, and no more where the fit streams its
+ * data.  A fit of enough iterations puts its samples in order once instead: 16 bytes per weight (fp32, up to
+ * 2^26 weights, and bf16 up to 3 * 2^19), or about 90 MB and 10 bytes per block (bf16 from there on).
+ * Medians do not depend on the workspace size, sums only by their rounding.  Host function, no CUDA call.
+ * Returns 0 for invalid arguments.
+ */
+BOF4_API size_t bof4_fit_workspace_bytes(int64_t n_total, int w_dtype, int block_size, int metric, int iters);
 
 /*
  * One E+M accumulation pass with the codebook held fixed (Sec. 3.2; Eq. 6 or Eq. 8 with the
@@ -132,7 +140,7 @@ BOF4_API size_t bof4_workspace_bytes(int op, int64_t n_max, int block_size, int 
  *             shorter block with its own constant: blocks never run across two tensors)
  *   d_codebook  [16] fp32 levels, read only
  *   d_stats   out: one bof4_em_stats record
- *   d_ws      workspace of at least bof4_workspace_bytes(BOF4_OP_EM, max_t h_n[t], ...)
+ *   d_ws      workspace of at least bof4_workspace_bytes(BOF4_OP_EM, sum_t h_n[t], ...) bytes, or less (see there)
  * The sums are accumulated in a fixed order that depends only on the shapes, so two calls on
  * the same inputs give bit-identical statistics.
  */
@@ -148,6 +156,7 @@ BOF4_API int bof4_em_step(const void* const* h_w, const int64_t* h_n, int n_tens
  *   d_codebook  in: initial levels (ascending), out: fitted levels
  *   d_err_log   [iters] fp64 or NULL: entry t = mean error (MSE or MAE over all weights,
  *               un-normalised domain) of the levels that ENTER iteration t
+ *   d_ws        workspace: bof4_fit_workspace_bytes, or any smaller one that BOF4_OP_EM accepts
  * No host synchronisation happens inside; the whole loop is enqueued on `stream`.
  */
 BOF4_API int bof4_fit_codebook(const void* const* h_w, const int64_t* h_n, int n_tensors, int w_dtype,

@@ -51,7 +51,7 @@ def mae_launches_per_call(n_tensors: int, n_total: int, iters: int) -> int:
     return chunks + iters * (1 + 4 * chunks + (2 if small else 3))
 
 
-EXPORTS = ("bof4_workspace_bytes", "bof4_em_step", "bof4_fit_codebook", "bof4_quantize",
+EXPORTS = ("bof4_workspace_bytes", "bof4_fit_workspace_bytes", "bof4_em_step", "bof4_fit_codebook", "bof4_quantize",
            "opq_split", "opq_split_static", "bof4_quantize_opq", "bof4_dequantize", "bof4_opq_threshold",
            "bof4_default_init", "bof4_last_error", "bof4_theoretical_codebook", "bof4_theoretical_codebook_batch",
            "bof4_gemv", "bof4_outlier_count", "bof4_scales_compress", "bof4_scales_expand",
@@ -84,6 +84,8 @@ def lib() -> ctypes.CDLL:
         vp, i64, i32, sz = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_size_t
         L.bof4_workspace_bytes.restype = sz
         L.bof4_workspace_bytes.argtypes = [i32, i64, i32, i32]
+        L.bof4_fit_workspace_bytes.restype = sz
+        L.bof4_fit_workspace_bytes.argtypes = [i64, i32, i32, i32, i32]
         L.bof4_em_step.restype = i32
         L.bof4_em_step.argtypes = [vp, vp, i32, i32, i32, i32, i32, vp, vp, vp, sz, vp]
         L.bof4_fit_codebook.restype = i32
@@ -226,6 +228,11 @@ def _workspace(op: int, n_max: int, block_size: int, metric: int, device) -> tor
 
 def bof4_workspace_bytes(op: int, n_max: int, block_size: int, metric: int = METRIC_MSE) -> int:
     return int(lib().bof4_workspace_bytes(op, n_max, block_size, metric))
+
+
+def bof4_fit_workspace_bytes(n_total: int, w_dtype: int, block_size: int, metric: int, iters: int) -> int:
+    """Bytes of the workspace with which a fit runs the fastest way it has (bof4_fit_codebook allocates that many)."""
+    return int(lib().bof4_fit_workspace_bytes(n_total, w_dtype, block_size, metric, iters))
 
 
 def bof4_opq_threshold(q: float, block_size: int) -> float:

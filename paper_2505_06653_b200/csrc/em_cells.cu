@@ -91,7 +91,7 @@ static size_t cells_layout(void* base, int64_t n, int block_size, CellsWs* W)
 
 size_t cells_workspace_bytes(int64_t n, int block_size)
 {
-    return n >= kCellsMinN ? cells_layout(nullptr, n, block_size, nullptr) : 0;
+    return cells_layout(nullptr, n, block_size, nullptr);
 }
 
 // ---------------------------------------------------------------- weights and cells of one magnitude

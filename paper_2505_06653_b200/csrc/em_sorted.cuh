@@ -49,9 +49,9 @@ struct SortWs {
     unsigned long long* cell_a;
 };
 
-// Bytes of workspace of the two ways (cells: 0 where they do not apply).
-size_t cells_workspace_bytes(int64_t n, int block_size);
+// Whether distinct weights serve as samples (em_cells.cu), and the bytes of workspace they take.
 bool cells_apply(int w_dtype, int64_t n);
+size_t cells_workspace_bytes(int64_t n, int block_size);
 
 // Carves the workspace for up to n samples; returns the bytes used.
 size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W);

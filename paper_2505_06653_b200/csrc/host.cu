@@ -1,4 +1,5 @@
 // Host-only parts of the C ABI: error strings, the OPQ threshold, the default starting codebook.
+#include <limits.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -78,20 +79,25 @@ const char* bof4_last_error(void) { return bof4::g_err; }
 size_t bof4_workspace_bytes(int op, int64_t n_max, int block_size, int metric)
 {
     if (n_max < 0 || !bof4::valid_block_size(block_size)) return 0;
-    if (op == BOF4_OP_EM || op == BOF4_OP_EM_BF16) {
+    if (op == BOF4_OP_EM) {
         if (metric < BOF4_METRIC_MSE || metric > BOF4_METRIC_MAE_NORMALIZED) return 0;
-        size_t need = bof4::em_workspace_bytes_for(n_max);
-        const size_t cells = bof4::cells_workspace_bytes(n_max, block_size);
-        if (need < cells) need = cells;
-        // one sample per weight: fp32 data, and bf16 data too small for the other way
-        if (n_max >= 1 && n_max <= bof4::kSortMaxDirect && (op == BOF4_OP_EM || cells == 0)) {
-            const size_t direct = bof4::sorted_layout(nullptr, n_max, false, nullptr);
-            if (need < direct) need = direct;
-        }
-        return need;
+        return bof4::em_workspace_bytes_for(n_max);
     }
+    if (op == BOF4_OP_EM_BF16) return bof4_fit_workspace_bytes(n_max, BOF4_BF16, block_size, metric, INT_MAX);
     if (op == BOF4_OP_OPQ) return bof4::opq_layout(n_max).total;
     return 0;
+}
+
+size_t bof4_fit_workspace_bytes(int64_t n_total, int w_dtype, int block_size, int metric, int iters)
+{
+    const size_t need = bof4_workspace_bytes(BOF4_OP_EM, n_total, block_size, metric);
+    if (need == 0 || (w_dtype != BOF4_F32 && w_dtype != BOF4_BF16)) return 0;
+    size_t order = 0;
+    if (iters >= bof4::kSortMinIters) {
+        if (bof4::cells_apply(w_dtype, n_total)) order = bof4::cells_workspace_bytes(n_total, block_size);
+        else if (n_total >= 1 && n_total <= bof4::kSortMaxDirect) order = bof4::sorted_layout(nullptr, n_total, false, nullptr);
+    }
+    return need < order ? order : need;
 }
 
 // The synchronising half of the two-call pattern: the outlier-producing calls only leave the true

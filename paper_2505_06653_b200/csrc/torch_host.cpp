@@ -139,12 +139,12 @@ const float* levels_ptr(const at::Tensor& t) { return t.const_data_ptr<float>();
 
 void* stream_of(at::Device d) { return c10::cuda::getCurrentCUDAStream(d.index()).stream(); }
 
-at::Tensor workspace(PyObject* given, int op, int64_t n, int block, int metric, at::Device d)
+// The workspace given, or a new one of the bytes a size query returned (0: it refused the arguments).
+at::Tensor workspace(PyObject* given, size_t bytes, at::Device d)
 {
     if (!none(given)) return tensor(given, "workspace");
-    const size_t bytes = bof4_workspace_bytes(op, n, block, metric);
     if (bytes == 0) {
-        if (PyObject* e = PyObject_CallFunction(g_error, "is", -2, "bof4_workspace_bytes rejected the arguments")) {
+        if (PyObject* e = PyObject_CallFunction(g_error, "is", -2, "the workspace size query rejected the arguments")) {
             PyErr_SetObject(g_error, e);
             Py_DECREF(e);
         }
@@ -341,7 +341,7 @@ PyObject* quantize_opq(PyObject* const* a)
     const int dt = dtype_code(w), sd = none(a[6]) ? dt : (int)integer(a[6]);
     const c10::cuda::CUDAGuard guard(d);
     const at::Tensor cb = codebook(a[3], d);
-    const at::Tensor ws = workspace(a[7], BOF4_OP_OPQ, n, (int)block, 0, d);
+    const at::Tensor ws = workspace(a[7], bof4_workspace_bytes(BOF4_OP_OPQ, n, (int)block, 0), d);
     Ref out(none(a[8]) ? PyTuple_New(5) : PySequence_Tuple(a[8]));
     if (none(a[8])) {
         const at::Tensor t[5] = {make((n + 1) / 2, at::kByte, d), make(blocks_of(n, block), torch_dtype(sd), d),
@@ -531,7 +531,7 @@ PyObject* fit_codebook(PyObject* const* a)
         if (!done) cb = codebook(a[4], w.d).clone();
         log = make(iters > 1 ? iters : 1, at::kDouble, w.d, iters < 1);  // the fit writes every entry
     }
-    const at::Tensor ws = workspace(a[7], w.dt == BOF4_BF16 ? BOF4_OP_EM_BF16 : BOF4_OP_EM, w.total, block, metric, w.d);
+    const at::Tensor ws = workspace(a[7], bof4_fit_workspace_bytes(w.total, w.dt, block, metric, (int)iters), w.d);
     check(bof4_fit_codebook(w.ptr.data(), w.n.data(), (int)w.ptr.size(), w.dt, block, norm, metric,
                             static_cast<float*>(cb.data_ptr()), (uint32_t)integer(a[5]), (int)iters,
                             static_cast<double*>(log.data_ptr()), ws.data_ptr(), (size_t)ws.numel(), st));

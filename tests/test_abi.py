@@ -77,6 +77,34 @@ def test_workspace_sizes(L):
     assert b.bof4_workspace_bytes(b.OP_OPQ, 0, 64, 0) >= 256
 
 
+def test_only_a_fit_that_orders_its_samples_asks_for_room_for_them(L):
+    """The E step, the joint fit and short fits stream: partial records and candidate lists, whatever the data's
+    size and type.  A long fit asks for 16 bytes per fp32 weight up to 2^26, or about 90 MB and 10 bytes per block (bf16)."""
+    from paper_2505_06653_b200 import binding as b
+    base = b.bof4_workspace_bytes(b.OP_EM, 0, 64, b.METRIC_MSE)
+    assert base < 10 << 20
+    for metric in range(4):
+        for n in (1, 1 << 20, 1 << 24, 1 << 26):
+            assert b.bof4_workspace_bytes(b.OP_EM, n, 64, metric) == base
+            for dt in (b.F32, b.BF16):
+                for iters in (-1, 0, 1, 3):
+                    assert b.bof4_fit_workspace_bytes(n, dt, 64, metric, iters) == base
+        big = 1 << 28
+        stream = b.bof4_workspace_bytes(b.OP_EM, big, 64, metric)
+        assert base < stream <= base + big // 8
+        assert b.bof4_fit_workspace_bytes(big, b.F32, 64, metric, 1000) == stream      # too large to order: no cell layout either
+        for n in (1 << 20, 1 << 24, 1 << 26):
+            assert 16 * n < b.bof4_fit_workspace_bytes(n, b.F32, 64, metric, 1000) < 17 * n + (16 << 20)
+        for n in (1 << 24, 1 << 26, 1 << 30):
+            cells = b.bof4_fit_workspace_bytes(n, b.BF16, 64, metric, 1000)
+            assert 10 * (n // 64) + (50 << 20) < max(cells, stream) and cells <= max(10 * (n // 64) + (100 << 20), base + n // 8)
+            assert b.bof4_workspace_bytes(b.OP_EM_BF16, n, 64, metric) == cells
+    assert b.bof4_fit_workspace_bytes(1 << 20, 7, 64, 0, 10) == 0
+    assert b.bof4_fit_workspace_bytes(1 << 20, b.F32, 48, 0, 10) == 0
+    assert b.bof4_fit_workspace_bytes(1 << 20, b.F32, 64, 9, 10) == 0
+    assert b.bof4_fit_workspace_bytes(-1, b.F32, 64, 0, 10) == 0
+
+
 def test_argument_validation_happens_before_any_cuda_call(L):
     """Bad shapes / dtypes / pointers are rejected on the host with the documented codes."""
     from paper_2505_06653_b200 import binding as b
