@@ -139,12 +139,16 @@ _host = None
 
 
 def _native():
-    """The native half of the binding.  Raises if it has not been built."""
+    """The native half of the binding.  Raises if it has not been built, or for another torch or Python."""
     global _host
     if _host is None:
         lib()
         if not os.path.exists(HOST_PATH):
             raise ImportError("%s not found: run `python -m paper_2505_06653_b200.build`" % HOST_PATH)
+        from . import build
+        if not build.host_matches(HOST_PATH):
+            raise ImportError("%s was not built for this torch and Python (%s): run `python -m paper_2505_06653_b200.build`"
+                              % (HOST_PATH, build.host_tag()))
         spec = importlib.util.spec_from_file_location("_bof4_torch", HOST_PATH)
         m = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(m)

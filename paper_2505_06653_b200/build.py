@@ -2,7 +2,8 @@
 half of the Python binding (``csrc/torch_host.cpp``) into ``_bof4_torch.so``.
 
 sm_100a only.  Both shared libraries are built in-tree so that they travel with the source tree;
-they are rebuilt when any source or header is newer than them.
+they are rebuilt when any source or header is newer than them, and the second one also when it was
+built for another torch or Python (it uses torch's C++ interface, which is only stable within a release).
 """
 from __future__ import annotations
 
@@ -49,8 +50,24 @@ def _host_deps():
     return [HOST_SRC] + [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE) if f.endswith(".h")]
 
 
+def host_tag() -> str:
+    """What the native half of the binding is built for; the module holds it as a string."""
+    import torch
+    return "bof4 host module for torch %s, Python %s;" % (torch.__version__, sysconfig.get_config_var("SOABI"))
+
+
+def host_matches(path: str) -> bool:
+    """Whether the module at `path` was built for the torch and Python that run now (it is not loaded for this)."""
+    with open(path, "rb") as f:
+        return host_tag().encode() in f.read()
+
+
+def _host_stale() -> bool:
+    return _older(HOST_LIB, _host_deps()) or not host_matches(HOST_LIB)
+
+
 def needs_build() -> bool:
-    return _older(LIB, _sources() + _deps()) or _older(HOST_LIB, _host_deps())
+    return _older(LIB, _sources() + _deps()) or _host_stale()
 
 
 def _build_host() -> None:
@@ -63,7 +80,7 @@ def _build_host() -> None:
     inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
            os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), *["-I" + p for p in inc], HOST_SRC,
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), '-DBOF4_HOST_TAG="%s"' % host_tag(), *["-I" + p for p in inc], HOST_SRC,
            "-o", HOST_LIB, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda",
            "-lc10", "-lc10_cuda", "-L" + os.path.join(cuda, "lib64"), "-lcudart", "-L" + _HERE, "-l:" + os.path.basename(LIB),
            "-Wl,-rpath,$ORIGIN"]
@@ -77,7 +94,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     if force or _older(LIB, _sources() + _deps()):
         _build_cuda(force, verbose)
-    if force or _older(HOST_LIB, _host_deps()):
+    if force or _host_stale():
         _build_host()
     return LIB
 

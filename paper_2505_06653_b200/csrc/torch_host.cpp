@@ -19,6 +19,9 @@
 
 #include "../../include/bof4.h"
 
+// The torch and Python this module is built for: the binding looks for it in the file before it loads the module.
+__attribute__((used)) static const char g_built_for[] = BOF4_HOST_TAG;
+
 namespace {
 
 struct PySet {};  // a Python exception has been set

@@ -176,6 +176,21 @@ def test_argument_validation_happens_before_any_cuda_call(L):
     assert batch(0, None, None, None, None, None, 1, None, 0, None) == 0
 
 
+def test_native_module_of_another_torch_is_rebuilt_and_not_loaded(L, tmp_path, monkeypatch):
+    """The native half of the binding is tied to the torch and Python it was compiled against."""
+    from paper_2505_06653_b200 import binding, build
+    assert build.host_matches(binding.HOST_PATH) and not build.needs_build()
+    other = tmp_path / "_bof4_torch.so"
+    data = open(binding.HOST_PATH, "rb").read()
+    other.write_bytes(data.replace(build.host_tag().encode(), build.host_tag().replace("torch ", "torch 0").encode()[:len(build.host_tag())]))
+    monkeypatch.setattr(build, "HOST_LIB", str(other))
+    monkeypatch.setattr(binding, "HOST_PATH", str(other))
+    monkeypatch.setattr(binding, "_host", None)
+    assert build.needs_build()              # newer than every source, and stale all the same
+    with pytest.raises(ImportError, match="not built for this torch"):
+        binding._native()
+
+
 def test_binding_refuses_cpu_tensors(L):
     import torch
     from paper_2505_06653_b200 import binding as b
