@@ -753,7 +753,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 // line in one that sixteen-byte reads of neighbouring rows find without bank conflicts.
 int make_map(const void* p, bool bytes, int64_t cols, int64_t rows, int box_rows, CUtensorMap* map)
 {
-    static EncodeTiledFn fn = nullptr;
+    static std::atomic<EncodeTiledFn> known{nullptr};
+    EncodeTiledFn fn = known.load(std::memory_order_relaxed);
     if (!fn) {
         void* f = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -763,6 +764,7 @@ int make_map(const void* p, bool bytes, int64_t cols, int64_t rows, int box_rows
             return BOF4_ERR_CUDA;
         }
         fn = reinterpret_cast<EncodeTiledFn>(f);
+        known.store(fn, std::memory_order_relaxed);
     }
     const int esize = bytes ? 1 : 2;
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};

@@ -6,6 +6,10 @@
 // call against 2 ... 7 us of device time.  Here it is a few hundred nanoseconds beside the
 // allocations and the launches.  Plain CPython entry points (positional vector call); binding.py keeps the
 // signatures and their documentation.
+//
+// Other Python threads run while the library enqueues (a launch waits where the stream's queue is full) and while
+// memory is allocated (which may synchronise): what such a stretch uses is owned by this call, not borrowed
+// from a list that another thread may change.
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
@@ -51,6 +55,26 @@ void check(int rc)
         Py_DECREF(e);
     }
     throw PySet{};
+}
+
+struct NoGil {  // other Python threads run during its lifetime
+    PyThreadState* state = PyEval_SaveThread();
+    NoGil() = default;
+    NoGil(const NoGil&) = delete;
+    NoGil& operator=(const NoGil&) = delete;
+    ~NoGil() { PyEval_RestoreThread(state); }
+};
+
+// A call of the library; the arguments are already plain pointers and numbers.
+template <class... P, class... A>
+void call(int (*fn)(P...), A... args)
+{
+    int rc;
+    {
+        const NoGil others;
+        rc = fn(args...);
+    }
+    check(rc);
 }
 
 struct Ref {  // owned reference
@@ -109,17 +133,35 @@ double real(PyObject* o)
 }
 bool none(PyObject* o) { return o == Py_None; }
 
+// k uninitialised buffers.
+struct Spec {
+    int64_t numel;
+    at::ScalarType dt;
+};
+void make(at::Tensor* out, const Spec* spec, size_t k, at::Device d)
+{
+    if (g_allocator) {
+        for (size_t i = 0; i < k; ++i) {
+            Ref device(THPDevice_New(d));
+            Ref r(PyObject_CallFunction(g_allocator, "LOOO", (long long)(spec[i].numel < 0 ? 0 : spec[i].numel),
+                                        (PyObject*)torch::getTHPDtype(spec[i].dt), device.p, Py_False));
+            out[i] = tensor(r.p, "the allocator's result");
+        }
+        return;
+    }
+    const NoGil others;
+    for (size_t i = 0; i < k; ++i)
+        out[i] = at::detail::empty_cuda({spec[i].numel < 0 ? 0 : spec[i].numel}, spec[i].dt, d, std::nullopt);
+}
 at::Tensor make(int64_t numel, at::ScalarType dt, at::Device d, bool zero = false)
 {
-    if (numel < 0) numel = 0;
-    if (g_allocator) {
-        Ref device(THPDevice_New(d));
-        Ref r(PyObject_CallFunction(g_allocator, "LOOO", (long long)numel, (PyObject*)torch::getTHPDtype(dt), device.p,
-                                    zero ? Py_True : Py_False));
-        return tensor(r.p, "the allocator's result");
+    at::Tensor t;
+    const Spec spec{numel, dt};
+    make(&t, &spec, 1, d);
+    if (zero) {
+        const NoGil others;
+        t.zero_();
     }
-    at::Tensor t = at::detail::empty_cuda({numel}, dt, d, std::nullopt);
-    if (zero) t.zero_();
     return t;
 }
 PyObject* wrap(const at::Tensor& t) { return THPVariable_Wrap(t); }
@@ -162,38 +204,47 @@ struct Outliers {
     const void* val = nullptr;
     const int64_t* cnt = nullptr;
     int64_t cap = 0;
+    at::Tensor own[3];
     explicit Outliers(PyObject* o)
     {
         if (none(o)) return;
         Ref f(PySequence_Fast(o, "outliers must be (idx, val, n_out)"));
         if (PySequence_Fast_GET_SIZE(f.p) != 3) fail(PyExc_ValueError, "outliers must be (idx, val, n_out)");
         PyObject** v = PySequence_Fast_ITEMS(f.p);
-        const at::Tensor &i = dev(v[0], "outliers"), &x = dev(v[1], "outliers"), &n = dev(v[2], "outliers");
-        idx = static_cast<const int32_t*>(i.const_data_ptr());
-        val = x.const_data_ptr();
-        cnt = static_cast<const int64_t*>(n.const_data_ptr());
-        cap = i.numel();
+        for (int k = 0; k < 3; ++k) own[k] = dev(v[k], "outliers");
+        idx = static_cast<const int32_t*>(own[0].const_data_ptr());
+        val = own[1].const_data_ptr();
+        cnt = static_cast<const int64_t*>(own[2].const_data_ptr());
+        cap = own[0].numel();
     }
 };
 
+// The items of a sequence as a tuple (a new reference), or NULL with a TypeError.
+PyObject* items(PyObject* o, const char* msg)
+{
+    PyObject* t = PySequence_Tuple(o);
+    if (!t && PyErr_ExceptionMatches(PyExc_TypeError)) PyErr_SetString(PyExc_TypeError, msg);
+    return t;
+}
+
 // A list of tensors (or one tensor) of one dtype: pointers and sizes.
 struct List {
+    Ref own;  // the tensor, or a tuple of the list's
     std::vector<const void*> ptr;
     std::vector<int64_t> n;
     int64_t total = 0;
     int dt = 0;
     at::Device d = at::kCUDA;
-    explicit List(PyObject* o)
+    explicit List(PyObject* o) : own(THPVariable_Check(o) ? Py_NewRef(o) : items(o, "weights must be a tensor or a list of tensors"))
     {
         if (THPVariable_Check(o)) {
             add(o);
         } else {
-            Ref f(PySequence_Fast(o, "weights must be a tensor or a list of tensors"));
-            const Py_ssize_t k = PySequence_Fast_GET_SIZE(f.p);
+            const Py_ssize_t k = PyTuple_GET_SIZE(own.p);
             if (k == 0) fail(PyExc_ValueError, "empty tensor list");
             ptr.reserve(k);
             n.reserve(k);
-            for (Py_ssize_t i = 0; i < k; ++i) add(PySequence_Fast_GET_ITEM(f.p, i));
+            for (Py_ssize_t i = 0; i < k; ++i) add(PyTuple_GET_ITEM(own.p, i));
         }
     }
     void add(PyObject* o)
@@ -251,18 +302,20 @@ PyObject* quantize(PyObject* const* a)
     const c10::cuda::CUDAGuard guard(w.device());
     const at::Tensor cb = codebook(a[3], w.device());
     if (none(a[5])) {
-        const at::Tensor codes = make((n + 1) / 2, at::kByte, w.device());
-        const at::Tensor scales = make(blocks_of(n, block), torch_dtype(sd), w.device());
-        check(bof4_quantize(w.const_data_ptr(), dt, n, (int)block, (int)integer(a[2]), levels_ptr(cb),
-                            static_cast<uint8_t*>(codes.data_ptr()), scales.data_ptr(), sd, stream_of(w.device())));
+        at::Tensor made[2];
+        const Spec spec[2] = {{(n + 1) / 2, at::kByte}, {blocks_of(n, block), torch_dtype(sd)}};
+        make(made, spec, 2, w.device());
+        const at::Tensor &codes = made[0], &scales = made[1];
+        call(bof4_quantize, w.const_data_ptr(), dt, n, (int)block, (int)integer(a[2]), levels_ptr(cb),
+             static_cast<uint8_t*>(codes.data_ptr()), scales.data_ptr(), sd, stream_of(w.device()));
         Ref c(wrap(codes)), s(wrap(scales));
         return PyTuple_Pack(2, c.p, s.p);
     }
     Ref out(PySequence_Tuple(a[5]));
     if (PyTuple_GET_SIZE(out.p) != 2) fail(PyExc_ValueError, "out must be (codes, scales)");
-    check(bof4_quantize(w.const_data_ptr(), dt, n, (int)block, (int)integer(a[2]), levels_ptr(cb),
-                        static_cast<uint8_t*>(tensor(PyTuple_GET_ITEM(out.p, 0), "codes").data_ptr()),
-                        tensor(PyTuple_GET_ITEM(out.p, 1), "scales").data_ptr(), sd, stream_of(w.device())));
+    call(bof4_quantize, w.const_data_ptr(), dt, n, (int)block, (int)integer(a[2]), levels_ptr(cb),
+         static_cast<uint8_t*>(tensor(PyTuple_GET_ITEM(out.p, 0), "codes").data_ptr()),
+         tensor(PyTuple_GET_ITEM(out.p, 1), "scales").data_ptr(), sd, stream_of(w.device()));
     return out.release();
 }
 
@@ -277,9 +330,9 @@ PyObject* dequantize(PyObject* const* a)
     const int od = (int)integer(a[4]);
     const Outliers o(a[5]);
     const at::Tensor out = none(a[6]) ? make(n, torch_dtype(od), codes.device()) : tensor(a[6], "out");
-    check(bof4_dequantize(static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), n,
-                          (int)integer(a[2]), levels_ptr(cb), o.idx, o.val, o.cnt, o.cap, out.data_ptr(), od,
-                          stream_of(codes.device())));
+    call(bof4_dequantize, static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), n,
+         (int)integer(a[2]), levels_ptr(cb), o.idx, o.val, o.cnt, o.cap, out.data_ptr(), od,
+         stream_of(codes.device()));
     if (!none(a[6])) {
         Py_INCREF(a[6]);
         return a[6];
@@ -298,9 +351,9 @@ PyObject* gemv(PyObject* const* a)
     const at::Tensor cb = codebook(a[5], codes.device());
     const Outliers o(a[7]);
     const at::Tensor out = none(a[8]) ? make(rows, at::kFloat, codes.device()) : tensor(a[8], "out");
-    check(bof4_gemv(static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), rows, cols,
-                    (int)integer(a[4]), levels_ptr(cb), x.const_data_ptr(), dtype_code(x), o.idx, o.val, o.cnt, o.cap,
-                    static_cast<float*>(out.data_ptr()), stream_of(codes.device())));
+    call(bof4_gemv, static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), rows, cols,
+         (int)integer(a[4]), levels_ptr(cb), x.const_data_ptr(), dtype_code(x), o.idx, o.val, o.cnt, o.cap,
+         static_cast<float*>(out.data_ptr()), stream_of(codes.device()));
     if (!none(a[8])) {
         Py_INCREF(a[8]);
         return a[8];
@@ -327,10 +380,10 @@ PyObject* gemm_tc(PyObject* const* a)
     else if (PyObject_IsTrue(a[8]))
         ws = make(rows / 16 + 256 + 148 * 2 * 128 * 4 * n_rhs, at::kByte, d);  // tickets; two parts of tiles per SM
     const Outliers o(a[9]);
-    check(bof4_gemm_tc(static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), rows,
-                       cols, (int)integer(a[4]), levels_ptr(cb), x.const_data_ptr(), (int)n_rhs, o.idx, o.val, o.cnt, o.cap,
-                       static_cast<float*>(y.data_ptr()), static_cast<int*>(status.data_ptr()),
-                       ws.defined() ? ws.data_ptr() : nullptr, ws.defined() ? (size_t)ws.numel() : 0, stream_of(d)));
+    call(bof4_gemm_tc, static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), rows,
+         cols, (int)integer(a[4]), levels_ptr(cb), x.const_data_ptr(), (int)n_rhs, o.idx, o.val, o.cnt, o.cap,
+         static_cast<float*>(y.data_ptr()), static_cast<int*>(status.data_ptr()),
+         ws.defined() ? ws.data_ptr() : nullptr, ws.defined() ? (size_t)ws.numel() : 0, stream_of(d));
     Ref ry(wrap(y)), rs(wrap(status));
     return PyTuple_Pack(2, ry.p, rs.p);
 }
@@ -347,15 +400,16 @@ PyObject* quantize_opq(PyObject* const* a)
     const at::Tensor ws = workspace(a[7], bof4_workspace_bytes(BOF4_OP_OPQ, n, (int)block, 0), d);
     Ref out(none(a[8]) ? PyTuple_New(5) : PySequence_Tuple(a[8]));
     if (none(a[8])) {
-        const at::Tensor t[5] = {make((n + 1) / 2, at::kByte, d), make(blocks_of(n, block), torch_dtype(sd), d),
-                                 make(cap, at::kInt, d), make(cap, at::kBFloat16, d), make(1, at::kLong, d)};
+        at::Tensor t[5];
+        const Spec spec[5] = {{(n + 1) / 2, at::kByte}, {blocks_of(n, block), torch_dtype(sd)}, {cap, at::kInt}, {cap, at::kBFloat16}, {1, at::kLong}};
+        make(t, spec, 5, d);
         for (int k = 0; k < 5; ++k) PyTuple_SET_ITEM(out.p, k, wrap(t[k]));
     }
     if (PyTuple_GET_SIZE(out.p) != 5) fail(PyExc_ValueError, "out must be (codes, scales, idx, val, n_out)");
     auto ptr = [&](int k) { return tensor(PyTuple_GET_ITEM(out.p, k), "out").data_ptr(); };
-    check(bof4_quantize_opq(w.const_data_ptr(), dt, n, (int)block, (int)integer(a[2]), levels_ptr(cb), (float)real(a[4]),
-                            static_cast<uint8_t*>(ptr(0)), ptr(1), sd, static_cast<int32_t*>(ptr(2)), ptr(3), cap,
-                            static_cast<int64_t*>(ptr(4)), ws.data_ptr(), (size_t)ws.numel(), stream_of(d)));
+    call(bof4_quantize_opq, w.const_data_ptr(), dt, n, (int)block, (int)integer(a[2]), levels_ptr(cb), (float)real(a[4]),
+         static_cast<uint8_t*>(ptr(0)), ptr(1), sd, static_cast<int32_t*>(ptr(2)), ptr(3), cap,
+         static_cast<int64_t*>(ptr(4)), ws.data_ptr(), (size_t)ws.numel(), stream_of(d));
     return out.release();
 }
 
@@ -368,11 +422,7 @@ PyObject* outlier_count(PyObject* const* a)
     const c10::cuda::CUDAGuard guard(n_out.device());
     const int64_t cap = integer(a[1]);
     int64_t host = 0;
-    int rc;
-    Py_BEGIN_ALLOW_THREADS  // waits for the stream
-    rc = bof4_outlier_count(static_cast<const int64_t*>(n_out.const_data_ptr()), cap, &host, stream_of(n_out.device()));
-    Py_END_ALLOW_THREADS
-    check(rc);
+    call(bof4_outlier_count, static_cast<const int64_t*>(n_out.const_data_ptr()), cap, &host, stream_of(n_out.device()));
     return PyLong_FromLongLong(host);
 }
 
@@ -387,6 +437,17 @@ PyObject* quantize_batch(PyObject* const* a)
     const at::Tensor cb = codebook(a[3], w.d);
     std::vector<uint8_t*> codes(k);
     std::vector<void*> scales(k);
+    std::vector<at::Tensor> made;
+    if (none(a[5])) {
+        std::vector<Spec> spec;
+        spec.reserve(2 * k);
+        for (size_t t = 0; t < k; ++t) {
+            spec.push_back({(w.n[t] + 1) / 2, at::kByte});
+            spec.push_back({blocks_of(w.n[t], block), torch_dtype(sd)});
+        }
+        made.resize(2 * k);
+        make(made.data(), spec.data(), 2 * k, w.d);
+    }
     PyObject *lc, *ls;
     if (none(a[5])) {
         lc = PyList_New((Py_ssize_t)k);
@@ -403,7 +464,7 @@ PyObject* quantize_batch(PyObject* const* a)
     for (size_t t = 0; t < k; ++t) {
         const int64_t nc = (w.n[t] + 1) / 2, ns = blocks_of(w.n[t], block);
         if (none(a[5])) {
-            const at::Tensor c = make(nc, at::kByte, w.d), s = make(ns, torch_dtype(sd), w.d);
+            const at::Tensor &c = made[2 * t], &s = made[2 * t + 1];
             codes[t] = static_cast<uint8_t*>(c.data_ptr());
             scales[t] = s.data_ptr();
             PyList_SET_ITEM(lc, (Py_ssize_t)t, wrap(c));
@@ -416,24 +477,24 @@ PyObject* quantize_batch(PyObject* const* a)
             scales[t] = s.data_ptr();
         }
     }
-    check(bof4_quantize_batch(w.ptr.data(), w.n.data(), (int)k, w.dt, (int)block, (int)integer(a[2]), levels_ptr(cb), codes.data(),
-                              scales.data(), sd, stream_of(w.d)));
+    call(bof4_quantize_batch, w.ptr.data(), w.n.data(), (int)k, w.dt, (int)block, (int)integer(a[2]), levels_ptr(cb), codes.data(),
+         scales.data(), sd, stream_of(w.d));
     return PyTuple_Pack(2, lc, ls);
 }
 
 // (codes, scales, sizes, block_size, levels, out_dtype, out)
 PyObject* dequantize_batch(PyObject* const* a)
 {
-    Ref fc(PySequence_Fast(a[0], "codes must be a list of tensors")), fs(PySequence_Fast(a[1], "scales must be a list of tensors")),
-        fn(PySequence_Fast(a[2], "sizes must be a list"));
-    const size_t k = (size_t)PySequence_Fast_GET_SIZE(fc.p);
+    Ref fc(items(a[0], "codes must be a list of tensors")), fs(items(a[1], "scales must be a list of tensors")),
+        fn(items(a[2], "sizes must be a list"));
+    const size_t k = (size_t)PyTuple_GET_SIZE(fc.p);
     if (k == 0) fail(PyExc_ValueError, "empty tensor list");
     const int64_t block = integer(a[3]);
     const int od = (int)integer(a[5]);
     Ref lo(none(a[6]) ? PyList_New((Py_ssize_t)k) : PySequence_List(a[6]));
-    if ((size_t)PySequence_Fast_GET_SIZE(fs.p) != k || (size_t)PySequence_Fast_GET_SIZE(fn.p) != k || (size_t)PyList_GET_SIZE(lo.p) != k)
+    if ((size_t)PyTuple_GET_SIZE(fs.p) != k || (size_t)PyTuple_GET_SIZE(fn.p) != k || (size_t)PyList_GET_SIZE(lo.p) != k)
         fail(PyExc_ValueError, "buffers do not match the sizes");
-    const at::Device d = dev(PySequence_Fast_GET_ITEM(fc.p, 0), "codes").device();
+    const at::Device d = dev(PyTuple_GET_ITEM(fc.p, 0), "codes").device();
     const c10::cuda::CUDAGuard guard(d);
     const at::Tensor cb = codebook(a[4], d);
     std::vector<const uint8_t*> codes(k);
@@ -443,8 +504,8 @@ PyObject* dequantize_batch(PyObject* const* a)
     int sd = 0;
     for (size_t t = 0; t < k; ++t) {
         const Py_ssize_t i = (Py_ssize_t)t;
-        const at::Tensor &c = dev(PySequence_Fast_GET_ITEM(fc.p, i), "codes"), &s = dev(PySequence_Fast_GET_ITEM(fs.p, i), "scales");
-        const int64_t n = ns[t] = integer(PySequence_Fast_GET_ITEM(fn.p, i));
+        const at::Tensor &c = dev(PyTuple_GET_ITEM(fc.p, i), "codes"), &s = dev(PyTuple_GET_ITEM(fs.p, i), "scales");
+        const int64_t n = ns[t] = integer(PyTuple_GET_ITEM(fn.p, i));
         if (t == 0) sd = dtype_code(s);
         if (c.numel() != (n + 1) / 2 || s.numel() != blocks_of(n, block) || dtype_code(s) != sd)
             fail(PyExc_ValueError, "buffers do not match the sizes");
@@ -460,8 +521,8 @@ PyObject* dequantize_batch(PyObject* const* a)
             outs[t] = o.data_ptr();
         }
     }
-    check(bof4_dequantize_batch(codes.data(), scales.data(), sd, ns.data(), (int)k, (int)block, levels_ptr(cb), outs.data(), od,
-                                stream_of(d)));
+    call(bof4_dequantize_batch, codes.data(), scales.data(), sd, ns.data(), (int)k, (int)block, levels_ptr(cb), outs.data(), od,
+         stream_of(d));
     return lo.release();
 }
 
@@ -473,12 +534,13 @@ PyObject* scales_compress(PyObject* const* a)
     const int64_t b = scales.numel();
     const int norm = (int)integer(a[1]);
     const c10::cuda::CUDAGuard guard(d);
-    const at::Tensor q = make(b, at::kByte, d), g = make((b + 255) / 256, at::kFloat, d);
-    at::Tensor sign;
-    if (norm == BOF4_NORM_SIGNED) sign = make((b + 7) / 8, at::kByte, d);
-    check(bof4_scales_compress(scales.const_data_ptr(), dtype_code(scales), b, norm, static_cast<uint8_t*>(q.data_ptr()),
-                               static_cast<float*>(g.data_ptr()),
-                               sign.defined() ? static_cast<uint8_t*>(sign.data_ptr()) : nullptr, stream_of(d)));
+    at::Tensor made[3];  // q, group, sign (signed normalisation)
+    const Spec spec[3] = {{b, at::kByte}, {(b + 255) / 256, at::kFloat}, {(b + 7) / 8, at::kByte}};
+    make(made, spec, norm == BOF4_NORM_SIGNED ? 3 : 2, d);
+    const at::Tensor &q = made[0], &g = made[1], &sign = made[2];
+    call(bof4_scales_compress, scales.const_data_ptr(), dtype_code(scales), b, norm, static_cast<uint8_t*>(q.data_ptr()),
+         static_cast<float*>(g.data_ptr()),
+         sign.defined() ? static_cast<uint8_t*>(sign.data_ptr()) : nullptr, stream_of(d));
     Ref rq(wrap(q)), rg(wrap(g));
     if (!sign.defined()) return PyTuple_Pack(3, rq.p, rg.p, Py_None);
     Ref rs(wrap(sign));
@@ -492,8 +554,8 @@ PyObject* scales_expand(PyObject* const* a)
     const uint8_t* sign = none(a[2]) ? nullptr : static_cast<const uint8_t*>(dev(a[2], "sign").const_data_ptr());
     const c10::cuda::CUDAGuard guard(q.device());
     const at::Tensor out = make(q.numel(), at::kFloat, q.device());
-    check(bof4_scales_expand(static_cast<const uint8_t*>(q.const_data_ptr()), static_cast<const float*>(g.const_data_ptr()), sign,
-                             q.numel(), static_cast<float*>(out.data_ptr()), stream_of(q.device())));
+    call(bof4_scales_expand, static_cast<const uint8_t*>(q.const_data_ptr()), static_cast<const float*>(g.const_data_ptr()), sign,
+         q.numel(), static_cast<float*>(out.data_ptr()), stream_of(q.device()));
     return wrap(out);
 }
 
@@ -514,6 +576,7 @@ PyObject* fit_codebook(PyObject* const* a)
         if (cb.scalar_type() != at::kFloat || cb.numel() != BOF4_LEVELS || log.scalar_type() != at::kDouble || log.numel() < iters)
             fail(PyExc_ValueError, "out must be (float32[16], float64[>= iters])");
         const at::Tensor src = codebook(a[4], w.d);
+        const NoGil others;
         if (src.data_ptr() != cb.data_ptr()) cb.copy_(src);  // levels may be the output buffer itself: continue in place
     } else {
         Py_buffer view;
@@ -523,6 +586,7 @@ PyObject* fit_codebook(PyObject* const* a)
             // 16 fp32 levels of a host array: straight into the result's buffer
             if (view.len == BOF4_LEVELS * 4 && view.format && view.format[0] == 'f' && view.format[1] == 0) {
                 // through a tensor: a copy from pageable memory of this size is staged before the call returns
+                const NoGil others;
                 cb = at::detail::empty_cuda({BOF4_LEVELS}, at::kFloat, w.d, std::nullopt);
                 done = cudaMemcpyAsync(cb.data_ptr(), view.buf, (size_t)view.len, cudaMemcpyHostToDevice,
                                        static_cast<cudaStream_t>(st)) == cudaSuccess;
@@ -531,18 +595,23 @@ PyObject* fit_codebook(PyObject* const* a)
         } else {
             PyErr_Clear();
         }
-        if (!done) cb = codebook(a[4], w.d).clone();
+        if (!done) {
+            const at::Tensor src = codebook(a[4], w.d);
+            const NoGil others;
+            cb = src.clone();
+        }
         log = make(iters > 1 ? iters : 1, at::kDouble, w.d, iters < 1);  // the fit writes every entry
     }
     const at::Tensor ws = workspace(a[7], bof4_fit_workspace_bytes(w.total, w.dt, block, metric, (int)iters), w.d);
-    check(bof4_fit_codebook(w.ptr.data(), w.n.data(), (int)w.ptr.size(), w.dt, block, norm, metric,
-                            static_cast<float*>(cb.data_ptr()), (uint32_t)integer(a[5]), (int)iters,
-                            static_cast<double*>(log.data_ptr()), ws.data_ptr(), (size_t)ws.numel(), st));
+    call(bof4_fit_codebook, w.ptr.data(), w.n.data(), (int)w.ptr.size(), w.dt, block, norm, metric,
+         static_cast<float*>(cb.data_ptr()), (uint32_t)integer(a[5]), (int)iters,
+         static_cast<double*>(log.data_ptr()), ws.data_ptr(), (size_t)ws.numel(), st);
     if (PyObject_IsTrue(a[8])) {
         cudaError_t e;
-        Py_BEGIN_ALLOW_THREADS
-        e = cudaStreamSynchronize(static_cast<cudaStream_t>(st));
-        Py_END_ALLOW_THREADS
+        {
+            const NoGil others;
+            e = cudaStreamSynchronize(static_cast<cudaStream_t>(st));
+        }
         if (e != cudaSuccess) failf(PyExc_RuntimeError, "CUDA error: %s", cudaGetErrorString(e));
     }
     Ref rc(wrap(cb)), rl(wrap(log.narrow(0, 0, iters < 0 ? 0 : iters)));
