@@ -314,16 +314,16 @@ struct SampleWeight {
     }
 };
 
+// First sample of every bin: sample i is the first of all bins behind the one of sample i - 1 up to its own; behind
+// the last sample come all bins that are left, which are all there are where no sample has a weight (bf16 zeros).
 __global__ void __launch_bounds__(256)
 sort_start_kernel(const float2* __restrict__ items, const uint32_t* __restrict__ head, uint32_t* __restrict__ start)
 {
     if (!after_previous()) return;
     const uint32_t n = *head;
-    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
-        const int b = sort_bin(items[i].x), prev = i ? sort_bin(items[i - 1].x) : -1;
+    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i <= n; i += gridDim.x * 256) {
+        const int b = i < n ? sort_bin(items[i].x) : kSortBins, prev = i ? sort_bin(items[i - 1].x) : -1;
         for (int t = prev + 1; t <= b; ++t) start[t] = i;
-        if (i == n - 1)
-            for (int t = b + 1; t <= kSortBins; ++t) start[t] = n;
     }
 }
 
@@ -973,7 +973,7 @@ int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
     SortWs V = W;  // the ordered samples are in the first array
     V.a = W.b;
     V.b = W.a;
-    const int64_t ctas = (F.n_max + 255) / 256;
+    const int64_t ctas = F.n_max / 256 + 1;  // one thread beyond the samples
     launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, V.b, V.n_items, V.start);
     BOF4_CUDA_TRY(cudaGetLastError());
     const bool mae = F.metric == BOF4_METRIC_MAE || F.metric == BOF4_METRIC_MAE_NORMALIZED;

@@ -100,3 +100,10 @@ def test_thresholds_in_one_bin(bof4, n, kind, metric):
 @pytest.mark.parametrize("metric", [0, 1])
 def test_length_from_which_samples_are_distinct_weights(bof4, n, metric):
     _check(bof4, [_weights(n, torch.bfloat16, 3, "plain")], 64, 1, metric, 4)
+
+
+@pytest.mark.parametrize("metric", [0, 1, 2, 3])
+def test_zeros_alone(bof4, metric):
+    """No weight counts under the metrics of the weights: there is not a single sample, and the levels stay."""
+    _check(bof4, [torch.zeros((3 << 19) + 70, dtype=torch.bfloat16)], 64, 0, metric, 12)
+    _check(bof4, [torch.zeros(70000, dtype=torch.float32)], 64, 1, metric, 12)
