@@ -133,12 +133,13 @@ double real(PyObject* o)
 }
 bool none(PyObject* o) { return o == Py_None; }
 
-// k uninitialised buffers.
+// k uninitialised buffers, then fn(), a call of the library that may use them.
 struct Spec {
     int64_t numel;
     at::ScalarType dt;
 };
-void make(at::Tensor* out, const Spec* spec, size_t k, at::Device d)
+template <class F>
+void make_and_call(at::Tensor* out, const Spec* spec, size_t k, at::Device d, F&& fn)
 {
     if (g_allocator) {
         for (size_t i = 0; i < k; ++i) {
@@ -147,11 +148,20 @@ void make(at::Tensor* out, const Spec* spec, size_t k, at::Device d)
                                         (PyObject*)torch::getTHPDtype(spec[i].dt), device.p, Py_False));
             out[i] = tensor(r.p, "the allocator's result");
         }
-        return;
+        k = 0;
     }
-    const NoGil others;
-    for (size_t i = 0; i < k; ++i)
-        out[i] = at::detail::empty_cuda({spec[i].numel < 0 ? 0 : spec[i].numel}, spec[i].dt, d, std::nullopt);
+    int rc;
+    {
+        const NoGil others;
+        for (size_t i = 0; i < k; ++i)
+            out[i] = at::detail::empty_cuda({spec[i].numel < 0 ? 0 : spec[i].numel}, spec[i].dt, d, std::nullopt);
+        rc = fn();
+    }
+    check(rc);
+}
+void make(at::Tensor* out, const Spec* spec, size_t k, at::Device d)
+{
+    make_and_call(out, spec, k, d, [] { return BOF4_OK; });
 }
 at::Tensor make(int64_t numel, at::ScalarType dt, at::Device d, bool zero = false)
 {
@@ -304,11 +314,12 @@ PyObject* quantize(PyObject* const* a)
     if (none(a[5])) {
         at::Tensor made[2];
         const Spec spec[2] = {{(n + 1) / 2, at::kByte}, {blocks_of(n, block), torch_dtype(sd)}};
-        make(made, spec, 2, w.device());
-        const at::Tensor &codes = made[0], &scales = made[1];
-        call(bof4_quantize, w.const_data_ptr(), dt, n, (int)block, (int)integer(a[2]), levels_ptr(cb),
-             static_cast<uint8_t*>(codes.data_ptr()), scales.data_ptr(), sd, stream_of(w.device()));
-        Ref c(wrap(codes)), s(wrap(scales));
+        const int norm = (int)integer(a[2]);
+        make_and_call(made, spec, 2, w.device(), [&] {
+            return bof4_quantize(w.const_data_ptr(), dt, n, (int)block, norm, levels_ptr(cb), static_cast<uint8_t*>(made[0].data_ptr()),
+                                 made[1].data_ptr(), sd, stream_of(w.device()));
+        });
+        Ref c(wrap(made[0])), s(wrap(made[1]));
         return PyTuple_Pack(2, c.p, s.p);
     }
     Ref out(PySequence_Tuple(a[5]));
@@ -329,10 +340,14 @@ PyObject* dequantize(PyObject* const* a)
     const at::Tensor cb = codebook(a[3], codes.device());
     const int od = (int)integer(a[4]);
     const Outliers o(a[5]);
-    const at::Tensor out = none(a[6]) ? make(n, torch_dtype(od), codes.device()) : tensor(a[6], "out");
-    call(bof4_dequantize, static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), n,
-         (int)integer(a[2]), levels_ptr(cb), o.idx, o.val, o.cnt, o.cap, out.data_ptr(), od,
-         stream_of(codes.device()));
+    const int sd = dtype_code(scales), block = (int)integer(a[2]);
+    at::Tensor out;
+    const Spec spec{n, torch_dtype(od)};
+    if (!none(a[6])) out = tensor(a[6], "out");
+    make_and_call(&out, &spec, none(a[6]) ? 1 : 0, codes.device(), [&] {
+        return bof4_dequantize(static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), sd, n, block, levels_ptr(cb),
+                               o.idx, o.val, o.cnt, o.cap, out.data_ptr(), od, stream_of(codes.device()));
+    });
     if (!none(a[6])) {
         Py_INCREF(a[6]);
         return a[6];
@@ -350,10 +365,14 @@ PyObject* gemv(PyObject* const* a)
     const c10::cuda::CUDAGuard guard(codes.device());
     const at::Tensor cb = codebook(a[5], codes.device());
     const Outliers o(a[7]);
-    const at::Tensor out = none(a[8]) ? make(rows, at::kFloat, codes.device()) : tensor(a[8], "out");
-    call(bof4_gemv, static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), rows, cols,
-         (int)integer(a[4]), levels_ptr(cb), x.const_data_ptr(), dtype_code(x), o.idx, o.val, o.cnt, o.cap,
-         static_cast<float*>(out.data_ptr()), stream_of(codes.device()));
+    const int sd = dtype_code(scales), xd = dtype_code(x), block = (int)integer(a[4]);
+    at::Tensor out;
+    const Spec spec{rows, at::kFloat};
+    if (!none(a[8])) out = tensor(a[8], "out");
+    make_and_call(&out, &spec, none(a[8]) ? 1 : 0, codes.device(), [&] {
+        return bof4_gemv(static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), sd, rows, cols, block, levels_ptr(cb),
+                         x.const_data_ptr(), xd, o.idx, o.val, o.cnt, o.cap, static_cast<float*>(out.data_ptr()), stream_of(codes.device()));
+    });
     if (!none(a[8])) {
         Py_INCREF(a[8]);
         return a[8];
@@ -372,18 +391,21 @@ PyObject* gemm_tc(PyObject* const* a)
     const at::Device d = codes.device();
     const c10::cuda::CUDAGuard guard(d);
     const at::Tensor cb = codebook(a[5], d);
-    const at::Tensor y = make(rows * n_rhs, at::kFloat, d).view({rows, n_rhs});
-    const at::Tensor status = make(1, at::kInt, d, rows == 0);  // written by the call, unless there is nothing to do
-    at::Tensor ws;
-    if (!none(a[7]))
-        ws = tensor(a[7], "workspace");
-    else if (PyObject_IsTrue(a[8]))
-        ws = make(rows / 16 + 256 + 148 * 2 * 128 * 4 * n_rhs, at::kByte, d);  // tickets; two parts of tiles per SM
     const Outliers o(a[9]);
-    call(bof4_gemm_tc, static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), dtype_code(scales), rows,
-         cols, (int)integer(a[4]), levels_ptr(cb), x.const_data_ptr(), (int)n_rhs, o.idx, o.val, o.cnt, o.cap,
-         static_cast<float*>(y.data_ptr()), static_cast<int*>(status.data_ptr()),
-         ws.defined() ? ws.data_ptr() : nullptr, ws.defined() ? (size_t)ws.numel() : 0, stream_of(d));
+    const int sd = dtype_code(scales), block = (int)integer(a[4]);
+    at::Tensor made[3];  // the product, its status (written by the call), the workspace: tickets and two parts of tiles per SM
+    const Spec spec[3] = {{rows * n_rhs, at::kFloat}, {1, at::kInt}, {rows / 16 + 256 + 148 * 2 * 128 * 4 * n_rhs, at::kByte}};
+    const bool split = none(a[7]) && PyObject_IsTrue(a[8]);
+    if (!none(a[7])) made[2] = tensor(a[7], "workspace");
+    make_and_call(made, spec, split ? 3 : 2, d, [&] {
+        if (rows == 0) made[1].zero_();  // nothing to do
+        const at::Tensor& ws = made[2];
+        return bof4_gemm_tc(static_cast<const uint8_t*>(codes.const_data_ptr()), scales.const_data_ptr(), sd, rows, cols, block,
+                            levels_ptr(cb), x.const_data_ptr(), (int)n_rhs, o.idx, o.val, o.cnt, o.cap,
+                            static_cast<float*>(made[0].data_ptr()), static_cast<int*>(made[1].data_ptr()),
+                            ws.defined() ? ws.data_ptr() : nullptr, ws.defined() ? (size_t)ws.numel() : 0, stream_of(d));
+    });
+    const at::Tensor y = made[0].view({rows, n_rhs}), &status = made[1];
     Ref ry(wrap(y)), rs(wrap(status));
     return PyTuple_Pack(2, ry.p, rs.p);
 }
@@ -536,11 +558,12 @@ PyObject* scales_compress(PyObject* const* a)
     const c10::cuda::CUDAGuard guard(d);
     at::Tensor made[3];  // q, group, sign (signed normalisation)
     const Spec spec[3] = {{b, at::kByte}, {(b + 255) / 256, at::kFloat}, {(b + 7) / 8, at::kByte}};
-    make(made, spec, norm == BOF4_NORM_SIGNED ? 3 : 2, d);
+    const int sd = dtype_code(scales);
     const at::Tensor &q = made[0], &g = made[1], &sign = made[2];
-    call(bof4_scales_compress, scales.const_data_ptr(), dtype_code(scales), b, norm, static_cast<uint8_t*>(q.data_ptr()),
-         static_cast<float*>(g.data_ptr()),
-         sign.defined() ? static_cast<uint8_t*>(sign.data_ptr()) : nullptr, stream_of(d));
+    make_and_call(made, spec, norm == BOF4_NORM_SIGNED ? 3 : 2, d, [&] {
+        return bof4_scales_compress(scales.const_data_ptr(), sd, b, norm, static_cast<uint8_t*>(q.data_ptr()), static_cast<float*>(g.data_ptr()),
+                                    sign.defined() ? static_cast<uint8_t*>(sign.data_ptr()) : nullptr, stream_of(d));
+    });
     Ref rq(wrap(q)), rg(wrap(g));
     if (!sign.defined()) return PyTuple_Pack(3, rq.p, rg.p, Py_None);
     Ref rs(wrap(sign));
@@ -553,9 +576,12 @@ PyObject* scales_expand(PyObject* const* a)
     const at::Tensor &q = dev(a[0], "q"), &g = dev(a[1], "group");
     const uint8_t* sign = none(a[2]) ? nullptr : static_cast<const uint8_t*>(dev(a[2], "sign").const_data_ptr());
     const c10::cuda::CUDAGuard guard(q.device());
-    const at::Tensor out = make(q.numel(), at::kFloat, q.device());
-    call(bof4_scales_expand, static_cast<const uint8_t*>(q.const_data_ptr()), static_cast<const float*>(g.const_data_ptr()), sign,
-         q.numel(), static_cast<float*>(out.data_ptr()), stream_of(q.device()));
+    at::Tensor out;
+    const Spec spec{q.numel(), at::kFloat};
+    make_and_call(&out, &spec, 1, q.device(), [&] {
+        return bof4_scales_expand(static_cast<const uint8_t*>(q.const_data_ptr()), static_cast<const float*>(g.const_data_ptr()), sign,
+                                  q.numel(), static_cast<float*>(out.data_ptr()), stream_of(q.device()));
+    });
     return wrap(out);
 }
 
