@@ -3,7 +3,7 @@
 //
 // Launches of a fit, whatever its number of iterations: samples (one per 64 tensors), two ordering
 // passes of eight bits (count and scatter each, least significant digit first, stable), first sample of
-// every bin, sums of the bins in two steps, iterations.  Nothing depends on the order in which CTAs run:
+// every bin, full order where a bin is crowded, sums of the bins in two steps, iterations.  Nothing depends on the order in which CTAs run:
 // the samples' order, the order of every sum and hence the result are reproducible.
 #include <type_traits>
 
@@ -40,6 +40,7 @@ size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W)
     L.trail = reinterpret_cast<SortSums*>(take(chunks * sizeof(SortSums)));
     L.a = reinterpret_cast<float2*>(take((size_t)n * 8));
     L.b = reinterpret_cast<float2*>(take((size_t)n * 8));
+    L.before = nullptr;
     L.cell_s = cells ? reinterpret_cast<double*>(take((size_t)n * 8)) : nullptr;
     L.cell_a = cells ? reinterpret_cast<unsigned long long*>(take((size_t)n * 8)) : nullptr;
     if (W) *W = L;
@@ -161,6 +162,7 @@ __global__ void sort_head_kernel(uint32_t* head, uint32_t n, double* w2)
     if (threadIdx.x == 0) {
         head[0] = n;
         head[1] = 0u;
+        head[4] = 0u;
     }
     for (int k = threadIdx.x; k < kSortParts; k += blockDim.x) w2[k] = 0.0;
 }
@@ -190,6 +192,29 @@ sort_count_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ he
         atomicAdd(&s_hist[tid >> 8][(sort_bin(in[i].x) >> SHIFT) & 255], 1u);
     __syncthreads();
     if (tid < 256) counts[blockIdx.x * 256 + tid] = s_hist[0][tid] + s_hist[1][tid] + s_hist[2][tid] + s_hist[3][tid];
+}
+
+// Ranks of a warp's PER x 32 items by a digit of eight bits: item k of a lane goes behind rank[k] others of its digit
+// (those of smaller k, and of lower lanes at the same k).  cnt[256], zero before, ends as the warp's histogram.
+template <int PER, class Digit, class Valid>
+__device__ __forceinline__ void rank_in_warp(uint32_t* cnt, int lane, Digit digit, Valid valid, uint32_t (&rank)[PER])
+{
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const bool ok = valid(k);
+        const uint32_t d = digit(k);
+        unsigned peers = __ballot_sync(kFull, ok);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const unsigned with = __ballot_sync(kFull, (d >> b) & 1u);
+            peers &= ((d >> b) & 1u) ? with : ~with;
+        }
+        const uint32_t old = cnt[d];
+        __syncwarp();
+        if (ok && lane == __ffs(peers) - 1) cnt[d] = old + __popc(peers);
+        __syncwarp();
+        rank[k] = old + __popc(peers & ((1u << lane) - 1u));
+    }
 }
 
 // Stable scatter by one digit.  A sample goes to: samples with a smaller digit + samples of the same
@@ -249,22 +274,8 @@ sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ 
 #pragma unroll
         for (int k = 0; k < 8; ++k) s_cnt[warp][lane + 32 * k] = 0u;
         __syncwarp();
-#pragma unroll
-        for (int k = 0; k < kSortPerThread; ++k) {
-            const bool ok = i0 + 32 * k < hi;
-            const uint32_t d = ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u;
-            unsigned peers = __ballot_sync(kFull, ok);
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                const unsigned with = __ballot_sync(kFull, (d >> b) & 1u);
-                peers &= ((d >> b) & 1u) ? with : ~with;
-            }
-            const uint32_t old = s_cnt[warp][d];
-            __syncwarp();
-            if (ok && lane == __ffs(peers) - 1) s_cnt[warp][d] = old + __popc(peers);
-            __syncwarp();
-            rank[k] = old + __popc(peers & ((1u << lane) - 1u));
-        }
+        rank_in_warp<kSortPerThread>(s_cnt[warp], lane, [&](int k) { return ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u; },
+                                     [&](int k) { return i0 + 32 * k < hi; }, rank);
         __syncthreads();
         if (tid < 256) {
             uint32_t c[32], run = s_base[tid];
@@ -321,9 +332,22 @@ sort_start_kernel(const float2* __restrict__ items, const uint32_t* __restrict__
 {
     if (!after_previous()) return;
     const uint32_t n = *head;
+    int far0 = 0, far1 = -1;  // a gap of many empty bins, if the thread meets one: filled by the warp below
+    uint32_t far_i = 0u;
     for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i <= n; i += gridDim.x * 256) {
         const int b = i < n ? sort_bin(items[i].x) : kSortBins, prev = i ? sort_bin(items[i - 1].x) : -1;
-        for (int t = prev + 1; t <= b; ++t) start[t] = i;
+        if (b - prev > 64 && far1 < 0) {
+            far0 = prev + 1, far1 = b;
+            far_i = i;
+        } else {
+            for (int t = prev + 1; t <= b; ++t) start[t] = i;
+        }
+    }
+    __syncwarp();
+    for (unsigned far = __ballot_sync(kFull, far1 >= 0); far; far &= far - 1u) {
+        const int who = __ffs(far) - 1, t0 = __shfl_sync(kFull, far0, who), t1 = __shfl_sync(kFull, far1, who);
+        const uint32_t i = __shfl_sync(kFull, far_i, who);
+        for (int t = t0 + (threadIdx.x & 31); t <= t1; t += 32) start[t] = i;
     }
 }
 
@@ -342,6 +366,178 @@ __device__ __forceinline__ void sums_add(SortSums& t, const SortSums& v)
     t.s += v.s;
     t.sx += v.sx;
     t.a += v.a;
+}
+
+// ---------------------------------------------------------------- crowded bins
+//
+// The bins are fine where normalised weights of model layers lie, but data can put any number of samples into one:
+// few distinct values (weights that have been quantised before) or a narrow range of x.  Looked through by a warp, such bins
+// made a fit of 2^24 weights of sixteen levels 4.4 ms long (MSE) and one of medians 100 ms, whatever streaming it takes (0.4
+// and 5.2 ms for 8 iterations).  So the windows that hold part of a crowded bin are put in full order, with running sums
+// beside them; what a threshold takes of the bin, and where its weight reaches a half, is then found by bisection in every
+// window, a lane each: 1.1 and 1.3 ms, of which 0.8 are the ordering that other data takes as well.  An iteration now costs
+// at most a few bisections (14 steps of an access to L2 each) per 2^20 samples of a crowded bin, and median step.
+// Other data pays for a launch that finds nothing to do and for the test of the flag: 165.8 -> 169.3 us for 50 iterations over
+// 2^20 weights.
+
+// One CTA per window of kSortWindow samples: four stable passes of eight bits by the key of x in shared memory, then the
+// running sums (exclusive within the window, every fourth sample).
+struct WindowScratch {
+    float2 item[kSortWindow];
+    uint32_t cnt[kSortThreads / 32][256];
+    uint32_t warp[8];
+    SortSums sum[kSortThreads / 32];
+};
+template <bool MAE>
+__global__ void __launch_bounds__(kSortThreads)
+sort_windows_kernel(const SortWs W, SampleWeight<MAE, false> weight)
+{
+    if (!after_previous()) return;
+    if (W.n_items[4] == 0u) return;
+    constexpr int NT = kSortThreads, PER = kSortWindow / NT, NW = NT / 32;
+    extern __shared__ __align__(16) unsigned char s_window[];
+    WindowScratch& S = *reinterpret_cast<WindowScratch*>(s_window);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t n = W.n_items[0];
+    weight.max_bits = W.n_items[1];
+    for (uint32_t lo = blockIdx.x * kSortWindow; lo < n; lo += gridDim.x * kSortWindow) {
+        const uint32_t len = min(kSortWindow, n - lo);
+        bool crowded = false;
+        for (uint32_t i = tid; i < len; i += NT) {
+            const float2 it = W.b[lo + i];
+            const int b = sort_bin(it.x);
+            crowded = crowded || (!one_value_bin(b) && W.start[b + 1] - W.start[b] > kSortCrowd);
+            S.item[i] = it;
+        }
+        if (!__syncthreads_or(crowded)) continue;
+        const uint32_t i0 = warp * (32 * PER) + lane;
+        for (int shift = 0; shift < 32; shift += 8) {
+            float2 item[PER];
+            uint32_t rank[PER];
+#pragma unroll
+            for (int k = 0; k < PER; ++k) item[k] = (i0 + 32 * k < len) ? S.item[i0 + 32 * k] : make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) S.cnt[warp][lane + 32 * k] = 0u;
+            __syncwarp();
+            rank_in_warp<PER>(S.cnt[warp], lane, [&](int k) { return (sort_key(item[k].x) >> shift) & 255u; },
+                              [&](int k) { return i0 + 32 * k < len; }, rank);
+            __syncthreads();
+            uint32_t mine = 0u, incl = 0u;  // samples of smaller digits, then those of the same digit in earlier warps
+            if (tid < 256) {
+                for (int w = 0; w < NW; ++w) mine += S.cnt[w][tid];
+                incl = mine;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const uint32_t t = __shfl_up_sync(kFull, incl, off);
+                    if (lane >= off) incl += t;
+                }
+                if (lane == 31) S.warp[warp] = incl;
+            }
+            __syncthreads();
+            if (tid < 256) {
+                for (int k = 0; k < warp; ++k) incl += S.warp[k];
+                uint32_t run = incl - mine;
+                for (int w = 0; w < NW; ++w) {
+                    const uint32_t c = S.cnt[w][tid];
+                    S.cnt[w][tid] = run;
+                    run += c;
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if (i0 + 32 * k < len) S.item[S.cnt[warp][(sort_key(item[k].x) >> shift) & 255u] + rank[k]] = item[k];
+            __syncthreads();
+        }
+        for (uint32_t i = tid; i < len; i += NT) W.b[lo + i] = S.item[i];
+        // a thread adds up PER samples in a row
+        auto add = [&](SortSums& t, uint32_t i) {
+            if (i >= len) return;
+            const float2 it = S.item[i];
+            SortSums v;
+            weight(it, v.s, v.a);
+            v.sx = v.s * (double)it.x;
+            sums_add(t, v);
+        };
+        SortSums incl{0.0, 0.0, 0ull};
+        for (int k = 0; k < PER; ++k) add(incl, tid * PER + k);
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const SortSums u{__shfl_up_sync(kFull, incl.s, off), __shfl_up_sync(kFull, incl.sx, off),
+                             MAE ? __shfl_up_sync(kFull, incl.a, off) : 0ull};
+            if (lane >= off) sums_add(incl, u);
+        }
+        if (lane == 31) S.sum[warp] = incl;
+        SortSums run{__shfl_up_sync(kFull, incl.s, 1), __shfl_up_sync(kFull, incl.sx, 1), MAE ? __shfl_up_sync(kFull, incl.a, 1) : 0ull};
+        if (lane == 0) run = SortSums{0.0, 0.0, 0ull};
+        __syncthreads();
+        for (int k = 0; k < warp; ++k) sums_add(run, S.sum[k]);
+        for (int k = 0; k < PER; ++k) {
+            const uint32_t i = tid * PER + k;
+            if (k % 4 == 0 && i < len) W.before[(lo + i) / 4] = run;
+            add(run, i);
+        }
+        __syncthreads();  // the next window overwrites the samples
+    }
+}
+
+// Windows that a warp looks into at once, per lane: as many independent bisections in flight.
+constexpr int kWindowsPerLane = 4;
+
+// Sums of the samples of a window in front of position i (`first`: the window's first sample).
+template <bool MAE>
+__device__ __forceinline__ SortSums sums_before(const SortWs& W, const SampleWeight<MAE, false>& weight, uint32_t first, uint32_t i)
+{
+    SortSums t{0.0, 0.0, 0ull};
+    if (i <= first) return t;
+    const uint32_t q = (i - 1) / 4;
+    t = W.before[q];
+    for (uint32_t j = 4 * q; j < i; ++j) {
+        const float2 it = W.b[j];
+        double s;
+        unsigned long long a;
+        weight(it, s, a);
+        t.s += s;
+        t.sx += s * (double)it.x;
+        t.a += a;
+    }
+    return t;
+}
+
+// This lane's share of the samples of a crowded bin, from ... to - 1, with p <= x < q; the warp's lanes together have all.
+template <bool MAE>
+__device__ __noinline__ void crowded_sums(const SortWs& W, const SampleWeight<MAE, false>& weight, uint32_t from, uint32_t to, float p,
+                                          float q, SortSums& t)
+{
+    constexpr int U = kWindowsPerLane;
+    const uint32_t last = (to - 1) / kSortWindow;
+    for (uint32_t w0 = from / kSortWindow + (threadIdx.x & 31); w0 <= last; w0 += 32 * U) {
+        uint32_t lo[U], hi[U], at_p[U], at_q[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t w = w0 + 32 * u;
+            lo[u] = max(from, w * kSortWindow);
+            hi[u] = min(to, (w + 1) * kSortWindow);
+            if (w > last) lo[u] = hi[u] = to;
+            at_p[u] = at_q[u] = lo[u];
+        }
+        for (uint32_t step = kSortWindow; step; step >>= 1) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (at_p[u] + step <= hi[u] && W.b[at_p[u] + step - 1].x < p) at_p[u] += step;
+                if (at_q[u] + step <= hi[u] && W.b[at_q[u] + step - 1].x < q) at_q[u] += step;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (at_q[u] <= at_p[u]) continue;
+            const uint32_t first = (lo[u] / kSortWindow) * kSortWindow;
+            const SortSums a = sums_before<MAE>(W, weight, first, at_p[u]), b = sums_before<MAE>(W, weight, first, at_q[u]);
+            t.s += b.s - a.s;
+            t.sx += b.sx - a.sx;
+            t.a += b.a - a.a;
+        }
+    }
 }
 
 // One warp per kSortChunk ordered samples, 32 at a time: a segmented scan over the runs of equal bins.
@@ -421,6 +617,11 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
             open_key = __shfl_sync(kFull, key[k], 31);
             early = early && heads == 0u;
         }
+        // a chunk inside one bin: a crowded one has many, the first of them says so
+        if (!CELLS && early && open_key == before && lane == 0 && !one_value_bin(before)) {
+            const uint32_t s = W.start[before];
+            if (lo - s <= kSortChunk && W.start[before + 1] - s > kSortCrowd) W.n_items[4] = 1u;
+        }
         if (lane == 0 && open_key != kNone) (early ? W.lead[c] : open_key == behind ? W.trail[c] : W.bin[open_key]) = open;
     }
 }
@@ -430,6 +631,9 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
 // Bound by the latency of its loads: with all crossing bins put together one after the other by the whole warp
 // it took 14.6 us for 2^20 samples, 3.7 with those of up to kSortFew chunks a lane each (cells of 2^26 weights 22.9, 10.5).
 constexpr uint32_t kSortFew = 16;
+// A bin of very many chunks (crowded, or one of a single value: the zeros of sparse data) is put together by the whole CTA:
+// 2^24 samples within a tenth of a binade took 1910 us by a warp; 2^20 took 132, 32 this way.
+constexpr uint32_t kSortMany = 128;
 template <bool MAE>
 __global__ void __launch_bounds__(256)
 sort_group_kernel(const SortWs W)
@@ -447,7 +651,32 @@ sort_group_kernel(const SortWs W)
 #pragma unroll 4
         for (uint32_t c = c0 + 1; c <= c1; ++c) sums_add(t, W.lead[c]);
     }
-    unsigned spans = __ballot_sync(kFull, e > s && c0 != c1 && !few);
+    __shared__ uint32_t s_first[256], s_last[256], s_many[8];
+    __shared__ SortSums s_part[8];
+    const bool many = e > s && c1 - c0 > kSortMany;
+    const unsigned wide = __ballot_sync(kFull, many);
+    s_first[threadIdx.x] = c0;
+    s_last[threadIdx.x] = c1;
+    if (lane == 0) s_many[threadIdx.x >> 5] = wide;
+    if (__syncthreads_or(many)) {
+        for (int w = 0; w < 8; ++w) {
+            for (unsigned left = s_many[w]; left; left &= left - 1u) {
+                const int who = w * 32 + __ffs(left) - 1;
+                const uint32_t f = s_first[who], l = s_last[who];
+                SortSums u{0.0, 0.0, 0ull};
+#pragma unroll 4
+                for (uint32_t c = f + threadIdx.x; c <= l; c += 256) sums_add(u, (c == f) ? W.trail[c] : W.lead[c]);
+                __syncwarp();
+                sums_reduce<MAE>(u);
+                if (lane == 0) s_part[threadIdx.x >> 5] = u;
+                __syncthreads();
+                if ((int)threadIdx.x == who)
+                    for (int k = 0; k < 8; ++k) sums_add(t, s_part[k]);
+                __syncthreads();
+            }
+        }
+    }
+    unsigned spans = __ballot_sync(kFull, e > s && c0 != c1 && !few && !many);
     while (spans) {
         const int who = __ffs(spans) - 1;
         spans &= spans - 1u;
@@ -503,11 +732,11 @@ constexpr int kMseOff = kSortGroups * 16;            // shared memory: group sum
 constexpr int kMseFirst = kMseOff + kSortBins * 2;   // of the groups
 constexpr int kMseSmem = kMseFirst + (kSortGroups + 1) * 4;
 
-template <bool CELLS>
-__global__ void __launch_bounds__(1024, 1)
-sort_fit_mse_kernel(const SortWs W, const SortFit F)
+// CROWDED: a copy of the loop that also knows crowded bins.  Apart, because the calls in it cost the other one registers: 0.4 us
+// an iteration with both in one.
+template <bool CELLS, bool CROWDED>
+__device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
 {
-    if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_fit[];
     double2* const s_group = reinterpret_cast<double2*>(s_fit);
     uint16_t* const s_off = reinterpret_cast<uint16_t*>(s_fit + kMseOff);
@@ -599,8 +828,16 @@ sort_fit_mse_kernel(const SortWs W, const SortFit F)
                     if (x >= c.p && x < c.above) hs += sv, hx += xv;
                 }
             };
-            if (c.from < c.to) add(std::integral_constant<int, 2>{}, c.from + lane);
-            for (uint32_t at = c.from + 64; at < c.to; at += 128) add(std::integral_constant<int, 4>{}, at + lane);
+            if (CROWDED && c.to - c.from > kSortCrowd) {
+                const SampleWeight<false, false> weight{};
+                SortSums in{0.0, 0.0, 0ull}, out = in;
+                if (c.low) crowded_sums<false>(W, weight, c.from, c.to, c.below, c.p, in);
+                crowded_sums<false>(W, weight, c.from, c.to, c.p, c.above, out);
+                ls = in.s, lx = in.sx, hs = out.s, hx = out.sx;
+            } else {
+                if (c.from < c.to) add(std::integral_constant<int, 2>{}, c.from + lane);
+                for (uint32_t at = c.from + 64; at < c.to; at += 128) add(std::integral_constant<int, 4>{}, at + lane);
+            }
             __syncwarp();
             // four sums at once: a quarter of the warp goes on with each
             const bool a = lane & 16, q = lane & 8;
@@ -662,6 +899,15 @@ sort_fit_mse_kernel(const SortWs W, const SortFit F)
     }
 }
 
+template <bool CELLS>
+__global__ void __launch_bounds__(1024, 1)
+sort_fit_mse_kernel(const SortWs W, const SortFit F)
+{
+    if (!after_previous()) return;
+    if (!CELLS && W.n_items[4] != 0u) fit_mse<CELLS, !CELLS>(W, F);
+    else fit_mse<CELLS, false>(W, F);
+}
+
 // ---------------------------------------------------------------- all iterations, absolute error
 
 // Sum of a 64-bit integer over the warp (modulo 2^64), 27 bits at a time.
@@ -683,12 +929,75 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v)
 // error log are filled in and the loop ends.  30 iterations over 2^24 fp32 weights: 1267 us with a median found by
 // halving the range of keys, 992 by the weights between them; over 3 * 2^20 bf16 weights 416 -> 390, eight layers of
 // a 7B-shaped model 213 -> 180.
-template <bool CELLS>
-__global__ void __launch_bounds__(1024, 1)
-sort_fit_mae_kernel(const SortWs W, const SortFit F)
+
+// The sample of a crowded bin, among those with p <= x < q, at which twice the weight `before` and up to it reaches `total`;
+// false, and `before` advanced past them, where it lies behind them.  Called by a whole warp.
+__device__ __noinline__ bool crowded_median(const SortWs& W, const SampleWeight<true, false>& weight, uint32_t from, uint32_t to, float p,
+                                            float q, unsigned long long total, unsigned long long& before, float& median)
 {
-    if (!after_previous()) return;
-    extern __shared__ __align__(16) SortSums s_group[];
+    constexpr int U = kWindowsPerLane;
+    const uint32_t last = (to - 1) / kSortWindow;
+    // weight of the bin's samples with keys up to k, the largest of these keys, and the smallest key beyond
+    auto upto = [&](uint32_t k, uint32_t& end, uint32_t& begin) -> unsigned long long {
+        unsigned long long sum = 0ull;
+        uint32_t top = 0u, next = 0xffffffffu;
+        for (uint32_t w0 = from / kSortWindow + (threadIdx.x & 31); w0 <= last; w0 += 32 * U) {
+            uint32_t lo[U], hi[U], at[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t w = w0 + 32 * u;
+                lo[u] = max(from, w * kSortWindow);
+                hi[u] = min(to, (w + 1) * kSortWindow);
+                if (w > last) lo[u] = hi[u] = to;
+                at[u] = lo[u];
+            }
+            for (uint32_t step = kSortWindow; step; step >>= 1) {
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (at[u] + step <= hi[u] && sort_key(W.b[at[u] + step - 1].x) <= k) at[u] += step;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (lo[u] == hi[u]) continue;
+                if (at[u] < hi[u]) next = min(next, sort_key(W.b[at[u]].x));
+                if (at[u] == lo[u]) continue;
+                top = max(top, sort_key(W.b[at[u] - 1].x));
+                const uint32_t first = (lo[u] / kSortWindow) * kSortWindow;
+                sum += sums_before<true>(W, weight, first, at[u]).a - sums_before<true>(W, weight, first, lo[u]).a;
+            }
+        }
+        __syncwarp();
+        end = __reduce_max_sync(kFull, top);
+        begin = __reduce_min_sync(kFull, next);
+        return warp_sum64(sum);
+    };
+    const float inf = __int_as_float(0x7f800000);
+    const uint32_t kp = (p == -inf) ? 1u : sort_key(p), kq = (q == inf) ? 0xffffffffu : sort_key(q);
+    uint32_t k0, k1, other;
+    const unsigned long long skip = upto(kp - 1u, other, k0), all = upto(kq - 1u, k1, other), sum = all - skip;
+    if (sum == 0ull || 2ull * (before + sum) < total) {
+        before += sum;
+        return false;
+    }
+    unsigned long long c0 = 0ull, c1 = sum;  // as in the search over few samples
+    for (int step = 1; k0 < k1; ++step) {
+        const uint32_t d = k1 - k0;
+        const float at = step % 3 == 0 ? 0.5f : (float)(total - 2ull * (before + c0)) / (2.0f * (float)(c1 - c0));
+        const uint32_t km = k0 + min((uint32_t)((float)d * at), d - 1u);
+        uint32_t end, begin;
+        const unsigned long long c = upto(km, end, begin) - skip;
+        if (2ull * (before + c) >= total) k1 = end, c1 = c;
+        else k0 = begin, c0 = c;
+    }
+    median = sort_key_value(k0);
+    return true;
+}
+
+template <bool CELLS, bool CROWDED>
+__device__ __forceinline__ void fit_mae(const SortWs& W, const SortFit& F)
+{
+    extern __shared__ __align__(16) unsigned char s_fit[];
+    SortSums* const s_group = reinterpret_cast<SortSums*>(s_fit);
     __shared__ float s_level[2][kLevels], s_med[kLevels];
     __shared__ SortSums s_half[32];
     __shared__ int s_stop;
@@ -737,6 +1046,16 @@ sort_fit_mae_kernel(const SortWs W, const SortFit F)
         uint32_t sp = 0u, ep = 0u, sq = 0u, eq = 0u;
         if (cut_p && !one_p) sp = __ldg(W.start + bp) + lane, ep = __ldg(W.start + bp + 1);
         if (cut_q && !one_q) sq = __ldg(W.start + bq) + lane, eq = __ldg(W.start + bq + 1);
+        if (CROWDED) {
+            if (ep > kSortCrowd && ep - kSortCrowd > sp - lane) {
+                crowded_sums<true>(W, weight, sp - lane, ep, p, q, t);
+                ep = 0u;
+            }
+            if (eq > kSortCrowd && eq - kSortCrowd > sq - lane) {
+                crowded_sums<true>(W, weight, sq - lane, eq, p, q, t);
+                eq = 0u;
+            }
+        }
         const bool in_p = sp < ep, in_q = sq < eq;
         float2 ip = make_float2(0.0f, 0.0f), iq = ip;
         if (in_p) ip = __ldg(W.b + sp);
@@ -791,6 +1110,12 @@ sort_fit_mae_kernel(const SortWs W, const SortFit F)
                     }
                     constexpr int R = 4;
                     const uint32_t s0 = __ldg(W.start + b), e = __ldg(W.start + b + 1);
+                    if (CROWDED && e - s0 > kSortCrowd) {
+                        float median;
+                        if (!crowded_median(W, weight, s0, e, p, q, total, before, median)) return false;
+                        if (lane == 0) s_med[l] = median;
+                        return true;
+                    }
                     uint32_t key[R], kmin = 0xffffffffu, kmax = 0u;
                     unsigned long long wt[R], sum = 0ull;
                     auto get = [&](uint32_t i, uint32_t& k, unsigned long long& a) {
@@ -920,6 +1245,15 @@ sort_fit_mae_kernel(const SortWs W, const SortFit F)
     if (tid < kLevels && !((F.fixed_mask >> tid) & 1u)) F.codebook[tid] = s_level[now][tid];
 }
 
+template <bool CELLS>
+__global__ void __launch_bounds__(1024, 1)
+sort_fit_mae_kernel(const SortWs W, const SortFit F)
+{
+    if (!after_previous()) return;
+    if (!CELLS && W.n_items[4] != 0u) fit_mae<CELLS, !CELLS>(W, F);
+    else fit_mae<CELLS, false>(W, F);
+}
+
 // ---------------------------------------------------------------- host side
 
 namespace {
@@ -934,6 +1268,15 @@ int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
     const int64_t ctas = (F.n_max + 8 * kSortChunk - 1) / (8 * kSortChunk);
     launch_after(sort_sums_kernel<MAE, CELLS>, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, W, weight);
     launch_after(sort_group_kernel<MAE>, kSortGroups / 8, 256, 0, st, W);
+    if constexpr (!CELLS) {  // cells never crowd a bin, and no more samples than make one cannot either
+        if (F.n_max > kSortCrowd) {
+            constexpr auto kern = sort_windows_kernel<MAE>;
+            constexpr int smem = (int)sizeof(WindowScratch);
+            if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
+            const int64_t windows = (F.n_max + kSortWindow - 1) / kSortWindow;
+            launch_after(kern, (int)(windows < kSMs ? windows : kSMs), kSortThreads, smem, st, W, weight);
+        }
+    }
     if constexpr (MAE) {
         constexpr int smem = kSortGroups * (int)sizeof(SortSums);
         constexpr auto kern = sort_fit_mae_kernel<CELLS>;
@@ -973,6 +1316,7 @@ int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
     SortWs V = W;  // the ordered samples are in the first array
     V.a = W.b;
     V.b = W.a;
+    V.before = reinterpret_cast<SortSums*>(W.b);
     const int64_t ctas = F.n_max / 256 + 1;  // one thread beyond the samples
     launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, V.b, V.n_items, V.start);
     BOF4_CUDA_TRY(cudaGetLastError());

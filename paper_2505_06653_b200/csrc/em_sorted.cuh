@@ -25,6 +25,10 @@ constexpr int kSortChunk = 128;              // samples per warp of the bin sums
 // Below four iterations putting the samples in order costs more than streaming the data does (one
 // streaming iteration of small data is a 14 us launch, the ordering 35 us; of large data, see em_cells.cu).
 constexpr int kSortMinIters = 4;
+// A bin of more samples than this, crowded, is not looked through sample by sample (em_sorted.cu).  Near-Gaussian data
+// of 2^26 weights, the most there can be, has up to 3500 in a bin; 4096 take a warp 10 us.
+constexpr uint32_t kSortCrowd = 4096;
+constexpr uint32_t kSortWindow = 8192;       // samples put in full order together
 constexpr int64_t kSortMaxDirect = (int64_t)1 << 26;  // one sample per weight: 16 bytes of workspace each
 constexpr int kSortParts = 2 * kSMs + 1;     // partial sums of w^2: CTAs of the sample kernels, and the short last blocks
 
@@ -35,7 +39,8 @@ struct SortSums {      // per bin, per group, or per part of a bin
 };
 
 struct SortWs {
-    uint32_t* n_items;    // device: [0] samples, [1] bits of the largest block constant, [2..3] scale (em_cells.cu)
+    uint32_t* n_items;    // device: [0] samples, [1] bits of the largest block constant, [2..3] scale (em_cells.cu),
+                          // [4] whether a bin is crowded
     double* w2;           // [kSortParts]
     uint32_t* counts;     // [kSortGrid][256]
     uint32_t* start;      // [kSortBins + 1] first sample of every bin
@@ -45,6 +50,7 @@ struct SortWs {
     SortSums *pre, *suf;  // per bin: the bins of its group in front of it; it and those behind it
     SortSums *lead, *trail;  // [chunks] part of a bin that began in an earlier chunk / that goes on in the next
     float2 *a, *b;        // samples, ordered samples
+    SortSums* before;     // crowded bins: sums of the window's samples in front of every fourth (in the place of a)
     double* cell_s;       // em_cells.cu: weights of the ordered samples (else NULL)
     unsigned long long* cell_a;
 };
@@ -78,19 +84,19 @@ int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iter
 int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters, double* d_err_log, void* d_ws,
               size_t ws_bytes, cudaStream_t st, bool* done);
 
-// Bin of a normalised weight, monotone in x: 32768 +- the bin of |x|, which is 0 for x = 0 alone, eight
-// bins per binade below 2^-7 (1 ... 254, all of |x| < 2^-38 in the first), bins of width 1 / 32767 from there on, and
-// 32767 for |x| = 1 alone.  Zeros (sparse data) and ones (a weight per block) are the only values that
-// data is likely to hold in any number, and no threshold ever has to look into a bin of one value.
+// Bin of a normalised weight, monotone in x: 32768 +- the bin of |x|, which is 0 for x = 0 alone, 128 bins per binade
+// below 2^-7 (1 ... 4318, all of |x| < 2^-40 in the first few), bins of width 1 / 28671 from there on (the width that the
+// binade below has as well), and 32767 for |x| = 1 alone.  Zeros (sparse data) and ones (a weight per block) are the only
+// values that data is likely to hold in any number, and no threshold ever has to look into a bin of one value.
 constexpr int kBinMinus = 1, kBinZero = 32768, kBinPlus = 65535;
 __device__ __forceinline__ int sort_bin(float x)
 {
     const float a = fminf(fabsf(x), 1.0f);
     int m;
     if (a >= 0.0078125f) {
-        m = (int)(a * 32767.0f);
+        m = 4096 + (int)(a * 28671.0f);
     } else {
-        m = 255 - (960 - (int)(__float_as_uint(a) >> 20));
+        m = 4319 - (15360 - (int)(__float_as_uint(a) >> 16));
         m = (a == 0.0f) ? 0 : max(m, 1);
     }
     return x < 0.0f ? kBinZero - m : kBinZero + m;

@@ -107,3 +107,61 @@ def test_zeros_alone(bof4, metric):
     """No weight counts under the metrics of the weights: there is not a single sample, and the levels stay."""
     _check(bof4, [torch.zeros((3 << 19) + 70, dtype=torch.bfloat16)], 64, 0, metric, 12)
     _check(bof4, [torch.zeros(70000, dtype=torch.float32)], 64, 1, metric, 12)
+
+
+def _crowded(n, kind, seed):
+    """fp32 weights whose blocks of 64 start with a one (x is the weight itself) and that share few bins of x, with levels
+    whose thresholds lie among them."""
+    g = torch.Generator().manual_seed(seed)
+    u = torch.rand(n, generator=g)
+    if kind == "grid":         # sixteenths: every other threshold is one of the values
+        w, lv = torch.round(32 * u - 16) / 16, np.linspace(-1, 1, 16)
+    elif kind == "jitter":     # a few neighbouring values in every crowded bin
+        w, lv = torch.round(16 * u - 8) / 8 * (1 + torch.randint(0, 4, (n,), generator=g) * 2.0 ** -23), np.linspace(-1, 1, 16)
+    elif kind == "octave":     # everything in two bins, all thresholds as well
+        w, lv = 2.0 ** -10 * (1 + 0.2 * u), 2.0 ** -10 * (1 + np.arange(16) / 80)
+    else:                      # "tiny": the outermost bins on either side of zero
+        w, lv = (u - 0.5) * 2.0 ** -39, (np.arange(16) - 7.5) * 2.0 ** -43
+    w[::64] = 1.0
+    return w, lv.astype(np.float32)
+
+
+@pytest.mark.parametrize("n", [4096 + 64, 8192 * 2 + 5, 70001, (1 << 20) + 77])
+@pytest.mark.parametrize("kind", ["grid", "jitter", "octave", "tiny"])
+@pytest.mark.parametrize("metric", [0, 1, 2, 3])
+def test_crowded_bins(bof4, n, kind, metric):
+    """Bins of more samples than are looked through: windows put in full order and searched."""
+    w, lv = _crowded(n, kind, 11)
+    iters = 12
+    dev = [w.cuda()]
+    cb, log = bof4.bof4_fit_codebook(dev, 64, 0, metric, lv, 0x8000, iters)
+    again, log2 = bof4.bof4_fit_codebook(dev, 64, 0, metric, lv, 0x8000, iters)
+    assert torch.equal(cb, again) and torch.equal(log, log2)
+    ref, ref_log = oracle.fit([w], 64, 0, metric, lv, 0x8000, iters)
+    if metric in (1, 3):
+        assert np.array_equal(cb.cpu().numpy(), ref)
+    else:
+        np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5)
+    # the squared error is the difference of two sums: their rounding, 2^-50 of the sum of squares, is what remains of it
+    np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5, atol=2.0 ** -50 * float((w.double() ** 2).mean()))
+
+
+def test_crowded_bins_take_bounded_time(bof4):
+    """2^22 weights that have been quantised before (sixteen levels, every block with its own constant): 150 000 samples and
+    more in a bin.  Looked through by one warp, a fit takes 16 ms (medians) and streaming the data 14."""
+    g = torch.Generator().manual_seed(3)
+    n = 1 << 22
+    q = torch.randint(-7, 9, (n // 64, 64), generator=g).float()
+    q[:, 0] = 8
+    w = (q * torch.rand(n // 64, 1, generator=g) * 0.01).reshape(-1).cuda()
+    lv, mask = bof4.bof4_default_init(0)
+    for metric in (0, 1):
+        best = 1e9
+        for _ in range(3):
+            s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            s.record()
+            bof4.bof4_fit_codebook(w, 64, 0, metric, lv, mask, 32, sync=False)
+            e.record()
+            torch.cuda.synchronize()
+            best = min(best, s.elapsed_time(e))
+        assert best < 5.0, (metric, best)
