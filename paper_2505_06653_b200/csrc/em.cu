@@ -3,9 +3,10 @@
 // MSE pass (Eq. 6): every lane owns 16 consecutive weights, a block is a group of I/16 lanes.
 // Per weight: x = w / m, region c by the one-probe table search, then
 //     s1[c] += m^2 x,   s0[c] += m^2            (one packed read-modify-write)
-// and, per lane, w2 += w^2.  The error of App. B.3 follows in the combine step from
+// and, per lane, w2 += m^2 x^2.  The error of App. B.3 follows in the combine step from
 //     sum (w - m xhat[c])^2 = w2 - sum_l xhat[l] (2 s1[l] - xhat[l] s0[l]),
-// evaluated in fp64.  The level-indexed sums live in shared memory as one private column per
+// evaluated in fp64.  Between folds into fp64 every thread keeps m in units of a power of two of its own (AccScale), so
+// that m^2 neither underflows nor overflows, whatever the magnitude of the weights.  The level-indexed sums live in shared memory as one private column per
 // thread (no atomics, no bank conflicts: the bank is the lane), are folded into fp64 per-CTA
 // totals in a fixed order, written as one partial record per CTA, and combined by a single-CTA
 // kernel that also updates the free levels.  Nothing depends on scheduling, so results are
@@ -36,6 +37,38 @@ static_assert(kEmFlushIters * kLaneW < 65536, "16-bit member counters must not o
 
 // Record layout in doubles: [0,16) s1, [16,32) s0, [32,48) count (uint64 bits), [48] sum w^2.
 constexpr int kRecS1 = 0, kRecS0 = 16, kRecCnt = 32, kRecW2 = 48;
+
+// The unit, 2^exp, in which a thread adds up its block constants between two folds: the magnitude of the first
+// one that is not zero, until one is met that is more than 2^40 times as large (2048 squares of such stay finite; what was
+// added before is then 2^-80 of it).  Smaller ones keep their full precision down to 2^-63 of the unit.
+struct AccScale {
+    float inv, limit;  // 2^-exp; constants beyond the limit need a larger unit
+    int exp;
+    __device__ __forceinline__ void reset(bool unit)  // unit: all weights are 1
+    {
+        inv = 1.0f;
+        limit = unit ? __int_as_float(0x7f800000) : 0.0f;
+        exp = 0;
+    }
+    // Takes a new unit for |m| > limit; the thread's sums so far are in `col`, one per level, row_bytes apart.
+    __device__ __forceinline__ void grow(float am, unsigned char* col, uint32_t row_bytes)
+    {
+        const int e = max((int)(__float_as_uint(am) >> 23) - 127, -126);
+        if (limit > 0.0f) shrink_sums(col, row_bytes, __uint_as_float((uint32_t)max(127 + exp - e, 0) << 23));
+        inv = e == 127 ? 0x1p-127f : __uint_as_float((uint32_t)(127 - e) << 23);
+        exp = e;
+        limit = e > 87 ? __int_as_float(0x7f800000) : __uint_as_float((uint32_t)(167 + e) << 23);
+    }
+    static __device__ __noinline__ void shrink_sums(unsigned char* col, uint32_t row_bytes, float f)  // by f^2; f is 0 where it underflows
+    {
+        for (int l = 0; l < kLevels; ++l) {
+            float2* p = reinterpret_cast<float2*>(col + l * row_bytes);
+            *p = make_float2(p->x * f * f, p->y * f * f);
+        }
+    }
+    // What turns a sum into the unit of m^2.
+    static __device__ __forceinline__ double square(int exp) { return __hiloint2double((1023 + 2 * exp) << 20, 0); }
+};
 
 // What the last accumulation CTA (or the stand-alone combine kernel) does with the records.
 //   stats    != NULL: receives the combined record
@@ -272,6 +305,7 @@ em_mse_kernel(const EmTensors T, const float* levels, double* partials, const Ms
     __shared__ double s_part[NSEG][3][kLevels];
     __shared__ double s_tot[3 * kLevels];  // s1, s0, count (as uint64 bits)
     __shared__ double s_w2[NW];
+    __shared__ short s_exp[NT];  // the threads' units, for the fold
     __shared__ const void* s_ptr[kEmMaxTensors];
     __shared__ int64_t s_n[kEmMaxTensors], s_row_end[kEmMaxTensors];
 
@@ -299,9 +333,13 @@ em_mse_kernel(const EmTensors T, const float* levels, double* partials, const Ms
     double w2sum = 0.0;
     int t_cur = 0;
     int since_flush = 0;
+    AccScale scale;
+    scale.reset(unit);
 
     // Folds the private fp32 columns into the fp64 CTA totals (fixed order) and clears them.
     auto flush = [&]() {
+        s_exp[tid] = (short)scale.exp;
+        scale.reset(unit);
         __syncthreads();
         {
             const int l = warp & (kLevels - 1), seg = warp >> 4;
@@ -313,8 +351,9 @@ em_mse_kernel(const EmTensors T, const float* levels, double* partials, const Ms
                 const int col = seg * (NT / NSEG) + k * 32 + lane;
                 float2* pa = reinterpret_cast<float2*>(s_acc + l * G::acc_row_bytes + col * 8);
                 const float2 a = *pa;
-                a1 += (double)a.x;
-                a0 += (double)a.y;
+                const double sq = AccScale::square(s_exp[col]);
+                a1 = fma((double)a.x, sq, a1);
+                a0 = fma((double)a.y, sq, a0);
                 *pa = make_float2(0.0f, 0.0f);
                 if (COUNT) {
                     uint16_t* pc = reinterpret_cast<uint16_t*>(s_cnt + l * (G::acc_row_bytes / 4) + col * 2);
@@ -377,22 +416,17 @@ em_mse_kernel(const EmTensors T, const float* levels, double* partials, const Ms
         float x[kLaneW];
         normalise16<false>(v, m, safe && DT::code == BF16::code, x);
         float2 sq = make_float2(0.0f, 0.0f);
-        if (unit) {  // App. D variant: the error is measured on x
 #pragma unroll
-            for (int k = 0; k < kLaneW / 2; ++k) {
-                const float2 vv = make_float2(x[2 * k], x[2 * k + 1]);
-                sq = __ffma2_rn(vv, vv, sq);
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < kLaneW / 2; ++k) {
-                const float2 vv = make_float2(v[2 * k], v[2 * k + 1]);
-                sq = __ffma2_rn(vv, vv, sq);
-            }
+        for (int k = 0; k < kLaneW / 2; ++k) {
+            const float2 xx = make_float2(x[2 * k], x[2 * k + 1]);
+            sq = __ffma2_rn(xx, xx, sq);
         }
-        if (ok) w2sum += (double)(sq.x + sq.y);
         if (ok) {
-            const float m2 = unit ? 1.0f : m * m;
+            const float am = fabsf(m);
+            if (am > scale.limit) scale.grow(am, s_acc + tid_off, G::acc_row_bytes);
+            const double md = unit ? 1.0 : (double)m;  // unit: App. D variant, the error is measured on x
+            w2sum += (double)(sq.x + sq.y) * (md * md);
+            const float ms = m * scale.inv, m2 = unit ? 1.0f : ms * ms;
             const float2 mm = make_float2(m2, m2);
             if (lut_ok && safe) {
 #pragma unroll
@@ -504,7 +538,7 @@ __device__ __forceinline__ void em_add(unsigned char* s_acc, unsigned char* s_cn
 // One row of a lane the slow way (true quotients, binary search against the true thresholds).
 // Out of line.
 template <bool COUNT>
-__device__ __noinline__ float em_row32_slow(Raw32 raw, float m, float mm, bool unit, const float* s_xi,
+__device__ __noinline__ float em_row32_slow(Raw32 raw, float m, float mm, const float* s_xi,
                                             unsigned char* s_acc, unsigned char* s_cnt, uint32_t tid_off,
                                             uint32_t row_bytes)
 {
@@ -515,9 +549,8 @@ __device__ __noinline__ float em_row32_slow(Raw32 raw, float m, float mm, bool u
     float2 sq = make_float2(0.0f, 0.0f);
 #pragma unroll 4
     for (int k = 0; k < 16; ++k) {
-        const float2 v = make_float2(bf_lo(u[k]), bf_hi(u[k]));
-        const float2 x = exact_quotient2(v, m, r, recip);
-        sq = unit ? __ffma2_rn(x, x, sq) : __ffma2_rn(v, v, sq);
+        const float2 x = exact_quotient2(make_float2(bf_lo(u[k]), bf_hi(u[k])), m, r, recip);
+        sq = __ffma2_rn(x, x, sq);
         em_add<COUNT>(s_acc, s_cnt, (uint32_t)region_of(x.x, s_xi) * row_bytes + tid_off, mm, x.x);
         em_add<COUNT>(s_acc, s_cnt, (uint32_t)region_of(x.y, s_xi) * row_bytes + tid_off, mm, x.y);
     }
@@ -540,6 +573,7 @@ em_mse32_kernel(const EmTensors T, const float* levels, double* partials, const 
     __shared__ double s_part[NSEG][3][kLevels];
     __shared__ double s_tot[3 * kLevels];  // s1, s0, count (as uint64 bits)
     __shared__ double s_w2[NW];
+    __shared__ short s_exp[NT];  // the threads' units, for the fold
     __shared__ const void* s_ptr[kEmMaxTensors];
     __shared__ int64_t s_n[kEmMaxTensors], s_row_end[kEmMaxTensors];
 
@@ -565,9 +599,13 @@ em_mse32_kernel(const EmTensors T, const float* levels, double* partials, const 
     double w2sum = 0.0;
     int t_cur = 0;
     int since_flush = 0;
+    AccScale scale;
+    scale.reset(unit);
 
     // Folds the private fp32 columns into the fp64 CTA totals (fixed order) and clears them.
     auto flush = [&]() {
+        s_exp[tid] = (short)scale.exp;
+        scale.reset(unit);
         __syncthreads();
         {
             const int l = warp & (kLevels - 1), seg = warp >> 4;
@@ -579,8 +617,9 @@ em_mse32_kernel(const EmTensors T, const float* levels, double* partials, const 
                 const int col = seg * (NT / NSEG) + k * 32 + lane;
                 float2* pa = reinterpret_cast<float2*>(s_acc + l * G::acc_row_bytes + col * 8);
                 const float2 a = *pa;
-                a1 += (double)a.x;
-                a0 += (double)a.y;
+                const double sq = AccScale::square(s_exp[col]);
+                a1 = fma((double)a.x, sq, a1);
+                a0 = fma((double)a.y, sq, a0);
                 *pa = make_float2(0.0f, 0.0f);
                 if (COUNT) {
                     uint16_t* pc = reinterpret_cast<uint16_t*>(s_cnt + l * (G::acc_row_bytes / 4) + col * 2);
@@ -637,7 +676,9 @@ em_mse32_kernel(const EmTensors T, const float* levels, double* partials, const 
         float mx, mn, g;
         lane_minmax32(u, mx, mn);
         const float m = block_constant32<I, SIGNED>(u, mx, mn, g, &s_wide);
-        const float mm = unit ? 1.0f : m * m;
+        const float am = fabsf(m);
+        if (am > scale.limit) scale.grow(am, s_acc + tid_off, G::acc_row_bytes);
+        const float ms = m * scale.inv, mm = unit ? 1.0f : ms * ms;
         float sq;
         if (row_is_fast(g, m, ok, fast_ok, &s_info)) {
             const float r = __frcp_rn(m);
@@ -648,16 +689,17 @@ em_mse32_kernel(const EmTensors T, const float* levels, double* partials, const 
                 const float2 v = make_float2(bf_lo(u[k]), bf_hi(u[k]));
                 const float2 x = __fmul2_rn(v, rr);
                 const float2 key = lut_key2(x);
-                sq2 = unit ? __ffma2_rn(x, x, sq2) : __ffma2_rn(v, v, sq2);
+                sq2 = __ffma2_rn(x, x, sq2);
                 const uint2 e0 = lut_probe<G::lut_rep>(key.x, lut_base), e1 = lut_probe<G::lut_rep>(key.y, lut_base);
                 em_add<COUNT>(s_acc, s_cnt, e0.y + ((x.x >= __uint_as_float(e0.x)) ? G::acc_row_bytes : 0u) + tid_off, mm, x.x);
                 em_add<COUNT>(s_acc, s_cnt, e1.y + ((x.y >= __uint_as_float(e1.x)) ? G::acc_row_bytes : 0u) + tid_off, mm, x.y);
             }
             sq = sq2.x + sq2.y;
         } else {
-            sq = ok ? em_row32_slow<COUNT>(raw, m, mm, unit, s_xi, s_acc, s_cnt, tid_off, G::acc_row_bytes) : 0.0f;
+            sq = ok ? em_row32_slow<COUNT>(raw, m, mm, s_xi, s_acc, s_cnt, tid_off, G::acc_row_bytes) : 0.0f;
         }
-        w2sum += (double)sq;
+        const double md = unit ? 1.0 : (double)m;
+        w2sum += (double)sq * (md * md);
         if (++since_flush == G::flush_rows) {
             flush();
             since_flush = 0;
