@@ -945,7 +945,7 @@ extern "C" int bof4_fit_codebook(const void* const* h_w, const int64_t* h_n, int
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     double* partials = static_cast<double*>(d_ws);
-    // Four or more iterations: put the samples in order once (em_cells.cu, em_sorted.cu); fewer, or a
+    // Enough iterations for it to pay (ordering_pays): put the samples in order once (em_cells.cu, em_sorted.cu); fewer, or a
     // workspace that does not hold them: stream the data in every iteration.
     bool done = false;
     if ((rc = cells_fit(a, d_codebook, fixed_mask, iters, d_err_log, d_ws, ws_bytes, st, &done)) || done) return rc;

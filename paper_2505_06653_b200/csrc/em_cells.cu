@@ -619,7 +619,7 @@ int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters
               size_t ws_bytes, cudaStream_t st, bool* done)
 {
     *done = false;
-    if (!cells_apply(a.w_dtype, a.n_total) || iters < kSortMinIters) return BOF4_OK;
+    if (!cells_apply(a.w_dtype, a.n_total) || !ordering_pays(a.w_dtype, a.n_total, a.metric, iters, true)) return BOF4_OK;
     CellsWs W;
     if (cells_layout(d_ws, a.n_total, a.block_size, &W) > ws_bytes) return BOF4_OK;
     *done = true;

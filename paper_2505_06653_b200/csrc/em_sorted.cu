@@ -732,7 +732,7 @@ constexpr int kMseOff = kSortGroups * 16;            // shared memory: group sum
 constexpr int kMseFirst = kMseOff + kSortBins * 2;   // of the groups
 constexpr int kMseSmem = kMseFirst + (kSortGroups + 1) * 4;
 
-// CROWDED: a copy of the loop that also knows crowded bins.  Apart, because the calls in it cost the other one registers: 0.4 us
+// CROWDED: a copy of the loop that also knows crowded bins.  Apart, because the calls in it cost the other one registers: 0.3 us
 // an iteration with both in one.
 template <bool CELLS, bool CROWDED>
 __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
@@ -1329,7 +1329,7 @@ int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iter
                size_t ws_bytes, cudaStream_t st, bool* done)
 {
     *done = false;
-    if (iters < kSortMinIters || a.n_total < 1 || a.n_total > kSortMaxDirect) return BOF4_OK;
+    if (a.n_total > kSortMaxDirect || !ordering_pays(a.w_dtype, a.n_total, a.metric, iters, false)) return BOF4_OK;
     SortWs W;
     if (sorted_layout(d_ws, a.n_total, false, &W) > ws_bytes) return BOF4_OK;
     *done = true;

@@ -92,11 +92,9 @@ size_t bof4_fit_workspace_bytes(int64_t n_total, int w_dtype, int block_size, in
 {
     const size_t need = bof4_workspace_bytes(BOF4_OP_EM, n_total, block_size, metric);
     if (need == 0 || (w_dtype != BOF4_F32 && w_dtype != BOF4_BF16)) return 0;
-    size_t order = 0;
-    if (iters >= bof4::kSortMinIters) {
-        if (bof4::cells_apply(w_dtype, n_total)) order = bof4::cells_workspace_bytes(n_total, block_size);
-        else if (n_total >= 1 && n_total <= bof4::kSortMaxDirect) order = bof4::sorted_layout(nullptr, n_total, false, nullptr);
-    }
+    const bool cells = bof4::cells_apply(w_dtype, n_total);
+    if ((!cells && n_total > bof4::kSortMaxDirect) || !bof4::ordering_pays(w_dtype, n_total, metric, iters, cells)) return need;
+    const size_t order = cells ? bof4::cells_workspace_bytes(n_total, block_size) : bof4::sorted_layout(nullptr, n_total, false, nullptr);
     return need < order ? order : need;
 }
 

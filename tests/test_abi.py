@@ -105,6 +105,28 @@ def test_only_a_fit_that_orders_its_samples_asks_for_room_for_them(L):
     assert b.bof4_fit_workspace_bytes(-1, b.F32, 64, 0, 10) == 0
 
 
+# (type, log2 of the weights, metric): iterations that are streamed, iterations that are ordered, by the times measured
+ROUTES = [("f32", 20, 0, 4, 8), ("f32", 22, 0, 8, 16), ("f32", 24, 0, 16, 32), ("f32", 26, 0, 32, 60),
+          ("f32", 20, 1, 3, 4), ("f32", 22, 1, 3, 4), ("f32", 24, 1, 8, 16), ("f32", 26, 1, 16, 32),
+          ("bf16", 21, 0, 4, 8), ("bf16", 22, 0, 4, 8), ("bf16", 24, 0, 3, 6), ("bf16", 26, 0, 3, 4), ("bf16", 30, 0, 3, 4),
+          ("bf16", 22, 1, 3, 4), ("bf16", 28, 1, 3, 4)]
+
+
+@pytest.mark.parametrize("dtype,lg,metric,few,many", ROUTES)
+def test_a_fit_is_ordered_where_that_is_faster(L, dtype, lg, metric, few, many):
+    """The rule that picks between streaming the data and ordering it once, on either side of where the two cross (seen by
+    the workspace a fit asks for)."""
+    from paper_2505_06653_b200 import binding as b
+    dt = b.F32 if dtype == "f32" else b.BF16
+    size = lambda iters: b.bof4_fit_workspace_bytes(1 << lg, dt, 64, metric, iters)  # noqa: E731
+    order = [size(it) for it in range(1, 101)]
+    assert order == sorted(order)
+    assert size(few) == b.bof4_workspace_bytes(b.OP_EM, 1 << lg, 64, metric)
+    assert size(many) == size(1000)
+    if lg < 30:      # beyond, the candidate lists of a streamed fit are larger than the cells
+        assert size(many) > size(few)
+
+
 def test_argument_validation_happens_before_any_cuda_call(L):
     """Bad shapes / dtypes / pointers are rejected on the host with the documented codes."""
     from paper_2505_06653_b200 import binding as b

@@ -1,4 +1,4 @@
-"""Fits of four and more iterations, which put the samples in order once: one sample per weight (fp32,
+"""Fits of enough iterations, which put the samples in order once: one sample per weight (fp32,
 small bf16) and one per distinct normalised weight (bf16 from 3 * 2^19 weights), against the oracle."""
 import numpy as np
 import pytest
@@ -63,6 +63,38 @@ def test_one_sample_per_weight(bof4, sizes, metric, dtype):
 @pytest.mark.parametrize("norm", [0, 1])
 def test_one_sample_per_distinct_weight(bof4, n, I, kind, mask, metric, norm):
     _check(bof4, [_weights(n, torch.bfloat16, 7, kind)], I, norm, metric, 4, mask)
+
+
+@pytest.mark.parametrize("sizes", [(8192 * 148 + 5,), (1 << 20, 70001)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_one_sample_per_weight_long(bof4, sizes, dtype):
+    """Sizes from which a few iterations are streamed, with more of them."""
+    _check(bof4, [_weights(n, dtype, 200 + k, "plain") for k, n in enumerate(sizes)], 64, 1, 0, 10)
+
+
+@pytest.mark.parametrize("n,I,kind,mask", [((1 << 22), 64, "plain", None), ((1 << 22) + 37, 32, "sparse", 0),
+                                           ((1 << 22) + 4095, 4096, "grid", 0), ((1 << 22) + 64, 64, "scales", None),
+                                           ((1 << 22) + 1, 1024, "subnormal", None), ((3 << 19), 64, "plain", None)])
+@pytest.mark.parametrize("norm", [0, 1])
+def test_one_sample_per_distinct_weight_long(bof4, n, I, kind, mask, norm):
+    _check(bof4, [_weights(n, torch.bfloat16, 7, kind)], I, norm, 0, 8, mask)
+
+
+def test_many_tensors_long(bof4):
+    ws = [_weights(70000 + 13 * k, torch.bfloat16, k, "plain") for k in range(66)]
+    _check(bof4, ws, 128, 0, 0, 8)
+
+
+@pytest.mark.parametrize("dtype,n,metric,iters", [(torch.float32, 1 << 20, 0, (5, 6)), (torch.float32, 1 << 21, 0, (7, 8)),
+                                                  (torch.float32, 1 << 23, 1, (6, 7)), (torch.bfloat16, 1 << 21, 0, (5, 6))])
+def test_both_sides_of_the_switch_over(bof4, dtype, n, metric, iters):
+    """One iteration apart, one fit is streamed and the other ordered; the same oracle."""
+    from paper_2505_06653_b200 import binding as b
+    dt = b.F32 if dtype == torch.float32 else b.BF16
+    a, z = (b.bof4_fit_workspace_bytes(n, dt, 64, metric, it) for it in iters)
+    assert a < z
+    for it in iters:
+        _check(bof4, [_weights(n, dtype, 9, "plain")], 64, 0, metric, it)
 
 
 def test_converged_fit_fills_the_rest_of_the_log(bof4):
