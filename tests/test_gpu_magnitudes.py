@@ -56,3 +56,26 @@ def test_squares_neither_underflow_nor_overflow(bof4, kind, dtype, metric):
         cb, log = bof4.bof4_fit_codebook(dev, 64, 1, metric, LV, 0x8080, iters, workspace=ws)
         np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5, atol=1e-7)
         np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5)
+
+
+def test_a_larger_workspace_makes_no_median_slower(bof4):
+    """2^24 weights of sixteen levels: candidate lists as long as a workspace of 16 bytes per weight would hold are never filled."""
+    g = torch.Generator().manual_seed(3)
+    n = 1 << 24
+    q = torch.randint(-7, 9, (n // 64, 64), generator=g).float()
+    q[:, 0] = 8
+    w = (q * torch.rand(n // 64, 1, generator=g) * 0.01).reshape(-1).cuda()
+    lv, mask = bof4.bof4_default_init(0)
+    ms = []
+    for nbytes in (bof4.bof4_workspace_bytes(bof4.OP_EM, n, 64, 1), 16 * n):
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        best = 1e9
+        for _ in range(3):
+            s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            s.record()
+            bof4.bof4_fit_codebook(w, 64, 0, 1, lv, mask, 2, workspace=ws, sync=False)
+            e.record()
+            torch.cuda.synchronize()
+            best = min(best, s.elapsed_time(e))
+        ms.append(best)
+    assert ms[1] < 2 * ms[0], ms
