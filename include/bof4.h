@@ -158,6 +158,9 @@ BOF4_API int bof4_em_step(const void* const* h_w, const int64_t* h_n, int n_tens
  *               un-normalised domain) of the levels that ENTER iteration t
  *   d_ws        workspace: bof4_fit_workspace_bytes, or any smaller one that BOF4_OP_EM accepts
  * No host synchronisation happens inside; the whole loop is enqueued on `stream`.
+ * Two limits of a fit over bf16 weights that puts its samples in order: a normalised weight of 2^-40 and less counts as the
+ * power of two at or below it, with its sign (so it falls on the right side of a threshold at zero, and a level moves by no more
+ * than 2^-40); and a block constant below 2^-38 of the largest enters the sums of m^2 with fewer bits, below 2^-46 not at all.
  */
 BOF4_API int bof4_fit_codebook(const void* const* h_w, const int64_t* h_n, int n_tensors, int w_dtype,
                       int block_size, int norm, int metric, float* d_codebook,

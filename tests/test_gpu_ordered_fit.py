@@ -197,3 +197,22 @@ def test_crowded_bins_take_bounded_time(bof4):
             torch.cuda.synchronize()
             best = min(best, s.elapsed_time(e))
         assert best < 5.0, (metric, best)
+
+
+@pytest.mark.parametrize("tail", [0, 37])
+@pytest.mark.parametrize("unit", [1.0, 2.0 ** -80])
+@pytest.mark.parametrize("metric", [0, 1, 2, 3])
+def test_normalised_weights_near_zero_keep_their_sign(bof4, tail, unit, metric):
+    """Weights below 2^-40 of their block's constant, of either sign, and a threshold that is exactly zero: which side they
+    fall on decides the levels beside it.  Their magnitude is known to a factor of two, which is 2^-40 absolute."""
+    n = (1 << 21) + tail
+    w = workloads.gaussian(n, 0.02, 21, torch.float32)
+    g = torch.Generator().manual_seed(22)
+    small = torch.rand(n, generator=g) < 0.4
+    sign = torch.where(torch.rand(n, generator=g) < 0.8, -1.0, 1.0)
+    w = (torch.where(small, sign * 1e-15 * (0.5 + torch.rand(n, generator=g)), w) * unit).to(torch.bfloat16)
+    lv = np.linspace(-1, 1, 16).astype(np.float32)
+    cb, log = bof4.bof4_fit_codebook(w.cuda(), 64, 0, metric, lv, 0x8001, 8)
+    ref, ref_log = oracle.fit([w], 64, 0, metric, lv, 0x8001, 8)
+    np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=0 if metric in (1, 3) else 1e-5, atol=2.0 ** -40 if metric in (1, 3) else 1e-7)
+    np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5)
