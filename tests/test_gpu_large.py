@@ -75,3 +75,25 @@ def test_quantise_dequantise_and_fit_beyond_four_giga_elements(bof4):
     same = gm["median"] == ma["median"]
     assert same.sum() >= 14, (gm["median"], ma["median"])     # at most the tail's few samples can shift a crossing
     assert np.all(np.abs(gm["median"] - ma["median"]) < 1e-4)
+
+
+@pytest.mark.parametrize("single", [True, False])
+def test_fit_in_order_beyond_four_giga_elements(bof4, single):
+    """A fit that reduces its data to distinct weights, over 257 copies of 2^24 weights (more than 2^32 in all) as one tensor
+    and as a list: levels, medians and errors are those of one copy."""
+    free, _ = torch.cuda.mem_get_info()
+    if free < 40 * (1 << 30):
+        pytest.skip("needs 40 GB of free device memory")
+    chunk = workloads.gaussian_student_mixture(1 << 24, 0.02, 0.01, 4, 93, torch.bfloat16)
+    w = [chunk.cuda().repeat(257)] if single else [chunk.cuda()] * 257
+    n = sum(t.numel() for t in w)
+    assert n > 1 << 32
+    lv, mask = bof4.bof4_default_init(1)
+    for metric in (bof4.METRIC_MSE, bof4.METRIC_MAE):
+        cb, log = bof4.bof4_fit_codebook(w, I, 1, metric, lv, mask, 6)
+        ref, ref_log = oracle.fit(chunk, I, 1, metric, lv, mask, 6)
+        if metric == bof4.METRIC_MAE:
+            assert np.array_equal(cb.cpu().numpy(), ref)
+        else:
+            np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5, atol=1e-7)
+        np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5)
