@@ -50,11 +50,12 @@ size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W)
 // ---------------------------------------------------------------- samples, one per weight
 
 // Every lane owns 16 consecutive weights; x = RN(w / m) and |m| (1 for the normalised-domain metrics) go
-// to the sample array in the order of the weights.  Bound by its stores (8 bytes per weight).
+// to the sample array in the order of the weights.  Bound by its stores (8 bytes per weight).  Every CTA leaves its sum of
+// squares and its largest constant in slots of its own; the first launch of a fit writes all slots, and the head.
 template <class DT, int I, bool SIGNED>
 __global__ void __launch_bounds__(512, 2)
-sort_samples_kernel(const EmTensors T, const uint32_t first, float2* __restrict__ items, uint32_t* __restrict__ head,
-                    double* __restrict__ w2)
+sort_samples_kernel(const EmTensors T, const uint32_t first, const uint32_t n, float2* __restrict__ items,
+                    uint32_t* __restrict__ head, double* __restrict__ w2, uint32_t* __restrict__ tops)
 {
     if (!after_previous()) return;
     constexpr int NT = 512;
@@ -116,15 +117,21 @@ sort_samples_kernel(const EmTensors T, const uint32_t first, float2* __restrict_
             bits = max(bits, s_max[k]);
         }
         w2[blockIdx.x] = T.accumulate ? w2[blockIdx.x] + a : a;
-        atomicMax(head + 1, bits);  // non-negative floats order like their bits
+        tops[blockIdx.x] = T.accumulate ? max(tops[blockIdx.x], bits) : bits;  // non-negative floats order like their bits
+        if (!T.accumulate && blockIdx.x == 0) {
+            head[0] = n;
+            head[4] = 0u;
+            w2[kSortParts - 1] = 0.0;  // the short last blocks'
+            tops[kSortParts - 1] = 0u;
+        }
     }
 }
 
-// The short last blocks, after all whole blocks in the sample array: one CTA.
+// The short last blocks, after all whole blocks in the sample array: one CTA.  `alone`: there are no whole blocks.
 template <class DT, bool SIGNED>
 __global__ void __launch_bounds__(kEmTailThreads)
-sort_tail_kernel(const EmTails Q, uint32_t at, float2* __restrict__ items, uint32_t* __restrict__ head,
-                 double* __restrict__ w2)
+sort_tail_kernel(const EmTails Q, uint32_t at, const uint32_t n, const bool alone, float2* __restrict__ items,
+                 uint32_t* __restrict__ head, double* __restrict__ w2, uint32_t* __restrict__ tops)
 {
     if (!after_previous()) return;
     __shared__ float s_w[4096];
@@ -132,9 +139,11 @@ sort_tail_kernel(const EmTails Q, uint32_t at, float2* __restrict__ items, uint3
     __shared__ double s_sum[kEmTailThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double sum = 0.0;
+    uint32_t top = 0u;
     for (int q = 0; q < Q.count; ++q) {
         const int len = Q.len[q];
         const float m = load_short_block<DT, SIGNED>(Q.ptr[q], len, s_w, s_red);
+        top = max(top, __float_as_uint(fabsf(m)));
         for (int i = tid; i < len; i += kEmTailThreads) {
             const float x = normalise(s_w[i], m), am = Q.unit ? 1.0f : fabsf(m);
             const double e = (double)x * (double)am;
@@ -142,7 +151,6 @@ sort_tail_kernel(const EmTails Q, uint32_t at, float2* __restrict__ items, uint3
             items[at + i] = make_float2(x, am);
         }
         at += (uint32_t)len;
-        if (tid == 0) atomicMax(head + 1, __float_as_uint(fabsf(m)));
         __syncthreads();  // before the next block overwrites s_w
     }
 #pragma unroll
@@ -153,18 +161,18 @@ sort_tail_kernel(const EmTails Q, uint32_t at, float2* __restrict__ items, uint3
         double a = 0.0;
         for (int k = 0; k < kEmTailThreads / 32; ++k) a += s_sum[k];
         w2[kSortParts - 1] = Q.accumulate ? w2[kSortParts - 1] + a : a;
+        tops[kSortParts - 1] = Q.accumulate ? max(tops[kSortParts - 1], top) : top;
+        if (alone && !Q.accumulate) {
+            head[0] = n;
+            head[4] = 0u;
+        }
     }
-}
-
-__global__ void sort_head_kernel(uint32_t* head, uint32_t n, double* w2)
-{
-    if (!after_previous()) return;
-    if (threadIdx.x == 0) {
-        head[0] = n;
-        head[1] = 0u;
-        head[4] = 0u;
+    if (alone && !Q.accumulate) {
+        for (int k = tid; k < kSortParts - 1; k += kEmTailThreads) {
+            w2[k] = 0.0;
+            tops[k] = 0u;
+        }
     }
-    for (int k = threadIdx.x; k < kSortParts; k += blockDim.x) w2[k] = 0.0;
 }
 
 // ---------------------------------------------------------------- ordering passes
@@ -327,11 +335,19 @@ struct SampleWeight {
 
 // First sample of every bin: sample i is the first of all bins behind the one of sample i - 1 up to its own; behind
 // the last sample come all bins that are left, which are all there are where no sample has a weight (bf16 zeros).
+// tops, or NULL: the largest constants of the samples' CTAs, of which one is made.
 __global__ void __launch_bounds__(256)
-sort_start_kernel(const float2* __restrict__ items, const uint32_t* __restrict__ head, uint32_t* __restrict__ start)
+sort_start_kernel(const float2* __restrict__ items, uint32_t* __restrict__ head, const uint32_t* __restrict__ tops,
+                  uint32_t* __restrict__ start)
 {
     if (!after_previous()) return;
     const uint32_t n = *head;
+    if (tops && blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) {
+        uint32_t top = 0u;
+        for (int k = threadIdx.x; k < kSortParts; k += 32) top = max(top, tops[k]);
+        top = __reduce_max_sync(kFull, top);
+        if (threadIdx.x == 0) head[1] = top;
+    }
     int far0 = 0, far1 = -1;  // a gap of many empty bins, if the thread meets one: filled by the warp below
     uint32_t far_i = 0u;
     for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i <= n; i += gridDim.x * 256) {
@@ -1292,10 +1308,10 @@ int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
 }
 
 template <class DT, bool SG>
-int samples(const EmTensors& T, int block_size, uint32_t first, const SortWs& W, cudaStream_t st)
+int samples(const EmTensors& T, int block_size, uint32_t first, uint32_t n, const SortWs& W, cudaStream_t st)
 {
 #define BOF4_SORT_I(I_) \
-    case I_: launch_after(sort_samples_kernel<DT, I_, SG>, 2 * kSMs, 512, 0, st, T, first, W.a, W.n_items, W.w2); break;
+    case I_: launch_after(sort_samples_kernel<DT, I_, SG>, 2 * kSMs, 512, 0, st, T, first, n, W.a, W.n_items, W.w2, W.first); break;
     switch (block_size) {
         BOF4_SORT_I(32) BOF4_SORT_I(64) BOF4_SORT_I(128) BOF4_SORT_I(256) BOF4_SORT_I(512) BOF4_SORT_I(1024)
         BOF4_SORT_I(2048) BOF4_SORT_I(4096)
@@ -1318,7 +1334,7 @@ int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
     V.b = W.a;
     V.before = reinterpret_cast<SortSums*>(W.b);
     const int64_t ctas = F.n_max / 256 + 1;  // one thread beyond the samples
-    launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, V.b, V.n_items, V.start);
+    launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, V.b, V.n_items, F.acc ? nullptr : V.first, V.start);
     BOF4_CUDA_TRY(cudaGetLastError());
     const bool mae = F.metric == BOF4_METRIC_MAE || F.metric == BOF4_METRIC_MAE_NORMALIZED;
     if (F.acc) return mae ? sums_and_iterations<true, true>(V, F, st) : sums_and_iterations<false, true>(V, F, st);
@@ -1333,7 +1349,8 @@ int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iter
     SortWs W;
     if (sorted_layout(d_ws, a.n_total, false, &W) > ws_bytes) return BOF4_OK;
     *done = true;
-    launch_after(sort_head_kernel, 1, 320, 0, st, W.n_items, (uint32_t)a.n_total, W.w2);
+    const uint32_t n = (uint32_t)a.n_total;
+    const bool alone = !has_whole_blocks(a);
     const bool sg = a.norm == BOF4_NORM_SIGNED;
     uint32_t at = 0;
     int calls = 0;
@@ -1341,17 +1358,17 @@ int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iter
         const uint32_t first = at;
         for (int t = 0; t < T.count; ++t) at += (uint32_t)T.n[t];
         if (a.w_dtype == BOF4_F32)
-            return sg ? samples<F32, true>(T, a.block_size, first, W, st) : samples<F32, false>(T, a.block_size, first, W, st);
-        return sg ? samples<BF16, true>(T, a.block_size, first, W, st) : samples<BF16, false>(T, a.block_size, first, W, st);
+            return sg ? samples<F32, true>(T, a.block_size, first, n, W, st) : samples<F32, false>(T, a.block_size, first, n, W, st);
+        return sg ? samples<BF16, true>(T, a.block_size, first, n, W, st) : samples<BF16, false>(T, a.block_size, first, n, W, st);
     }, &calls);
     if (rc) return rc;
     rc = for_each_tail_chunk(a, [&](const EmTails& Q) -> int {
         if (a.w_dtype == BOF4_F32) {
-            if (sg) launch_after(sort_tail_kernel<F32, true>, 1, kEmTailThreads, 0, st, Q, at, W.a, W.n_items, W.w2);
-            else launch_after(sort_tail_kernel<F32, false>, 1, kEmTailThreads, 0, st, Q, at, W.a, W.n_items, W.w2);
+            if (sg) launch_after(sort_tail_kernel<F32, true>, 1, kEmTailThreads, 0, st, Q, at, n, alone, W.a, W.n_items, W.w2, W.first);
+            else launch_after(sort_tail_kernel<F32, false>, 1, kEmTailThreads, 0, st, Q, at, n, alone, W.a, W.n_items, W.w2, W.first);
         } else {
-            if (sg) launch_after(sort_tail_kernel<BF16, true>, 1, kEmTailThreads, 0, st, Q, at, W.a, W.n_items, W.w2);
-            else launch_after(sort_tail_kernel<BF16, false>, 1, kEmTailThreads, 0, st, Q, at, W.a, W.n_items, W.w2);
+            if (sg) launch_after(sort_tail_kernel<BF16, true>, 1, kEmTailThreads, 0, st, Q, at, n, alone, W.a, W.n_items, W.w2, W.first);
+            else launch_after(sort_tail_kernel<BF16, false>, 1, kEmTailThreads, 0, st, Q, at, n, alone, W.a, W.n_items, W.w2, W.first);
         }
         for (int q = 0; q < Q.count; ++q) at += (uint32_t)Q.len[q];
         BOF4_CUDA_TRY(cudaGetLastError());

@@ -42,7 +42,7 @@ struct SortWs {
     double* w2;           // [kSortParts]
     uint32_t* counts;     // [kSortGrid][256]
     uint32_t* start;      // [kSortBins + 1] first sample of every bin
-    uint32_t* first;      // [kSortGroups + 1] first sample of every group
+    uint32_t* first;      // [kSortGroups + 1] first sample of every group; before, the largest constants of the samples' CTAs
     uint16_t* off;        // [kSortBins] first sample of a bin in its group, kFarBin: too far, see start
     SortSums *bin, *group;
     SortSums *pre, *suf;  // per bin: the bins of its group in front of it; it and those behind it

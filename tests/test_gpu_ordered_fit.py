@@ -216,3 +216,24 @@ def test_normalised_weights_near_zero_keep_their_sign(bof4, tail, unit, metric):
     ref, ref_log = oracle.fit([w], 64, 0, metric, lv, 0x8001, 8)
     np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=0 if metric in (1, 3) else 1e-5, atol=2.0 ** -40 if metric in (1, 3) else 1e-7)
     np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5)
+
+
+@pytest.mark.parametrize("size", [3000, 20])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("metric", [0, 1])
+def test_many_small_tensors(bof4, size, dtype, metric):
+    """One sample per weight of more tensors than one launch takes; of 20 weights and a few there are short blocks only.  The
+    workspace holds what another fit has left."""
+    ws = [_weights(size + 13 * k % 11, dtype, k, "plain") for k in range(140)]
+    n = sum(w.numel() for w in ws)
+    lv, mask = bof4.bof4_default_init(0)
+    room = torch.empty(bof4.bof4_fit_workspace_bytes(1 << 20, bof4.F32, 64, metric, 100), dtype=torch.uint8, device="cuda")
+    bof4.bof4_fit_codebook(_weights(1 << 20, torch.float32, 1, "grid").cuda() * 1e9, 64, 0, metric, lv, mask, 9, workspace=room)
+    cb, log = bof4.bof4_fit_codebook([w.cuda() for w in ws], 64, 0, metric, lv, mask, 9, workspace=room)
+    ref, ref_log = oracle.fit(ws, 64, 0, metric, lv, mask, 9)
+    assert n < 1 << 20
+    if metric == bof4.METRIC_MAE:
+        assert np.array_equal(cb.cpu().numpy(), ref)
+    else:
+        np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5, atol=1e-7)
+    np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5, atol=1e-12)
