@@ -12,8 +12,9 @@
 //   accumulate  a unit is some blocks of ONE magnitude |m|: with m fixed, the cell of a weight is the
 //               difference of the two bit patterns, so the counts of a unit are 10240 words of shared
 //               memory and a weight costs a subtraction, a comparison and one shared-memory reduction
-//               (about 3.5 wavefronts per 32 weights on random banks, which bounds the pass); when the
-//               unit is done its counts times the weight of |m| are added to the cells
+//               on random banks (2^28 weights, 168 us: 83 % of the LSU data path, 4.6 wavefronts per 32 weights,
+//               and 82 % of the issue slots, 16.6 instructions a weight); when the unit is done its counts times
+//               the weight of |m| are added to the cells
 //   items       the occupied cells in a fixed order, as samples for the ordering passes
 //
 // A cell is (significand of m, sign, distance of the bit patterns).  Cell sums are integers (128 bits, a

@@ -22,8 +22,11 @@
 //                 K = 16), tcgen05.commit hands the stage back
 //   4 results     read the accumulators of a part of a tile (there are two sets) while the next part runs
 //
-// What bounds it: shared memory, 8192 weights of a k-block at 32 weights per 128-byte wavefront and clock (256
-// cycles; 300 with codes, constants and X), against 80 for what HBM delivers.  A decoded tile in shared memory
+// What bounds it: the data path of shared memory.  The accesses of a k-block need 300 wavefronts (its 8192 weights at 32 per
+// 128-byte wavefront, 256; codes, constants and X the rest); its codes take HBM 182 cycles (4096 bytes at 22.5 bytes a clock and
+// SM).  Counted are 473 wavefronts and 551 cycles a k-block while an SM is active (28672 x 8192 x 32, 194 k-blocks per SM; with
+// an outlier list 490 and 746, 65 % of the issue slots); what the other 170 wavefronts are is not known.  The rest of a
+// launch, about 9 us at any size, is set-up, first loads, cut tiles and drain.  A decoded tile in shared memory
 // would add as much again for its write and the tensor cores' read; decoding in registers by byte permutes
 // takes 460 cycles of the half-rate integer pipe.  Warps with global loads of their own in flight paid their
 // latency at every publication of a k-block, hence the TMA ring; one issuing warp takes 500 cycles per k-block
@@ -34,7 +37,7 @@
 // entries of a batch of lines into short lists per line, warp and half k-block beforehand (two searches and one
 // pass over the tile's entries, beside the main loop).
 //
-// Measured: 28672 x 8192 x 32 68 us (87 with a list of 0.1 %), 4096 x 4096 x 32 13 us (17); the form with one CTA
+// Measured: 28672 x 8192 x 32 69 us (90 with a list of 0.06 %), 4096 x 4096 x 32 13 us (17); the form with one CTA
 // per tile and K split that stored its tile in shared memory took 170 (210) and 13 (17) us.
 //
 // Every wait is bounded: a time-out sets the status word, everybody leaves, and the kernel frees its tensor

@@ -55,7 +55,9 @@ inline uint32_t mae_cand_capacity(size_t ws_bytes)
 
 // ---------------------------------------------------------------- OPQ workspace
 // The weights are cut into tiles of kOpqTile elements (one warp iteration).  Each tile has a
-// count and a staging slot of kOpqStage outliers; tiles are scanned in chunks of kOpqChunk.
+// count and a staging slot of kOpqStage outliers; tiles are scanned in chunks of kOpqChunk, a CTA of
+// the gathering kernel each.  512 against 2048 tiles: 2^20 weights 16.3 against 18.6 us, 2^24 29 against 32, 2^27 the same (191);
+// where every tile has more outliers than slots and is looked through again, 143 against 484, 193 against 533 and 675 against 983.
 constexpr int kOpqTile = 512;
 constexpr int kOpqStage = 16;
 constexpr int kOpqChunk = 512;
