@@ -108,19 +108,19 @@ int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iter
 int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters, double* d_err_log, void* d_ws,
               size_t ws_bytes, cudaStream_t st, bool* done);
 
-// Bin of a normalised weight, monotone in x: 32768 +- the bin of |x|, which is 0 for x = 0 alone, 128 bins per binade
-// below 2^-7 (1 ... 4318, all of |x| < 2^-40 in the first few), bins of width 1 / 28671 from there on (the width that the
-// binade below has as well), and 32767 for |x| = 1 alone.  Zeros (sparse data) and ones (a weight per block) are the only
+// Bin of a normalised weight, monotone in x: 32768 +- the bin of |x|, which is 0 for x = 0 alone, eight bins per binade
+// below 2^-11 (1 ... 215, all of |x| < 2^-38 in the first), bins of width 1 / 32566 from there on (at least the width of the
+// ones below), and 32767 for |x| = 1 alone.  Zeros (sparse data) and ones (a weight per block) are the only
 // values that data is likely to hold in any number, and no threshold ever has to look into a bin of one value.
 constexpr int kBinMinus = 1, kBinZero = 32768, kBinPlus = 65535;
 __device__ __forceinline__ int sort_bin(float x)
 {
     const float a = fminf(fabsf(x), 1.0f);
     int m;
-    if (a >= 0.0078125f) {
-        m = 4096 + (int)(a * 28671.0f);
+    if (a >= 0x1p-11f) {
+        m = 201 + (int)(a * 32566.0f);
     } else {
-        m = 4319 - (15360 - (int)(__float_as_uint(a) >> 16));
+        m = 215 - (927 - (int)(__float_as_uint(a) >> 20));
         m = (a == 0.0f) ? 0 : max(m, 1);
     }
     return x < 0.0f ? kBinZero - m : kBinZero + m;
