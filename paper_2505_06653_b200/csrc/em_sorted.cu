@@ -335,22 +335,25 @@ struct SampleWeight {
 
 // First sample of every bin: sample i is the first of all bins behind the one of sample i - 1 up to its own; behind
 // the last sample come all bins that are left, which are all there are where no sample has a weight (bf16 zeros).
-// tops, or NULL: the largest constants of the samples' CTAs, of which one is made.
+// tops, or NULL: the largest constants of the samples' CTAs, of which the last CTA makes one.
 __global__ void __launch_bounds__(256)
 sort_start_kernel(const float2* __restrict__ items, uint32_t* __restrict__ head, const uint32_t* __restrict__ tops,
                   uint32_t* __restrict__ start)
 {
     if (!after_previous()) return;
     const uint32_t n = *head;
-    if (tops && blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) {
+    if (blockIdx.x == gridDim.x - 1) {
+        if (!tops || threadIdx.x >= 32) return;
         uint32_t top = 0u;
-        for (int k = threadIdx.x; k < kSortParts; k += 32) top = max(top, tops[k]);
+#pragma unroll
+        for (int k = 0; k < kSortParts; k += 32) top = max(top, k + threadIdx.x < kSortParts ? tops[k + threadIdx.x] : 0u);
         top = __reduce_max_sync(kFull, top);
         if (threadIdx.x == 0) head[1] = top;
+        return;
     }
     int far0 = 0, far1 = -1;  // a gap of many empty bins, if the thread meets one: filled by the warp below
     uint32_t far_i = 0u;
-    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i <= n; i += gridDim.x * 256) {
+    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i <= n; i += (gridDim.x - 1) * 256) {
         const int b = i < n ? sort_bin(items[i].x) : kSortBins, prev = i ? sort_bin(items[i - 1].x) : -1;
         if (b - prev > 64 && far1 < 0) {
             far0 = prev + 1, far1 = b;
@@ -393,8 +396,8 @@ __device__ __forceinline__ void sums_add(SortSums& t, const SortSums& v)
 // beside them; what a threshold takes of the bin, and where its weight reaches a half, is then found by bisection in every
 // window, a lane each: 1.1 and 1.3 ms, of which 0.8 are the ordering that other data takes as well.  An iteration now costs
 // at most a few bisections (14 steps of an access to L2 each) per 2^20 samples of a crowded bin, and median step.
-// Other data pays for a launch that finds nothing to do and for the test of the flag: 165.8 -> 169.3 us for 50 iterations over
-// 2^20 weights.
+// Other data pays for a launch that finds nothing to do (two for medians) and for the test of the flag: 50 iterations over 2^20
+// weights 166.7 -> 167.7 us, 12 of medians 146 -> 150.
 
 // One CTA per window of kSortWindow samples: four stable passes of eight bits by the key of x in shared memory, then the
 // running sums (exclusive within the window, every fourth sample).
@@ -668,14 +671,27 @@ sort_group_kernel(const SortWs W)
 #pragma unroll 4
         for (uint32_t c = c0 + 1; c <= c1; ++c) sums_add(t, W.lead[c]);
     }
+    const bool many = e > s && c1 - c0 > kSortMany;
+    unsigned spans = __ballot_sync(kFull, e > s && c0 != c1 && !few && !many);
+    while (spans) {
+        const int who = __ffs(spans) - 1;
+        spans &= spans - 1u;
+        const uint32_t f = __shfl_sync(kFull, c0, who), l = __shfl_sync(kFull, c1, who);
+        SortSums u{0.0, 0.0, 0ull};
+#pragma unroll 4
+        for (uint32_t c = f + lane; c <= l; c += 32) sums_add(u, (c == f) ? W.trail[c] : W.lead[c]);
+        __syncwarp();
+        sums_reduce<MAE>(u);
+        if (lane == who) t = u;
+    }
     __shared__ uint32_t s_first[256], s_last[256], s_many[8];
     __shared__ SortSums s_part[8];
-    const bool many = e > s && c1 - c0 > kSortMany;
-    const unsigned wide = __ballot_sync(kFull, many);
-    s_first[threadIdx.x] = c0;
-    s_last[threadIdx.x] = c1;
-    if (lane == 0) s_many[threadIdx.x >> 5] = wide;
     if (__syncthreads_or(many)) {
+        const unsigned wide = __ballot_sync(kFull, many);
+        s_first[threadIdx.x] = c0;
+        s_last[threadIdx.x] = c1;
+        if (lane == 0) s_many[threadIdx.x >> 5] = wide;
+        __syncthreads();
         for (int w = 0; w < 8; ++w) {
             for (unsigned left = s_many[w]; left; left &= left - 1u) {
                 const int who = w * 32 + __ffs(left) - 1;
@@ -692,18 +708,6 @@ sort_group_kernel(const SortWs W)
                 __syncthreads();
             }
         }
-    }
-    unsigned spans = __ballot_sync(kFull, e > s && c0 != c1 && !few && !many);
-    while (spans) {
-        const int who = __ffs(spans) - 1;
-        spans &= spans - 1u;
-        const uint32_t f = __shfl_sync(kFull, c0, who), l = __shfl_sync(kFull, c1, who);
-        SortSums u{0.0, 0.0, 0ull};
-#pragma unroll 4
-        for (uint32_t c = f + lane; c <= l; c += 32) sums_add(u, (c == f) ? W.trail[c] : W.lead[c]);
-        __syncwarp();
-        sums_reduce<MAE>(u);
-        if (lane == who) t = u;
     }
     W.bin[b] = t;
     SortSums up = t, down = t;  // this bin and those in front of it; and those behind it
@@ -750,7 +754,7 @@ constexpr int kMseFirst = kMseOff + kSortBins * 2;   // of the groups
 constexpr int kMseSmem = kMseFirst + (kSortGroups + 1) * 4;
 
 // CROWDED: a copy of the loop that also knows crowded bins.  Apart, because the calls in it cost the other one registers: 0.3 us
-// an iteration with both in one.
+// an iteration with both in one.  (Two kernels, as for the absolute error, of which the flag picks one: 2 us slower.)
 template <bool CELLS, bool CROWDED>
 __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
 {
@@ -1010,9 +1014,15 @@ __device__ __noinline__ bool crowded_median(const SortWs& W, const SampleWeight<
     return true;
 }
 
+// CROWDED: the kernel for data with crowded bins.  Both are launched, the flag of such bins tells which one runs: with both
+// loops in one kernel 2^22 fp32 weights, 12 iterations, took 299 us against 293.5, 2^20 153.8 against 152.4.
 template <bool CELLS, bool CROWDED>
-__device__ __forceinline__ void fit_mae(const SortWs& W, const SortFit& F)
+__global__ void __launch_bounds__(1024, 1)
+sort_fit_mae_kernel(const SortWs W, const SortFit F)
 {
+    if (!after_previous()) return;
+    if (CROWDED && W.n_items[4] == 0u) return;
+    const uint32_t other = CELLS || CROWDED ? 0u : W.n_items[4];
     extern __shared__ __align__(16) unsigned char s_fit[];
     SortSums* const s_group = reinterpret_cast<SortSums*>(s_fit);
     __shared__ float s_level[2][kLevels], s_med[kLevels];
@@ -1025,6 +1035,7 @@ __device__ __forceinline__ void fit_mae(const SortWs& W, const SortFit& F)
     for (int k = tid; k < kSortGroups; k += 1024) s_group[k] = W.group[k];
     if (tid < kLevels) s_level[0][tid] = F.codebook[tid];
     if (tid == 0) s_stop = 0;
+    if (other) return;
     __syncthreads();
     const int l = warp >> 1, h = warp & 1;
     const float inf = __int_as_float(0x7f800000);
@@ -1262,15 +1273,6 @@ __device__ __forceinline__ void fit_mae(const SortWs& W, const SortFit& F)
     if (tid < kLevels && !((F.fixed_mask >> tid) & 1u)) F.codebook[tid] = s_level[now][tid];
 }
 
-template <bool CELLS>
-__global__ void __launch_bounds__(1024, 1)
-sort_fit_mae_kernel(const SortWs W, const SortFit F)
-{
-    if (!after_previous()) return;
-    if (!CELLS && W.n_items[4] != 0u) fit_mae<CELLS, !CELLS>(W, F);
-    else fit_mae<CELLS, false>(W, F);
-}
-
 // ---------------------------------------------------------------- host side
 
 namespace {
@@ -1285,21 +1287,32 @@ int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
     const int64_t ctas = (F.n_max + 8 * kSortChunk - 1) / (8 * kSortChunk);
     launch_after(sort_sums_kernel<MAE, CELLS>, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, W, weight);
     launch_after(sort_group_kernel<MAE>, kSortGroups / 8, 256, 0, st, W);
-    if constexpr (!CELLS) {  // cells never crowd a bin, and no more samples than make one cannot either
-        if (F.n_max > kSortCrowd) {
+    // cells never crowd a bin, and no more samples than make one cannot either
+    auto order_windows = [&]() -> int {
+        if constexpr (!CELLS) {
             constexpr auto kern = sort_windows_kernel<MAE>;
             constexpr int smem = (int)sizeof(WindowScratch);
             if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
             const int64_t windows = (F.n_max + kSortWindow - 1) / kSortWindow;
             launch_after(kern, (int)(windows < kSMs ? windows : kSMs), kSortThreads, smem, st, W, weight);
         }
-    }
+        return BOF4_OK;
+    };
+    const bool may_crowd = !CELLS && F.n_max > kSortCrowd;
     if constexpr (MAE) {
         constexpr int smem = kSortGroups * (int)sizeof(SortSums);
-        constexpr auto kern = sort_fit_mae_kernel<CELLS>;
-        if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
-        launch_after(kern, 1, 1024, smem, st, W, F);
+        constexpr auto plain = sort_fit_mae_kernel<CELLS, false>;
+        if (const int rc = ensure_dynamic_smem<plain>(smem)) return rc;
+        launch_after(plain, 1, 1024, smem, st, W, F);
+        if (may_crowd) {
+            if (const int rc = order_windows()) return rc;
+            constexpr auto crowded = sort_fit_mae_kernel<CELLS, !CELLS>;
+            if (const int rc = ensure_dynamic_smem<crowded>(smem)) return rc;
+            launch_after(crowded, 1, 1024, smem, st, W, F);
+        }
     } else {
+        if (may_crowd)
+            if (const int rc = order_windows()) return rc;
         constexpr auto kern = sort_fit_mse_kernel<CELLS>;
         if (const int rc = ensure_dynamic_smem<kern>(kMseSmem)) return rc;
         launch_after(kern, 1, 1024, kMseSmem, st, W, F);
@@ -1335,7 +1348,7 @@ int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
     V.b = W.a;
     V.before = reinterpret_cast<SortSums*>(W.b);
     const int64_t ctas = F.n_max / 256 + 1;  // one thread beyond the samples
-    launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, V.b, V.n_items, F.acc ? nullptr : V.first, V.start);
+    launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs) + 1, 256, 0, st, V.b, V.n_items, F.acc ? nullptr : V.first, V.start);
     BOF4_CUDA_TRY(cudaGetLastError());
     const bool mae = F.metric == BOF4_METRIC_MAE || F.metric == BOF4_METRIC_MAE_NORMALIZED;
     if (F.acc) return mae ? sums_and_iterations<true, true>(V, F, st) : sums_and_iterations<false, true>(V, F, st);
