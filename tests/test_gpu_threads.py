@@ -37,6 +37,16 @@ def test_a_full_queue_stops_no_other_thread(make):
     call = make(bof4, w, cb)
     call()
     torch.cuda.synchronize()
+    for attempt in range(3):  # a busy machine may stop a thread for a while by itself; the lock does every time
+        waited, gap = _longest_gap(call)
+        assert waited > 0.4, "the queue did not fill"
+        if gap < 0.2:
+            return
+    raise AssertionError("another thread stood still for %.3f s of %.3f s" % (gap, waited))
+
+
+def _longest_gap(call):
+    """Seconds that 3000 calls behind a kernel of 0.6 s and more take, and the longest that another thread stood still."""
     seen, stop = [], threading.Event()
 
     def watch():
@@ -47,7 +57,7 @@ def test_a_full_queue_stops_no_other_thread(make):
     t = threading.Thread(target=watch)
     t.start()
     time.sleep(0.05)
-    torch.cuda._sleep(int(1.2e9))            # 0.6 s and more of an idle kernel; the calls below pile up behind it
+    torch.cuda._sleep(int(1.2e9))
     start = time.perf_counter()
     for _ in range(3000):
         call()
@@ -55,6 +65,4 @@ def test_a_full_queue_stops_no_other_thread(make):
     stop.set()
     t.join()
     torch.cuda.synchronize()
-    assert waited > 0.4, "the queue did not fill"
-    gap = max(b - a for a, b in zip(seen, seen[1:]))
-    assert gap < 0.2, "another thread stood still for %.3f s of %.3f s" % (gap, waited)
+    return waited, max(b - a for a, b in zip(seen, seen[1:]))
