@@ -56,14 +56,14 @@ struct SortWs {
 // Whether a fit of `iters` iterations over n weights is faster with its samples in order than streamed: the ordering is
 // paid once, an iteration is cheaper by what it streams.  Both sides by measurement, in us with k = n / 2^20 (blocks of 64;
 // other block sizes differ by a few per cent):
-//   ordering  one sample per weight 85 (k = 1), 195 (4), 390 (8), 770 (16), 1560 (32), 4040 (64: beyond the L2's reach);
+//   ordering  one sample per weight 81 (k = 1), 185 (4), 370 (8), 755 (16), 1580 (32), 4230 (64: beyond the L2's reach);
 //             distinct bf16 weights 102 (2), 107 (4), 135 (16), 190 (64), 400 (256), 1140 (1024)
 //   streamed iteration less an ordered one
-//             fp32: MSE 15 (1), 17 (4), 24 (8), 31 (16), 57 (32), 97 (64), medians 45, 52, 65, 75, 107, 132
+//             fp32: MSE 15 (1), 19 (4), 26 (8), 34 (16), 64 (32), 112 (64), medians 46, 52, 63, 73, 108, 148
 //             bf16: MSE 17 (1), 18 (4), 34 (16), 73 (64), 970 (1024), medians 50, 52, 76, 173, 2000
-// The lines below are fits to these.  Where they cross, in iterations: fp32 MSE 6 at 2^20, 11 at 2^22, 24 at 2^24, 45 at 2^26,
-// medians 4, 4, 11, 31; bf16 MSE 6 from 3 * 2^19 to 2^22, 4 from 2^24 on, medians 4.  With four iterations for all,
-// fits of 4 and 8 over 2^24 fp32 weights took 787 and 796 us (MSE) against 150 and 284 streamed.
+// The lines below are fits to these.  Where they cross, in iterations: fp32 MSE 6 at 2^20, 11 at 2^22, 22 at 2^24, 37 at 2^26,
+// medians 4, 4, 11, 29; bf16 MSE 6 from 3 * 2^19 to 2^22, 4 from 2^24 on, medians 4.  With four iterations for all,
+// fits of 4 and 8 over 2^24 fp32 weights took 787 and 796 us (MSE) against 160 and 307 streamed.
 // Fewer than four iterations are not ordered, although two or three would pay for bf16 data from 2^26 weights on (2^28, three: 1120
 // us streamed, about 400 ordered): such a fit gets by with the small workspace.
 inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool cells)
@@ -73,8 +73,8 @@ inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool ce
     const bool mae = metric == BOF4_METRIC_MAE || metric == BOF4_METRIC_MAE_NORMALIZED;
     double order = 105.0 + 1.1 * k, gain = mae ? 50.0 + 1.9 * k : 16.5 + 0.9 * k;
     if (!cells) {
-        order = fmax(fmax(46.0 + 35.0 * k, 48.0 * k), 78.0 * k - 1000.0);
-        gain = mae ? fmin(43.0 + 1.85 * k, 85.0 + 0.75 * k) : (w_dtype == BOF4_BF16 ? 18.0 : 13.0) + 1.2 * k;
+        order = fmax(fmax(46.0 + 35.0 * k, 48.0 * k), 82.0 * k - 1000.0);
+        gain = mae ? fmin(43.0 + 1.85 * k, 85.0 + k) : (w_dtype == BOF4_BF16 ? 18.0 : 13.0) + 1.3 * k + 0.005 * k * k;
     }
     return iters * gain >= order;
 }
