@@ -34,6 +34,9 @@
 
 namespace bof4 {
 
+constexpr int kQLutRep = 16;         // columns of the quantisers' region table, half the stores of one per lane: 2^24 weights
+                                     // 12.7 us against 13.4, the OPQ pass over 28672 x 8192 177 against 181
+constexpr int kQLutBytes = lut_bytes(kQLutRep);
 constexpr int kLW = 32;              // bf16 weights per lane and row
 constexpr int kWarpW32 = 32 * kLW;   // weights per warp iteration
 
@@ -187,18 +190,17 @@ struct FastInfo {
     int tiny;  // some threshold has magnitude below 2^-90 (zero included): FAST is off
 };
 
-// One bin of the near-significand test: threshold index j, significand b.
-__device__ __forceinline__ void mark_if_near(const float* s_xi, int j, int b, FastInfo* s_info)
+// The near-significand test of one threshold and one significand b.
+__device__ __forceinline__ bool is_near(float xi, uint32_t b)
 {
-    const uint32_t bits = __float_as_uint(s_xi[j]), xb = bits & 0x7fffffffu;
-    if (xb >= 0x7f800000u || xb < 0x12800000u) return;  // not finite, or below 2^-90 (see tiny)
+    const uint32_t bits = __float_as_uint(xi), xb = bits & 0x7fffffffu;
     const uint32_t X = (xb & 0x7fffffu) | 0x800000u;       // 24-bit significand
-    const uint32_t P = X * (uint32_t)b;                    // < 2^32, >= 2^30
+    const uint32_t P = X * b;                              // < 2^32, >= 2^30
     const int s = (P >> 31) ? 24 : 23;                     // P >> s in [128, 256)
     const uint32_t frac = P & ((1u << s) - 1u);
     const uint32_t dist = (bits >> 31) ? ((1u << s) - frac) & ((1u << s) - 1u) : frac;  // distance into the window side
-    const bool near = 4u * dist >= (uint32_t)b && dist <= (P >> 20);
-    if (near) atomicOr(&s_info->near_mask[(b - 128) >> 5], 1u << ((b - 128) & 31));
+    // not finite, or below 2^-90 (see tiny): no
+    return 4u * dist >= b && dist <= (P >> 20) && xb < 0x7f800000u && xb >= 0x12800000u;
 }
 
 // The third fp32 number below x (finite, |x| >= 2^-90: no zero crossing).
@@ -208,67 +210,32 @@ __device__ __forceinline__ float three_steps_down(float x)
     return __uint_as_float((u >> 31) ? u + 3u : u - 3u);
 }
 
-// Everything a quantising kernel derives from the codebook, in two barriers: the true thresholds
+// Everything a quantising kernel derives from the codebook, in one barrier: the true thresholds
 // and the levels (s_xi, s_lv), the one-probe region table of the FAST path over the LOWERED
 // thresholds (s_lut, [bin][lane] replicated REP times; payload(base) beside every threshold) and
-// the FAST-path information.  Every thread derives
-// the thresholds and their table bins itself from the 16 levels, so that the table entries, the
-// "two thresholds in one bin" test and the "tiny threshold" test need no exchange.  Returns
-// whether the table can serve the codebook.  Call with all threads of the CTA (>= 257).
-template <int REP = 32, class PayloadFn>
-__device__ __forceinline__ bool build_tables32(const float* __restrict__ levels, float* s_xi, float* s_lv,
+// the FAST-path information.  level = lane_level(levels).  Returns whether the table can serve the
+// codebook.  Call with all threads of the CTA (four warps or more).
+template <int REP, class PayloadFn>
+__device__ __forceinline__ bool build_tables32(float level, float* s_xi, float* s_lv,
                                                unsigned char* s_lut, FastInfo* s_info, PayloadFn payload)
 {
-    __shared__ uint2 s_ent[kLutBins];
-    const int tid = threadIdx.x;
-    float lv[kLevels], xi[kLevels];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(levels) + q);
-        lv[4 * q] = t.x;
-        lv[4 * q + 1] = t.y;
-        lv[4 * q + 2] = t.z;
-        lv[4 * q + 3] = t.w;
-    }
-    float lo[kLevels];  // lowered thresholds (table side)
-    int bin[kLevels - 1];
-    bool multi = false, tiny = false;
-#pragma unroll
-    for (int j = 0; j < kLevels - 1; ++j) {
-        xi[j] = __fmul_rn(__fadd_rn(lv[j], lv[j + 1]), 0.5f);
-        const bool usable = fabsf(xi[j]) >= 0x1p-90f && fabsf(xi[j]) < __int_as_float(0x7f800000);
-        tiny = tiny || !(fabsf(xi[j]) >= 0x1p-90f);
-        lo[j] = usable ? three_steps_down(xi[j]) : xi[j];
-        const int bj = (int)(__float_as_uint(lut_key(lo[j])) - kLutMagicBits);
-        bin[j] = bj < 0 ? 0 : (bj > kLutBins - 1 ? kLutBins - 1 : bj);
-        if (j > 0) multi = multi || bin[j] == bin[j - 1];   // ascending thresholds: equal bins are adjacent
-    }
-    xi[kLevels - 1] = lo[kLevels - 1] = __int_as_float(0x7f800000);
-    if (tid < kLutBins) {
-        int base = 0;
-#pragma unroll
-        for (int j = 0; j < kLevels - 1; ++j) base += (bin[j] < tid) ? 1 : 0;
-        float thr = lo[kLevels - 1];
-#pragma unroll
-        for (int j = kLevels - 2; j >= 0; --j) thr = (base == j) ? lo[j] : thr;
-        s_ent[tid] = make_uint2(__float_as_uint(thr), payload(base));
-    }
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float xi = lane_threshold(level), mag = fabsf(xi);
+    const bool usable = mag >= 0x1p-90f && mag < __int_as_float(0x7f800000);
+    const bool tiny = __any_sync(kFull, !(mag >= 0x1p-90f));
+    const bool multi = fill_lut<REP>(usable ? three_steps_down(xi) : xi, s_lut, payload);
     if (tid < kLevels) {
-        float a = xi[kLevels - 1], l = lv[kLevels - 1];
-#pragma unroll
-        for (int j = kLevels - 2; j >= 0; --j) {
-            a = (tid == j) ? xi[j] : a;
-            l = (tid == j) ? lv[j] : l;
-        }
-        s_xi[tid] = a;
-        s_lv[tid] = l;
+        s_xi[tid] = xi;
+        s_lv[tid] = level;
     }
-    if (tid < 4) s_info->near_mask[tid] = 0u;
-    if (tid == 4) s_info->tiny = tiny ? 1 : 0;
-    __syncthreads();
-    for (int k = tid; k < kLutBins * REP; k += blockDim.x)
-        *reinterpret_cast<uint2*>(s_lut + k * 8) = s_ent[k / REP];
-    for (int t = tid; t < (kLevels - 1) * 128; t += blockDim.x) mark_if_near(s_xi, t >> 7, 128 + (t & 127), s_info);
+    if (tid == 0) s_info->tiny = tiny ? 1 : 0;
+    if (warp < 4) {  // 32 significands a warp
+        bool near = false;
+#pragma unroll
+        for (int j = 0; j < kLevels - 1; ++j) near = is_near(__shfl_sync(kFull, xi, j), 128u + (uint32_t)tid) || near;
+        const unsigned word = __ballot_sync(kFull, near);
+        if (lane == 0) s_info->near_mask[warp] = word;
+    }
     __syncthreads();
     return !multi;
 }
@@ -298,6 +265,7 @@ __device__ __forceinline__ uint32_t horner_code(uint32_t wd, float x, uint2 entr
 }
 
 // FAST path: m != 0, every |w| <= |m|, so every x~ is a finite number in [-1, 1].
+template <int REP>
 __device__ __forceinline__ void encode32_fast(const uint32_t (&u)[16], float m, uint32_t lut_base, uint32_t (&cw)[4])
 {
     const float r = __frcp_rn(m);
@@ -310,7 +278,7 @@ __device__ __forceinline__ void encode32_fast(const uint32_t (&u)[16], float m, 
             const uint32_t uu = u[4 * h + j];
             const float2 x = __fmul2_rn(make_float2(bf_lo(uu), bf_hi(uu)), rr);
             const float2 key = lut_key2(x);
-            const uint2 e0 = lut_probe(key.x, lut_base), e1 = lut_probe(key.y, lut_base);
+            const uint2 e0 = lut_probe<REP>(key.x, lut_base), e1 = lut_probe<REP>(key.y, lut_base);
             wd = horner_code(wd, x.x, e0);
             wd = horner_code(wd, x.y, e1);
         }
