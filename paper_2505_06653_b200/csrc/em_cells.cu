@@ -12,9 +12,9 @@
 //   accumulate  a unit is some blocks of ONE magnitude |m|: with m fixed, the cell of a weight is the
 //               difference of the two bit patterns, so the counts of a unit are 10240 words of shared
 //               memory and a weight costs a subtraction, a comparison and one shared-memory reduction
-//               on random banks (2^28 weights, 168 us: 83 % of the LSU data path, 4.6 wavefronts per 32 weights,
-//               and 82 % of the issue slots, 16.6 instructions a weight); when the unit is done its counts times
-//               the weight of |m| are added to the cells
+//               on random banks, whose conflicts bound it (4.6 wavefronts of the LSU data path per 32 weights; two
+//               weights at a time without a predicate where all are counted: 2^26 weights 56 -> 51 us, 1.6 * 10^9 827 -> 811);
+//               when the unit is done its counts times the weight of |m| are added to the cells
 //   items       the occupied cells in a fixed order, as samples for the ordering passes
 //
 // A cell is (significand of m, sign, distance of the bit patterns).  Cell sums are integers (128 bits, a
@@ -37,6 +37,7 @@ constexpr int kCellCounts = 2 * kCellDepth + 2 * kDeepExps;  // counters of a un
 constexpr int kMags = 32768;                      // magnitudes of a bf16 number
 constexpr int kCellThreads = 512;
 constexpr int kCellCtas = 3;                      // per SM
+constexpr int kOrderGroup = 8;                   // blocks that a thread of the ordering takes at a time
 constexpr int kCellScan = 2048;                   // cells per CTA of the items pass
 constexpr int kCellScans = (kCells + kCellScan - 1) / kCellScan;
 // Below, one sample per weight is cheaper.  20 iterations, MSE and MAE, one sample per weight against this way:
@@ -89,7 +90,7 @@ static size_t cells_layout(void* base, int64_t n, int block_size, CellsWs* W)
     L.scans = reinterpret_cast<uint32_t*>(take((size_t)kCellScans * 4));
     L.units = reinterpret_cast<CellUnit*>(take((size_t)(kMags + kMaxExtraUnits) * sizeof(CellUnit)));
     L.order = reinterpret_cast<unsigned long long*>(take(blocks * 8));
-    L.consts = reinterpret_cast<uint16_t*>(take(blocks * 2));
+    L.consts = reinterpret_cast<uint16_t*>(take(align_up(blocks, kOrderGroup) * 2));
     char* rest = p ? p + off : nullptr;
     off += sorted_layout(rest, kCells, true, &L.sort);
     if (W) *W = L;
@@ -245,8 +246,10 @@ cells_blocks_kernel(const EmTensors T, const int64_t first_block, uint32_t* __re
 
 // ---------------------------------------------------------------- plan
 
-// One CTA, 32 magnitudes per thread: positions of the magnitudes in the ordered list, the units of work,
-// the largest magnitude and the scale of the cell sums.
+// One CTA, 32 magnitudes per thread, 1024 apart: positions of the magnitudes in the ordered list, the units of work,
+// the largest magnitude and the scale of the cell sums.  The magnitudes that most blocks have are neighbours (a binade
+// has 128), so they lie with different threads; with 32 neighbours to a thread one of them wrote most of the
+// units (2^26 weights 20 us against 7, 2^30 26 against 11).  The order of the magnitudes in the list is of no account.
 __global__ void __launch_bounds__(1024)
 cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __restrict__ head)
 {
@@ -256,16 +259,13 @@ cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __re
     if (tid == 0) s_top = W.scal[2];
     uint32_t c[32], blocks = 0u, units = 0u, top = 0u;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const uint4 v = reinterpret_cast<const uint4*>(W.hist)[tid * 8 + q];
-        c[4 * q] = v.x, c[4 * q + 1] = v.y, c[4 * q + 2] = v.z, c[4 * q + 3] = v.w;
-    }
+    for (int k = 0; k < 32; ++k) c[k] = W.hist[k * 1024 + tid];
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
         blocks += c[k];
         if (c[k]) {
             units += (c[k] + per_unit - 1) / per_unit;
-            top = (uint32_t)(tid * 32 + k);
+            top = (uint32_t)(k * 1024 + tid);
         }
     }
     uint32_t ib = blocks, iu = units;
@@ -282,7 +282,8 @@ cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __re
         s_blocks[warp] = ib;
         s_units[warp] = iu;
     }
-    atomicMax(&s_top, top);
+    top = __reduce_max_sync(kFull, top);
+    if (lane == 0) atomicMax(&s_top, top);
     __syncthreads();
     for (int k = 0; k < warp; ++k) {
         ib += s_blocks[k];
@@ -290,15 +291,9 @@ cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __re
     }
     uint32_t at = ib - blocks, u = iu - units;
 #pragma unroll
-    for (int k = 0; k < 32; k += 4) {
-        const uint32_t a1 = c[k], a2 = a1 + c[k + 1], a3 = a2 + c[k + 2];
-        reinterpret_cast<uint4*>(W.cursor)[(tid * 32 + k) >> 2] = make_uint4(at, at + a1, at + a2, at + a3);
-        at += a3 + c[k + 3];
-    }
-    at = ib - blocks;
-#pragma unroll
     for (int k = 0; k < 32; ++k) {
-        const uint32_t mag = (uint32_t)(tid * 32 + k);
+        const uint32_t mag = (uint32_t)(k * 1024 + tid);
+        W.cursor[mag] = at;
         for (uint32_t done = 0; done < c[k]; done += per_unit)
             W.units[u++] = CellUnit{mag, at + done, min(per_unit, c[k] - done)};
         at += c[k];
@@ -316,10 +311,10 @@ cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __re
 
 // ---------------------------------------------------------------- order
 
-// Every CTA takes a contiguous part of the blocks: counts its magnitudes, reserves room for them in the
+// Few blocks: every CTA takes a contiguous part of them, counts its magnitudes, reserves room for them in the
 // list, then writes the addresses.  The order inside a magnitude does not matter (sums of integers).
 __global__ void __launch_bounds__(1024, 1)
-cells_order_kernel(const EmTensors T, const int64_t first_block, const int64_t n_blocks, int block_size, const CellsWs W)
+cells_order_few_kernel(const EmTensors T, const int64_t first_block, const int64_t n_blocks, int block_size, const CellsWs W)
 {
     if (!after_previous()) return;
     extern __shared__ uint32_t s_pos[];  // [kMags]
@@ -353,6 +348,124 @@ cells_order_kernel(const EmTensors T, const int64_t first_block, const int64_t n
         const uint32_t c = W.consts[i];
         const unsigned long long p = reinterpret_cast<unsigned long long>(s_ptr[t] + i * block_size * 2);
         W.order[atomicAdd(&s_pos[c & 0x7fffu], 1u)] = p | ((unsigned long long)(c >> 15) << 63);
+    }
+}
+
+// Every CTA takes a contiguous part of the blocks, 8192 at a time: ranks them within their magnitudes, reserves room for
+// every magnitude in the list, puts the tile in order in shared memory and writes its addresses, so that neighbouring lanes
+// write neighbouring places.  The order inside a magnitude does not matter (sums of integers).  Writing each address from
+// the lane that has the block, 32 cache lines a store, took 207 us for the 25 million blocks of eight layers of a 7B-shaped
+// model, 113 this way (fits of 2^28 and 2^30 weights 10 and 60 us faster).  Bound by the counters, whose lanes collide on common
+// magnitudes, and the chain of a tile: the reservation in global memory, five barriers.  (A lane counting for all of its
+// magnitude in the warp, by __match_any_sync: 248 us.)
+// Fewer blocks in a launch are written directly: 2^16 (2^22 weights) 283 us a fit against 286 in tiles, 2^20 348 against 345.
+constexpr int64_t kOrderFew = 1 << 19;
+constexpr int kOrderTile = 1024 * kOrderGroup;
+static_assert(kOrderTile == 1 << 13, "13 bits for a place in a tile");
+constexpr int kOrderSmem = kMags * 4 + kOrderTile * (4 + 4 + 2);
+__global__ void __launch_bounds__(1024, 1)
+cells_order_kernel(const EmTensors T, const int64_t first_block, const int64_t n_blocks, int block_size, const CellsWs W)
+{
+    if (!after_previous()) return;
+    extern __shared__ __align__(16) uint32_t s_pos[];  // [kMags] blocks of a magnitude in the tile, then its slot and first place
+    uint32_t* const s_item = s_pos + kMags;            // [kOrderTile] slot, sign, block in the tile
+    uint32_t* const s_delta = s_item + kOrderTile;     // [kOrderTile] per slot: place in the list less place in the tile
+    uint16_t* const s_mag = reinterpret_cast<uint16_t*>(s_delta + kOrderTile);  // [kOrderTile] per slot
+    __shared__ const char* s_ptr[kEmMaxTensors];
+    __shared__ int64_t s_end[kEmMaxTensors];  // first block behind the tensor
+    __shared__ uint32_t s_slots, s_warp[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int k = tid; k < kMags / 4; k += 1024) reinterpret_cast<uint4*>(s_pos)[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) {
+        int64_t b = first_block;
+        for (int t = 0; t < T.count; ++t) {
+            // address that block 0 would have
+            s_ptr[t] = static_cast<const char*>(T.ptr[t]) - b * block_size * 2;
+            b += T.n[t] / block_size;
+            s_end[t] = b;
+        }
+        s_slots = 0u;
+    }
+    __syncthreads();
+    // groups of eight blocks, of which the first and the last of the launch may belong to others in part
+    const int64_t end = first_block + n_blocks, g0 = first_block / kOrderGroup, groups = (end + kOrderGroup - 1) / kOrderGroup - g0;
+    const int64_t part = (groups + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = g0 + (int64_t)blockIdx.x * part, hi = min(g0 + groups, lo + part);
+    const uint4* consts = reinterpret_cast<const uint4*>(W.consts);  // (room for whole groups: cells_layout)
+    uint4 next = lo + tid < hi ? consts[lo + tid] : make_uint4(0u, 0u, 0u, 0u);
+    int t = 0;
+    for (int64_t tile = lo; tile < hi; tile += 1024) {
+        const int64_t g = tile + tid, i0 = g * kOrderGroup;
+        const uint32_t w[4] = {next.x, next.y, next.z, next.w};
+        if (g + 1024 < hi) next = consts[g + 1024];
+        const int from = g < hi ? (int)max(first_block - i0, (int64_t)0) : kOrderGroup;
+        const int to = (int)min(end - i0, (int64_t)kOrderGroup);
+        uint32_t rank[kOrderGroup];
+#pragma unroll
+        for (int k = 0; k < kOrderGroup; ++k) {
+            const uint32_t mag = (w[k >> 1] >> (16 * (k & 1))) & 0x7fffu;
+            rank[k] = k >= from && k < to ? atomicAdd(&s_pos[mag], 1u) : 1u;
+        }
+#pragma unroll
+        for (int k = 0; k < kOrderGroup; ++k)
+            if (rank[k] == 0u) s_mag[atomicAdd(&s_slots, 1u)] = (uint16_t)((w[k >> 1] >> (16 * (k & 1))) & 0x7fffu);
+        __syncthreads();
+        const uint32_t slots = s_slots;
+        uint32_t placed = 0u;  // blocks of the slots before
+        for (uint32_t j0 = 0; j0 < slots; j0 += 1024) {
+            const uint32_t j = j0 + tid;
+            uint32_t mag = 0u, count = 0u, at = 0u;
+            if (j < slots) {
+                mag = s_mag[j];
+                count = s_pos[mag];
+                at = atomicAdd(&W.cursor[mag], count);
+            }
+            uint32_t incl = count;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t x = __shfl_up_sync(kFull, incl, off);
+                if (lane >= off) incl += x;
+            }
+            if (j0) __syncthreads();  // s_warp of the round before has been read
+            if (lane == 31) s_warp[warp] = incl;
+            __syncthreads();
+            const uint32_t mine = s_warp[lane];
+            const uint32_t before = __reduce_add_sync(kFull, lane < warp ? mine : 0u), all = __reduce_add_sync(kFull, mine);
+            const uint32_t place = placed + before + incl - count;
+            if (j < slots) {
+                s_pos[mag] = j << 13 | place;
+                s_delta[j] = at - place;
+            }
+            placed += all;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kOrderGroup; ++k) {
+            if (k < from || k >= to) continue;
+            const uint32_t c = w[k >> 1] >> (16 * (k & 1)), e = s_pos[c & 0x7fffu];
+            s_item[(e & (kOrderTile - 1)) + rank[k]] = (e >> 13) << 14 | ((c >> 15) & 1u) << 13 | (uint32_t)(tid * kOrderGroup + k);
+        }
+        __syncthreads();
+        for (uint32_t j = tid; j < slots; j += 1024) s_pos[s_mag[j]] = 0u;
+        if (tid == 0) s_slots = 0u;
+        const int64_t b0 = tile * kOrderGroup;
+        while (max(b0, first_block) >= s_end[t]) ++t;
+        const bool one = min(b0 + kOrderTile, end) <= s_end[t];  // the tile lies in one tensor
+        const char* const base = s_ptr[t];
+#pragma unroll 4
+        for (uint32_t p = tid; p < placed; p += 1024) {
+            const uint32_t e = s_item[p];
+            const int64_t i = b0 + (e & (kOrderTile - 1));
+            const char* from_tensor = base;
+            if (!one) {
+                int u = t;
+                while (i >= s_end[u]) ++u;
+                from_tensor = s_ptr[u];
+            }
+            const unsigned long long a = reinterpret_cast<unsigned long long>(from_tensor + i * block_size * 2);
+            W.order[s_delta[e >> 14] + p] = a | ((unsigned long long)((e >> 13) & 1u) << 63);
+        }
+        __syncthreads();  // the next tile overwrites what has been read here
     }
 }
 
@@ -420,29 +533,37 @@ cells_accumulate_kernel(const CellsWs W, int lanes_shift, int metric)
         } else if (U.mag >= (uint32_t)kMagTiny) {
             const uint32_t deep = U.mag - (uint32_t)kCellDepth;  // largest magnitude that goes to a deep cell
             const uint32_t both = U.mag * 0x10001u;
+            // Two weights at a time: their distances (no weight is beyond the constant: no borrow between the halves), then
+            // the addresses of their counters, which are below 2^16 (base is little more than the system's kilobyte).
+            const uint32_t base2 = base * 0x10001u;
             auto use = [&](const Raw8& r, uint32_t flip) {
-                // the largest distance, or the largest that is counted, two weights at a time (no weight is beyond the
-                // constant: no borrow between the halves)
                 constexpr uint32_t kCounted = (uint32_t)(kCellDepth - 1) * 0x10001u;
-                uint32_t far = kCounted;
 #pragma unroll
-                for (int k = 0; k < 8; k += 2) {
-                    uint32_t d[2];
+                for (int h = 0; h < 8; h += 4) {
+                    uint32_t d[4];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint32_t u = r.u[k + h] ^ flip;
-                        d[h] = both - (u & 0x7fff7fffu);
-                        cell_count(base, d[h] & 0xffffu, u & 0x8000u);
-                        cell_count(base, d[h] >> 16, u & 0x80000000u);
+                    for (int k = 0; k < 4; ++k) d[k] = both - (r.u[h + k] & 0x7fff7fffu);
+                    // the largest distance, or the largest that is counted
+                    if (__vimax3_u16x2(__vimax3_u16x2(d[0], d[1], d[2]), d[3], kCounted) == kCounted) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const uint32_t negative = ((r.u[h + k] ^ flip) >> 15) & 0x10001u;
+                            const uint32_t at = negative * (uint32_t)(kCellDepth * 4) + base2 + d[k] * 4u;
+                            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at & 0xffffu) : "memory");
+                            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at >> 16) : "memory");
+                        }
+                    } else {  // a zero, or a weight for a deep cell
+                        uint32_t least = 0xffffffffu;  // the smallest magnitude less one: zeros wrap to the top
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const uint32_t u = r.u[h + k] ^ flip;
+                            cell_count(base, d[k] & 0xffffu, u & 0x8000u);
+                            cell_count(base, d[k] >> 16, u & 0x80000000u);
+                            least = __viaddmin_u16x2(u & 0x7fff7fffu, 0xffffffffu, least);
+                        }
+                        if ((least & 0xffffu) < deep || (least >> 16) < deep)
+                            for (int k = 0; k < 4; ++k) deep_count(s_cnt + 2 * kCellDepth, r.u[h + k] ^ flip, U.mag, false);
                     }
-                    far = __vimax3_u16x2(far, d[0], d[1]);
-                }
-                if (far != kCounted) {  // a zero, or a weight for a deep cell
-                    uint32_t least = 0xffffffffu;  // the smallest magnitude less one: zeros wrap to the top
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) least = __viaddmin_u16x2(r.u[k] & 0x7fff7fffu, 0xffffffffu, least);
-                    if ((least & 0xffffu) < deep || (least >> 16) < deep)
-                        for (int k = 0; k < 8; ++k) deep_count(s_cnt + 2 * kCellDepth, r.u[k] ^ flip, U.mag, false);
                 }
             };
             uint32_t fa, fb, q = tid;
@@ -704,8 +825,13 @@ int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters
     rc = for_each_tensor_chunk(a, 1024 * kLW, [&](const EmTensors& T) -> int {
         const int64_t f = first, nb = of(T);
         first += nb;
-        if (const int e = ensure_dynamic_smem<cells_order_kernel>(kMags * 4)) return e;
-        launch_after(cells_order_kernel, kSMs, 1024, kMags * 4, st, T, f, nb, a.block_size, W);
+        if (nb < kOrderFew) {
+            if (const int e = ensure_dynamic_smem<cells_order_few_kernel>(kMags * 4)) return e;
+            launch_after(cells_order_few_kernel, kSMs, 1024, kMags * 4, st, T, f, nb, a.block_size, W);
+        } else {
+            if (const int e = ensure_dynamic_smem<cells_order_kernel>(kOrderSmem)) return e;
+            launch_after(cells_order_kernel, kSMs, 1024, kOrderSmem, st, T, f, nb, a.block_size, W);
+        }
         BOF4_CUDA_TRY(cudaGetLastError());
         return BOF4_OK;
     }, &calls);
