@@ -18,6 +18,8 @@ namespace bof4 {
 constexpr int kQThreads = 512;              // quantise / OPQ pass 1
 constexpr int kQRow = kQThreads * kLaneW;   // weights per CTA row
 constexpr int kQCtasPerSm = 2;              // two CTAs, each with its own region table
+// The batch kernels keep the table once per lane: 28 tensors of 872 million bf16 weights 356 us against 383.
+constexpr int kQBatchRep = 32;
 constexpr int kDThreads = 512;              // dequantise
 constexpr int kDCtasPerSm = 3;              // each with its own 64 KiB level-pair table
 constexpr int kDTableBytes = 256 * 32 * 8;  // [code byte][lane] pairs of levels
@@ -101,10 +103,11 @@ struct QuantTables {
 };
 
 // level = lane_level(levels)
+template <int REP>
 __device__ __forceinline__ QuantTables setup_tables(float level, float* s_xi, unsigned char* s_lut)
 {
     const float xi = lane_threshold(level);
-    const bool multi = fill_lut<kQLutRep>(xi, s_lut, [](int base) { return (uint32_t)base; });
+    const bool multi = fill_lut<REP>(xi, s_lut, [](int base) { return (uint32_t)base; });
     if (threadIdx.x < kLevels) s_xi[threadIdx.x] = xi;
     __syncthreads();
     return QuantTables{s_xi, s_lut, !multi};
@@ -114,6 +117,7 @@ __device__ __forceinline__ QuantTables setup_tables(float level, float* s_xi, un
 // the high nibble of its byte.  Each word is built by Horner steps w = 16 w + code over its 8
 // codes in the order 6 7 4 5 2 3 0 1, which leaves byte k = (code[2k] << 4) | code[2k+1].
 // use_lut (warp-uniform) requires finite x in [-1, 1].
+template <int REP>
 __device__ __forceinline__ void encode16(const float (&x)[kLaneW], const QuantTables& T, bool use_lut,
                                          uint32_t lut_base, uint32_t& w0, uint32_t& w1)
 {
@@ -132,7 +136,7 @@ __device__ __forceinline__ void encode16(const float (&x)[kLaneW], const QuantTa
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int k = 8 * h + (6 - 2 * (j >> 1)) + (j & 1);
-                const uint2 e = lut_probe<kQLutRep>(key[k], lut_base);
+                const uint2 e = lut_probe<REP>(key[k], lut_base);
                 w = w * 16u + e.y;
                 if (x[k] >= __uint_as_float(e.x)) w += 1u;
             }
@@ -155,7 +159,7 @@ __device__ __forceinline__ void encode16(const float (&x)[kLaneW], const QuantTa
 }
 
 // Block constant, normalisation, codes and stores for one lane-row of (cleaned) weights.
-template <class DT, int I, bool SIGNED, class ST>
+template <class DT, int I, bool SIGNED, class ST, int REP>
 __device__ __forceinline__ void quantize_row(const float (&v)[kLaneW], float mx, float mn, int64_t idx,
                                              bool ok, const QuantTables& T, uint32_t lut_base, int lane,
                                              uint8_t* __restrict__ codes, void* __restrict__ scales,
@@ -167,7 +171,7 @@ __device__ __forceinline__ void quantize_row(const float (&v)[kLaneW], float mx,
     float x[kLaneW];
     normalise16<true>(v, m, safe && DT::code == BF16::code, x);
     uint32_t w0, w1;
-    encode16(x, T, safe && T.lut_ok, lut_base, w0, w1);
+    encode16<REP>(x, T, safe && T.lut_ok, lut_base, w0, w1);
     if (ok) {
         st_stream64(codes + idx / 2, w0, w1);
         if ((idx & (I - 1)) == 0) store_scale<ST>(scales, idx / I, m);  // the block's first lane
@@ -204,26 +208,29 @@ __device__ __forceinline__ int first_row_of(int start)
 }
 
 // The rows r0, r0 + G, ... of one tensor of n weights (G = CTAs of the grid), its short last block included; `first` is
-// row r0 already on its way.
-template <class DT, int I, bool SIGNED, class ST>
+// row r0 already on its way.  behind() requests the row that the CTA takes after these; it is left in `first`.
+template <class DT, int I, bool SIGNED, class ST, int REP, class Behind>
 __device__ __forceinline__ void quantize_rows(const void* __restrict__ w, int64_t n, uint8_t* __restrict__ codes,
-                                              void* __restrict__ scales, const int r0, const RawRow<DT>& first,
-                                              const QuantTables& T, uint32_t lut_base, WideScratch* ws)
+                                              void* __restrict__ scales, const int r0, RawRow<DT>& first,
+                                              const QuantTables& T, uint32_t lut_base, WideScratch* ws, Behind behind)
 {
     const int lane = threadIdx.x & 31, G = gridDim.x, tail = (int)(n & (I - 1));
     const RowMap map(n - tail, kQRow, threadIdx.x);
     int r = r0;
     if (r < map.rows) {
-        RawRow<DT> raw = first;
         for (; r < map.rows; r += G) {
             const int rn = r + G;
-            const RawRow<DT> next = map.ok(rn) ? load_raw<DT>(w, map.idx(rn)) : zero_raw<DT>();
+            RawRow<DT> next = zero_raw<DT>();
+            if (map.ok(rn)) next = load_raw<DT>(w, map.idx(rn));
+            else if (rn >= map.rows) next = behind();
             float v[kLaneW], mx, mn;
-            widen(raw, v);
+            widen(first, v);
             lane_minmax(v, mx, mn);
-            quantize_row<DT, I, SIGNED, ST>(v, mx, mn, map.idx(r), map.ok(r), T, lut_base, lane, codes, scales, ws);
-            raw = next;
+            quantize_row<DT, I, SIGNED, ST, REP>(v, mx, mn, map.idx(r), map.ok(r), T, lut_base, lane, codes, scales, ws);
+            first = next;
         }
+    } else {
+        first = behind();
     }
     if (tail && r == map.rows) quantize_tail<DT, SIGNED, ST>(w, n - tail, tail, T.xi, codes, scales, n / I);
 }
@@ -238,9 +245,10 @@ quantize_kernel(const void* __restrict__ w, int64_t n, const float* __restrict__
     __shared__ float s_xi[kLevels];
     __shared__ WideScratch s_wide;
     const float level = lane_level(levels);
-    const RawRow<DT> first = first_row<DT>(w, n, (int)(n & (I - 1)), (int)blockIdx.x);
-    const QuantTables T = setup_tables(level, s_xi, s_lut);
-    quantize_rows<DT, I, SIGNED, ST>(w, n, codes, scales, (int)blockIdx.x, first, T, lut_lane_base<kQLutRep>(s_lut, threadIdx.x & 31), &s_wide);
+    RawRow<DT> first = first_row<DT>(w, n, (int)(n & (I - 1)), (int)blockIdx.x);
+    const QuantTables T = setup_tables<kQLutRep>(level, s_xi, s_lut);
+    quantize_rows<DT, I, SIGNED, ST, kQLutRep>(w, n, codes, scales, (int)blockIdx.x, first, T, lut_lane_base<kQLutRep>(s_lut, threadIdx.x & 31),
+                                               &s_wide, [] { return zero_raw<DT>(); });
 }
 
 template <class DT, int I, bool SIGNED, class ST>
@@ -253,15 +261,15 @@ quantize_batch_kernel(const __grid_constant__ QuantBatch B, const float* __restr
     __shared__ WideScratch s_wide;
     const int G = gridDim.x;
     auto row_of = [&](int t) { return first_row_of(B.start[t]); };
-    auto fetch = [&](int t) { return first_row<DT>(B.w[t], B.n[t], (int)(B.n[t] & (I - 1)), row_of(t)); };
+    auto fetch = [&](int t) {
+        return t < B.count ? first_row<DT>(B.w[t], B.n[t], (int)(B.n[t] & (I - 1)), row_of(t)) : zero_raw<DT>();
+    };
     const float level = lane_level(levels);
     RawRow<DT> first = fetch(0);
-    const QuantTables T = setup_tables(level, s_xi, s_lut);
-    for (int t = 0; t < B.count; ++t) {
-        if (t > 0) first = fetch(t);
-        quantize_rows<DT, I, SIGNED, ST>(B.w[t], B.n[t], B.codes[t], B.scales[t], row_of(t), first, T,
-                                         lut_lane_base<kQLutRep>(s_lut, threadIdx.x & 31), &s_wide);
-    }
+    const QuantTables T = setup_tables<kQBatchRep>(level, s_xi, s_lut);
+    for (int t = 0; t < B.count; ++t)
+        quantize_rows<DT, I, SIGNED, ST, kQBatchRep>(B.w[t], B.n[t], B.codes[t], B.scales[t], row_of(t), first, T,
+                                                     lut_lane_base<kQBatchRep>(s_lut, threadIdx.x & 31), &s_wide, [&] { return fetch(t + 1); });
 }
 
 // ---------------------------------------------------------------- quantise, bf16 weights
@@ -270,8 +278,7 @@ quantize_batch_kernel(const __grid_constant__ QuantBatch B, const float* __restr
 // after next is issued before a row is processed and no register is copied between iterations.
 
 constexpr int kQRow32 = kQThreads * kLW;  // weights per CTA row
-// The batch kernel keeps the table once per lane: 28 tensors of 872 million weights 356 us against 383.
-constexpr int kQBatchRep = 32;
+
 
 struct QuantShared32 {
     float xi[kLevels], lv[kLevels];
@@ -769,7 +776,7 @@ opq_pass1_kernel(const void* __restrict__ w, int64_t n, const float* __restrict_
     __shared__ float s_xi[kLevels];
     __shared__ WideScratch s_wide;
     QuantTables T{s_xi, s_lut, false};
-    if (QUANT) T = setup_tables(lane_level(levels), s_xi, s_lut);
+    if (QUANT) T = setup_tables<kQLutRep>(lane_level(levels), s_xi, s_lut);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lut_base = lut_lane_base<kQLutRep>(s_lut, lane);  // table base of this lane
     const RowMap map(n, kQRow, threadIdx.x);
@@ -819,7 +826,7 @@ opq_pass1_kernel(const void* __restrict__ w, int64_t n, const float* __restrict_
             counts[tile] = 0;
         }
         if (QUANT) {
-            quantize_row<DT, I, SIGNED, ST>(v, mx, mn, idx, ok, T, lut_base, lane, codes, scales, &s_wide);
+            quantize_row<DT, I, SIGNED, ST, kQLutRep>(v, mx, mn, idx, ok, T, lut_base, lane, codes, scales, &s_wide);
         } else if (w_clean != nullptr && ok) {
             store_row(DT{}, w_clean, idx, v);
         }
@@ -1608,8 +1615,8 @@ extern "C" int bof4_quantize_batch(const void* const* h_w, const int64_t* h_n, i
                 BOF4_DISPATCH_I(block_size,
                     BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                         { constexpr auto kern = quantize_batch_kernel<F32, I_, SG, F32>;
-                          if ((rc = ensure_dynamic_smem<kern>(kQLutBytes))) return rc;
-                          launch_after(kern, grid, kQThreads, kQLutBytes, st, B, d_codebook); }));
+                          if ((rc = ensure_dynamic_smem<kern>(lut_bytes(kQBatchRep)))) return rc;
+                          launch_after(kern, grid, kQThreads, lut_bytes(kQBatchRep), st, B, d_codebook); }));
             }
             BOF4_CUDA_TRY(cudaGetLastError());
             B.count = 0;
