@@ -52,6 +52,12 @@ size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W)
 // Every lane owns 16 consecutive weights; x = RN(w / m) and |m| (1 for the normalised-domain metrics) go
 // to the sample array in the order of the weights.  Bound by its stores (8 bytes per weight).  Every CTA leaves its sum of
 // squares and its largest constant in slots of its own; the first launch of a fit writes all slots, and the head.
+__device__ __forceinline__ void st_256(void* p, const Raw8& r)
+{
+    asm volatile("st.global.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(r.u[0]), "r"(r.u[1]), "r"(r.u[2]), "r"(r.u[3]),
+                 "r"(r.u[4]), "r"(r.u[5]), "r"(r.u[6]), "r"(r.u[7])
+                 : "memory");
+}
 template <class DT, int I, bool SIGNED>
 __global__ void __launch_bounds__(512, 2)
 sort_samples_kernel(const EmTensors T, const uint32_t first, const uint32_t n, float2* __restrict__ items,
@@ -90,14 +96,24 @@ sort_samples_kernel(const EmTensors T, const uint32_t first, const uint32_t n, f
         if (!ok) continue;
         top = fmaxf(top, gmax);
         const float am = unit ? 1.0f : fabsf(m);
+        double part[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
         for (int k = 0; k < kLaneW; ++k) {  // (m x)^2: with the x of the other sums the error is free of cancellation
             const double e = (double)x[k] * (double)am;
-            sum = fma(e, e, sum);
+            part[k & 3] = fma(e, e, part[k & 3]);
         }
-        float4* dst = reinterpret_cast<float4*>(items + s_item0[t] + idx);
+        sum += (part[0] + part[1]) + (part[2] + part[3]);
+        float2* dst = items + s_item0[t] + idx;
+        const uint32_t payload = __float_as_uint(am);
+        if ((s_item0[t] & 3u) == 0u) {
 #pragma unroll
-        for (int k = 0; k < kLaneW; k += 2) dst[k >> 1] = make_float4(x[k], am, x[k + 1], am);
+            for (int k = 0; k < kLaneW; k += 4)
+                st_256(dst + k, Raw8{{__float_as_uint(x[k]), payload, __float_as_uint(x[k + 1]), payload, __float_as_uint(x[k + 2]), payload,
+                                      __float_as_uint(x[k + 3]), payload}});
+        } else {  // behind a tensor whose length is no multiple of four
+#pragma unroll
+            for (int k = 0; k < kLaneW; k += 2) reinterpret_cast<float4*>(dst)[k >> 1] = make_float4(x[k], am, x[k + 1], am);
+        }
     }
     uint32_t bits = __float_as_uint(top);
 #pragma unroll
@@ -227,15 +243,25 @@ __device__ __forceinline__ void rank_in_warp(uint32_t* cnt, int lane, Digit digi
 
 // Stable scatter by one digit.  A sample goes to: samples with a smaller digit + samples of the same
 // digit in earlier CTAs + in earlier tiles of this CTA + in earlier warps of the tile + earlier in the
-// warp (each warp owns 256 consecutive samples of a tile, 32 at a time).
-template <int SHIFT>
+// warp (each warp owns 256 consecutive samples of a tile, 32 at a time).  STAGED: a tile is put in order in shared memory first,
+// so that neighbouring lanes store neighbouring samples, not 32 cache lines a store.
+constexpr int kScatterSmem = kSortTile * 8;
+// Fits over so many samples, one per weight, stage them: the ordering of 2^20 takes 88 us instead of 92, of 2^23 316 instead of
+// 384, of 2^26 2215 instead of 3790.  Fewer (and cells, of which
+// there are some 10^5) fill a tile in part, and the barriers cost more than the stores: 2^16 weights 97.5 us against 100,
+// cells of 2^22 weights 282 against 285.
+constexpr int64_t kStagedMin = 1 << 19;
+template <int SHIFT, bool STAGED>
 __global__ void __launch_bounds__(kSortThreads)
 sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ head, const uint32_t* __restrict__ counts,
                     float2* __restrict__ out)
 {
     if (!after_previous()) return;
+    extern __shared__ __align__(16) unsigned char s_window[];
+    float2* const s_item = reinterpret_cast<float2*>(s_window);  // [kSortTile] STAGED
     __shared__ uint32_t s_cnt[32][256];
     __shared__ uint32_t s_base[256], s_warp[8];
+    __shared__ uint32_t s_place[256];  // of a digit: where its first sample of the tile goes, less its place in the tile
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t lo, hi;
     sort_part(*head, blockIdx.x, lo, hi);
@@ -284,23 +310,70 @@ sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ 
         __syncwarp();
         rank_in_warp<kSortPerThread>(s_cnt[warp], lane, [&](int k) { return ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u; },
                                      [&](int k) { return i0 + 32 * k < hi; }, rank);
-        __syncthreads();
-        if (tid < 256) {
-            uint32_t c[32], run = s_base[tid];
+        if constexpr (STAGED) {
+            __syncthreads();
+            uint32_t c[32], mine = 0u, incl = 0u;
+            if (tid < 256) {
 #pragma unroll
-            for (int w = 0; w < 32; ++w) c[w] = s_cnt[w][tid];
+                for (int w = 0; w < 32; ++w) {
+                    c[w] = s_cnt[w][tid];
+                    mine += c[w];
+                }
+                incl = mine;
 #pragma unroll
-            for (int w = 0; w < 32; ++w) {
-                s_cnt[w][tid] = run;
-                run += c[w];
+                for (int off = 1; off < 32; off <<= 1) {
+                    const uint32_t t = __shfl_up_sync(kFull, incl, off);
+                    if (lane >= off) incl += t;
+                }
+                if (lane == 31) s_warp[warp] = incl;
             }
-            s_base[tid] = run;
-        }
-        __syncthreads();
+            __syncthreads();
+            if (tid < 256) {
+                for (int k = 0; k < warp; ++k) incl += s_warp[k];
+                uint32_t run = incl - mine;
+                s_place[tid] = s_base[tid] - run;
+                s_base[tid] += mine;
 #pragma unroll
-        for (int k = 0; k < kSortPerThread; ++k) {
-            const uint32_t d = ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u;
-            if (i0 + 32 * k < hi) out[s_cnt[warp][d] + rank[k]] = item[k];
+                for (int w = 0; w < 32; ++w) {
+                    s_cnt[w][tid] = run;
+                    run += c[w];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kSortPerThread; ++k) {
+                const uint32_t d = ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u;
+                if (i0 + 32 * k < hi) s_item[s_cnt[warp][d] + rank[k]] = item[k];
+            }
+            __syncthreads();
+            const uint32_t len = min((uint32_t)kSortTile, hi - t0);
+#pragma unroll
+            for (int k = 0; k < kSortPerThread; ++k) {
+                const uint32_t j = tid + k * kSortThreads;
+                if (j < len) {
+                    const float2 it = s_item[j];
+                    out[s_place[((uint32_t)sort_bin(it.x) >> SHIFT) & 255u] + j] = it;
+                }
+            }
+        } else {
+            __syncthreads();
+            if (tid < 256) {
+                uint32_t c[32], run = s_base[tid];
+#pragma unroll
+                for (int w = 0; w < 32; ++w) c[w] = s_cnt[w][tid];
+#pragma unroll
+                for (int w = 0; w < 32; ++w) {
+                    s_cnt[w][tid] = run;
+                    run += c[w];
+                }
+                s_base[tid] = run;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kSortPerThread; ++k) {
+                const uint32_t d = ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u;
+                if (i0 + 32 * k < hi) out[s_cnt[warp][d] + rank[k]] = item[k];
+            }
         }
         __syncthreads();  // s_cnt is cleared for the next tile
     }
@@ -1339,10 +1412,21 @@ int samples(const EmTensors& T, int block_size, uint32_t first, uint32_t n, cons
 
 int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
 {
-    launch_after(sort_count_kernel<0>, kSortGrid, kSortThreads, 0, st, W.a, W.n_items, W.counts);
-    launch_after(sort_scatter_kernel<0>, kSortGrid, kSortThreads, 0, st, W.a, W.n_items, W.counts, W.b);
-    launch_after(sort_count_kernel<8>, kSortGrid, kSortThreads, 0, st, W.b, W.n_items, W.counts);
-    launch_after(sort_scatter_kernel<8>, kSortGrid, kSortThreads, 0, st, W.b, W.n_items, W.counts, W.a);
+    const bool staged = !F.acc && F.n_max >= kStagedMin;
+    auto pass = [&](auto shift, const float2* in, float2* out) -> int {
+        constexpr int S = decltype(shift)::value;
+        launch_after(sort_count_kernel<S>, kSortGrid, kSortThreads, 0, st, in, W.n_items, W.counts);
+        if (staged) {
+            constexpr auto kern = sort_scatter_kernel<S, true>;
+            if (const int rc = ensure_dynamic_smem<kern>(kScatterSmem)) return rc;
+            launch_after(kern, kSortGrid, kSortThreads, kScatterSmem, st, in, W.n_items, W.counts, out);
+        } else {
+            launch_after(sort_scatter_kernel<S, false>, kSortGrid, kSortThreads, 0, st, in, W.n_items, W.counts, out);
+        }
+        return BOF4_OK;
+    };
+    int rc;
+    if ((rc = pass(std::integral_constant<int, 0>{}, W.a, W.b)) || (rc = pass(std::integral_constant<int, 8>{}, W.b, W.a))) return rc;
     SortWs V = W;  // the ordered samples are in the first array
     V.a = W.b;
     V.b = W.a;

@@ -64,6 +64,9 @@ struct SortWs {
 // The lines below are fits to these.  Where they cross, in iterations: fp32 MSE 6 at 2^20, 11 at 2^22, 22 at 2^24, 37 at 2^26,
 // medians 4, 4, 11, 29; bf16 MSE 6 from 3 * 2^19 to 2^22, 4 from 2^24 on, medians 4.  With four iterations for all,
 // fits of 4 and 8 over 2^24 fp32 weights took 787 and 796 us (MSE) against 160 and 307 streamed.
+// Samples that are staged (em_sorted.cu) and cells are ordered faster since: 88, 185, 316, 601, 1120 and 2215 us for k = 1, 4, ... 64
+// fp32, some 7 % less for cells.  The lines have stayed where they were, so fp32 fits of 2^24 and more are streamed up to twice as many
+// iterations as would pay (2^26 MSE: 20).
 // Fewer than four iterations are not ordered, although two or three would pay for bf16 data from 2^26 weights on (2^28, three: 1120
 // us streamed, about 400 ordered): such a fit gets by with the small workspace.
 inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool cells)
