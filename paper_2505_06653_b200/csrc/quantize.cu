@@ -18,7 +18,7 @@ namespace bof4 {
 constexpr int kQThreads = 512;              // quantise / OPQ pass 1
 constexpr int kQRow = kQThreads * kLaneW;   // weights per CTA row
 constexpr int kQCtasPerSm = 2;              // two CTAs, each with its own region table
-// The batch kernels keep the table once per lane: 28 tensors of 872 million bf16 weights 356 us against 383.
+// The batch kernels keep the table once per lane: 28 tensors of 872 million bf16 weights 357 us against 383.
 constexpr int kQBatchRep = 32;
 constexpr int kDThreads = 512;              // dequantise
 constexpr int kDCtasPerSm = 3;              // each with its own 64 KiB level-pair table
@@ -189,6 +189,7 @@ struct QuantBatch {
     void* scales[kQBatch];
     int64_t n[kQBatch];
     int start[kQBatch];  // CTA that takes the tensor's first row
+    int rows[kQBatch];   // its rows, a short last block included
     int count;
 };
 
@@ -205,6 +206,21 @@ __device__ __forceinline__ int first_row_of(int start)
 {
     const int r = (int)blockIdx.x - start;
     return r < 0 ? r + (int)gridDim.x : r;
+}
+
+// Whether this CTA takes a row of tensor t.  (Most CTAs have none of a small tensor: this is all that it costs them.)
+template <class Batch>
+__device__ __forceinline__ bool takes(const Batch& B, int t)
+{
+    return t < B.count && first_row_of(B.start[t]) < B.rows[t];
+}
+// The next tensor behind t that it takes a row of, or the number of tensors.
+template <class Batch>
+__device__ __forceinline__ int next_tensor(const Batch& B, int t)
+{
+    do ++t;
+    while (t < B.count && !takes(B, t));
+    return t;
 }
 
 // The rows r0, r0 + G, ... of one tensor of n weights (G = CTAs of the grid), its short last block included; `first` is
@@ -259,17 +275,19 @@ quantize_batch_kernel(const __grid_constant__ QuantBatch B, const float* __restr
     extern __shared__ __align__(16) unsigned char s_lut[];
     __shared__ float s_xi[kLevels];
     __shared__ WideScratch s_wide;
-    const int G = gridDim.x;
-    auto row_of = [&](int t) { return first_row_of(B.start[t]); };
     auto fetch = [&](int t) {
-        return t < B.count ? first_row<DT>(B.w[t], B.n[t], (int)(B.n[t] & (I - 1)), row_of(t)) : zero_raw<DT>();
+        return t < B.count ? first_row<DT>(B.w[t], B.n[t], (int)(B.n[t] & (I - 1)), first_row_of(B.start[t])) : zero_raw<DT>();
     };
     const float level = lane_level(levels);
-    RawRow<DT> first = fetch(0);
+    int t = next_tensor(B, -1);
+    RawRow<DT> first = fetch(t);
     const QuantTables T = setup_tables<kQBatchRep>(level, s_xi, s_lut);
-    for (int t = 0; t < B.count; ++t)
-        quantize_rows<DT, I, SIGNED, ST, kQBatchRep>(B.w[t], B.n[t], B.codes[t], B.scales[t], row_of(t), first, T,
-                                                     lut_lane_base<kQBatchRep>(s_lut, threadIdx.x & 31), &s_wide, [&] { return fetch(t + 1); });
+    while (t < B.count) {
+        const int then = next_tensor(B, t);
+        quantize_rows<DT, I, SIGNED, ST, kQBatchRep>(B.w[t], B.n[t], B.codes[t], B.scales[t], first_row_of(B.start[t]), first, T,
+                                                     lut_lane_base<kQBatchRep>(s_lut, threadIdx.x & 31), &s_wide, [&] { return fetch(then); });
+        t = then;
+    }
 }
 
 // ---------------------------------------------------------------- quantise, bf16 weights
@@ -426,11 +444,10 @@ quantize32_batch_kernel(const __grid_constant__ QuantBatch B, const float* __res
     extern __shared__ __align__(16) unsigned char s_lut[];
     __shared__ QuantShared32 S;
     const int G = gridDim.x;
-    auto row_of = [&](int t) { return first_row_of(B.start[t]); };
     auto fetch = [&](int t) -> Raw32 {
-        if (t >= B.count) return zero_raw32();
+        if (!takes(B, t)) return zero_raw32();
         const RowMap32 map(B.n[t] & ~(int64_t)(I - 1), kQRow32, threadIdx.x);
-        const int r = row_of(t);
+        const int r = first_row_of(B.start[t]);
         return map.ok(r) ? load_raw32(B.w[t], map.idx(r)) : zero_raw32();
     };
     const float level = lane_level(levels);
@@ -439,9 +456,15 @@ quantize32_batch_kernel(const __grid_constant__ QuantBatch B, const float* __res
     const bool fast_ok = lut_ok && !S.info.tiny;
     const uint32_t lut_base = lut_lane_base<kQBatchRep>(s_lut, threadIdx.x & 31);
     for (int t = 0; t < B.count; ++t) {
+        // (Going from one tensor with a row of this CTA to the next, as the fp32 kernel does, takes the 28 tensors 365 us, not
+        // 357: a register more in the loop over rows.)
+        if (!takes(B, t)) {
+            first = fetch(t + 1);
+            continue;
+        }
         const int tail = (int)(B.n[t] & (I - 1));
         const int64_t n = B.n[t] - tail;
-        const int rows = (int)((n + kQRow32 - 1) / kQRow32), r0 = row_of(t);
+        const int rows = (int)((n + kQRow32 - 1) / kQRow32), r0 = first_row_of(B.start[t]);
         // The next tensor's first row is requested with this one's last: a row's latency for every tensor otherwise (28 tensors
         // of 872 million weights 382 us against 356, 14 of 77 million 52 against 46).
         quantize32_rows<I, SIGNED, ST, kQBatchRep>(B.w[t], n, B.codes[t], B.scales[t], r0, first, fast_ok, lut_base, &S, [&] { return fetch(t + 1); });
@@ -596,7 +619,7 @@ struct DequantBatch {
     const void* scales[kQBatch];
     void* out[kQBatch];
     int64_t n[kQBatch];
-    int start[kQBatch];
+    int start[kQBatch], rows[kQBatch];
     int count;
 };
 
@@ -608,11 +631,15 @@ dequantize_batch_kernel(const __grid_constant__ DequantBatch B, const float* __r
     extern __shared__ __align__(16) unsigned char s_tab[];
     auto fetch = [&](int t) { return dequant_load<ST, I>(B.codes[t], B.scales[t], B.n[t] & ~(int64_t)(I - 1), first_row_of(B.start[t])); };
     const float level = lane_level(levels);
-    DequantRow first = fetch(0);
+    int t = next_tensor(B, -1);
+    if (t >= B.count) return;
+    DequantRow first = fetch(t);
     build_pair_table(level, s_tab);
-    for (int t = 0; t < B.count; ++t) {
-        if (t > 0) first = fetch(t);
+    while (true) {
         dequantize_rows<ST, OT, I>(B.codes[t], B.scales[t], B.n[t], B.out[t], s_tab, first_row_of(B.start[t]), first);
+        t = next_tensor(B, t);
+        if (t >= B.count) break;
+        first = fetch(t);
     }
 }
 
@@ -1599,7 +1626,8 @@ extern "C" int bof4_quantize_batch(const void* const* h_w, const int64_t* h_n, i
             B.scales[B.count] = h_scales[t];
             B.n[B.count] = h_n[t];
             B.start[B.count] = (int)(rows % G);
-            rows += (n_whole + row - 1) / row + (h_n[t] > n_whole ? 1 : 0);
+            B.rows[B.count] = (int)((n_whole + row - 1) / row + (h_n[t] > n_whole ? 1 : 0));
+            rows += B.rows[B.count];
             ++B.count;
         }
         if (B.count == kQBatch || (t == n_tensors && B.count > 0)) {
@@ -1667,7 +1695,8 @@ extern "C" int bof4_dequantize_batch(const uint8_t* const* h_codes, const void* 
             B.out[B.count] = h_out[t];
             B.n[B.count] = h_n[t];
             B.start[B.count] = (int)(rows % G);
-            rows += (n_whole + kDRow - 1) / kDRow + (h_n[t] > n_whole ? 1 : 0);
+            B.rows[B.count] = (int)((n_whole + kDRow - 1) / kDRow + (h_n[t] > n_whole ? 1 : 0));
+            rows += B.rows[B.count];
             ++B.count;
         }
         if (B.count == kQBatch || (t == n_tensors && B.count > 0)) {
