@@ -102,14 +102,19 @@ struct QuantTables {
     bool lut_ok;
 };
 
-// level = lane_level(levels)
-template <int REP>
+// level = lane_level(levels).  READ_BACK: whether the table serves the codebook is read back from shared memory.  Kept from the
+// ballots it cost the loop of the absolute variants of quantize_kernel two spilled registers: blocks of 64, 2^24 and 2^26 weights
+// 20.2 and 69.1 us, 19.7 and 67.6 this way.  (The OPQ pass spills with it, and has it from the ballots.)
+template <int REP, bool READ_BACK = false>
 __device__ __forceinline__ QuantTables setup_tables(float level, float* s_xi, unsigned char* s_lut)
 {
     const float xi = lane_threshold(level);
-    const bool multi = fill_lut<REP>(xi, s_lut, [](int base) { return (uint32_t)base; });
+    bool multi = fill_lut<REP>(xi, s_lut, [](int base) { return (uint32_t)base; });
     if (threadIdx.x < kLevels) s_xi[threadIdx.x] = xi;
+    __shared__ int s_multi;
+    if (READ_BACK && threadIdx.x == 0) s_multi = multi ? 1 : 0;
     __syncthreads();
+    if (READ_BACK) multi = s_multi != 0;
     return QuantTables{s_xi, s_lut, !multi};
 }
 
@@ -236,9 +241,7 @@ __device__ __forceinline__ void quantize_rows(const void* __restrict__ w, int64_
     if (r < map.rows) {
         for (; r < map.rows; r += G) {
             const int rn = r + G;
-            RawRow<DT> next = zero_raw<DT>();
-            if (map.ok(rn)) next = load_raw<DT>(w, map.idx(rn));
-            else if (rn >= map.rows) next = behind();
+            const RawRow<DT> next = rn < map.rows ? (map.ok(rn) ? load_raw<DT>(w, map.idx(rn)) : zero_raw<DT>()) : behind();
             float v[kLaneW], mx, mn;
             widen(first, v);
             lane_minmax(v, mx, mn);
@@ -262,7 +265,7 @@ quantize_kernel(const void* __restrict__ w, int64_t n, const float* __restrict__
     __shared__ WideScratch s_wide;
     const float level = lane_level(levels);
     RawRow<DT> first = first_row<DT>(w, n, (int)(n & (I - 1)), (int)blockIdx.x);
-    const QuantTables T = setup_tables<kQLutRep>(level, s_xi, s_lut);
+    const QuantTables T = setup_tables<kQLutRep, true>(level, s_xi, s_lut);
     quantize_rows<DT, I, SIGNED, ST, kQLutRep>(w, n, codes, scales, (int)blockIdx.x, first, T, lut_lane_base<kQLutRep>(s_lut, threadIdx.x & 31),
                                                &s_wide, [] { return zero_raw<DT>(); });
 }
