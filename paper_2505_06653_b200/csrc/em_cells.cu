@@ -35,6 +35,8 @@ constexpr int kDeepCells = 128 * kCellRow;        // first deep cell: positive o
 constexpr int kCells = kDeepCells + 2 * kDeepExps;
 constexpr int kCellCounts = 2 * kCellDepth + 2 * kDeepExps;  // counters of a unit: one magnitude, zeros left out
 constexpr int kMags = 32768;                      // magnitudes of a bf16 number
+constexpr int kCellBaseMax = 8192;                // bound on where a unit's counters begin in shared memory: behind the system's
+                                                  // kilobyte and the kernel's own variables
 constexpr int kCellThreads = 512;
 constexpr int kCellCtas = 3;                      // per SM
 constexpr int kOrderGroup = 8;                   // blocks that a thread of the ordering takes at a time
@@ -507,6 +509,7 @@ cells_accumulate_kernel(const CellsWs W, int lanes_shift, int metric)
     extern __shared__ uint32_t s_cnt[];  // [kCellCounts]
     __shared__ CellUnit s_unit;
     __shared__ uint32_t s_seen[kCellThreads / 32];
+    static_assert(1024 + sizeof(s_unit) + sizeof(s_seen) + 256 <= kCellBaseMax, "base below");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(s_cnt);
     const uint32_t units = W.scal[0], max_mag = W.scal[3];
@@ -534,7 +537,8 @@ cells_accumulate_kernel(const CellsWs W, int lanes_shift, int metric)
             const uint32_t deep = U.mag - (uint32_t)kCellDepth;  // largest magnitude that goes to a deep cell
             const uint32_t both = U.mag * 0x10001u;
             // Two weights at a time: their distances (no weight is beyond the constant: no borrow between the halves), then
-            // the addresses of their counters, which are below 2^16 (base is little more than the system's kilobyte).
+            // the addresses of their counters, two to a word: they have to stay below 2^16.
+            static_assert(2 * kCellDepth * 4 + kCellBaseMax <= 1 << 16, "an address would carry into the other half");
             const uint32_t base2 = base * 0x10001u;
             auto use = [&](const Raw8& r, uint32_t flip) {
                 constexpr uint32_t kCounted = (uint32_t)(kCellDepth - 1) * 0x10001u;
