@@ -244,7 +244,8 @@ __device__ __forceinline__ void rank_in_warp(uint32_t* cnt, int lane, Digit digi
 // Stable scatter by one digit.  A sample goes to: samples with a smaller digit + samples of the same
 // digit in earlier CTAs + in earlier tiles of this CTA + in earlier warps of the tile + earlier in the
 // warp (each warp owns 256 consecutive samples of a tile, 32 at a time).  STAGED: a tile is put in order in shared memory first,
-// so that neighbouring lanes store neighbouring samples, not 32 cache lines a store.
+// so that neighbouring lanes store neighbouring samples, not 32 cache lines a store.  (A digit's counts per warp go back to shared memory
+// as they are added up: kept in registers over the barriers they spilled 90 bytes.)
 constexpr int kScatterSmem = kSortTile * 8;
 // Fits over so many samples, one per weight, stage them: the ordering of 2^20 takes 88 us instead of 92, of 2^23 316 instead of
 // 384, of 2^26 2215 instead of 3790.  Fewer (and cells, of which
@@ -261,7 +262,8 @@ sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ 
     float2* const s_item = reinterpret_cast<float2*>(s_window);  // [kSortTile] STAGED
     __shared__ uint32_t s_cnt[32][256];
     __shared__ uint32_t s_base[256], s_warp[8];
-    __shared__ uint32_t s_place[256];  // of a digit: where its first sample of the tile goes, less its place in the tile
+    // of a digit: the place of its first sample in the tile, and where that goes less this place
+    __shared__ uint32_t s_first[256], s_place[256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t lo, hi;
     sort_part(*head, blockIdx.x, lo, hi);
@@ -312,12 +314,13 @@ sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ 
                                      [&](int k) { return i0 + 32 * k < hi; }, rank);
         if constexpr (STAGED) {
             __syncthreads();
-            uint32_t c[32], mine = 0u, incl = 0u;
+            uint32_t mine = 0u, incl = 0u;
             if (tid < 256) {
-#pragma unroll
+#pragma unroll 8
                 for (int w = 0; w < 32; ++w) {
-                    c[w] = s_cnt[w][tid];
-                    mine += c[w];
+                    const uint32_t c = s_cnt[w][tid];
+                    s_cnt[w][tid] = mine;
+                    mine += c;
                 }
                 incl = mine;
 #pragma unroll
@@ -330,20 +333,16 @@ sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ 
             __syncthreads();
             if (tid < 256) {
                 for (int k = 0; k < warp; ++k) incl += s_warp[k];
-                uint32_t run = incl - mine;
-                s_place[tid] = s_base[tid] - run;
+                const uint32_t first = incl - mine;
+                s_first[tid] = first;
+                s_place[tid] = s_base[tid] - first;
                 s_base[tid] += mine;
-#pragma unroll
-                for (int w = 0; w < 32; ++w) {
-                    s_cnt[w][tid] = run;
-                    run += c[w];
-                }
             }
             __syncthreads();
 #pragma unroll
             for (int k = 0; k < kSortPerThread; ++k) {
                 const uint32_t d = ((uint32_t)sort_bin(item[k].x) >> SHIFT) & 255u;
-                if (i0 + 32 * k < hi) s_item[s_cnt[warp][d] + rank[k]] = item[k];
+                if (i0 + 32 * k < hi) s_item[s_first[d] + s_cnt[warp][d] + rank[k]] = item[k];
             }
             __syncthreads();
             const uint32_t len = min((uint32_t)kSortTile, hi - t0);
