@@ -96,24 +96,20 @@ sort_samples_kernel(const EmTensors T, const uint32_t first, const uint32_t n, f
         if (!ok) continue;
         top = fmaxf(top, gmax);
         const float am = unit ? 1.0f : fabsf(m);
-        double part[4] = {0.0, 0.0, 0.0, 0.0};
+        double part[2] = {0.0, 0.0};
 #pragma unroll
         for (int k = 0; k < kLaneW; ++k) {  // (m x)^2: with the x of the other sums the error is free of cancellation
             const double e = (double)x[k] * (double)am;
-            part[k & 3] = fma(e, e, part[k & 3]);
+            part[k & 1] = fma(e, e, part[k & 1]);
         }
-        sum += (part[0] + part[1]) + (part[2] + part[3]);
+        sum += part[0] + part[1];
+        // 32-byte aligned: the tensors of a launch are whole blocks, of 32 weights at least, and so is what lies before them
         float2* dst = items + s_item0[t] + idx;
         const uint32_t payload = __float_as_uint(am);
-        if ((s_item0[t] & 3u) == 0u) {
 #pragma unroll
-            for (int k = 0; k < kLaneW; k += 4)
-                st_256(dst + k, Raw8{{__float_as_uint(x[k]), payload, __float_as_uint(x[k + 1]), payload, __float_as_uint(x[k + 2]), payload,
-                                      __float_as_uint(x[k + 3]), payload}});
-        } else {  // behind a tensor whose length is no multiple of four
-#pragma unroll
-            for (int k = 0; k < kLaneW; k += 2) reinterpret_cast<float4*>(dst)[k >> 1] = make_float4(x[k], am, x[k + 1], am);
-        }
+        for (int k = 0; k < kLaneW; k += 4)
+            st_256(dst + k, Raw8{{__float_as_uint(x[k]), payload, __float_as_uint(x[k + 1]), payload, __float_as_uint(x[k + 2]), payload,
+                                  __float_as_uint(x[k + 3]), payload}});
     }
     uint32_t bits = __float_as_uint(top);
 #pragma unroll
@@ -247,10 +243,10 @@ __device__ __forceinline__ void rank_in_warp(uint32_t* cnt, int lane, Digit digi
 // so that neighbouring lanes store neighbouring samples, not 32 cache lines a store.  (A digit's counts per warp go back to shared memory
 // as they are added up: kept in registers over the barriers they spilled 90 bytes.)
 constexpr int kScatterSmem = kSortTile * 8;
-// Fits over so many samples, one per weight, stage them: the ordering of 2^20 takes 88 us instead of 92, of 2^23 316 instead of
-// 384, of 2^26 2215 instead of 3790.  Fewer (and cells, of which
-// there are some 10^5) fill a tile in part, and the barriers cost more than the stores: 2^16 weights 97.5 us against 100,
-// cells of 2^22 weights 282 against 285.
+// Fits over so many samples, one per weight, stage them: the ordering of 2^20 takes 87 us instead of 92, of 2^23 298 instead of
+// 384, of 2^24 563 instead of 778, of 2^26 2030 instead of 3790.  Fewer (and cells, of which there are some 10^5) fill a tile in
+// part, and the barriers cost what the stores save.  Staged and not, 40 iterations: 2^18 weights 140.8 and 138.7 us, 2^19 147.4
+// and 147.5, 3 * 2^18 152 and 155, 2^20 157 and 163.
 constexpr int64_t kStagedMin = 1 << 19;
 template <int SHIFT, bool STAGED>
 __global__ void __launch_bounds__(kSortThreads)
