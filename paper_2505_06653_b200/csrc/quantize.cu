@@ -22,7 +22,8 @@ constexpr int kQCtasPerSm = 2;              // two CTAs, each with its own regio
 constexpr int kQBatchRep = 32;
 constexpr int kDThreads = 512;              // dequantise
 constexpr int kDCtasPerSm = 3;              // each with its own 64 KiB level-pair table
-constexpr int kDTableBytes = 256 * 32 * 8;  // [code byte][lane] pairs of levels
+constexpr int kDTableRow = 256;              // 16 columns of 8 bytes, and as many bytes that are not used
+constexpr int kDTableBytes = 256 * kDTableRow;  // [code byte][lane & 15] pairs of levels
 constexpr int kDLaneW = 32;                 // outputs per lane and row (16 code bytes in)
 constexpr int kDRow = kDThreads * kDLaneW;  // outputs per CTA row (dequantise)
 
@@ -501,16 +502,22 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 
 // One code byte holds two weights, so the levels are tabulated per byte: entry b is the pair
 // (xhat[b >> 4], xhat[b & 15]); one 8-byte shared-memory read and one packed multiplication by
-// the block constant give both products (Eq. 3).  The table is kept once per lane ([byte][lane],
-// 64 KiB): the code bytes of the 32 lanes are unrelated, and a shared table of 256 entries made
-// every read a three-fold bank conflict on average, which bound the kernel; with a column per
-// lane the bank only depends on the lane.
+// the block constant give both products (Eq. 3).  The code bytes of the lanes are unrelated, and a
+// shared table of 256 entries made every read a three-fold bank conflict on average, which bound the
+// kernel; with a column per lane the bank only depends on the lane.  An 8-byte read is served in half-warps, so 16
+// columns do: a row is 128 bytes, every 256 (the offset of an entry is then one byte permute).  A half-warp writes a row,
+// and the second level of a lane's rows is the same for all of them.  One B200, columns for 32 lanes and two shuffles a row before:
+// bf16 2^18 2.57 -> 1.94 us, 2^22 3.94 -> 3.02, 2^24 9.72 -> 8.25, from 2^26 on within the spread; seven tensors of 2^20 6.9 -> 5.5.
+__device__ __forceinline__ uint32_t pair_column() { return (threadIdx.x & 15u) * 8u; }
 __device__ __forceinline__ void build_pair_table(float level, unsigned char* s_tab)
 {
-    const int lane = threadIdx.x & 31;
-    for (int b = threadIdx.x >> 5; b < 256; b += kDThreads / 32)
-        *reinterpret_cast<float2*>(s_tab + (b * 32 + lane) * 8) =
-            make_float2(__shfl_sync(kFull, level, b >> 4), __shfl_sync(kFull, level, b & 15));
+    constexpr int kRows = 2 * kDThreads / 32;  // rows that the CTA writes at a time
+    static_assert(kRows % 16 == 0 && 256 % kRows == 0, "a lane's rows have the same low half");
+    const int row = threadIdx.x >> 4;
+    const float low = __shfl_sync(kFull, level, row & 15);
+#pragma unroll
+    for (int b = 0; b < 256; b += kRows)
+        *reinterpret_cast<float2*>(s_tab + (b + row) * kDTableRow + pair_column()) = make_float2(__shfl_sync(kFull, level, (b + row) >> 4), low);
     __syncthreads();
 }
 
@@ -522,7 +529,7 @@ __device__ __forceinline__ void dequantize_tail(const uint8_t* __restrict__ code
     const float m = load_scale<ST>(scales, scale_index);
     for (int i = threadIdx.x; i < len; i += kDThreads) {
         const int64_t k = first + i;
-        const float2 lv = *reinterpret_cast<const float2*>(s_tab + (size_t)codes[k >> 1] * 256 + (threadIdx.x & 31u) * 8u);
+        const float2 lv = *reinterpret_cast<const float2*>(s_tab + (size_t)codes[k >> 1] * kDTableRow + pair_column());
         const float v = __fmul_rn(m, (k & 1) ? lv.y : lv.x);
         if (OT::code == BF16::code)
             static_cast<uint16_t*>(out)[k] = (uint16_t)bf16_rne(v);
@@ -536,11 +543,10 @@ struct DequantRow {
     uint4 cc;
     float m;
 };
-// n: whole blocks, a multiple of 32, so a lane's 32 outputs are all inside the tensor or all outside
+// idx: the lane's first weight; n: whole blocks, a multiple of 32, so its 32 outputs are all inside the tensor or all outside
 template <class ST, int I>
-__device__ __forceinline__ DequantRow dequant_load(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t n, int64_t row)
+__device__ __forceinline__ DequantRow dequant_load(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t n, int64_t idx)
 {
-    const int64_t idx = (row * kDThreads + threadIdx.x) * kDLaneW;
     DequantRow d{make_uint4(0u, 0u, 0u, 0u), 0.0f};
     if (idx < n) {
         asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -550,6 +556,7 @@ __device__ __forceinline__ DequantRow dequant_load(const uint8_t* __restrict__ c
     }
     return d;
 }
+__device__ __forceinline__ int64_t dequant_index(int row) { return ((int64_t)row * kDThreads + threadIdx.x) * kDLaneW; }
 
 // The rows r0, r0 + G, ... of one tensor; `first` is row r0 already on its way.
 template <class ST, class OT, int I>
@@ -563,10 +570,11 @@ __device__ __forceinline__ void dequantize_rows(const uint8_t* __restrict__ code
     int r = r0;
     if (tail && rows >= r0 && (rows - r0) % G == 0) dequantize_tail<ST, OT>(codes, scales, n, tail, n / I, s_tab, out);
     if (r >= rows) return;
-    const uint32_t lane8 = (threadIdx.x & 31u) * 8u;
+    const uint32_t lane8 = pair_column();
+    int64_t idx = dequant_index(r);
     for (; r < rows; r += G) {
-        const int64_t idx = ((int64_t)r * kDThreads + threadIdx.x) * kDLaneW;
-        const DequantRow next = dequant_load<ST, I>(codes, scales, n, (int64_t)r + G);
+        const int64_t idx_next = idx + (int64_t)G * kDRow;
+        const DequantRow next = dequant_load<ST, I>(codes, scales, n, idx_next);
         if (idx < n) {
             const float2 mm = make_float2(first.m, first.m);
             const uint32_t word[4] = {first.cc.x, first.cc.y, first.cc.z, first.cc.w};
@@ -575,7 +583,7 @@ __device__ __forceinline__ void dequantize_rows(const uint8_t* __restrict__ code
                 float2 o[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    // byte offset of this lane's entry of the code byte: byte * 256 + lane * 8, one permute
+                    // byte offset of this lane's entry of the code byte: byte * kDTableRow + its column, one permute
                     const uint32_t off = __byte_perm(word[2 * h + (k >> 2)], lane8, 0x5504u | ((uint32_t)(k & 3) << 4));
                     o[k] = __fmul2_rn(mm, *reinterpret_cast<const float2*>(s_tab + off));
                 }
@@ -599,6 +607,7 @@ __device__ __forceinline__ void dequantize_rows(const uint8_t* __restrict__ code
             }
         }
         first = next;
+        idx = idx_next;
     }
 }
 
@@ -610,7 +619,7 @@ dequantize_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ sc
     if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_tab[];
     const float level = lane_level(levels);
-    const DequantRow first = dequant_load<ST, I>(codes, scales, n & ~(int64_t)(I - 1), (int64_t)blockIdx.x);  // on its way meanwhile
+    const DequantRow first = dequant_load<ST, I>(codes, scales, n & ~(int64_t)(I - 1), dequant_index((int)blockIdx.x));  // on its way meanwhile
     build_pair_table(level, s_tab);
     dequantize_rows<ST, OT, I>(codes, scales, n, out, s_tab, (int)blockIdx.x, first);
 }
@@ -632,7 +641,7 @@ dequantize_batch_kernel(const __grid_constant__ DequantBatch B, const float* __r
 {
     if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_tab[];
-    auto fetch = [&](int t) { return dequant_load<ST, I>(B.codes[t], B.scales[t], B.n[t] & ~(int64_t)(I - 1), first_row_of(B.start[t])); };
+    auto fetch = [&](int t) { return dequant_load<ST, I>(B.codes[t], B.scales[t], B.n[t] & ~(int64_t)(I - 1), dequant_index(first_row_of(B.start[t]))); };
     const float level = lane_level(levels);
     int t = next_tensor(B, -1);
     if (t >= B.count) return;
