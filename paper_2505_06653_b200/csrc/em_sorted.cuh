@@ -56,19 +56,19 @@ struct SortWs {
 // Whether a fit of `iters` iterations over n weights is faster with its samples in order than streamed: the ordering is
 // paid once, an iteration is cheaper by what it streams.  Both sides by measurement, in us with k = n / 2^20 (blocks of 64;
 // other block sizes differ by a few per cent):
-//   ordering  one sample per weight 81 (k = 1), 185 (4), 370 (8), 755 (16), 1580 (32), 4230 (64: beyond the L2's reach);
-//             distinct bf16 weights 102 (2), 107 (4), 135 (16), 190 (64), 400 (256), 1140 (1024)
+//   ordering, less what a streamed fit takes before its first iteration
+//             one sample per weight, fp32: 66 (k = 1), 94 (2), 162 (4), 267 (8), 534 (16), 778 (24), 1026 (32), 1514 (48), 2001 (64)
+//             distinct bf16 weights 75 to 83 (2), 90 (4), 93 to 113 (16), 143 to 175 (64), 192 to 413 (256)
 //   streamed iteration less an ordered one
-//             fp32: MSE 15 (1), 19 (4), 26 (8), 34 (16), 64 (32), 112 (64), medians 46, 52, 63, 73, 108, 148
-//             bf16: MSE 17 (1), 18 (4), 34 (16), 73 (64), 970 (1024), medians 50, 52, 76, 173, 2000
-// The lines below are fits to these.  Where they cross, in iterations: fp32 MSE 6 at 2^20, 11 at 2^22, 22 at 2^24, 37 at 2^26,
-// medians 4, 4, 11, 29; bf16 MSE 6 from 3 * 2^19 to 2^22, 4 from 2^24 on, medians 4.  With four iterations for all,
-// fits of 4 and 8 over 2^24 fp32 weights took 787 and 796 us (MSE) against 160 and 307 streamed.
-// Samples that are staged (em_sorted.cu) and cells are ordered faster since: 88, 185, 316, 601, 1120 and 2215 us for k = 1, 4, ... 64
-// fp32, some 7 % less for cells.  The lines have stayed where they were, so fp32 fits of 2^24 and more are streamed up to twice as many
-// iterations as would pay (2^26 MSE: 20).
-// Fewer than four iterations are not ordered, although two or three would pay for bf16 data from 2^26 weights on (2^28, three: 1120
-// us streamed, about 400 ordered): such a fit gets by with the small workspace.
+//             fp32: MSE 15 (1), 15 (2), 19 (4), 24 (8), 33 (16), 50 (24), 61 (32), 83 (48), 105 (64),
+//             medians 43, 45, 51, 63, 69, 91, 101, 125, 141
+//             bf16: MSE 15 (1), 15 (2), 16 (4), 31 (16), 82 (64), 259 (256), medians 48, 51, 51, 78, 179, 569
+// The lines below are fits to these, the one for medians of fp32 data between 2^22 and 2^23 weights an iteration or two on the
+// streamed side (2^23: 7, by the figures 5).  Where they cross, in iterations, and by the figures: fp32 MSE 6 (5) at
+// 2^20, 10 (9) at 2^22, 16 (16) at 2^24, 18 (17) at 2^25, 20 (19) at 2^26, medians 4 (4), 4 (4), 9 (8), 11 (11), 15 (15);
+// bf16 MSE 6 from 3 * 2^19 to 2^22, 4 from 2^24 on, medians 4.
+// Fewer than four iterations are not ordered, although two or three would pay for bf16 data from 2^26 weights on (2^28, three: 1000
+// us streamed, about 410 ordered): such a fit gets by with the small workspace.
 inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool cells)
 {
     if (iters < kSortMinIters || n < 1) return false;
@@ -76,8 +76,8 @@ inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool ce
     const bool mae = metric == BOF4_METRIC_MAE || metric == BOF4_METRIC_MAE_NORMALIZED;
     double order = 105.0 + 1.1 * k, gain = mae ? 50.0 + 1.9 * k : 16.5 + 0.9 * k;
     if (!cells) {
-        order = fmax(fmax(46.0 + 35.0 * k, 48.0 * k), 82.0 * k - 1000.0);
-        gain = mae ? fmin(43.0 + 1.85 * k, 85.0 + k) : (w_dtype == BOF4_BF16 ? 18.0 : 13.0) + 1.3 * k + 0.005 * k * k;
+        order = fmin(46.0 + 35.0 * k, 50.0 + 31.0 * k);
+        gain = mae ? fmin(fmax(46.0, 31.0 + 2.3 * k), 55.0 + 1.35 * k) : (w_dtype == BOF4_BF16 ? 18.0 : 13.0) + 1.42 * k;
     }
     return iters * gain >= order;
 }
