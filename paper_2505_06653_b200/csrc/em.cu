@@ -595,7 +595,7 @@ em_mse32_kernel(const EmTensors T, const float* levels, double* partials, const 
         *reinterpret_cast<float2*>(s_acc + l * G::acc_row_bytes + tid * 8) = make_float2(0.0f, 0.0f);
         if (COUNT) *reinterpret_cast<uint16_t*>(s_cnt + l * (G::acc_row_bytes / 4) + tid * 2) = 0;
     }
-    const bool lut_ok = build_tables32<G::lut_rep>(lane_level(levels), s_xi, s_lv, s_lut, &s_info,
+    const bool lut_ok = build_tables32<G::lut_rep, G::threads / 32>(lane_level(levels), s_xi, s_lv, s_lut, &s_info,
                                                    [](int base) { return (uint32_t)base * G::acc_row_bytes; });
     const bool fast_ok = lut_ok && !s_info.tiny;
 
