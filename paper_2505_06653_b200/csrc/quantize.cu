@@ -18,8 +18,9 @@ namespace bof4 {
 constexpr int kQThreads = 512;              // quantise / OPQ pass 1
 constexpr int kQRow = kQThreads * kLaneW;   // weights per CTA row
 constexpr int kQCtasPerSm = 2;              // two CTAs, each with its own region table
-// The batch kernels keep the table once per lane: 28 tensors of 872 million bf16 weights 357 us against 383.
-constexpr int kQBatchRep = 32;
+// Columns of the bf16 quantiser's and the batch kernels' region table: one per lane.  28 tensors of 872 million bf16 weights 357 us against
+// 383 with 16, one of 2^28 in blocks of 2048 148 against 165; below 2^24 weights as fast as with 16.
+constexpr int kQTableRep = 32;
 constexpr int kDThreads = 512;              // dequantise
 constexpr int kDCtasPerSm = 3;              // each with its own 64 KiB level-pair table
 constexpr int kDTableRow = 256;              // 16 columns of 8 bytes, and as many bytes that are not used
@@ -229,6 +230,9 @@ __device__ __forceinline__ int next_tensor(const Batch& B, int t)
     return t;
 }
 
+// In the place of a request for the row behind a tensor's: there is none.
+struct Nothing {};
+
 // The rows r0, r0 + G, ... of one tensor of n weights (G = CTAs of the grid), its short last block included; `first` is
 // row r0 already on its way.  behind() requests the row that the CTA takes after these; it is left in `first`.
 template <class DT, int I, bool SIGNED, class ST, int REP, class Behind>
@@ -285,11 +289,11 @@ quantize_batch_kernel(const __grid_constant__ QuantBatch B, const float* __restr
     const float level = lane_level(levels);
     int t = next_tensor(B, -1);
     RawRow<DT> first = fetch(t);
-    const QuantTables T = setup_tables<kQBatchRep>(level, s_xi, s_lut);
+    const QuantTables T = setup_tables<kQTableRep>(level, s_xi, s_lut);
     while (t < B.count) {
         const int then = next_tensor(B, t);
-        quantize_rows<DT, I, SIGNED, ST, kQBatchRep>(B.w[t], B.n[t], B.codes[t], B.scales[t], first_row_of(B.start[t]), first, T,
-                                                     lut_lane_base<kQBatchRep>(s_lut, threadIdx.x & 31), &s_wide, [&] { return fetch(then); });
+        quantize_rows<DT, I, SIGNED, ST, kQTableRep>(B.w[t], B.n[t], B.codes[t], B.scales[t], first_row_of(B.start[t]), first, T,
+                                                     lut_lane_base<kQTableRep>(s_lut, threadIdx.x & 31), &s_wide, [&] { return fetch(then); });
         t = then;
     }
 }
@@ -345,21 +349,27 @@ __device__ __noinline__ void quantize_row32_generic(Raw32 raw, int64_t idx, bool
 
 // The rows r, r + G, r + 2G, ... of one tensor (G = CTAs of the grid), `first` being row r already
 // on its way.  behind() requests the row that the CTA takes after these; it is left in `first`.  Called by all threads of
-// the CTA with the tables in place.
+// the CTA with the tables in place.  (A call on one tensor passes Nothing: with a row of zeros requested there, the loop kept more
+// of its values in local memory, 80 / 100 bytes of stores / loads and not 56 / 8, and absolute normalisation took 66 us for 2^27 weights, not 61.)
 template <int I, bool SIGNED, class ST, int REP, class Behind>
 __device__ __forceinline__ void quantize32_rows(const void* __restrict__ w, int64_t n, uint8_t* __restrict__ codes,
                                                 void* __restrict__ scales, const int r0, Raw32& first,
                                                 const bool fast_ok, const uint32_t lut_base, QuantShared32* S, Behind behind)
 {
+    constexpr bool kMore = !std::is_same_v<Behind, Nothing>;
     const RowMap32 map(n, kQRow32, threadIdx.x);
     const int G = gridDim.x;
     int r = r0;
     auto fetch = [&](int rr) { return map.ok(rr) ? load_raw32(w, map.idx(rr)) : zero_raw32(); };
     if constexpr (Geo32<I>::WPB > 1) {
         // blocks of several warps: every thread of the CTA takes every step (barriers inside)
-        if (r >= map.rows) first = behind();
+        if constexpr (kMore) {
+            if (r >= map.rows) first = behind();
+        }
         for (; r < map.rows; r += G) {
-            const Raw32 next = r + G < map.rows ? fetch(r + G) : behind();
+            Raw32 next;
+            if constexpr (kMore) next = r + G < map.rows ? fetch(r + G) : behind();
+            else next = fetch(r + G);
             uint32_t u[16];
             words_of(first, u);
             float mx, mn;
@@ -396,24 +406,24 @@ __device__ __forceinline__ void quantize32_rows(const void* __restrict__ w, int6
             Raw32 a = first, b = first;
             while (true) {
                 int rn = r + G;
-                if (rn < full) b = load_raw32(w, map.idx(rn)); else b = behind();
+                if (rn < full) b = load_raw32(w, map.idx(rn)); else if constexpr (kMore) b = behind();
                 row(a, r);
                 if (rn >= full) break;
                 r = rn;
                 rn = r + G;
-                if (rn < full) a = load_raw32(w, map.idx(rn)); else a = behind();
+                if (rn < full) a = load_raw32(w, map.idx(rn)); else if constexpr (kMore) a = behind();
                 row(b, r);
                 if (rn >= full) {
-                    b = a;
+                    if constexpr (kMore) b = a;
                     break;
                 }
                 r = rn;
             }
             if (partial) last(fetch(full));
-            first = b;
+            if constexpr (kMore) first = b;
         } else {
             if (partial) last(first);
-            first = behind();
+            if constexpr (kMore) first = behind();
         }
     }
 }
@@ -431,11 +441,11 @@ quantize32_kernel(const void* __restrict__ w, int64_t n, const float* __restrict
     const int r = blockIdx.x;
     const float level = lane_level(levels);
     Raw32 first = map.ok(r) ? load_raw32(w, map.idx(r)) : zero_raw32();  // on its way while the tables are built
-    const bool lut_ok = build_tables32<kQLutRep>(level, S.xi, S.lv, s_lut, &S.info, [](int base) { return (uint32_t)base; });
+    const bool lut_ok = build_tables32<kQTableRep>(level, S.xi, S.lv, s_lut, &S.info, [](int base) { return (uint32_t)base; });
     const bool fast_ok = lut_ok && !S.info.tiny;
-    const uint32_t lut_base = lut_lane_base<kQLutRep>(s_lut, threadIdx.x & 31);
+    const uint32_t lut_base = lut_lane_base<kQTableRep>(s_lut, threadIdx.x & 31);
     if (r < map.rows)
-        quantize32_rows<I, SIGNED, ST, kQLutRep>(w, n - tail, codes, scales, r, first, fast_ok, lut_base, &S, [] { return zero_raw32(); });
+        quantize32_rows<I, SIGNED, ST, kQTableRep>(w, n - tail, codes, scales, r, first, fast_ok, lut_base, &S, Nothing{});
     if (tail && r <= map.rows && (map.rows - r) % (int)gridDim.x == 0)
         quantize_tail<BF16, SIGNED, ST>(w, n - tail, tail, S.xi, codes, scales, n / I);
 }
@@ -456,9 +466,9 @@ quantize32_batch_kernel(const __grid_constant__ QuantBatch B, const float* __res
     };
     const float level = lane_level(levels);
     Raw32 first = fetch(0);
-    const bool lut_ok = build_tables32<kQBatchRep>(level, S.xi, S.lv, s_lut, &S.info, [](int base) { return (uint32_t)base; });
+    const bool lut_ok = build_tables32<kQTableRep>(level, S.xi, S.lv, s_lut, &S.info, [](int base) { return (uint32_t)base; });
     const bool fast_ok = lut_ok && !S.info.tiny;
-    const uint32_t lut_base = lut_lane_base<kQBatchRep>(s_lut, threadIdx.x & 31);
+    const uint32_t lut_base = lut_lane_base<kQTableRep>(s_lut, threadIdx.x & 31);
     for (int t = 0; t < B.count; ++t) {
         // (Going from one tensor with a row of this CTA to the next, as the fp32 kernel does, takes the 28 tensors 365 us, not
         // 357: a register more in the loop over rows.)
@@ -471,7 +481,7 @@ quantize32_batch_kernel(const __grid_constant__ QuantBatch B, const float* __res
         const int rows = (int)((n + kQRow32 - 1) / kQRow32), r0 = first_row_of(B.start[t]);
         // The next tensor's first row is requested with this one's last: a row's latency for every tensor otherwise (28 tensors
         // of 872 million weights 382 us against 356, 14 of 77 million 52 against 46).
-        quantize32_rows<I, SIGNED, ST, kQBatchRep>(B.w[t], n, B.codes[t], B.scales[t], r0, first, fast_ok, lut_base, &S, [&] { return fetch(t + 1); });
+        quantize32_rows<I, SIGNED, ST, kQTableRep>(B.w[t], n, B.codes[t], B.scales[t], r0, first, fast_ok, lut_base, &S, [&] { return fetch(t + 1); });
         if (tail && r0 <= rows && (rows - r0) % G == 0)
             quantize_tail<BF16, SIGNED, ST>(B.w[t], n, tail, S.xi, B.codes[t], B.scales[t], n / I);
     }
@@ -1526,8 +1536,8 @@ extern "C" int bof4_quantize(const void* d_w, int w_dtype, int64_t n, int block_
             BOF4_DISPATCH_I(block_size,
                 BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                     { constexpr auto kern = quantize32_kernel<I_, SG, ST>;
-                      if ((rc = ensure_dynamic_smem<kern>(kQLutBytes))) return rc;
-                      launch_after(kern, grid, kQThreads, kQLutBytes, st, d_w, n, d_codebook, d_codes, d_scales); })));
+                      if ((rc = ensure_dynamic_smem<kern>(lut_bytes(kQTableRep)))) return rc;
+                      launch_after(kern, grid, kQThreads, lut_bytes(kQTableRep), st, d_w, n, d_codebook, d_codes, d_scales); })));
     } else {
         const int grid = grid_for((n_whole + kQRow - 1) / kQRow + more, kQCtasPerSm);
         BOF4_DISPATCH_I(block_size,
@@ -1649,14 +1659,14 @@ extern "C" int bof4_quantize_batch(const void* const* h_w, const int64_t* h_n, i
                     BOF4_DISPATCH_I(block_size,
                         BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                             { constexpr auto kern = quantize32_batch_kernel<I_, SG, ST>;
-                              if ((rc = ensure_dynamic_smem<kern>(lut_bytes(kQBatchRep)))) return rc;
-                              launch_after(kern, grid, kQThreads, lut_bytes(kQBatchRep), st, B, d_codebook); })));
+                              if ((rc = ensure_dynamic_smem<kern>(lut_bytes(kQTableRep)))) return rc;
+                              launch_after(kern, grid, kQThreads, lut_bytes(kQTableRep), st, B, d_codebook); })));
             } else {
                 BOF4_DISPATCH_I(block_size,
                     BOF4_DISPATCH_BOOL(norm == BOF4_NORM_SIGNED, SG,
                         { constexpr auto kern = quantize_batch_kernel<F32, I_, SG, F32>;
-                          if ((rc = ensure_dynamic_smem<kern>(lut_bytes(kQBatchRep)))) return rc;
-                          launch_after(kern, grid, kQThreads, lut_bytes(kQBatchRep), st, B, d_codebook); }));
+                          if ((rc = ensure_dynamic_smem<kern>(lut_bytes(kQTableRep)))) return rc;
+                          launch_after(kern, grid, kQThreads, lut_bytes(kQTableRep), st, B, d_codebook); }));
             }
             BOF4_CUDA_TRY(cudaGetLastError());
             B.count = 0;
