@@ -63,10 +63,11 @@ struct SortWs {
 //             fp32: MSE 15 (1), 15 (2), 19 (4), 24 (8), 33 (16), 50 (24), 61 (32), 83 (48), 105 (64),
 //             medians 43, 45, 51, 63, 69, 91, 101, 125, 141
 //             bf16: MSE 15 (1), 15 (2), 16 (4), 31 (16), 82 (64), 259 (256), medians 48, 51, 51, 78, 179, 569
-// The lines below are fits to these, the one for medians of fp32 data between 2^22 and 2^23 weights an iteration or two on the
-// streamed side (2^23: 7, by the figures 5).  Where they cross, in iterations, and by the figures: fp32 MSE 6 (5) at
-// 2^20, 10 (9) at 2^22, 16 (16) at 2^24, 18 (17) at 2^25, 20 (19) at 2^26, medians 4 (4), 4 (4), 9 (8), 11 (11), 15 (15);
-// bf16 MSE 6 from 3 * 2^19 to 2^22, 4 from 2^24 on, medians 4.
+// The lines below are fits to these, a little on the streamed side, which takes 9 MB of workspace where ordering takes 16 bytes a weight;
+// from 2^25 weights on (more than half a gigabyte) ordering has to save more than it costs: fits of 2^26 weights and up to 32 iterations
+// (medians 23) get by with the small workspace, as callers are promised.  Where they cross, in iterations, and by the figures: fp32
+// MSE 6 (5) at 2^20, 10 (9) at 2^22, 13 (12) at 2^23, 17 (16) at 2^24, 20 (17) at 2^25, 33 (19) at 2^26, medians 4, 4, 7 (5), 9 (8), 12 (11),
+// 24 (15); bf16 MSE 6 from 3 * 2^19 to 2^22, 4 from 2^24 on, medians 4.
 // Fewer than four iterations are not ordered, although two or three would pay for bf16 data from 2^26 weights on (2^28, three: 1000
 // us streamed, about 410 ordered): such a fit gets by with the small workspace.
 inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool cells)
@@ -76,8 +77,8 @@ inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool ce
     const bool mae = metric == BOF4_METRIC_MAE || metric == BOF4_METRIC_MAE_NORMALIZED;
     double order = 105.0 + 1.1 * k, gain = mae ? 50.0 + 1.9 * k : 16.5 + 0.9 * k;
     if (!cells) {
-        order = fmin(46.0 + 35.0 * k, 50.0 + 31.0 * k);
-        gain = mae ? fmin(fmax(46.0, 31.0 + 2.3 * k), 55.0 + 1.35 * k) : (w_dtype == BOF4_BF16 ? 18.0 : 13.0) + 1.42 * k;
+        order = fmax(fmin(46.0 + 35.0 * k, 50.0 + 33.0 * k), 70.0 * k - 1120.0);
+        gain = mae ? fmin(fmax(47.5, 31.0 + 2.3 * k), 55.0 + 1.35 * k) : (w_dtype == BOF4_BF16 ? 18.0 : 13.0) + 1.42 * k;
     }
     return iters * gain >= order;
 }

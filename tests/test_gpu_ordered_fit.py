@@ -87,8 +87,8 @@ def test_many_tensors_long(bof4):
 
 @pytest.mark.parametrize("dtype,n,metric,iters", [(torch.float32, 1 << 20, 0, (5, 6)), (torch.float32, 1 << 21, 0, (7, 8)),
                                                   (torch.float32, 1 << 23, 1, (6, 7)), (torch.bfloat16, 1 << 21, 0, (5, 6)),
-                                                  (torch.float32, 1 << 23, 0, (12, 13)), (torch.float32, 1 << 24, 0, (15, 16)),
-                                                  (torch.float32, 1 << 24, 1, (8, 9)), (torch.float32, 1 << 26, 0, (19, 20))])
+                                                  (torch.float32, 1 << 23, 0, (12, 13)), (torch.float32, 1 << 24, 0, (16, 17)),
+                                                  (torch.float32, 1 << 24, 1, (8, 9)), (torch.float32, 1 << 25, 0, (19, 20))])
 def test_both_sides_of_the_switch_over(bof4, dtype, n, metric, iters):
     """One iteration apart, one fit is streamed and the other ordered; the same oracle."""
     from paper_2505_06653_b200 import binding as b
