@@ -360,7 +360,9 @@ cells_order_few_kernel(const EmTensors T, const int64_t first_block, const int64
 // model, 113 this way (fits of 2^28 and 2^30 weights 10 and 60 us faster).  Bound by the counters, whose lanes collide on common
 // magnitudes, and the chain of a tile: the reservation in global memory, five barriers.  (A lane counting for all of its
 // magnitude in the warp, by __match_any_sync: 248 us.)
-// Fewer blocks in a launch are written directly: 2^16 (2^22 weights) 283 us a fit against 286 in tiles, 2^20 348 against 345.
+// Fewer blocks in a launch are written directly.  Fits of 8 iterations, directly and in tiles: 2^16 blocks (2^22 weights) 132.7 us and
+// 136.6, 3 * 2^17 156 and 163, 2^19 173.3 and 173.7, 2^20 207 and 205.5, 2^22 417 and 404.  (Constants spread over six binades in every
+// tensor: 2^19 the same, 2^20 210 and 216, 2^21 295 and 299, 2^22 445 and 445.)
 constexpr int64_t kOrderFew = 1 << 19;
 constexpr int kOrderTile = 1024 * kOrderGroup;
 static_assert(kOrderTile == 1 << 13, "13 bits for a place in a tile");
