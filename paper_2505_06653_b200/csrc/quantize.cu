@@ -23,6 +23,7 @@ constexpr int kQCtasPerSm = 2;              // two CTAs, each with its own regio
 constexpr int kQTableRep = 32;
 constexpr int kDThreads = 512;              // dequantise
 constexpr int kDCtasPerSm = 3;              // each with its own 64 KiB level-pair table
+constexpr int64_t kDNarrowBelow = 1 << 27;
 constexpr int kDTableRow = 256;              // 16 columns of 8 bytes, and as many bytes that are not used
 constexpr int kDTableBytes = 256 * kDTableRow;  // [code byte][lane & 15] pairs of levels
 constexpr int kDLaneW = 32;                 // outputs per lane and row (16 code bytes in)
@@ -525,22 +526,36 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 // shared table of 256 entries made every read a three-fold bank conflict on average, which bound the
 // kernel; with a column per lane the bank only depends on the lane.  An 8-byte read is served in half-warps, so 16
 // columns do: a row is 128 bytes, every 256 (the offset of an entry is then one byte permute).  A half-warp writes a row,
-// and the second level of a lane's rows is the same for all of them.  One B200, columns for 32 lanes and two shuffles a row before:
-// bf16 2^18 2.57 -> 1.94 us, 2^22 3.94 -> 3.02, 2^24 9.72 -> 8.25, from 2^26 on within the spread; seven tensors of 2^20 6.9 -> 5.5.
-__device__ __forceinline__ uint32_t pair_column() { return (threadIdx.x & 15u) * 8u; }
+// and the second level of a lane's rows is the same for all of them.  One B200, 32 columns and 16: bf16 2^18 2.57 and 1.95 us, 2^22
+// 3.93 and 3.06, 2^24 9.6 and 8.3, 2^26 30.9 and 30.1, 2^27 59.7 and 59.2; seven tensors of 2^20 6.6 and 5.6.  From kDNarrowBelow weights on
+// the set-up is lost in the spread, and 32 columns are the faster: 28672 x 8192 with outliers, a new output each call, 109.5 and 112.4.
+template <int COLS>
+__device__ __forceinline__ uint32_t pair_column()
+{
+    return (threadIdx.x & (COLS - 1u)) * 8u;
+}
+template <int COLS>
 __device__ __forceinline__ void build_pair_table(float level, unsigned char* s_tab)
 {
+    if constexpr (COLS == 32) {
+        const int lane = threadIdx.x & 31;
+        for (int b = threadIdx.x >> 5; b < 256; b += kDThreads / 32)
+            *reinterpret_cast<float2*>(s_tab + (b * 32 + lane) * 8) =
+                make_float2(__shfl_sync(kFull, level, b >> 4), __shfl_sync(kFull, level, b & 15));
+        __syncthreads();
+        return;
+    }
     constexpr int kRows = 2 * kDThreads / 32;  // rows that the CTA writes at a time
     static_assert(kRows % 16 == 0 && 256 % kRows == 0, "a lane's rows have the same low half");
     const int row = threadIdx.x >> 4;
     const float low = __shfl_sync(kFull, level, row & 15);
 #pragma unroll
     for (int b = 0; b < 256; b += kRows)
-        *reinterpret_cast<float2*>(s_tab + (b + row) * kDTableRow + pair_column()) = make_float2(__shfl_sync(kFull, level, (b + row) >> 4), low);
+        *reinterpret_cast<float2*>(s_tab + (b + row) * kDTableRow + pair_column<COLS>()) = make_float2(__shfl_sync(kFull, level, (b + row) >> 4), low);
     __syncthreads();
 }
 
-template <class ST, class OT>
+template <class ST, class OT, int COLS>
 __device__ __forceinline__ void dequantize_tail(const uint8_t* __restrict__ codes, const void* __restrict__ scales,
                                                 int64_t first, int len, int64_t scale_index, const unsigned char* s_tab,
                                                 void* __restrict__ out)
@@ -548,7 +563,7 @@ __device__ __forceinline__ void dequantize_tail(const uint8_t* __restrict__ code
     const float m = load_scale<ST>(scales, scale_index);
     for (int i = threadIdx.x; i < len; i += kDThreads) {
         const int64_t k = first + i;
-        const float2 lv = *reinterpret_cast<const float2*>(s_tab + (size_t)codes[k >> 1] * kDTableRow + pair_column());
+        const float2 lv = *reinterpret_cast<const float2*>(s_tab + (size_t)codes[k >> 1] * kDTableRow + pair_column<COLS>());
         const float v = __fmul_rn(m, (k & 1) ? lv.y : lv.x);
         if (OT::code == BF16::code)
             static_cast<uint16_t*>(out)[k] = (uint16_t)bf16_rne(v);
@@ -562,10 +577,12 @@ struct DequantRow {
     uint4 cc;
     float m;
 };
-// idx: the lane's first weight; n: whole blocks, a multiple of 32, so its 32 outputs are all inside the tensor or all outside
+__device__ __forceinline__ int64_t dequant_index(int64_t row) { return (row * kDThreads + threadIdx.x) * kDLaneW; }
+// n: whole blocks, a multiple of 32, so a lane's 32 outputs are all inside the tensor or all outside
 template <class ST, int I>
-__device__ __forceinline__ DequantRow dequant_load(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t n, int64_t idx)
+__device__ __forceinline__ DequantRow dequant_load(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t n, int64_t row)
 {
+    const int64_t idx = dequant_index(row);
     DequantRow d{make_uint4(0u, 0u, 0u, 0u), 0.0f};
     if (idx < n) {
         asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -575,10 +592,9 @@ __device__ __forceinline__ DequantRow dequant_load(const uint8_t* __restrict__ c
     }
     return d;
 }
-__device__ __forceinline__ int64_t dequant_index(int row) { return ((int64_t)row * kDThreads + threadIdx.x) * kDLaneW; }
 
 // The rows r0, r0 + G, ... of one tensor; `first` is row r0 already on its way.
-template <class ST, class OT, int I>
+template <class ST, class OT, int I, int COLS>
 __device__ __forceinline__ void dequantize_rows(const uint8_t* __restrict__ codes, const void* __restrict__ scales,
                                                 int64_t n, void* __restrict__ out, const unsigned char* s_tab, const int r0,
                                                 DequantRow first)
@@ -587,13 +603,12 @@ __device__ __forceinline__ void dequantize_rows(const uint8_t* __restrict__ code
     n -= tail;
     const int rows = (int)((n + kDRow - 1) / kDRow), G = gridDim.x;
     int r = r0;
-    if (tail && rows >= r0 && (rows - r0) % G == 0) dequantize_tail<ST, OT>(codes, scales, n, tail, n / I, s_tab, out);
+    if (tail && rows >= r0 && (rows - r0) % G == 0) dequantize_tail<ST, OT, COLS>(codes, scales, n, tail, n / I, s_tab, out);
     if (r >= rows) return;
-    const uint32_t lane8 = pair_column();
-    int64_t idx = dequant_index(r);
+    const uint32_t lane8 = pair_column<COLS>();
     for (; r < rows; r += G) {
-        const int64_t idx_next = idx + (int64_t)G * kDRow;
-        const DequantRow next = dequant_load<ST, I>(codes, scales, n, idx_next);
+        const int64_t idx = dequant_index(r);
+        const DequantRow next = dequant_load<ST, I>(codes, scales, n, (int64_t)r + G);
         if (idx < n) {
             const float2 mm = make_float2(first.m, first.m);
             const uint32_t word[4] = {first.cc.x, first.cc.y, first.cc.z, first.cc.w};
@@ -626,11 +641,10 @@ __device__ __forceinline__ void dequantize_rows(const uint8_t* __restrict__ code
             }
         }
         first = next;
-        idx = idx_next;
     }
 }
 
-template <class ST, class OT, int I>
+template <class ST, class OT, int I, int COLS>
 __global__ void __launch_bounds__(kDThreads, kDCtasPerSm)
 dequantize_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ scales, int64_t n,
                   const float* __restrict__ levels, void* __restrict__ out)
@@ -638,9 +652,9 @@ dequantize_kernel(const uint8_t* __restrict__ codes, const void* __restrict__ sc
     if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_tab[];
     const float level = lane_level(levels);
-    const DequantRow first = dequant_load<ST, I>(codes, scales, n & ~(int64_t)(I - 1), dequant_index((int)blockIdx.x));  // on its way meanwhile
-    build_pair_table(level, s_tab);
-    dequantize_rows<ST, OT, I>(codes, scales, n, out, s_tab, (int)blockIdx.x, first);
+    const DequantRow first = dequant_load<ST, I>(codes, scales, n & ~(int64_t)(I - 1), (int64_t)blockIdx.x);  // on its way meanwhile
+    build_pair_table<COLS>(level, s_tab);
+    dequantize_rows<ST, OT, I, COLS>(codes, scales, n, out, s_tab, (int)blockIdx.x, first);
 }
 
 // Several tensors in one launch, their rows dealt round-robin over the CTAs as in
@@ -660,14 +674,14 @@ dequantize_batch_kernel(const __grid_constant__ DequantBatch B, const float* __r
 {
     if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_tab[];
-    auto fetch = [&](int t) { return dequant_load<ST, I>(B.codes[t], B.scales[t], B.n[t] & ~(int64_t)(I - 1), dequant_index(first_row_of(B.start[t]))); };
+    auto fetch = [&](int t) { return dequant_load<ST, I>(B.codes[t], B.scales[t], B.n[t] & ~(int64_t)(I - 1), first_row_of(B.start[t])); };
     const float level = lane_level(levels);
     int t = next_tensor(B, -1);
     if (t >= B.count) return;
     DequantRow first = fetch(t);
-    build_pair_table(level, s_tab);
+    build_pair_table<16>(level, s_tab);
     while (true) {
-        dequantize_rows<ST, OT, I>(B.codes[t], B.scales[t], B.n[t], B.out[t], s_tab, first_row_of(B.start[t]), first);
+        dequantize_rows<ST, OT, I, 16>(B.codes[t], B.scales[t], B.n[t], B.out[t], s_tab, first_row_of(B.start[t]), first);
         t = next_tensor(B, t);
         if (t >= B.count) break;
         first = fetch(t);
@@ -1594,9 +1608,10 @@ extern "C" int bof4_dequantize(const uint8_t* d_codes, const void* d_scales, int
     const int grid = grid_for(rows, kDCtasPerSm);
 #define BOF4_DEQ(ST_, OT_)                                                                                   \
     BOF4_DISPATCH_I(block_size, {                                                                            \
-        constexpr auto kern = dequantize_kernel<ST_, OT_, I_>;                                               \
-        if ((rc = ensure_dynamic_smem<kern>(kDTableBytes))) return rc;                                       \
-        launch_after(kern, grid, kDThreads, kDTableBytes, st, d_codes, d_scales, n, d_codebook, d_out); })
+        BOF4_DISPATCH_BOOL(n < kDNarrowBelow, NARROW, {                                                      \
+            constexpr auto kern = dequantize_kernel<ST_, OT_, I_, NARROW ? 16 : 32>;                         \
+            if ((rc = ensure_dynamic_smem<kern>(kDTableBytes))) return rc;                                   \
+            launch_after(kern, grid, kDThreads, kDTableBytes, st, d_codes, d_scales, n, d_codebook, d_out); }) })
     if (scale_dtype == BOF4_F32 && out_dtype == BOF4_F32) { BOF4_DEQ(F32, F32) }
     else if (scale_dtype == BOF4_F32) { BOF4_DEQ(F32, BF16) }
     else if (out_dtype == BOF4_F32) { BOF4_DEQ(BF16, F32) }
