@@ -799,105 +799,232 @@ sort_group_kernel(const SortWs W)
 
 // ---------------------------------------------------------------- all iterations, squared error
 //
-// One CTA.  An iteration is a chain of latencies, and what one SM can issue: 32 warps that each find their
-// thresholds' bins, samples and sums take 4000 cycles, most of them issue slots.  So the work is dealt out once:
-// warp 0 turns the levels into 15 cuts (bin, samples, neighbours; a cut per lane), warps 1 to 15 add up the
-// samples of a cut's bin on either side of it, warps 16 to 31 the whole bins of a region: groups from shared
-// memory, the bins beside whole groups as one sum each (pre, suf).  The first samples of all bins are in shared
-// memory as well (16 bits beside the group's first), which leaves one access to L2 in the chain.  Warp 0 divides,
-// compares and goes straight on to the next cuts; the error of an iteration is worked out while the others add up
-// the next.  Iterations of a fit of 2^20 weights, 50 of them: 115 us with
-// a warp per half region, 87 this way; of 2^26 bf16 weights, 100: 230 -> 165; of 2^24 fp32 weights, 30: 172 -> 129.
+// One CTA.  An iteration is a chain of latencies, so it is kept short: warp w adds up what lies below threshold w, the bins in
+// front of its bin as two sums that are at hand (whole groups, bins of its group) and the samples of its bin, and a region is
+// the difference of two such sums.  Behind the one barrier of an iteration every warp works the levels out for itself (a
+// lane each) and goes straight on to its next threshold; the sixteenth warp has no threshold and writes the error meanwhile.
+// The first samples of all bins are in shared memory (16 bits beside the group's first), which leaves one access to L2 in the
+// chain: 1.12 us an iteration (2^20 fp32 and 2^26 bf16 weights; 1.60 with cuts found by one warp, whole groups added up between them and three
+// barriers), 3.5 for 2^24 fp32 weights (3.9).  Of its 2200 cycles the bin takes 130, its first sample 220, the samples 430 or 820, by
+// where in L2 they are, their reduction 230, the barrier and what it waits for 200, the differences 300 and the quotients with
+// the test of the sums 330.  (The next iteration's samples requested ahead, by the last steps of the threshold: 1 to 13 % slower.)
+//
+// Sums of whole groups are kept in two doubles each, so that their difference is as good as adding the region up; the rest
+// (bins and samples beside whole groups, at most a group's weight) is rounded once to a double.  A region that
+// is very light beside its neighbours, or stands beside sums that are not finite, is added up by itself (region_sums).
 //
 // When an iteration leaves every level unchanged the remaining ones would repeat it bit for bit: their entries
 // of the error log are filled in and the loop ends.
-struct SortCut {
-    float p, below, above;      // the threshold and the ones beside it
-    uint32_t from, to;          // samples of its bin (none: a bin of one value, which is in or out as a whole)
-    int end, begin;             // whole bins: the region below ends before `end`, the one above starts at `begin`
-    int low;                    // the bin's samples below p belong to this cut (no cut before it in the same bin)
-};
-constexpr int kMseOff = kSortGroups * 16;            // shared memory: group sums, first samples of the bins,
-constexpr int kMseFirst = kMseOff + kSortBins * 2;   // of the groups
+constexpr int kMseThreads = 32 * kLevels;
+constexpr int kMseLow = (kSortGroups + 1) * 16;      // shared memory: sums of the groups in front, high and low halves,
+constexpr int kMseOff = 2 * kMseLow;                 // first samples of the bins,
+constexpr int kMseFirst = kMseOff + kSortBins * 2 + 16;  // (and the end) of the groups
 constexpr int kMseSmem = kMseFirst + (kSortGroups + 1) * 4;
 
-// CROWDED: a copy of the loop that also knows crowded bins.  Apart, because the calls in it cost the other one registers: 0.3 us
-// an iteration with both in one.  (Two kernels, as for the absolute error, of which the flag picks one: 2 us slower.)
+// The first samples of all bins, into shared memory: 16 bits beside the first of the bin's group (or kFarBin).  Asynchronous.
+__device__ __forceinline__ void copy_starts(const SortWs& W, uint16_t* s_off, uint32_t* s_first)
+{
+    auto copy = [](void* to, const void* from, auto bytes) {
+        constexpr int B = decltype(bytes)::value;
+        const uint32_t a = (uint32_t)__cvta_generic_to_shared(to);
+        if constexpr (B == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(from) : "memory");
+        else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(from) : "memory");
+    };
+    for (int k = threadIdx.x; k < kSortBins / 8; k += blockDim.x) copy(s_off + 8 * k, W.off + 8 * k, std::integral_constant<int, 16>{});
+    for (int k = threadIdx.x; k <= kSortGroups; k += blockDim.x) copy(s_first + k, W.first + k, std::integral_constant<int, 4>{});
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// A sum in two doubles, high + low with |low| at most half a unit of high.
+struct TwoSum {
+    double h, l;
+};
+__device__ __forceinline__ TwoSum two_add(const TwoSum& a, const TwoSum& b)
+{
+    const double s = a.h + b.h, t = s - a.h;
+    const double e = ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l);
+    const double h = s + e;
+    return TwoSum{h, e - (h - s)};
+}
+__device__ __forceinline__ TwoSum two_shfl_up(const TwoSum& a, int off)
+{
+    return TwoSum{__shfl_up_sync(kFull, a.h, off), __shfl_up_sync(kFull, a.l, off)};
+}
+
+// Sums of the samples with p <= x < q, by a warp; the result is the same in all lanes.
+template <bool CELLS, bool CROWDED>
+__device__ __noinline__ double2 region_sums(const SortWs& W, float p, float q)
+{
+    const int lane = threadIdx.x & 31;
+    const float inf = __int_as_float(0x7f800000);
+    const int bp = (p == -inf) ? -1 : sort_bin(p), bq = (q == inf) ? kSortBins : sort_bin(q);
+    const int b0 = bp + 1, b1 = max(bq, b0);  // bins strictly inside, as whole groups with up to 31 single bins on either side
+    const int g0 = (b0 + kSortGroup - 1) / kSortGroup, g1 = b1 / kSortGroup;
+    SortSums t{0.0, 0.0, 0ull};
+    auto whole = [&](const SortSums* v) { t.s += __ldg(&v->s), t.sx += __ldg(&v->sx); };
+    if (b0 + lane < min(b1, g0 * kSortGroup)) whole(W.bin + b0 + lane);
+    for (int g = g0 + lane; g < g1; g += 32) whole(W.group + g);
+    if (g1 >= g0 && g1 * kSortGroup + lane < b1) whole(W.bin + g1 * kSortGroup + lane);
+    auto cut = [&](int b) {
+        if (one_value_bin(b)) {  // in or out as a whole
+            if (lane == 0 && value_of_bin(b) >= p && value_of_bin(b) < q) whole(W.bin + b);
+            return;
+        }
+        const uint32_t from = __ldg(W.start + b), to = __ldg(W.start + b + 1);
+        if (CROWDED && to - from > kSortCrowd) {
+            crowded_sums<false>(W, SampleWeight<false, false>{}, from, to, p, q, t);
+            return;
+        }
+        for (uint32_t i = from + lane; i < to; i += 32) {
+            const float2 it = __ldg(W.b + i);
+            if (!(it.x >= p && it.x < q)) continue;
+            const double m = (double)it.y, s = CELLS ? __ldg(W.cell_s + i) : m * m;
+            t.s += s;
+            t.sx += s * (double)it.x;
+        }
+        __syncwarp();
+    };
+    if (bp >= 0) cut(bp);
+    if (bq < kSortBins && bq != bp) cut(bq);
+    __syncwarp();
+    sums_reduce<false>(t);
+    return make_double2(t.s, t.sx);
+}
+
+// CROWDED: a copy of the loop that also knows crowded bins.  Apart, because the calls in it cost the other one registers.
 template <bool CELLS, bool CROWDED>
 __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
 {
     extern __shared__ __align__(16) unsigned char s_fit[];
-    double2* const s_group = reinterpret_cast<double2*>(s_fit);
+    double2* const s_high = reinterpret_cast<double2*>(s_fit);           // {s, sx} of the groups in front of a group
+    double2* const s_low = reinterpret_cast<double2*>(s_fit + kMseLow);
     uint16_t* const s_off = reinterpret_cast<uint16_t*>(s_fit + kMseOff);
     uint32_t* const s_first = reinterpret_cast<uint32_t*>(s_fit + kMseFirst);
-    __shared__ SortCut s_cut[kLevels - 1];
-    __shared__ double2 s_low[kLevels], s_high[kLevels + 1], s_mid[kLevels];  // s_low[15] and s_high[0] stay zero
-    __shared__ int s_stop;
+    // What lies below threshold k - 1: whole groups (high, low), the rest.  Entry 0: nothing, entry 16: everything.  Two sets, used
+    // in turn.
+    __shared__ double2 s_below[2][3][kLevels + 1];
+    __shared__ float2 s_cut[2][kLevels + 1];  // the threshold, and how many samples lie below it
+    __shared__ float s_level[2][kLevels];
+    __shared__ int s_stop;  // the iteration behind whose barrier all leave
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int k = tid; k < kSortBins / 8; k += 1024) reinterpret_cast<uint4*>(s_off)[k] = reinterpret_cast<const uint4*>(W.off)[k];
-    for (int k = tid; k < kSortGroups; k += 1024) s_group[k] = make_double2(W.group[k].s, W.group[k].sx);
-    for (int k = tid; k <= kSortGroups; k += 1024) s_first[k] = W.first[k];
-    if (tid == 0) {
-        s_stop = 0;
-        s_low[kLevels - 1] = s_high[0] = make_double2(0.0, 0.0);
+    const float inf = __int_as_float(0x7f800000);
+    if (tid == 0) s_stop = 0x7fffffff, s_off[kSortBins] = 0u;
+    copy_starts(W, s_off, s_first);
+    // running sums of the groups, four to a thread
+    {
+        constexpr int PER = kSortGroups / kMseThreads;
+        TwoSum s[PER], x[PER];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const SortSums* g = W.group + tid * PER + k;
+            s[k] = TwoSum{g->s, 0.0}, x[k] = TwoSum{g->sx, 0.0};
+        }
+        static_assert(PER == 4, "a tree of two levels");
+        TwoSum ts = two_add(two_add(s[0], s[1]), two_add(s[2], s[3])), tx = two_add(two_add(x[0], x[1]), two_add(x[2], x[3]));
+        auto scan = [&](TwoSum& as, TwoSum& ax) {  // inclusive, over the warp
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const TwoSum us = two_shfl_up(as, off), ux = two_shfl_up(ax, off);
+                if (lane >= off) as = two_add(us, as), ax = two_add(ux, ax);
+            }
+        };
+        scan(ts, tx);
+        // (the room of the loop's sums serves for the warps' totals)
+        if (lane == 31) s_below[0][0][warp] = make_double2(ts.h, tx.h), s_below[0][1][warp] = make_double2(ts.l, tx.l);
+        __syncthreads();
+        TwoSum ws{0.0, 0.0}, wx = ws;
+        if (lane < warp) {
+            const double2 h = s_below[0][0][lane], l = s_below[0][1][lane];
+            ws = TwoSum{h.x, l.x}, wx = TwoSum{h.y, l.y};
+        }
+        scan(ws, wx);  // lane 31: all warps in front of this one
+        TwoSum rs = two_shfl_up(ts, 1), rx = two_shfl_up(tx, 1);
+        if (lane == 0) rs = rx = TwoSum{0.0, 0.0};
+        rs = two_add(TwoSum{__shfl_sync(kFull, ws.h, 31), __shfl_sync(kFull, ws.l, 31)}, rs);
+        rx = two_add(TwoSum{__shfl_sync(kFull, wx.h, 31), __shfl_sync(kFull, wx.l, 31)}, rx);
+#pragma unroll
+        for (int k = 0; k <= PER; ++k) {
+            if (k == PER && tid < kMseThreads - 1) break;  // behind the last group: everything
+            s_high[tid * PER + k] = make_double2(rs.h, rx.h);
+            s_low[tid * PER + k] = make_double2(rs.l, rx.l);
+            if (k < PER) rs = two_add(rs, s[k]), rx = two_add(rx, x[k]);
+        }
     }
+    // warps 0 to 14: lane k has level warp + k % 2, those on either side of the warp's threshold; the last warp: lane l has level l
+    const bool last = warp == kLevels - 1;
+    const int mine = last ? lane & (kLevels - 1) : warp + (lane & 1);
+    const bool fixed = (F.fixed_mask >> mine) & 1u;
+    float lv = F.codebook[mine];
     double w2 = 0.0;
-    float lv = 0.0f;
-    const bool level = lane < kLevels;
-    if (warp == 0) {
+    if (last) {
         for (int k = lane; k < kSortParts; k += 32) w2 += W.w2[k];
 #pragma unroll
         for (int off = 16; off; off >>= 1) w2 += __shfl_xor_sync(kFull, w2, off);
-        lv = level ? F.codebook[lane] : 0.0f;
     }
+    copies_done();
     __syncthreads();
-    const float inf = __int_as_float(0x7f800000);
-    auto start_of = [&](int b) -> uint32_t {  // first sample of bin b <= kSortBins
-        if (b == kSortBins) return s_first[kSortGroups];
-        const uint32_t o = s_off[b];
-        return o == kFarBin ? __ldg(W.start + b) : s_first[b / kSortGroup] + o;
-    };
-    // the error of the iteration `at`, whose levels and sums lane l has (warp 0)
-    auto error_of = [&](float old, double s0, double s1, int at) -> double {
-        const double o = (double)old;
-        double err = level ? o * (2.0 * s1 - o * s0) : 0.0;
-#pragma unroll
-        for (int off = 8; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
-        err = fmax(w2 - err, 0.0) / (double)F.n_total;
-        if (lane == 0 && F.err_log) F.err_log[at] = err;
-        return err;
-    };
-    float old = 0.0f;
-    double s0 = 0.0, s1 = 0.0;
+    if (tid < 2) {
+        const double2 none = make_double2(0.0, 0.0);
+        for (int k = 0; k < 3; ++k) s_below[tid][k][0] = none;
+        s_below[tid][0][kLevels] = s_high[kSortGroups];
+        s_below[tid][1][kLevels] = s_low[kSortGroups];
+        s_below[tid][2][kLevels] = none;
+        s_cut[tid][0] = make_float2(-inf, __uint_as_float(0u));
+        s_cut[tid][kLevels] = make_float2(inf, __uint_as_float(s_first[kSortGroups]));
+    }
     int iter = 0;
-    for (;; ++iter) {
-        // cuts of this iteration; the last one's stop
-        if (warp == 0) {
-            const float up = __shfl_down_sync(kFull, lv, 1);
-            const float p = (lane < kLevels - 1) ? __fmul_rn(__fadd_rn(lv, up), 0.5f) : inf;
-            const int b = sort_bin(p);
-            const float above = __shfl_down_sync(kFull, p, 1), below = __shfl_up_sync(kFull, p, 1);
-            const int before = __shfl_up_sync(kFull, b, 1);
-            if (lane < kLevels - 1) {
-                SortCut c;
-                const bool one = one_value_bin(b);
-                c.p = p, c.above = above, c.below = lane ? below : -inf;
-                c.from = one ? 0u : start_of(b);
-                c.to = one ? 0u : start_of(b + 1);
-                c.end = c.begin = b + 1;
-                if (!one || !(value_of_bin(b) < p)) c.end = b;
-                if (one) c.begin = c.end;
-                c.low = lane == 0 || before != b;
-                s_cut[lane] = c;
-            }
+    if (last) {
+        // Iteration by iteration, beside the others' next one: the error, and whether the levels have stopped to move.
+        float before = __int_as_float(0x7fc00001);
+        double err = 0.0;
+        for (; iter < F.iters; ++iter) {
+            const int set = iter & 1;
+            __syncthreads();
+            if (s_stop <= iter) break;
+            lv = s_level[set][mine];
+            const double2 h0 = s_below[set][0][mine], h1 = s_below[set][0][mine + 1], l0 = s_below[set][1][mine], l1 = s_below[set][1][mine + 1];
+            const double2 r0 = s_below[set][2][mine], r1 = s_below[set][2][mine + 1];
+            const double s0 = ((h1.x - h0.x) + (l1.x - l0.x)) + (r1.x - r0.x);
+            const double s1 = ((h1.y - h0.y) + (l1.y - l0.y)) + (r1.y - r0.y);
+            const double o = (double)lv;
+            err = o * (2.0 * s1 - o * s0);
+#pragma unroll
+            for (int off = 8; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
+            err = fmax(w2 - err, 0.0) / (double)F.n_total;
+            if (lane == 0 && F.err_log) F.err_log[iter] = err;
+            if (__all_sync(kFull, __float_as_uint(lv) == __float_as_uint(before)) && lane == 0) s_stop = iter + 1;
+            before = lv;
         }
-        __syncthreads();
-        if (s_stop || iter == F.iters) break;
-        if (warp == 0) {
-            if (iter) error_of(old, s0, s1, iter - 1);
-        } else if (warp < kLevels) {
-            const SortCut c = s_cut[warp - 1];
-            double ls = 0.0, lx = 0.0, hs = 0.0, hx = 0.0;
+        err = __shfl_sync(kFull, err, 0);
+        if (F.err_log)
+            for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = err;
+        return;
+    }
+    for (; iter < F.iters; ++iter) {
+        const int set = iter & 1;
+        const float p = __fmul_rn(__fadd_rn(lv, __shfl_xor_sync(kFull, lv, 1)), 0.5f);
+        const int b = sort_bin(p);
+        const bool one = one_value_bin(b);                        // in or out as a whole
+        const int at = (one && value_of_bin(b) < p) ? b + 1 : b;  // whole bins in front of this one
+        // All loads are requested before anything is used, and without branches around them: a lane that has nothing to load loads
+        // something else.
+        const uint32_t o0 = s_off[at], o1 = s_off[b + 1], f0 = s_first[at / kSortGroup], f1 = s_first[(b + 1) / kSortGroup];
+        const double2 whole = ((lane & 1) ? s_low : s_high)[at / kSortGroup];
+        uint32_t from = f0 + o0, to = f1 + o1;
+        if (max(o0, o1) == kFarBin) {
+            if (o0 == kFarBin) from = __ldg(W.start + at);
+            if (o1 == kFarBin) to = __ldg(W.start + b + 1);
+        }
+        if (one) to = from;
+        const double rest = __ldg(reinterpret_cast<const double*>(W.pre + min(at, kSortBins - 1)) + (lane >> 4));
+        double ls = 0.0, lx = 0.0;
+        uint32_t below = 0u;
+        if (CROWDED && to - from > kSortCrowd) {
+            SortSums in{0.0, 0.0, 0ull};
+            crowded_sums<false>(W, SampleWeight<false, false>{}, from, to, -inf, p, in);
+            ls = in.s, lx = in.sx;
+            below = lane == 0 ? ~from - (uint32_t)warp : 0u;  // not counted: no two thresholds alike
+        } else {
             // 64 samples at once, which is all of most bins, then 128
             auto add = [&](auto count, uint32_t i) {
                 constexpr int U = decltype(count)::value;
@@ -905,91 +1032,68 @@ __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
                 double s[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const bool in = i + 32 * u < c.to;
-                    it[u] = in ? __ldg(W.b + i + 32 * u) : make_float2(__int_as_float(0x7fffffff), 0.0f);  // NaN: on neither side
-                    s[u] = (CELLS && in) ? __ldg(W.cell_s + i + 32 * u) : 0.0;
+                    const uint32_t j = i + 32 * u < to ? i + 32 * u : 0u;
+                    it[u] = __ldg(W.b + j);
+                    s[u] = CELLS ? __ldg(W.cell_s + j) : 0.0;
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const float x = it[u].x;
-                    const double m = (double)it[u].y, sv = CELLS ? s[u] : m * m, xv = sv * (double)x;
-                    if (x < c.p && x >= c.below && c.low) ls += sv, lx += xv;
-                    if (x >= c.p && x < c.above) hs += sv, hx += xv;
+                    const bool in = i + 32 * u < to && it[u].x < p;
+                    const double x = (double)it[u].x, m = (double)it[u].y, sv = CELLS ? s[u] : m * m, xv = sv * x;
+                    ls += in ? sv : 0.0;
+                    lx += in ? xv : 0.0;
+                    below += in ? 1u : 0u;
                 }
             };
-            if (CROWDED && c.to - c.from > kSortCrowd) {
-                const SampleWeight<false, false> weight{};
-                SortSums in{0.0, 0.0, 0ull}, out = in;
-                if (c.low) crowded_sums<false>(W, weight, c.from, c.to, c.below, c.p, in);
-                crowded_sums<false>(W, weight, c.from, c.to, c.p, c.above, out);
-                ls = in.s, lx = in.sx, hs = out.s, hx = out.sx;
-            } else {
-                if (c.from < c.to) add(std::integral_constant<int, 2>{}, c.from + lane);
-                for (uint32_t at = c.from + 64; at < c.to; at += 128) add(std::integral_constant<int, 4>{}, at + lane);
-            }
-            __syncwarp();
-            // four sums at once: a quarter of the warp goes on with each
-            const bool a = lane & 16, q = lane & 8;
-            double u = (a ? hs : ls) + __shfl_xor_sync(kFull, a ? ls : hs, 16);
-            double v = (a ? hx : lx) + __shfl_xor_sync(kFull, a ? lx : hx, 16);
-            u = (q ? v : u) + __shfl_xor_sync(kFull, q ? u : v, 8);
-#pragma unroll
-            for (int off = 4; off; off >>= 1) u += __shfl_xor_sync(kFull, u, off);
-            if ((lane & 7) == 0) {
-                double2* to = a ? &s_high[warp] : &s_low[warp - 1];
-                (q ? to->y : to->x) = u;
-            }
-        } else {
-            const int l = warp - kLevels;
-            const int b0 = l ? s_cut[l - 1].begin : 0, b1 = l < kLevels - 1 ? s_cut[l].end : kSortBins;
-            const int g0 = (b0 + kSortGroup - 1) / kSortGroup, g1 = b1 / kSortGroup;
-            const SortSums* side = nullptr;  // what this lane adds of the bins beside whole groups
-            if (g1 < g0) {                   // all inside one group
-                if (b0 + lane < b1) side = W.bin + b0 + lane;
-            } else if (b0 < b1) {
-                if (lane == 0 && b0 < g0 * kSortGroup) side = W.suf + b0;
-                if (lane == 1 && b1 > g1 * kSortGroup) side = W.pre + b1;
-            }
-            double s = 0.0, x = 0.0;
-            if (side) s = __ldg(&side->s), x = __ldg(&side->sx);
-            double gs = 0.0, gx = 0.0;
-#pragma unroll 4
-            for (int g = g0 + lane; g < g1; g += 32) {
-                const double2 t = s_group[g];
-                gs += t.x;
-                gx += t.y;
-            }
-            s += gs;
-            x += gx;
-            __syncwarp();
-            const bool a = lane & 16;
-            double v = (a ? x : s) + __shfl_xor_sync(kFull, a ? s : x, 16);
-#pragma unroll
-            for (int off = 8; off; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
-            if ((lane & 15) == 0) (a ? s_mid[l].y : s_mid[l].x) = v;
+            add(std::integral_constant<int, 2>{}, from + lane);
+            for (uint32_t i = from + 64; i < to; i += 128) add(std::integral_constant<int, 4>{}, i + lane);
         }
+        __syncwarp();
+        below = __reduce_add_sync(kFull, below);
+        // both sums at once: half the warp goes on with each
+        const bool a = lane & 16;
+        double v = (a ? lx : ls) + __shfl_xor_sync(kFull, a ? ls : lx, 16);
+        v += ((lane & 15) || at == kSortBins) ? 0.0 : rest;
+#pragma unroll
+        for (int off = 8; off; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
+        if ((lane & 15) == 0) (a ? s_below[set][2][warp + 1].y : s_below[set][2][warp + 1].x) = v;
+        if ((lane | 1) == 3) s_below[set][lane & 1][warp + 1] = whole;
+        if (lane == 4) s_cut[set][warp + 1] = make_float2(p, __uint_as_float(from + below));
+        if (lane == 8 || (lane == 9 && warp == kLevels - 2)) s_level[set][mine] = lv;
         __syncthreads();
-        if (warp == 0) {
-            old = lv;
-            if (level) {
-                s0 = s_high[lane].x + s_mid[lane].x + s_low[lane].x;
-                s1 = s_high[lane].y + s_mid[lane].y + s_low[lane].y;
-                if (!((F.fixed_mask >> lane) & 1u) && s0 > 0.0) lv = (float)(s1 / s0);
+        // the sums of the two regions, and their levels
+        const int stop = s_stop;
+        const double2 r0 = s_below[set][2][mine], r1 = s_below[set][2][mine + 1], h0 = s_below[set][0][mine], h1 = s_below[set][0][mine + 1];
+        const double2 l0 = s_below[set][1][mine], l1 = s_below[set][1][mine + 1];
+        const float2 c0 = s_cut[set][mine], c1 = s_cut[set][mine + 1];
+        double s0 = ((h1.x - h0.x) + (l1.x - l0.x)) + (r1.x - r0.x);
+        const double s1 = ((h1.y - h0.y) + (l1.y - l0.y)) + (r1.y - r0.y);
+        float moved = (float)(s1 / s0);
+        const bool empty = __float_as_uint(c0.y) == __float_as_uint(c1.y);
+        // Too small beside what was rounded (2^-20 of it) or the groups in front (2^-50), negative, or not finite: by the upper
+        // halves of the doubles, whose exponents begin at bit 20.
+        auto top = [](double d) { return __double2hiint(d) & 0x7fffffff; };
+        const int least0 = max(max(top(r0.x), top(r1.x)) - (20 << 20), top(h1.x) - (50 << 20)), least1 = max(top(r0.y), top(r1.y)) - (20 << 20);
+        const int t0 = __double2hiint(s0), t1 = top(s1);
+        const bool light = !empty && (t0 < max(least0, 0) || t1 < least1 || max(t0, t1) >= 0x7ff00000);
+        const unsigned by_itself = __ballot_sync(kFull, light);
+        if (stop <= iter) break;
+        if (by_itself & 3u) {
+            for (int k = 0; k < 2; ++k) {
+                if (!((by_itself >> k) & 1u)) continue;
+                const double2 t = region_sums<CELLS, CROWDED>(W, __shfl_sync(kFull, c0.x, k), __shfl_sync(kFull, c1.x, k));
+                if ((lane & 1) == k) s0 = t.x, moved = (float)(t.y / t.x);
             }
-            const bool same = __all_sync(kFull, __float_as_uint(lv) == __float_as_uint(old));
-            if (lane == 0 && same) s_stop = 1;
         }
+        if (!fixed && !empty && s0 > 0.0) lv = moved;
     }
-    if (warp == 0 && iter > 0) {
-        const double err = __shfl_sync(kFull, error_of(old, s0, s1, iter - 1), 0);
-        if (F.err_log)
-            for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = err;
-        if (level && !((F.fixed_mask >> lane) & 1u)) F.codebook[lane] = lv;
-    }
+    // (a stop: the levels have not moved since the iteration before)
+    if (lane == 0 || (lane == 1 && warp == kLevels - 2))
+        if (!fixed) F.codebook[mine] = lv;
 }
 
 template <bool CELLS>
-__global__ void __launch_bounds__(1024, 1)
+__global__ void __launch_bounds__(kMseThreads, 1)
 sort_fit_mse_kernel(const SortWs W, const SortFit F)
 {
     if (!after_previous()) return;
@@ -1383,7 +1487,7 @@ int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
             if (const int rc = order_windows()) return rc;
         constexpr auto kern = sort_fit_mse_kernel<CELLS>;
         if (const int rc = ensure_dynamic_smem<kern>(kMseSmem)) return rc;
-        launch_after(kern, 1, 1024, kMseSmem, st, W, F);
+        launch_after(kern, 1, kMseThreads, kMseSmem, st, W, F);
     }
     BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;

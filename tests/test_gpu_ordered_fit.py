@@ -239,3 +239,40 @@ def test_many_small_tensors(bof4, size, dtype, metric):
     else:
         np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5, atol=1e-7)
     np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5, atol=1e-12)
+
+
+def _light(n, light, seed):
+    """fp32 weights whose blocks of 64 start with their constant: a region of `light` samples whose blocks are 2^-20 of the others', and
+    beside it, in the same bins of x or the next ones, the others' samples; seen from every other level it is nothing."""
+    g = torch.Generator().manual_seed(seed)
+    u = torch.rand(n // 64, 64, generator=g)
+    x = torch.where(torch.rand(n // 64, 64, generator=g) < 0.5, 0.49992 + 3e-5 * u, 0.50006 + 3e-5 * u)
+    x[:light] = 0.49998 + 5e-5 * u[:light]
+    x[:, 0] = 1.0
+    m = torch.ones(n // 64, 1)
+    m[:light] = 2.0 ** -20
+    lv = np.array([-1, -0.5, -0.4, -0.3, -0.2, -0.1, 0, 0.1, 0.2, 0.3, 0.4, 0.4999, 0.50001, 0.5001, 0.7, 1], np.float32)
+    return (x * m).reshape(-1), lv
+
+
+@pytest.mark.parametrize("n,light", [(64 * 300, 1), (1 << 16, 40)])
+def test_a_region_that_is_light_beside_its_neighbours(bof4, n, light):
+    """Its weight is 2^-40 of what lies in front of it in its group of bins: as the difference of two sums of doubles its level
+    would be off by 1e-3 and more."""
+    w, lv = _light(n, light, 31)
+    cb, log = bof4.bof4_fit_codebook(w.cuda(), 64, 0, 0, lv, 0xffff ^ (1 << 12), 8)
+    ref, ref_log = oracle.fit([w], 64, 0, 0, lv, 0xffff ^ (1 << 12), 8)
+    assert ref[12] != lv[12]
+    np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-7)
+    np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5)
+
+
+def test_an_infinite_weight_reaches_no_other_region(bof4):
+    """Its block counts as zeros of infinite weight and one weight that is not a number: the fixed levels' regions."""
+    w = _weights(1 << 16, torch.float32, 17, "plain")
+    w[(1 << 15) + 5] = float("inf")
+    lv, mask = bof4.bof4_default_init(0)
+    cb, _ = bof4.bof4_fit_codebook(w.cuda(), 64, 0, 0, lv, mask, 8)
+    w[1 << 15:][:64] = 0
+    ref, _ = oracle.fit([w], 64, 0, 0, lv, mask, 8)
+    np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5)
