@@ -33,7 +33,6 @@ size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W)
     L.first = reinterpret_cast<uint32_t*>(take((size_t)(kSortGroups + 1) * 4));
     L.off = reinterpret_cast<uint16_t*>(take((size_t)kSortBins * 2));
     L.pre = reinterpret_cast<SortSums*>(take((size_t)kSortBins * sizeof(SortSums)));
-    L.suf = reinterpret_cast<SortSums*>(take((size_t)kSortBins * sizeof(SortSums)));
     L.bin = reinterpret_cast<SortSums*>(take((size_t)kSortBins * sizeof(SortSums)));
     L.group = reinterpret_cast<SortSums*>(take((size_t)kSortGroups * sizeof(SortSums)));
     L.lead = reinterpret_cast<SortSums*>(take(chunks * sizeof(SortSums)));
@@ -714,7 +713,7 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
 }
 
 // One warp per group of 32 bins: empty bins are cleared, bins that cross chunks put together (in the
-// order of the chunks), and the sums of the group, of the bins in front of each and from each on formed.
+// order of the chunks), and the sums of the group, of the bins in front of each formed.
 // Bound by the latency of its loads: with all crossing bins put together one after the other by the whole warp
 // it took 14.6 us for 2^20 samples, 3.7 with those of up to kSortFew chunks a lane each (cells of 2^26 weights 22.9, 10.5).
 // Between 4 and 64 chunks as the line the fits of 2^18 to 2^24 weights differ by less than 2 us; at 64 those of 2^18 are 1.5 slower.
@@ -778,16 +777,12 @@ sort_group_kernel(const SortWs W)
         }
     }
     W.bin[b] = t;
-    SortSums up = t, down = t;  // this bin and those in front of it; and those behind it
+    SortSums up = t;  // this bin and those in front of it
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const SortSums u{__shfl_up_sync(kFull, up.s, o), __shfl_up_sync(kFull, up.sx, o), MAE ? __shfl_up_sync(kFull, up.a, o) : 0ull};
-        const SortSums d{__shfl_down_sync(kFull, down.s, o), __shfl_down_sync(kFull, down.sx, o),
-                         MAE ? __shfl_down_sync(kFull, down.a, o) : 0ull};
         if (lane >= o) sums_add(up, u);
-        if (lane + o < 32) sums_add(down, d);
     }
-    W.suf[b] = down;
     if (lane == 0) W.pre[b] = SortSums{0.0, 0.0, 0ull};
     if (lane < 31) W.pre[b + 1] = up;
     else W.group[g] = up;
@@ -1113,15 +1108,18 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v)
 }
 
 //
-// One CTA.  Warp 2 l + h owns half h of region l: the samples from the region's lower threshold to its
-// level (h = 0) or from the level to the upper threshold (h = 1); the split is what the MAE error needs.
-// An iteration is a chain of latencies (thresholds -> first samples of the two cut bins -> those samples
-// -> butterfly -> level update), so everything that does not depend on one another is requested
-// together; the cut bins are mostly those of the iteration before and come from L1.  When an iteration
-// leaves every level unchanged the remaining ones would repeat it bit for bit: their entries of the
-// error log are filled in and the loop ends.  30 iterations over 2^24 fp32 weights: 1267 us with a median found by
-// halving the range of keys, 992 by the weights between them; over 3 * 2^20 bf16 weights 416 -> 390, eight layers of
-// a 7B-shaped model 213 -> 180.
+// One CTA, and as for the squared error what lies below a threshold is one sum that its own warp forms (whole groups and bins from
+// running sums, the samples of its bin).  Behind a barrier warp l looks for the median of region l: the weight at which half of
+// the region is reached is a place in the running sums of all groups (shared memory, 64 entries a step), then of the group's bins
+// (one load), then among the samples of one bin.  A second barrier, and the levels are there.  Eight more warps add up
+// beside this what lies below each level, which the error of the iteration needs and nothing else, and warp 15, which has no
+// threshold, writes the error of the iteration before.  The weights are integers, so a region is exactly the difference of two sums.
+// When an iteration leaves every level unchanged the remaining ones would repeat it bit for bit: their entries of the
+// error log are filled in and the loop ends.
+// An iteration over eight layers of a 7B-shaped model or 2^26 bf16 weights 5.6 -> 2.5 us, over 2^20 fp32 weights 6.5 -> 3.1, over 2^24
+// 33 -> 14 (before: two warps to a region, whole groups added up and searched one after the other, cut bins first).  Bound by its
+// chain: three loads from L2 of 430 or 820 cycles each, the reductions, two barriers; over 2^24 weights by the passes over the 500 samples
+// of a bin (of up to 64 samples every lane adds up what is not behind its own, in one pass: 2^26 bf16 3.0 -> 2.5, 2^20 fp32 3.75 -> 3.1).
 
 // The sample of a crowded bin, among those with p <= x < q, at which twice the weight `before` and up to it reaches `total`;
 // false, and `before` advanced past them, where it lies behind them.  Called by a whole warp.
@@ -1186,31 +1184,76 @@ __device__ __noinline__ bool crowded_median(const SortWs& W, const SampleWeight<
     return true;
 }
 
+constexpr int kMaeScan = 32 * kLevels, kMaeThreads = kMaeScan + 32 * kLevels / 2;
+constexpr int kMaeSums = ((kSortGroups + 1) * 8 + 15) / 16 * 16;  // shared memory: what lies in front of the groups: fixed-point weights, {s, sx},
+constexpr int kMaeOff = kMaeSums + (kSortGroups + 1) * 16;      // first samples of the bins,
+constexpr int kMaeFirst = kMaeOff + kSortBins * 2 + 16;         // (and the end) of the groups
+constexpr int kMaeSmem = kMaeFirst + (kSortGroups + 1) * 4;
+
 // CROWDED: the kernel for data with crowded bins.  Both are launched, the flag of such bins tells which one runs: with both
 // loops in one kernel 2^22 fp32 weights, 12 iterations, took 299 us against 293.5, 2^20 153.8 against 152.4.
 template <bool CELLS, bool CROWDED>
-__global__ void __launch_bounds__(1024, 1)
+__global__ void __launch_bounds__(kMaeThreads, 1)
 sort_fit_mae_kernel(const SortWs W, const SortFit F)
 {
     if (!after_previous()) return;
-    if (CROWDED && W.n_items[4] == 0u) return;
-    const uint32_t other = CELLS || CROWDED ? 0u : W.n_items[4];
+    if (!CELLS && (W.n_items[4] != 0u) != CROWDED) return;
     extern __shared__ __align__(16) unsigned char s_fit[];
-    SortSums* const s_group = reinterpret_cast<SortSums*>(s_fit);
-    __shared__ float s_level[2][kLevels], s_med[kLevels];
-    __shared__ SortSums s_half[32];
+    unsigned long long* const s_a = reinterpret_cast<unsigned long long*>(s_fit);
+    double2* const s_sums = reinterpret_cast<double2*>(s_fit + kMaeSums);
+    uint16_t* const s_off = reinterpret_cast<uint16_t*>(s_fit + kMaeOff);
+    uint32_t* const s_first = reinterpret_cast<uint32_t*>(s_fit + kMaeFirst);
+    __shared__ unsigned long long s_below[2][kLevels + 1];  // fixed-point weight below threshold k - 1; entry 0: nothing, entry 16: everything
+    __shared__ float s_level[2][kLevels];
+    __shared__ double s_err[2][2 * kLevels];  // parts of the error: the thresholds' and the levels'
+    __shared__ SortSums s_warp[kLevels];
     __shared__ int s_stop;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     SampleWeight<true, false> weight;
     weight.max_bits = W.n_items[1];
     weight.unit = F.metric >= 2;
-    for (int k = tid; k < kSortGroups; k += 1024) s_group[k] = W.group[k];
+    if (tid == 0) s_stop = 0, s_off[kSortBins] = 0u;
+    copy_starts(W, s_off, s_first);
     if (tid < kLevels) s_level[0][tid] = F.codebook[tid];
-    if (tid == 0) s_stop = 0;
-    if (other) return;
+    {  // running sums of the groups, four to a thread of the first warps
+        constexpr int PER = kSortGroups / kMaeScan;
+        const bool has = warp < kLevels;
+        SortSums g[PER], t{0.0, 0.0, 0ull};
+#pragma unroll
+        for (int k = 0; k < PER; ++k) g[k] = W.group[(has ? tid : 0) * PER + k];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) sums_add(t, g[k]);
+        auto scan = [&](SortSums& v) {  // inclusive, over the warp
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const SortSums u{__shfl_up_sync(kFull, v.s, off), __shfl_up_sync(kFull, v.sx, off), __shfl_up_sync(kFull, v.a, off)};
+                if (lane >= off) sums_add(v, u);
+            }
+        };
+        scan(t);
+        if (lane == 31 && has) s_warp[warp] = t;
+        __syncthreads();
+        SortSums w{0.0, 0.0, 0ull};
+        if (lane < warp && lane < kLevels) w = s_warp[lane];
+        scan(w);
+        SortSums run{__shfl_up_sync(kFull, t.s, 1), __shfl_up_sync(kFull, t.sx, 1), __shfl_up_sync(kFull, t.a, 1)};
+        if (lane == 0) run = SortSums{0.0, 0.0, 0ull};
+        sums_add(run, SortSums{__shfl_sync(kFull, w.s, 31), __shfl_sync(kFull, w.sx, 31), __shfl_sync(kFull, w.a, 31)});
+#pragma unroll
+        for (int k = 0; k <= PER; ++k) {
+            if (!has || (k == PER && tid < kMaeScan - 1)) break;  // behind the last group: everything
+            s_a[tid * PER + k] = run.a;
+            s_sums[tid * PER + k] = make_double2(run.s, run.sx);
+            if (k < PER) sums_add(run, g[k]);
+        }
+    }
+    copies_done();
     __syncthreads();
-    const int l = warp >> 1, h = warp & 1;
-    const float inf = __int_as_float(0x7f800000);
+    if (tid < 2) s_below[tid][0] = 0ull, s_below[tid][kLevels] = s_a[kSortGroups];
+    auto start_of = [&](int b) -> uint32_t {  // first sample of bin b <= kSortBins
+        const uint32_t o = s_off[b], f = s_first[b / kSortGroup];
+        return o == kFarBin ? __ldg(W.start + b) : f + o;
+    };
     auto use = [&](uint32_t i, float2 it, double& s, unsigned long long& a) {
         if (CELLS) {
             s = __ldg(W.cell_s + i);
@@ -1219,230 +1262,253 @@ sort_fit_mae_kernel(const SortWs W, const SortFit F)
             weight(it, s, a);
         }
     };
-    auto bin_sums = [&](int b) {
-        SortSums v;
-        v.s = __ldg(&W.bin[b].s);
-        v.sx = __ldg(&W.bin[b].sx);
-        v.a = __ldg(&W.bin[b].a);
-        return v;
-    };
-    int now = 0;
-    for (int iter = 0; iter < F.iters; ++iter, now ^= 1) {
-        const float* s_lv = s_level[now];
-        const float lv = s_lv[l];
-        const float lo = l ? __fmul_rn(__fadd_rn(s_lv[l - 1], lv), 0.5f) : -inf;
-        const float hi = l < kLevels - 1 ? __fmul_rn(__fadd_rn(lv, s_lv[l + 1]), 0.5f) : inf;
-        const float mid = fminf(fmaxf(lv, lo), hi);
-        const float p = h ? mid : lo, q = h ? hi : mid;  // this warp: samples with p <= x < q
-        const int bp = (p == -inf) ? -1 : sort_bin(p), bq = (q == inf) ? kSortBins : sort_bin(q);
-        // bins strictly inside, as whole groups with up to 31 single bins on either side
-        const int b0 = bp + 1, b1 = max(bq, b0);
-        const int g0 = (b0 + kSortGroup - 1) / kSortGroup, g1 = b1 / kSortGroup;
-        const int head_end = min(b1, g0 * kSortGroup), tail0 = (g1 >= g0) ? g1 * kSortGroup : b1;
-        const bool cut_p = bp >= 0, cut_q = bq < kSortBins && bq != bp;
-        const bool one_p = one_value_bin(bp), one_q = one_value_bin(bq);
-        SortSums t{0.0, 0.0, 0ull};
-        // the cut bins' samples: the first 32 of both are on their way before anything is added up
-        uint32_t sp = 0u, ep = 0u, sq = 0u, eq = 0u;
-        if (cut_p && !one_p) sp = __ldg(W.start + bp) + lane, ep = __ldg(W.start + bp + 1);
-        if (cut_q && !one_q) sq = __ldg(W.start + bq) + lane, eq = __ldg(W.start + bq + 1);
-        if (CROWDED) {
-            if (ep > kSortCrowd && ep - kSortCrowd > sp - lane) {
-                crowded_sums<true>(W, weight, sp - lane, ep, p, q, t);
-                ep = 0u;
-            }
-            if (eq > kSortCrowd && eq - kSortCrowd > sq - lane) {
-                crowded_sums<true>(W, weight, sq - lane, eq, p, q, t);
-                eq = 0u;
-            }
-        }
-        const bool in_p = sp < ep, in_q = sq < eq;
-        float2 ip = make_float2(0.0f, 0.0f), iq = ip;
-        if (in_p) ip = __ldg(W.b + sp);
-        if (in_q) iq = __ldg(W.b + sq);
-        auto take = [&](uint32_t i, float2 it) {
-            if (!(it.x >= p && it.x < q)) return;
-            double s;
-            unsigned long long a;
-            use(i, it, s, a);
-            t.s += s;
-            t.sx += s * (double)it.x;
-            t.a += a;
-        };
-        if (b0 + lane < head_end) sums_add(t, bin_sums(b0 + lane));
-        if (tail0 + lane < b1) sums_add(t, bin_sums(tail0 + lane));
-        for (int g = g0 + lane; g < g1; g += 32) sums_add(t, s_group[g]);
-        if (lane == 0) {  // bins of one value are in or out as a whole
-            if (cut_p && one_p && value_of_bin(bp) >= p && value_of_bin(bp) < q) sums_add(t, bin_sums(bp));
-            if (cut_q && one_q && value_of_bin(bq) >= p && value_of_bin(bq) < q) sums_add(t, bin_sums(bq));
-        }
-        if (in_p) {
-            take(sp, ip);
-            for (uint32_t i = sp + 32; i < ep; i += 32) take(i, __ldg(W.b + i));
-        }
-        if (in_q) {
-            take(sq, iq);
-            for (uint32_t i = sq + 32; i < eq; i += 32) take(i, __ldg(W.b + i));
+    // What lies below v, less the whole groups in front of the one that is returned: this lane's share.
+    auto below = [&](float v, SortSums& t) -> int {
+        const int b = sort_bin(v);
+        const bool one = one_value_bin(b);                        // in or out as a whole
+        const int at = (one && value_of_bin(b) < v) ? b + 1 : b;  // whole bins in front of this one
+        const uint32_t from = start_of(at), to = one ? from : start_of(b + 1);
+        t = SortSums{0.0, 0.0, 0ull};
+        const unsigned long long pre = __ldg(reinterpret_cast<const unsigned long long*>(W.pre + min(at, kSortBins - 1)) + (lane < 3 ? lane : 0));
+        if (CROWDED && to - from > kSortCrowd) {
+            crowded_sums<true>(W, weight, from, to, -__int_as_float(0x7f800000), v, t);
+        } else {
+            auto add = [&](auto count, uint32_t i) {  // 64 samples at once, which is all of most bins, then 128
+                constexpr int U = decltype(count)::value;
+                float2 it[U];
+                double s[U];
+                unsigned long long a[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const uint32_t j = i + 32 * u < to ? i + 32 * u : 0u;
+                    it[u] = __ldg(W.b + j);
+                    if (CELLS) use(j, it[u], s[u], a[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!CELLS) use(i, it[u], s[u], a[u]);
+                    const bool in = i + 32 * u < to && it[u].x < v;
+                    const double sx = s[u] * (double)it[u].x;
+                    t.s += in ? s[u] : 0.0;
+                    t.sx += in ? sx : 0.0;
+                    t.a += in ? a[u] : 0ull;
+                }
+            };
+            add(std::integral_constant<int, 2>{}, from + lane);
+            for (uint32_t i = from + 64; i < to; i += 128) add(std::integral_constant<int, 4>{}, i + lane);
         }
         __syncwarp();
-        sums_reduce<false>(t);
-        t.a = warp_sum64(t.a);
-        if (lane == 0) s_half[warp] = t;
+        if (at < kSortBins) {
+            if (lane == 0) t.s += __longlong_as_double((long long)pre);
+            if (lane == 1) t.sx += __longlong_as_double((long long)pre);
+            if (lane == 2) t.a += pre;
+        }
+        return at / kSortGroup;
+    };
+    // the lanes' shares of two sums together: {s, sx} in all lanes
+    auto both = [&](double s, double x) -> double2 {
+        const bool h = lane & 16;
+        double v = (h ? x : s) + __shfl_xor_sync(kFull, h ? s : x, 16);
+#pragma unroll
+        for (int off = 8; off; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
+        return make_double2(__shfl_sync(kFull, v, 0), __shfl_sync(kFull, v, 16));
+    };
+    // the error of iteration `at`, by warp 15: it has no threshold
+    auto error_of = [&](int at) {
+        double err = s_err[at & 1][lane];
+#pragma unroll
+        for (int off = 16; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
+        err = fmax(err, 0.0) / (double)F.n_total;
+        if (lane == 0 && F.err_log) F.err_log[at] = err;
+        return err;
+    };
+    int iter = 0;
+    if (warp >= kLevels) {
+        // ---- the levels' parts of the error, two levels to a warp, beside the others' search for the next ones
+        float known[2];
+        double part[2];
+        for (; iter < F.iters; ++iter) {
+            const int set = iter & 1;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int l = 2 * (warp - kLevels) + k;
+                const float lv = s_level[set][l];
+                if (iter == 0 || __float_as_uint(lv) != __float_as_uint(known[k])) {
+                    SortSums t;
+                    const int g = below(lv, t);
+                    const double2 r = both(t.s, t.sx), p = s_sums[g];
+                    known[k] = lv;
+                    part[k] = 2.0 * ((double)lv * (r.x + p.x) - (r.y + p.y));
+                }
+                if (lane == 0) s_err[set][kLevels + l] = part[k];
+                __syncthreads();
+                if (k == 0 && s_stop) return;
+            }
+        }
+        return;
+    }
+    // ---- warp w: threshold w and level w
+    const bool fixed = (F.fixed_mask >> warp) & 1u, cuts = warp < kLevels - 1;
+    float lv = s_level[0][warp];
+    for (; iter < F.iters; ++iter) {
+        const int set = iter & 1;
+        SortSums t{0.0, 0.0, 0ull};
+        float above = 0.0f;  // the next level
+        int group = 0;
+        if (cuts) {
+            above = s_level[set][warp + 1];
+            group = below(__fmul_rn(__fadd_rn(lv, above), 0.5f), t);
+            const unsigned long long a = warp_sum64(t.a) + s_a[group];
+            if (lane == 0) s_below[set][warp + 1] = a;
+        } else {
+            if (iter) {
+                const double err = error_of(iter - 1);
+                const int l = lane & (kLevels - 1);
+                // no level has moved: the remaining iterations would repeat this one bit for bit
+                if (__all_sync(kFull, __float_as_uint(s_level[set][l]) == __float_as_uint(s_level[set ^ 1][l]))) {
+                    if (lane == 0) s_stop = 1;
+                    if (F.err_log)
+                        for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = err;
+                }
+            }
+        }
         __syncthreads();
-        {
-            // The warp whose half holds the crossing of half the region's weight finds the sample.
-            const unsigned long long below = s_half[2 * l].a, total = below + s_half[2 * l + 1].a;
-            const bool in_lower = 2ull * below >= total;
-            if (total > 0ull && in_lower == (h == 0) && !((F.fixed_mask >> l) & 1u)) {
-                unsigned long long before = h ? below : 0ull;
-                // the samples of bin b inside [p, q): smallest key with 2 (before + weight up to it) >= total;
-                // false (and `before` advanced) if the crossing lies behind them
-                auto pick = [&](int b) -> bool {
-                    if (one_value_bin(b)) {
-                        const float x = value_of_bin(b);
-                        const unsigned long long a = (x >= p && x < q) ? bin_sums(b).a : 0ull;
-                        if (a == 0ull || 2ull * (before + a) < total) {
-                            before += a;
-                            return false;
-                        }
-                        if (lane == 0) s_med[l] = x;
-                        return true;
-                    }
-                    constexpr int R = 4;
-                    const uint32_t s0 = __ldg(W.start + b), e = __ldg(W.start + b + 1);
-                    if (CROWDED && e - s0 > kSortCrowd) {
-                        float median;
-                        if (!crowded_median(W, weight, s0, e, p, q, total, before, median)) return false;
-                        if (lane == 0) s_med[l] = median;
-                        return true;
-                    }
-                    uint32_t key[R], kmin = 0xffffffffu, kmax = 0u;
-                    unsigned long long wt[R], sum = 0ull;
+        if (s_stop) break;
+        // The median of the region: the first sample, in the order of x, with which the weight reaches half.
+        const unsigned long long a0 = s_below[set][warp], a1 = s_below[set][warp + 1];
+        const float from_left = warp ? s_level[set][warp - 1] : 0.0f;
+        // (levels that do not ascend have regions without samples)
+        const bool some = a1 != a0 && !(warp && cuts && __fadd_rn(from_left, lv) * 0.5f > __fadd_rn(lv, above) * 0.5f);
+        const bool search = some && !fixed;
+        const unsigned long long goal = a0 + (a1 - a0) - (a1 - a0) / 2ull;
+        int g = 0;
+        SortSums pre{0.0, 0.0, 0ull};
+        if (search) {
+            // the last group in front of which there is less than the goal: 32 groups of 64, then one of 64
+            int c = __popc(__ballot_sync(kFull, s_a[64 * (lane + 1)] < goal));
+            const unsigned long long u = s_a[64 * c + 1 + lane], v = s_a[64 * c + 33 + lane];
+            g = 64 * c + __popc(__ballot_sync(kFull, u < goal)) + __popc(__ballot_sync(kFull, v < goal));
+            pre.a = __ldg(&W.pre[g * kSortGroup + lane].a);
+        }
+        {  // beside the search: the threshold's part of the error (the last warp: that of everything)
+            const double2 s = cuts ? both(t.s, t.sx) : s_sums[kSortGroups], p = cuts ? s_sums[group] : make_double2(0.0, 0.0);
+            double err = (s.y + p.y) - (double)lv * (s.x + p.x);
+            if (cuts) err -= (double)above * (s.x + p.x) - (s.y + p.y);
+            if (lane == 0) s_err[set][warp] = err;
+        }
+        if (search) {
+            const unsigned long long before = s_a[g];
+            const int in = __popc(__ballot_sync(kFull, before + pre.a < goal)) - 1, b = g * kSortGroup + in;
+            const unsigned long long front = before + __shfl_sync(kFull, pre.a, in), need = goal - front;
+            if (one_value_bin(b)) {
+                lv = value_of_bin(b);
+            } else {
+                const uint32_t s0 = start_of(b), e = start_of(b + 1);
+                if (CROWDED && e - s0 > kSortCrowd) {
+                    unsigned long long none = 0ull;
+                    const float inf = __int_as_float(0x7f800000);
+                    crowded_median(W, weight, s0, e, -inf, inf, 2ull * need, none, lv);
+                } else {
                     auto get = [&](uint32_t i, uint32_t& k, unsigned long long& a) {
-                        k = 0xffffffffu;
-                        a = 0ull;
-                        if (i < e) {
-                            const float2 it = __ldg(W.b + i);
-                            double s;
-                            if (it.x >= p && it.x < q) {
-                                use(i, it, s, a);
-                                k = sort_key(it.x);
+                        const uint32_t j = i < e ? i : s0;
+                        const float2 it = __ldg(W.b + j);
+                        double s;
+                        use(j, it, s, a);
+                        k = i < e ? sort_key(it.x) : 0xffffffffu;
+                        a = i < e ? a : 0ull;
+                    };
+                    // Few samples: one or two to a lane, which adds up for each all those that are not behind it.
+                    auto among = [&](auto count) {
+                        constexpr int N = decltype(count)::value;
+                        using Weight = typename std::conditional<CELLS, unsigned long long, uint32_t>::type;  // (31 bits, one sample per weight)
+                        uint32_t key[N], first = 0xffffffffu;
+                        Weight mine[N];
+                        unsigned long long a, sum[N];
+#pragma unroll
+                        for (int r = 0; r < N; ++r) {
+                            get(s0 + 32 * r + lane, key[r], a);
+                            mine[r] = (Weight)a;
+                            sum[r] = 0ull;
+                        }
+#pragma unroll
+                        for (int r = 0; r < N; ++r) {
+                            const int here = min((int)(e - s0) - 32 * r, 32);
+#pragma unroll 4
+                            for (int j = 0; j < here; ++j) {
+                                const uint32_t k = __shfl_sync(kFull, key[r], j);
+                                const Weight w = __shfl_sync(kFull, mine[r], j);
+#pragma unroll
+                                for (int q = 0; q < N; ++q) sum[q] += k <= key[q] ? w : 0;
                             }
                         }
+#pragma unroll
+                        for (int q = 0; q < N; ++q)
+                            if (sum[q] >= need) first = min(first, key[q]);  // (no sample: the last key of all)
+                        lv = sort_key_value(__reduce_min_sync(kFull, first));
                     };
+                    if (e - s0 <= 32u) {
+                        among(std::integral_constant<int, 1>{});
+                    } else if (e - s0 <= 64u) {
+                        among(std::integral_constant<int, 2>{});
+                    } else {
+                        // The goal is reached at one of the keys k0 ... k1 of the bin's samples; c0 of the bin's weight lies
+                        // below k0, c1 up to k1.  The next key to split at is where even weights would put it (every third
+                        // time the middle), and the ends move to samples: a handful of steps, where halving the keys
+                        // takes one per bit in which they differ.
+                        constexpr int R = 4;
+                        uint32_t key[R], kmin = 0xffffffffu, kmax = 0u;
+                        unsigned long long wt[R];
+                        unsigned long long c0 = 0ull, c1 = __ldg(&W.bin[b].a);
 #pragma unroll
-                    for (int r = 0; r < R; ++r) get(s0 + 32 * r + lane, key[r], wt[r]);
-                    auto each = [&](auto fn) {
+                        for (int r = 0; r < R; ++r) get(s0 + 32 * r + lane, key[r], wt[r]);
+                        auto each = [&](auto fn) {
 #pragma unroll
-                        for (int r = 0; r < R; ++r) fn(key[r], wt[r]);
-                        for (uint32_t i = s0 + 32 * R + lane; i < e; i += 32 * R) {
-                            uint32_t k[R];
-                            unsigned long long a[R];
+                            for (int r = 0; r < R; ++r) fn(key[r], wt[r]);
+                            for (uint32_t i = s0 + 32 * R + lane; i < e; i += 32 * 2 * R) {
+                                uint32_t k[2 * R];
+                                unsigned long long a[2 * R];
 #pragma unroll
-                            for (int r = 0; r < R; ++r) get(i + 32 * r, k[r], a[r]);
+                                for (int r = 0; r < 2 * R; ++r) get(i + 32 * r, k[r], a[r]);
 #pragma unroll
-                            for (int r = 0; r < R; ++r) fn(k[r], a[r]);
-                        }
-                        __syncwarp();
-                    };
-                    each([&](uint32_t k, unsigned long long a) {
-                        if (k != 0xffffffffu) {
-                            kmin = min(kmin, k);
-                            kmax = max(kmax, k);
-                        }
-                        sum += a;
-                    });
-                    sum = warp_sum64(sum);
-                    if (2ull * (before + sum) < total || sum == 0ull) {
-                        before += sum;
-                        return false;
-                    }
-                    // The crossing is at one of the keys k0 ... k1 of the bin's samples; c0 of the bin's weight lies
-                    // below k0, c1 up to k1.  The next key to split at is where even weights would put it (every third
-                    // time the middle), and the ends move to samples: a handful of steps, where halving the keys
-                    // takes one per bit in which they differ.
-                    uint32_t k0 = __reduce_min_sync(kFull, kmin), k1 = __reduce_max_sync(kFull, kmax);
-                    unsigned long long c0 = 0ull, c1 = sum;
-                    for (int step = 1; k0 < k1; ++step) {
-                        const uint32_t d = k1 - k0;
-                        const float at = step % 3 == 0 ? 0.5f : (float)(total - 2ull * (before + c0)) / (2.0f * (float)(c1 - c0));
-                        const uint32_t km = k0 + min((uint32_t)((float)d * at), d - 1u);
-                        uint32_t end = 0u, begin = 0xffffffffu;
-                        sum = 0ull;
-                        each([&](uint32_t k, unsigned long long a) {
-                            if (k <= km) {
-                                sum += a;
-                                end = max(end, k);
-                            } else {
-                                begin = min(begin, k);
+                                for (int r = 0; r < 2 * R; ++r) fn(k[r], a[r]);
+                            }
+                            __syncwarp();
+                        };
+                        each([&](uint32_t k, unsigned long long) {
+                            if (k != 0xffffffffu) {
+                                kmin = min(kmin, k);
+                                kmax = max(kmax, k);
                             }
                         });
-                        sum = warp_sum64(sum);
-                        if (2ull * (before + sum) >= total) k1 = __reduce_max_sync(kFull, end), c1 = sum;
-                        else k0 = __reduce_min_sync(kFull, begin), c0 = sum;
+                        uint32_t k0 = __reduce_min_sync(kFull, kmin), k1 = __reduce_max_sync(kFull, kmax);
+                        for (int step = 1; k0 < k1; ++step) {
+                            const uint32_t d = k1 - k0;
+                            const float part = step % 3 == 0 ? 0.5f : (float)(need - c0) / (float)(c1 - c0);
+                            const uint32_t km = k0 + min((uint32_t)((float)d * part), d - 1u);
+                            uint32_t end = 0u, begin = 0xffffffffu;
+                            unsigned long long sum = 0ull;
+                            each([&](uint32_t k, unsigned long long a) {
+                                if (k <= km) {
+                                    sum += a;
+                                    end = max(end, k);
+                                } else {
+                                    begin = min(begin, k);
+                                }
+                            });
+                            sum = warp_sum64(sum);
+                            if (sum >= need) k1 = __reduce_max_sync(kFull, end), c1 = sum;
+                            else k0 = __reduce_min_sync(kFull, begin), c0 = sum;
+                        }
+                        lv = sort_key_value(k0);
                     }
-                    if (lane == 0) s_med[l] = sort_key_value(k0);
-                    return true;
-                };
-                // 32 entries, this lane's `mine`: the first that reaches half, or -1; `before` advanced past those in front
-                auto first_of = [&](unsigned long long mine) -> int {
-                    unsigned long long incl = mine;
-#pragma unroll
-                    for (int off = 1; off < 32; off <<= 1) {
-                        const unsigned long long v = __shfl_up_sync(kFull, incl, off);
-                        if (lane >= off) incl += v;
-                    }
-                    const unsigned hit = __ballot_sync(kFull, 2ull * (before + incl) >= total && mine > 0ull);
-                    const int at = __ffs(hit) - 1;
-                    const unsigned long long upto = __shfl_sync(kFull, incl, at < 0 ? 31 : at);
-                    before += (at < 0) ? upto : upto - __shfl_sync(kFull, mine, at);
-                    return at;
-                };
-                auto bins = [&](int from, int to) -> bool {  // at most 32 whole bins
-                    const int at = first_of((from + lane < to) ? bin_sums(from + lane).a : 0ull);
-                    return at >= 0 && pick(from + at);
-                };
-                bool found = cut_p && pick(bp);
-                if (!found && b0 < head_end) found = bins(b0, head_end);
-                for (int g = g0; !found && g < g1; g += 32) {
-                    const int at = first_of((g + lane < g1) ? s_group[g + lane].a : 0ull);
-                    if (at >= 0) found = bins((g + at) * kSortGroup, (g + at + 1) * kSortGroup);
                 }
-                if (!found && tail0 < b1) found = bins(tail0, b1);
-                if (!found && cut_q) pick(bq);
-            }
-            __syncthreads();
-        }
-        double err = 0.0;
-        if (warp < 2 && lane < kLevels) {
-            const SortSums u = s_half[2 * lane], v = s_half[2 * lane + 1];
-            const float old = s_lv[lane];
-            const double o = (double)old;
-            if (warp == 0) {
-                float next = old;
-                if (!((F.fixed_mask >> lane) & 1u)) {
-                    if (u.a + v.a > 0ull) next = s_med[lane];
-                }
-                s_level[now ^ 1][lane] = next;
-                const bool same = __all_sync(0xffffu, __float_as_uint(next) == __float_as_uint(old));
-                if (lane == 0) s_stop = same ? 1 : 0;
-            } else {
-                err = (o * u.s - u.sx) + (v.sx - o * v.s);
-#pragma unroll
-                for (int off = 8; off; off >>= 1) err += __shfl_xor_sync(0xffffu, err, off);
-                err = fmax(err, 0.0) / (double)F.n_total;
-                if (lane == 0 && F.err_log) F.err_log[iter] = err;
             }
         }
+        if (lane == 0) s_level[set ^ 1][warp] = lv;
         __syncthreads();
-        if (s_stop) {
-            if (warp == 1 && lane < kLevels && F.err_log)
-                for (int k = iter + 1 + lane; k < F.iters; k += kLevels) F.err_log[k] = err;
-            now ^= 1;
-            break;
-        }
     }
-    if (tid < kLevels && !((F.fixed_mask >> tid) & 1u)) F.codebook[tid] = s_level[now][tid];
+    if (warp == kLevels - 1 && iter == F.iters && iter) error_of(iter - 1);
+    if (lane == 0 && !fixed) F.codebook[warp] = lv;
 }
 
 // ---------------------------------------------------------------- host side
@@ -1472,15 +1538,15 @@ int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
     };
     const bool may_crowd = !CELLS && F.n_max > kSortCrowd;
     if constexpr (MAE) {
-        constexpr int smem = kSortGroups * (int)sizeof(SortSums);
+        constexpr int smem = kMaeSmem;
         constexpr auto plain = sort_fit_mae_kernel<CELLS, false>;
         if (const int rc = ensure_dynamic_smem<plain>(smem)) return rc;
-        launch_after(plain, 1, 1024, smem, st, W, F);
+        launch_after(plain, 1, kMaeThreads, smem, st, W, F);
         if (may_crowd) {
             if (const int rc = order_windows()) return rc;
             constexpr auto crowded = sort_fit_mae_kernel<CELLS, !CELLS>;
             if (const int rc = ensure_dynamic_smem<crowded>(smem)) return rc;
-            launch_after(crowded, 1, 1024, smem, st, W, F);
+            launch_after(crowded, 1, kMaeThreads, smem, st, W, F);
         }
     } else {
         if (may_crowd)

@@ -45,7 +45,7 @@ struct SortWs {
     uint32_t* first;      // [kSortGroups + 1] first sample of every group; before, the largest constants of the samples' CTAs
     uint16_t* off;        // [kSortBins] first sample of a bin in its group, kFarBin: too far, see start
     SortSums *bin, *group;
-    SortSums *pre, *suf;  // per bin: the bins of its group in front of it; it and those behind it
+    SortSums* pre;        // per bin: the bins of its group in front of it
     SortSums *lead, *trail;  // [chunks] part of a bin that began in an earlier chunk / that goes on in the next
     float2 *a, *b;        // samples, ordered samples
     SortSums* before;     // crowded bins: sums of the window's samples in front of every fourth (in the place of a)

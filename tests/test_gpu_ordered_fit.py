@@ -276,3 +276,17 @@ def test_an_infinite_weight_reaches_no_other_region(bof4):
     w[1 << 15:][:64] = 0
     ref, _ = oracle.fit([w], 64, 0, 0, lv, mask, 8)
     np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-5)
+
+
+@pytest.mark.parametrize("each", [31, 32, 33, 63, 64, 65, 127, 129, 700])
+def test_median_among_the_samples_of_one_bin(bof4, each):
+    """`each` samples in every occupied bin, near the sizes at which they are looked through in another way; equal samples among
+    them, and medians that lie at the first and the last of a bin."""
+    g = torch.Generator().manual_seed(each)
+    bins = 90
+    x = (torch.arange(bins).repeat_interleave(each) * 137 + 800 + (0.05 + 0.9 * torch.rand(bins * each, generator=g))) / 32566
+    x = torch.where(torch.rand(x.numel(), generator=g) < 0.2, x.roll(1), x)[torch.randperm(x.numel(), generator=g)]
+    x = x[:x.numel() // 31 * 31].view(-1, 31)
+    w = torch.cat([torch.ones(len(x), 1), x, x.neg().flip(0)], 1)
+    w = torch.nn.functional.pad(w, (0, 1)) * (0.5 + torch.rand(len(x), 1, generator=g))
+    _check(bof4, [w.reshape(-1)], 64, 0, bof4.METRIC_MAE, 12)
