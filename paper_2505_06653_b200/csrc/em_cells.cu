@@ -4,10 +4,10 @@
 // the size of the data, the normalised weights of magnitude 2^-40 and more take at most 128 * 128 * 2 * 40
 // values, and the fit only needs the sum of the sample weights (m^2 or |m|) of each.  The data is read
 // twice, once for the block constants and once for the counts; then a fit of any number of iterations
-// works on at most 1.3 million samples (about 0.4 million for near-Gaussian data).
+// works on 1.3 million cells (of which near-Gaussian data occupies about 0.4 million).
 //
 //   blocks      block constants (bf16, stored) and the number of blocks per magnitude; HBM bound
-//   plan        first position of every magnitude, units of work
+//   plan        first position of every magnitude, units of work; the order of the fractions a / b
 //   order       block addresses grouped by magnitude
 //   accumulate  a unit is some blocks of ONE magnitude |m|: with m fixed, the cell of a weight is the
 //               difference of the two bit patterns, so the counts of a unit are 10240 words of shared
@@ -15,7 +15,7 @@
 //               on random banks, whose conflicts bound it (4.6 wavefronts of the LSU data path per 32 weights; two
 //               weights at a time without a predicate where all are counted: 2^26 weights 56 -> 51 us, 1.6 * 10^9 827 -> 811);
 //               when the unit is done its counts times the weight of |m| are added to the cells
-//   items       the occupied cells in a fixed order, as samples for the ordering passes
+//   then        sums of the cells in the order of x, and all iterations (em_cells_fit.cu)
 //
 // A cell is (significand of m, sign, distance of the bit patterns).  Cell sums are integers (128 bits, a
 // fixed-point scale relative to the largest |m|; exact while |m| is within 2^-38 of it), so they do not
@@ -23,16 +23,11 @@
 // exponent only (deep cells): they count as the power of two at or below them.  Whether a lane's sixteen weights have
 // any is seen from the largest distance among them, a three-way maximum per four weights: eight layers of a 7B-shaped model, medians,
 // 1850 -> 1857 us (1897 with a two-way maximum, 1994 with the smallest magnitude that is not zero).
-#include "em_sorted.cuh"
+#include "em_cells.cuh"
 #include "lane32.cuh"
 
 namespace bof4 {
 
-constexpr int kCellDepth = 40 * 128;              // bit-pattern distances told apart: 40 binades
-constexpr int kCellRow = 2 * kCellDepth + 1;      // positive, negative, zero
-constexpr int kDeepExps = 88;                     // biased exponents of fp32 numbers up to 2^-40
-constexpr int kDeepCells = 128 * kCellRow;        // first deep cell: positive ones by exponent, then negative ones
-constexpr int kCells = kDeepCells + 2 * kDeepExps;
 constexpr int kCellCounts = 2 * kCellDepth + 2 * kDeepExps;  // counters of a unit: one magnitude, zeros left out
 constexpr int kMags = 32768;                      // magnitudes of a bf16 number
 constexpr int kCellBaseMax = 8192;                // bound on where a unit's counters begin in shared memory: behind the system's
@@ -40,30 +35,12 @@ constexpr int kCellBaseMax = 8192;                // bound on where a unit's cou
 constexpr int kCellThreads = 512;
 constexpr int kCellCtas = 3;                      // per SM
 constexpr int kOrderGroup = 8;                   // blocks that a thread of the ordering takes at a time
-constexpr int kCellScan = 2048;                   // cells per CTA of the items pass
-constexpr int kCellScans = (kCells + kCellScan - 1) / kCellScan;
 // Below, one sample per weight is cheaper.  20 iterations, MSE and MAE, one sample per weight against this way:
 // 2^20 weights 132 and 241 us against 151 and 236, 2^21 171 and 330 against 157 and 242.
 constexpr int64_t kCellsMinN = (int64_t)3 << 19;
 constexpr int kMagTiny = 48 * 128;                // |m| below 2^-79: subnormal weights within 40 binades
 
 bool cells_apply(int w_dtype, int64_t n) { return w_dtype == BOF4_BF16 && n >= kCellsMinN; }
-
-struct CellUnit {
-    uint32_t mag, first, count;  // bit pattern of |m|, first block in the ordered list, blocks
-};
-struct CellsWs {
-    uint32_t* hist;      // [kMags] blocks per magnitude
-    uint32_t* cursor;    // [kMags] next free position of the ordered list
-    uint32_t* scal;      // [0] units, [1] next unit, [2] largest magnitude of the short last blocks, [3] of all
-    uint32_t* scans;     // [kCellScans]
-    ulonglong2* acc;     // [kCells]
-    unsigned long long* acc_a;
-    CellUnit* units;
-    unsigned long long* order;  // [blocks] address, sign of the constant in bit 63
-    uint16_t* consts;           // [blocks]
-    SortWs sort;
-};
 
 constexpr int kMaxExtraUnits = 16 * kSMs;  // units beyond one per magnitude: blocks / unit size
 
@@ -89,12 +66,14 @@ static size_t cells_layout(void* base, int64_t n, int block_size, CellsWs* W)
     L.acc = reinterpret_cast<ulonglong2*>(take((size_t)kCells * 16));
     L.acc_a = reinterpret_cast<unsigned long long*>(take((size_t)kCells * 8));  // the four arrays above are cleared together
     L.cursor = reinterpret_cast<uint32_t*>(take((size_t)kMags * 4));
-    L.scans = reinterpret_cast<uint32_t*>(take((size_t)kCellScans * 4));
     L.units = reinterpret_cast<CellUnit*>(take((size_t)(kMags + kMaxExtraUnits) * sizeof(CellUnit)));
     L.order = reinterpret_cast<unsigned long long*>(take(blocks * 8));
     L.consts = reinterpret_cast<uint16_t*>(take(align_up(blocks, kOrderGroup) * 2));
-    char* rest = p ? p + off : nullptr;
-    off += sorted_layout(rest, kCells, true, &L.sort);
+    L.value_of = reinterpret_cast<uint16_t*>(take((size_t)(kCellFractions + kCellParts) * 2));
+    L.front = reinterpret_cast<double2*>(take((size_t)kCellBlocks * kCellBlock * 16));
+    L.front_a = reinterpret_cast<unsigned long long*>(take((size_t)kCellBlocks * kCellBlock * 8));
+    L.block = reinterpret_cast<CellBlock*>(take((size_t)kCellBlocks * sizeof(CellBlock)));
+    L.part_a = reinterpret_cast<unsigned long long*>(take((size_t)kCellPartsAll * 8));
     if (W) *W = L;
     return off;
 }
@@ -252,10 +231,18 @@ cells_blocks_kernel(const EmTensors T, const int64_t first_block, uint32_t* __re
 // the largest magnitude and the scale of the cell sums.  The magnitudes that most blocks have are neighbours (a binade
 // has 128), so they lie with different threads; with 32 neighbours to a thread one of them wrote most of the
 // units (2^26 weights 20 us against 7, 2^30 26 against 11).  The order of the magnitudes in the list is of no account.
+// The other CTAs put the fractions in order meanwhile.
 __global__ void __launch_bounds__(1024)
-cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __restrict__ head)
+cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric)
 {
     if (!after_previous()) return;
+    if (blockIdx.x) {
+        const uint32_t f = (blockIdx.x - 1) * kFractionThreads + threadIdx.x;
+        if (threadIdx.x >= kFractionThreads) return;
+        if (f < kCellFractions) W.value_of[fraction_rank(f >> 7, f & 127u)] = (uint16_t)f;
+        else W.value_of[f] = (uint16_t)fractions_below(f - kCellFractions);
+        return;
+    }
     __shared__ uint32_t s_blocks[32], s_units[32], s_top;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) s_top = W.scal[2];
@@ -306,8 +293,7 @@ cells_plan_kernel(const CellsWs W, uint32_t per_unit, int metric, uint32_t* __re
     }
     if (tid == 0) {
         W.scal[3] = s_top;
-        head[1] = s_top << 16;
-        *reinterpret_cast<double*>(head + 2) = cell_scale(s_top, metric);
+        *cells_scale(W) = cell_scale(s_top, metric);
     }
 }
 
@@ -606,7 +592,9 @@ cells_accumulate_kernel(const CellsWs W, int lanes_shift, int metric)
             if (v) {
                 s_cnt[k] = 0u;
                 seen += v;
-                cell_add(W, (k < 2 * kCellDepth ? row : (uint32_t)(kDeepCells - 2 * kCellDepth)) + (uint32_t)k, v, m, mae);
+                // (all of +-1 share a cell, whatever the significand)
+                const uint32_t first = k >= 2 * kCellDepth ? (uint32_t)(kDeepCells - 2 * kCellDepth) : k % kCellDepth ? row : 0u;
+                cell_add(W, first + (uint32_t)k, v, m, mae);
             }
         }
 #pragma unroll
@@ -617,7 +605,7 @@ cells_accumulate_kernel(const CellsWs W, int lanes_shift, int metric)
             for (int k = 1; k < kCellThreads / 32; ++k) seen += s_seen[k];
             const uint32_t zeros = pieces * 16u - seen;
             // an all-zero block has weight zero, except where every sample weighs one
-            if (zeros && (U.mag != 0u || metric >= 2)) cell_add(W, row + 2 * kCellDepth, zeros, m, mae);
+            if (zeros && (U.mag != 0u || metric >= 2)) cell_add(W, kZeroCell, zeros, m, mae);
         }
     }
 }
@@ -646,124 +634,16 @@ cells_tail_kernel(const EmTails Q, const CellsWs W, int metric, int add)
                 const uint32_t w = tiny ? scaled16(w0) : w0, d = ms - (w & 0x7fffu);
                 const bool deep = mag != 0u && d >= (uint32_t)kCellDepth && (w0 & 0x7fffu) != 0u;
                 const int at = deep ? deep_cell(w0, mag) : -1;
-                const uint32_t in_row = (mag == 0u || d >= (uint32_t)kCellDepth) ? 2u * kCellDepth : d + ((w & 0x8000u) ? kCellDepth : 0u);
-                cell_add(W, at >= 0 ? (uint32_t)(kDeepCells + at) : (mw.b - 128u) * (uint32_t)kCellRow + in_row, 1ull, mw, mae);
+                uint32_t cell = kZeroCell;
+                if (at >= 0) cell = (uint32_t)(kDeepCells + at);
+                else if (mag != 0u && d < (uint32_t)kCellDepth)
+                    cell = (d ? (mw.b - 128u) * (uint32_t)kCellRow : 0u) + d + ((w & 0x8000u) ? kCellDepth : 0u);
+                cell_add(W, cell, 1ull, mw, mae);
             }
         }
         __syncthreads();  // before the next block overwrites s_w
     }
 }
-
-// ---------------------------------------------------------------- items
-
-// Occupied cells per CTA of the items pass.  A cell of weight zero (|m| far below the largest) has no say.
-__global__ void __launch_bounds__(512)
-cells_scan_kernel(const CellsWs W)
-{
-    if (!after_previous()) return;
-    __shared__ uint32_t s_n[16];
-    const int tid = threadIdx.x;
-    uint32_t n = 0u;
-#pragma unroll
-    for (int k = 0; k < kCellScan / 512; ++k) {
-        const int c = blockIdx.x * kCellScan + k * 512 + tid;
-        if (c < kCells) {
-            const ulonglong2 v = W.acc[c];
-            n += (v.x | v.y) ? 1u : 0u;
-        }
-    }
-    n = __reduce_add_sync(kFull, n);
-    if ((tid & 31) == 0) s_n[tid >> 5] = n;
-    __syncthreads();
-    if (tid == 0) {
-        for (int k = 1; k < 16; ++k) n += s_n[k];
-        W.scans[blockIdx.x] = n;
-    }
-}
-
-// Writes the samples {x, cell} of the occupied cells in the order of the cells, and the sums of m^2 x^2 for
-// the error of the MSE metrics.
-__global__ void __launch_bounds__(512)
-cells_items_kernel(const CellsWs W)
-{
-    if (!after_previous()) return;
-    constexpr int PER = kCellScan / 512;
-    __shared__ uint32_t s_warp[16], s_before[16];
-    __shared__ double s_sum[16];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t before = 0u;
-    for (int k = tid; k < (int)blockIdx.x; k += 512) before += W.scans[k];
-    before = __reduce_add_sync(kFull, before);
-    if (lane == 0) s_before[warp] = before;
-    const double scale = *reinterpret_cast<const double*>(W.sort.n_items + 2);
-    const int c0 = blockIdx.x * kCellScan + tid * PER;
-    ulonglong2 v[PER];
-    uint32_t mine = 0u;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        v[k] = (c0 + k < kCells) ? W.acc[c0 + k] : make_ulonglong2(0ull, 0ull);
-        mine += (v[k].x | v[k].y) ? 1u : 0u;
-    }
-    uint32_t incl = mine;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t t = __shfl_up_sync(kFull, incl, off);
-        if (lane >= off) incl += t;
-    }
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    before = 0u;
-    for (int k = 0; k < 16; ++k) before += s_before[k] + (k < warp ? s_warp[k] : 0u);
-    uint32_t at = before + incl - mine;
-    double sum = 0.0;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        if (!(v[k].x | v[k].y)) continue;
-        const uint32_t cell = (uint32_t)(c0 + k), b = cell / kCellRow, r = cell % kCellRow;
-        float x = 0.0f;
-        if (cell >= (uint32_t)kDeepCells) {
-            const uint32_t at = cell - (uint32_t)kDeepCells, e = at % kDeepExps;
-            x = __uint_as_float((e ? e << 23 : 0x400000u) | (at >= (uint32_t)kDeepExps ? 0x80000000u : 0u));
-            const double e2 = (double)x;
-            sum += ((double)v[k].y * 18446744073709551616.0 + (double)v[k].x) * scale * e2 * e2;
-        } else if (r < 2u * kCellDepth) {
-            const bool neg = r >= (uint32_t)kCellDepth;
-            const uint32_t mb = 0x3f80u + b, wb = mb - (neg ? r - kCellDepth : r);
-            const float m = __uint_as_float(mb << 16), w = __uint_as_float(wb << 16);
-            x = __fdiv_rn(neg ? -w : w, m);
-            const double e = (double)x;
-            sum += ((double)v[k].y * 18446744073709551616.0 + (double)v[k].x) * scale * e * e;
-        }
-        W.sort.a[at++] = make_float2(x, __uint_as_float(cell));
-    }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
-    if (lane == 0) s_sum[warp] = sum;
-    __syncthreads();
-    if (tid == 0) {
-        for (int k = 1; k < 16; ++k) sum += s_sum[k];
-        reinterpret_cast<double*>(W.sort.counts)[blockIdx.x] = sum;  // folded by the next kernel
-        if (blockIdx.x == gridDim.x - 1) {
-            uint32_t n = before;  // of all earlier CTAs (warp 0 has added nothing of its own CTA)
-            for (int k = 0; k < 16; ++k) n += s_warp[k];
-            W.sort.n_items[0] = n;
-        }
-    }
-}
-
-// The CTAs' sums of squares into the slots that the iterations add up.
-__global__ void __launch_bounds__(320)
-cells_square_kernel(const CellsWs W)
-{
-    if (!after_previous()) return;
-    const double* part = reinterpret_cast<const double*>(W.sort.counts);
-    for (int k = threadIdx.x; k < kSortParts; k += blockDim.x) {
-        double a = 0.0;
-        for (int c = k; c < kCellScans; c += kSortParts) a += part[c];
-        W.sort.w2[k] = a;
-    }
-}
-static_assert((size_t)kCellScans * 8 <= (size_t)kSortGrid * 256 * 4, "partial sums fit the ordering passes' counters");
 
 // ---------------------------------------------------------------- host side
 
@@ -825,7 +705,7 @@ int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters
         return sg ? blocks_pass<true>(T, a.block_size, f, W, st) : blocks_pass<false>(T, a.block_size, f, W, st);
     }, &calls);
     if (rc) return rc;
-    launch_after(cells_plan_kernel, 1, 1024, 0, st, W, (uint32_t)unit_blocks(blocks, a.block_size), a.metric, W.sort.n_items);
+    launch_after(cells_plan_kernel, 1 + (kCellFractions + kCellParts) / kFractionThreads, 1024, 0, st, W, (uint32_t)unit_blocks(blocks, a.block_size), a.metric);
     BOF4_CUDA_TRY(cudaGetLastError());
     first = 0;
     rc = for_each_tensor_chunk(a, 1024 * kLW, [&](const EmTensors& T) -> int {
@@ -849,21 +729,14 @@ int cells_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters
     launch_after(cells_accumulate_kernel, kCellCtas * kSMs, kCellThreads, smem, st, W, shift, a.metric);
     BOF4_CUDA_TRY(cudaGetLastError());
     if ((rc = tails(1))) return rc;
-    launch_after(cells_scan_kernel, kCellScans, 512, 0, st, W);
-    launch_after(cells_items_kernel, kCellScans, 512, 0, st, W);
-    launch_after(cells_square_kernel, 1, 320, 0, st, W);
-    BOF4_CUDA_TRY(cudaGetLastError());
     SortFit F{};
-    F.acc = reinterpret_cast<const unsigned long long*>(W.acc);
-    F.acc_a = W.acc_a;
     F.metric = a.metric;
     F.n_total = a.n_total;
-    F.n_max = kCells;
     F.codebook = d_codebook;
     F.fixed_mask = fixed_mask;
     F.iters = iters;
     F.err_log = d_err_log;
-    return sorted_run(W.sort, F, st);
+    return cells_run(W, F, st);
 }
 
 }  // namespace bof4

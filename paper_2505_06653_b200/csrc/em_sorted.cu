@@ -7,7 +7,7 @@
 // the samples' order, the order of every sum and hence the result are reproducible.
 #include <type_traits>
 
-#include "em_sorted.cuh"
+#include "em_fit.cuh"
 
 namespace bof4 {
 
@@ -15,7 +15,7 @@ constexpr int kSortThreads = 1024;
 constexpr int kSortPerThread = 8;
 constexpr int kSortTile = kSortThreads * kSortPerThread;
 
-size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W)
+size_t sorted_layout(void* base, int64_t n, SortWs* W)
 {
     char* p = static_cast<char*>(base);
     size_t off = 0;
@@ -40,8 +40,6 @@ size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W)
     L.a = reinterpret_cast<float2*>(take((size_t)n * 8));
     L.b = reinterpret_cast<float2*>(take((size_t)n * 8));
     L.before = nullptr;
-    L.cell_s = cells ? reinterpret_cast<double*>(take((size_t)n * 8)) : nullptr;
-    L.cell_a = cells ? reinterpret_cast<unsigned long long*>(take((size_t)n * 8)) : nullptr;
     if (W) *W = L;
     return off;
 }
@@ -243,7 +241,7 @@ __device__ __forceinline__ void rank_in_warp(uint32_t* cnt, int lane, Digit digi
 // as they are added up: kept in registers over the barriers they spilled 90 bytes.)
 constexpr int kScatterSmem = kSortTile * 8;
 // Fits over so many samples, one per weight, stage them: the ordering of 2^20 takes 87 us instead of 92, of 2^23 298 instead of
-// 384, of 2^24 563 instead of 778, of 2^26 2030 instead of 3790.  Fewer (and cells, of which there are some 10^5) fill a tile in
+// 384, of 2^24 563 instead of 778, of 2^26 2030 instead of 3790.  Fewer fill a tile in
 // part, and the barriers cost what the stores save.  Staged and not, 40 iterations: 2^18 weights 140.8 and 138.7 us, 2^19 147.4
 // and 147.5, 3 * 2^18 152 and 155, 2^20 157 and 163.
 constexpr int64_t kStagedMin = 1 << 19;
@@ -375,34 +373,23 @@ sort_scatter_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ 
 
 // ---------------------------------------------------------------- sums of the bins
 
-// What a sample contributes.
-template <bool MAE, bool CELLS>
+// What a sample contributes; its payload is |m|.
+template <bool MAE>
 struct SampleWeight {
     uint32_t max_bits;
     bool unit;
-    double scale;                    // CELLS: undoes the fixed-point scale of the weights
-    const ulonglong2* acc;           // CELLS, by cell
-    const unsigned long long* acc_a;
-    // A direct sample's payload is its |m|; a cell's is its number.
     __device__ __forceinline__ void operator()(float2 it, double& s, unsigned long long& a) const
     {
         a = 0ull;
-        if (CELLS) {
-            const uint32_t cell = __float_as_uint(it.y);
-            const ulonglong2 v = acc[cell];
-            s = ((double)v.y * 18446744073709551616.0 + (double)v.x) * scale;
-            if (MAE) a = acc_a[cell];
-        } else {
-            const double m = (double)it.y;
-            s = MAE ? m : m * m;
-            if (MAE) a = unit ? 1ull : (unsigned long long)sort_fixed_weight(it.y, max_bits);
-        }
+        const double m = (double)it.y;
+        s = MAE ? m : m * m;
+        if (MAE) a = unit ? 1ull : (unsigned long long)sort_fixed_weight(it.y, max_bits);
     }
 };
 
 // First sample of every bin: sample i is the first of all bins behind the one of sample i - 1 up to its own; behind
 // the last sample come all bins that are left, which are all there are where no sample has a weight (bf16 zeros).
-// tops, or NULL: the largest constants of the samples' CTAs, of which the last CTA makes one.
+// tops: the largest constants of the samples' CTAs, of which the last CTA makes one.
 __global__ void __launch_bounds__(256)
 sort_start_kernel(const float2* __restrict__ items, uint32_t* __restrict__ head, const uint32_t* __restrict__ tops,
                   uint32_t* __restrict__ start)
@@ -410,7 +397,7 @@ sort_start_kernel(const float2* __restrict__ items, uint32_t* __restrict__ head,
     if (!after_previous()) return;
     const uint32_t n = *head;
     if (blockIdx.x == gridDim.x - 1) {
-        if (!tops || threadIdx.x >= 32) return;
+        if (threadIdx.x >= 32) return;
         uint32_t top = 0u;
 #pragma unroll
         for (int k = 0; k < kSortParts; k += 32) top = max(top, k + threadIdx.x < kSortParts ? tops[k + threadIdx.x] : 0u);
@@ -476,7 +463,7 @@ struct WindowScratch {
 };
 template <bool MAE>
 __global__ void __launch_bounds__(kSortThreads)
-sort_windows_kernel(const SortWs W, SampleWeight<MAE, false> weight)
+sort_windows_kernel(const SortWs W, SampleWeight<MAE> weight)
 {
     if (!after_previous()) return;
     if (W.n_items[4] == 0u) return;
@@ -572,7 +559,7 @@ constexpr int kWindowsPerLane = 4;
 
 // Sums of the samples of a window in front of position i (`first`: the window's first sample).
 template <bool MAE>
-__device__ __forceinline__ SortSums sums_before(const SortWs& W, const SampleWeight<MAE, false>& weight, uint32_t first, uint32_t i)
+__device__ __forceinline__ SortSums sums_before(const SortWs& W, const SampleWeight<MAE>& weight, uint32_t first, uint32_t i)
 {
     SortSums t{0.0, 0.0, 0ull};
     if (i <= first) return t;
@@ -592,7 +579,7 @@ __device__ __forceinline__ SortSums sums_before(const SortWs& W, const SampleWei
 
 // This lane's share of the samples of a crowded bin, from ... to - 1, with p <= x < q; the warp's lanes together have all.
 template <bool MAE>
-__device__ __noinline__ void crowded_sums(const SortWs& W, const SampleWeight<MAE, false>& weight, uint32_t from, uint32_t to, float p,
+__device__ __noinline__ void crowded_sums(const SortWs& W, const SampleWeight<MAE>& weight, uint32_t from, uint32_t to, float p,
                                           float q, SortSums& t)
 {
     constexpr int U = kWindowsPerLane;
@@ -630,15 +617,14 @@ __device__ __noinline__ void crowded_sums(const SortWs& W, const SampleWeight<MA
 // A run that lies inside the chunk is a bin's sum; parts of runs that cross the chunk's edges go to
 // lead / trail and are put together by sort_group_kernel.  The work is even whatever the distribution (the bins
 // of x = +-1 hold 1 / I of the data; a bin of small data is mostly empty).
-template <bool MAE, bool CELLS>
+template <bool MAE>
 __global__ void __launch_bounds__(256)
-sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
+sort_sums_kernel(const SortWs W, SampleWeight<MAE> weight)
 {
     if (!after_previous()) return;
     constexpr int STEPS = kSortChunk / 32, kNone = 1 << 20;
     const uint32_t n = W.n_items[0];
     weight.max_bits = W.n_items[1];
-    if (CELLS) weight.scale = *reinterpret_cast<const double*>(W.n_items + 2);
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * 8u;
     for (uint32_t c = blockIdx.x * 8u + (threadIdx.x >> 5); (uint64_t)c * kSortChunk < n; c += warps) {
@@ -661,16 +647,6 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
                 key[k] = sort_bin(it[k].x);
                 weight(it[k], v[k].s, v[k].a);
                 v[k].sx = v[k].s * (double)it[k].x;
-            }
-        }
-        if (CELLS) {
-#pragma unroll
-            for (int k = 0; k < STEPS; ++k) {
-                const uint32_t i = lo + 32 * k + lane;
-                if (i < hi) {
-                    W.cell_s[i] = v[k].s;
-                    if (MAE) W.cell_a[i] = v[k].a;
-                }
             }
         }
         SortSums open{0.0, 0.0, 0ull};  // the run that reaches the end of the steps so far (the same in all lanes)
@@ -704,7 +680,7 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE, CELLS> weight)
             early = early && heads == 0u;
         }
         // a chunk inside one bin: a crowded one has many, the first of them says so
-        if (!CELLS && early && open_key == before && lane == 0 && !one_value_bin(before)) {
+        if (early && open_key == before && lane == 0 && !one_value_bin(before)) {
             const uint32_t s = W.start[before];
             if (lo - s <= kSortChunk && W.start[before + 1] - s > kSortCrowd) W.n_items[4] = 1u;
         }
@@ -794,23 +770,13 @@ sort_group_kernel(const SortWs W)
 
 // ---------------------------------------------------------------- all iterations, squared error
 //
-// One CTA.  An iteration is a chain of latencies, so it is kept short: warp w adds up what lies below threshold w, the bins in
-// front of its bin as two sums that are at hand (whole groups, bins of its group) and the samples of its bin, and a region is
-// the difference of two such sums.  Behind the one barrier of an iteration every warp works the levels out for itself (a
-// lane each) and goes straight on to its next threshold; the sixteenth warp has no threshold and writes the error meanwhile.
-// The first samples of all bins are in shared memory (16 bits beside the group's first), which leaves one access to L2 in the
-// chain: 1.12 us an iteration (2^20 fp32 and 2^26 bf16 weights; 1.60 with cuts found by one warp, whole groups added up between them and three
-// barriers), 3.5 for 2^24 fp32 weights (3.9).  Of its 2200 cycles the bin takes 130, its first sample 220, the samples 430 or 820, by
-// where in L2 they are, their reduction 230, the barrier and what it waits for 200, the differences 300 and the quotients with
-// the test of the sums 330.  (The next iteration's samples requested ahead, by the last steps of the threshold: 1 to 13 % slower.)
-//
-// Sums of whole groups are kept in two doubles each, so that their difference is as good as adding the region up; the rest
-// (bins and samples beside whole groups, at most a group's weight) is rounded once to a double.  A region that
-// is very light beside its neighbours, or stands beside sums that are not finite, is added up by itself (region_sums).
-//
-// When an iteration leaves every level unchanged the remaining ones would repeat it bit for bit: their entries
-// of the error log are filled in and the loop ends.
-constexpr int kMseThreads = 32 * kLevels;
+// What lies below a threshold (em_fit.cuh): the groups in front of its bin's, in shared memory, the bins of the group in front of it
+// (one load), and the samples of its bin.  The first samples of all bins are in shared memory (16 bits beside the group's first),
+// which leaves one access to L2 in the chain: 1.12 us an iteration over 2^20 fp32 weights (1.60 with cuts found by one warp, whole
+// groups added up between them and three barriers), 3.5 over 2^24 (3.9).  Of its 2200 cycles the bin takes 130, its first sample 220,
+// the samples 430 or 820, by where in L2 they are, their reduction 230, the barrier and what it waits for 200, the differences 300
+// and the quotients with the test of the sums 330.  (The next iteration's samples requested ahead, by the last steps of the
+// threshold: 1 to 13 % slower.)
 constexpr int kMseLow = (kSortGroups + 1) * 16;      // shared memory: sums of the groups in front, high and low halves,
 constexpr int kMseOff = 2 * kMseLow;                 // first samples of the bins,
 constexpr int kMseFirst = kMseOff + kSortBins * 2 + 16;  // (and the end) of the groups
@@ -828,26 +794,9 @@ __device__ __forceinline__ void copy_starts(const SortWs& W, uint16_t* s_off, ui
     for (int k = threadIdx.x; k < kSortBins / 8; k += blockDim.x) copy(s_off + 8 * k, W.off + 8 * k, std::integral_constant<int, 16>{});
     for (int k = threadIdx.x; k <= kSortGroups; k += blockDim.x) copy(s_first + k, W.first + k, std::integral_constant<int, 4>{});
 }
-__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// A sum in two doubles, high + low with |low| at most half a unit of high.
-struct TwoSum {
-    double h, l;
-};
-__device__ __forceinline__ TwoSum two_add(const TwoSum& a, const TwoSum& b)
-{
-    const double s = a.h + b.h, t = s - a.h;
-    const double e = ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l);
-    const double h = s + e;
-    return TwoSum{h, e - (h - s)};
-}
-__device__ __forceinline__ TwoSum two_shfl_up(const TwoSum& a, int off)
-{
-    return TwoSum{__shfl_up_sync(kFull, a.h, off), __shfl_up_sync(kFull, a.l, off)};
-}
 
 // Sums of the samples with p <= x < q, by a warp; the result is the same in all lanes.
-template <bool CELLS, bool CROWDED>
+template <bool CROWDED>
 __device__ __noinline__ double2 region_sums(const SortWs& W, float p, float q)
 {
     const int lane = threadIdx.x & 31;
@@ -867,13 +816,13 @@ __device__ __noinline__ double2 region_sums(const SortWs& W, float p, float q)
         }
         const uint32_t from = __ldg(W.start + b), to = __ldg(W.start + b + 1);
         if (CROWDED && to - from > kSortCrowd) {
-            crowded_sums<false>(W, SampleWeight<false, false>{}, from, to, p, q, t);
+            crowded_sums<false>(W, SampleWeight<false>{}, from, to, p, q, t);
             return;
         }
         for (uint32_t i = from + lane; i < to; i += 32) {
             const float2 it = __ldg(W.b + i);
             if (!(it.x >= p && it.x < q)) continue;
-            const double m = (double)it.y, s = CELLS ? __ldg(W.cell_s + i) : m * m;
+            const double m = (double)it.y, s = m * m;
             t.s += s;
             t.sx += s * (double)it.x;
         }
@@ -887,7 +836,7 @@ __device__ __noinline__ double2 region_sums(const SortWs& W, float p, float q)
 }
 
 // CROWDED: a copy of the loop that also knows crowded bins.  Apart, because the calls in it cost the other one registers.
-template <bool CELLS, bool CROWDED>
+template <bool CROWDED>
 __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
 {
     extern __shared__ __align__(16) unsigned char s_fit[];
@@ -907,7 +856,7 @@ __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
     copy_starts(W, s_off, s_first);
     // running sums of the groups, four to a thread
     {
-        constexpr int PER = kSortGroups / kMseThreads;
+        constexpr int PER = kSortGroups / kFitThreads;
         TwoSum s[PER], x[PER];
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
@@ -939,7 +888,7 @@ __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
         rx = two_add(TwoSum{__shfl_sync(kFull, wx.h, 31), __shfl_sync(kFull, wx.l, 31)}, rx);
 #pragma unroll
         for (int k = 0; k <= PER; ++k) {
-            if (k == PER && tid < kMseThreads - 1) break;  // behind the last group: everything
+            if (k == PER && tid < kFitThreads - 1) break;  // behind the last group: everything
             s_high[tid * PER + k] = make_double2(rs.h, rx.h);
             s_low[tid * PER + k] = make_double2(rs.l, rx.l);
             if (k < PER) rs = two_add(rs, s[k]), rx = two_add(rx, x[k]);
@@ -1016,7 +965,7 @@ __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
         uint32_t below = 0u;
         if (CROWDED && to - from > kSortCrowd) {
             SortSums in{0.0, 0.0, 0ull};
-            crowded_sums<false>(W, SampleWeight<false, false>{}, from, to, -inf, p, in);
+            crowded_sums<false>(W, SampleWeight<false>{}, from, to, -inf, p, in);
             ls = in.s, lx = in.sx;
             below = lane == 0 ? ~from - (uint32_t)warp : 0u;  // not counted: no two thresholds alike
         } else {
@@ -1024,17 +973,15 @@ __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
             auto add = [&](auto count, uint32_t i) {
                 constexpr int U = decltype(count)::value;
                 float2 it[U];
-                double s[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const uint32_t j = i + 32 * u < to ? i + 32 * u : 0u;
                     it[u] = __ldg(W.b + j);
-                    s[u] = CELLS ? __ldg(W.cell_s + j) : 0.0;
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const bool in = i + 32 * u < to && it[u].x < p;
-                    const double x = (double)it[u].x, m = (double)it[u].y, sv = CELLS ? s[u] : m * m, xv = sv * x;
+                    const double x = (double)it[u].x, m = (double)it[u].y, sv = m * m, xv = sv * x;
                     ls += in ? sv : 0.0;
                     lx += in ? xv : 0.0;
                     below += in ? 1u : 0u;
@@ -1065,18 +1012,13 @@ __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
         const double s1 = ((h1.y - h0.y) + (l1.y - l0.y)) + (r1.y - r0.y);
         float moved = (float)(s1 / s0);
         const bool empty = __float_as_uint(c0.y) == __float_as_uint(c1.y);
-        // Too small beside what was rounded (2^-20 of it) or the groups in front (2^-50), negative, or not finite: by the upper
-        // halves of the doubles, whose exponents begin at bit 20.
-        auto top = [](double d) { return __double2hiint(d) & 0x7fffffff; };
-        const int least0 = max(max(top(r0.x), top(r1.x)) - (20 << 20), top(h1.x) - (50 << 20)), least1 = max(top(r0.y), top(r1.y)) - (20 << 20);
-        const int t0 = __double2hiint(s0), t1 = top(s1);
-        const bool light = !empty && (t0 < max(least0, 0) || t1 < least1 || max(t0, t1) >= 0x7ff00000);
+        const bool light = !empty && too_rough(s0, s1, r0, r1, h1.x);
         const unsigned by_itself = __ballot_sync(kFull, light);
         if (stop <= iter) break;
         if (by_itself & 3u) {
             for (int k = 0; k < 2; ++k) {
                 if (!((by_itself >> k) & 1u)) continue;
-                const double2 t = region_sums<CELLS, CROWDED>(W, __shfl_sync(kFull, c0.x, k), __shfl_sync(kFull, c1.x, k));
+                const double2 t = region_sums<CROWDED>(W, __shfl_sync(kFull, c0.x, k), __shfl_sync(kFull, c1.x, k));
                 if ((lane & 1) == k) s0 = t.x, moved = (float)(t.y / t.x);
             }
         }
@@ -1087,13 +1029,12 @@ __device__ __forceinline__ void fit_mse(const SortWs& W, const SortFit& F)
         if (!fixed) F.codebook[mine] = lv;
 }
 
-template <bool CELLS>
-__global__ void __launch_bounds__(kMseThreads, 1)
+__global__ void __launch_bounds__(kFitThreads, 1)
 sort_fit_mse_kernel(const SortWs W, const SortFit F)
 {
     if (!after_previous()) return;
-    if (!CELLS && W.n_items[4] != 0u) fit_mse<CELLS, !CELLS>(W, F);
-    else fit_mse<CELLS, false>(W, F);
+    if (W.n_items[4] != 0u) fit_mse<true>(W, F);
+    else fit_mse<false>(W, F);
 }
 
 // ---------------------------------------------------------------- all iterations, absolute error
@@ -1107,23 +1048,10 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v)
     return (unsigned long long)lo + ((unsigned long long)mi << 27) + ((unsigned long long)hi << 54);
 }
 
-//
-// One CTA, and as for the squared error what lies below a threshold is one sum that its own warp forms (whole groups and bins from
-// running sums, the samples of its bin).  Behind a barrier warp l looks for the median of region l: the weight at which half of
-// the region is reached is a place in the running sums of all groups (shared memory, 64 entries a step), then of the group's bins
-// (one load), then among the samples of one bin.  A second barrier, and the levels are there.  Eight more warps add up
-// beside this what lies below each level, which the error of the iteration needs and nothing else, and warp 15, which has no
-// threshold, writes the error of the iteration before.  The weights are integers, so a region is exactly the difference of two sums.
-// When an iteration leaves every level unchanged the remaining ones would repeat it bit for bit: their entries of the
-// error log are filled in and the loop ends.
-// An iteration over eight layers of a 7B-shaped model or 2^26 bf16 weights 5.6 -> 2.5 us, over 2^20 fp32 weights 6.5 -> 3.1, over 2^24
-// 33 -> 14 (before: two warps to a region, whole groups added up and searched one after the other, cut bins first).  Bound by its
-// chain: three loads from L2 of 430 or 820 cycles each, the reductions, two barriers; over 2^24 weights by the passes over the 500 samples
-// of a bin (of up to 64 samples every lane adds up what is not behind its own, in one pass: 2^26 bf16 3.0 -> 2.5, 2^20 fp32 3.75 -> 3.1).
 
 // The sample of a crowded bin, among those with p <= x < q, at which twice the weight `before` and up to it reaches `total`;
 // false, and `before` advanced past them, where it lies behind them.  Called by a whole warp.
-__device__ __noinline__ bool crowded_median(const SortWs& W, const SampleWeight<true, false>& weight, uint32_t from, uint32_t to, float p,
+__device__ __noinline__ bool crowded_median(const SortWs& W, const SampleWeight<true>& weight, uint32_t from, uint32_t to, float p,
                                             float q, unsigned long long total, unsigned long long& before, float& median)
 {
     constexpr int U = kWindowsPerLane;
@@ -1184,138 +1112,32 @@ __device__ __noinline__ bool crowded_median(const SortWs& W, const SampleWeight<
     return true;
 }
 
-constexpr int kMaeScan = 32 * kLevels, kMaeThreads = kMaeScan + 32 * kLevels / 2;
-constexpr int kMaeSums = ((kSortGroups + 1) * 8 + 15) / 16 * 16;  // shared memory: what lies in front of the groups: fixed-point weights, {s, sx},
-constexpr int kMaeOff = kMaeSums + (kSortGroups + 1) * 16;      // first samples of the bins,
-constexpr int kMaeFirst = kMaeOff + kSortBins * 2 + 16;         // (and the end) of the groups
-constexpr int kMaeSmem = kMaeFirst + (kSortGroups + 1) * 4;
+constexpr int kFitMaeThreads = 2 * kFitThreads;  // a warp per threshold and level, as many for the error
 
-// CROWDED: the kernel for data with crowded bins.  Both are launched, the flag of such bins tells which one runs: with both
-// loops in one kernel 2^22 fp32 weights, 12 iterations, took 299 us against 293.5, 2^20 153.8 against 152.4.
-template <bool CELLS, bool CROWDED>
-__global__ void __launch_bounds__(kMaeThreads, 1)
-sort_fit_mae_kernel(const SortWs W, const SortFit F)
+// Behind a barrier warp l looks for the median of region l: the first sample, in the order of x, with which the weight reaches half
+// of the region's.  The weights are integers, so a region is exactly the difference of two sums.  A second barrier, and the levels
+// are there.  Sixteen more warps add up beside this what the error of the iteration needs, and warp 15, which has no threshold, writes
+// the error of the iteration before.
+//
+// The source, by a warp, results the same in all lanes:  weight(v): of what lies below v;  sums(v): {s, sx} of what lies below v;
+//              median(goal): the first sample with which the weight of all samples from the first on reaches the goal
+struct FitMaeShared {
+    unsigned long long below[2][kLevels + 1];  // weight below threshold k - 1; entry 0: nothing, entry 16: everything
+    float level[2][kLevels];
+    double err[2][2 * kLevels];                // parts of the error: the thresholds' and the levels'
+    int stop;
+};
+template <class Source>
+__device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, double2 everything, unsigned long long weight, const SortFit& F)
 {
-    if (!after_previous()) return;
-    if (!CELLS && (W.n_items[4] != 0u) != CROWDED) return;
-    extern __shared__ __align__(16) unsigned char s_fit[];
-    unsigned long long* const s_a = reinterpret_cast<unsigned long long*>(s_fit);
-    double2* const s_sums = reinterpret_cast<double2*>(s_fit + kMaeSums);
-    uint16_t* const s_off = reinterpret_cast<uint16_t*>(s_fit + kMaeOff);
-    uint32_t* const s_first = reinterpret_cast<uint32_t*>(s_fit + kMaeFirst);
-    __shared__ unsigned long long s_below[2][kLevels + 1];  // fixed-point weight below threshold k - 1; entry 0: nothing, entry 16: everything
-    __shared__ float s_level[2][kLevels];
-    __shared__ double s_err[2][2 * kLevels];  // parts of the error: the thresholds' and the levels'
-    __shared__ SortSums s_warp[kLevels];
-    __shared__ int s_stop;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    SampleWeight<true, false> weight;
-    weight.max_bits = W.n_items[1];
-    weight.unit = F.metric >= 2;
-    if (tid == 0) s_stop = 0, s_off[kSortBins] = 0u;
-    copy_starts(W, s_off, s_first);
-    if (tid < kLevels) s_level[0][tid] = F.codebook[tid];
-    {  // running sums of the groups, four to a thread of the first warps
-        constexpr int PER = kSortGroups / kMaeScan;
-        const bool has = warp < kLevels;
-        SortSums g[PER], t{0.0, 0.0, 0ull};
-#pragma unroll
-        for (int k = 0; k < PER; ++k) g[k] = W.group[(has ? tid : 0) * PER + k];
-#pragma unroll
-        for (int k = 0; k < PER; ++k) sums_add(t, g[k]);
-        auto scan = [&](SortSums& v) {  // inclusive, over the warp
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const SortSums u{__shfl_up_sync(kFull, v.s, off), __shfl_up_sync(kFull, v.sx, off), __shfl_up_sync(kFull, v.a, off)};
-                if (lane >= off) sums_add(v, u);
-            }
-        };
-        scan(t);
-        if (lane == 31 && has) s_warp[warp] = t;
-        __syncthreads();
-        SortSums w{0.0, 0.0, 0ull};
-        if (lane < warp && lane < kLevels) w = s_warp[lane];
-        scan(w);
-        SortSums run{__shfl_up_sync(kFull, t.s, 1), __shfl_up_sync(kFull, t.sx, 1), __shfl_up_sync(kFull, t.a, 1)};
-        if (lane == 0) run = SortSums{0.0, 0.0, 0ull};
-        sums_add(run, SortSums{__shfl_sync(kFull, w.s, 31), __shfl_sync(kFull, w.sx, 31), __shfl_sync(kFull, w.a, 31)});
-#pragma unroll
-        for (int k = 0; k <= PER; ++k) {
-            if (!has || (k == PER && tid < kMaeScan - 1)) break;  // behind the last group: everything
-            s_a[tid * PER + k] = run.a;
-            s_sums[tid * PER + k] = make_double2(run.s, run.sx);
-            if (k < PER) sums_add(run, g[k]);
-        }
-    }
-    copies_done();
+    if (tid < 2) S.below[tid][0] = 0ull, S.below[tid][kLevels] = weight;
+    if (tid == 0) S.stop = 0;
+    if (tid < kLevels) S.level[0][tid] = F.codebook[tid];
     __syncthreads();
-    if (tid < 2) s_below[tid][0] = 0ull, s_below[tid][kLevels] = s_a[kSortGroups];
-    auto start_of = [&](int b) -> uint32_t {  // first sample of bin b <= kSortBins
-        const uint32_t o = s_off[b], f = s_first[b / kSortGroup];
-        return o == kFarBin ? __ldg(W.start + b) : f + o;
-    };
-    auto use = [&](uint32_t i, float2 it, double& s, unsigned long long& a) {
-        if (CELLS) {
-            s = __ldg(W.cell_s + i);
-            a = __ldg(W.cell_a + i);
-        } else {
-            weight(it, s, a);
-        }
-    };
-    // What lies below v, less the whole groups in front of the one that is returned: this lane's share.
-    auto below = [&](float v, SortSums& t) -> int {
-        const int b = sort_bin(v);
-        const bool one = one_value_bin(b);                        // in or out as a whole
-        const int at = (one && value_of_bin(b) < v) ? b + 1 : b;  // whole bins in front of this one
-        const uint32_t from = start_of(at), to = one ? from : start_of(b + 1);
-        t = SortSums{0.0, 0.0, 0ull};
-        const unsigned long long pre = __ldg(reinterpret_cast<const unsigned long long*>(W.pre + min(at, kSortBins - 1)) + (lane < 3 ? lane : 0));
-        if (CROWDED && to - from > kSortCrowd) {
-            crowded_sums<true>(W, weight, from, to, -__int_as_float(0x7f800000), v, t);
-        } else {
-            auto add = [&](auto count, uint32_t i) {  // 64 samples at once, which is all of most bins, then 128
-                constexpr int U = decltype(count)::value;
-                float2 it[U];
-                double s[U];
-                unsigned long long a[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const uint32_t j = i + 32 * u < to ? i + 32 * u : 0u;
-                    it[u] = __ldg(W.b + j);
-                    if (CELLS) use(j, it[u], s[u], a[u]);
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (!CELLS) use(i, it[u], s[u], a[u]);
-                    const bool in = i + 32 * u < to && it[u].x < v;
-                    const double sx = s[u] * (double)it[u].x;
-                    t.s += in ? s[u] : 0.0;
-                    t.sx += in ? sx : 0.0;
-                    t.a += in ? a[u] : 0ull;
-                }
-            };
-            add(std::integral_constant<int, 2>{}, from + lane);
-            for (uint32_t i = from + 64; i < to; i += 128) add(std::integral_constant<int, 4>{}, i + lane);
-        }
-        __syncwarp();
-        if (at < kSortBins) {
-            if (lane == 0) t.s += __longlong_as_double((long long)pre);
-            if (lane == 1) t.sx += __longlong_as_double((long long)pre);
-            if (lane == 2) t.a += pre;
-        }
-        return at / kSortGroup;
-    };
-    // the lanes' shares of two sums together: {s, sx} in all lanes
-    auto both = [&](double s, double x) -> double2 {
-        const bool h = lane & 16;
-        double v = (h ? x : s) + __shfl_xor_sync(kFull, h ? s : x, 16);
-#pragma unroll
-        for (int off = 8; off; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
-        return make_double2(__shfl_sync(kFull, v, 0), __shfl_sync(kFull, v, 16));
-    };
-    // the error of iteration `at`, by warp 15: it has no threshold
+    // the error of iteration `at`, by warp 15
     auto error_of = [&](int at) {
-        double err = s_err[at & 1][lane];
+        double err = S.err[at & 1][lane];
 #pragma unroll
         for (int off = 16; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
         err = fmax(err, 0.0) / (double)F.n_total;
@@ -1324,236 +1146,322 @@ sort_fit_mae_kernel(const SortWs W, const SortFit F)
     };
     int iter = 0;
     if (warp >= kLevels) {
-        // ---- the levels' parts of the error, two levels to a warp, beside the others' search for the next ones
-        float known[2];
-        double part[2];
+        // ---- the error's parts of a threshold and of a level, beside the others' search for the next levels
+        const int l = warp - kLevels;
+        float known = 0.0f;
+        double part = 0.0;
         for (; iter < F.iters; ++iter) {
             const int set = iter & 1;
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int l = 2 * (warp - kLevels) + k;
-                const float lv = s_level[set][l];
-                if (iter == 0 || __float_as_uint(lv) != __float_as_uint(known[k])) {
-                    SortSums t;
-                    const int g = below(lv, t);
-                    const double2 r = both(t.s, t.sx), p = s_sums[g];
-                    known[k] = lv;
-                    part[k] = 2.0 * ((double)lv * (r.x + p.x) - (r.y + p.y));
-                }
-                if (lane == 0) s_err[set][kLevels + l] = part[k];
-                __syncthreads();
-                if (k == 0 && s_stop) return;
+            const float lv = S.level[set][l];
+            if (l < kLevels - 1) {
+                const float above = S.level[set][l + 1];
+                const double2 p = source.sums(__fmul_rn(__fadd_rn(lv, above), 0.5f));
+                if (lane == 0) S.err[set][l] = 2.0 * p.y - ((double)lv + (double)above) * p.x;
+            } else if (lane == 0) {
+                S.err[set][l] = everything.y - (double)lv * everything.x;
             }
+            __syncthreads();
+            if (S.stop) return;
+            if (iter == 0 || __float_as_uint(lv) != __float_as_uint(known)) {
+                const double2 p = source.sums(lv);
+                known = lv;
+                part = 2.0 * ((double)lv * p.x - p.y);
+            }
+            if (lane == 0) S.err[set][kLevels + l] = part;
+            __syncthreads();
         }
         return;
     }
     // ---- warp w: threshold w and level w
     const bool fixed = (F.fixed_mask >> warp) & 1u, cuts = warp < kLevels - 1;
-    float lv = s_level[0][warp];
+    float lv = S.level[0][warp];
     for (; iter < F.iters; ++iter) {
         const int set = iter & 1;
-        SortSums t{0.0, 0.0, 0ull};
         float above = 0.0f;  // the next level
-        int group = 0;
         if (cuts) {
-            above = s_level[set][warp + 1];
-            group = below(__fmul_rn(__fadd_rn(lv, above), 0.5f), t);
-            const unsigned long long a = warp_sum64(t.a) + s_a[group];
-            if (lane == 0) s_below[set][warp + 1] = a;
+            above = S.level[set][warp + 1];
+            const unsigned long long a = source.weight(__fmul_rn(__fadd_rn(lv, above), 0.5f));
+            if (lane == 0) S.below[set][warp + 1] = a;
         } else {
             if (iter) {
                 const double err = error_of(iter - 1);
                 const int l = lane & (kLevels - 1);
                 // no level has moved: the remaining iterations would repeat this one bit for bit
-                if (__all_sync(kFull, __float_as_uint(s_level[set][l]) == __float_as_uint(s_level[set ^ 1][l]))) {
-                    if (lane == 0) s_stop = 1;
+                if (__all_sync(kFull, __float_as_uint(S.level[set][l]) == __float_as_uint(S.level[set ^ 1][l]))) {
+                    if (lane == 0) S.stop = 1;
                     if (F.err_log)
                         for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = err;
                 }
             }
         }
         __syncthreads();
-        if (s_stop) break;
-        // The median of the region: the first sample, in the order of x, with which the weight reaches half.
-        const unsigned long long a0 = s_below[set][warp], a1 = s_below[set][warp + 1];
-        const float from_left = warp ? s_level[set][warp - 1] : 0.0f;
+        if (S.stop) break;
+        const unsigned long long a0 = S.below[set][warp], a1 = S.below[set][warp + 1];
+        const float from_left = warp ? S.level[set][warp - 1] : 0.0f;
         // (levels that do not ascend have regions without samples)
         const bool some = a1 != a0 && !(warp && cuts && __fadd_rn(from_left, lv) * 0.5f > __fadd_rn(lv, above) * 0.5f);
-        const bool search = some && !fixed;
-        const unsigned long long goal = a0 + (a1 - a0) - (a1 - a0) / 2ull;
-        int g = 0;
-        SortSums pre{0.0, 0.0, 0ull};
-        if (search) {
-            // the last group in front of which there is less than the goal: 32 groups of 64, then one of 64
-            int c = __popc(__ballot_sync(kFull, s_a[64 * (lane + 1)] < goal));
-            const unsigned long long u = s_a[64 * c + 1 + lane], v = s_a[64 * c + 33 + lane];
-            g = 64 * c + __popc(__ballot_sync(kFull, u < goal)) + __popc(__ballot_sync(kFull, v < goal));
-            pre.a = __ldg(&W.pre[g * kSortGroup + lane].a);
-        }
-        {  // beside the search: the threshold's part of the error (the last warp: that of everything)
-            const double2 s = cuts ? both(t.s, t.sx) : s_sums[kSortGroups], p = cuts ? s_sums[group] : make_double2(0.0, 0.0);
-            double err = (s.y + p.y) - (double)lv * (s.x + p.x);
-            if (cuts) err -= (double)above * (s.x + p.x) - (s.y + p.y);
-            if (lane == 0) s_err[set][warp] = err;
-        }
-        if (search) {
-            const unsigned long long before = s_a[g];
-            const int in = __popc(__ballot_sync(kFull, before + pre.a < goal)) - 1, b = g * kSortGroup + in;
-            const unsigned long long front = before + __shfl_sync(kFull, pre.a, in), need = goal - front;
-            if (one_value_bin(b)) {
-                lv = value_of_bin(b);
-            } else {
-                const uint32_t s0 = start_of(b), e = start_of(b + 1);
-                if (CROWDED && e - s0 > kSortCrowd) {
-                    unsigned long long none = 0ull;
-                    const float inf = __int_as_float(0x7f800000);
-                    crowded_median(W, weight, s0, e, -inf, inf, 2ull * need, none, lv);
-                } else {
-                    auto get = [&](uint32_t i, uint32_t& k, unsigned long long& a) {
-                        const uint32_t j = i < e ? i : s0;
-                        const float2 it = __ldg(W.b + j);
-                        double s;
-                        use(j, it, s, a);
-                        k = i < e ? sort_key(it.x) : 0xffffffffu;
-                        a = i < e ? a : 0ull;
-                    };
-                    // Few samples: one or two to a lane, which adds up for each all those that are not behind it.
-                    auto among = [&](auto count) {
-                        constexpr int N = decltype(count)::value;
-                        using Weight = typename std::conditional<CELLS, unsigned long long, uint32_t>::type;  // (31 bits, one sample per weight)
-                        uint32_t key[N], first = 0xffffffffu;
-                        Weight mine[N];
-                        unsigned long long a, sum[N];
-#pragma unroll
-                        for (int r = 0; r < N; ++r) {
-                            get(s0 + 32 * r + lane, key[r], a);
-                            mine[r] = (Weight)a;
-                            sum[r] = 0ull;
-                        }
-#pragma unroll
-                        for (int r = 0; r < N; ++r) {
-                            const int here = min((int)(e - s0) - 32 * r, 32);
-#pragma unroll 4
-                            for (int j = 0; j < here; ++j) {
-                                const uint32_t k = __shfl_sync(kFull, key[r], j);
-                                const Weight w = __shfl_sync(kFull, mine[r], j);
-#pragma unroll
-                                for (int q = 0; q < N; ++q) sum[q] += k <= key[q] ? w : 0;
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < N; ++q)
-                            if (sum[q] >= need) first = min(first, key[q]);  // (no sample: the last key of all)
-                        lv = sort_key_value(__reduce_min_sync(kFull, first));
-                    };
-                    if (e - s0 <= 32u) {
-                        among(std::integral_constant<int, 1>{});
-                    } else if (e - s0 <= 64u) {
-                        among(std::integral_constant<int, 2>{});
-                    } else {
-                        // The goal is reached at one of the keys k0 ... k1 of the bin's samples; c0 of the bin's weight lies
-                        // below k0, c1 up to k1.  The next key to split at is where even weights would put it (every third
-                        // time the middle), and the ends move to samples: a handful of steps, where halving the keys
-                        // takes one per bit in which they differ.
-                        constexpr int R = 4;
-                        uint32_t key[R], kmin = 0xffffffffu, kmax = 0u;
-                        unsigned long long wt[R];
-                        unsigned long long c0 = 0ull, c1 = __ldg(&W.bin[b].a);
-#pragma unroll
-                        for (int r = 0; r < R; ++r) get(s0 + 32 * r + lane, key[r], wt[r]);
-                        auto each = [&](auto fn) {
-#pragma unroll
-                            for (int r = 0; r < R; ++r) fn(key[r], wt[r]);
-                            for (uint32_t i = s0 + 32 * R + lane; i < e; i += 32 * 2 * R) {
-                                uint32_t k[2 * R];
-                                unsigned long long a[2 * R];
-#pragma unroll
-                                for (int r = 0; r < 2 * R; ++r) get(i + 32 * r, k[r], a[r]);
-#pragma unroll
-                                for (int r = 0; r < 2 * R; ++r) fn(k[r], a[r]);
-                            }
-                            __syncwarp();
-                        };
-                        each([&](uint32_t k, unsigned long long) {
-                            if (k != 0xffffffffu) {
-                                kmin = min(kmin, k);
-                                kmax = max(kmax, k);
-                            }
-                        });
-                        uint32_t k0 = __reduce_min_sync(kFull, kmin), k1 = __reduce_max_sync(kFull, kmax);
-                        for (int step = 1; k0 < k1; ++step) {
-                            const uint32_t d = k1 - k0;
-                            const float part = step % 3 == 0 ? 0.5f : (float)(need - c0) / (float)(c1 - c0);
-                            const uint32_t km = k0 + min((uint32_t)((float)d * part), d - 1u);
-                            uint32_t end = 0u, begin = 0xffffffffu;
-                            unsigned long long sum = 0ull;
-                            each([&](uint32_t k, unsigned long long a) {
-                                if (k <= km) {
-                                    sum += a;
-                                    end = max(end, k);
-                                } else {
-                                    begin = min(begin, k);
-                                }
-                            });
-                            sum = warp_sum64(sum);
-                            if (sum >= need) k1 = __reduce_max_sync(kFull, end), c1 = sum;
-                            else k0 = __reduce_min_sync(kFull, begin), c0 = sum;
-                        }
-                        lv = sort_key_value(k0);
-                    }
-                }
-            }
-        }
-        if (lane == 0) s_level[set ^ 1][warp] = lv;
+        if (some && !fixed) lv = source.median(a0 + (a1 - a0) - (a1 - a0) / 2ull);
+        if (lane == 0) S.level[set ^ 1][warp] = lv;
         __syncthreads();
     }
     if (warp == kLevels - 1 && iter == F.iters && iter) error_of(iter - 1);
     if (lane == 0 && !fixed) F.codebook[warp] = lv;
 }
 
+// What lies below a threshold: as for the squared error.  The place of a median: in the running sums of the groups (shared memory,
+// 64 entries a step), then of the group's bins (one load), then among the samples of one bin.
+// An iteration over 2^20 fp32 weights 6.5 -> 3.1 us, over 2^24 33 -> 14 (before: two warps to a region, whole groups added up and
+// searched one after the other, cut bins first).  Bound by its chain: three loads from L2 of 430 or 820 cycles each, the
+// reductions, two barriers; over 2^24 weights by the passes over the 500 samples of a bin (of up to 64 samples every lane adds
+// up what is not behind its own, in one pass: 2^20 weights 3.75 -> 3.1).
+constexpr int kMaeSums = ((kSortGroups + 1) * 8 + 15) / 16 * 16;  // shared memory: what lies in front of the groups: weights, {s, sx},
+constexpr int kMaeOff = kMaeSums + (kSortGroups + 1) * 16;      // first samples of the bins,
+constexpr int kMaeFirst = kMaeOff + kSortBins * 2 + 16;         // (and the end) of the groups
+constexpr int kMaeSmem = kMaeFirst + (kSortGroups + 1) * 4;
+
+template <bool CROWDED>
+struct MaeSamples {
+    const SortWs& W;
+    const SampleWeight<true>& weights;
+    SharedTable<double2> group_sums;          // what lies in front of a group
+    SharedTable<unsigned long long> group_a;
+    SharedTable<uint16_t> off;
+    SharedTable<uint32_t> group_first;
+    __device__ __forceinline__ uint32_t start_of(int b) const  // first sample of bin b <= kSortBins
+    {
+        const uint32_t o = off[b], f = group_first[b / kSortGroup];
+        return o == kFarBin ? __ldg(W.start + b) : f + o;
+    }
+    // This lane's share of what lies below v, less the whole groups in front of the one that is returned.
+    template <bool SUMS>
+    __device__ __forceinline__ int below(float v, SortSums& t) const
+    {
+        const int lane = threadIdx.x & 31;
+        const int b = sort_bin(v);
+        const bool one = one_value_bin(b);                        // in or out as a whole
+        const int at = (one && value_of_bin(b) < v) ? b + 1 : b;  // whole bins in front of this one
+        const uint32_t from = start_of(at), to = one ? from : start_of(b + 1);
+        t = SortSums{0.0, 0.0, 0ull};
+        const unsigned long long pre =
+            __ldg(reinterpret_cast<const unsigned long long*>(W.pre + min(at, kSortBins - 1)) + (SUMS ? (lane & 1) : 2));
+        if (CROWDED && to - from > kSortCrowd) {
+            crowded_sums<true>(W, weights, from, to, -__int_as_float(0x7f800000), v, t);
+        } else {
+            auto add = [&](auto count, uint32_t i) {  // 64 samples at once, which is all of most bins, then 128
+                constexpr int U = decltype(count)::value;
+                float2 it[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) it[u] = __ldg(W.b + (i + 32 * u < to ? i + 32 * u : 0u));
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    double s;
+                    unsigned long long a;
+                    weights(it[u], s, a);
+                    const bool in = i + 32 * u < to && it[u].x < v;
+                    const double sx = s * (double)it[u].x;
+                    if (SUMS) {
+                        t.s += in ? s : 0.0;
+                        t.sx += in ? sx : 0.0;
+                    } else {
+                        t.a += in ? a : 0ull;
+                    }
+                }
+            };
+            add(std::integral_constant<int, 2>{}, from + lane);
+            for (uint32_t i = from + 64; i < to; i += 128) add(std::integral_constant<int, 4>{}, i + lane);
+        }
+        __syncwarp();
+        if (at < kSortBins) {
+            if (SUMS && lane == 0) t.s += __longlong_as_double((long long)pre);
+            if (SUMS && lane == 1) t.sx += __longlong_as_double((long long)pre);
+            if (!SUMS && lane == 0) t.a += pre;
+        }
+        return at / kSortGroup;
+    }
+    __device__ __forceinline__ unsigned long long weight(float v) const
+    {
+        SortSums t;
+        const int g = below<false>(v, t);
+        return warp_sum64(t.a) + group_a[g];
+    }
+    __device__ __forceinline__ double2 sums(float v) const
+    {
+        SortSums t;
+        const double2 g = group_sums[below<true>(v, t)];
+        const bool h = threadIdx.x & 16;
+        double u = (h ? t.sx : t.s) + __shfl_xor_sync(kFull, h ? t.s : t.sx, 16);
+#pragma unroll
+        for (int o = 8; o; o >>= 1) u += __shfl_xor_sync(kFull, u, o);
+        return make_double2(g.x + __shfl_sync(kFull, u, 0), g.y + __shfl_sync(kFull, u, 16));
+    }
+    __device__ __forceinline__ float median(unsigned long long goal) const
+    {
+        // the last group in front of which there is less than the goal: 32 groups of 64, then one of 64
+        const int lane = threadIdx.x & 31, c = __popc(__ballot_sync(kFull, group_a[64 * (lane + 1)] < goal));
+        const unsigned long long u = group_a[64 * c + 1 + lane], v = group_a[64 * c + 33 + lane];
+        const int g = 64 * c + __popc(__ballot_sync(kFull, u < goal)) + __popc(__ballot_sync(kFull, v < goal));
+        const unsigned long long before = group_a[g], pre = __ldg(&W.pre[g * kSortGroup + lane].a);
+        const int in = __popc(__ballot_sync(kFull, before + pre < goal)) - 1, b = g * kSortGroup + in;
+        const unsigned long long need = goal - (before + __shfl_sync(kFull, pre, in));  // of the bin's weight
+        if (one_value_bin(b)) return value_of_bin(b);
+        const uint32_t s0 = start_of(b), e = start_of(b + 1);
+        if (CROWDED && e - s0 > kSortCrowd) {
+            unsigned long long none = 0ull;
+            const float inf = __int_as_float(0x7f800000);
+            float median = 0.0f;
+            crowded_median(W, weights, s0, e, -inf, inf, 2ull * need, none, median);
+            return median;
+        }
+        auto get = [&](uint32_t i, uint32_t& k, uint32_t& a) {
+            const float2 it = __ldg(W.b + (i < e ? i : s0));
+            double s;
+            unsigned long long w;
+            weights(it, s, w);
+            k = i < e ? sort_key(it.x) : 0xffffffffu;
+            a = i < e ? (uint32_t)w : 0u;  // (31 bits)
+        };
+        if (e - s0 <= 64u) {
+            // Few samples: one or two to a lane, which adds up for each all those that are not behind it.
+            auto among = [&](auto count) -> float {
+                constexpr int N = decltype(count)::value;
+                uint32_t key[N], mine[N], first = 0xffffffffu;
+                unsigned long long sum[N];
+#pragma unroll
+                for (int r = 0; r < N; ++r) {
+                    get(s0 + 32 * r + lane, key[r], mine[r]);
+                    sum[r] = 0ull;
+                }
+#pragma unroll
+                for (int r = 0; r < N; ++r) {
+                    const int here = min((int)(e - s0) - 32 * r, 32);
+#pragma unroll 4
+                    for (int j = 0; j < here; ++j) {
+                        const uint32_t k = __shfl_sync(kFull, key[r], j), w = __shfl_sync(kFull, mine[r], j);
+#pragma unroll
+                        for (int q = 0; q < N; ++q) sum[q] += k <= key[q] ? w : 0u;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < N; ++q)
+                    if (sum[q] >= need) first = min(first, key[q]);  // (no sample: the last key of all)
+                return sort_key_value(__reduce_min_sync(kFull, first));
+            };
+            return e - s0 <= 32u ? among(std::integral_constant<int, 1>{}) : among(std::integral_constant<int, 2>{});
+        }
+        // The goal is reached at one of the keys k0 ... k1 of the bin's samples; c0 of the bin's weight lies below k0, c1 up to
+        // k1.  The next key to split at is where even weights would put it (every third time the middle), and the ends move to
+        // samples: a handful of steps, where halving the keys takes one per bit in which they differ.
+        constexpr int R = 4;
+        uint32_t key[R], wt[R], kmin = 0xffffffffu, kmax = 0u;
+        unsigned long long c0 = 0ull, c1 = __ldg(&W.bin[b].a);
+#pragma unroll
+        for (int r = 0; r < R; ++r) get(s0 + 32 * r + lane, key[r], wt[r]);
+        auto each = [&](auto fn) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) fn(key[r], wt[r]);
+            for (uint32_t i = s0 + 32 * R + lane; i < e; i += 32 * 2 * R) {
+                uint32_t k[2 * R], a[2 * R];
+#pragma unroll
+                for (int r = 0; r < 2 * R; ++r) get(i + 32 * r, k[r], a[r]);
+#pragma unroll
+                for (int r = 0; r < 2 * R; ++r) fn(k[r], a[r]);
+            }
+            __syncwarp();
+        };
+        each([&](uint32_t k, uint32_t) {
+            if (k != 0xffffffffu) {
+                kmin = min(kmin, k);
+                kmax = max(kmax, k);
+            }
+        });
+        uint32_t k0 = __reduce_min_sync(kFull, kmin), k1 = __reduce_max_sync(kFull, kmax);
+        for (int step = 1; k0 < k1; ++step) {
+            const uint32_t d = k1 - k0;
+            const float part = step % 3 == 0 ? 0.5f : (float)(need - c0) / (float)(c1 - c0);
+            const uint32_t km = k0 + min((uint32_t)((float)d * part), d - 1u);
+            uint32_t end = 0u, begin = 0xffffffffu;
+            unsigned long long sum = 0ull;
+            each([&](uint32_t k, uint32_t a) {
+                if (k <= km) {
+                    sum += a;
+                    end = max(end, k);
+                } else {
+                    begin = min(begin, k);
+                }
+            });
+            sum = warp_sum64(sum);
+            if (sum >= need) k1 = __reduce_max_sync(kFull, end), c1 = sum;
+            else k0 = __reduce_min_sync(kFull, begin), c0 = sum;
+        }
+        return sort_key_value(k0);
+    }
+};
+
+// CROWDED: the kernel for data with crowded bins.  Both are launched, the flag of such bins tells which one runs: with both
+// loops in one kernel 2^22 fp32 weights, 12 iterations, took 299 us against 293.5, 2^20 153.8 against 152.4.
+template <bool CROWDED>
+__global__ void __launch_bounds__(kFitMaeThreads, 1)
+sort_fit_mae_kernel(const __grid_constant__ SortWs W, const __grid_constant__ SortFit F)
+{
+    if (!after_previous()) return;
+    if ((W.n_items[4] != 0u) != CROWDED) return;
+    extern __shared__ __align__(16) unsigned char s_fit[];
+    unsigned long long* const s_a = reinterpret_cast<unsigned long long*>(s_fit);
+    double2* const s_sums = reinterpret_cast<double2*>(s_fit + kMaeSums);
+    uint16_t* const s_off = reinterpret_cast<uint16_t*>(s_fit + kMaeOff);
+    uint32_t* const s_first = reinterpret_cast<uint32_t*>(s_fit + kMaeFirst);
+    __shared__ FitMaeShared S;
+    SampleWeight<true> weights;
+    weights.max_bits = W.n_items[1];
+    weights.unit = F.metric >= 2;
+    if (threadIdx.x == 0) s_off[kSortBins] = 0u;
+    copy_starts(W, s_off, s_first);
+    running_sums<kSortGroups / kFitThreads, PairSum>(kSortGroups, [&](int g) { return PairSum{W.group[g].s, W.group[g].sx}; },
+                                                     [&](int g, const PairSum& v) { s_sums[g] = make_double2(v.s, v.sx); });
+    running_sums<kSortGroups / kFitThreads, unsigned long long>(kSortGroups, [&](int g) { return W.group[g].a; },
+                                                                [&](int g, unsigned long long v) { s_a[g] = v; });
+    copies_done();
+    __syncthreads();
+    MaeSamples<CROWDED> source{W, weights, SharedTable(s_sums), SharedTable(s_a), SharedTable(s_off), SharedTable(s_first)};
+    fit_mae_loop(source, S, s_sums[kSortGroups], s_a[kSortGroups], F);
+}
+
 // ---------------------------------------------------------------- host side
 
 namespace {
 
-template <bool MAE, bool CELLS>
+template <bool MAE>
 int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
 {
-    SampleWeight<MAE, CELLS> weight{};
+    SampleWeight<MAE> weight{};
     weight.unit = F.metric >= 2;
-    weight.acc = reinterpret_cast<const ulonglong2*>(F.acc);
-    weight.acc_a = F.acc_a;
     const int64_t ctas = (F.n_max + 8 * kSortChunk - 1) / (8 * kSortChunk);
-    launch_after(sort_sums_kernel<MAE, CELLS>, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, W, weight);
+    launch_after(sort_sums_kernel<MAE>, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, W, weight);
     launch_after(sort_group_kernel<MAE>, kSortGroups / 8, 256, 0, st, W);
-    // cells never crowd a bin, and no more samples than make one cannot either
     auto order_windows = [&]() -> int {
-        if constexpr (!CELLS) {
-            constexpr auto kern = sort_windows_kernel<MAE>;
-            constexpr int smem = (int)sizeof(WindowScratch);
-            if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
-            const int64_t windows = (F.n_max + kSortWindow - 1) / kSortWindow;
-            launch_after(kern, (int)(windows < kSMs ? windows : kSMs), kSortThreads, smem, st, W, weight);
-        }
+        constexpr auto kern = sort_windows_kernel<MAE>;
+        constexpr int smem = (int)sizeof(WindowScratch);
+        if (const int rc = ensure_dynamic_smem<kern>(smem)) return rc;
+        const int64_t windows = (F.n_max + kSortWindow - 1) / kSortWindow;
+        launch_after(kern, (int)(windows < kSMs ? windows : kSMs), kSortThreads, smem, st, W, weight);
         return BOF4_OK;
     };
-    const bool may_crowd = !CELLS && F.n_max > kSortCrowd;
+    const bool may_crowd = F.n_max > kSortCrowd;  // no more samples than make a crowded bin do not
     if constexpr (MAE) {
-        constexpr int smem = kMaeSmem;
-        constexpr auto plain = sort_fit_mae_kernel<CELLS, false>;
-        if (const int rc = ensure_dynamic_smem<plain>(smem)) return rc;
-        launch_after(plain, 1, kMaeThreads, smem, st, W, F);
+        constexpr auto plain = sort_fit_mae_kernel<false>;
+        if (const int rc = ensure_dynamic_smem<plain>(kMaeSmem)) return rc;
+        launch_after(plain, 1, kFitMaeThreads, kMaeSmem, st, W, F);
         if (may_crowd) {
             if (const int rc = order_windows()) return rc;
-            constexpr auto crowded = sort_fit_mae_kernel<CELLS, !CELLS>;
-            if (const int rc = ensure_dynamic_smem<crowded>(smem)) return rc;
-            launch_after(crowded, 1, kMaeThreads, smem, st, W, F);
+            constexpr auto crowded = sort_fit_mae_kernel<true>;
+            if (const int rc = ensure_dynamic_smem<crowded>(kMaeSmem)) return rc;
+            launch_after(crowded, 1, kFitMaeThreads, kMaeSmem, st, W, F);
         }
     } else {
         if (may_crowd)
             if (const int rc = order_windows()) return rc;
-        constexpr auto kern = sort_fit_mse_kernel<CELLS>;
-        if (const int rc = ensure_dynamic_smem<kern>(kMseSmem)) return rc;
-        launch_after(kern, 1, kMseThreads, kMseSmem, st, W, F);
+        if (const int rc = ensure_dynamic_smem<sort_fit_mse_kernel>(kMseSmem)) return rc;
+        launch_after(sort_fit_mse_kernel, 1, kFitThreads, kMseSmem, st, W, F);
     }
     BOF4_CUDA_TRY(cudaGetLastError());
     return BOF4_OK;
@@ -1575,9 +1483,10 @@ int samples(const EmTensors& T, int block_size, uint32_t first, uint32_t n, cons
 
 }  // namespace
 
-int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
+// Samples are in W.a, their number in *W.n_items: orders them, sums the bins, runs the iterations.
+static int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
 {
-    const bool staged = !F.acc && F.n_max >= kStagedMin;
+    const bool staged = F.n_max >= kStagedMin;
     auto pass = [&](auto shift, const float2* in, float2* out) -> int {
         constexpr int S = decltype(shift)::value;
         launch_after(sort_count_kernel<S>, kSortGrid, kSortThreads, 0, st, in, W.n_items, W.counts);
@@ -1597,11 +1506,10 @@ int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
     V.b = W.a;
     V.before = reinterpret_cast<SortSums*>(W.b);
     const int64_t ctas = F.n_max / 256 + 1;  // one thread beyond the samples
-    launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs) + 1, 256, 0, st, V.b, V.n_items, F.acc ? nullptr : V.first, V.start);
+    launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs) + 1, 256, 0, st, V.b, V.n_items, V.first, V.start);
     BOF4_CUDA_TRY(cudaGetLastError());
     const bool mae = F.metric == BOF4_METRIC_MAE || F.metric == BOF4_METRIC_MAE_NORMALIZED;
-    if (F.acc) return mae ? sums_and_iterations<true, true>(V, F, st) : sums_and_iterations<false, true>(V, F, st);
-    return mae ? sums_and_iterations<true, false>(V, F, st) : sums_and_iterations<false, false>(V, F, st);
+    return mae ? sums_and_iterations<true>(V, F, st) : sums_and_iterations<false>(V, F, st);
 }
 
 int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iters, double* d_err_log, void* d_ws,
@@ -1610,7 +1518,7 @@ int sorted_fit(const EmArgs& a, float* d_codebook, uint32_t fixed_mask, int iter
     *done = false;
     if (a.n_total > kSortMaxDirect || !ordering_pays(a.w_dtype, a.n_total, a.metric, iters, false)) return BOF4_OK;
     SortWs W;
-    if (sorted_layout(d_ws, a.n_total, false, &W) > ws_bytes) return BOF4_OK;
+    if (sorted_layout(d_ws, a.n_total, &W) > ws_bytes) return BOF4_OK;
     *done = true;
     const uint32_t n = (uint32_t)a.n_total;
     const bool alone = !has_whole_blocks(a);

@@ -1,11 +1,10 @@
-// Codebook fit over samples that are put in order ONCE: interface between the two ways of making the
-// samples (em_sorted.cu: one per weight; em_cells.cu: one per distinct normalised weight of bf16
-// data) and what follows them (order, sums per bin, all iterations in one launch).
+// Codebook fit over samples that are put in order ONCE: what the two ways share (em_sorted.cu: one sample per weight, put in the order of
+// bins of x; em_cells.cu and em_cells_fit.cu: one per distinct normalised weight of bf16 data, whose order is known).
 //
 // The normalised weights x and the block constants do not change from one Lloyd iteration to the next;
-// only the thresholds move.  With the samples in ascending order of a 16-bit bin of x and the sums of
-// every bin at hand, an iteration needs no pass over the data: a region's sums are those of the bins
-// inside it plus the few samples of the two bins that its thresholds cut, and the weighted median is
+// only the thresholds move.  With the samples in ascending order of a 16-bit bin of x and running sums of
+// the bins at hand, an iteration needs no pass over the data: what lies below a threshold is a running sum
+// plus a few samples of the bin that the threshold cuts, a region is the difference of two such sums, and the weighted median is
 // found the same way.  An iteration costs about as much as a handful of L2 accesses, whatever the size
 // of the data.
 #pragma once
@@ -30,15 +29,14 @@ constexpr uint32_t kSortWindow = 8192;       // samples put in full order togeth
 constexpr int64_t kSortMaxDirect = (int64_t)1 << 26;  // one sample per weight: 16 bytes of workspace each
 constexpr int kSortParts = 2 * kSMs + 1;     // partial sums of w^2: CTAs of the sample kernels, and the short last blocks
 
-// A sample is {x, payload}: the magnitude of its block constant, or (em_cells.cu) the number of its cell.
+// A sample is {x, the magnitude of its block constant}.
 struct SortSums {      // per bin, per group, or per part of a bin
     double s, sx;      // sum of the sample weights, sum of weight * x
     unsigned long long a;  // MAE: sum of the fixed-point weights of the median
 };
 
 struct SortWs {
-    uint32_t* n_items;    // device: [0] samples, [1] bits of the largest block constant, [2..3] scale (em_cells.cu),
-                          // [4] whether a bin is crowded
+    uint32_t* n_items;    // device: [0] samples, [1] bits of the largest block constant, [4] whether a bin is crowded
     double* w2;           // [kSortParts]
     uint32_t* counts;     // [kSortGrid][256]
     uint32_t* start;      // [kSortBins + 1] first sample of every bin
@@ -49,8 +47,6 @@ struct SortWs {
     SortSums *lead, *trail;  // [chunks] part of a bin that began in an earlier chunk / that goes on in the next
     float2 *a, *b;        // samples, ordered samples
     SortSums* before;     // crowded bins: sums of the window's samples in front of every fourth (in the place of a)
-    double* cell_s;       // em_cells.cu: weights of the ordered samples (else NULL)
-    unsigned long long* cell_a;
 };
 
 // Whether a fit of `iters` iterations over n weights is faster with its samples in order than streamed: the ordering is
@@ -58,16 +54,16 @@ struct SortWs {
 // other block sizes differ by a few per cent):
 //   ordering, less what a streamed fit takes before its first iteration
 //             one sample per weight, fp32: 66 (k = 1), 94 (2), 162 (4), 267 (8), 534 (16), 778 (24), 1026 (32), 1514 (48), 2001 (64)
-//             distinct bf16 weights 75 to 83 (2), 90 (4), 93 to 113 (16), 143 to 175 (64), 192 to 413 (256)
+//             distinct bf16 weights 72 (2), 73 (4), 95 (16), 150 (64), 340 (256)
 //   streamed iteration less an ordered one
-//             fp32: MSE 15 (1), 15 (2), 19 (4), 24 (8), 33 (16), 50 (24), 61 (32), 83 (48), 105 (64),
-//             medians 43, 45, 51, 63, 69, 91, 101, 125, 141
-//             bf16: MSE 15 (1), 15 (2), 16 (4), 31 (16), 82 (64), 259 (256), medians 48, 51, 51, 78, 179, 569
+//             fp32: MSE 15 (1), 15 (2), 19 (4), 24 (8), 34 (16), 50 (24), 61 (32), 83 (48), 105 (64),
+//             medians 47 (1), 55 (4), 90 (16), 227 (64)
+//             bf16: MSE 17 (2), 16 (4), 32 (16), 80 (64), 255 (256), medians 55, 57, 82, 176, 681
 // The lines below are fits to these, a little on the streamed side, which takes 9 MB of workspace where ordering takes 16 bytes a weight;
 // from 2^25 weights on (more than half a gigabyte) ordering has to save more than it costs: fits of 2^26 weights and up to 32 iterations
 // (medians 23) get by with the small workspace, as callers are promised.  Where they cross, in iterations, and by the figures: fp32
-// MSE 6 (5) at 2^20, 10 (9) at 2^22, 13 (12) at 2^23, 17 (16) at 2^24, 20 (17) at 2^25, 33 (19) at 2^26, medians 4, 4, 7 (5), 9 (8), 12 (11),
-// 24 (15); bf16 MSE 6 from 3 * 2^19 to 2^22, 4 from 2^24 on, medians 4.
+// MSE 6 (5) at 2^20, 10 (9) at 2^22, 13 (12) at 2^23, 17 (16) at 2^24, 20 (17) at 2^25, 33 (19) at 2^26, medians 4, 4 (3) at 2^22, 9 (7) at
+// 2^24, 24 (9) at 2^26; bf16 MSE 6 (5) from 3 * 2^19 to 2^22, 4 (3) from 2^24 on, medians 4 (2).
 // Fewer than four iterations are not ordered, although two or three would pay for bf16 data from 2^26 weights on (2^28, three: 1000
 // us streamed, about 410 ordered): such a fit gets by with the small workspace.
 inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool cells)
@@ -88,11 +84,9 @@ bool cells_apply(int w_dtype, int64_t n);
 size_t cells_workspace_bytes(int64_t n, int block_size);
 
 // Carves the workspace for up to n samples; returns the bytes used.
-size_t sorted_layout(void* base, int64_t n, bool cells, SortWs* W);
+size_t sorted_layout(void* base, int64_t n, SortWs* W);
 
 struct SortFit {
-    const unsigned long long* acc;   // em_cells.cu: [cell] {low, high} 128-bit sum of weights, else NULL
-    const unsigned long long* acc_a; // [cell] fixed-point weights (MAE)
     int metric;
     int64_t n_total;
     int64_t n_max;                   // at most this many samples
@@ -101,9 +95,6 @@ struct SortFit {
     int iters;
     double* err_log;
 };
-
-// Samples are in W.a, their number in *W.n_items: orders them, sums the bins, runs the iterations.
-int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st);
 
 // The whole fit by one of the two ways; *done tells whether it was taken (workspace, size, type,
 // number of iterations).

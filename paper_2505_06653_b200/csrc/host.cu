@@ -94,7 +94,7 @@ size_t bof4_fit_workspace_bytes(int64_t n_total, int w_dtype, int block_size, in
     if (need == 0 || (w_dtype != BOF4_F32 && w_dtype != BOF4_BF16)) return 0;
     const bool cells = bof4::cells_apply(w_dtype, n_total);
     if ((!cells && n_total > bof4::kSortMaxDirect) || !bof4::ordering_pays(w_dtype, n_total, metric, iters, cells)) return need;
-    const size_t order = cells ? bof4::cells_workspace_bytes(n_total, block_size) : bof4::sorted_layout(nullptr, n_total, false, nullptr);
+    const size_t order = cells ? bof4::cells_workspace_bytes(n_total, block_size) : bof4::sorted_layout(nullptr, n_total, nullptr);
     return need < order ? order : need;
 }
 
