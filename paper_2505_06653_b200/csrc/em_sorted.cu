@@ -2,8 +2,8 @@
 // the sums per bin and the iterations.
 //
 // Launches of a fit, whatever its number of iterations: samples (one per 64 tensors), two ordering
-// passes of eight bits (count and scatter each, least significant digit first, stable), first sample of
-// every bin, full order where a bin is crowded, sums of the bins in two steps, iterations.  Nothing depends on the order in which CTAs run:
+// passes of eight bits (count and scatter each, least significant digit first, stable), first samples and sums
+// of the bins in two steps, full order where a bin is crowded, iterations.  Nothing depends on the order in which CTAs run:
 // the samples' order, the order of every sum and hence the result are reproducible.
 #include <type_traits>
 
@@ -194,11 +194,19 @@ __device__ __forceinline__ void sort_part(uint32_t n, uint32_t c, uint32_t& lo, 
     hi = min(n, lo + len);
 }
 
+// tops (the second pass): the largest constants of the samples' CTAs, of which one CTA makes one.
 template <int SHIFT>
 __global__ void __launch_bounds__(kSortThreads)
-sort_count_kernel(const float2* __restrict__ in, const uint32_t* __restrict__ head, uint32_t* __restrict__ counts)
+sort_count_kernel(const float2* __restrict__ in, uint32_t* __restrict__ head, uint32_t* __restrict__ counts, const uint32_t* __restrict__ tops)
 {
     if (!after_previous()) return;
+    if (SHIFT && blockIdx.x == 0 && threadIdx.x < 32) {
+        uint32_t top = 0u;
+#pragma unroll
+        for (int k = 0; k < kSortParts; k += 32) top = max(top, k + threadIdx.x < kSortParts ? tops[k + threadIdx.x] : 0u);
+        top = __reduce_max_sync(kFull, top);
+        if (threadIdx.x == 0) head[1] = top;
+    }
     __shared__ uint32_t s_hist[4][256];  // a copy per eight warps: fewer collisions on crowded digits
     const int tid = threadIdx.x;
     (&s_hist[0][0])[tid] = 0u;
@@ -386,43 +394,6 @@ struct SampleWeight {
         if (MAE) a = unit ? 1ull : (unsigned long long)sort_fixed_weight(it.y, max_bits);
     }
 };
-
-// First sample of every bin: sample i is the first of all bins behind the one of sample i - 1 up to its own; behind
-// the last sample come all bins that are left, which are all there are where no sample has a weight (bf16 zeros).
-// tops: the largest constants of the samples' CTAs, of which the last CTA makes one.
-__global__ void __launch_bounds__(256)
-sort_start_kernel(const float2* __restrict__ items, uint32_t* __restrict__ head, const uint32_t* __restrict__ tops,
-                  uint32_t* __restrict__ start)
-{
-    if (!after_previous()) return;
-    const uint32_t n = *head;
-    if (blockIdx.x == gridDim.x - 1) {
-        if (threadIdx.x >= 32) return;
-        uint32_t top = 0u;
-#pragma unroll
-        for (int k = 0; k < kSortParts; k += 32) top = max(top, k + threadIdx.x < kSortParts ? tops[k + threadIdx.x] : 0u);
-        top = __reduce_max_sync(kFull, top);
-        if (threadIdx.x == 0) head[1] = top;
-        return;
-    }
-    int far0 = 0, far1 = -1;  // a gap of many empty bins, if the thread meets one: filled by the warp below
-    uint32_t far_i = 0u;
-    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i <= n; i += (gridDim.x - 1) * 256) {
-        const int b = i < n ? sort_bin(items[i].x) : kSortBins, prev = i ? sort_bin(items[i - 1].x) : -1;
-        if (b - prev > 64 && far1 < 0) {
-            far0 = prev + 1, far1 = b;
-            far_i = i;
-        } else {
-            for (int t = prev + 1; t <= b; ++t) start[t] = i;
-        }
-    }
-    __syncwarp();
-    for (unsigned far = __ballot_sync(kFull, far1 >= 0); far; far &= far - 1u) {
-        const int who = __ffs(far) - 1, t0 = __shfl_sync(kFull, far0, who), t1 = __shfl_sync(kFull, far1, who);
-        const uint32_t i = __shfl_sync(kFull, far_i, who);
-        for (int t = t0 + (threadIdx.x & 31); t <= t1; t += 32) start[t] = i;
-    }
-}
 
 template <bool MAE>
 __device__ __forceinline__ void sums_reduce(SortSums& t)
@@ -613,7 +584,8 @@ __device__ __noinline__ void crowded_sums(const SortWs& W, const SampleWeight<MA
     }
 }
 
-// One warp per kSortChunk ordered samples, 32 at a time: a segmented scan over the runs of equal bins.
+// One warp per kSortChunk ordered samples, 32 at a time: a segmented scan over the runs of equal bins; the first samples of all bins
+// on the way (with a launch of their own fits of 2^20 weights took 3 us longer).
 // A run that lies inside the chunk is a bin's sum; parts of runs that cross the chunk's edges go to
 // lead / trail and are put together by sort_group_kernel.  The work is even whatever the distribution (the bins
 // of x = +-1 hold 1 / I of the data; a bin of small data is mostly empty).
@@ -657,6 +629,17 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE> weight)
             int left = __shfl_up_sync(kFull, key[k], 1);
             if (lane == 0) left = open_key;
             const unsigned heads = __ballot_sync(kFull, key[k] != left);
+            // the sample is the first of all bins behind the one of the sample before it up to its own; a gap of many empty bins is
+            // filled by the warp
+            const bool starts = key[k] != left && key[k] != kNone, wide = starts && key[k] - left > 64;
+            const uint32_t i = lo + 32 * k + lane;
+            if (starts && !wide)
+                for (int t = left + 1; t <= key[k]; ++t) W.start[t] = i;
+            for (unsigned far = __ballot_sync(kFull, wide); far; far &= far - 1u) {
+                const int who = __ffs(far) - 1, t1 = __shfl_sync(kFull, key[k], who);
+                const uint32_t first = __shfl_sync(kFull, i, who);
+                for (int t = __shfl_sync(kFull, left, who) + 1 + lane; t <= t1; t += 32) W.start[t] = first;
+            }
             if ((heads & 1u) && k > 0 && lane == 0 && open_key != kNone) (early ? W.lead[c] : W.bin[open_key]) = open;
             const unsigned upto = heads & ((2u << lane) - 1u);
             const int from = upto ? 31 - __clz(upto) : 0;
@@ -679,10 +662,12 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE> weight)
             open_key = __shfl_sync(kFull, key[k], 31);
             early = early && heads == 0u;
         }
-        // a chunk inside one bin: a crowded one has many, the first of them says so
-        if (early && open_key == before && lane == 0 && !one_value_bin(before)) {
-            const uint32_t s = W.start[before];
-            if (lo - s <= kSortChunk && W.start[before + 1] - s > kSortCrowd) W.n_items[4] = 1u;
+        if (hi == n) {  // behind the last sample come all bins that are left
+            int top = -1;
+#pragma unroll
+            for (int k = 0; k < STEPS; ++k) top = max(top, key[k] == kNone ? -1 : key[k]);
+            top = __reduce_max_sync(kFull, top);
+            for (int t = top + 1 + lane; t <= kSortBins; t += 32) W.start[t] = n;
         }
         if (lane == 0 && open_key != kNone) (early ? W.lead[c] : open_key == behind ? W.trail[c] : W.bin[open_key]) = open;
     }
@@ -707,6 +692,7 @@ sort_group_kernel(const SortWs W)
     SortSums t{0.0, 0.0, 0ull};
     const uint32_t c0 = s / kSortChunk, c1 = (e > s) ? (e - 1) / kSortChunk : c0;
     if (e > s && c0 == c1) t = W.bin[b];
+    if (e > s && e - s > kSortCrowd && !one_value_bin(b)) W.n_items[4] = 1u;
     // a bin of a few chunks by its lane, the lanes side by side; a longer one by the warp
     const bool few = e > s && c0 != c1 && c1 - c0 <= kSortFew;
     if (few) {
@@ -1489,7 +1475,7 @@ static int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
     const bool staged = F.n_max >= kStagedMin;
     auto pass = [&](auto shift, const float2* in, float2* out) -> int {
         constexpr int S = decltype(shift)::value;
-        launch_after(sort_count_kernel<S>, kSortGrid, kSortThreads, 0, st, in, W.n_items, W.counts);
+        launch_after(sort_count_kernel<S>, kSortGrid, kSortThreads, 0, st, in, W.n_items, W.counts, W.first);
         if (staged) {
             constexpr auto kern = sort_scatter_kernel<S, true>;
             if (const int rc = ensure_dynamic_smem<kern>(kScatterSmem)) return rc;
@@ -1505,8 +1491,6 @@ static int sorted_run(const SortWs& W, const SortFit& F, cudaStream_t st)
     V.a = W.b;
     V.b = W.a;
     V.before = reinterpret_cast<SortSums*>(W.b);
-    const int64_t ctas = F.n_max / 256 + 1;  // one thread beyond the samples
-    launch_after(sort_start_kernel, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs) + 1, 256, 0, st, V.b, V.n_items, V.first, V.start);
     BOF4_CUDA_TRY(cudaGetLastError());
     const bool mae = F.metric == BOF4_METRIC_MAE || F.metric == BOF4_METRIC_MAE_NORMALIZED;
     return mae ? sums_and_iterations<true>(V, F, st) : sums_and_iterations<false>(V, F, st);
