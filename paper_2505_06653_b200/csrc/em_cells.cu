@@ -11,8 +11,9 @@
 //   order       block addresses grouped by magnitude
 //   accumulate  a unit is some blocks of ONE magnitude |m|: with m fixed, the cell of a weight is the
 //               difference of the two bit patterns, so the counts of a unit are 10240 words of shared
-//               memory and a weight costs a subtraction, a comparison and one shared-memory reduction
-//               on random banks, whose conflicts bound it (4.6 wavefronts of the LSU data path per 32 weights; two
+//               memory and a weight costs a subtraction, a comparison and one shared-memory reduction,
+//               whose rate bounds it (4.6 cycles per 32 weights; a counter per lane for four binades, so that no two
+//               lanes meet at a bank, takes two reductions of 4.4 each: 811 -> 1570 us; two
 //               weights at a time without a predicate where all are counted: 2^26 weights 56 -> 51 us, 1.6 * 10^9 827 -> 811);
 //               when the unit is done its counts times the weight of |m| are added to the cells
 //   then        sums of the cells in the order of x, and all iterations (em_cells_fit.cu)
