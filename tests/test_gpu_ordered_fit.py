@@ -290,3 +290,21 @@ def test_median_among_the_samples_of_one_bin(bof4, each):
     w = torch.cat([torch.ones(len(x), 1), x, x.neg().flip(0)], 1)
     w = torch.nn.functional.pad(w, (0, 1)) * (0.5 + torch.rand(len(x), 1, generator=g))
     _check(bof4, [w.reshape(-1)], 64, 0, bof4.METRIC_MAE, 12)
+
+
+def test_a_light_region_among_distinct_weights(bof4):
+    """The same for bf16 data: quotients near one half of blocks that are 2^-20 of the others', whose own lie just beside the region."""
+    n, light = 1 << 21, 200
+    g = torch.Generator().manual_seed(5)
+    x = torch.where(torch.rand(n // 64, 64, generator=g) < 0.5, 255 / 512, 129 / 256)
+    m = torch.ones(n // 64, 1)
+    m[:light] = 2.0 ** -20 * (1 + torch.randint(0, 128, (light, 1), generator=g) / 128)
+    x[:light] = 0.5005
+    x[:, 0] = 1.0
+    w = (x * m).to(torch.bfloat16).reshape(-1)
+    lv = np.array([-1, -0.5, -0.4, -0.3, -0.2, -0.1, 0, 0.1, 0.2, 0.3, 0.4, 0.498, 0.5004, 0.5039, 0.7, 1], np.float32)
+    cb, log = bof4.bof4_fit_codebook(w.cuda(), 64, 0, 0, lv, 0xffff ^ (1 << 12), 8)
+    ref, ref_log = oracle.fit([w], 64, 0, 0, lv, 0xffff ^ (1 << 12), 8)
+    assert ref[12] != lv[12]
+    np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-7)
+    np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5)
