@@ -209,11 +209,6 @@ __device__ __noinline__ double2 cell_region(const CellsWs& W, float p, float q)
 }
 
 constexpr int kCellValues = (kCellFractions + kCellParts) * 2;  // bytes of value_of
-__device__ __forceinline__ void copy_values(const CellsWs& W, uint16_t* s_value)
-{
-    for (int k = threadIdx.x; k < kCellValues / 16; k += blockDim.x)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(s_value + 8 * k)), "l"(W.value_of + 8 * k) : "memory");
-}
 
 // ---- squared error
 
@@ -280,7 +275,7 @@ cells_fit_mse_kernel(const __grid_constant__ CellsWs W, const __grid_constant__ 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float inf = __int_as_float(0x7f800000);
     if (tid == 0) s_stop = 0x7fffffff;
-    copy_values(W, s_value);
+    copy_in(s_value, W.value_of, kCellValues);
     double w2 = 0.0;
     if (warp == kLevels - 1) {
 #pragma unroll 8
@@ -419,13 +414,15 @@ cells_fit_mse_kernel(const __grid_constant__ CellsWs W, const __grid_constant__ 
 //
 // Warp l forms what lies below the two thresholds beside level l and looks for the median between them: the first cell, in the order of
 // x, with which the weight reaches half of the region's.  Its part is found by three steps of 32 entries in shared memory, its place
-// among the 128 of the part by one round of loads.  One more warp, with a level or a threshold per lane, adds up the error
+// among the 128 of the part by one round of loads.  One more warp, with half a region per lane, adds up the error
 // and stops the others when no level has moved.
 // An iteration over eight layers of a 7B-shaped model 5.6 us with sorted cells, 2.5 with running sums over 65,536 bins, 1.9 with places and
-// sixteen warps for the error, a barrier before the medians, 1.41 this way.
+// sixteen warps for the error, a barrier before the medians, 1.41 with one warp for it and no such barrier, 1.30 with what an iteration's
+// error needs loaded behind the one before and 32 errors divided at once (2^22 and 2^26 weights).
 constexpr int kCellsMaeThreads = kFitThreads + 32;
-constexpr int kCellsMaeSums = ((kCellPartsAll + 1) * 8 + 15) / 16 * 16;       // shared memory: weights in front of the parts, {s, sx} of
-constexpr int kCellsMaeValues = kCellsMaeSums + (kCellBlocks + 1) * 16;       // the blocks, value_of
+constexpr int kCellsMaeHigh = ((kCellPartsAll + 1) * 8 + 15) / 16 * 16;       // shared memory: weights in front of the parts, {s, sx} in
+constexpr int kCellsMaeLow = kCellsMaeHigh + (kCellBlocks + 1) * 16;          // front of the blocks, high and low halves,
+constexpr int kCellsMaeValues = kCellsMaeLow + (kCellBlocks + 1) * 16;        // value_of
 constexpr int kCellsMaeSmem = kCellsMaeValues + kCellValues;
 __global__ void __launch_bounds__(kCellsMaeThreads, 1)
 cells_fit_mae_kernel(const __grid_constant__ CellsWs W, const __grid_constant__ SortFit F)
@@ -433,51 +430,72 @@ cells_fit_mae_kernel(const __grid_constant__ CellsWs W, const __grid_constant__ 
     if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char s_fit[];
     unsigned long long* const s_a = reinterpret_cast<unsigned long long*>(s_fit);
-    double2* const s_sums = reinterpret_cast<double2*>(s_fit + kCellsMaeSums);
+    double2* const s_high = reinterpret_cast<double2*>(s_fit + kCellsMaeHigh);
+    double2* const s_low = reinterpret_cast<double2*>(s_fit + kCellsMaeLow);
     uint16_t* const s_value = reinterpret_cast<uint16_t*>(s_fit + kCellsMaeValues);
     __shared__ float s_level[2][kLevels];
     __shared__ int s_stop;  // the iteration behind whose barrier all leave
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    copy_values(W, s_value);
+    copy_in(s_value, W.value_of, kCellValues);
     if (tid < kLevels) s_level[0][tid] = F.codebook[tid];
     if (tid == 0) s_stop = 0x7fffffff;
-    running_sums<kCellPer, PairSum>(kCellBlocks, [&](int b) { return PairSum{W.block[b].s, W.block[b].sx}; },
-                                    [&](int b, const PairSum& v) { s_sums[b] = make_double2(v.s, v.sx); });
-    running_sums<kCellPartsAll / kFitThreads + 1, unsigned long long>(kCellPartsAll, [&](int p) { return W.part_a[p]; },
-                                                                     [&](int p, unsigned long long v) { s_a[p] = v; });
+    CellBlock* const s_block = reinterpret_cast<CellBlock*>(s_high);  // the blocks' sums, before the running sums take their place
+    static_assert(kCellBlocks * sizeof(CellBlock) + 16 <= 2 * (kCellBlocks + 1) * sizeof(double2), "room for the blocks' sums");
+    copy_in(s_block, W.block, kCellBlocks * (int)sizeof(CellBlock));
+    copy_in(s_a, W.part_a, kCellPartsAll * 8);
     copies_done();
+    __syncthreads();
+    running_sums<kCellPer, TwoPair>(kCellBlocks, [&](int b) { return TwoPair{{s_block[b].s, 0.0}, {s_block[b].sx, 0.0}}; },
+                                    [&](int b, const TwoPair& v) {
+                                        s_high[b] = make_double2(v.s.h, v.x.h);
+                                        s_low[b] = make_double2(v.s.l, v.x.l);
+                                    });
+    running_sums<kCellPartsAll / kFitThreads + 1, unsigned long long>(kCellPartsAll, [&](int p) { return s_a[p]; },
+                                                                     [&](int p, unsigned long long v) { s_a[p] = v; });
     __syncthreads();
     const SharedTable<uint16_t> value_of(s_value);
     const SharedTable<unsigned long long> parts_a(s_a);
     if (warp == kLevels) {
-        // ---- the error: lane l has level l, lane 16 + l threshold l (the last one: everything)
-        const SharedTable<double2> block_sums(s_sums);
-        const int l = lane & (kLevels - 1);
+        // ---- the error, a half region to a lane
+        const SharedTable<double2> high(s_high), low(s_low);
+        const int l = lane & (kLevels - 1), from = lower_end_of(lane);
         float before = __int_as_float(0x7fc00001);
-        double err = 0.0;
+        double err = 0.0, kept = 0.0;
+        // Of iteration k, formed behind the loads of the next one; 32 are kept, a lane each, and written together.
+        Below end;
+        double2 rest;
+        FitPoints at;
+        auto add_up = [&](int k) {
+            end.low.x += rest.x, end.low.y += rest.y;
+            const Below begin{make_double2(__shfl_sync(kFull, end.high.x, from), __shfl_sync(kFull, end.high.y, from)),
+                              make_double2(__shfl_sync(kFull, end.low.x, from), __shfl_sync(kFull, end.low.y, from))};
+            err = half_error(lane, at, before, begin, end);
+#pragma unroll
+            for (int off = 16; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
+            if (lane == (k & 31)) kept = err;
+            if ((k & 31) == 31 && F.err_log) F.err_log[k - 31 + lane] = fmax(kept, 0.0) / (double)F.n_total;
+        };
         int iter = 0;
         for (; iter < F.iters; ++iter) {
-            const float lv = s_level[iter & 1][l], above = s_level[iter & 1][min(l + 1, kLevels - 1)];
-            const bool threshold = lane >= kLevels, all = lane == 31;
-            const int place = place_of<1>(all ? __int_as_float(0x7f800000) : threshold ? __fmul_rn(__fadd_rn(lv, above), 0.5f) : lv, value_of);
-            const double2 f = __ldg(W.front + place), b = block_sums[place / kCellBlock];
+            const float* const lvs = s_level[iter & 1];
+            const float lv = lvs[l];
+            const FitPoints now = points_of(l, lvs[max(l - 1, 0)], lv, lvs[min(l + 1, kLevels - 1)]);
+            const int place = place_of<1>(lane < kLevels ? now.mid : now.hi, value_of);
+            const double2 next = __ldg(W.front + place);
+            if (iter) add_up(iter - 1);
             // the levels have stopped to move: the iterations from this one on repeat the one before bit for bit
             const bool same = __all_sync(kFull, __float_as_uint(lv) == __float_as_uint(before));
-            before = lv;
             if (same && lane == 0) s_stop = iter;
             __syncthreads();
             if (same) break;
-            const double s = b.x + f.x, x = b.y + f.y;
-            if (all) err = x - (double)lv * s;
-            else if (threshold) err = 2.0 * x - ((double)lv + (double)above) * s;
-            else err = 2.0 * ((double)lv * s - x);
-#pragma unroll
-            for (int off = 16; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
-            err = fmax(err, 0.0) / (double)F.n_total;
-            if (lane == 0 && F.err_log) F.err_log[iter] = err;
+            before = lv, at = now, rest = next;
+            end = Below{high[place / kCellBlock], low[place / kCellBlock]};
         }
-        if (F.err_log)
-            for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = err;
+        if (iter == F.iters) add_up(iter - 1);
+        if (F.err_log) {
+            if (lane < (iter & 31)) F.err_log[(iter & ~31) + lane] = fmax(kept, 0.0) / (double)F.n_total;
+            for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = fmax(err, 0.0) / (double)F.n_total;
+        }
         return;
     }
     // ---- warp l: level l

@@ -2,9 +2,11 @@
 // em_cells_fit.cu: the distinct normalised weights of bf16 data).
 //
 // An iteration is a chain of latencies, so it is kept short: what lies below a threshold is one sum, and a region is the difference of
-// two such sums.  For the squared error the sums of large parts of the samples are kept in two doubles each, so that their
-// difference is as good as adding the region up; the rest is rounded once to a double.  A region that is very light beside its
-// neighbours, or stands beside sums that are not finite, is added up by itself.  The weights of the medians are integers.
+// two such sums.  The sums of large parts of the samples are kept in two doubles each, so that their difference is as good as
+// adding the region up; the rest is rounded once to a double.  For the squared error a region that is very light beside its
+// neighbours, or stands beside sums that are not finite, is added up by itself; the absolute error, which only goes to the log, is known to
+// the rounding of these differences, 2^-53 of the weight in each (with one double for a sum over all parts it was off by 30 times as much).
+// The weights of the medians are integers.
 //
 // When an iteration leaves every level unchanged the remaining ones would repeat it bit for bit: their entries of the error log
 // are filled in and the loop ends.
@@ -18,6 +20,14 @@ constexpr int kFitThreads = 32 * kLevels;  // those that form the running sums
 
 // This thread's asynchronous copies have arrived.
 __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Asynchronous copy of `bytes` (rounded up to 16) to shared memory, by all threads of the CTA.
+__device__ __forceinline__ void copy_in(void* to, const void* from, int bytes)
+{
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(to);
+    for (int k = threadIdx.x; k < (bytes + 15) / 16; k += blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a + 16u * k), "l"(static_cast<const char*>(from) + 16 * k) : "memory");
+}
 
 // A table in shared memory that is complete: made behind the barrier that its writers pass.  Holds its address in that space,
 // which the compiler does not find out for pointers in the sources.
@@ -58,14 +68,24 @@ __device__ __forceinline__ TwoSum two_shfl_up(const TwoSum& a, int off)
 
 __device__ __forceinline__ unsigned long long shfl_up(unsigned long long v, int off) { return __shfl_up_sync(kFull, v, off); }
 __device__ __forceinline__ unsigned long long shfl(unsigned long long v, int from) { return __shfl_sync(kFull, v, from); }
-struct PairSum {
-    double s, sx;
+// {s, sx} in two doubles each, of which the low ones take up what the high ones are rounded by (they are not made small again
+// after an addition: a few units of the high ones at most, and three operations of eleven less).
+struct TwoPair {
+    TwoSum s, x;
 };
-__device__ __forceinline__ PairSum operator+(const PairSum& a, const PairSum& b) { return PairSum{a.s + b.s, a.sx + b.sx}; }
-__device__ __forceinline__ PairSum shfl_up(const PairSum& v, int off) { return PairSum{__shfl_up_sync(kFull, v.s, off), __shfl_up_sync(kFull, v.sx, off)}; }
-__device__ __forceinline__ PairSum shfl(const PairSum& v, int from) { return PairSum{__shfl_sync(kFull, v.s, from), __shfl_sync(kFull, v.sx, from)}; }
+__device__ __forceinline__ TwoSum two_gather(const TwoSum& a, const TwoSum& b)
+{
+    const double s = a.h + b.h, t = s - a.h;
+    return TwoSum{s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l)};
+}
+__device__ __forceinline__ TwoPair operator+(const TwoPair& a, const TwoPair& b) { return TwoPair{two_gather(a.s, b.s), two_gather(a.x, b.x)}; }
+__device__ __forceinline__ TwoPair shfl_up(const TwoPair& v, int off) { return TwoPair{two_shfl_up(v.s, off), two_shfl_up(v.x, off)}; }
+__device__ __forceinline__ TwoSum two_shfl(const TwoSum& a, int from) { return TwoSum{__shfl_sync(kFull, a.h, from), __shfl_sync(kFull, a.l, from)}; }
+__device__ __forceinline__ TwoPair shfl(const TwoPair& v, int from) { return TwoPair{two_shfl(v.s, from), two_shfl(v.x, from)}; }
 
-// The same for values of any type with a sum.
+// put(k, sum of part(0) ... part(k - 1)), k = 0 ... n, by all threads of the CTA; n <= PER * kFitThreads.  All parts have been read before
+// anything is put, so a sum may take the place of its part.  (The parts come from shared memory, see copy_in: a thread's are
+// neighbours, and the lines that they share do not stay in the L1 that the tables leave: read from global memory, 11 us more for the cells.)
 template <int PER, class T, class Part, class Put>
 __device__ __forceinline__ void running_sums(int n, Part part, Put put)
 {
@@ -73,33 +93,72 @@ __device__ __forceinline__ void running_sums(int n, Part part, Put put)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool has = warp < kLevels;
     T v[PER], t{};
+    auto scan = [&](T& u, int width) {  // inclusive, over the first `width` lanes of the warp
 #pragma unroll
-    for (int k = 0; k < PER; ++k) v[k] = has && tid * PER + k < n ? part(tid * PER + k) : T{};
-#pragma unroll
-    for (int k = 0; k < PER; ++k) t = t + v[k];
-    auto scan = [&](T& u) {  // inclusive, over the warp
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
+        for (int off = 1; off < width; off <<= 1) {
             const T w = shfl_up(u, off);
             if (lane >= off) u = w + u;
         }
     };
-    scan(t);
-    if (lane == 31 && has) s_warp[warp] = t;
+    if (has) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) v[k] = tid * PER + k < n ? part(tid * PER + k) : T{};
+        t = v[0];
+#pragma unroll
+        for (int k = 1; k < PER; ++k) t = t + v[k];
+        scan(t, 32);
+        if (lane == 31) s_warp[warp] = t;
+    }
     __syncthreads();
+    if (!has) return;
     T w{};
-    if (lane < warp && lane < kLevels) w = s_warp[lane];
-    scan(w);
+    if (lane < warp) w = s_warp[lane];
+    scan(w, kLevels);
     T run = shfl_up(t, 1);
     if (lane == 0) run = T{};
-    run = shfl(w, 31) + run;
-    if (!has) return;
+    run = shfl(w, kLevels - 1) + run;
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         if (tid * PER + k <= n) put(tid * PER + k, run);
         run = run + v[k];
     }
     if (tid == kFitThreads - 1 && n == kFitThreads * PER) put(n, run);
+}
+
+// {s, sx} of what lies below a point, in two doubles each.
+struct Below {
+    double2 high, low;
+};
+__device__ __forceinline__ Below below_of(double2 high, double2 low, double2 rest) { return Below{high, make_double2(low.x + rest.x, low.y + rest.y)}; }
+
+// The absolute error is added up half region by half region, each the difference of two such sums.  Lane l has what lies below level l,
+// lane 16 + l what lies below the threshold above it (lane 31: everything): a lane's half ends there and begins at the point of the
+// lane that `lower_end_of` says.
+__device__ __forceinline__ int lower_end_of(int lane) { return lane < kLevels ? lane + kLevels - 1 : lane - kLevels; }
+
+// The points of level l: the thresholds on either side and the level itself, within them whatever the levels are.
+struct FitPoints {
+    float lo, mid, hi;
+};
+__device__ __forceinline__ FitPoints points_of(int l, float left, float lv, float right)
+{
+    const float inf = __int_as_float(0x7f800000);
+    FitPoints p;
+    p.lo = l ? __fmul_rn(__fadd_rn(left, lv), 0.5f) : -inf;
+    p.hi = l < kLevels - 1 ? __fmul_rn(__fadd_rn(lv, right), 0.5f) : inf;
+    p.mid = fminf(fmaxf(lv, p.lo), p.hi);
+    return p;
+}
+
+// What the samples of a lane's half add to the error of level lv (levels that do not ascend have regions without samples).
+__device__ __forceinline__ double half_error(int lane, const FitPoints& p, float lv, const Below& begin, const Below& end)
+{
+    if (p.lo > p.hi) return 0.0;
+    const bool first = lane == 0;  // nothing lies in front of it
+    auto part = [&](double b, double e) { return e - (first ? 0.0 : b); };
+    const double s = part(begin.high.x, end.high.x) + part(begin.low.x, end.low.x);
+    const double x = part(begin.high.y, end.high.y) + part(begin.low.y, end.low.y);
+    return lane < kLevels ? (double)lv * s - x : x - (double)lv * s;
 }
 
 // Whether the difference of two sums {s, sx}, s0 and s1, is too rough to be a region's: small beside what was rounded (2^-20 of it; `rest`: what

@@ -1105,16 +1105,16 @@ constexpr int kFitMaeThreads = 2 * kFitThreads;  // a warp per threshold and lev
 // are there.  Sixteen more warps add up beside this what the error of the iteration needs, and warp 15, which has no threshold, writes
 // the error of the iteration before.
 //
-// The source, by a warp, results the same in all lanes:  weight(v): of what lies below v;  sums(v): {s, sx} of what lies below v;
+// The source, by a warp, results the same in all lanes:  weight(v): of what lies below v;  sums(v): {s, sx} of it;  all(): of everything;
 //              median(goal): the first sample with which the weight of all samples from the first on reaches the goal
 struct FitMaeShared {
     unsigned long long below[2][kLevels + 1];  // weight below threshold k - 1; entry 0: nothing, entry 16: everything
     float level[2][kLevels];
-    double err[2][2 * kLevels];                // parts of the error: the thresholds' and the levels'
+    Below at[2][2 * kLevels];                  // what lies below the levels, and below the thresholds above them
     int stop;
 };
 template <class Source>
-__device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, double2 everything, unsigned long long weight, const SortFit& F)
+__device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, unsigned long long weight, const SortFit& F)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < 2) S.below[tid][0] = 0ull, S.below[tid][kLevels] = weight;
@@ -1123,7 +1123,10 @@ __device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, do
     __syncthreads();
     // the error of iteration `at`, by warp 15
     auto error_of = [&](int at) {
-        double err = S.err[at & 1][lane];
+        const int l = lane & (kLevels - 1);
+        const float* const lvs = S.level[at & 1];
+        const FitPoints p = points_of(l, lvs[max(l - 1, 0)], lvs[l], lvs[min(l + 1, kLevels - 1)]);
+        double err = half_error(lane, p, lvs[l], S.at[at & 1][lower_end_of(lane)], S.at[at & 1][lane]);
 #pragma unroll
         for (int off = 16; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
         err = fmax(err, 0.0) / (double)F.n_total;
@@ -1132,28 +1135,25 @@ __device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, do
     };
     int iter = 0;
     if (warp >= kLevels) {
-        // ---- the error's parts of a threshold and of a level, beside the others' search for the next levels
+        // ---- what the error needs of a threshold and of a level, beside the others' search for the next levels
         const int l = warp - kLevels;
         float known = 0.0f;
-        double part = 0.0;
+        Below part = source.all();
+        if (l == kLevels - 1 && lane < 2) S.at[lane][2 * kLevels - 1] = part;
         for (; iter < F.iters; ++iter) {
             const int set = iter & 1;
-            const float lv = S.level[set][l];
+            const FitPoints at = points_of(l, S.level[set][max(l - 1, 0)], S.level[set][l], S.level[set][min(l + 1, kLevels - 1)]);
             if (l < kLevels - 1) {
-                const float above = S.level[set][l + 1];
-                const double2 p = source.sums(__fmul_rn(__fadd_rn(lv, above), 0.5f));
-                if (lane == 0) S.err[set][l] = 2.0 * p.y - ((double)lv + (double)above) * p.x;
-            } else if (lane == 0) {
-                S.err[set][l] = everything.y - (double)lv * everything.x;
+                const Below p = source.sums(at.hi);
+                if (lane == 0) S.at[set][kLevels + l] = p;
             }
             __syncthreads();
             if (S.stop) return;
-            if (iter == 0 || __float_as_uint(lv) != __float_as_uint(known)) {
-                const double2 p = source.sums(lv);
-                known = lv;
-                part = 2.0 * ((double)lv * p.x - p.y);
+            if (iter == 0 || __float_as_uint(at.mid) != __float_as_uint(known)) {
+                part = source.sums(at.mid);
+                known = at.mid;
             }
-            if (lane == 0) S.err[set][kLevels + l] = part;
+            if (lane == 0) S.at[set][l] = part;
             __syncthreads();
         }
         return;
@@ -1200,8 +1200,9 @@ __device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, do
 // searched one after the other, cut bins first).  Bound by its chain: three loads from L2 of 430 or 820 cycles each, the
 // reductions, two barriers; over 2^24 weights by the passes over the 500 samples of a bin (of up to 64 samples every lane adds
 // up what is not behind its own, in one pass: 2^20 weights 3.75 -> 3.1).
-constexpr int kMaeSums = ((kSortGroups + 1) * 8 + 15) / 16 * 16;  // shared memory: what lies in front of the groups: weights, {s, sx},
-constexpr int kMaeOff = kMaeSums + (kSortGroups + 1) * 16;      // first samples of the bins,
+constexpr int kMaeHigh = ((kSortGroups + 1) * 8 + 15) / 16 * 16;  // shared memory: what lies in front of the groups: weights, {s, sx},
+constexpr int kMaeLow = kMaeHigh + (kSortGroups + 1) * 16;      // high and low halves,
+constexpr int kMaeOff = kMaeLow + (kSortGroups + 1) * 16;       // first samples of the bins,
 constexpr int kMaeFirst = kMaeOff + kSortBins * 2 + 16;         // (and the end) of the groups
 constexpr int kMaeSmem = kMaeFirst + (kSortGroups + 1) * 4;
 
@@ -1209,7 +1210,7 @@ template <bool CROWDED>
 struct MaeSamples {
     const SortWs& W;
     const SampleWeight<true>& weights;
-    SharedTable<double2> group_sums;          // what lies in front of a group
+    SharedTable<double2> group_high, group_low;  // what lies in front of a group
     SharedTable<unsigned long long> group_a;
     SharedTable<uint16_t> off;
     SharedTable<uint32_t> group_first;
@@ -1270,16 +1271,17 @@ struct MaeSamples {
         const int g = below<false>(v, t);
         return warp_sum64(t.a) + group_a[g];
     }
-    __device__ __forceinline__ double2 sums(float v) const
+    __device__ __forceinline__ Below sums(float v) const
     {
         SortSums t;
-        const double2 g = group_sums[below<true>(v, t)];
+        const int g = below<true>(v, t);
         const bool h = threadIdx.x & 16;
         double u = (h ? t.sx : t.s) + __shfl_xor_sync(kFull, h ? t.s : t.sx, 16);
 #pragma unroll
         for (int o = 8; o; o >>= 1) u += __shfl_xor_sync(kFull, u, o);
-        return make_double2(g.x + __shfl_sync(kFull, u, 0), g.y + __shfl_sync(kFull, u, 16));
+        return below_of(group_high[g], group_low[g], make_double2(__shfl_sync(kFull, u, 0), __shfl_sync(kFull, u, 16)));
     }
+    __device__ __forceinline__ Below all() const { return Below{group_high[kSortGroups], group_low[kSortGroups]}; }
     __device__ __forceinline__ float median(unsigned long long goal) const
     {
         // the last group in front of which there is less than the goal: 32 groups of 64, then one of 64
@@ -1393,7 +1395,8 @@ sort_fit_mae_kernel(const __grid_constant__ SortWs W, const __grid_constant__ So
     if ((W.n_items[4] != 0u) != CROWDED) return;
     extern __shared__ __align__(16) unsigned char s_fit[];
     unsigned long long* const s_a = reinterpret_cast<unsigned long long*>(s_fit);
-    double2* const s_sums = reinterpret_cast<double2*>(s_fit + kMaeSums);
+    double2* const s_high = reinterpret_cast<double2*>(s_fit + kMaeHigh);
+    double2* const s_low = reinterpret_cast<double2*>(s_fit + kMaeLow);
     uint16_t* const s_off = reinterpret_cast<uint16_t*>(s_fit + kMaeOff);
     uint32_t* const s_first = reinterpret_cast<uint32_t*>(s_fit + kMaeFirst);
     __shared__ FitMaeShared S;
@@ -1401,15 +1404,23 @@ sort_fit_mae_kernel(const __grid_constant__ SortWs W, const __grid_constant__ So
     weights.max_bits = W.n_items[1];
     weights.unit = F.metric >= 2;
     if (threadIdx.x == 0) s_off[kSortBins] = 0u;
-    copy_starts(W, s_off, s_first);
-    running_sums<kSortGroups / kFitThreads, PairSum>(kSortGroups, [&](int g) { return PairSum{W.group[g].s, W.group[g].sx}; },
-                                                     [&](int g, const PairSum& v) { s_sums[g] = make_double2(v.s, v.sx); });
-    running_sums<kSortGroups / kFitThreads, unsigned long long>(kSortGroups, [&](int g) { return W.group[g].a; },
-                                                                [&](int g, unsigned long long v) { s_a[g] = v; });
+    SortSums* const s_group = reinterpret_cast<SortSums*>(s_high);  // the groups' sums, before the running sums take their place
+    static_assert(kSortGroups * sizeof(SortSums) <= 2 * (kSortGroups + 1) * sizeof(double2), "room for the groups' sums");
+    copy_in(s_group, W.group, kSortGroups * (int)sizeof(SortSums));
     copies_done();
     __syncthreads();
-    MaeSamples<CROWDED> source{W, weights, SharedTable(s_sums), SharedTable(s_a), SharedTable(s_off), SharedTable(s_first)};
-    fit_mae_loop(source, S, s_sums[kSortGroups], s_a[kSortGroups], F);
+    copy_starts(W, s_off, s_first);
+    running_sums<kSortGroups / kFitThreads, unsigned long long>(kSortGroups, [&](int g) { return s_group[g].a; },
+                                                                [&](int g, unsigned long long v) { s_a[g] = v; });
+    running_sums<kSortGroups / kFitThreads, TwoPair>(kSortGroups, [&](int g) { return TwoPair{{s_group[g].s, 0.0}, {s_group[g].sx, 0.0}}; },
+                                                     [&](int g, const TwoPair& v) {
+                                                         s_high[g] = make_double2(v.s.h, v.x.h);
+                                                         s_low[g] = make_double2(v.s.l, v.x.l);
+                                                     });
+    copies_done();
+    __syncthreads();
+    MaeSamples<CROWDED> source{W, weights, SharedTable(s_high), SharedTable(s_low), SharedTable(s_a), SharedTable(s_off), SharedTable(s_first)};
+    fit_mae_loop(source, S, s_a[kSortGroups], F);
 }
 
 // ---------------------------------------------------------------- host side

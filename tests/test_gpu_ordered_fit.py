@@ -308,3 +308,37 @@ def test_a_light_region_among_distinct_weights(bof4):
     assert ref[12] != lv[12]
     np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=1e-7)
     np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5)
+
+
+def _absolute_error(w, lv, I=64):
+    """Mean of |m| |x - level| over the weights (whole blocks), absolute normalisation, and the mean of |w|, in long double."""
+    b = w.float().numpy().reshape(-1, I)
+    m = np.abs(b).max(1, keepdims=True)
+    x = np.divide(b, m, out=np.zeros_like(b), where=m > 0)
+    lv = np.asarray(lv, np.float32)
+    level = lv[np.searchsorted((lv[:-1] + lv[1:]) * np.float32(0.5), x, side="right")]
+    m = m.astype(np.longdouble)
+    n = np.longdouble(b.size)
+    return (np.abs(x.astype(np.longdouble) - level) * m).sum() / n, (np.abs(x.astype(np.longdouble)) * m).sum() / n
+
+
+@pytest.mark.parametrize("n,dtype", [(1 << 14, torch.float32), (1 << 18, torch.float32), (1 << 20, torch.float32), (1 << 21, torch.bfloat16)])
+@pytest.mark.parametrize("kind", ["plain", "levels"])
+def test_the_absolute_error_is_added_up_by_regions(bof4, n, dtype, kind):
+    """The logged error against sums in long double.  A half region is the difference of two sums in two doubles each, so what is
+    left is the rounding of the halves, 2^-53 of each and of random sign: less than 2^-53 of the mean of |w| in all.  (As 32 differences
+    of sums over all the data, each in one double, it would be 2^-51 to 2^-50.)  "levels": most weights lie on one."""
+    lv, _ = bof4.bof4_default_init(0)
+    for seed in range(4):
+        w = _weights(n, torch.float32, 40 + seed, "plain")
+        if kind == "levels":
+            g = torch.Generator().manual_seed(seed)
+            w = torch.randint(-1, 9, (n // 64, 64), generator=g).float() / 8
+            w = torch.where(w < 0, -1.0, w)
+            w[:, 0] = 1.0
+            w = (w * (0.5 + torch.rand(n // 64, 1, generator=g))).reshape(-1)
+        w = w.to(dtype)
+        _, log = bof4.bof4_fit_codebook(w.cuda(), 64, 0, bof4.METRIC_MAE, lv, 0xffff, 12)
+        ref, mean = _absolute_error(w, lv)
+        assert abs(log[0].item() - ref) <= 2.0 ** -53 * mean, (seed, float((log[0].item() - ref) / mean))
+        assert (log == log[0]).all()
