@@ -161,15 +161,16 @@ __device__ __forceinline__ double half_error(int lane, const FitPoints& p, float
     return lane < kLevels ? (double)lv * s - x : x - (double)lv * s;
 }
 
-// Whether the difference of two sums {s, sx}, s0 and s1, is too rough to be a region's: small beside what was rounded (2^-20 of it; `rest`: what
-// was in the two sums) or beside all that lies in front (2^-50), negative, or not finite.  By the upper halves of the
-// doubles, whose exponents begin at bit 20.
-__device__ __forceinline__ bool too_rough(double s0, double s1, double2 rest0, double2 rest1, double front)
+// Whether the difference of two sums {s, sx}, s0 and s1, is too rough to be a region's: not finite, negative, or small beside all that lies
+// in front (2^-50) or beside what was rounded: the `rest` of either sum, and what is compared with it is what the region is known to
+// hold.  Its weight is s0; of sum |weight x|, which s1 may cancel, the upper rest is a part if the points have different parts in
+// front of them.  By the upper halves of the doubles, whose exponents begin at bit 20.
+__device__ __forceinline__ bool too_rough(double s0, double s1, double2 rest0, double2 rest1, double front0, double front1)
 {
     auto top = [](double d) { return __double2hiint(d) & 0x7fffffff; };
-    const int least0 = max(max(top(rest0.x), top(rest1.x)) - (20 << 20), top(front) - (50 << 20)), least1 = max(top(rest0.y), top(rest1.y)) - (20 << 20);
-    const int t0 = __double2hiint(s0), t1 = top(s1);
-    return t0 < max(least0, 0) || t1 < least1 || max(t0, t1) >= 0x7ff00000;
+    const int t0 = __double2hiint(s0), t1 = top(s1), held = front0 != front1 ? max(t1, top(rest1.y)) : t1;
+    const int least0 = max(max(top(rest0.x), top(rest1.x)) - (20 << 20), top(front1) - (50 << 20));
+    return t0 < max(least0, 0) || held < top(rest0.y) - (20 << 20) || max(t0, t1) >= 0x7ff00000;
 }
 
 }  // namespace bof4
