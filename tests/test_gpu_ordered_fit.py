@@ -373,3 +373,45 @@ def test_a_level_at_zero_costs_what_others_do(bof4, mask):
     other = lv.copy()
     other[8] = 0.11
     assert _iteration_us(bof4, w, lv, mask, 0) < 1.35 * _iteration_us(bof4, w, other, 0x81c1, 0)
+
+
+def _halfway(dtype, seed):
+    """Weights with a region of which the level lies exactly halfway between two floats, and sums are exact if they are added up by
+    themselves: its blocks' constant is a power of two.  Its weight is 2^-18 of what lies below it in the same group of bins (of
+    places), where constants are arbitrary and sums are rounded.  Returns the weights, the levels, the free level's index and value."""
+    g = torch.Generator().manual_seed(seed)
+    lv = np.linspace(-1, 1, 16).astype(np.float32)
+    if dtype == torch.float32:
+        u = torch.rand(64, 64, generator=g)
+        w = torch.where(torch.rand(64, 64, generator=g) < 0.5, 0.49991 + 2e-5 * u, 0.50007 + 2e-5 * u)
+        w[:, 0] = 1.0
+        w *= 0.5 + 0.5 * torch.rand(64, 1, generator=g)
+        a = np.float32(0.49999) + np.float32(2.0 ** -24) * np.float32(seed)
+        b = np.nextafter(a, np.float32(1))
+        lv[10:14] = 0.4, 0.4999, 0.50001, 0.5001
+        x = torch.zeros(64 * 63)
+        x[:1999], x[1999:2 * 1999] = float(a), float(b)     # (the sums have bits that the others' are rounded by)
+        light = torch.cat([torch.ones(64, 1), x.view(64, 63)], 1)
+        return torch.cat([w, light * 2.0 ** -10]).reshape(-1), lv, 12, np.float32((np.float64(a) + np.float64(b)) / 2)
+    blocks, samples = 2081, 1 << 17
+    m = torch.randint(192, 256, ((1 << 15) - blocks, 1), generator=g).float()
+    w = torch.where(torch.rand(len(m), 64, generator=g) < 0.5, (m - 1) / 2, m / 8)    # (m - 1) / 2 m: from 0.4973 to 0.498
+    w[:, :1] = m
+    w /= 256
+    high = 2 * int(torch.randint(1 << 13, 1 << 15, (1,), generator=g)) + 1
+    x = torch.zeros(blocks * 63)
+    x[:samples] = 0.5
+    x[:high] = 129 / 256
+    light = torch.cat([torch.ones(blocks, 1), x[torch.randperm(len(x), generator=g)].view(blocks, 63)], 1)
+    lv[10:14] = 0.4, 0.498, 0.5005, 0.51
+    return torch.cat([w, light * 2.0 ** -8]).to(dtype).reshape(-1), lv, 12, np.float32(0.5 + high * 2.0 ** -25)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_a_light_region_is_as_exact_as_by_itself(bof4, dtype):
+    """As the difference of rounded sums its level would be off by 2^-34, which decides to which side a level halfway between two
+    floats is rounded: to the even one if it is exact."""
+    for seed in range(16):
+        w, lv, free, level = _halfway(dtype, seed)
+        cb, _ = bof4.bof4_fit_codebook(w.cuda(), 64, 0, 0, lv, 0xffff ^ (1 << free), 8)
+        assert cb[free].item() == level, seed
