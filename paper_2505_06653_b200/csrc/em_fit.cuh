@@ -3,10 +3,10 @@
 //
 // An iteration is a chain of latencies, so it is kept short: what lies below a threshold is one sum, and a region is the difference of
 // two such sums.  The sums of large parts of the samples are kept in two doubles each, so that their difference is as good as
-// adding the region up; the rest is rounded once to a double.  For the squared error a region that is light beside this rest
-// (an eighth, so that its weight is good to 2^-50), or stands beside sums that are not finite, is added up by itself; the absolute error, which only goes to the log, is known to
-// the rounding of these differences, 2^-53 of the weight in each (with one double for a sum over all parts it was off by 30 times as much).
-// The weights of the medians are integers.
+// adding the region up; the rest is rounded once to a double.  For the squared error a region that is light beside this rest (2^-8, so that
+// its level is good to 2^-45), or stands beside sums that are not finite, is added up by itself; the absolute error, which only goes to the
+// log, is known to the rounding of these differences, 2^-53 of the weight in each (with one double for a sum over all parts it was off by 30
+// times as much).  The weights of the medians are integers.
 //
 // When an iteration leaves every level unchanged the remaining ones would repeat it bit for bit: their entries of the error log
 // are filled in and the loop ends.
@@ -162,15 +162,15 @@ __device__ __forceinline__ double half_error(int lane, const FitPoints& p, float
 }
 
 // Whether the difference of two sums {s, sx}, s0 and s1, is too rough to be a region's: not finite, negative, or small beside all that lies
-// in front (2^-50) or beside what was rounded: the `rest` of either sum, and what is compared with it is what the region is known to
-// hold.  Its weight is s0 (2^-3 of the rests); of sum |weight x|, which s1 may cancel, the upper rest is a part if the points have different
-// parts in front of them (2^-8: thresholds at random places of their parts would be below 2^-3 in one of ten iterations).  By the upper
-// halves of the doubles, whose exponents begin at bit 20.
+// in front (2^-50) or beside what was rounded, the `rest` of either sum (2^-8).  What is compared with it is what the region is known to
+// hold: its weight, s0, and of sum |weight x|, which s1 may cancel, the upper rest if the points have different parts in front of them.
+// (From 2^-3 on all regions go the long way where one group of bins holds all the data: 2^20 weights 53 us an iteration, 16 this way.)  By
+// the upper halves of the doubles, whose exponents begin at bit 20.
 __device__ __forceinline__ bool too_rough(double s0, double s1, double2 rest0, double2 rest1, double front0, double front1)
 {
     auto top = [](double d) { return __double2hiint(d) & 0x7fffffff; };
     const int t0 = __double2hiint(s0), t1 = top(s1), held = front0 != front1 ? max(t1, top(rest1.y)) : t1;
-    const int least0 = max(max(top(rest0.x), top(rest1.x)) - (3 << 20), top(front1) - (50 << 20));
+    const int least0 = max(max(top(rest0.x), top(rest1.x)) - (8 << 20), top(front1) - (50 << 20));
     return t0 < max(least0, 0) || held < top(rest0.y) - (8 << 20) || max(t0, t1) >= 0x7ff00000;
 }
 
