@@ -445,12 +445,12 @@ cells_fit_mae_kernel(const __grid_constant__ CellsWs W, const __grid_constant__ 
     copy_in(s_a, W.part_a, kCellPartsAll * 8);
     copies_done();
     __syncthreads();
-    running_sums<kCellPer, TwoPair>(kCellBlocks, [&](int b) { return TwoPair{{s_block[b].s, 0.0}, {s_block[b].sx, 0.0}}; },
+    running_sums<kCellPer, TwoPair>(warp < kLevels, kCellBlocks, [&](int b) { return TwoPair{{s_block[b].s, 0.0}, {s_block[b].sx, 0.0}}; },
                                     [&](int b, const TwoPair& v) {
                                         s_high[b] = make_double2(v.s.h, v.x.h);
                                         s_low[b] = make_double2(v.s.l, v.x.l);
                                     });
-    running_sums<kCellPartsAll / kFitThreads + 1, unsigned long long>(kCellPartsAll, [&](int p) { return s_a[p]; },
+    running_sums<kCellPartsAll / kFitThreads + 1, unsigned long long>(warp < kLevels, kCellPartsAll, [&](int p) { return s_a[p]; },
                                                                      [&](int p, unsigned long long v) { s_a[p] = v; });
     __syncthreads();
     const SharedTable<uint16_t> value_of(s_value);

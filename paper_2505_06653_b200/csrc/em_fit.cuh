@@ -83,15 +83,15 @@ __device__ __forceinline__ TwoPair shfl_up(const TwoPair& v, int off) { return T
 __device__ __forceinline__ TwoSum two_shfl(const TwoSum& a, int from) { return TwoSum{__shfl_sync(kFull, a.h, from), __shfl_sync(kFull, a.l, from)}; }
 __device__ __forceinline__ TwoPair shfl(const TwoPair& v, int from) { return TwoPair{two_shfl(v.s, from), two_shfl(v.x, from)}; }
 
-// put(k, sum of part(0) ... part(k - 1)), k = 0 ... n, by all threads of the CTA; n <= PER * kFitThreads.  All parts have been read before
-// anything is put, so a sum may take the place of its part.  (The parts come from shared memory, see copy_in: a thread's are
-// neighbours, and the lines that they share do not stay in the L1 that the tables leave: read from global memory, 11 us more for the cells.)
+// put(k, sum of part(0) ... part(k - 1)), k = 0 ... n <= PER * kFitThreads, by the CTA's first kFitThreads threads or its next ones (`has`;
+// the others only pass the barrier).  All parts have been read before anything is put, so a sum may take the place of its part.
+// (The cells' parts come from shared memory, see copy_in: a thread's are neighbours, and the lines that they share do not stay in the
+// L1 that those tables leave: read from global memory, 11 us more.)
 template <int PER, class T, class Part, class Put>
-__device__ __forceinline__ void running_sums(int n, Part part, Put put)
+__device__ __forceinline__ void running_sums(bool has, int n, Part part, Put put)
 {
     __shared__ T s_warp[kLevels];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool has = warp < kLevels;
+    const int tid = threadIdx.x & (kFitThreads - 1), lane = tid & 31, warp = tid >> 5;
     T v[PER], t{};
     auto scan = [&](T& u, int width) {  // inclusive, over the first `width` lanes of the warp
 #pragma unroll
@@ -129,7 +129,6 @@ __device__ __forceinline__ void running_sums(int n, Part part, Put put)
 struct Below {
     double2 high, low;
 };
-__device__ __forceinline__ Below below_of(double2 high, double2 low, double2 rest) { return Below{high, make_double2(low.x + rest.x, low.y + rest.y)}; }
 
 // The absolute error is added up half region by half region, each the difference of two such sums.  Lane l has what lies below level l,
 // lane 16 + l what lies below the threshold above it (lane 31: everything): a lane's half ends there and begins at the point of the

@@ -1105,7 +1105,8 @@ constexpr int kFitMaeThreads = 2 * kFitThreads;  // a warp per threshold and lev
 // are there.  Sixteen more warps add up beside this what the error of the iteration needs, and warp 15, which has no threshold, writes
 // the error of the iteration before.
 //
-// The source, by a warp, results the same in all lanes:  weight(v): of what lies below v;  sums(v): {s, sx} of it;  all(): of everything;
+// The source, by a warp, results the same in all lanes:  weight(v): of what lies below v;  sums(v): {s, sx} of it, all(): of everything, in
+//              lanes 0 to 3 the doubles of a Below;
 //              median(goal): the first sample with which the weight of all samples from the first on reaches the goal
 struct FitMaeShared {
     unsigned long long below[2][kLevels + 1];  // weight below threshold k - 1; entry 0: nothing, entry 16: everything
@@ -1138,22 +1139,22 @@ __device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, un
         // ---- what the error needs of a threshold and of a level, beside the others' search for the next levels
         const int l = warp - kLevels;
         float known = 0.0f;
-        Below part = source.all();
-        if (l == kLevels - 1 && lane < 2) S.at[lane][2 * kLevels - 1] = part;
+        double part = source.all();
+        auto put = [&](int set, int at, double v) {
+            if (lane < 4) reinterpret_cast<double*>(&S.at[set][at])[lane] = v;
+        };
+        if (l == kLevels - 1) put(0, 2 * kLevels - 1, part), put(1, 2 * kLevels - 1, part);
         for (; iter < F.iters; ++iter) {
             const int set = iter & 1;
             const FitPoints at = points_of(l, S.level[set][max(l - 1, 0)], S.level[set][l], S.level[set][min(l + 1, kLevels - 1)]);
-            if (l < kLevels - 1) {
-                const Below p = source.sums(at.hi);
-                if (lane == 0) S.at[set][kLevels + l] = p;
-            }
+            if (l < kLevels - 1) put(set, kLevels + l, source.sums(at.hi));
             __syncthreads();
             if (S.stop) return;
             if (iter == 0 || __float_as_uint(at.mid) != __float_as_uint(known)) {
                 part = source.sums(at.mid);
                 known = at.mid;
             }
-            if (lane == 0) S.at[set][l] = part;
+            put(set, l, part);
             __syncthreads();
         }
         return;
@@ -1200,9 +1201,7 @@ __device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, un
 // searched one after the other, cut bins first).  Bound by its chain: three loads from L2 of 430 or 820 cycles each, the
 // reductions, two barriers; over 2^24 weights by the passes over the 500 samples of a bin (of up to 64 samples every lane adds
 // up what is not behind its own, in one pass: 2^20 weights 3.75 -> 3.1).
-constexpr int kMaeHigh = ((kSortGroups + 1) * 8 + 15) / 16 * 16;  // shared memory: what lies in front of the groups: weights, {s, sx},
-constexpr int kMaeLow = kMaeHigh + (kSortGroups + 1) * 16;      // high and low halves,
-constexpr int kMaeOff = kMaeLow + (kSortGroups + 1) * 16;       // first samples of the bins,
+constexpr int kMaeOff = ((kSortGroups + 1) * 8 + 15) / 16 * 16;  // shared memory: weights in front of the groups, first samples of the bins,
 constexpr int kMaeFirst = kMaeOff + kSortBins * 2 + 16;         // (and the end) of the groups
 constexpr int kMaeSmem = kMaeFirst + (kSortGroups + 1) * 4;
 
@@ -1210,7 +1209,7 @@ template <bool CROWDED>
 struct MaeSamples {
     const SortWs& W;
     const SampleWeight<true>& weights;
-    SharedTable<double2> group_high, group_low;  // what lies in front of a group
+    const double* group_sums;                 // what lies in front of a group, the four doubles of a Below
     SharedTable<unsigned long long> group_a;
     SharedTable<uint16_t> off;
     SharedTable<uint32_t> group_first;
@@ -1219,9 +1218,10 @@ struct MaeSamples {
         const uint32_t o = off[b], f = group_first[b / kSortGroup];
         return o == kFarBin ? __ldg(W.start + b) : f + o;
     }
-    // This lane's share of what lies below v, less the whole groups in front of the one that is returned.
+    // This lane's share of what lies below v, less the whole groups in front of the one that is returned; what lies in front of that one, a double
+    // to a lane (asked for before the samples).
     template <bool SUMS>
-    __device__ __forceinline__ int below(float v, SortSums& t) const
+    __device__ __forceinline__ int below(float v, SortSums& t, double& front) const
     {
         const int lane = threadIdx.x & 31;
         const int b = sort_bin(v);
@@ -1231,6 +1231,7 @@ struct MaeSamples {
         t = SortSums{0.0, 0.0, 0ull};
         const unsigned long long pre =
             __ldg(reinterpret_cast<const unsigned long long*>(W.pre + min(at, kSortBins - 1)) + (SUMS ? (lane & 1) : 2));
+        if (SUMS) front = group_sums[4 * (at / kSortGroup) + (lane & 3)];
         if (CROWDED && to - from > kSortCrowd) {
             crowded_sums<true>(W, weights, from, to, -__int_as_float(0x7f800000), v, t);
         } else {
@@ -1268,20 +1269,24 @@ struct MaeSamples {
     __device__ __forceinline__ unsigned long long weight(float v) const
     {
         SortSums t;
-        const int g = below<false>(v, t);
+        double none;
+        const int g = below<false>(v, t, none);
         return warp_sum64(t.a) + group_a[g];
     }
-    __device__ __forceinline__ Below sums(float v) const
+    __device__ __forceinline__ double sums(float v) const
     {
         SortSums t;
-        const int g = below<true>(v, t);
-        const bool h = threadIdx.x & 16;
+        double front;
+        below<true>(v, t, front);
+        const int lane = threadIdx.x & 31;
+        const bool h = lane & 16;
         double u = (h ? t.sx : t.s) + __shfl_xor_sync(kFull, h ? t.s : t.sx, 16);
 #pragma unroll
         for (int o = 8; o; o >>= 1) u += __shfl_xor_sync(kFull, u, o);
-        return below_of(group_high[g], group_low[g], make_double2(__shfl_sync(kFull, u, 0), __shfl_sync(kFull, u, 16)));
+        const double rest = __shfl_sync(kFull, u, lane & 1 ? 16 : 0);
+        return (lane & 2) ? front + rest : front;
     }
-    __device__ __forceinline__ Below all() const { return Below{group_high[kSortGroups], group_low[kSortGroups]}; }
+    __device__ __forceinline__ double all() const { return group_sums[4 * kSortGroups + (threadIdx.x & 3)]; }
     __device__ __forceinline__ float median(unsigned long long goal) const
     {
         // the last group in front of which there is less than the goal: 32 groups of 64, then one of 64
@@ -1395,8 +1400,6 @@ sort_fit_mae_kernel(const __grid_constant__ SortWs W, const __grid_constant__ So
     if ((W.n_items[4] != 0u) != CROWDED) return;
     extern __shared__ __align__(16) unsigned char s_fit[];
     unsigned long long* const s_a = reinterpret_cast<unsigned long long*>(s_fit);
-    double2* const s_high = reinterpret_cast<double2*>(s_fit + kMaeHigh);
-    double2* const s_low = reinterpret_cast<double2*>(s_fit + kMaeLow);
     uint16_t* const s_off = reinterpret_cast<uint16_t*>(s_fit + kMaeOff);
     uint32_t* const s_first = reinterpret_cast<uint32_t*>(s_fit + kMaeFirst);
     __shared__ FitMaeShared S;
@@ -1404,22 +1407,22 @@ sort_fit_mae_kernel(const __grid_constant__ SortWs W, const __grid_constant__ So
     weights.max_bits = W.n_items[1];
     weights.unit = F.metric >= 2;
     if (threadIdx.x == 0) s_off[kSortBins] = 0u;
-    SortSums* const s_group = reinterpret_cast<SortSums*>(s_high);  // the groups' sums, before the running sums take their place
-    static_assert(kSortGroups * sizeof(SortSums) <= 2 * (kSortGroups + 1) * sizeof(double2), "room for the groups' sums");
-    copy_in(s_group, W.group, kSortGroups * (int)sizeof(SortSums));
-    copies_done();
-    __syncthreads();
     copy_starts(W, s_off, s_first);
-    running_sums<kSortGroups / kFitThreads, unsigned long long>(kSortGroups, [&](int g) { return s_group[g].a; },
-                                                                [&](int g, unsigned long long v) { s_a[g] = v; });
-    running_sums<kSortGroups / kFitThreads, TwoPair>(kSortGroups, [&](int g) { return TwoPair{{s_group[g].s, 0.0}, {s_group[g].sx, 0.0}}; },
-                                                     [&](int g, const TwoPair& v) {
-                                                         s_high[g] = make_double2(v.s.h, v.x.h);
-                                                         s_low[g] = make_double2(v.s.l, v.x.l);
-                                                     });
+    // What lies in front of the groups goes where the digits' counts were, which have served: in shared memory beside the first samples it would leave
+    // 28 KB of L1, and bisections in crowded bins live on L1 (2^20 weights in two bins 58 us an iteration, 68 without it).
+    static_assert((kSortGroups + 1) * sizeof(Below) <= (size_t)kSortGrid * 256 * 4, "room for the running sums");
+    Below* const sums = reinterpret_cast<Below*>(W.counts);
+    if (threadIdx.x < kFitThreads)
+        running_sums<kSortGroups / kFitThreads, TwoPair>(true, kSortGroups, [&](int g) { return TwoPair{{W.group[g].s, 0.0}, {W.group[g].sx, 0.0}}; },
+                                                         [&](int g, const TwoPair& v) {
+                                                             sums[g] = Below{make_double2(v.s.h, v.x.h), make_double2(v.s.l, v.x.l)};
+                                                         });
+    else
+        running_sums<kSortGroups / kFitThreads, unsigned long long>(true, kSortGroups, [&](int g) { return W.group[g].a; },
+                                                                    [&](int g, unsigned long long v) { s_a[g] = v; });
     copies_done();
     __syncthreads();
-    MaeSamples<CROWDED> source{W, weights, SharedTable(s_high), SharedTable(s_low), SharedTable(s_a), SharedTable(s_off), SharedTable(s_first)};
+    MaeSamples<CROWDED> source{W, weights, reinterpret_cast<const double*>(sums), SharedTable(s_a), SharedTable(s_off), SharedTable(s_first)};
     fit_mae_loop(source, S, s_a[kSortGroups], F);
 }
 
