@@ -344,23 +344,24 @@ def test_the_absolute_error_is_added_up_by_regions(bof4, n, dtype, kind):
         assert (log == log[0]).all()
 
 
-def _iteration_us(bof4, w, lv, mask, metric):
-    """Time of an iteration: 100 less 20 of them, with the launches queued behind a wait so that the host's time is not in it."""
-    room = torch.empty(bof4.bof4_fit_workspace_bytes(w.numel(), bof4.F32, 64, metric, 100), dtype=torch.uint8, device="cuda")
+def _best_ms(bof4, w, lv, mask, metric, iters):
+    """Time of a fit, with the launches queued behind a wait so that the host's time is not in it."""
+    room = torch.empty(bof4.bof4_fit_workspace_bytes(w.numel(), bof4.F32, 64, metric, iters), dtype=torch.uint8, device="cuda")
+    best = 1e9
+    for _ in range(9):
+        s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda._sleep(2_000_000)
+        s.record()
+        bof4.bof4_fit_codebook(w, 64, 0, metric, lv, mask, iters, workspace=room, sync=False)
+        e.record()
+        torch.cuda.synchronize()
+        best = min(best, s.elapsed_time(e))
+    return best
 
-    def best(iters):
-        out = 1e9
-        for _ in range(9):
-            s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            torch.cuda._sleep(2_000_000)
-            s.record()
-            bof4.bof4_fit_codebook(w, 64, 0, metric, lv, mask, iters, workspace=room, sync=False)
-            e.record()
-            torch.cuda.synchronize()
-            out = min(out, s.elapsed_time(e))
-        return out
-    best(20)
-    return (best(100) - best(20)) / 80 * 1000
+
+def _iteration_us(bof4, w, lv, mask, metric):
+    """100 iterations less 20."""
+    return (_best_ms(bof4, w, lv, mask, metric, 100) - _best_ms(bof4, w, lv, mask, metric, 20)) / 80 * 1000
 
 
 @pytest.mark.parametrize("mask", [0x81c1, 0x8141])
@@ -415,3 +416,10 @@ def test_a_light_region_is_as_exact_as_by_itself(bof4, dtype):
         w, lv, free, level = _halfway(dtype, seed)
         cb, _ = bof4.bof4_fit_codebook(w.cuda(), 64, 0, 0, lv, 0xffff ^ (1 << free), 8)
         assert cb[free].item() == level, seed
+
+
+def test_a_median_in_a_crowded_bin_is_looked_for_between_its_thresholds(bof4):
+    """2^20 weights about zero, all thresholds in the outermost bins of it: 18 iterations 1.8 ms.  Among all samples of a bin, whose keys
+    span fourteen binades, and from nowhere in particular, they took 3.4."""
+    w, lv = _crowded(1 << 20, "tiny", 11)
+    assert _best_ms(bof4, w.cuda(), lv, 0x8000, bof4.METRIC_MAE, 18) < 2.6
