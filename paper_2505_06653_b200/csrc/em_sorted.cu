@@ -548,13 +548,15 @@ __device__ __forceinline__ SortSums sums_before(const SortWs& W, const SampleWei
     return t;
 }
 
-// This lane's share of the samples of a crowded bin, from ... to - 1, with p <= x < q; the warp's lanes together have all.
+// This lane's share of the samples of a crowded bin, from ... to - 1, with p <= x < q; the warp's lanes together have all.  (Nothing is looked
+// for where p is minus infinity, as it is for what lies below a threshold: 2^20 weights in two bins, squared error, 16.2 -> 11.1 us an iteration.)
 template <bool MAE>
 __device__ __noinline__ void crowded_sums(const SortWs& W, const SampleWeight<MAE>& weight, uint32_t from, uint32_t to, float p,
                                           float q, SortSums& t)
 {
     constexpr int U = kWindowsPerLane;
     const uint32_t last = (to - 1) / kSortWindow;
+    const bool cut = p > -__int_as_float(0x7f800000);
     for (uint32_t w0 = from / kSortWindow + (threadIdx.x & 31); w0 <= last; w0 += 32 * U) {
         uint32_t lo[U], hi[U], at_p[U], at_q[U];
 #pragma unroll
@@ -568,7 +570,7 @@ __device__ __noinline__ void crowded_sums(const SortWs& W, const SampleWeight<MA
         for (uint32_t step = kSortWindow; step; step >>= 1) {
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                if (at_p[u] + step <= hi[u] && W.b[at_p[u] + step - 1].x < p) at_p[u] += step;
+                if (cut && at_p[u] + step <= hi[u] && W.b[at_p[u] + step - 1].x < p) at_p[u] += step;
                 if (at_q[u] + step <= hi[u] && W.b[at_q[u] + step - 1].x < q) at_q[u] += step;
             }
         }
