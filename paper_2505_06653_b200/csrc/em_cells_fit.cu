@@ -345,35 +345,11 @@ cells_fit_mse_kernel(const __grid_constant__ CellsWs W, const __grid_constant__ 
         s_cut[tid][0] = make_float2(-inf, __uint_as_float(0u));
         s_cut[tid][kLevels] = make_float2(inf, __uint_as_float((uint32_t)kCellPlaces));
     }
-    int iter = 0;
     if (last) {
-        // Iteration by iteration, beside the others' next one: the error, and whether the levels have stopped to move.
-        float before = __int_as_float(0x7fc00001);
-        double err = 0.0;
-        for (; iter < F.iters; ++iter) {
-            const int set = iter & 1;
-            __syncthreads();
-            if (s_stop <= iter) break;
-            lv = s_level[set][mine];
-            const double2 h0 = s_below[set][0][mine], h1 = s_below[set][0][mine + 1], l0 = s_below[set][1][mine], l1 = s_below[set][1][mine + 1];
-            const double2 r0 = s_below[set][2][mine], r1 = s_below[set][2][mine + 1];
-            const double s0 = ((h1.x - h0.x) + (l1.x - l0.x)) + (r1.x - r0.x);
-            const double s1 = ((h1.y - h0.y) + (l1.y - l0.y)) + (r1.y - r0.y);
-            const double o = (double)lv;
-            err = o * (2.0 * s1 - o * s0);
-#pragma unroll
-            for (int off = 8; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
-            err = fmax(w2 - err, 0.0) / (double)F.n_total;
-            if (lane == 0 && F.err_log) F.err_log[iter] = err;
-            if (__all_sync(kFull, __float_as_uint(lv) == __float_as_uint(before)) && lane == 0) s_stop = iter + 1;
-            before = lv;
-        }
-        err = __shfl_sync(kFull, err, 0);
-        if (F.err_log)
-            for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = err;
+        squared_errors(F, w2, s_level, s_below, s_stop);
         return;
     }
-    for (; iter < F.iters; ++iter) {
+    for (int iter = 0; iter < F.iters; ++iter) {
         const int set = iter & 1;
         const float p = __fmul_rn(__fadd_rn(lv, __shfl_xor_sync(kFull, lv, 1)), 0.5f);
         const int place = place_of<32>(p, value_of);

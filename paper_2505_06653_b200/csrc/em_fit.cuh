@@ -160,6 +160,37 @@ __device__ __forceinline__ double half_error(int lane, const FitPoints& p, float
     return lane < kLevels ? (double)lv * s - x : x - (double)lv * s;
 }
 
+// The last warp of a fit of squared errors.  Iteration by iteration, beside the others' next one: the error, and whether the levels have
+// stopped to move (`stop`: the iteration behind whose barrier all leave).  w2: the sum of squares of all samples.
+__device__ __forceinline__ void squared_errors(const SortFit& F, double w2, const float (&level)[2][kLevels], const double2 (&below)[2][3][kLevels + 1], int& stop)
+{
+    const int lane = threadIdx.x & 31, l = lane & (kLevels - 1);
+    float before = __int_as_float(0x7fc00001);
+    double err = 0.0;
+    int iter = 0;
+    for (; iter < F.iters; ++iter) {
+        const int set = iter & 1;
+        __syncthreads();
+        if (stop <= iter) break;
+        const float lv = level[set][l];
+        const double2 h0 = below[set][0][l], h1 = below[set][0][l + 1], l0 = below[set][1][l], l1 = below[set][1][l + 1];
+        const double2 r0 = below[set][2][l], r1 = below[set][2][l + 1];
+        const double s0 = ((h1.x - h0.x) + (l1.x - l0.x)) + (r1.x - r0.x);
+        const double s1 = ((h1.y - h0.y) + (l1.y - l0.y)) + (r1.y - r0.y);
+        const double o = (double)lv;
+        err = o * (2.0 * s1 - o * s0);
+#pragma unroll
+        for (int off = 8; off; off >>= 1) err += __shfl_xor_sync(kFull, err, off);
+        err = fmax(w2 - err, 0.0) / (double)F.n_total;
+        if (lane == 0 && F.err_log) F.err_log[iter] = err;
+        if (__all_sync(kFull, __float_as_uint(lv) == __float_as_uint(before)) && lane == 0) stop = iter + 1;
+        before = lv;
+    }
+    err = __shfl_sync(kFull, err, 0);
+    if (F.err_log)
+        for (int k = iter + lane; k < F.iters; k += 32) F.err_log[k] = err;
+}
+
 // Whether the difference of two sums {s, sx}, s0 and s1, is too rough to be a region's: not finite, negative, or small beside all that lies
 // in front (2^-50) or beside what was rounded, the `rest` of either sum (2^-8).  What is compared with it is what the region is known to
 // hold: its weight, s0, and of sum |weight x|, which s1 may cancel, the upper rest if the points have different parts in front of them.
