@@ -53,17 +53,18 @@ struct SortWs {
 // paid once, an iteration is cheaper by what it streams.  Both sides by measurement, in us with k = n / 2^20 (blocks of 64;
 // other block sizes differ by a few per cent):
 //   ordering, less what a streamed fit takes before its first iteration
-//             one sample per weight, fp32: 66 (k = 1), 94 (2), 162 (4), 267 (8), 534 (16), 778 (24), 1026 (32), 1514 (48), 2001 (64)
-//             distinct bf16 weights 72 (2), 73 (4), 95 (16), 150 (64), 340 (256)
+//             one sample per weight, fp32: 66 (k = 1), 87 (2), 150 (4), 263 (8), 510 (16), 715 (24), 925 (32), 1360 (48), 1815 (64)
+//             distinct bf16 weights 43 to 56 (2), 48 to 60 (4), 65 to 80 (16), 81 to 120 (64), 109 to 255 (256)
 //   streamed iteration less an ordered one
-//             fp32: MSE 15 (1), 15 (2), 19 (4), 24 (8), 34 (16), 50 (24), 61 (32), 83 (48), 105 (64),
-//             medians 47 (1), 55 (4), 90 (16), 227 (64)
-//             bf16: MSE 17 (2), 16 (4), 32 (16), 80 (64), 255 (256), medians 55, 57, 82, 176, 681
-// The lines below are fits to these, a little on the streamed side, which takes 9 MB of workspace where ordering takes 16 bytes a weight;
-// from 2^25 weights on (more than half a gigabyte) ordering has to save more than it costs: fits of 2^26 weights and up to 32 iterations
-// (medians 23) get by with the small workspace, as callers are promised.  Where they cross, in iterations, and by the figures: fp32
-// MSE 6 (5) at 2^20, 10 (9) at 2^22, 13 (12) at 2^23, 17 (16) at 2^24, 20 (17) at 2^25, 33 (19) at 2^26, medians 4, 4 (3) at 2^22, 9 (7) at
-// 2^24, 24 (9) at 2^26; bf16 MSE 6 (5) from 3 * 2^19 to 2^22, 4 (3) from 2^24 on, medians 4 (2).
+//             fp32: MSE 15 (1), 15 (2), 19 (4), 25 (8), 34 (16), 49 (24), 61 (32), 83 (48), 105 (64),
+//             medians 47 (1), 50 (2), 56 (4), 71 (8), 90 (16), 120 (24), 142 (32), 188 (48), 231 (64)
+//             bf16: MSE 16 (2), 16 (4), 31 (16), 76 (64), 264 (256), medians 54, 58, 82, 180, 679
+// The lines below lie on the streamed side of these, which takes 9 MB of workspace where ordering takes 16 bytes a weight (64 MB and 10
+// bytes a block for bf16 data): a fit at the line has streamed at most two and a half times what the ordering costs.  From 2^25 weights on
+// (more than half a gigabyte) that is on purpose: ordering has to save more than it costs, and squared errors over 2^26 weights get by with the
+// small workspace up to 32 iterations.  Where they cross, in iterations, and by the figures: fp32 MSE 6 (5) at 2^20, 10 (9) at 2^22, 13 (11) at
+// 2^23, 17 (15) at 2^24, 20 (16) at 2^25, 33 (18) at 2^26, medians 4, 4 (3) at 2^22, 7 (4) at 2^23, 9 (6) at 2^24, 11 (7) at 2^25, 19 (8) at
+// 2^26; bf16 MSE 6 (3) from 3 * 2^19 to 2^22, 4 (3) from 2^24 on, medians 4 (2).
 // Fewer than four iterations are not ordered, although two or three would pay for bf16 data from 2^26 weights on (2^28, three: 1000
 // us streamed, about 410 ordered): such a fit gets by with the small workspace.
 inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool cells)
@@ -74,7 +75,7 @@ inline bool ordering_pays(int w_dtype, int64_t n, int metric, int iters, bool ce
     double order = 105.0 + 1.1 * k, gain = mae ? 50.0 + 1.9 * k : 16.5 + 0.9 * k;
     if (!cells) {
         order = fmax(fmin(46.0 + 35.0 * k, 50.0 + 33.0 * k), 70.0 * k - 1120.0);
-        gain = mae ? fmin(fmax(47.5, 31.0 + 2.3 * k), 55.0 + 1.35 * k) : (w_dtype == BOF4_BF16 ? 18.0 : 13.0) + 1.42 * k;
+        gain = mae ? fmax(47.5, 31.0 + 2.3 * k) : (w_dtype == BOF4_BF16 ? 18.0 : 13.0) + 1.42 * k;
     }
     return iters * gain >= order;
 }

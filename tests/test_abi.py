@@ -79,7 +79,7 @@ def test_workspace_sizes(L):
 
 def test_only_a_fit_that_orders_its_samples_asks_for_room_for_them(L):
     """The E step, the joint fit and short fits stream: partial records and candidate lists, whatever the data's
-    size and type.  A long fit asks for 16 bytes per fp32 weight up to 2^26, or about 90 MB and 10 bytes per block (bf16)."""
+    size and type.  A long fit asks for 16 bytes per fp32 weight up to 2^26, or about 64 MB and 10 bytes per block (bf16)."""
     from paper_2505_06653_b200 import binding as b
     base = b.bof4_workspace_bytes(b.OP_EM, 0, 64, b.METRIC_MSE)
     assert base < 10 << 20
@@ -125,6 +125,22 @@ def test_a_fit_is_ordered_where_that_is_faster(L, dtype, lg, metric, few, many):
     assert size(many) == size(1000)
     if lg < 30:      # beyond, the candidate lists of a streamed fit are larger than the cells
         assert size(many) > size(few)
+
+
+# (type, log2 of the weights, metric): what ordering costs and what it gains per iteration, in us
+GAINS = [("f32", 20, 0, 66, 15), ("f32", 22, 0, 156, 19), ("f32", 23, 0, 262, 25), ("f32", 24, 0, 502, 34), ("f32", 25, 0, 937, 61),
+         ("f32", 26, 0, 1830, 105), ("f32", 23, 1, 264, 71), ("f32", 24, 1, 517, 90), ("f32", 25, 1, 911, 142), ("f32", 26, 1, 1814, 231),
+         ("bf16", 21, 0, 43, 16), ("bf16", 24, 0, 65, 31)]
+
+
+@pytest.mark.parametrize("dtype,lg,metric,cost,gain", GAINS)
+def test_a_fit_is_ordered_soon_after_that_pays(L, dtype, lg, metric, cost, gain):
+    """The first number of iterations that is ordered gains what ordering costs, and not more than two and a half times that."""
+    from paper_2505_06653_b200 import binding as b
+    dt = b.F32 if dtype == "f32" else b.BF16
+    small = b.bof4_workspace_bytes(b.OP_EM, 1 << lg, 64, metric)
+    first = next(it for it in range(1, 100) if b.bof4_fit_workspace_bytes(1 << lg, dt, 64, metric, it) > small)
+    assert cost <= first * gain <= 2.5 * cost + gain
 
 
 def test_argument_validation_happens_before_any_cuda_call(L):
