@@ -125,7 +125,7 @@ BOF4_API size_t bof4_workspace_bytes(int op, int64_t n_max, int block_size, int 
  * Bytes of device workspace with which bof4_fit_codebook runs `iters` iterations over n_total weights of
  * w_dtype the fastest way it has.  Never less than BOF4_OP_EM asks for, and no more where the fit streams its
  * data.  A fit of enough iterations puts its samples in order once instead: 16 bytes per weight (fp32, up to
- * 2^26 weights, and bf16 up to 3 * 2^19), or about 90 MB and 10 bytes per block (bf16 from there on).
+ * 2^26 weights, and bf16 up to 3 * 2^19), or about 64 MB and 10 bytes per block (bf16 from there on).
  * Medians do not depend on the workspace size, sums only by their rounding.  Host function, no CUDA call.
  * Returns 0 for invalid arguments.
  */

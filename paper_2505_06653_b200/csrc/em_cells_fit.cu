@@ -369,7 +369,7 @@ cells_fit_mse_kernel(const __grid_constant__ CellsWs W, const __grid_constant__ 
         const double s1 = ((h1.y - h0.y) + (l1.y - l0.y)) + (r1.y - r0.y);
         float moved = (float)(s1 / s0);
         const bool empty = __float_as_uint(c0.y) == __float_as_uint(c1.y);
-        const unsigned by_itself = __ballot_sync(kFull, !fixed && !empty && too_rough(s0, s1, r0, r1, h0.x, h1.x));
+        const unsigned by_itself = __ballot_sync(kFull, !fixed & !empty & too_rough(s0, s1, r0, r1, h0.x, h1.x));
         if (stop <= iter) break;
         if (by_itself & 3u) {
             for (int k = 0; k < 2; ++k) {

@@ -423,3 +423,74 @@ def test_a_median_in_a_crowded_bin_is_looked_for_between_its_thresholds(bof4):
     span fourteen binades, and from nowhere in particular, they took 3.4."""
     w, lv = _crowded(1 << 20, "tiny", 11)
     assert _best_ms(bof4, w.cuda(), lv, 0x8000, bof4.METRIC_MAE, 18) < 2.6
+
+
+def _few_values(dtype, seed):
+    """Blocks of 64 with one of 24 constants of any significand and twelve weights of its own, from 2^-45 of it on (powers of two below
+    2^-40), zeros and the constant's own size among them: a few hundred normalised weights, so that one on the wrong side of a threshold
+    shows.  Returns the weights and, by ascending x: x, sum of m^2, sum of |m|."""
+    rng = np.random.default_rng(seed)
+    blocks = (3 << 19) // 64 if dtype == torch.bfloat16 else 1 << 11
+    sig = rng.integers(128, 256, 24)
+    m = sig * 2.0 ** rng.integers(-9, -6, 24)
+    d = (rng.uniform(0, 45, (24, 12)) ** 1.5 / 45 ** 0.5 * 128).astype(int)       # distances of the bit patterns, small ones more often
+    e, a = -(-(d - sig[:, None] + 128) // 128), (sig[:, None] - 128 - d) % 128 + 128
+    w = np.where(d < 5120, m[:, None] * (a / sig[:, None]) * 2.0 ** -e, m[:, None] * 2.0 ** -(d // 128))
+    w[:, 0], w[:, 1] = 0.0, -m
+    w[:, 2:] *= rng.choice([-1, 1], (24, 10))
+    which = rng.integers(0, 24, blocks)
+    data = np.concatenate([m[which][:, None], w[which[:, None], rng.integers(0, 12, (blocks, 63))]], 1).astype(np.float32)
+    assert np.array_equal(torch.from_numpy(data).to(torch.bfloat16).float().numpy(), data)
+    x, at = np.unique(data / data[:, :1], return_inverse=True)
+    c = np.broadcast_to(data[:, :1].astype(np.float64), data.shape).reshape(-1)
+    return torch.from_numpy(data).to(dtype).reshape(-1), x, np.bincount(at.reshape(-1), c * c), np.bincount(at.reshape(-1), c)
+
+
+def _lloyd(x, s, lv, metric, iters, n):
+    """By the definition: a region is what lies between its thresholds, and nothing where they do not ascend."""
+    lv, log = lv.copy(), []
+    for _ in range(iters):
+        t = (lv[:-1] + lv[1:]) * np.float32(0.5)
+        lo, hi = np.append(np.float32(-np.inf), t), np.append(t, np.float32(np.inf))
+        new, err = lv.copy(), 0.0
+        for k in range(16):
+            i = (x >= lo[k]) & (x < hi[k])
+            v, u = s[i], x[i].astype(np.float64)
+            d = np.abs(u - np.float64(lv[k]))
+            err += (v * (d if metric == 1 else d * d)).sum()
+            if v.sum() > 0:
+                new[k] = x[i][np.argmax(2 * np.cumsum(v) >= v.sum())] if metric == 1 else np.float32((v * u).sum() / v.sum())
+        log.append(err / n)
+        lv = new
+    return lv, np.array(log)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("metric", [0, 1])
+@pytest.mark.parametrize("ascend", [True, False])
+def test_thresholds_at_the_samples(bof4, dtype, metric, ascend):
+    """Eight thresholds of every fit are a normalised weight that occurs, the next number below it or above it; and levels that do not
+    ascend, whose regions are empty (the log of the squared error is not defined for them)."""
+    for seed in range(4):
+        w, x, m2, m1 = _few_values(dtype, seed)
+        dev, rng = w.cuda(), np.random.default_rng(100 + seed)
+        inside = x[(np.abs(x) < 0.99)]
+        for _ in range(12):
+            p = np.sort(rng.choice(inside[np.abs(inside) > 2.0 ** -60], 8, replace=False))
+            p = np.where(rng.random(8) < 0.34, p, np.nextafter(p, np.where(rng.random(8) < 0.5, -9, 9).astype(np.float32)))
+            step = np.spacing(np.abs(p)) * 2
+            step = np.where(((p - step) + (p + step)) * np.float32(0.5) == p, step, step * np.float32(1.5))     # (beside a power of two)
+            lv = np.stack([p - step, p + step], 1).reshape(-1)
+            assert np.array_equal((lv[::2] + lv[1::2]) * np.float32(0.5), p)
+            if not ascend:
+                k = rng.choice(15, 3, replace=False)
+                lv[k], lv[k + 1] = lv[k + 1].copy(), lv[k].copy()
+                lv[rng.integers(1, 16)] = lv[rng.integers(0, 15)]
+            ref, ref_log = _lloyd(x, m1 if metric == 1 else m2, lv, metric, 6, w.numel())
+            cb, log = bof4.bof4_fit_codebook(dev, 64, 0, metric, lv, 0, 6)
+            if metric == 1:
+                assert np.array_equal(cb.cpu().numpy(), ref)
+            else:
+                np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=2e-7, atol=1e-30)
+            if metric == 1 or ascend:
+                np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-9, atol=2.0 ** -50 * float((m1 if metric == 1 else m2).sum()) / w.numel())
