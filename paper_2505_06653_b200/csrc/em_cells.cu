@@ -36,8 +36,10 @@ constexpr int kCellBaseMax = 8192;                // bound on where a unit's cou
 constexpr int kCellThreads = 512;
 constexpr int kCellCtas = 3;                      // per SM
 constexpr int kOrderGroup = 8;                   // blocks that a thread of the ordering takes at a time
-// Below, one sample per weight is cheaper.  20 iterations, MSE and MAE, one sample per weight against this way:
-// 2^20 weights 132 and 241 us against 151 and 236, 2^21 171 and 330 against 157 and 242.
+// Below, a fit has one sample per weight.  That is no longer the faster way (20 iterations, MSE and MAE, one sample per weight against
+// this way: 2^17 weights 77 and 106 us against 73 and 85, 2^19 83 and 120 against 73 and 85, 2^20 93 and 142 against 74 and 87, 2^21 126 and
+// 187 against 75 and 89; the two crossed here while the cells were sorted), but small fits have not got the limits that the cells have (weights
+// below 2^-40 and constants below 2^-38, see the header), and take 16 bytes a weight where the cells take 64 MB.
 constexpr int64_t kCellsMinN = (int64_t)3 << 19;
 constexpr int kMagTiny = 48 * 128;                // |m| below 2^-79: subnormal weights within 40 binades
 

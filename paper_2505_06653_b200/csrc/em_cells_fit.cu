@@ -251,7 +251,7 @@ struct Window {
 };
 
 // An iteration over 2^26 bf16 weights took 1.61 us with cells put in the order of 65,536 bins by sorting, 1.10 with running sums over
-// these bins, 1.11 with places and all sums loaded, 0.85 this way; 1.45 with all thresholds in one warp, a lane each, and no barrier (the chain
+// these bins, 1.11 with places and all sums loaded, 0.9 this way; 1.45 with all thresholds in one warp, a lane each, and no barrier (the chain
 // of a single warp is longer than a barrier and the waiting for others).
 constexpr int kWindow = 256;
 constexpr int kCellsMseLow = (kCellBlocks + 1) * 16;

@@ -248,10 +248,9 @@ __device__ __forceinline__ void rank_in_warp(uint32_t* cnt, int lane, Digit digi
 // so that neighbouring lanes store neighbouring samples, not 32 cache lines a store.  (A digit's counts per warp go back to shared memory
 // as they are added up: kept in registers over the barriers they spilled 90 bytes.)
 constexpr int kScatterSmem = kSortTile * 8;
-// Fits over so many samples, one per weight, stage them: the ordering of 2^20 takes 87 us instead of 92, of 2^23 298 instead of
-// 384, of 2^24 563 instead of 778, of 2^26 2030 instead of 3790.  Fewer fill a tile in
-// part, and the barriers cost what the stores save.  Staged and not, 40 iterations: 2^18 weights 140.8 and 138.7 us, 2^19 147.4
-// and 147.5, 3 * 2^18 152 and 155, 2^20 157 and 163.
+// Fits over so many samples, one per weight, stage them.  Fewer fill a tile in part, and the barriers cost what the stores save.  Staged and
+// not, 50 iterations: 2^18 weights 127.8 and 126.9 us, 2^19 129.4 and 130.7, 3 * 2^18 135.0 and 138.4, 2^20 139.9 and 145.6, 2^23 384 and
+// 459, 2^24 702 and 890.
 constexpr int64_t kStagedMin = 1 << 19;
 template <int SHIFT, bool STAGED>
 __global__ void __launch_bounds__(kSortThreads)
@@ -421,8 +420,8 @@ __device__ __forceinline__ void sums_add(SortSums& t, const SortSums& v)
 // beside them; what a threshold takes of the bin, and where its weight reaches a half, is then found by bisection in every
 // window, a lane each: 1.1 and 1.3 ms, of which 0.8 are the ordering that other data takes as well.  An iteration now costs
 // at most a few bisections (14 steps of an access to L2 each) per 2^20 samples of a crowded bin, and median step.
-// Other data pays for a launch that finds nothing to do (two for medians) and for the test of the flag: 50 iterations over 2^20
-// weights 166.7 -> 167.7 us, 12 of medians 146 -> 150.
+// Other data pays for a launch that finds nothing to do (two for medians) and for the test of the flag: 12 iterations over 2^20
+// weights 92.9 -> 97.0 us (50 of them 140.5 -> 137.6, for no known reason), 12 of medians 119.5 -> 124.9.
 
 // One CTA per window of kSortWindow samples: four stable passes of eight bits by the key of x in shared memory, then the
 // running sums (exclusive within the window, every fourth sample).
@@ -678,7 +677,7 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE> weight)
 // One warp per group of 32 bins: empty bins are cleared, bins that cross chunks put together (in the
 // order of the chunks), and the sums of the group, of the bins in front of each formed.
 // Bound by the latency of its loads: with all crossing bins put together one after the other by the whole warp
-// it took 14.6 us for 2^20 samples, 3.7 with those of up to kSortFew chunks a lane each (cells of 2^26 weights 22.9, 10.5).
+// it took 14.6 us for 2^20 samples, 3.7 with those of up to kSortFew chunks a lane each.
 // Between 4 and 64 chunks as the line the fits of 2^18 to 2^24 weights differ by less than 2 us; at 64 those of 2^18 are 1.5 slower.
 constexpr uint32_t kSortFew = 16;
 // A bin of very many chunks (crowded, or one of a single value: the zeros of sparse data) is put together by the whole CTA:
@@ -760,7 +759,7 @@ sort_group_kernel(const SortWs W)
 //
 // What lies below a threshold (em_fit.cuh): the groups in front of its bin's, in shared memory, the bins of the group in front of it
 // (one load), and the samples of its bin.  The first samples of all bins are in shared memory (16 bits beside the group's first),
-// which leaves one access to L2 in the chain: 1.12 us an iteration over 2^20 fp32 weights (1.60 with cuts found by one warp, whole
+// which leaves one access to L2 in the chain: 1.14 us an iteration over 2^20 fp32 weights (1.60 with cuts found by one warp, whole
 // groups added up between them and three barriers), 3.5 over 2^24 (3.9).  Of its 2200 cycles the bin takes 130, its first sample 220,
 // the samples 430 or 820, by where in L2 they are, their reduction 230, the barrier and what it waits for 200, the differences 300
 // and the quotients with the test of the sums 330.  (The next iteration's samples requested ahead, by the last steps of the
@@ -1174,7 +1173,7 @@ __device__ __forceinline__ void fit_mae_loop(Source& source, FitMaeShared& S, un
 
 // What lies below a threshold: as for the squared error.  The place of a median: in the running sums of the groups (shared memory,
 // 64 entries a step), then of the group's bins (one load), then among the samples of one bin.
-// An iteration over 2^20 fp32 weights 6.5 -> 3.1 us, over 2^24 33 -> 14 (before: two warps to a region, whole groups added up and
+// An iteration over 2^20 fp32 weights 6.5 -> 3.1 us, over 2^24 33 -> 14.5 (before: two warps to a region, whole groups added up and
 // searched one after the other, cut bins first).  Bound by its chain: three loads from L2 of 430 or 820 cycles each, the
 // reductions, two barriers; over 2^24 weights by the passes over the 500 samples of a bin (of up to 64 samples every lane adds
 // up what is not behind its own, in one pass: 2^20 weights 3.75 -> 3.1).
@@ -1363,7 +1362,7 @@ struct MaeSamples {
 };
 
 // CROWDED: the kernel for data with crowded bins.  Both are launched, the flag of such bins tells which one runs: with both
-// loops in one kernel 2^22 fp32 weights, 12 iterations, took 299 us against 293.5, 2^20 153.8 against 152.4.
+// loops in one kernel 2^22 fp32 weights, 12 iterations, take 252.9 us against 246.2, 2^20 125.2 against 124.9.
 template <bool CROWDED>
 __global__ void __launch_bounds__(kFitMaeThreads, 1)
 sort_fit_mae_kernel(const __grid_constant__ SortWs W, const __grid_constant__ SortFit F)

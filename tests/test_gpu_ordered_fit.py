@@ -180,6 +180,22 @@ def test_crowded_bins(bof4, n, kind, metric):
     np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-5, atol=2.0 ** -50 * float((w.double() ** 2).mean()))
 
 
+def _best_ms(bof4, w, lv, mask, metric, iters):
+    """Time of a fit, with the launches queued behind a wait of 10 ms: the host's time is not in it, nor are its pauses, which on a shared
+    machine can be longer than any fit here (85 ms were seen)."""
+    room = torch.empty(bof4.bof4_fit_workspace_bytes(w.numel(), bof4.F32, 64, metric, iters), dtype=torch.uint8, device="cuda")
+    best = 1e9
+    for _ in range(9):
+        s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda._sleep(20_000_000)
+        s.record()
+        bof4.bof4_fit_codebook(w, 64, 0, metric, lv, mask, iters, workspace=room, sync=False)
+        e.record()
+        torch.cuda.synchronize()
+        best = min(best, s.elapsed_time(e))
+    return best
+
+
 def test_crowded_bins_take_bounded_time(bof4):
     """2^22 weights that have been quantised before (sixteen levels, every block with its own constant): 150 000 samples and
     more in a bin.  Looked through by one warp, a fit takes 16 ms (medians) and streaming the data 14."""
@@ -190,14 +206,7 @@ def test_crowded_bins_take_bounded_time(bof4):
     w = (q * torch.rand(n // 64, 1, generator=g) * 0.01).reshape(-1).cuda()
     lv, mask = bof4.bof4_default_init(0)
     for metric in (0, 1):
-        best = 1e9
-        for _ in range(3):
-            s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            s.record()
-            bof4.bof4_fit_codebook(w, 64, 0, metric, lv, mask, 32, sync=False)
-            e.record()
-            torch.cuda.synchronize()
-            best = min(best, s.elapsed_time(e))
+        best = _best_ms(bof4, w, lv, mask, metric, 32)
         assert best < 5.0, (metric, best)
 
 
@@ -342,21 +351,6 @@ def test_the_absolute_error_is_added_up_by_regions(bof4, n, dtype, kind):
         ref, mean = _absolute_error(w, lv)
         assert abs(log[0].item() - ref) <= 2.0 ** -53 * mean, (seed, float((log[0].item() - ref) / mean))
         assert (log == log[0]).all()
-
-
-def _best_ms(bof4, w, lv, mask, metric, iters):
-    """Time of a fit, with the launches queued behind a wait so that the host's time is not in it."""
-    room = torch.empty(bof4.bof4_fit_workspace_bytes(w.numel(), bof4.F32, 64, metric, iters), dtype=torch.uint8, device="cuda")
-    best = 1e9
-    for _ in range(9):
-        s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        torch.cuda._sleep(2_000_000)
-        s.record()
-        bof4.bof4_fit_codebook(w, 64, 0, metric, lv, mask, iters, workspace=room, sync=False)
-        e.record()
-        torch.cuda.synchronize()
-        best = min(best, s.elapsed_time(e))
-    return best
 
 
 def _iteration_us(bof4, w, lv, mask, metric):
