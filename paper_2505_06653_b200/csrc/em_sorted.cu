@@ -585,11 +585,16 @@ __device__ __noinline__ void crowded_sums(const SortWs& W, const SampleWeight<MA
     }
 }
 
-// One warp per kSortChunk ordered samples, 32 at a time: a segmented scan over the runs of equal bins; the first samples of all bins
-// on the way (with a launch of their own fits of 2^20 weights took 3 us longer).
+// First samples of all bins: a thread each, by bisection, in CTAs of their own beside those that form the sums.  (Written by the sums' warps as they
+// come to the ends of runs, the gaps between few samples are long chains of stores: 1000 weights, 12 iterations, 89 us and 70 this way,
+// 2^14 81.7 and 75.4, 2^20 93.9 and 93.4, medians of 2^24 710 and 701; with a launch before, 80, 81, 99.6 and 969 for the fit as it was then.
+// By halves, quarters and eighths 2^18 82.5, 80.9 and 81.3, 2^24 699, 701 and 705.)
+//
+// Sums: one warp per kSortChunk ordered samples, 32 at a time: a segmented scan over the runs of equal bins.
 // A run that lies inside the chunk is a bin's sum; parts of runs that cross the chunk's edges go to
 // lead / trail and are put together by sort_group_kernel.  The work is even whatever the distribution (the bins
 // of x = +-1 hold 1 / I of the data; a bin of small data is mostly empty).
+constexpr int kStartCtas = kSortBins / 256;
 template <bool MAE>
 __global__ void __launch_bounds__(256)
 sort_sums_kernel(const SortWs W, SampleWeight<MAE> weight)
@@ -597,10 +602,29 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE> weight)
     if (!after_previous()) return;
     constexpr int STEPS = kSortChunk / 32, kNone = 1 << 20;
     const uint32_t n = W.n_items[0];
+    if (blockIdx.x < kStartCtas) {
+        const int bin = (int)(blockIdx.x * 256 + threadIdx.x);
+        uint32_t from = 0u, to = n;
+        while (from < to) {  // quarters: half the dependent loads that halves take
+            const uint32_t part = (to - from + 3u) / 4u;
+            uint32_t in_front = 0u;
+#pragma unroll
+            for (int u = 1; u < 4; ++u) {
+                const uint32_t last = from + u * part - 1u;
+                const int at = sort_bin(W.b[min(last, to - 1u)].x);
+                in_front += (last < to && at < bin) ? 1u : 0u;
+            }
+            from += in_front * part;
+            if (in_front < 3u) to = min(to, from + part - 1u);
+        }
+        W.start[bin] = from;
+        if (bin == 0) W.start[kSortBins] = n;
+        return;
+    }
     weight.max_bits = W.n_items[1];
     const int lane = threadIdx.x & 31;
-    const uint32_t warps = gridDim.x * 8u;
-    for (uint32_t c = blockIdx.x * 8u + (threadIdx.x >> 5); (uint64_t)c * kSortChunk < n; c += warps) {
+    const uint32_t warps = (gridDim.x - kStartCtas) * 8u;
+    for (uint32_t c = (blockIdx.x - kStartCtas) * 8u + (threadIdx.x >> 5); (uint64_t)c * kSortChunk < n; c += warps) {
         const uint32_t lo = c * kSortChunk, hi = min(n, lo + kSortChunk);
         float2 it[STEPS];
         SortSums v[STEPS];
@@ -630,17 +654,6 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE> weight)
             int left = __shfl_up_sync(kFull, key[k], 1);
             if (lane == 0) left = open_key;
             const unsigned heads = __ballot_sync(kFull, key[k] != left);
-            // the sample is the first of all bins behind the one of the sample before it up to its own; a gap of many empty bins is
-            // filled by the warp
-            const bool starts = key[k] != left && key[k] != kNone, wide = starts && key[k] - left > 64;
-            const uint32_t i = lo + 32 * k + lane;
-            if (starts && !wide)
-                for (int t = left + 1; t <= key[k]; ++t) W.start[t] = i;
-            for (unsigned far = __ballot_sync(kFull, wide); far; far &= far - 1u) {
-                const int who = __ffs(far) - 1, t1 = __shfl_sync(kFull, key[k], who);
-                const uint32_t first = __shfl_sync(kFull, i, who);
-                for (int t = __shfl_sync(kFull, left, who) + 1 + lane; t <= t1; t += 32) W.start[t] = first;
-            }
             if ((heads & 1u) && k > 0 && lane == 0 && open_key != kNone) (early ? W.lead[c] : W.bin[open_key]) = open;
             const unsigned upto = heads & ((2u << lane) - 1u);
             const int from = upto ? 31 - __clz(upto) : 0;
@@ -662,13 +675,6 @@ sort_sums_kernel(const SortWs W, SampleWeight<MAE> weight)
             if (MAE) open.a = __shfl_sync(kFull, t.a, 31);
             open_key = __shfl_sync(kFull, key[k], 31);
             early = early && heads == 0u;
-        }
-        if (hi == n) {  // behind the last sample come all bins that are left
-            int top = -1;
-#pragma unroll
-            for (int k = 0; k < STEPS; ++k) top = max(top, key[k] == kNone ? -1 : key[k]);
-            top = __reduce_max_sync(kFull, top);
-            for (int t = top + 1 + lane; t <= kSortBins; t += 32) W.start[t] = n;
         }
         if (lane == 0 && open_key != kNone) (early ? W.lead[c] : open_key == behind ? W.trail[c] : W.bin[open_key]) = open;
     }
@@ -1407,7 +1413,7 @@ int sums_and_iterations(const SortWs& W, const SortFit& F, cudaStream_t st)
     SampleWeight<MAE> weight{};
     weight.unit = F.metric >= 2;
     const int64_t ctas = (F.n_max + 8 * kSortChunk - 1) / (8 * kSortChunk);
-    launch_after(sort_sums_kernel<MAE>, (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, W, weight);
+    launch_after(sort_sums_kernel<MAE>, kStartCtas + (int)(ctas < 8 * kSMs ? ctas : 8 * kSMs), 256, 0, st, W, weight);
     launch_after(sort_group_kernel<MAE>, kSortGroups / 8, 256, 0, st, W);
     auto order_windows = [&]() -> int {
         constexpr auto kern = sort_windows_kernel<MAE>;

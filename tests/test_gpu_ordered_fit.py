@@ -488,3 +488,11 @@ def test_thresholds_at_the_samples(bof4, dtype, metric, ascend):
                 np.testing.assert_allclose(cb.cpu().numpy(), ref, rtol=2e-7, atol=1e-30)
             if metric == 1 or ascend:
                 np.testing.assert_allclose(log.cpu().numpy(), ref_log, rtol=1e-9, atol=2.0 ** -50 * float((m1 if metric == 1 else m2).sum()) / w.numel())
+
+
+@pytest.mark.parametrize("metric", [0, 1])
+def test_few_weights_take_no_longer_than_many(bof4, metric):
+    """1000 weights leave most bins empty: finding the bins' first samples took longer than all else was shorter (86 us against 71)."""
+    lv, mask = bof4.bof4_default_init(0)
+    few, many = (_best_ms(bof4, _weights(n, torch.float32, 3, "plain").cuda(), lv, mask, metric, 6) for n in (1000, 1 << 16))
+    assert few < many
