@@ -38,7 +38,7 @@ struct SortSums {      // per bin, per group, or per part of a bin
 struct SortWs {
     uint32_t* n_items;    // device: [0] samples, [1] bits of the largest block constant, [4] whether a bin is crowded
     double* w2;           // [kSortParts]
-    uint32_t* counts;     // [kSortGrid][256]
+    uint32_t* counts;     // [kSortGrid][256]; behind the ordering passes running sums of the groups, see sort_fit_mae_kernel
     uint32_t* start;      // [kSortBins + 1] first sample of every bin
     uint32_t* first;      // [kSortGroups + 1] first sample of every group; before, the largest constants of the samples' CTAs
     uint16_t* off;        // [kSortBins] first sample of a bin in its group, kFarBin: too far, see start
